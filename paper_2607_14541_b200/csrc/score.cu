@@ -1,4 +1,4 @@
-// Roofline score aggregation (Eq. 4-6), batched over candidates: one CTA per candidate.
+// Roofline score aggregation (Eq. 4-6), batched over candidates.
 //
 //   Eq. 4  S_j = T_roofline,j / T_cand,j for units that passed correctness (a value above 1, or a
 //          candidate time that is not a finite positive number, is counted as an evaluation
@@ -7,12 +7,26 @@
 //          0 when there is none
 //   Eq. 6  S_agg = sum_i w_i S_i, accumulated in operator order
 //
-// Every floating-point step is one explicit round-to-nearest operation in a fixed order, so
-// the result has one bit pattern.  The median of a small group is found by ranking (each value's
-// rank is the number of values that sort before it, ties broken by position), that of a large one
-// by a bitwise search for the wanted order statistics; neither needs a sorting network or scratch
-// memory beyond the CTA's shared memory.
+// Every floating-point step of a result is one explicit round-to-nearest operation in a fixed order, so
+// the result has one bit pattern.
+//
+// Where a unit goes when units are grouped by operator is the same for every candidate, so a CTA works
+// that out once and then goes through its candidates.  Two kernels:
+//   score_warp_kernel  one candidate per warp, no barriers: many candidates of few units
+//   score_cta_kernel   one candidate per CTA: few candidates, or more units than a warp should hold
+// The kernel before these (one candidate per CTA, grouping redone for every candidate, exact scores ranked
+// against each other) was bound by its barriers and shared-memory atomics: 65 536 candidates x 440 units x
+// 30 operators in 594 us, 1 000 x 12 001 units x 7 operators in 1 179 us.
+//
+// Ranking does not need exact quotients.  A unit's approximate score is formed in binary32 -- two
+// conversions, a reciprocal and a product, within six units in the last place of the exact quotient -- and
+// its bit pattern is the key; only the one or two middle units of an operator are divided in binary64.
+// That is right as long as no other key of the operator is close to a middle one: then the middle units by
+// key are the middle units by score.  Where one is (ties among them), or an operand is outside the range
+// the approximation is good for, the operator's candidates for the middle are ranked by exact quotients.
+#include <cmath>
 #include <mutex>
+#include <utility>
 
 #include "kernels.h"
 
@@ -20,131 +34,779 @@ using namespace atrex;
 
 namespace {
 
-constexpr int SCORE_THREADS = 256;
+constexpr uint32_t FULL = 0xFFFFFFFFu;
+constexpr uint32_t SELECT_BINS = 128;
 
-// Order statistics of a large group.  A double's bit pattern, with the sign bit flipped for positive
-// values and all bits flipped for negative ones, orders like the value; the k-th smallest key (k from
-// 0) is the largest v with #{key < v} <= k, found one bit at a time.  Called by a whole warp; every
-// lane returns the value.
-constexpr uint32_t SELECT_ABOVE = 128;   // below this, ranking every value against every other is cheaper
-__device__ __forceinline__ unsigned long long order_key(double x) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+// Order-preserving key of an exact score: a double's bit pattern with the sign bit flipped for positive values
+// and all bits flipped for negative ones.  Any NaN (a unit without a roofline) gets one pattern, above +inf.
+__device__ __forceinline__ ull key_of_score(double x) {
+    if (x != x) return 0xFFF8000000000000ull;
+    const ull b = (ull)__double_as_longlong(x);
     return b ^ ((b >> 63) ? ~0ull : (1ull << 63));
 }
-__device__ __forceinline__ double select_kth(const double* v, uint32_t m, uint32_t k, uint32_t lane) {
-    unsigned long long ans = 0;
-    for (int bit = 63; bit >= 0; --bit) {
-        const unsigned long long trial = ans | (1ull << bit);
-        uint32_t below = 0;
-        for (uint32_t a = lane; a < m; a += 32) below += order_key(v[a]) < trial ? 1u : 0u;
-        below = __reduce_add_sync(0xFFFFFFFFu, below);
-        if (below <= k) ans = trial;
-    }
-    const unsigned long long b = ans ^ ((ans >> 63) ? (1ull << 63) : ~0ull);
-    return __longlong_as_double((long long)b);
+__device__ __forceinline__ double score_of_key(ull k) { return __longlong_as_double((long long)(k ^ ((k >> 63) ? (1ull << 63) : ~0ull))); }
+__device__ __forceinline__ double median_of_keys(ull lo, ull hi, bool odd) {
+    const double h = score_of_key(hi);
+    return odd ? h : __dmul_rn(__dadd_rn(score_of_key(lo), h), 0.5);
+}
+// Eq. 4 for one unit: its exact key, or all ones where it has no usable score.
+__device__ __forceinline__ ull exact_key(double roofline, double t, bool ok) {
+    return ok && t > 0.0 && !isinf(t) ? key_of_score(__ddiv_rn(roofline, t)) : ~0ull;
 }
 
-__global__ void __launch_bounds__(SCORE_THREADS) score_kernel(const double* __restrict__ roofline_s,
-                                                              const uint32_t* __restrict__ unit_op, uint32_t n_units,
-                                                              const double* __restrict__ t_cand,
-                                                              const uint8_t* __restrict__ correct,
-                                                              const double* __restrict__ w, uint32_t n_ops,
-                                                              double* s_agg, double* s_op_out, ull* errors_out) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    double* s_val = reinterpret_cast<double*>(smem_raw);                   // [n_units] S_j grouped by operator
-    double* s_med = s_val + n_units;                                       // [n_ops]   S_i
-    uint32_t* s_start = reinterpret_cast<uint32_t*>(s_med + n_ops);        // [n_ops + 1]
-    uint32_t* s_fill = s_start + n_ops + 1;                                // [n_ops]
-    __shared__ unsigned int s_errors;
-    const ull cand = blockIdx.x;
-    const double* t = t_cand + cand * n_units;
-    const uint8_t* ok = correct + cand * n_units;
+constexpr uint32_t K_ABSENT = 0x7FFFFFFFu;       // no usable score: sorts last
+constexpr uint32_t K_UNKNOWN = 0x7FFFFFC0u;      // usable, but outside the approximation's range (above every approximation)
+constexpr uint32_t K_APART = 16;                 // keys further apart than this are in the order of the exact scores
+// Operands between 2^-60 and 2^60 keep every step of the approximation a normal number.
+constexpr uint32_t SAFE_LOW = (1023u - 60u) << 20, SAFE_SPAN = 120u << 20;
+__device__ __forceinline__ bool in_safe_range(double x) { return (uint32_t)__double2hiint(x) - SAFE_LOW < SAFE_SPAN; }
+__device__ __forceinline__ float approx_roofline(double r) { return in_safe_range(r) ? (float)r : __int_as_float(0x7FFFFFFF); }
 
-    for (uint32_t i = threadIdx.x; i < n_ops; i += blockDim.x) s_fill[i] = 0;
-    if (threadIdx.x == 0) s_errors = 0;
+// Key of one unit and its evaluation errors; `r` = approx_roofline(*roofline), no branch on the usual way.
+__device__ __forceinline__ uint32_t approx_key(float r, const double* roofline, double t, bool use, uint32_t& errors) {
+    uint32_t key = (uint32_t)__float_as_int(__fdividef(r, (float)t));
+    // fl(roofline / t) > 1 exactly when roofline > t; the approximation settles it away from 1
+    const bool special = !in_safe_range(t) | (key > 0x3F800000u - K_APART);   // (a NaN is far above)
+    key = use ? key : K_ABSENT;
+    if (use & special) {
+        if (!(t > 0.0) || isinf(t)) {
+            key = K_ABSENT;
+            ++errors;
+        } else {
+            if (!in_safe_range(t) || r != r) key = K_UNKNOWN;
+            errors += __ldg(roofline) > t ? 1u : 0u;
+        }
+    }
+    return key;
+}
+
+// The k-th and (k+1)-th smallest (from 0) of the usable keys among the g keys key_at(0 .. g - 1), by one warp:
+// the range that holds the k-th is cut into up to 128 equal bins, counted, and narrowed to one bin until
+// that bin's keys fit the lanes (two rounds for a thousand spread-out values), where they are ranked.
+// A range of one value ends the search as well, so ties cost nothing; each round narrows the range at
+// least 64-fold, so there are at most eleven.  K: 32- or 64-bit keys, all ones = no usable score.
+// `bins`: SELECT_BINS words of this warp's.
+template <typename K, typename KeyAt>
+__device__ __noinline__ void warp_select(KeyAt key_at, uint32_t g, uint32_t k, uint32_t* bins, K* out_k, K* out_next) {
+    constexpr K NONE = ~(K)0;
+    const uint32_t lane = threadIdx.x & 31u;
+    K lo = NONE, hi = 0;
+#pragma unroll 4
+    for (uint32_t a = lane; a < g; a += 32) {
+        const K x = key_at(a);
+        if (x == NONE) continue;
+        lo = min(lo, x);
+        hi = max(hi, x);
+    }
+#pragma unroll
+    for (int d = 16; d; d >>= 1) {
+        lo = min(lo, __shfl_xor_sync(FULL, lo, d));
+        hi = max(hi, __shfl_xor_sync(FULL, hi, d));
+    }
+    K next_above = NONE;         // smallest key above the current range
+    while (lo != hi) {
+        const int len = 64 - __clzll((long long)(ull)(hi - lo));
+        const int shift = len > 7 ? len - 7 : 0;
+        reinterpret_cast<uint4*>(bins)[lane] = make_uint4(0, 0, 0, 0);
+        __syncwarp();
+#pragma unroll 4
+        for (uint32_t a = lane; a < g; a += 32) {
+            const K x = key_at(a);
+            if (x >= lo && x <= hi) atomicAdd(&bins[(uint32_t)((x - lo) >> shift)], 1u);
+        }
+        __syncwarp();
+        const uint4 c = reinterpret_cast<const uint4*>(bins)[lane];
+        const uint32_t own = c.x + c.y + c.z + c.w;
+        uint32_t incl = own;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t o = __shfl_up_sync(FULL, incl, d);
+            if (lane >= (uint32_t)d) incl += o;
+        }
+        const uint32_t src = __ffs(__ballot_sync(FULL, incl > k)) - 1;   // the lane whose four bins hold the k-th
+        uint32_t before = incl - own, bin = lane * 4, n = c.x;
+        if (k >= before + n) { before += n; ++bin; n = c.y; if (k >= before + n) { before += n; ++bin; n = c.z; if (k >= before + n) { before += n; ++bin; n = c.w; } } }
+        bin = __shfl_sync(FULL, bin, src);
+        k -= __shfl_sync(FULL, before, src);
+        n = __shfl_sync(FULL, n, src);
+        __syncwarp();   // the bins are reused
+        lo += (K)bin << shift;
+        hi = min(hi, lo + (((K)1 << shift) - 1));
+        if (n <= 32) break;
+    }
+    // keys in [lo, hi] to the lanes (at most 32 unless the range is one value), and the smallest key above it
+    uint32_t n = 0;
+    K* list = reinterpret_cast<K*>(bins);
+#pragma unroll 4
+    for (uint32_t a0 = 0; a0 < g; a0 += 32) {
+        const K x = a0 + lane < g ? key_at(a0 + lane) : NONE;
+        const bool in = x >= lo && x <= hi;
+        if (x > hi) next_above = min(next_above, x);
+        const uint32_t votes = __ballot_sync(FULL, in);
+        const uint32_t pos = n + __popc(votes & ((1u << lane) - 1u));
+        if (in && pos < 32) list[pos] = x;
+        n += __popc(votes);
+    }
+#pragma unroll
+    for (int d = 16; d; d >>= 1) next_above = min(next_above, __shfl_xor_sync(FULL, next_above, d));
+    __syncwarp();
+    if (lo == hi) {
+        *out_k = lo;
+        *out_next = k + 1 < n ? lo : next_above;
+    } else {
+        const K x = lane < n ? list[lane] : NONE;
+        uint32_t less = 0, leq = 0;
+        for (uint32_t b = 0; b < n; ++b) {
+            const K y = list[b];
+            less += y < x ? 1u : 0u;
+            leq += y <= x ? 1u : 0u;
+        }
+        const uint32_t at_k = __ffs(__ballot_sync(FULL, lane < n && less <= k && k < leq)) - 1;
+        *out_k = __shfl_sync(FULL, x, at_k);
+        const uint32_t at_next = __ballot_sync(FULL, lane < n && less <= k + 1 && k + 1 < leq);
+        const K in_list = __shfl_sync(FULL, x, at_next ? __ffs(at_next) - 1 : 0);
+        *out_next = k + 1 < n ? in_list : next_above;
+    }
+    __syncwarp();   // `bins` may be overwritten from here on
+}
+
+// The middle of one operator's keys, by one warp: number of usable units, the lower and upper middle keys (no
+// key lies between them), how many keys are within K_APART of them, how many are below those.
+struct Middle {
+    uint32_t m, v_lo, v_up, close, below;
+    bool unknown;                                       // a key outside the approximation's range: nothing else is valid
+    __device__ __forceinline__ uint32_t from() const { return v_lo - K_APART; }
+    __device__ __forceinline__ uint32_t span() const { return v_up - v_lo + 2 * K_APART; }
+    __device__ __forceinline__ bool clear() const { return close == 2 - (m & 1u) && ((m & 1u) || v_up - v_lo > K_APART); }
+};
+
+// Up to 32 R keys held in registers: the range of the wanted key is halved (a count over the warp each time)
+// until one key is left in it.
+template <int R>
+__device__ __forceinline__ Middle middle_in_registers(const uint32_t* keys, uint32_t g) {
+    const uint32_t lane = threadIdx.x & 31u;
+    uint32_t x[R], least = ~0u, most = 0, usable = 0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const uint32_t a = lane + 32 * r;
+        x[r] = a < g ? keys[a] : K_ABSENT;
+        least = min(least, x[r]);
+        most = max(most, x[r] == K_ABSENT ? 0u : x[r]);
+        usable += x[r] != K_ABSENT ? 1u : 0u;
+    }
+    Middle d;
+    d.m = __reduce_add_sync(FULL, usable);
+    uint32_t lo = __reduce_min_sync(FULL, least), hi = __reduce_max_sync(FULL, most);
+    d.unknown = hi == K_UNKNOWN;
+    d.v_lo = d.v_up = d.close = d.below = 0;
+    if (d.m == 0 || d.unknown) return d;
+    const uint32_t k = (d.m - 1) / 2;
+    uint32_t before = 0, through = d.m;    // keys below lo, keys up to hi
+    while (through - before > 1 && lo < hi) {
+        const uint32_t half = lo + (hi - lo) / 2 + 1;
+        uint32_t c = 0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) c += x[r] < half ? 1u : 0u;
+        c = __reduce_add_sync(FULL, c);
+        if (k < c) {
+            hi = half - 1;
+            through = c;
+        } else {
+            lo = half;
+            before = c;
+        }
+    }
+    uint32_t v = ~0u;
+#pragma unroll
+    for (int r = 0; r < R; ++r) v = min(v, x[r] >= lo ? x[r] : ~0u);
+    d.v_lo = d.v_up = __reduce_min_sync(FULL, v);
+    if (!(d.m & 1u)) {
+        uint32_t leq = 0, up = ~0u;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            leq += x[r] <= d.v_lo ? 1u : 0u;
+            up = min(up, x[r] > d.v_lo ? x[r] : ~0u);
+        }
+        up = __reduce_min_sync(FULL, up);
+        if (__reduce_add_sync(FULL, leq) == k + 1) d.v_up = up;
+    }
+    uint32_t close = 0, below = 0;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        close += x[r] - d.from() <= d.span() ? 1u : 0u;
+        below += x[r] < d.from() ? 1u : 0u;
+    }
+    d.close = __reduce_add_sync(FULL, close);
+    d.below = __reduce_add_sync(FULL, below);
+    return d;
+}
+
+__device__ __noinline__ Middle group_middle(const uint32_t* keys, uint32_t g, uint32_t* bins) {
+    if (g <= 32) return middle_in_registers<1>(keys, g);
+    if (g <= 64) return middle_in_registers<2>(keys, g);
+    if (g <= 128) return middle_in_registers<4>(keys, g);
+    if (g <= 256) return middle_in_registers<8>(keys, g);
+    const uint32_t lane = threadIdx.x & 31u;
+    Middle d;
+    uint32_t m = 0, unknown = 0;
+#pragma unroll 4
+    for (uint32_t a = lane; a < g; a += 32) {
+        const uint32_t x = keys[a];
+        m += x != K_ABSENT ? 1u : 0u;
+        unknown |= x == K_UNKNOWN ? 1u : 0u;
+    }
+    d.m = __reduce_add_sync(FULL, m);
+    d.unknown = __any_sync(FULL, unknown);
+    d.v_lo = d.v_up = d.close = d.below = 0;
+    if (d.m == 0 || d.unknown) return d;
+    uint32_t next;
+    warp_select<uint32_t>([=](uint32_t a) { const uint32_t k = keys[a]; return k == K_ABSENT ? ~0u : k; }, g, (d.m - 1) / 2, bins, &d.v_lo, &next);
+    d.v_up = (d.m & 1u) ? d.v_lo : next;
+    uint32_t close = 0, below = 0;
+#pragma unroll 4
+    for (uint32_t a = lane; a < g; a += 32) {
+        const uint32_t x = keys[a];
+        close += x - d.from() <= d.span() ? 1u : 0u;
+        below += x < d.from() ? 1u : 0u;
+    }
+    d.close = __reduce_add_sync(FULL, close);
+    d.below = __reduce_add_sync(FULL, below);
+    return d;
+}
+
+// Sizes of the operators' groups (whole CTA).
+__device__ __forceinline__ void count_groups(const uint32_t* __restrict__ unit_op, uint32_t n_units, uint32_t n_ops, uint32_t* size) {
+    for (uint32_t i = threadIdx.x; i < n_ops; i += blockDim.x) size[i] = 0;
     __syncthreads();
-    // count the usable units of each operator
     for (uint32_t j = threadIdx.x; j < n_units; j += blockDim.x) {
         const uint32_t op = unit_op[j];
-        if (!ok[j] || op >= n_ops) continue;
-        const double tj = t[j];
-        if (!(tj > 0.0) || isinf(tj)) {
-            atomicAdd(&s_errors, 1u);
-            continue;
-        }
-        atomicAdd(&s_fill[op], 1u);
+        if (op < n_ops) atomicAdd(&size[op], 1u);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        uint32_t run = 0;
-        for (uint32_t i = 0; i < n_ops; ++i) {
-            s_start[i] = run;
-            run += s_fill[i];
-            s_fill[i] = 0;
-        }
-        s_start[n_ops] = run;
+}
+
+// ---- one candidate per warp ---------------------------------------------------------------------
+// Bound by the integer pipe.  A lane sorts its operator's keys in registers (up to 32, a pruned odd-even
+// merge network: two instructions per comparator, no divergence; each key carries its slot in its low five
+// bits).  Groups above 32 are searched by the whole warp, operators whose keys cannot decide on exact
+// quotients.  65 536 candidates x 440 units x 30 operators: 145 us (1 410 warp instructions per candidate,
+// half of the issue slots; the inputs alone take 42 us); ranking exact keys by counting took 4 050
+// instructions and 319 us.
+constexpr uint32_t NET_MAX = 32;                 // largest group that a lane sorts
+constexpr uint32_t K_SLOT = 31u;                 // low bits of a lane's keys: their slots
+constexpr uint32_t NET_APART = 64;               // keys with slots: further apart than this is the order of the exact scores
+
+// Ascending sort of v[0 .. N - 1]: Batcher's odd-even merge network for 32 with the comparators beyond N left
+// out, spelled out at compile time (an index that is not a constant would put v in local memory).
+template <int N>
+struct Network {
+    int n = 0, a[191] = {}, b[191] = {};
+    constexpr Network() {
+        for (int p = 1; p < 32; p *= 2)
+            for (int k = p; k >= 1; k /= 2)
+                for (int j = k % p; j + k < 32; j += 2 * k)
+                    for (int i = 0; i < k; ++i)
+                        if ((i + j) / (2 * p) == (i + j + k) / (2 * p) && i + j + k < N) {
+                            a[n] = i + j;
+                            b[n++] = i + j + k;
+                        }
     }
-    __syncthreads();
-    // Eq. 4, placed into the operator's segment
-    for (uint32_t j = threadIdx.x; j < n_units; j += blockDim.x) {
-        const uint32_t op = unit_op[j];
-        if (!ok[j] || op >= n_ops) continue;
-        const double tj = t[j];
-        if (!(tj > 0.0) || isinf(tj)) continue;
-        const double s = __ddiv_rn(roofline_s[j], tj);
-        if (s > 1.0) atomicAdd(&s_errors, 1u);
-        s_val[s_start[op] + atomicAdd(&s_fill[op], 1u)] = s;
+};
+template <int A, int B, int N>
+__device__ __forceinline__ void compare_exchange(uint32_t (&v)[N]) {
+    const uint32_t x = v[A], y = v[B];
+    v[A] = min(x, y);
+    v[B] = max(x, y);
+}
+template <int N, int... I>
+__device__ __forceinline__ void sort_steps(uint32_t (&v)[N], std::integer_sequence<int, I...>) {
+    constexpr Network<N> net;
+    (compare_exchange<net.a[I], net.b[I]>(v), ...);
+}
+template <int N>
+__device__ __forceinline__ void sort_network(uint32_t (&v)[N]) {
+    constexpr Network<N> net;
+    sort_steps(v, std::make_integer_sequence<int, net.n>());
+}
+
+// One lane's operator: N keys at col[0], col[32], ..., the unused ones absent (sorted in place).  Returns the number of usable units; the slots of the lower and upper middle in `low` and `up`; `search`
+// where the keys cannot decide.
+template <int N>
+__device__ __forceinline__ uint32_t middle_slots(uint32_t* col, uint32_t& low, uint32_t& up, bool& search) {
+    uint32_t v[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) v[i] = (col[32 * i] & ~K_SLOT) | (uint32_t)i;
+    sort_network<N>(v);
+#pragma unroll
+    for (int i = 0; i < N; ++i) col[32 * i] = v[i];
+    // (an absent unit's key has a slot in its low bits too: absent means at or above K_ABSENT without them)
+    uint32_t m = 0;
+#pragma unroll
+    for (int step = 16; step; step >>= 1)
+        if (m + step <= N) m += col[32 * (m + step - 1)] < (K_ABSENT & ~K_SLOT) ? step : 0;
+    if (N == 32 && m == 31 && col[32 * 31] < (K_ABSENT & ~K_SLOT)) m = 32;
+    low = up = 0;
+    search = false;
+    if (m == 0) return 0;
+    const uint32_t kl = (m - 1) / 2, ku = m / 2;
+    const uint32_t vl = col[32 * kl], vu = col[32 * ku];
+    const uint32_t below = kl > 0 ? col[32 * (kl - 1)] : 0u, above = ku + 1 < m ? col[32 * (ku + 1)] : K_ABSENT;
+    search = col[32 * (m - 1)] >= K_UNKNOWN || (kl > 0 && vl - below <= NET_APART) || (kl != ku && vu - vl <= NET_APART) ||
+             above - vu <= NET_APART;
+    low = vl & K_SLOT;
+    up = vu & K_SLOT;
+    return m;
+}
+
+constexpr uint32_t WARP_ILP = 4;           // units per lane in flight
+__host__ __device__ __forceinline__ uint32_t padded_units(uint32_t n) { return (n + 32u * WARP_ILP - 1u) / (32u * WARP_ILP) * (32u * WARP_ILP); }
+
+struct WarpLayout {   // byte offsets; from `prod` on relative to the warp's own block (which starts with its keys)
+    uint32_t roof, place, group, chunk, unit_at, warps, prod, bins, warp_bytes;
+    __host__ __device__ WarpLayout(uint32_t n, uint32_t n_ops, uint32_t slots) {
+        uint32_t o = 0;
+        roof = o;    o += 4u * padded_units(n);            // f32 rooflines, NaN outside the safe range
+        group = o;   o += 8u * n_ops;                      // {first list entry (large groups), size | large << 31}
+        chunk = o;   o += 4u * ((n_ops + 31u) / 32u + 1u); // first slot of each chunk of 32 operators
+        place = o;   o += 2u * padded_units(n);            // slot of each unit, NO_GROUP flag
+        unit_at = o; o += 2u * (slots + n);                // unit of each slot; behind the columns, the large groups' units
+        warps = (o + 15u) & ~15u;
+        o = 4u * (slots + n + 1u);
+        bins = o = (o + 15u) & ~15u;  o += 4u * SELECT_BINS;
+        prod = o;    o += 8u * n_ops;
+        warp_bytes = (o + 15u) & ~15u;
     }
-    __syncthreads();
-    // Eq. 5: one warp per operator, median by ranking
+};
+// Columns come in the lengths of the networks.
+__host__ __device__ __forceinline__ uint32_t column_length(uint32_t g) { return g <= 8 ? 8u : (g <= 16 ? 16u : (g + 3u) & ~3u); }
+// Slots to provide: the group sizes are in device memory, so every chunk of operators gets room for groups
+// three standard deviations above the mean (units falling to operators at random); what does not fit is
+// treated as a large group.
+inline uint32_t warp_slots(uint32_t n, uint32_t n_ops) {
+    const double mean = (double)n / n_ops;
+    double width = std::ceil(mean + 3.0 * std::sqrt(mean)) + 2.0;
+    if (mean > NET_MAX) width = 8;         // (hardly any group is small enough)
+    if (width > NET_MAX) width = NET_MAX;
+    return (n_ops + 31u) / 32u * 32u * column_length((uint32_t)width);
+}
+
+constexpr uint32_t NO_GROUP = 0x8000u;     // flag of a unit of an operator outside [0, n_ops)
+constexpr uint32_t SLOT_MASK = 0x7FFFu;    // (units without a group write to a slot behind all others)
+constexpr uint32_t WARP_KERNEL_THREADS = 256, WARP_KERNEL_CTAS = 3;   // per SM (80 registers a thread; four CTAs of 64 were 3 % slower)
+
+__global__ void __launch_bounds__(WARP_KERNEL_THREADS, WARP_KERNEL_CTAS)
+    score_warp_kernel(const double* __restrict__ roofline_s, const uint32_t* __restrict__ unit_op, uint32_t n_units,
+                      const double* __restrict__ t_cand, const uint8_t* __restrict__ correct, uint32_t n_cand,
+                      const double* __restrict__ w, uint32_t n_ops, uint32_t max_slots, double* s_agg, double* s_op_out, ull* errors_out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const WarpLayout L(n_units, n_ops, max_slots);
+    float* roof = reinterpret_cast<float*>(smem_raw + L.roof);
+    uint16_t* place = reinterpret_cast<uint16_t*>(smem_raw + L.place);
+    uint2* group = reinterpret_cast<uint2*>(smem_raw + L.group);
+    uint32_t* chunk = reinterpret_cast<uint32_t*>(smem_raw + L.chunk);
+    uint16_t* unit_at = reinterpret_cast<uint16_t*>(smem_raw + L.unit_at);
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u, n_warps = blockDim.x >> 5;
-    for (uint32_t op = warp; op < n_ops; op += n_warps) {
-        const uint32_t lo = s_start[op], m = s_start[op + 1] - lo;
-        if (m == 0) {
-            if (lane == 0) s_med[op] = 0.0;
-            continue;
-        }
-        const uint32_t want_hi = m / 2, want_lo = (m & 1u) ? m / 2 : m / 2 - 1;
-        double v_hi = 0.0, v_lo = 0.0;
-        if (m > SELECT_ABOVE) {
-            // a large group: the wanted order statistics by a bitwise search over order-preserving keys
-            // (64 counting passes over the group instead of m)
-            const double hi = select_kth(s_val + lo, m, want_hi, lane);
-            const double lw = (m & 1u) ? hi : select_kth(s_val + lo, m, want_lo, lane);
-            if (lane == 0) s_med[op] = (m & 1u) ? hi : __dmul_rn(__dadd_rn(lw, hi), 0.5);
-            continue;
-        }
-        for (uint32_t a = lane; a < m; a += 32) {
-            const double x = s_val[lo + a];
-            uint32_t rank = 0;
-            for (uint32_t b = 0; b < m; ++b) {
-                const double y = s_val[lo + b];
-                rank += (y < x || (y == x && b < a)) ? 1u : 0u;
+    unsigned char* mine = smem_raw + L.warps + warp * L.warp_bytes;
+    uint32_t* keys = reinterpret_cast<uint32_t*>(mine);
+    uint32_t* bins = reinterpret_cast<uint32_t*>(mine + L.bins);
+    double* prod = reinterpret_cast<double*>(mine + L.prod);
+
+    // where each unit goes: operators in chunks of 32, one lane's column each
+    uint32_t* size = reinterpret_cast<uint32_t*>(smem_raw + L.warps + L.prod);   // [n_ops], in the first warp's block for now
+    for (uint32_t j = threadIdx.x; j < padded_units(n_units); j += blockDim.x) {
+        roof[j] = approx_roofline(j < n_units ? roofline_s[j] : 0.0);
+        if (j >= n_units) place[j] = (uint16_t)((max_slots + n_units) | NO_GROUP);
+    }
+    count_groups(unit_op, n_units, n_ops, size);
+    if (threadIdx.x < 32) {
+        uint32_t slot = 0, large = 0;
+        for (uint32_t op0 = 0; op0 < n_ops; op0 += 32) {
+            const uint32_t op = op0 + lane, g = op < n_ops ? size[op] : 0u;
+            const bool is_large = g > NET_MAX || slot + 32 * column_length(g) > max_slots;
+            const uint32_t widest = __reduce_max_sync(FULL, is_large ? 0u : g);
+            uint32_t incl = is_large ? g : 0u;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t o = __shfl_up_sync(FULL, incl, d);
+                if (lane >= (uint32_t)d) incl += o;
             }
-            if (rank == want_hi) v_hi = x;
-            if (rank == want_lo) v_lo = x;
+            if (op < n_ops) {
+                group[op] = is_large ? make_uint2(max_slots + large + incl - g, g | 0x80000000u) : make_uint2(0u, g);
+                size[op] = 0;
+            }
+            if (lane == 0) chunk[op0 / 32] = slot;
+            slot += widest ? 32 * column_length(widest) : 0u;
+            large += __shfl_sync(FULL, incl, 31);
         }
-        // exactly one lane holds each of the two wanted values; the others contribute +0.0
-        for (int off = 16; off > 0; off >>= 1) {
-            v_hi += __shfl_xor_sync(0xFFFFFFFFu, v_hi, off);
-            v_lo += __shfl_xor_sync(0xFFFFFFFFu, v_lo, off);
-        }
-        if (lane == 0) s_med[op] = (m & 1u) ? v_hi : __dmul_rn(__dadd_rn(v_lo, v_hi), 0.5);
+        if (lane == 0) chunk[(n_ops + 31) / 32] = slot;
     }
     __syncthreads();
-    if (s_op_out)
-        for (uint32_t i = threadIdx.x; i < n_ops; i += blockDim.x) s_op_out[cand * n_ops + i] = s_med[i];
-    if (threadIdx.x == 0) {
-        double agg = 0.0;  // Eq. 6 in operator order
-        for (uint32_t i = 0; i < n_ops; ++i) agg = __dadd_rn(agg, __dmul_rn(w[i], s_med[i]));
-        s_agg[cand] = agg;
-        if (errors_out) errors_out[cand] = s_errors;
+    for (uint32_t j = threadIdx.x; j < n_units; j += blockDim.x) {
+        const uint32_t op = unit_op[j];
+        uint32_t to = (max_slots + n_units) | NO_GROUP;
+        if (op < n_ops) {
+            const uint2 g = group[op];
+            const uint32_t i = atomicAdd(&size[op], 1u);
+            if (g.y >> 31) {
+                to = g.x + i;
+            } else {
+                to = chunk[op / 32] + (op & 31u) + 32 * i;
+            }
+            unit_at[to] = (uint16_t)j;
+        }
+        place[j] = (uint16_t)to;
+    }
+    __syncthreads();   // (the sizes lie in the first warp's block)
+    for (uint32_t i = lane; i < chunk[(n_ops + 31) / 32]; i += 32) keys[i] = K_ABSENT;   // unused slots stay absent
+    __syncwarp();
+
+    for (uint32_t cand = blockIdx.x * n_warps + warp; cand < n_cand; cand += gridDim.x * n_warps) {
+        const double* t = t_cand + (size_t)cand * n_units;
+        const uint8_t* ok = correct + (size_t)cand * n_units;
+        if (cand + gridDim.x * n_warps < n_cand) {   // the warp's next candidate starts towards L2
+            const size_t ahead = (size_t)gridDim.x * n_warps * n_units;
+            for (uint32_t o = lane * 16u; o < n_units; o += 512u) asm volatile("prefetch.global.L2 [%0];" ::"l"(t + ahead + o));
+            for (uint32_t o = lane * 128u; o < n_units; o += 4096u) asm volatile("prefetch.global.L2 [%0];" ::"l"(ok + ahead + o));
+        }
+        uint32_t errors = 0;
+        for (uint32_t j0 = lane; j0 < n_units; j0 += 32 * WARP_ILP) {
+            double tj[WARP_ILP];
+            uint32_t okj[WARP_ILP];
+#pragma unroll
+            for (uint32_t u = 0; u < WARP_ILP; ++u) {
+                const uint32_t j = min(j0 + 32 * u, n_units - 1);
+                tj[u] = __ldg(t + j);
+                okj[u] = __ldg(ok + j);
+            }
+#pragma unroll
+            for (uint32_t u = 0; u < WARP_ILP; ++u) {
+                const uint32_t j = j0 + 32 * u, to = place[j];          // (padded with units that do not count)
+                const bool use = (okj[u] != 0) & ((to & NO_GROUP) == 0);
+                const uint32_t key = approx_key(roof[j], roofline_s + j, tj[u], use, errors);
+                keys[to & SLOT_MASK] = key;
+            }
+        }
+        __syncwarp();
+        for (uint32_t op0 = 0; op0 < n_ops; op0 += 32) {
+            const uint32_t op = op0 + lane;
+            const uint2 g = op < n_ops ? group[op] : make_uint2(0, 0);
+            const bool is_large = g.y >> 31;
+            const uint32_t first_slot = chunk[op0 / 32] + lane, length = (chunk[op0 / 32 + 1] - chunk[op0 / 32]) / 32;
+            uint32_t* col = keys + first_slot;
+            uint32_t low = 0, up = 0, m = 0;
+            bool search = false;
+            if (length == 8) m = middle_slots<8>(col, low, up, search);
+            else if (length == 16) m = middle_slots<16>(col, low, up, search);
+            else if (length == 20) m = middle_slots<20>(col, low, up, search);
+            else if (length == 24) m = middle_slots<24>(col, low, up, search);
+            else if (length == 28) m = middle_slots<28>(col, low, up, search);
+            else if (length == 32) m = middle_slots<32>(col, low, up, search);
+            double s = 0.0;
+            if (m != 0 && !search) {
+                const uint32_t ju = unit_at[first_slot + 32 * up], jl = unit_at[first_slot + 32 * low];
+                s = __ddiv_rn(__ldg(roofline_s + ju), __ldg(t + ju));
+                if (!(m & 1u)) s = __dmul_rn(__dadd_rn(__ddiv_rn(__ldg(roofline_s + jl), __ldg(t + jl)), s), 0.5);
+            }
+            for (uint32_t todo = __ballot_sync(FULL, search || is_large); todo; todo &= todo - 1) {
+                const uint32_t src = __ffs(todo) - 1;
+                const uint32_t first = __shfl_sync(FULL, is_large ? g.x : first_slot, src), packed = __shfl_sync(FULL, g.y, src);
+                const uint32_t n = packed & 0x7FFFFFFFu, stride = packed >> 31 ? 1u : 32u;
+                auto key_at = [=](uint32_t a) {
+                    const uint32_t j = unit_at[first + a * stride];
+                    return exact_key(__ldg(roofline_s + j), __ldg(t + j), __ldg(ok + j) != 0);
+                };
+                uint32_t usable = 0;
+                ull k_lo, k_hi;
+                bool found = false;
+                if (stride == 1) {
+                    const Middle d = group_middle(keys + first, n, bins);
+                    usable = d.m;
+                    if (!d.unknown && usable != 0 && d.close <= 32) {
+                        // the exact scores of the units close to the middle, ranked
+                        ull* list = reinterpret_cast<ull*>(bins);
+                        uint32_t filled = 0;
+                        for (uint32_t a0 = 0; a0 < n; a0 += 32) {
+                            const bool in = a0 + lane < n && keys[first + a0 + lane] - d.from() <= d.span();
+                            const uint32_t votes = __ballot_sync(FULL, in);
+                            if (in) list[filled + __popc(votes & ((1u << lane) - 1u))] = key_at(a0 + lane);
+                            filled += __popc(votes);
+                        }
+                        __syncwarp();
+                        const ull x = lane < filled ? list[lane] : ~0ull;
+                        uint32_t less = 0, leq = 0;
+                        for (uint32_t i = 0; i < filled; ++i) {
+                            less += list[i] < x ? 1u : 0u;
+                            leq += list[i] <= x ? 1u : 0u;
+                        }
+                        const uint32_t kl = (usable - 1) / 2 - d.below, ku = usable / 2 - d.below;
+                        k_lo = __shfl_sync(FULL, x, __ffs(__ballot_sync(FULL, lane < filled && less <= kl && kl < leq)) - 1);
+                        k_hi = __shfl_sync(FULL, x, __ffs(__ballot_sync(FULL, lane < filled && less <= ku && ku < leq)) - 1);
+                        __syncwarp();
+                        found = true;
+                    }
+                }
+                if (!found) {
+                    usable = 0;
+                    for (uint32_t a = lane; a < n; a += 32) usable += key_at(a) != ~0ull ? 1u : 0u;
+                    usable = __reduce_add_sync(FULL, usable);
+                    if (usable == 0) continue;
+                    warp_select<ull>(key_at, n, (usable - 1) / 2, bins, &k_lo, &k_hi);
+                }
+                if (lane == src) s = median_of_keys(k_lo, (usable & 1u) ? k_lo : k_hi, usable & 1u);
+            }
+            if (op < n_ops) {
+                prod[op] = __dmul_rn(w[op], s);
+                if (s_op_out) s_op_out[(size_t)cand * n_ops + op] = s;
+            }
+        }
+        errors = __reduce_add_sync(FULL, errors);
+        __syncwarp();
+        if (lane == 0) {
+            double agg = 0.0;  // Eq. 6 in operator order
+#pragma unroll 4
+            for (uint32_t i = 0; i < n_ops; ++i) agg = __dadd_rn(agg, prod[i]);
+            s_agg[cand] = agg;
+            if (errors_out) errors_out[cand] = errors;
+        }
+        __syncwarp();
+    }
+}
+
+// The same for g <= N keys in a row that stay where they are; the middle keys come with their slots.
+template <int N>
+__device__ __forceinline__ uint32_t middle_keys(const uint32_t* keys, uint32_t g, uint32_t& vl, uint32_t& vu, bool& search) {
+    uint32_t v[N], m = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const uint32_t k = (uint32_t)i < g ? keys[i] : K_ABSENT;
+        m += k != K_ABSENT ? 1u : 0u;
+        v[i] = (k & ~K_SLOT) | (uint32_t)i;
+    }
+    sort_network<N>(v);
+    const int kl = ((int)m - 1) / 2, ku = (int)m / 2;
+    uint32_t below = 0, above = K_ABSENT, last = 0;
+    vl = vu = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        below = i == kl - 1 ? v[i] : below;
+        vl = i == kl ? v[i] : vl;
+        vu = i == ku ? v[i] : vu;
+        above = i == ku + 1 && i < (int)m ? v[i] : above;
+        last = i == (int)m - 1 ? v[i] : last;
+    }
+    search = m != 0 && (last >= K_UNKNOWN || (kl > 0 && vl - below <= NET_APART) || (kl != ku && vu - vl <= NET_APART) || above - vu <= NET_APART);
+    return m;
+}
+
+// ---- one candidate per CTA ------------------------------------------------------------------------
+// Bound by latency: the loads of Eq. 4, then the search rounds of the largest groups (one warp each).  Keys
+// of four bytes and positions of two let two or three CTAs share an SM at ten thousand units, so that one's
+// loads cover another's search: 1 000 candidates x 12 001 units x 7 operators in 142 us (with 64-bit exact
+// keys, one CTA per SM: 166 us).
+constexpr uint32_t MARK = 0x80000000u;        // top bit of a key: a middle unit of its operator, or close to one
+// flags beside an operator's count of usable units: the marked units' exact scores are ranked / all are searched
+constexpr uint32_t M_RANK = 0x40000000u, M_SEARCH = 0x80000000u, M_COUNT = 0x3FFFFFFFu;
+constexpr uint32_t POOL_MAX = 128;            // exact scores kept for such ranking, per candidate
+
+struct CtaLayout {
+    uint32_t mid, bins, start, upper, count, place, total;
+    __host__ __device__ CtaLayout(uint32_t n, uint32_t n_ops, uint32_t threads) {
+        uint32_t o = (4u * n + 15u) & ~15u;          // (keys first)
+        mid = o;    o += 16u * n_ops;                // exact scores of the lower and upper middle, then w * S in the first
+        bins = o;   o += threads / 32u * 4u * SELECT_BINS;
+        start = o;  o += 4u * (n_ops + 1u);
+        upper = o;  o += 4u * n_ops;                 // key of the upper middle, or units below the marked ones (at first: group sizes)
+        count = o;  o += 4u * n_ops;
+        place = o;  o += 2u * n;
+        total = o;
+    }
+};
+
+__global__ void __launch_bounds__(1024)
+    score_cta_kernel(const double* __restrict__ roofline_s, const uint32_t* __restrict__ unit_op, uint32_t n_units,
+                     const double* __restrict__ t_cand, const uint8_t* __restrict__ correct, uint32_t n_cand,
+                     const double* __restrict__ w, uint32_t n_ops, double* s_agg, double* s_op_out, ull* errors_out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ ull s_pool[POOL_MAX];
+    __shared__ uint16_t s_pool_op[POOL_MAX];
+    __shared__ uint32_t s_errors, s_pooled;
+    const CtaLayout L(n_units, n_ops, blockDim.x);
+    uint32_t* keys = reinterpret_cast<uint32_t*>(smem_raw);              // grouped by operator
+    double* mid = reinterpret_cast<double*>(smem_raw + L.mid);
+    uint32_t* start = reinterpret_cast<uint32_t*>(smem_raw + L.start);
+    uint32_t* upper = reinterpret_cast<uint32_t*>(smem_raw + L.upper);
+    uint32_t* count = reinterpret_cast<uint32_t*>(smem_raw + L.count);
+    uint16_t* place = reinterpret_cast<uint16_t*>(smem_raw + L.place);   // position, 0xFFFF = none (positions stay below 2^14)
+    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u, n_warps = blockDim.x >> 5;
+    uint32_t* bins = reinterpret_cast<uint32_t*>(smem_raw + L.bins) + warp * SELECT_BINS;
+    if (threadIdx.x == 0) s_errors = s_pooled = 0;
+    {   // where each unit goes: segments of the operators one behind the other
+        uint32_t* fill = upper;
+        count_groups(unit_op, n_units, n_ops, fill);
+        if (threadIdx.x < 32) {
+            uint32_t run = 0;
+            for (uint32_t i0 = 0; i0 < n_ops; i0 += 32) {
+                const uint32_t i = i0 + lane, c = i < n_ops ? fill[i] : 0u;
+                uint32_t incl = c;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint32_t o = __shfl_up_sync(FULL, incl, d);
+                    if (lane >= (uint32_t)d) incl += o;
+                }
+                if (i < n_ops) {
+                    start[i] = run + incl - c;
+                    fill[i] = 0;
+                }
+                run += __shfl_sync(FULL, incl, 31);
+            }
+            if (lane == 0) start[n_ops] = run;
+        }
+        __syncthreads();
+        for (uint32_t j = threadIdx.x; j < n_units; j += blockDim.x) {
+            const uint32_t op = unit_op[j];
+            place[j] = op < n_ops ? (uint16_t)(start[op] + atomicAdd(&fill[op], 1u)) : (uint16_t)0xFFFFu;
+        }
+        __syncthreads();
+    }
+
+    // One operator's middle keys are marked, with whatever comes close to them (one warp).
+    auto mark_middle = [&](uint32_t op) {
+        const uint32_t b = start[op], g = start[op + 1] - b;
+        const Middle d = group_middle(keys + b, g, bins);
+        uint32_t flag = 0;
+        if (d.unknown) {
+            flag = M_SEARCH;
+        } else if (d.m != 0) {
+            if (!d.clear()) flag = d.close <= 32 ? M_RANK : M_SEARCH;
+            for (uint32_t a = lane; a < g; a += 32) {
+                const uint32_t k = keys[b + a];
+                if (k - d.from() <= d.span()) keys[b + a] = k | MARK;
+            }
+        }
+        if (lane == 0) {
+            upper[op] = flag ? d.below : d.v_up;
+            count[op] = d.m | flag;
+        }
+    };
+    const bool lane_sorted = n_ops >= 4 * n_warps;   // (fewer operators: a warp for each is quicker than a lane for each)
+    for (uint32_t cand = blockIdx.x; cand < n_cand; cand += gridDim.x) {
+        const double* t = t_cand + (size_t)cand * n_units;
+        const uint8_t* ok = correct + (size_t)cand * n_units;
+        // 1. approximate keys
+        uint32_t errors = 0;
+        constexpr uint32_t U = 4;
+        for (uint32_t j0 = threadIdx.x; j0 < n_units; j0 += blockDim.x * U) {
+            double tj[U], rj[U];
+            uint32_t okj[U];
+#pragma unroll
+            for (uint32_t u = 0; u < U; ++u) {
+                const uint32_t j = min(j0 + blockDim.x * u, n_units - 1);
+                tj[u] = __ldg(t + j);
+                okj[u] = __ldg(ok + j);
+                rj[u] = __ldg(roofline_s + j);
+            }
+#pragma unroll
+            for (uint32_t u = 0; u < U; ++u) {
+                const uint32_t j = j0 + blockDim.x * u;
+                const uint32_t pos = j < n_units ? place[j] : 0xFFFFu;
+                if (pos != 0xFFFFu) keys[pos] = approx_key(approx_roofline(rj[u]), roofline_s + j, tj[u], okj[u] != 0, errors);
+            }
+        }
+        errors = __reduce_add_sync(FULL, errors);
+        if (lane == 0 && errors) atomicAdd(&s_errors, errors);
+        __syncthreads();
+        // 2. the middle keys of each operator are marked
+        //    Groups of up to 32: one lane each, 32 operators to a warp, where that keeps the warps busy
+        for (uint32_t op0 = warp * 32; lane_sorted && op0 < n_ops; op0 += n_warps * 32) {
+            const uint32_t op = op0 + lane, b = op < n_ops ? start[op] : 0u, g = op < n_ops ? start[op + 1] - b : 0u;
+            const bool small = g != 0 && g <= NET_MAX;
+            const uint32_t widest = __reduce_max_sync(FULL, small ? g : 0u);
+            uint32_t vl = 0, vu = 0, m = 0;
+            bool search = false;
+            if (widest == 0) {
+            } else if (widest <= 8) m = middle_keys<8>(keys + b, small ? g : 0u, vl, vu, search);
+            else if (widest <= 16) m = middle_keys<16>(keys + b, small ? g : 0u, vl, vu, search);
+            else if (widest <= 24) m = middle_keys<24>(keys + b, small ? g : 0u, vl, vu, search);
+            else m = middle_keys<32>(keys + b, small ? g : 0u, vl, vu, search);
+            if (op < n_ops && g <= NET_MAX && !search) {
+                if (m != 0) {
+                    upper[op] = keys[b + (vu & K_SLOT)];
+                    keys[b + (vu & K_SLOT)] |= MARK;
+                    if (!(m & 1u)) keys[b + (vl & K_SLOT)] |= MARK;
+                }
+                count[op] = m;
+            }
+            for (uint32_t todo = __ballot_sync(FULL, search); todo; todo &= todo - 1) mark_middle(__ffs(todo) - 1 + op0);
+        }
+        for (uint32_t op = warp; op < n_ops; op += n_warps)
+            if (!lane_sorted || start[op + 1] - start[op] > NET_MAX) mark_middle(op);
+        __syncthreads();
+        // 3. the marked units are divided exactly
+        for (uint32_t j = threadIdx.x; j < n_units; j += blockDim.x) {
+            const uint32_t pos = place[j];
+            if (pos == 0xFFFFu) continue;
+            const uint32_t k = keys[pos];
+            if ((k & MARK) == 0) continue;
+            const uint32_t op = __ldg(unit_op + j), m = count[op];
+            const double s = __ddiv_rn(__ldg(roofline_s + j), __ldg(t + j));
+            if (m & M_RANK) {
+                const uint32_t at = atomicAdd(&s_pooled, 1u);
+                if (at < POOL_MAX) {
+                    s_pool[at] = key_of_score(s);
+                    s_pool_op[at] = (uint16_t)op;
+                }
+            } else if (!(m & M_SEARCH)) {
+                mid[2 * op + ((k & ~MARK) == upper[op] ? 1 : 0)] = s;
+            }
+        }
+        __syncthreads();
+        // 4. Eq. 5, and the products of Eq. 6
+        for (uint32_t op0 = warp * 32; op0 < n_ops; op0 += n_warps * 32) {
+            const uint32_t op = op0 + lane;
+            const uint32_t m = op < n_ops ? count[op] : 0u;
+            double s = 0.0;
+            if (m != 0 && !(m & (M_RANK | M_SEARCH))) {
+                s = mid[2 * op + 1];
+                if (!(m & 1u)) s = __dmul_rn(__dadd_rn(mid[2 * op], s), 0.5);
+            }
+            for (uint32_t todo = __ballot_sync(FULL, m & (M_RANK | M_SEARCH)); todo; todo &= todo - 1) {
+                const uint32_t src = __ffs(todo) - 1, o = op0 + src, flags = count[o], usable = flags & M_COUNT, k = (usable - 1) / 2;
+                ull k_lo, k_hi;
+                if ((flags & M_RANK) && s_pooled <= POOL_MAX) {
+                    auto key_at = [=](uint32_t i) { return s_pool_op[i] == o ? s_pool[i] : ~0ull; };
+                    warp_select<ull>(key_at, s_pooled, k - upper[o], bins, &k_lo, &k_hi);
+                } else {
+                    auto key_at = [=](uint32_t j) {   // (rare: every unit is asked whether it is the operator's)
+                        return __ldg(unit_op + j) == o ? exact_key(__ldg(roofline_s + j), __ldg(t + j), __ldg(ok + j) != 0) : ~0ull;
+                    };
+                    warp_select<ull>(key_at, n_units, k, bins, &k_lo, &k_hi);
+                }
+                if (lane == src) s = median_of_keys(k_lo, (usable & 1u) ? k_lo : k_hi, usable & 1u);
+            }
+            __syncwarp();
+            if (op < n_ops) {
+                mid[2 * op] = __dmul_rn(w[op], s);
+                if (s_op_out) s_op_out[(size_t)cand * n_ops + op] = s;
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double agg = 0.0;  // Eq. 6 in operator order
+#pragma unroll 4
+            for (uint32_t i = 0; i < n_ops; ++i) agg = __dadd_rn(agg, mid[2 * i]);
+            s_agg[cand] = agg;
+            if (errors_out) errors_out[cand] = s_errors;
+            s_errors = s_pooled = 0;
+        }
+        __syncthreads();   // the keys, counts and s_errors are reused
     }
 }
 
 constexpr int SCORE_MAX_DEVICES = 64;
 std::mutex g_score_lock;
-bool g_score_prepared[SCORE_MAX_DEVICES];   // per device: the kernel's shared-memory limit has been raised
+int g_score_sms[SCORE_MAX_DEVICES];   // per device: its SM count, once the kernels' shared-memory limit has been raised there
+constexpr int SCORE_SMEM_MAX = 232448 - 1536;   // (the CTA kernel has 1.3 KB of its own beside the dynamic part)
+constexpr size_t SM_SMEM = 233472;              // shared memory of one SM; a CTA takes 1 KB beside its own
 
 struct ScoreDeviceGuard {
     int prev = -1;
@@ -172,7 +834,6 @@ extern "C" int atrex_score_aggregate(const double* d_roofline_s, const uint32_t*
     if (n_units == 0 || n_ops == 0) return ATREX_ERR_INVALID;
     if (n_units > ATREX_SCORE_MAX_UNITS || n_ops > ATREX_SCORE_MAX_OPS || n_candidates > 0x7FFFFFFFull)
         return ATREX_ERR_TOO_LARGE;
-    const size_t smem = (size_t)n_units * 8 + (size_t)n_ops * 8 + ((size_t)2 * n_ops + 1) * 4;
     // the inputs live on some device: run there, and raise that device's shared-memory limit once
     cudaPointerAttributes attr;
     if (cudaPointerGetAttributes(&attr, d_t_cand) != cudaSuccess || attr.type != cudaMemoryTypeDevice || attr.device < 0 ||
@@ -185,18 +846,42 @@ extern "C" int atrex_score_aggregate(const double* d_roofline_s, const uint32_t*
         cudaGetLastError();
         return ATREX_ERR_CUDA;
     }
+    int n_sms;
     {
         std::lock_guard<std::mutex> hold(g_score_lock);
-        if (!g_score_prepared[attr.device]) {
-            if (cudaFuncSetAttribute(score_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess) {
+        if (g_score_sms[attr.device] == 0) {
+            int v = 0;
+            if (cudaFuncSetAttribute(score_warp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SCORE_SMEM_MAX) != cudaSuccess ||
+                cudaFuncSetAttribute(score_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SCORE_SMEM_MAX) != cudaSuccess ||
+                cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, attr.device) != cudaSuccess) {
                 cudaGetLastError();
                 return ATREX_ERR_CUDA;
             }
-            g_score_prepared[attr.device] = true;
+            g_score_sms[attr.device] = v;
         }
+        n_sms = g_score_sms[attr.device];
     }
-    score_kernel<<<(unsigned)n_candidates, SCORE_THREADS, smem, (cudaStream_t)stream>>>(
-        d_roofline_s, d_unit_op, (uint32_t)n_units, d_t_cand, d_correct, d_w, n_ops, d_s_agg, d_s_op,
-        reinterpret_cast<ull*>(d_errors));
+    const uint32_t n = (uint32_t)n_units, b = (uint32_t)n_candidates;
+    ull* errors = reinterpret_cast<ull*>(d_errors);
+    // One candidate per warp pays once there are candidates enough for several warps on every SM, and as
+    // long as an SM's shared memory holds 16 warps' keys; otherwise a CTA works on each candidate.
+    const uint32_t slots = warp_slots(n, n_ops);
+    const WarpLayout wl(n, n_ops, slots);
+    const size_t warp_smem = wl.warps + (size_t)wl.warp_bytes * (WARP_KERNEL_THREADS / 32);
+    if (b >= (uint32_t)n_sms * 16u && slots + n < SLOT_MASK && warp_smem * 2 <= SM_SMEM - 2048) {
+        const uint32_t fit = (uint32_t)(SM_SMEM / (warp_smem + 1024)), per_sm = fit < WARP_KERNEL_CTAS ? fit : WARP_KERNEL_CTAS;
+        const uint32_t warps = WARP_KERNEL_THREADS / 32, want = (b + warps - 1) / warps, most = (uint32_t)n_sms * per_sm;
+        score_warp_kernel<<<want < most ? want : most, WARP_KERNEL_THREADS, warp_smem, (cudaStream_t)stream>>>(
+            d_roofline_s, d_unit_op, n, d_t_cand, d_correct, b, d_w, n_ops, slots, d_s_agg, d_s_op, errors);
+    } else {
+        const uint32_t threads = n <= 4096 ? 256u : (n <= 13000 ? 512u : 1024u);
+        const size_t smem = CtaLayout(n, n_ops, threads).total;
+        uint32_t per_sm = (uint32_t)(SM_SMEM / (smem + 2560));
+        if (per_sm > 1024u / threads) per_sm = 1024u / threads;   // (64 registers a thread)
+        if (per_sm < 1) per_sm = 1;
+        const uint32_t most = (uint32_t)n_sms * per_sm;
+        score_cta_kernel<<<b < most ? b : most, threads, smem, (cudaStream_t)stream>>>(
+            d_roofline_s, d_unit_op, n, d_t_cand, d_correct, b, d_w, n_ops, d_s_agg, d_s_op, errors);
+    }
     return cudaGetLastError() == cudaSuccess ? ATREX_OK : ATREX_ERR_CUDA;
 }

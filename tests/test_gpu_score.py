@@ -59,3 +59,30 @@ def test_score_limits():
     assert p.atrex_score_aggregate(None, z.data_ptr(), 4, z.data_ptr(), z.data_ptr(), 1, z.data_ptr(), 1, z.data_ptr(),
                                    None, None, None) == p.ATREX_ERR_INVALID
     assert p.atrex_score_aggregate(None, None, 4, None, None, 0, None, 1, None, None, None, None) == p.ATREX_OK
+
+
+# group sizes at the edges of the lane-sorted columns, the register searches and the shared-memory search
+EDGE_GROUPS = {"lanes": [1, 2, 7, 8, 9, 15, 16, 17, 20, 24, 25, 28, 31, 32, 0, 5], "mixed": [32, 33, 3, 64, 65, 1, 128, 129, 0, 40],
+               "wide": [255, 256, 257, 600, 31, 33], "many": [3, 0, 9, 1] * 40}
+
+
+@pytest.mark.parametrize("batch", [3, 2500])       # one candidate per CTA, one per warp
+@pytest.mark.parametrize("groups", sorted(EDGE_GROUPS))
+def test_score_parity_at_group_size_edges(groups, batch):
+    sizes = EDGE_GROUPS[groups]
+    n_ops, n_units = len(sizes), sum(sizes)
+    rng = np.random.default_rng(n_units + batch)
+    unit_op = rng.permutation(np.repeat(np.arange(n_ops), sizes)).astype(np.uint32)
+    roof = np.exp(rng.uniform(np.log(1e-6), np.log(1e-1), n_units))
+    t = roof[None, :] / rng.uniform(0.01, 1.02, (batch, n_units))
+    t[0::5] = roof / np.round(rng.uniform(0.1, 1.0, n_units), 1)          # ties
+    t[1::5] = roof / 0.5 * (1 + rng.integers(0, 4, (len(t[1::5]), n_units)) * 2.0 ** -50)   # scores a few units in the last place apart
+    t[2::5, : n_units // 2] *= 2.0 ** -100                                # far outside the usual range
+    ok = rng.random((batch, n_units)) < 0.8
+    t[3::5, ::9] = 0.0
+    w = rng.dirichlet(np.ones(n_ops))
+    exp = oracle.score_candidates(roof, unit_op, t, ok, w)
+    got = run_gpu(roof, unit_op, t, ok, w)
+    assert got[0].tobytes() == exp[0].tobytes()
+    assert got[1].tobytes() == exp[1].tobytes()
+    assert np.array_equal(got[2], exp[2])
