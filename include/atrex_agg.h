@@ -124,7 +124,8 @@ typedef struct {
     uint64_t total_hi[ATREX_MAX_PHASES];
     uint64_t keys_per_phase[ATREX_MAX_PHASES];
     uint64_t table_slots;                 /* capacity of the key table                 */
-    uint64_t hot_slots;                   /* keys currently in the shared-memory hot directory */
+    uint64_t hot_slots;                   /* keys in the shared-memory stage: the hot directory, or after small calls
+                                             only, the most that one thread block's table held */
     uint64_t n_spilled;                   /* records that went through the partition spill buffers */
     uint64_t n_overflow;                  /* records that found their spill buffer full (slow exact path) */
     uint64_t max_spill_fill;              /* fullest spill buffer seen since reset, in entries */

@@ -19,7 +19,7 @@ constexpr size_t STAGING_BYTES = 64ull << 20;          // per staging buffer (tw
 constexpr uint32_t LP_MIN = 8, LP_MAX = 12;             // 256 .. 4096 partitions
 constexpr ull MAX_KEYS = 1ull << 25;
 constexpr ull MAX_RECORDS_TOTAL = 1ull << 40;
-constexpr uint32_t HOT_MIN_RECORDS = 32768;             // smaller calls run without a directory
+constexpr size_t L2_TABLE_BYTES = 48ull << 20;           // a table up to this size stays in the 126 MB L2
 constexpr uint32_t HOT_SAMPLE = 1u << 20;
 constexpr uint32_t CAND_BITS = 17;                     // candidate table of the directory build
 constexpr size_t SKETCH_BYTES = (size_t)4 << 20;        // 2^20 counters (ingest.cu SKETCH_BITS)
@@ -432,8 +432,25 @@ static int drain_spill(atrex_agg* h, bool force, cudaStream_t s) {
 }
 
 static int ingest_launch(atrex_agg* h, const atrex_record_t* recs, uint64_t n, cudaStream_t s) {
-    // hot directory from a sample of the first sufficiently large call after create/reset
-    if (h->L.hot_slots && !h->hot_ready && n >= HOT_MIN_RECORDS) {
+    // Small calls go straight into the table (direct.cu).  The line lies where the two-pass route's fixed
+    // costs are made up for by its higher rate: at 2^20 records for tables that L2 holds beside everything
+    // else, at 2^18 for larger ones, whose global atomics wait for DRAM.  Without the shared-memory stage only the smallest.
+    const uint64_t direct_max = h->L.hot_slots == 0 ? DIRECT_RECORDS_MAX : (h->L.n_slots * 24 > L2_TABLE_BYTES ? 1ull << 18 : 1ull << 20);
+    if (n <= direct_max) {
+        DirectParams d;
+        memset(&d, 0, sizeof(d));
+        d.recs = (const uint4*)recs;
+        d.n = (uint32_t)n;
+        d.n_apps = h->cfg.n_apps;
+        d.phase_lim = h->cfg.n_phases << 16;
+        d.app_w = h->d_appw;
+        d.t = h->table_ref();
+        CU(h, launch_direct(d, h->n_sms, s));
+        h->launches++;
+        return ATREX_OK;
+    }
+    // hot directory from a sample of the first call after create/reset that takes the two-pass route
+    if (h->L.hot_slots && !h->hot_ready) {
         HotBuildParams b;
         b.recs = (const uint4*)recs;
         b.n_sample = (uint32_t)(n < HOT_SAMPLE ? n : HOT_SAMPLE);

@@ -164,6 +164,12 @@ __device__ __forceinline__ ull ld_relaxed(const ull* p) {
     return v;
 }
 
+// Chained launches (launch_chained in kernels.h): a kernel may be set up while its predecessor on the stream
+// is still running, and waits here before it touches memory; the predecessor says where its successor may
+// start to be set up.
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 struct TableRef {
     ull* keys;            // [P * C]
     ulonglong2* vals;     // [P * C] {lo, cnthi}

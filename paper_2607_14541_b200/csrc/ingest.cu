@@ -684,6 +684,7 @@ __global__ void __launch_bounds__(256) merge_kernel(const atrex_entry_t* in, ull
 
 cudaError_t ingest_prepare() {
     cudaError_t e = scatter_prepare();
+    if (e == cudaSuccess) e = direct_prepare();
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(partition_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448 - 2048);
     if (e != cudaSuccess) return e;

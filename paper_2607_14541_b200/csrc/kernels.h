@@ -53,6 +53,19 @@ struct IngestParams {
     ull seq;                   // sequence number of this launch
 };
 
+// Small calls (direct.cu): records straight into the table.
+constexpr uint32_t DIRECT_RECORDS_MAX = 8192;   // up to here a thread per record, beyond it a shared-memory table per CTA
+struct DirectParams {
+    const uint4* recs;
+    uint32_t n;
+    uint32_t n_apps;
+    uint32_t phase_lim;        // n_phases << 16
+    const uint32_t* app_w;
+    TableRef t;
+    uint32_t share;            // records per CTA
+    uint32_t slots;            // slots of a CTA's table
+};
+
 struct PartitionParams {
     TableRef t;
     const unsigned char* spill;
@@ -126,7 +139,26 @@ struct TopkAllParams {
     uint32_t sel_cap;
 };
 
+// Launches a kernel whose set-up may overlap its predecessor on the stream (the kernel starts with
+// grid_dependency_wait): between kernels of a few microseconds the gap is a third of their time.
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), uint32_t grid, uint32_t block, size_t smem, cudaStream_t stream, const A&... args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(block);
+    c.dynamicSmemBytes = smem;
+    c.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = attr;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+
 cudaError_t ingest_prepare();
+cudaError_t direct_prepare();
+cudaError_t launch_direct(DirectParams p, int n_sms, cudaStream_t stream);
 cudaError_t scatter_prepare();
 cudaError_t launch_scatter(const IngestParams& p, bool hot, int grid, cudaStream_t stream);
 cudaError_t launch_partition(const PartitionParams& p, int n_sms, cudaStream_t stream);
