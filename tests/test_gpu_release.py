@@ -222,3 +222,28 @@ def test_refresh_round_trip(lib):
     exp = o.finalize(PEAK_BW, PEAK_FLOPS)
     ent2, n2 = b.finalize(PEAK_BW, PEAK_FLOPS)
     assert host(lib.sort_entries_by_key(ent2, n2), lib.ENTRY_DTYPE).tobytes() == exp.tobytes()
+
+
+@pytest.mark.parametrize("n", [1, 2, 33, 4_095, 4_096, 4_097, 6_145, 40_000, 300_001])
+@pytest.mark.parametrize("shape", ["dense", "clustered", "equal weights"])
+def test_binned_sort_at_its_edges(lib, n, shape):
+    """Key order and ranking where one CTA's sort ends, where a bin outgrows a tile (clustered keys and
+    thousands of equal weights: the radix sort takes over), and where local bins crowd."""
+    rng = np.random.default_rng(n)
+    e = np.zeros(n, dtype=oracle.ENTRY_DTYPE)
+    key = np.arange(n, dtype=np.uint64)
+    if shape == "clustered":                                  # nearly all keys in a sliver of the range
+        key[n // 2:] += np.uint64(1 << 20)
+        key[-1] = np.uint64((7 << 48) | (0xFFFF << 32) | 0xFFFFFFFF)
+        e["wt_lo"] = np.where(np.arange(n) % 50 == 0, rng.integers(1, 1 << 62, n), (1 << 40) + np.arange(n) // 3)
+    elif shape == "equal weights":
+        e["wt_lo"] = 77
+    else:
+        key = (key % np.uint64(48) << np.uint64(32)) | (key // np.uint64(48))
+        e["wt_lo"], e["wt_hi"] = rng.integers(0, 1 << 63, n), rng.integers(0, 1 << 12, n) * (rng.random(n) < 0.2)
+    e["key"] = rng.permutation(key)
+    e["count"] = np.arange(n)
+    d = dev(e)
+    assert host(lib.sort_entries_by_key(d, n), oracle.ENTRY_DTYPE).tobytes() == oracle.sort_by_key(e).tobytes()
+    check_rank(lib, e, d, n, (0, 7), ppms=(0, 500_000, 1_000_000))
+    check_rank(lib, e, d, n, (0,), ppms=(900_000,), out_cap=n // 2)
