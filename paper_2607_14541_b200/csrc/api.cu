@@ -44,7 +44,7 @@ ull pow2_at_least(ull x) {
 }
 
 struct Layout {
-    size_t off_ctl, off_keys, off_vals, off_work, off_appw, off_hot, off_staging[2], off_sel, off_topk_out, off_hist_all,
+    size_t off_ctl, off_keys, off_vals, off_work, off_appw, off_hot, off_staging[2], off_sel, off_pick, off_topk_out, off_hist_all,
         off_spill_cnt, off_spill, off_hot_scratch, off_queue, off_hot_img, total;
     ull n_slots, work_slots;
     uint32_t lp, C;              // partitions = 1 << lp, slots per partition
@@ -107,7 +107,9 @@ void compute_layout(const atrex_agg_config_t* c, size_t smem_optin, int n_sms, L
     L->hot_slots = scatter_hot_slots(L->lp);   // what the scatter pass's shared memory holds for this partition count
     if (c->flags & ATREX_FLAG_NO_HOT_DIRECTORY) L->hot_slots = 0;
     size_t o = 0;
+    // (control block, spill counts and table are neighbours: a reset clears them in one piece)
     L->off_ctl = o;            o += round_up(sizeof(Control), ALIGN);
+    L->off_spill_cnt = o;      o += round_up(((size_t)L->n_groups << L->lp) * 4, ALIGN);
     L->off_keys = o;           o += round_up(L->n_slots * 8, ALIGN);
     L->off_vals = o;           o += round_up(L->n_slots * 16, ALIGN);
     L->off_work = o;           o += round_up(L->work_slots * sizeof(WorkSlot), ALIGN);
@@ -117,11 +119,11 @@ void compute_layout(const atrex_agg_config_t* c, size_t smem_optin, int n_sms, L
     L->off_staging[0] = o;     o += STAGING_BYTES;
     L->off_staging[1] = o;     o += STAGING_BYTES;
     L->off_sel = o;            o += round_up((size_t)SEL_CAP * 32 * c->n_phases, ALIGN);   // one region per phase
+    L->off_pick = o;           o += round_up((size_t)TOPK_PICK_MAX * 32 * c->n_phases, ALIGN);
     L->off_hist_all = o;       o += round_up((size_t)ATREX_MAX_PHASES * TOPK_BINS * 4, ALIGN);
     L->off_topk_out = o;       o += round_up((size_t)ATREX_MAX_TOPK * sizeof(atrex_entry_t), ALIGN);
     L->off_hot_scratch = o;    o += round_up(HOT_SCRATCH_BYTES, ALIGN);
     L->off_queue = o;          o += round_up((size_t)L->n_groups * L->queue_cap * 16, ALIGN);
-    L->off_spill_cnt = o;      o += round_up(((size_t)L->n_groups << L->lp) * 4, ALIGN);
     L->off_spill = o;          o += round_up(((size_t)L->n_groups << L->lp) * L->cap * SPILL_ENTRY_BYTES, ALIGN) + ALIGN;  // + prefetch overrun
     L->total = o;
 }
@@ -139,15 +141,16 @@ struct DeviceGuard {
 
 }  // namespace
 
-// What one ranking request worked out for every phase, kept until the next finalize: the
-// first-digit histograms (one pass over the table for all phases) and, for the last k asked for,
-// each phase's selection (one more pass for all phases).  A second phase's top-k of the same k then
-// costs no pass over the table at all.
+// What ranking requests worked out, kept until the next finalize: the first-digit counts and, for the last k
+// asked for, every phase's answer (in pinned memory).  A phase that could not be answered that way keeps the
+// selection of its last k.
 struct TopkCache {
-    ull hist_gen = 0;                       // finalize generation the histograms belong to (0 = none)
-    ull sel_gen = 0;                        // ... and the selections
-    uint32_t k = 0;                         // k the selections were made for
-    ull total[ATREX_MAX_PHASES] = {};       // candidates collected per phase
+    ull hist_gen = 0;                       // finalize generation the counts belong to (0 = none)
+    ull pick_gen = 0;                       // ... and the answers
+    uint32_t k = 0;                         // k of the answers
+    ull sel_gen[ATREX_MAX_PHASES] = {};     // the long way, per phase
+    uint32_t sel_k[ATREX_MAX_PHASES] = {};
+    ull total[ATREX_MAX_PHASES] = {};       // candidates selected
 };
 
 struct atrex_agg {
@@ -172,8 +175,10 @@ struct atrex_agg {
     ull* sel = nullptr;
     atrex_entry_t* topk_out = nullptr;
     Control* h_ctl = nullptr;  // pinned mirror
-    uint32_t* hist_all = nullptr;     // [ATREX_MAX_PHASES][TOPK_BINS] first-digit histograms of all phases
-    uint32_t* h_hist_all = nullptr;   // pinned mirror
+    uint32_t* hist_all = nullptr;     // [ATREX_MAX_PHASES][TOPK_BINS] first-digit counts of all phases
+    ull* pick = nullptr;              // [n_phases][TOPK_PICK_MAX][4] candidates
+    atrex_entry_t* h_top = nullptr;   // pinned: [n_phases][TOPK_PICK_K] the best k of each phase, then u32 [n_phases] how many
+    bool merged = false;              // entries were folded in since reset: their phases may be any
     TopkCache topk;
     ull fin_gen = 0;                  // bumped by every successful finalize
     bool hot_ready = false;
@@ -316,15 +321,15 @@ int atrex_agg_create(const atrex_agg_config_t* cfg, atrex_agg_t** out) {
         h->sel = (ull*)(h->ws + L.off_sel);
         h->topk_out = (atrex_entry_t*)(h->ws + L.off_topk_out);
         h->hist_all = (uint32_t*)(h->ws + L.off_hist_all);
+        h->pick = (ull*)(h->ws + L.off_pick);
         cudaError_t e = cudaSuccess;
-        if (e == cudaSuccess) e = cudaMemset(h->ws + L.off_ctl, 0, L.off_appw - L.off_ctl);  // control, table, work
+        if (e == cudaSuccess) e = cudaMemset(h->ws + L.off_ctl, 0, L.off_appw - L.off_ctl);  // control, spill counts, table, work
         if (e == cudaSuccess) e = cudaMemcpy(h->d_appw, cfg->app_weights, (size_t)cfg->n_apps * 4, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemset(h->hot_keys, 0, (size_t)(L.hot_slots ? L.hot_slots : 2) * 8);
         if (e == cudaSuccess) e = cudaMemset(h->hot_img, 0, (size_t)L.n_groups * (L.hot_slots ? L.hot_slots : 2) * 16);
-        if (e == cudaSuccess) e = cudaMemset(h->spill_cnt, 0, ((size_t)L.n_groups << L.lp) * 4);
-        if (e == cudaSuccess) e = cudaHostAlloc((void**)&h->h_ctl, sizeof(Control), cudaHostAllocDefault);
+        if (e == cudaSuccess) e = cudaHostAlloc((void**)&h->h_ctl, sizeof(Control), cudaHostAllocMapped);
         if (e == cudaSuccess)
-            e = cudaHostAlloc((void**)&h->h_hist_all, (size_t)ATREX_MAX_PHASES * TOPK_BINS * 4, cudaHostAllocDefault);
+            e = cudaHostAlloc((void**)&h->h_top, (size_t)cfg->n_phases * (TOPK_PICK_K * sizeof(atrex_entry_t) + 4), cudaHostAllocMapped);
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking);
         for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
             e = cudaEventCreateWithFlags(&h->ev_ready[i], cudaEventDisableTiming);
@@ -353,7 +358,7 @@ void atrex_agg_destroy(atrex_agg_t* h) {
     }
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
     if (h->h_ctl) cudaFreeHost(h->h_ctl);
-    if (h->h_hist_all) cudaFreeHost(h->h_hist_all);
+    if (h->h_top) cudaFreeHost(h->h_top);
     if (h->owns_workspace && h->ws) cudaFree(h->ws);
     delete h;
 }
@@ -363,14 +368,14 @@ int atrex_agg_reset(atrex_agg_t* h, void* stream) {
     if (!h) return ATREX_ERR_INVALID;
     DeviceGuard guard(h->cfg.device);
     cudaStream_t s = (cudaStream_t)stream;
-    CU(h, cudaMemsetAsync(h->ctl, 0, sizeof(Control), s));
-    CU(h, cudaMemsetAsync(h->keys, 0, h->L.off_work - h->L.off_keys, s));  // keys and vals
-    CU(h, cudaMemsetAsync(h->spill_cnt, 0, ((size_t)h->L.n_groups << h->L.lp) * 4, s));  // discard undrained entries
+    // control block, spill counts (undrained entries are discarded), keys and values
+    CU(h, cudaMemsetAsync(h->ctl, 0, h->L.off_work - h->L.off_ctl, s));
     if (h->hot_dirty) CU(h, cudaMemsetAsync(h->hot_img, 0, (size_t)h->L.n_groups * (h->L.hot_slots ? h->L.hot_slots : 2) * 16, s));
     h->hot_dirty = false;
     h->spill_pending = false;
     h->hot_ready = false;
     h->finalized = false;
+    h->merged = false;
     h->n_records = 0;
     return ATREX_OK;
 }
@@ -418,7 +423,6 @@ static int drain_spill(atrex_agg* h, bool force, cudaStream_t s) {
     q.queue_cap = h->L.queue_cap;
     q.force = force ? 1u : 0u;
     q.seq = h->scatter_seq;
-    CU(h, cudaMemsetAsync(&h->ctl->part_cursor, 0, sizeof(ull), s));
     CU(h, launch_partition(q, h->n_sms, s));
     h->launches++;
     if (force && h->hot_dirty) {
@@ -557,16 +561,25 @@ int atrex_agg_merge(atrex_agg_t* h, const atrex_entry_t* d_entries, uint64_t n, 
     if (!d_entries || ((uintptr_t)d_entries & 15u) != 0) return ATREX_ERR_INVALID;
     DeviceGuard guard(h->cfg.device);
     h->finalized = false;
+    h->merged = true;
     CU(h, launch_merge(d_entries, n, h->table_ref(), h->scan_grid(n, 256), (cudaStream_t)stream));
     h->launches++;
     return ATREX_OK;
 }
 
-static int run_totals(atrex_agg* h, cudaStream_t s) {
-    size_t off = offsetof(Control, total_lo);
-    CU(h, cudaMemsetAsync((unsigned char*)h->ctl + off, 0, offsetof(Control, hist) - off, s));
-    CU(h, launch_totals(h->table_ref(), h->L.n_slots, h->scan_grid(h->L.n_slots, 128 * 8), s));
+static int run_totals(atrex_agg* h, const uint64_t* total_lo, const uint64_t* total_hi, cudaStream_t s) {
+    GivenTotals given;
+    memset(&given, 0, sizeof(given));
+    if (total_lo) {
+        // normalise by the totals over all shards instead of this handle's own
+        memcpy(given.lo, total_lo, sizeof(given.lo));
+        memcpy(given.hi, total_hi, sizeof(given.hi));
+        given.use = 1;
+    }
+    const uint32_t n_phases = h->merged ? ATREX_MAX_PHASES : h->cfg.n_phases;
+    CU(h, launch_totals(h->table_ref(), h->L.n_slots, n_phases, given, h->hist_all, h->scan_grid(h->L.n_slots, 128 * 8), s));
     h->launches++;
+    h->topk.hist_gen = 0;   // (the counts were cleared)
     return ATREX_OK;
 }
 
@@ -575,6 +588,7 @@ static FinalizeParams finalize_params(const atrex_agg* h, atrex_entry_t* out, ui
     p.t = h->table_ref();
     p.n_slots = h->L.n_slots;
     p.ctl = h->ctl;
+    p.mirror = h->h_ctl;
     p.work = h->work_ref();
     p.peaks = h->peaks;
     p.out = out;
@@ -613,17 +627,10 @@ static int finalize_impl(atrex_agg_t* h, const atrex_hw_peaks_t* peaks, const ui
     h->peaks = *peaks;
     int rc = drain_spill(h, /*force=*/true, s);
     if (rc != ATREX_OK) return rc;
-    rc = run_totals(h, s);
+    rc = run_totals(h, total_lo, total_hi, s);
     if (rc != ATREX_OK) return rc;
-    if (total_lo) {
-        // normalise by the totals over all shards instead of this handle's own
-        CU(h, cudaMemcpyAsync(h->ctl->total_lo, total_lo, sizeof(ull) * ATREX_MAX_PHASES, cudaMemcpyHostToDevice, s));
-        CU(h, cudaMemcpyAsync(h->ctl->total_hi, total_hi, sizeof(ull) * ATREX_MAX_PHASES, cudaMemcpyHostToDevice, s));
-    }
-    CU(h, cudaMemsetAsync(&h->ctl->n_out, 0, sizeof(ull), s));
-    CU(h, launch_emit(finalize_params(h, d_out, out_cap), h->scan_grid(h->L.n_slots, 256 * 4), s));
+    CU(h, launch_emit(finalize_params(h, d_out, out_cap), h->scan_grid(h->L.n_slots, 256 * 4), s));   // (fills the mirror h_ctl)
     h->launches++;
-    CU(h, cudaMemcpyAsync(h->h_ctl, h->ctl, offsetof(Control, hist), cudaMemcpyDeviceToHost, s));
     CU(h, cudaStreamSynchronize(s));
     *n_out = h->h_ctl->n_out;
     rc = device_status_to_error(h->h_ctl);
@@ -635,16 +642,10 @@ static int finalize_impl(atrex_agg_t* h, const atrex_hw_peaks_t* peaks, const ui
 }
 
 // Radix-select plan of one phase for the best k: fixes leading digits of the ranking composite until
-// the class holding the k-th entry is small enough to sort.  The first digit comes from the cached
-// all-phase histograms; deeper digits (only when more than TOPK_CAND_CAP keys share the leading
-// digits) take one single-phase pass each.
+// the class holding the k-th entry is small enough to sort, one single-phase pass per digit.
 static int plan_phase(atrex_agg_t* h, uint32_t q, uint32_t k, TopkAllParams* all, ull* total, cudaStream_t s) {
     const ull n_phase = h->h_ctl->keys_per_phase[q];
     all->n_prefix_digits[q] = 0;
-    if (n_phase == 0) {
-        *total = 0;
-        return ATREX_OK;
-    }
     all->active_mask |= 1u << q;
     if (n_phase <= k) {
         all->collect_all_mask |= 1u << q;
@@ -653,19 +654,7 @@ static int plan_phase(atrex_agg_t* h, uint32_t q, uint32_t k, TopkAllParams* all
     }
     const uint32_t n_digits = (144 - all->shift[q] + 11) / 12;
     ull need = k, cand = 0;
-    const uint32_t* hist = h->h_hist_all + (size_t)q * TOPK_BINS;
     while (true) {
-        ull above = 0;
-        int bin = TOPK_BINS - 1;
-        for (; bin > 0; --bin) {
-            if (above + hist[bin] >= need) break;
-            above += hist[bin];
-        }
-        need -= above;
-        cand = hist[bin];
-        all->prefix_digit[q][all->n_prefix_digits[q]++] = (uint16_t)bin;
-        if (cand <= TOPK_CAND_CAP || all->n_prefix_digits[q] == n_digits) break;
-        // next digit of this phase alone
         TopkParams p;
         memset(&p, 0, sizeof(p));
         p.t = h->table_ref();
@@ -680,9 +669,48 @@ static int plan_phase(atrex_agg_t* h, uint32_t q, uint32_t k, TopkAllParams* all
         h->launches++;
         CU(h, cudaMemcpyAsync(h->h_ctl->hist, h->ctl->hist, sizeof(h->ctl->hist), cudaMemcpyDeviceToHost, s));
         CU(h, cudaStreamSynchronize(s));
-        hist = h->h_ctl->hist;
+        const uint32_t* hist = h->h_ctl->hist;
+        ull above = 0;
+        int bin = TOPK_BINS - 1;
+        for (; bin > 0; --bin) {
+            if (above + hist[bin] >= need) break;
+            above += hist[bin];
+        }
+        need -= above;
+        cand = hist[bin];
+        all->prefix_digit[q][all->n_prefix_digits[q]++] = (uint16_t)bin;
+        if (cand <= TOPK_CAND_CAP || all->n_prefix_digits[q] == n_digits) break;
     }
     *total = (k - need) + cand;
+    return ATREX_OK;
+}
+
+// One phase's candidates for the best k, sorted, in its selection region.
+static int select_phase(atrex_agg_t* h, uint32_t q, uint32_t k, cudaStream_t s) {
+    TopkCache& cache = h->topk;
+    if (cache.sel_gen[q] == h->fin_gen && cache.sel_k[q] == k) return ATREX_OK;
+    TopkAllParams all;
+    memset(&all, 0, sizeof(all));
+    all.t = h->table_ref();
+    all.n_slots = h->L.n_slots;
+    all.sel = h->sel;
+    all.sel_count = h->ctl->sel_count_all;
+    all.sel_cap = SEL_CAP;
+    // digits start at the highest bit the phase's total has (no key's weighted time exceeds it)
+    const ull hi = h->h_ctl->total_hi[q], lo = h->h_ctl->total_lo[q];
+    const int top_bit = hi ? 64 + (63 - __builtin_clzll(hi)) : (lo ? 63 - __builtin_clzll(lo) : 0);
+    all.shift[q] = (uint32_t)(143 - (top_bit + 56));
+    int rc = plan_phase(h, q, k, &all, &cache.total[q], s);
+    if (rc != ATREX_OK) return rc;
+    if (cache.total[q] > SEL_CAP) return ATREX_ERR_STATE;  // cannot happen: composites are unique
+    const uint32_t n_pow2 = (uint32_t)pow2_at_least(cache.total[q] < 2 ? 2 : cache.total[q]);
+    CU(h, cudaMemsetAsync(h->ctl->sel_count_all, 0, sizeof(h->ctl->sel_count_all), s));
+    CU(h, cudaMemsetAsync(h->sel + (size_t)q * SEL_CAP * 4, 0, (size_t)n_pow2 * 32, s));   // (the sort wants zeros behind the candidates)
+    CU(h, launch_topk_collect_all(all, h->scan_grid(h->L.n_slots, 256 * 4), s));
+    CU(h, launch_topk_sort(h->sel + (size_t)q * SEL_CAP * 4, n_pow2, s));
+    h->launches += 2;
+    cache.sel_gen[q] = h->fin_gen;
+    cache.sel_k[q] = k;
     return ATREX_OK;
 }
 
@@ -692,63 +720,39 @@ int atrex_agg_topk(atrex_agg_t* h, uint32_t phase, uint32_t k, atrex_entry_t* h_
     *n_out = 0;
     if (!h->finalized) return ATREX_ERR_STATE;
     if (k == 0) return ATREX_OK;
+    if (h->h_ctl->keys_per_phase[phase] == 0) return ATREX_OK;
     DeviceGuard guard(h->cfg.device);
     cudaStream_t s = (cudaStream_t)stream;
-    if (h->h_ctl->keys_per_phase[phase] == 0) return ATREX_OK;
-    const uint32_t n_phases = h->cfg.n_phases;
     TopkCache& cache = h->topk;
-
-    if (cache.sel_gen != h->fin_gen || cache.k != k) {
-        TopkAllParams all;
-        memset(&all, 0, sizeof(all));
-        all.t = h->table_ref();
-        all.n_slots = h->L.n_slots;
-        all.hist = h->hist_all;
-        all.sel = h->sel;
-        all.sel_count = h->ctl->sel_count_all;
-        all.sel_cap = SEL_CAP;
-        // digits start at the highest bit a phase's total has (no key's weighted time exceeds it)
-        for (uint32_t q = 0; q < n_phases; ++q) {
-            ull hi = h->h_ctl->total_hi[q], lo = h->h_ctl->total_lo[q];
-            int top_bit = hi ? 64 + (63 - __builtin_clzll(hi)) : (lo ? 63 - __builtin_clzll(lo) : 0);
-            all.shift[q] = (uint32_t)(143 - (top_bit + 56));
-        }
-        if (cache.hist_gen != h->fin_gen) {
-            // first digit of every non-empty phase: one pass over the table
-            for (uint32_t q = 0; q < n_phases; ++q)
-                if (h->h_ctl->keys_per_phase[q] != 0) all.active_mask |= 1u << q;
-            CU(h, cudaMemsetAsync(h->hist_all, 0, (size_t)ATREX_MAX_PHASES * TOPK_BINS * 4, s));
-            CU(h, launch_topk_hist_all(all, h->n_sms, s));
-            h->launches++;
-            CU(h, cudaMemcpyAsync(h->h_hist_all, h->hist_all, (size_t)ATREX_MAX_PHASES * TOPK_BINS * 4,
-                                  cudaMemcpyDeviceToHost, s));
+    if (k <= TOPK_PICK_K) {
+        // every phase's answer in one go
+        const volatile uint32_t* answered = (const uint32_t*)(h->h_top + (size_t)h->cfg.n_phases * TOPK_PICK_K);
+        if (cache.pick_gen != h->fin_gen || cache.k != k) {
+            PickParams p;
+            p.fin = finalize_params(h, nullptr, 0);
+            p.n_phases = h->cfg.n_phases;
+            p.k = k;
+            p.hist = h->hist_all;
+            p.sel = h->pick;
+            p.host_top = h->h_top;
+            p.host_n = (uint32_t*)answered;
+            const bool count = cache.hist_gen != h->fin_gen;
+            cache.pick_gen = 0;
+            CU(h, launch_topk_pick(p, count, h->n_sms, s));
+            h->launches += count ? 4 : 3;
             CU(h, cudaStreamSynchronize(s));
-            cache.hist_gen = h->fin_gen;
-            all.active_mask = 0;
+            cache.hist_gen = cache.pick_gen = h->fin_gen;
+            cache.k = k;
         }
-        for (uint32_t q = 0; q < n_phases; ++q) {
-            int rc = plan_phase(h, q, k, &all, &cache.total[q], s);
-            if (rc != ATREX_OK) return rc;
-            if (cache.total[q] > SEL_CAP) return ATREX_ERR_STATE;  // cannot happen: composites are unique
+        const uint32_t m = answered[phase];
+        if (m != PICK_NONE) {
+            memcpy(h_out, h->h_top + (size_t)phase * TOPK_PICK_K, (size_t)m * sizeof(atrex_entry_t));
+            *n_out = m;
+            return ATREX_OK;
         }
-        // every phase's candidates in one pass, each into its own zero-padded region
-        CU(h, cudaMemsetAsync(h->ctl->sel_count_all, 0, sizeof(h->ctl->sel_count_all), s));
-        for (uint32_t q = 0; q < n_phases; ++q) {
-            if (cache.total[q] == 0) continue;
-            const size_t n_pow2 = pow2_at_least(cache.total[q] < 2 ? 2 : cache.total[q]);
-            CU(h, cudaMemsetAsync(h->sel + (size_t)q * SEL_CAP * 4, 0, n_pow2 * 32, s));
-        }
-        CU(h, launch_topk_collect_all(all, h->scan_grid(h->L.n_slots, 256 * 4), s));
-        h->launches++;
-        for (uint32_t q = 0; q < n_phases; ++q) {   // sorted once, read by this and later calls
-            if (cache.total[q] == 0) continue;
-            const uint32_t n_pow2 = (uint32_t)pow2_at_least(cache.total[q] < 2 ? 2 : cache.total[q]);
-            CU(h, launch_topk_sort(h->sel + (size_t)q * SEL_CAP * 4, n_pow2, s));
-            h->launches++;
-        }
-        cache.sel_gen = h->fin_gen;
-        cache.k = k;
     }
+    int rc = select_phase(h, phase, k, s);
+    if (rc != ATREX_OK) return rc;
     const ull total = cache.total[phase];
     const uint32_t m = (uint32_t)(total < k ? total : k);
     CU(h, launch_topk_emit(finalize_params(h, h->topk_out, m), h->sel + (size_t)phase * SEL_CAP * 4, m, s));
@@ -776,9 +780,9 @@ int atrex_agg_stats(atrex_agg_t* h, atrex_stats_t* out, void* stream) {
     cudaStream_t s = (cudaStream_t)stream;
     int rc = drain_spill(h, /*force=*/true, s);
     if (rc != ATREX_OK) return rc;
-    rc = run_totals(h, s);
+    rc = run_totals(h, nullptr, nullptr, s);
     if (rc != ATREX_OK) return rc;
-    CU(h, cudaMemcpyAsync(h->h_ctl, h->ctl, offsetof(Control, hist), cudaMemcpyDeviceToHost, s));
+    CU(h, cudaMemcpyAsync(h->h_ctl, h->ctl, offsetof(Control, acc_lo), cudaMemcpyDeviceToHost, s));
     CU(h, cudaStreamSynchronize(s));
     memset(out, 0, sizeof(*out));
     const Control* c = h->h_ctl;

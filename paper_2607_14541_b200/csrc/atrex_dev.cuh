@@ -51,13 +51,16 @@ constexpr ull ST_BOUNDS = 32;   // debug build: an index was outside its array
 constexpr int TOPK_BINS = 4096;       // 12-bit digits
 constexpr int TOPK_DIGITS = 12;       // 144-bit composite = 88-bit weighted time, 56-bit ~key
 constexpr uint32_t TOPK_CAND_CAP = 65536;
+constexpr uint32_t TOPK_PICK_MAX = 2048;     // candidates of a phase that one CTA ranks in shared memory
+constexpr uint32_t TOPK_PICK_K = 1024;       // ... and the largest k answered that way
+constexpr uint32_t PICK_NONE = 0xFFFFFFFFu;
 
 struct Control {
     ull status;
     ull n_rejected;
     ull n_dropped;
     ull n_out;                 // entries emitted by the last finalize
-    ull sel_count;             // top-k: selected candidates
+    ull pad0;
     ull hot_n;                 // keys in the hot directory
     ull work_status;           // ST_WORK_* bits of the last work-table load
     ull hot_skew;              // 1 if one key dominates the sample: combine equal lanes per warp
@@ -68,12 +71,16 @@ struct Control {
     ull n_drains;              // partition passes that actually ran
     ull dir_mult;              // multiplier of the hot directory's bucket hash chosen at build time
     ull part_cursor;           // partition pass: next partition to hand out (zeroed before each launch)
-    ull pad1[1];
+    ull part_done;             // partition pass: CTAs that are through (the last one rewinds part_cursor)
     ull total_lo[ATREX_MAX_PHASES];
     ull total_hi[ATREX_MAX_PHASES];
     ull keys_per_phase[ATREX_MAX_PHASES];
     ull count_per_phase[ATREX_MAX_PHASES];
+    // ---- up to here mirrored in pinned host memory by every finalize
+    ull acc_lo[ATREX_MAX_PHASES], acc_hi[ATREX_MAX_PHASES], acc_keys[ATREX_MAX_PHASES], acc_count[ATREX_MAX_PHASES];   // totals pass: sums so far
+    ull tot_done, emit_done;              // CTAs that are through; the last one moves the sums on / fills the mirror
     ull sel_count_all[ATREX_MAX_PHASES];  // top-k: candidates collected per phase
+    uint32_t pick_bin[ATREX_MAX_PHASES];  // top-k: first digit of the last bin that is collected, PICK_NONE = too many candidates
     uint32_t hist[TOPK_BINS];
 };
 

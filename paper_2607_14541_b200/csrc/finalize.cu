@@ -4,6 +4,8 @@
 // All floating-point results come from explicit round-to-nearest intrinsics on exact
 // integers, so they have one correct bit pattern: fl(fl(wt) / fl(T)) and
 // fmax(fl(F) / P, fl(M) / beta).
+#include <cstddef>
+
 #include "atrex_dev.cuh"
 #include "kernels.h"
 
@@ -33,19 +35,36 @@ __device__ __forceinline__ SlotView load_slot(const TableRef& t, ull i) {
 }
 
 // ---- per-phase totals -------------------------------------------------------------------
-// Each thread keeps private per-phase 128-bit sums in its own shared-memory column; columns
-// are added per CTA and folded into the control block with a carry-aware pair of atomics.
-__global__ void __launch_bounds__(TOT_THREADS) totals_kernel(TableRef tab, ull n_slots) {
+// Each thread keeps private per-phase 128-bit sums in its own shared-memory column; columns are added per
+// CTA and folded into accumulators in the control block with a carry-aware pair of atomics.  The last CTA
+// moves the accumulators to their place and clears them (and the emit kernel's output count), so that no
+// launch is spent on clearing; the top-k histogram is cleared on the way.
+__device__ __forceinline__ bool last_cta(ull* done) {
+    __shared__ bool s_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(done, 1ull) == gridDim.x - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    return s_last;
+}
+
+__global__ void __launch_bounds__(TOT_THREADS) totals_kernel(TableRef tab, ull n_slots, uint32_t n_phases, const __grid_constant__ GivenTotals given,
+                                                             uint32_t* hist) {
     Control* ctl = tab.ctl;
     __shared__ ull s_lo[ATREX_MAX_PHASES][TOT_THREADS];
     __shared__ ull s_hi[ATREX_MAX_PHASES][TOT_THREADS];
     __shared__ ull s_cnt[ATREX_MAX_PHASES][TOT_THREADS];
     __shared__ uint32_t s_nk[ATREX_MAX_PHASES][TOT_THREADS];
     const int t = threadIdx.x;
-#pragma unroll
-    for (int p = 0; p < ATREX_MAX_PHASES; ++p) {
+    for (uint32_t p = 0; p < n_phases; ++p) {
         s_lo[p][t] = 0; s_hi[p][t] = 0; s_cnt[p][t] = 0; s_nk[p][t] = 0;
     }
+    grid_dependency_wait();
+    for (uint32_t i = blockIdx.x * TOT_THREADS + t; i < n_phases * TOPK_BINS / 4; i += gridDim.x * TOT_THREADS)
+        reinterpret_cast<uint4*>(hist)[i] = make_uint4(0, 0, 0, 0);
     // four slots per thread in flight: all key loads first, then the values of the live ones
     constexpr int ILP = 4;
     const ull stride = (ull)gridDim.x * blockDim.x;
@@ -59,7 +78,8 @@ __global__ void __launch_bounds__(TOT_THREADS) totals_kernel(TableRef tab, ull n
 #pragma unroll
         for (int u = 0; u < ILP; ++u) {
             if (sk[u] == 0) continue;
-            const int p = (int)(~sk[u] >> 48) & (ATREX_MAX_PHASES - 1);
+            const uint32_t p = (uint32_t)(~sk[u] >> 48) & (ATREX_MAX_PHASES - 1);
+            if (p >= n_phases) continue;
             const ull o = s_lo[p][t], n = o + x[u].x;
             s_lo[p][t] = n;
             s_hi[p][t] += (x[u].y >> HI_SHIFT) + (n < o ? 1ull : 0ull);
@@ -67,23 +87,42 @@ __global__ void __launch_bounds__(TOT_THREADS) totals_kernel(TableRef tab, ull n
             s_nk[p][t] += 1;
         }
     }
+    grid_dependents_launch();
     __syncthreads();
-    if (t < ATREX_MAX_PHASES) {
+    const uint32_t lane = t & 31;
+    for (uint32_t p = t >> 5; p < n_phases; p += TOT_THREADS / 32) {   // a warp per phase
         ull lo = 0, hi = 0, cnt = 0, nk = 0;
-        for (int j = 0; j < TOT_THREADS; ++j) {
-            ull n = lo + s_lo[t][j];
-            hi += s_hi[t][j] + (n < lo ? 1ull : 0ull);
+        for (int j = lane; j < TOT_THREADS; j += 32) {
+            const ull n = lo + s_lo[p][j];
+            hi += s_hi[p][j] + (n < lo ? 1ull : 0ull);
             lo = n;
-            cnt += s_cnt[t][j];
-            nk += s_nk[t][j];
+            cnt += s_cnt[p][j];
+            nk += s_nk[p][j];
         }
-        if (nk != 0) {
-            ull old = atomicAdd(&ctl->total_lo[t], lo);
-            atomicAdd(&ctl->total_hi[t], hi + (old + lo < old ? 1ull : 0ull));
-            atomicAdd(&ctl->count_per_phase[t], cnt);
-            atomicAdd(&ctl->keys_per_phase[t], nk);
+#pragma unroll
+        for (int d = 16; d; d >>= 1) {
+            const ull olo = __shfl_xor_sync(0xFFFFFFFFu, lo, d), ohi = __shfl_xor_sync(0xFFFFFFFFu, hi, d), n = lo + olo;
+            hi += ohi + (n < lo ? 1ull : 0ull);
+            lo = n;
+            cnt += __shfl_xor_sync(0xFFFFFFFFu, cnt, d);
+            nk += __shfl_xor_sync(0xFFFFFFFFu, nk, d);
+        }
+        if (lane == 0 && nk != 0) {
+            const ull old = atomicAdd(&ctl->acc_lo[p], lo);
+            atomicAdd(&ctl->acc_hi[p], hi + (old + lo < old ? 1ull : 0ull));
+            atomicAdd(&ctl->acc_count[p], cnt);
+            atomicAdd(&ctl->acc_keys[p], nk);
         }
     }
+    if (!last_cta(&ctl->tot_done)) return;
+    if (t < ATREX_MAX_PHASES) {
+        ctl->total_lo[t] = given.use ? given.lo[t] : ld_relaxed(&ctl->acc_lo[t]);
+        ctl->total_hi[t] = given.use ? given.hi[t] : ld_relaxed(&ctl->acc_hi[t]);
+        ctl->keys_per_phase[t] = ld_relaxed(&ctl->acc_keys[t]);
+        ctl->count_per_phase[t] = ld_relaxed(&ctl->acc_count[t]);
+        ctl->acc_lo[t] = ctl->acc_hi[t] = ctl->acc_keys[t] = ctl->acc_count[t] = 0;
+    }
+    if (t == 0) ctl->tot_done = ctl->n_out = 0;
 }
 
 // ---- per-key results ----------------------------------------------------------------------
@@ -157,6 +196,7 @@ __global__ void __launch_bounds__(FIN_THREADS) emit_kernel(FinalizeParams p) {
     __shared__ bool zeroT[ATREX_MAX_PHASES];
     __shared__ ull q_key[EMIT_WARPS][32 * EMIT_ILP];
     __shared__ ulonglong2 q_val[EMIT_WARPS][32 * EMIT_ILP];
+    grid_dependency_wait();
     load_phase_totals(p.ctl, dT, zeroT);
     const unsigned lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
     const ull stride = (ull)gridDim.x * blockDim.x;
@@ -199,6 +239,12 @@ __global__ void __launch_bounds__(FIN_THREADS) emit_kernel(FinalizeParams p) {
         }
         __syncwarp();  // the queue is refilled in the next round
     }
+    grid_dependents_launch();
+    if (!last_cta(&p.ctl->emit_done)) return;
+    // the host's copy of the counters and totals, straight to pinned memory
+    constexpr uint32_t WORDS = offsetof(Control, acc_lo) / 8;
+    if (threadIdx.x < WORDS) reinterpret_cast<ull*>(p.mirror)[threadIdx.x] = ld_relaxed(reinterpret_cast<const ull*>(p.ctl) + threadIdx.x);
+    if (threadIdx.x == 0) p.ctl->emit_done = 0;
 }
 
 // ---- work table ---------------------------------------------------------------------------
@@ -236,7 +282,198 @@ __global__ void __launch_bounds__(256) work_insert_kernel(const atrex_work_t* ro
     }
 }
 
-// ---- top-k --------------------------------------------------------------------------------
+// ---- top-k, the usual way -----------------------------------------------------------------
+// All phases at once, without a word from the host in between: a first digit on a logarithmic scale (bit
+// length and the five bits below the leading one: 3 % steps) is counted per phase; one CTA per phase finds
+// the digit of its k-th key; the keys at or above it are collected; one CTA per phase ranks them exactly and
+// writes the best k to pinned host memory.  Weights that span orders of magnitude leave a few dozen
+// candidates beside the winners.  (Digits on a linear scale below the phase total's highest bit put every
+// key of a flat trace into the lowest one: 26 000 candidates in one CTA's global-memory sort took 4 ms.)
+__device__ __forceinline__ uint32_t topk_first_digit(ull lo, ull hi) {
+    if ((lo | hi) == 0) return 0;
+    const int e = hi ? 128 - __clzll((long long)hi) : 64 - __clzll((long long)lo);      // 1 .. 88
+    uint32_t m;
+    if (e > 69) m = (uint32_t)(hi >> (e - 70));
+    else if (e > 64) m = (uint32_t)((hi << (70 - e)) | (lo >> (e - 6)));
+    else m = (uint32_t)(e >= 6 ? lo >> (e - 6) : lo << (6 - e));
+    return ((uint32_t)e << 5) | (m & 31u);
+}
+static_assert((88 << 5) + 31 < TOPK_BINS, "first digits fit the histogram");
+
+constexpr int PICK_THREADS = 1024;
+
+// first-digit counts of every phase
+__global__ void __launch_bounds__(PICK_THREADS) topk_count_kernel(const __grid_constant__ PickParams p) {
+    extern __shared__ uint32_t s_hist[];  // [n_phases][TOPK_BINS]
+    for (uint32_t i = threadIdx.x; i < p.n_phases * TOPK_BINS; i += PICK_THREADS) s_hist[i] = 0;
+    __syncthreads();
+    grid_dependency_wait();
+    const TableRef& tab = p.fin.t;
+    constexpr int ILP = 4;
+    const ull stride = (ull)gridDim.x * PICK_THREADS, n_slots = p.fin.n_slots;
+    for (ull i0 = (ull)blockIdx.x * PICK_THREADS + threadIdx.x; i0 < n_slots; i0 += stride * ILP) {
+        ull sk[ILP];
+        ulonglong2 x[ILP];
+#pragma unroll
+        for (int u = 0; u < ILP; ++u) {
+            const ull i = i0 + u * stride;
+            sk[u] = i < n_slots ? tab.keys[i] : 0ull;
+            x[u] = i < n_slots ? tab.vals[i] : make_ulonglong2(0, 0);  // no wait for the keys
+        }
+#pragma unroll
+        for (int u = 0; u < ILP; ++u) {
+            const uint32_t q = (uint32_t)(~sk[u] >> 48) & (ATREX_MAX_PHASES - 1);
+            if (sk[u] != 0 && q < p.n_phases) atomicAdd(&s_hist[q * TOPK_BINS + topk_first_digit(x[u].x, x[u].y >> HI_SHIFT)], 1u);
+        }
+    }
+    grid_dependents_launch();
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < p.n_phases * TOPK_BINS; i += PICK_THREADS)
+        if (s_hist[i] != 0) atomicAdd(&p.hist[i], s_hist[i]);
+}
+
+// the digit of each phase's k-th key (one CTA per phase)
+__global__ void __launch_bounds__(PICK_THREADS) topk_plan_kernel(const __grid_constant__ PickParams p) {
+    __shared__ uint32_t s_warp[32];
+    grid_dependency_wait();
+    const uint32_t q = blockIdx.x, t = threadIdx.x, lane = t & 31u, w = t >> 5;
+    // thread t holds the four bins below TOPK_BINS - 4 t, highest first
+    const uint4 v = reinterpret_cast<const uint4*>(p.hist + (size_t)q * TOPK_BINS)[TOPK_BINS / 4 - 1 - t];
+    const uint32_t c[4] = {v.w, v.z, v.y, v.x};
+    const uint32_t own = c[0] + c[1] + c[2] + c[3];
+    uint32_t incl = own;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+        if (lane >= (uint32_t)d) incl += o;
+    }
+    if (lane == 31) s_warp[w] = incl;
+    __syncthreads();
+    if (w == 0) {
+        uint32_t s = s_warp[lane];
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, s, d);
+            if (lane >= (uint32_t)d) s += o;
+        }
+        s_warp[lane] = s;
+    }
+    __syncthreads();
+    const uint32_t all = s_warp[31];
+    uint32_t above = incl - own + (w ? s_warp[w - 1] : 0u);
+    if (t == 0) {
+        p.fin.ctl->sel_count_all[q] = 0;
+        if (all <= p.k) p.fin.ctl->pick_bin[q] = all <= TOPK_PICK_MAX ? 0u : PICK_NONE;
+    }
+    if (all > p.k && above < p.k) {
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u) {
+            if (above < p.k && above + c[u] >= p.k)
+                p.fin.ctl->pick_bin[q] = above + c[u] <= TOPK_PICK_MAX ? TOPK_BINS - 1 - (4 * t + u) : PICK_NONE;
+            above += c[u];
+        }
+    }
+}
+
+// the keys at or above that digit
+__global__ void __launch_bounds__(FIN_THREADS) topk_collect_kernel(const __grid_constant__ PickParams p) {
+    __shared__ uint32_t s_bin[ATREX_MAX_PHASES];
+    grid_dependency_wait();
+    if (threadIdx.x < ATREX_MAX_PHASES) s_bin[threadIdx.x] = threadIdx.x < p.n_phases ? p.fin.ctl->pick_bin[threadIdx.x] : PICK_NONE;
+    __syncthreads();
+    const TableRef& tab = p.fin.t;
+    constexpr int ILP = 4;
+    const ull stride = (ull)gridDim.x * FIN_THREADS, n_slots = p.fin.n_slots;
+    for (ull i0 = (ull)blockIdx.x * FIN_THREADS + threadIdx.x; i0 < n_slots; i0 += stride * ILP) {
+        ull sk[ILP];
+        ulonglong2 x[ILP];
+#pragma unroll
+        for (int u = 0; u < ILP; ++u) {
+            const ull i = i0 + u * stride;
+            sk[u] = i < n_slots ? tab.keys[i] : 0ull;
+            x[u] = i < n_slots ? tab.vals[i] : make_ulonglong2(0, 0);
+        }
+#pragma unroll
+        for (int u = 0; u < ILP; ++u) {
+            if (sk[u] == 0) continue;
+            const uint32_t q = (uint32_t)(~sk[u] >> 48) & (ATREX_MAX_PHASES - 1);
+            const ull hi = x[u].y >> HI_SHIFT;
+            if (topk_first_digit(x[u].x, hi) < s_bin[q]) continue;      // (PICK_NONE: never)
+            const ull pos = atomicAdd(&p.fin.ctl->sel_count_all[q], 1ull);
+            if (pos < TOPK_PICK_MAX) {
+                ull* dst = p.sel + ((ull)q * TOPK_PICK_MAX + pos) * 4;
+                dst[0] = hi; dst[1] = x[u].x; dst[2] = ~sk[u]; dst[3] = i0 + u * stride;
+            }
+        }
+    }
+    grid_dependents_launch();
+}
+
+// the candidates of each phase ranked: weighted time descending, key ascending (one CTA per phase)
+__global__ void __launch_bounds__(512) topk_rank_kernel(const __grid_constant__ PickParams p) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    ull* s_hi = reinterpret_cast<ull*>(smem_raw);
+    ull* s_lo = s_hi + TOPK_PICK_MAX;
+    ull* s_key = s_lo + TOPK_PICK_MAX;
+    uint32_t* s_at = reinterpret_cast<uint32_t*>(s_key + TOPK_PICK_MAX);
+    __shared__ double dT[ATREX_MAX_PHASES];
+    __shared__ bool zeroT[ATREX_MAX_PHASES];
+    grid_dependency_wait();
+    const uint32_t q = blockIdx.x;
+    if (p.fin.ctl->pick_bin[q] == PICK_NONE) {
+        if (threadIdx.x == 0) p.host_n[q] = PICK_NONE;
+        return;
+    }
+    load_phase_totals(p.fin.ctl, dT, zeroT);
+    const uint32_t n = (uint32_t)p.fin.ctl->sel_count_all[q];      // <= TOPK_PICK_MAX by the plan
+    const ull* sel = p.sel + (size_t)q * TOPK_PICK_MAX * 4;
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
+        s_hi[i] = sel[4 * i];
+        s_lo[i] = sel[4 * i + 1];
+        s_key[i] = sel[4 * i + 2];
+        s_at[i] = (uint32_t)sel[4 * i + 3];
+    }
+    __syncthreads();
+    auto before = [&](uint32_t a, uint32_t b) {
+        if (s_hi[a] != s_hi[b]) return s_hi[a] > s_hi[b];
+        if (s_lo[a] != s_lo[b]) return s_lo[a] > s_lo[b];
+        return s_key[a] < s_key[b];
+    };
+    auto emit = [&](uint32_t row, uint32_t i) {
+        const SlotView v = load_slot(p.fin.t, s_at[i]);
+        store_entry(p.host_top + (size_t)q * TOPK_PICK_K + row, make_entry(v, dT, zeroT, p.fin));
+    };
+    if (n <= 512) {     // every candidate counts those before it
+        if (threadIdx.x < n) {
+            uint32_t row = 0;
+            for (uint32_t j = 0; j < n; ++j) row += before(j, threadIdx.x) ? 1u : 0u;
+            if (row < p.k) emit(row, threadIdx.x);
+        }
+    } else {
+        // bitonic network over positions 0 .. n - 1 (every comparator puts the better one first, so that
+        // positions beyond n can be left out)
+        for (uint32_t k = 2; k / 2 < n; k <<= 1) {
+            for (uint32_t j = k >> 1; j; j >>= 1) {
+                for (uint32_t t = threadIdx.x; t < n; t += blockDim.x) {
+                    const uint32_t lo = (t / j) * 2 * j + (t & (j - 1));
+                    const uint32_t hi = j == k >> 1 ? (lo | (k - 1)) - (lo & (k - 1)) : lo + j;
+                    if (hi < n && before(hi, lo)) {
+                        ull x = s_hi[lo]; s_hi[lo] = s_hi[hi]; s_hi[hi] = x;
+                        x = s_lo[lo]; s_lo[lo] = s_lo[hi]; s_lo[hi] = x;
+                        x = s_key[lo]; s_key[lo] = s_key[hi]; s_key[hi] = x;
+                        const uint32_t y = s_at[lo]; s_at[lo] = s_at[hi]; s_at[hi] = y;
+                    }
+                }
+                __syncthreads();
+            }
+        }
+        for (uint32_t i = threadIdx.x; i < min(n, p.k); i += blockDim.x) emit(i, i);
+    }
+    if (threadIdx.x == 0) p.host_n[q] = min(n, p.k);
+}
+
+// ---- top-k, the long way ------------------------------------------------------------------
+// For k above TOPK_PICK_K, and where more than TOPK_PICK_MAX keys share the first digit of the k-th.
 // Ranking composite, larger = better: bits 56..143 hold the 88-bit weighted time, bits 0..55
 // the complemented key (so the smaller key wins a tie).  Unique per key.  A most-significant-
 // digit radix select (12-bit digits) narrows the table down to the definite winners plus a
@@ -297,46 +534,6 @@ __device__ __forceinline__ int compare_prefix_of(const Composite& x, const TopkA
         if (a != b) return a > b ? 1 : -1;
     }
     return 0;
-}
-
-// Next-digit histograms of all active phases in one pass (shared memory: one row per phase).
-__global__ void __launch_bounds__(1024) topk_hist_all_kernel(const __grid_constant__ TopkAllParams p) {
-    extern __shared__ uint32_t h_all[];  // [ATREX_MAX_PHASES][TOPK_BINS], rows of inactive phases unused
-    for (uint32_t i = threadIdx.x; i < ATREX_MAX_PHASES * TOPK_BINS; i += blockDim.x)
-        if ((p.active_mask >> (i / TOPK_BINS)) & 1u) h_all[i] = 0;
-    __syncthreads();
-    constexpr int ILP = 4;
-    const ull stride = (ull)gridDim.x * blockDim.x;
-    for (ull i0 = (ull)blockIdx.x * blockDim.x + threadIdx.x; i0 < p.n_slots; i0 += stride * ILP) {
-        ull sk[ILP];
-        ulonglong2 x[ILP];
-#pragma unroll
-        for (int u = 0; u < ILP; ++u) sk[u] = i0 + u * stride < p.n_slots ? p.t.keys[i0 + u * stride] : 0ull;
-#pragma unroll
-        for (int u = 0; u < ILP; ++u) {
-            x[u] = i0 + u * stride < p.n_slots ? p.t.vals[i0 + u * stride] : make_ulonglong2(0, 0);  // no wait for the keys
-        }
-#pragma unroll
-        for (int u = 0; u < ILP; ++u) {
-            const uint32_t q = (uint32_t)(~sk[u] >> 48) & (ATREX_MAX_PHASES - 1);
-            if (!(sk[u] != 0 && ((p.active_mask >> q) & 1u))) sk[u] = 0;
-        }
-#pragma unroll
-        for (int u = 0; u < ILP; ++u) {
-            if (sk[u] == 0) continue;
-            SlotView v;
-            v.key = ~sk[u];
-            v.lo = x[u].x;
-            v.hi = x[u].y >> HI_SHIFT;
-            const uint32_t q = (uint32_t)(v.key >> 48) & (ATREX_MAX_PHASES - 1);
-            const Composite c = composite_of(v);
-            if (compare_prefix_of(c, p, q) != 0) continue;
-            atomicAdd(&h_all[q * TOPK_BINS + digit_of(c, (int)p.n_prefix_digits[q], (int)p.shift[q])], 1u);
-        }
-    }
-    __syncthreads();
-    for (uint32_t i = threadIdx.x; i < ATREX_MAX_PHASES * TOPK_BINS; i += blockDim.x)
-        if (((p.active_mask >> (i / TOPK_BINS)) & 1u) && h_all[i] != 0) atomicAdd(&p.hist[i], h_all[i]);
 }
 
 // Candidates of all active phases in one pass, each phase into its own selection region.
@@ -418,19 +615,22 @@ __global__ void __launch_bounds__(FIN_THREADS) topk_emit_kernel(FinalizeParams p
 }
 
 // ---- launchers ----------------------------------------------------------------------------
+constexpr size_t PICK_SMEM = (size_t)TOPK_PICK_MAX * 28;
+
 cudaError_t finalize_prepare() {
-    return cudaFuncSetAttribute(topk_hist_all_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(ATREX_MAX_PHASES * TOPK_BINS * sizeof(uint32_t)));
+    cudaError_t e = cudaFuncSetAttribute(topk_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(ATREX_MAX_PHASES * TOPK_BINS * sizeof(uint32_t)));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(topk_rank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PICK_SMEM);
+    return e;
 }
 
-cudaError_t launch_totals(const TableRef& t, ull n_slots, int grid, cudaStream_t stream) {
-    totals_kernel<<<grid, TOT_THREADS, 0, stream>>>(t, n_slots);
-    return cudaGetLastError();
+cudaError_t launch_totals(const TableRef& t, ull n_slots, uint32_t n_phases, const GivenTotals& given, uint32_t* hist, int grid,
+                          cudaStream_t stream) {
+    return launch_chained(totals_kernel, grid, TOT_THREADS, 0, stream, t, n_slots, n_phases, given, hist);
 }
 
 cudaError_t launch_emit(const FinalizeParams& p, int grid, cudaStream_t stream) {
-    emit_kernel<<<grid, FIN_THREADS, 0, stream>>>(p);
-    return cudaGetLastError();
+    return launch_chained(emit_kernel, grid, FIN_THREADS, 0, stream, p);
 }
 
 cudaError_t launch_work_insert(const atrex_work_t* rows, ull n, const WorkRef& w, Control* ctl, int grid,
@@ -439,10 +639,18 @@ cudaError_t launch_work_insert(const atrex_work_t* rows, ull n, const WorkRef& w
     return cudaGetLastError();
 }
 
-cudaError_t launch_topk_hist_all(const TopkAllParams& p, int n_sms, cudaStream_t stream) {
-    const size_t smem = (size_t)ATREX_MAX_PHASES * TOPK_BINS * sizeof(uint32_t);
-    topk_hist_all_kernel<<<n_sms, 1024, smem, stream>>>(p);
-    return cudaGetLastError();
+cudaError_t launch_topk_pick(const PickParams& p, bool count, int n_sms, cudaStream_t stream) {
+    const ull per_cta = PICK_THREADS * 4;
+    ull grid = (p.fin.n_slots + per_cta - 1) / per_cta;
+    if (grid > (ull)n_sms) grid = n_sms;
+    cudaError_t e = cudaSuccess;
+    if (count) e = launch_chained(topk_count_kernel, (uint32_t)grid, PICK_THREADS, p.n_phases * TOPK_BINS * sizeof(uint32_t), stream, p);
+    if (e == cudaSuccess) e = launch_chained(topk_plan_kernel, p.n_phases, PICK_THREADS, 0, stream, p);
+    ull wide = (p.fin.n_slots + FIN_THREADS * 4 - 1) / (FIN_THREADS * 4);
+    if (wide > (ull)n_sms * 8) wide = (ull)n_sms * 8;
+    if (e == cudaSuccess) e = launch_chained(topk_collect_kernel, (uint32_t)wide, FIN_THREADS, 0, stream, p);
+    if (e == cudaSuccess) e = launch_chained(topk_rank_kernel, p.n_phases, 512, PICK_SMEM, stream, p);
+    return e;
 }
 
 cudaError_t launch_topk_collect_all(const TopkAllParams& p, int grid, cudaStream_t stream) {

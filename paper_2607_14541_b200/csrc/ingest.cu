@@ -482,6 +482,11 @@ __global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(PartitionP
         for (uint32_t g = threadIdx.x; g < q.n_used; g += blockDim.x) q.spill_cnt[((ull)g << q.t.lp) + part] = 0;
         part = next;
     }
+    // the last CTA rewinds the hand-out counter for the next launch
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&q.t.ctl->part_done, 1ull) == gridDim.x - 1) q.t.ctl->part_cursor = q.t.ctl->part_done = 0;
+    }
 }
 
 // --------------------------------------------------------------------------------------

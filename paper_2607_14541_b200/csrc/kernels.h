@@ -104,10 +104,26 @@ struct FinalizeParams {
     TableRef t;
     ull n_slots;
     Control* ctl;
+    Control* mirror;     // pinned host memory, filled by the emit kernel
     WorkRef work;
     atrex_hw_peaks_t peaks;
     atrex_entry_t* out;
     ull out_cap;
+};
+
+struct GivenTotals {     // totals to normalise by instead of the table's own
+    ull lo[ATREX_MAX_PHASES], hi[ATREX_MAX_PHASES];
+    uint32_t use;
+};
+
+// Top-k of every phase at once (the usual way): see topk_first_digit in finalize.cu.
+struct PickParams {
+    FinalizeParams fin;
+    uint32_t n_phases, k;
+    uint32_t* hist;            // [n_phases][TOPK_BINS] first-digit counts
+    ull* sel;                  // [n_phases][TOPK_PICK_MAX][4]
+    atrex_entry_t* host_top;   // pinned: [n_phases][TOPK_PICK_K]
+    uint32_t* host_n;          // pinned: [n_phases] entries written, PICK_NONE = not answered this way
 };
 
 struct TopkParams {
@@ -133,7 +149,6 @@ struct TopkAllParams {
     uint32_t shift[ATREX_MAX_PHASES];
     uint32_t n_prefix_digits[ATREX_MAX_PHASES];
     uint16_t prefix_digit[ATREX_MAX_PHASES][12];
-    uint32_t* hist;                                    // [ATREX_MAX_PHASES][TOPK_BINS] next-digit counts
     ull* sel;                                          // [ATREX_MAX_PHASES][sel_cap][4]
     ull* sel_count;                                    // [ATREX_MAX_PHASES]
     uint32_t sel_cap;
@@ -168,11 +183,12 @@ cudaError_t launch_hot_fold(const ull* hot_keys, ulonglong2* hot_img, uint32_t n
 cudaError_t launch_merge(const atrex_entry_t* in, ull n, const TableRef& t, int grid, cudaStream_t stream);
 
 cudaError_t finalize_prepare();
-cudaError_t launch_totals(const TableRef& t, ull n_slots, int grid, cudaStream_t stream);
+cudaError_t launch_totals(const TableRef& t, ull n_slots, uint32_t n_phases, const GivenTotals& given, uint32_t* hist, int grid,
+                          cudaStream_t stream);
 cudaError_t launch_emit(const FinalizeParams& p, int grid, cudaStream_t stream);
 cudaError_t launch_work_insert(const atrex_work_t* rows, ull n, const WorkRef& w, Control* ctl, int grid,
                                cudaStream_t stream);
-cudaError_t launch_topk_hist_all(const TopkAllParams& p, int n_sms, cudaStream_t stream);
+cudaError_t launch_topk_pick(const PickParams& p, bool count, int n_sms, cudaStream_t stream);
 cudaError_t launch_topk_collect_all(const TopkAllParams& p, int grid, cudaStream_t stream);
 cudaError_t launch_topk_hist(const TopkParams& p, int grid, cudaStream_t stream);
 cudaError_t launch_topk_sort(ull* sel, uint32_t n_pow2, cudaStream_t stream);
