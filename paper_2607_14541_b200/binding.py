@@ -171,6 +171,13 @@ class AtrexError(RuntimeError):
         super().__init__(msg)
 
 
+def _raw_stream(torch, device: int) -> int:
+    """cudaStream_t of the device's current torch stream (the raw handle: building a Stream object for it takes
+    longer than a kernel launch)."""
+    get = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return get(device) if get is not None else torch.cuda.current_stream(device).cuda_stream
+
+
 def make_peaks(peak_bw: float, peak_flops) -> atrex_hw_peaks_t:
     pk = atrex_hw_peaks_t()
     pk.peak_bw = float(peak_bw)
@@ -196,7 +203,7 @@ class OperatorWeights:
         self._h = h
 
     def _stream(self, stream=None):
-        return self._torch.cuda.current_stream(self.device).cuda_stream if stream is None else stream.cuda_stream
+        return _raw_stream(self._torch, self.device) if stream is None else stream.cuda_stream
 
     def ingest(self, records, n: int | None = None, stream=None):
         if n is None:
@@ -237,7 +244,7 @@ def score_aggregate(roofline_s, unit_op, t_cand, correct, w, stream=None):
     s_agg = torch.empty(b, dtype=torch.float64, device=dev)
     s_op = torch.empty(b, n_ops, dtype=torch.float64, device=dev)
     err = torch.empty(b, dtype=torch.int64, device=dev)
-    s = torch.cuda.current_stream(dev).cuda_stream if stream is None else stream.cuda_stream
+    s = _raw_stream(torch, dev.index or 0) if stream is None else stream.cuda_stream
     rc = atrex_score_aggregate(roofline_s.data_ptr(), unit_op.data_ptr(), n, t_cand.data_ptr(), correct.data_ptr(), b,
                                w.data_ptr(), n_ops, s_agg.data_ptr(), s_op.data_ptr(), err.data_ptr(), s)
     if rc != ATREX_OK:
@@ -370,7 +377,7 @@ class Aggregator:
     # -- helpers
     def _stream(self, stream=None):
         if stream is None:
-            return self._torch.cuda.current_stream(self.device).cuda_stream
+            return _raw_stream(self._torch, self.device)
         return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
     def _check(self, rc, where):

@@ -204,6 +204,7 @@ struct atrex_agg {
         }
         return strides;
     }
+    ull key_strides = 0, work_strides = 0;   // worked out once by create
     TableRef table_ref() const {
         TableRef t;
         t.keys = keys;
@@ -211,7 +212,7 @@ struct atrex_agg {
         t.lp = L.lp;
         t.C = L.C;
         t.ctl = ctl;
-        t.strides = strides_for(L.C / 2);   // in slot pairs
+        t.strides = key_strides;
         return t;
     }
     WorkRef work_ref() const {
@@ -219,7 +220,7 @@ struct atrex_agg {
         w.table = L.work_slots ? work : nullptr;
         w.lp = L.lp;
         w.Cw = L.Cw;
-        w.strides = strides_for(L.Cw ? L.Cw : 1);
+        w.strides = work_strides;
         return w;
     }
     int scan_grid(ull n_items, int threads) const {
@@ -305,6 +306,8 @@ int atrex_agg_create(const atrex_agg_config_t* cfg, atrex_agg_t** out) {
             h->owns_workspace = true;
         }
         const Layout& L = h->L;
+        h->key_strides = atrex_agg::strides_for(L.C / 2);   // in slot pairs
+        h->work_strides = atrex_agg::strides_for(L.Cw ? L.Cw : 1);
         h->ctl = (Control*)(h->ws + L.off_ctl);
         h->keys = (ull*)(h->ws + L.off_keys);
         h->vals = (ulonglong2*)(h->ws + L.off_vals);
@@ -562,7 +565,7 @@ int atrex_agg_merge(atrex_agg_t* h, const atrex_entry_t* d_entries, uint64_t n, 
     DeviceGuard guard(h->cfg.device);
     h->finalized = false;
     h->merged = true;
-    CU(h, launch_merge(d_entries, n, h->table_ref(), h->scan_grid(n, 256), (cudaStream_t)stream));
+    CU(h, launch_merge(d_entries, n, h->table_ref(), (cudaStream_t)stream));
     h->launches++;
     return ATREX_OK;
 }
@@ -577,7 +580,7 @@ static int run_totals(atrex_agg* h, const uint64_t* total_lo, const uint64_t* to
         given.use = 1;
     }
     const uint32_t n_phases = h->merged ? ATREX_MAX_PHASES : h->cfg.n_phases;
-    CU(h, launch_totals(h->table_ref(), h->L.n_slots, n_phases, given, h->hist_all, h->scan_grid(h->L.n_slots, 128 * 8), s));
+    CU(h, launch_totals(h->table_ref(), h->L.n_slots, n_phases, given, h->hist_all, h->n_sms, s));
     h->launches++;
     h->topk.hist_gen = 0;   // (the counts were cleared)
     return ATREX_OK;
@@ -629,7 +632,7 @@ static int finalize_impl(atrex_agg_t* h, const atrex_hw_peaks_t* peaks, const ui
     if (rc != ATREX_OK) return rc;
     rc = run_totals(h, total_lo, total_hi, s);
     if (rc != ATREX_OK) return rc;
-    CU(h, launch_emit(finalize_params(h, d_out, out_cap), h->scan_grid(h->L.n_slots, 256 * 4), s));   // (fills the mirror h_ctl)
+    CU(h, launch_emit(finalize_params(h, d_out, out_cap), h->n_sms, s));   // (fills the mirror h_ctl)
     h->launches++;
     CU(h, cudaStreamSynchronize(s));
     *n_out = h->h_ctl->n_out;

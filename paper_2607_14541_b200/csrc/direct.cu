@@ -70,12 +70,14 @@ __device__ __forceinline__ uint32_t combine_first(const Record& r, ull& lo, ull&
 }
 
 __global__ void __launch_bounds__(RECORDS_THREADS) direct_records_kernel(DirectParams p) {
-    grid_dependency_wait();
     const uint32_t i = blockIdx.x * RECORDS_THREADS + threadIdx.x;
     const bool present = i < p.n;
+    // (a prefetch into L2, where every write arrives, may come before the predecessor's writes are waited for)
+    if (present && (threadIdx.x & 7u) == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.recs + i));
+    grid_dependents_launch();   // (its successor does the same before it waits)
+    grid_dependency_wait();
     const uint4 v = present ? __ldcs(p.recs + i) : make_uint4(0, 0, 0, 0);
     const Record r = decode(p, v, present);
-    grid_dependents_launch();
     count_rejected(p, present && !r.valid);
     ull lo, hi;
     const uint32_t count = combine_first(r, lo, hi);

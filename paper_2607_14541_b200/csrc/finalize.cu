@@ -624,13 +624,15 @@ cudaError_t finalize_prepare() {
     return e;
 }
 
-cudaError_t launch_totals(const TableRef& t, ull n_slots, uint32_t n_phases, const GivenTotals& given, uint32_t* hist, int grid,
+cudaError_t launch_totals(const TableRef& t, ull n_slots, uint32_t n_phases, const GivenTotals& given, uint32_t* hist, int n_sms,
                           cudaStream_t stream) {
-    return launch_chained(totals_kernel, grid, TOT_THREADS, 0, stream, t, n_slots, n_phases, given, hist);
+    static const uint32_t per_sm = resident_ctas(totals_kernel, TOT_THREADS, 0);
+    return launch_chained(totals_kernel, grid_for_work(n_slots, TOT_THREADS * 8, n_sms, per_sm), TOT_THREADS, 0, stream, t, n_slots, n_phases, given, hist);
 }
 
-cudaError_t launch_emit(const FinalizeParams& p, int grid, cudaStream_t stream) {
-    return launch_chained(emit_kernel, grid, FIN_THREADS, 0, stream, p);
+cudaError_t launch_emit(const FinalizeParams& p, int n_sms, cudaStream_t stream) {
+    static const uint32_t per_sm = resident_ctas(emit_kernel, FIN_THREADS, 0);
+    return launch_chained(emit_kernel, grid_for_work(p.n_slots, FIN_THREADS * EMIT_ILP, n_sms, per_sm), FIN_THREADS, 0, stream, p);
 }
 
 cudaError_t launch_work_insert(const atrex_work_t* rows, ull n, const WorkRef& w, Control* ctl, int grid,
@@ -640,15 +642,11 @@ cudaError_t launch_work_insert(const atrex_work_t* rows, ull n, const WorkRef& w
 }
 
 cudaError_t launch_topk_pick(const PickParams& p, bool count, int n_sms, cudaStream_t stream) {
-    const ull per_cta = PICK_THREADS * 4;
-    ull grid = (p.fin.n_slots + per_cta - 1) / per_cta;
-    if (grid > (ull)n_sms) grid = n_sms;
+    static const uint32_t per_sm = resident_ctas(topk_collect_kernel, FIN_THREADS, 0);
     cudaError_t e = cudaSuccess;
-    if (count) e = launch_chained(topk_count_kernel, (uint32_t)grid, PICK_THREADS, p.n_phases * TOPK_BINS * sizeof(uint32_t), stream, p);
+    if (count) e = launch_chained(topk_count_kernel, grid_for_work(p.fin.n_slots, PICK_THREADS * 4, n_sms, 1), PICK_THREADS, p.n_phases * TOPK_BINS * sizeof(uint32_t), stream, p);
     if (e == cudaSuccess) e = launch_chained(topk_plan_kernel, p.n_phases, PICK_THREADS, 0, stream, p);
-    ull wide = (p.fin.n_slots + FIN_THREADS * 4 - 1) / (FIN_THREADS * 4);
-    if (wide > (ull)n_sms * 8) wide = (ull)n_sms * 8;
-    if (e == cudaSuccess) e = launch_chained(topk_collect_kernel, (uint32_t)wide, FIN_THREADS, 0, stream, p);
+    if (e == cudaSuccess) e = launch_chained(topk_collect_kernel, grid_for_work(p.fin.n_slots, FIN_THREADS * 4, n_sms, per_sm), FIN_THREADS, 0, stream, p);
     if (e == cudaSuccess) e = launch_chained(topk_rank_kernel, p.n_phases, 512, PICK_SMEM, stream, p);
     return e;
 }

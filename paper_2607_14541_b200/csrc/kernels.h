@@ -155,7 +155,10 @@ struct TopkAllParams {
 };
 
 // Launches a kernel whose set-up may overlap its predecessor on the stream (the kernel starts with
-// grid_dependency_wait): between kernels of a few microseconds the gap is a third of their time.
+// grid_dependency_wait): between kernels of a few microseconds the gap is a third of their time.  Only grids of
+// up to two CTAs per SM: the CTAs of a wide grid that fill up the SMs while the predecessor drains end up
+// unevenly spread (emit kernel over a 566 MB table: 1 120 us chained, 614 us not).
+constexpr uint32_t CHAIN_MAX_CTAS = 296;
 template <typename... P, typename... A>
 inline cudaError_t launch_chained(void (*kernel)(P...), uint32_t grid, uint32_t block, size_t smem, cudaStream_t stream, const A&... args) {
     cudaLaunchConfig_t c = {};
@@ -167,8 +170,21 @@ inline cudaError_t launch_chained(void (*kernel)(P...), uint32_t grid, uint32_t 
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     c.attrs = attr;
-    c.numAttrs = 1;
+    c.numAttrs = grid <= CHAIN_MAX_CTAS ? 1 : 0;
     return cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+
+// CTAs of a grid-stride kernel: as many as the SMs hold at once (a second, partly filled wave would cost as
+// much as a full one), fewer when there is less work.  `per_sm` comes from resident_ctas, asked once.
+template <typename K>
+inline uint32_t resident_ctas(K* kernel, int threads, size_t smem) {
+    int n = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, threads, smem) != cudaSuccess || n < 1) n = 1;
+    return (uint32_t)n;
+}
+inline uint32_t grid_for_work(ull items, ull items_per_cta, int n_sms, uint32_t per_sm) {
+    const ull want = (items + items_per_cta - 1) / items_per_cta, most = (ull)n_sms * per_sm;
+    return (uint32_t)(want < 1 ? 1 : (want < most ? want : most));
 }
 
 cudaError_t ingest_prepare();
@@ -180,12 +196,12 @@ cudaError_t launch_partition(const PartitionParams& p, int n_sms, cudaStream_t s
 cudaError_t launch_hot_build(const HotBuildParams& p, int n_sms, cudaStream_t stream);
 cudaError_t launch_hot_fold(const ull* hot_keys, ulonglong2* hot_img, uint32_t n_groups, uint32_t hot_slots,
                             const TableRef& t, cudaStream_t stream);
-cudaError_t launch_merge(const atrex_entry_t* in, ull n, const TableRef& t, int grid, cudaStream_t stream);
+cudaError_t launch_merge(const atrex_entry_t* in, ull n, const TableRef& t, cudaStream_t stream);
 
 cudaError_t finalize_prepare();
-cudaError_t launch_totals(const TableRef& t, ull n_slots, uint32_t n_phases, const GivenTotals& given, uint32_t* hist, int grid,
+cudaError_t launch_totals(const TableRef& t, ull n_slots, uint32_t n_phases, const GivenTotals& given, uint32_t* hist, int n_sms,
                           cudaStream_t stream);
-cudaError_t launch_emit(const FinalizeParams& p, int grid, cudaStream_t stream);
+cudaError_t launch_emit(const FinalizeParams& p, int n_sms, cudaStream_t stream);
 cudaError_t launch_work_insert(const atrex_work_t* rows, ull n, const WorkRef& w, Control* ctl, int grid,
                                cudaStream_t stream);
 cudaError_t launch_topk_pick(const PickParams& p, bool count, int n_sms, cudaStream_t stream);

@@ -428,7 +428,7 @@ constexpr uint32_t TILE_STEP = 2048;        // a tile is the bins that start in 
 constexpr uint32_t TILE_CAP = 6144;         // ... and has at most this many items
 constexpr uint32_t TILE_LOCAL_BINS = 4096, TILE_THREADS = 512;
 constexpr uint32_t TILE_CLASH_MAX = 24;     // larger local bins send the tile to the comparison network
-constexpr size_t TILE_SMEM = (size_t)TILE_CAP * 12 + TILE_LOCAL_BINS * 4;
+constexpr size_t TILE_SMEM = (size_t)TILE_CAP * 8 + TILE_LOCAL_BINS * 4;    // three CTAs per SM
 constexpr uint32_t SMALL_SORT_MAX = 4096;   // up to here one CTA does everything
 
 struct BinCtl {                  // at the start of the scratch, cleared by every call (with the bins behind it)
@@ -450,10 +450,9 @@ struct BinSort {                 // what the kernels share
     BinCtl* ctl;
     BinReport* report;
     const atrex_entry_t* entries;
-    ull* words;                  // [n] raw words (keys), then items' words in bin order at items_word
-    uint32_t* idx;               // [n] (ranking) entry of each word; null: the position itself
-    ull* items_word;
-    uint32_t* items_idx;
+    ull* words;                  // [n] raw words: keys (key order), words (ranking)
+    uint32_t* idx;               // [n] (ranking) entry of each word, later the entries' order
+    ull* items;                  // [n] in bin order: leading 32 bits of the word's place in the range, then the entry
     uint32_t* bins;              // [1 << bits] counts, then cursors
     uint32_t* tile_start;        // [tiles + 1]
     ull* tile_sum;               // [tiles][2]
@@ -487,16 +486,23 @@ struct KeyRadix {
     }
 };
 
+// The words' range cut into equal bins, and into 2^32 steps for the items (all of it, where it is no wider).
 struct BinRange {
-    ull low;
+    ull low, scale;
+    uint32_t last;
     int shift;
     __device__ __forceinline__ BinRange(const BinSort& b, const KeyRadix& r) {
         low = b.ranking ? ~b.ctl->max_nword : 0ull;
-        const ull high = b.ranking ? b.ctl->max_word : ((b.ctl->max_phase + 1) * r.ops * r.shapes - 1);
-        const int len = 64 - __clzll((long long)(high - low));
-        shift = len > (int)b.bits ? len - (int)b.bits : 0;
+        const ull span = b.ranking ? b.ctl->max_word - low : (b.ctl->max_phase + 1) * r.ops * r.shapes - 1;
+        const int len = 64 - __clzll((long long)span);
+        shift = len > 32 ? len - 32 : 0;
+        last = (1u << b.bits) - 1u;
+        // bin = floor(place * bins / (span + 1)) up to rounding, which keeps the order of the bins
+        const double s = ldexp((double)(1u << b.bits), 64) / ((double)span + 1.0);
+        scale = s >= 18446744073709549568.0 ? ~0ull : (ull)s;
     }
-    __device__ __forceinline__ uint32_t bin(ull word) const { return (uint32_t)((word - low) >> shift); }
+    __device__ __forceinline__ uint32_t bin(ull word) const { return min(last, (uint32_t)__umul64hi(word - low, scale)); }
+    __device__ __forceinline__ ull item(ull word, uint32_t entry) const { return ((word - low) >> shift) << 32 | entry; }
 };
 
 template <typename T>
@@ -657,8 +663,20 @@ __global__ void __launch_bounds__(1024) bin_scan_kernel(const BinSort b) {
     uint32_t c[1u << (BIN_BITS_MAX - 10)];
     uint32_t sum = 0, most = 0;
 #pragma unroll
+    for (uint32_t u = 0; u < 1u << (BIN_BITS_MAX - 10); u += 4) {
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (u < per && first + u < n_bins) {
+            if (per >= 4) {
+                v = *reinterpret_cast<const uint4*>(b.bins + first + u);
+            } else {
+                v.x = b.bins[first];
+                if (per == 2) v.y = b.bins[first + 1];
+            }
+        }
+        c[u] = v.x; c[u + 1] = v.y; c[u + 2] = v.z; c[u + 3] = v.w;
+    }
+#pragma unroll
     for (uint32_t u = 0; u < 1u << (BIN_BITS_MAX - 10); ++u) {
-        c[u] = u < per && first + u < n_bins ? b.bins[first + u] : 0u;
         sum += c[u];
         most = max(most, c[u]);
     }
@@ -732,43 +750,39 @@ __global__ void __launch_bounds__(BIN_THREADS) bin_scatter_kernel(const BinSort 
             if (i0 + u * BIN_THREADS >= end) continue;
             if (!b.ranking) w[u] = radix.word(w[u]);
             const uint32_t pos = atomicAdd(&s_bins[range.bin(w[u])], 1u);
-            b.items_word[pos] = w[u];
-            b.items_idx[pos] = idx[u];
+            b.items[pos] = range.item(w[u], idx[u]);
         }
     }
 }
 
-// Order of two items: by word; equal words by what the word leaves out.
-__device__ __forceinline__ bool item_less(const atrex_entry_t* entries, bool ranking, ull wa, uint32_t ia, ull wb, uint32_t ib) {
-    if (wa != wb) return wa < wb;
-    if (!ranking || ia == ib) return ia < ib;           // equal keys keep their input order
-    const atrex_entry_t *a = entries + ia, *c = entries + ib;
-    if (a->wt_hi != c->wt_hi) return a->wt_hi > c->wt_hi;
-    if (a->wt_lo != c->wt_lo) return a->wt_lo > c->wt_lo;
+// Order of two items: by their leading bits; equal ones by what those leave out.
+__device__ __forceinline__ bool item_less(const atrex_entry_t* entries, bool ranking, ull x, ull y) {
+    if ((x ^ y) >> 32) return x < y;
+    const atrex_entry_t *a = entries + (uint32_t)x, *c = entries + (uint32_t)y;
+    if (ranking) {
+        if (a->wt_hi != c->wt_hi) return a->wt_hi > c->wt_hi;
+        if (a->wt_lo != c->wt_lo) return a->wt_lo > c->wt_lo;
+    }
     if (a->key != c->key) return a->key < c->key;
-    return ia < ib;
+    return x < y;               // equal keys keep their input order
 }
 
-// Sorts n <= TILE_CAP items whose words lie in [low, high] into s_word / s_idx.  `load(i, word, idx)` gives item
-// i (twice).  Each item goes to one of 4 096 local bins of equal width -- less than one item per bin, so that
+// Sorts n <= TILE_CAP items whose leading bits lie in [low, high] into s_item.  `load(i)` gives item i (twice).  Each item goes to one of 4 096 local bins of equal width -- less than one item per bin, so that
 // a thread puts a bin in order by insertion; crowded local bins (words that cluster) send the whole tile
 // through a bitonic network instead, with absent items behind the last one.
 template <typename Load>
-__device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ranking, uint32_t n, ull low, ull high, Load load, ull* s_word,
-                                          uint32_t* s_idx, uint32_t* s_local) {
+__device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ranking, uint32_t n, uint32_t low, uint32_t high, Load load, ull* s_item,
+                                          uint32_t* s_local) {
     __shared__ uint32_t s_warp[32];
     __shared__ uint32_t s_crowded;
     const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
-    const int len = 64 - __clzll((long long)(high - low));
+    const int len = 32 - __clz((int)(high - low));
     const int shift = len > 12 ? len - 12 : 0;
     for (uint32_t i = threadIdx.x; i < TILE_LOCAL_BINS; i += blockDim.x) s_local[i] = 0;
     if (threadIdx.x == 0) s_crowded = 0;
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
-        ull word;
-        uint32_t idx;
-        load(i, word, idx);
-        if (atomicAdd(&s_local[(uint32_t)((word - low) >> shift)], 1u) >= TILE_CLASH_MAX) s_crowded = 1;
+        if (atomicAdd(&s_local[((uint32_t)(load(i) >> 32) - low) >> shift], 1u) >= TILE_CLASH_MAX) s_crowded = 1;
     }
     __syncthreads();
     // exclusive scan of the local bins: each thread a run of them
@@ -801,12 +815,8 @@ __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ran
     }
     __syncthreads();
     for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
-        ull word;
-        uint32_t idx;
-        load(i, word, idx);
-        const uint32_t pos = atomicAdd(&s_local[(uint32_t)((word - low) >> shift)], 1u);
-        s_word[pos] = word;
-        s_idx[pos] = idx;
+        const ull item = load(i);
+        s_item[atomicAdd(&s_local[((uint32_t)(item >> 32) - low) >> shift], 1u)] = item;
     }
     __syncthreads();
     if (!s_crowded) {
@@ -814,16 +824,13 @@ __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ran
         for (uint32_t d = threadIdx.x; d < TILE_LOCAL_BINS; d += blockDim.x) {
             const uint32_t b0 = d ? s_local[d - 1] : 0u, b1 = s_local[d];
             for (uint32_t i = b0 + 1; i < b1; ++i) {
-                const ull wi = s_word[i];
-                const uint32_t ii = s_idx[i];
+                const ull item = s_item[i];
                 uint32_t j = i;
-                while (j > b0 && item_less(entries, ranking, wi, ii, s_word[j - 1], s_idx[j - 1])) {
-                    s_word[j] = s_word[j - 1];
-                    s_idx[j] = s_idx[j - 1];
+                while (j > b0 && item_less(entries, ranking, item, s_item[j - 1])) {
+                    s_item[j] = s_item[j - 1];
                     --j;
                 }
-                s_word[j] = wi;
-                s_idx[j] = ii;
+                s_item[j] = item;
             }
         }
     } else {
@@ -836,13 +843,10 @@ __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ran
                 for (uint32_t t = threadIdx.x; t < pow2 / 2; t += blockDim.x) {
                     const uint32_t lo = (t / j) * 2 * j + (t & (j - 1));
                     const uint32_t hi = j == k >> 1 ? (lo | (k - 1)) - (lo & (k - 1)) : lo + j;
-                    if (hi < n && item_less(entries, ranking, s_word[hi], s_idx[hi], s_word[lo], s_idx[lo])) {
-                        const ull tw = s_word[lo];
-                        const uint32_t ti = s_idx[lo];
-                        s_word[lo] = s_word[hi];
-                        s_idx[lo] = s_idx[hi];
-                        s_word[hi] = tw;
-                        s_idx[hi] = ti;
+                    if (hi < n && item_less(entries, ranking, s_item[hi], s_item[lo])) {
+                        const ull x = s_item[lo];
+                        s_item[lo] = s_item[hi];
+                        s_item[hi] = x;
                     }
                 }
                 __syncthreads();
@@ -855,7 +859,7 @@ __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ran
 // Entries of the sorted items to out[first .. first + n), as far as out_cap: three lanes to an entry, so that
 // the stores are contiguous and an entry's read is three 16-byte pieces of one or two lines (8-byte pieces
 // where a caller's buffer is only 8-byte aligned).
-__device__ __forceinline__ void gather_tile(const atrex_entry_t* entries, const uint32_t* s_idx, uint32_t n, atrex_entry_t* out, uint32_t first,
+__device__ __forceinline__ void gather_tile(const atrex_entry_t* entries, const ull* s_item, uint32_t n, atrex_entry_t* out, uint32_t first,
                                             uint32_t out_cap) {
     const uint32_t rows = first < out_cap ? min(n, out_cap - first) : 0u;
     if ((((uintptr_t)entries | (uintptr_t)out) & 15u) == 0) {
@@ -866,7 +870,7 @@ __device__ __forceinline__ void gather_tile(const atrex_entry_t* entries, const 
 #pragma unroll
             for (uint32_t u = 0; u < 4; ++u) {
                 const uint32_t x = i + u * blockDim.x;
-                if (x < rows * 3) v[u] = __ldg(src + (size_t)s_idx[x / 3] * 3 + x % 3);
+                if (x < rows * 3) v[u] = __ldg(src + (size_t)(uint32_t)s_item[x / 3] * 3 + x % 3);
             }
 #pragma unroll
             for (uint32_t u = 0; u < 4; ++u)
@@ -875,17 +879,17 @@ __device__ __forceinline__ void gather_tile(const atrex_entry_t* entries, const 
     } else {
         const ull* src = reinterpret_cast<const ull*>(entries);
         ull* dst = reinterpret_cast<ull*>(out + first);
-        for (uint32_t i = threadIdx.x; i < rows * 6; i += blockDim.x) dst[i] = src[(size_t)s_idx[i / 6] * 6 + i % 6];
+        for (uint32_t i = threadIdx.x; i < rows * 6; i += blockDim.x) dst[i] = src[(size_t)(uint32_t)s_item[i / 6] * 6 + i % 6];
     }
 }
 
 // 5. a tile's items in order, their entries gathered; (ranking) the tile's weighted time, and the order itself
 __global__ void __launch_bounds__(TILE_THREADS) bin_tile_kernel(const BinSort b, atrex_entry_t* out, uint32_t out_cap) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    ull* s_word = reinterpret_cast<ull*>(smem_raw);
-    uint32_t* s_idx = reinterpret_cast<uint32_t*>(s_word + TILE_CAP);
-    uint32_t* s_local = s_idx + TILE_CAP;
-    __shared__ ull s_part[32], s_sum[2];
+    ull* s_item = reinterpret_cast<ull*>(smem_raw);
+    uint32_t* s_local = reinterpret_cast<uint32_t*>(s_item + TILE_CAP);
+    __shared__ ull s_sum[2];
+    __shared__ uint32_t s_range[2];
     grid_dependency_wait();
     if (b.ctl->overflow) return;
     const uint32_t first = b.tile_start[blockIdx.x], n = b.tile_start[blockIdx.x + 1] - first;
@@ -893,33 +897,32 @@ __global__ void __launch_bounds__(TILE_THREADS) bin_tile_kernel(const BinSort b,
         if (b.ranking && threadIdx.x < 2) b.tile_sum[2 * blockIdx.x + threadIdx.x] = 0;
         return;
     }
-    ull top = 0, ntop = 0;
+    uint32_t top = 0, ntop = 0;
     for (uint32_t i = threadIdx.x; i < n; i += TILE_THREADS) {
-        const ull w = b.items_word[first + i];
-        top = max_ull(top, w);
-        ntop = max_ull(ntop, ~w);
+        const uint32_t w = (uint32_t)(b.items[first + i] >> 32);
+        top = max(top, w);
+        ntop = max(ntop, ~w);
     }
-    top = block_reduce(top, max_ull, s_part);
-    ntop = block_reduce(ntop, max_ull, s_part);
-    if (threadIdx.x == 0) {
-        s_sum[0] = ~ntop;
-        s_sum[1] = top;
+    if (threadIdx.x == 0) s_range[0] = s_range[1] = 0;
+    __syncthreads();
+    top = __reduce_max_sync(FULL, top);
+    ntop = __reduce_max_sync(FULL, ntop);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&s_range[0], ntop);
+        atomicMax(&s_range[1], top);
     }
     __syncthreads();
-    const ull low = s_sum[0], high = s_sum[1];
-    sort_tile(b.entries, b.ranking, n, low, high, [&](uint32_t i, ull& word, uint32_t& idx) {
-        word = b.items_word[first + i];
-        idx = b.items_idx[first + i];
-    }, s_word, s_idx, s_local);
+    sort_tile(b.entries, b.ranking, n, ~s_range[0], s_range[1], [&](uint32_t i) { return b.items[first + i]; }, s_item, s_local);
     grid_dependents_launch();
     if (b.ranking) {
         if (threadIdx.x < 2) s_sum[threadIdx.x] = 0;
         __syncthreads();
         ull lo = 0, hi = 0;
         for (uint32_t i = threadIdx.x; i < n; i += TILE_THREADS) {
-            const atrex_entry_t* e = b.entries + s_idx[i];
+            const uint32_t at = (uint32_t)s_item[i];
+            const atrex_entry_t* e = b.entries + at;
             add128(lo, hi, e->wt_lo, e->wt_hi);
-            b.items_idx[first + i] = s_idx[i];
+            b.idx[first + i] = at;
         }
 #pragma unroll
         for (int d = 16; d; d >>= 1) {
@@ -930,15 +933,14 @@ __global__ void __launch_bounds__(TILE_THREADS) bin_tile_kernel(const BinSort b,
         __syncthreads();
         if (threadIdx.x < 2) b.tile_sum[2 * blockIdx.x + threadIdx.x] = s_sum[threadIdx.x];
     }
-    gather_tile(b.entries, s_idx, n, out, first, out_cap);
+    gather_tile(b.entries, s_item, n, out, first, out_cap);
 }
 
 // Key order of up to SMALL_SORT_MAX entries, all of it in one CTA.
 __global__ void __launch_bounds__(1024) small_sort_kernel(const atrex_entry_t* entries, uint32_t n, atrex_entry_t* out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    ull* s_word = reinterpret_cast<ull*>(smem_raw);
-    uint32_t* s_idx = reinterpret_cast<uint32_t*>(s_word + TILE_CAP);
-    uint32_t* s_local = s_idx + TILE_CAP;
+    ull* s_item = reinterpret_cast<ull*>(smem_raw);
+    uint32_t* s_local = reinterpret_cast<uint32_t*>(s_item + TILE_CAP);
     __shared__ ull s_part[32];
     __shared__ BinCtl s_ctl;
     ull key[SMALL_SORT_MAX / 1024];
@@ -965,15 +967,15 @@ __global__ void __launch_bounds__(1024) small_sort_kernel(const atrex_entry_t* e
     }
     __syncthreads();
     const KeyRadix radix(&s_ctl);
-    const ull high = (s_ctl.max_phase + 1) * radix.ops * radix.shapes - 1;
-    sort_tile(entries, false, n, 0ull, high, [&](uint32_t i, ull& word, uint32_t& idx) {
+    const ull span = (s_ctl.max_phase + 1) * radix.ops * radix.shapes - 1;
+    const int len = 64 - __clzll((long long)span), shift = len > 32 ? len - 32 : 0;
+    sort_tile(entries, false, n, 0u, (uint32_t)(span >> shift), [&](uint32_t i) {
         ull k = key[0];
 #pragma unroll
         for (uint32_t u = 1; u < SMALL_SORT_MAX / 1024; ++u) k = i / 1024 == u ? key[u] : k;
-        word = radix.word(k);
-        idx = i;
-    }, s_word, s_idx, s_local);
-    gather_tile(entries, s_idx, n, out, 0, n);
+        return radix.word(k) >> shift << 32 | i;
+    }, s_item, s_local);
+    gather_tile(entries, s_item, n, out, 0, n);
 }
 
 // 6. (ranking) exclusive scan of the tiles' weighted times, and the sum the coverage cut needs: the smallest
@@ -1036,7 +1038,7 @@ __global__ void __launch_bounds__(SCAN_BLOCK) bin_share_kernel(const BinSort b, 
         const uint32_t r = base + threadIdx.x;
         ull lo = 0, hi = 0;
         if (r < end) {
-            const atrex_entry_t* e = r < out_cap ? ranked + r : b.entries + b.items_idx[r];
+            const atrex_entry_t* e = r < out_cap ? ranked + r : b.entries + b.idx[r];
             lo = e->wt_lo;
             hi = e->wt_hi;
         }
@@ -1202,17 +1204,17 @@ BinSort carve_bins(void* base, const atrex_entry_t* entries, uint64_t n, bool ra
     b.entries = entries;
     b.n = (uint32_t)n;
     b.ranking = ranking;
-    b.bits = 4;                                    // about 256 items per bin, as far as the bins go
-    while (b.bits < BIN_BITS_MAX && (256ull << b.bits) < n) ++b.bits;
+    // about 256 items per bin, a thousand beyond 2^12 bins (more open ranges than that cost the scattered writes)
+    b.bits = 4;
+    while (b.bits < BIN_BITS_MAX && ((b.bits < 12 ? 256ull : 1024ull) << b.bits) < n) ++b.bits;
     p += sizeof(BinCtl);
     b.bins = (uint32_t*)p;       p += 4ull << b.bits;
     b.tile_sum = (ull*)p;        p += tiles * 16;
     b.tile_start = (uint32_t*)p; p += (tiles + 1) * 4;
     p = (unsigned char*)base + align256(p - (unsigned char*)base);
     b.words = (ull*)p;           p += align256(n * 8);
-    b.items_word = (ull*)p;      p += align256(n * 8);
-    b.idx = (uint32_t*)p;        p += align256(n * 4);
-    b.items_idx = (uint32_t*)p;
+    b.items = (ull*)p;           p += align256(n * 8);
+    b.idx = (uint32_t*)p;
     return b;
 }
 // (what it needs beyond the pairs is less than the radix sort's digit counts, as long as there are a few tiles)
