@@ -5,33 +5,49 @@
 //   Eq. 3  wtilde_i = sum_a p_a (1/|Phi_i|) sum_{phi in Phi_i} D[i][a][phi] / D_a[phi];
 //          w_i = wtilde_i / sum over retained j of wtilde_j
 //
-// The group-by runs over (operator, application, phase) cells, a space of at most a few million
-// cells that stays resident in L2.  With uniformly spread applications no subset of the cells is hot
-// and equal cells hardly ever meet inside a warp, so there is nothing to pre-aggregate: ingest is one
-// 64-bit reduction per record into L2, and what matters is that it does not return a value.  While
-// fewer than 2^32 records have been ingested no cell can overflow 64 bits (durations are below 2^32),
-// so the reduction is fire-and-forget; from then on every add returns the old value and wraps are
-// counted in a second limb.  The floating-point part sums in ascending phase, application and
-// operator order with every operation rounded once, which gives one bit pattern.
+// The group-by runs over (operator, application, phase) cells.  Two routes:
+//   local   the cells fit a CTA's shared memory and there are records enough: every CTA sums its share there
+//           and adds its cells to the global ones at the end (70 M records into 11 560 cells: 1 056 -> 197 us,
+//           most of it DRAM time; the few hot cells of a small trace no longer queue at L2)
+//   direct  one 64-bit reduction per record into L2.  (Binning the records by cell first, entries kept in L2, one
+//           CTA summing each bin in shared memory, was measured for 10^6 cells: 2.0 ms per 2^28 records against
+//           1.8 by reductions; the bin pass spends its time between barriers.)
+// While fewer than 2^32 records have been ingested no cell can overflow 64 bits (durations are below 2^32), so
+// reductions need not return a value; from then on every add does and wraps are counted in a second limb.
+// The floating-point part sums in ascending phase, application and operator order with every operation
+// rounded once, which gives one bit pattern.
 #include <cmath>
+#include <cstring>
 #include <new>
+#include <vector>
 
 #include "kernels.h"
 
 using namespace atrex;
 
+namespace {
+
+constexpr uint32_t FULL = 0xFFFFFFFFu;
+constexpr uint32_t LOCAL_CELLS_MAX = 28 * 1024; // 8 bytes each
+
+}  // namespace
+
 struct atrex_eq3 {
     uint32_t n_apps = 0, n_ops = 0, n_phases = 0;
     int device = 0, n_sms = 0;
-    uint32_t* d_appw = nullptr;   // [n_apps]
+    unsigned char* arena = nullptr;   // one allocation for everything below
     ull* d_lo = nullptr;          // [n_phases][n_ops][n_apps] low 64 bits of D
     ull* d_hi = nullptr;          //                           wraps of the low limb
-    ull* d_tot = nullptr;         // [n_phases][n_apps][2] D_a (lo, hi)
+    double* d_den = nullptr;      // [n_phases][n_apps] fl(D_a[phi])
+    double* d_pa = nullptr;       // [n_apps] card-hour fractions
     double* d_wt = nullptr;       // [n_ops] wtilde
-    double* d_w = nullptr;        // [n_ops] w
-    uint8_t* d_ret = nullptr;     // [n_ops] retained flags
-    ull* d_rejected = nullptr;
+    uint32_t* d_present = nullptr;   // [n_ops] bit phi: operator i has time in phase phi (cleared by every finalize)
+    ull* d_ctl = nullptr;         // [0] rejected, [1] finalize: operators done
+    size_t h_bytes = 0;
+    double* h_out = nullptr;      // pinned: w [n_ops], wtilde [n_ops], rejected; then the retained flags [n_ops]
     size_t cells = 0;
+    double c_total = 0.0;
+    bool hi_used = false;
     ull n_ingested = 0;           // records handed to ingest since create/reset (decides the carry handling)
 };
 
@@ -48,151 +64,251 @@ struct Guard {
     }
 };
 
+struct Eq3Params {
+    const uint4* recs;
+    ull n;
+    uint32_t n_apps, n_ops, n_phases, cells;
+    ull *lo, *hi, *rejected;
+};
+
 __device__ __forceinline__ void red_add_u64(ull* p, ull v) {
     asm volatile("red.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
-
-// One record's duration into its cell.  CARRY: the low limb may wrap, so the add returns the old value.
 template <bool CARRY>
-__device__ __forceinline__ uint32_t eq3_add(uint32_t app, uint32_t w1, uint32_t dur, uint32_t n_apps, uint32_t n_ops,
-                                            uint32_t n_phases, ull* lo, ull* hi) {
-    const uint32_t op = w1 & 0xFFFFu, phase = (w1 >> 16) & 0xFFu;
-    if (app >= n_apps || op >= n_ops || phase >= n_phases) return 1u;
-    const size_t cell = ((size_t)phase * n_ops + op) * n_apps + app;
+__device__ __forceinline__ void add_cell(const Eq3Params& p, uint32_t cell, ull v) {
     if (CARRY) {
-        const ull d = dur, old = atomicAdd(&lo[cell], d);
-        if (old + d < old) atomicAdd(&hi[cell], 1ull);
+        const ull old = atomicAdd(&p.lo[cell], v);
+        if (old + v < old) atomicAdd(&p.hi[cell], 1ull);
     } else {
-        red_add_u64(&lo[cell], (ull)dur);
+        red_add_u64(&p.lo[cell], v);
     }
-    return 0u;
+}
+__device__ __forceinline__ bool cell_of(const Eq3Params& p, const uint4& r, uint32_t& cell) {
+    const uint32_t op = r.y & 0xFFFFu, phase = (r.y >> 16) & 0xFFu;
+    cell = (phase * p.n_ops + op) * p.n_apps + r.x;
+    return r.x < p.n_apps && op < p.n_ops && phase < p.n_phases;
+}
+__device__ __forceinline__ void count_rejected(const Eq3Params& p, uint32_t bad) {
+    bad = __reduce_add_sync(FULL, bad);
+    if ((threadIdx.x & 31u) == 0 && bad) atomicAdd(p.rejected, (ull)bad);
 }
 
-// Two records per 32-byte load, two loads in flight per thread.
+// ---- direct: bound by the L2's reduction rate, ~150 G/s for random 8-byte targets
 template <bool CARRY>
-__global__ void __launch_bounds__(512) eq3_ingest_kernel(const unsigned char* __restrict__ body, ull n_pairs, const uint4* head,
-                                                         const uint4* tail, uint32_t n_apps, uint32_t n_ops, uint32_t n_phases,
-                                                         ull* lo, ull* hi, ull* rejected) {
+__global__ void __launch_bounds__(512) eq3_direct_kernel(const Eq3Params p) {
+    grid_dependency_wait();
+    uint32_t bad = 0;
+    const ull stride = (ull)gridDim.x * 512;
+    for (ull i0 = (ull)blockIdx.x * 512 + threadIdx.x; i0 < p.n; i0 += 4 * stride) {
+        uint4 r[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i0 + u * stride < p.n) r[u] = __ldcs(p.recs + i0 + u * stride);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (i0 + u * stride >= p.n) continue;
+            uint32_t cell;
+            if (cell_of(p, r[u], cell)) add_cell<CARRY>(p, cell, r[u].w);
+            else ++bad;
+        }
+    }
+    grid_dependents_launch();
+    count_rejected(p, bad);
+}
+
+// ---- local: {u32 low, u32 wraps} per cell in shared memory; bound by the records' DRAM reads
+__device__ __forceinline__ void smem_add(uint32_t* lo, uint32_t* hi, uint32_t at, uint32_t v) {
+    const uint32_t o = atomicAdd(lo + at, v);
+    if (o + v < o) atomicAdd(hi + at, 1u);
+}
+template <bool CARRY>
+__global__ void __launch_bounds__(1024) eq3_local_kernel(const Eq3Params p) {
+    extern __shared__ __align__(16) uint32_t s_cells[];
+    uint32_t *s_lo = s_cells, *s_hi = s_cells + p.cells;
+    for (uint32_t i = threadIdx.x; i < 2 * p.cells; i += blockDim.x) s_cells[i] = 0;
+    __syncthreads();
+    grid_dependency_wait();
     uint32_t bad = 0;
     const ull stride = (ull)gridDim.x * blockDim.x;
-    for (ull i = (ull)blockIdx.x * blockDim.x + threadIdx.x; i < n_pairs; i += 2 * stride) {
-        uint32_t a[8], b[8];
-        const bool second = i + stride < n_pairs;
-        asm volatile("ld.global.L1::no_allocate.L2::evict_first.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                     : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7])
-                     : "l"(body + i * 32));
-        if (second)
-            asm volatile("ld.global.L1::no_allocate.L2::evict_first.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                         : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]), "=r"(b[4]), "=r"(b[5]), "=r"(b[6]), "=r"(b[7])
-                         : "l"(body + (i + stride) * 32));
-        bad += eq3_add<CARRY>(a[0], a[1], a[3], n_apps, n_ops, n_phases, lo, hi);
-        bad += eq3_add<CARRY>(a[4], a[5], a[7], n_apps, n_ops, n_phases, lo, hi);
-        if (second) {
-            bad += eq3_add<CARRY>(b[0], b[1], b[3], n_apps, n_ops, n_phases, lo, hi);
-            bad += eq3_add<CARRY>(b[4], b[5], b[7], n_apps, n_ops, n_phases, lo, hi);
+    for (ull i0 = (ull)blockIdx.x * blockDim.x + threadIdx.x; i0 < p.n; i0 += 4 * stride) {
+        uint4 r[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i0 + u * stride < p.n) r[u] = __ldcs(p.recs + i0 + u * stride);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (i0 + u * stride >= p.n) continue;
+            uint32_t cell;
+            if (cell_of(p, r[u], cell)) smem_add(s_lo, s_hi, cell, r[u].w);
+            else ++bad;
         }
     }
-    if (blockIdx.x == 0 && threadIdx.x < 2) {   // records outside the 32-byte aligned body
-        const uint4* one = threadIdx.x == 0 ? head : tail;
-        if (one) {
-            const uint4 r = *one;
-            bad += eq3_add<CARRY>(r.x, r.y, r.w, n_apps, n_ops, n_phases, lo, hi);
-        }
+    grid_dependents_launch();
+    count_rejected(p, bad);
+    __syncthreads();
+    // the CTAs start at different cells, so that they do not queue at the same ones
+    const uint32_t first = (uint32_t)((ull)p.cells * blockIdx.x / gridDim.x);
+    for (uint32_t i = threadIdx.x; i < p.cells; i += blockDim.x) {
+        uint32_t cell = first + i;
+        if (cell >= p.cells) cell -= p.cells;
+        const ull v = (ull)s_lo[cell] | ((ull)s_hi[cell] << 32);
+        if (v != 0) add_cell<CARRY>(p, cell, v);
     }
-    bad = __reduce_add_sync(0xFFFFFFFFu, bad);
-    if ((threadIdx.x & 31u) == 0 && bad) atomicAdd(rejected, (ull)bad);
 }
 
-// D_a[phi]: one thread per (phase, application), summing over operators
-__global__ void eq3_app_totals_kernel(const ull* lo, const ull* hi, uint32_t n_apps, uint32_t n_ops, uint32_t n_phases, ull* tot) {
-    const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (size_t)n_phases * n_apps) return;
-    const uint32_t phase = (uint32_t)(idx / n_apps), app = (uint32_t)(idx % n_apps);
-    ull s_lo = 0, s_hi = 0;
-    for (uint32_t i = 0; i < n_ops; ++i) {
-        const size_t cell = ((size_t)phase * n_ops + i) * n_apps + app;
-        const ull x = lo[cell];
-        const ull nl = s_lo + x;
-        s_hi += hi[cell] + (nl < s_lo ? 1ull : 0ull);
-        s_lo = nl;
-    }
-    tot[2 * idx] = s_lo;
-    tot[2 * idx + 1] = s_hi;
-}
-
-// wtilde_i: one CTA per operator.  The CTA finds Phi_i, then every thread works out the terms
-// p_a * (1/|Phi_i|) * sum_phi D[i][a][phi] / D_a[phi] of its applications (each a fixed sequence of
-// rounded operations, independent of the others) into shared memory in chunks; only the running sum
-// over the applications, whose order is part of the result, is left to one thread.
-constexpr int WT_THREADS = 256;
-constexpr uint32_t WT_CHUNK = 2048;   // terms held in shared memory at a time
-
-__global__ void __launch_bounds__(WT_THREADS) eq3_wtilde_kernel(const ull* lo, const ull* hi, const ull* tot, const uint32_t* appw,
-                                                                uint32_t n_apps, uint32_t n_ops, uint32_t n_phases, double* wt) {
-    __shared__ double s_term[WT_CHUNK];
-    __shared__ uint32_t s_present;
-    __shared__ ull s_weights;
-    const uint32_t i = blockIdx.x;
-    if (threadIdx.x == 0) {
-        s_present = 0;
-        s_weights = 0;
-    }
-    __syncthreads();
-    uint32_t present = 0;  // bit phi: operator i has time in phase phi
-    ull c_part = 0;
-    for (uint32_t a = threadIdx.x; a < n_apps; a += WT_THREADS) {
-        c_part += appw[a];  // < 2^64 in total: fewer than 2^32 weights below 2^32
-        for (uint32_t p = 0; p < n_phases; ++p) {
-            const size_t cell = ((size_t)p * n_ops + i) * n_apps + a;
-            if ((lo[cell] | hi[cell]) != 0) present |= 1u << p;
+// ---- D_a[phi] and Phi_i: a CTA per 32 applications and phase, its warps share the operators
+constexpr int TOTAL_WARPS = 16;
+__global__ void __launch_bounds__(TOTAL_WARPS * 32) eq3_app_totals_kernel(const ull* lo, const ull* hi, uint32_t n_apps, uint32_t n_ops, double* den,
+                                                                          uint32_t* present) {
+    __shared__ ull s_lo[TOTAL_WARPS][32], s_hi[TOTAL_WARPS][32];
+    grid_dependency_wait();
+    const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5, app = blockIdx.x * 32 + lane, phase = blockIdx.y;
+    ull t_lo = 0, t_hi = 0;
+    for (uint32_t i0 = w; i0 < n_ops; i0 += 4 * TOTAL_WARPS) {
+        ull x[4], y[4];
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u) {
+            const uint32_t i = i0 + u * TOTAL_WARPS;
+            const bool in = i < n_ops && app < n_apps;
+            const size_t cell = ((size_t)phase * n_ops + i) * n_apps + app;
+            x[u] = in ? lo[cell] : 0ull;
+            y[u] = in && hi ? hi[cell] : 0ull;
+        }
+#pragma unroll
+        for (uint32_t u = 0; u < 4; ++u) {
+            const ull s = t_lo + x[u];
+            t_hi += y[u] + (s < t_lo ? 1ull : 0ull);
+            t_lo = s;
+            if (__any_sync(FULL, (x[u] | y[u]) != 0) && lane == 0) atomicOr(&present[i0 + u * TOTAL_WARPS], 1u << phase);
         }
     }
-    if (present) atomicOr(&s_present, present);
-    atomicAdd(&s_weights, c_part);
+    grid_dependents_launch();
+    s_lo[w][lane] = t_lo;
+    s_hi[w][lane] = t_hi;
     __syncthreads();
-    present = s_present;
-    const ull c_lo = s_weights;
-    const int n_phi = __popc(present);
-    if (n_phi == 0 || c_lo == 0) {
-        if (threadIdx.x == 0) wt[i] = 0.0;
-        return;
+    if (w != 0 || app >= n_apps) return;
+    for (int k = 1; k < TOTAL_WARPS; ++k) {
+        const ull s = t_lo + s_lo[k][lane];
+        t_hi += s_hi[k][lane] + (s < t_lo ? 1ull : 0ull);
+        t_lo = s;
     }
-    const double c_total = __ull2double_rn(c_lo), d_phi = (double)n_phi;
+    den[(size_t)phase * n_apps + app] = u128_to_f64_rn(t_hi, t_lo);   // (+0.0: no time, nothing to divide)
+}
+
+// ---- wtilde_i: one CTA per operator.  The terms p_a * (1/|Phi_i|) * sum_phi D[i][a][phi] / D_a[phi] (each a fixed
+// sequence of rounded operations, independent of the others) are worked out by all warps but the first, in
+// chunks; the running sum over the applications, whose order is part of the result, by one thread of the
+// first warp, a chunk behind.  Bound by that chain: 4 096 additions.  The last CTA forms w.
+constexpr int WT_THREADS = 512;
+constexpr uint32_t WT_CHUNK = 960;    // two terms per computing thread
+
+__global__ void __launch_bounds__(WT_THREADS) eq3_wtilde_kernel(const ull* lo, const ull* hi, const double* den, const double* pa, uint32_t* present,
+                                                                uint32_t n_apps, uint32_t n_ops, uint32_t n_phases, bool any_weight, double* wt,
+                                                                const uint8_t* retained, ull* ctl, double* h_out) {
+    __shared__ __align__(16) double s_term[2][WT_CHUNK];
+    __shared__ double s_total;
+    __shared__ bool s_last;
+    grid_dependency_wait();
+    const uint32_t i = blockIdx.x, mask = present[i];
+    const int n_phi = __popc(mask);
     double acc = 0.0;   // thread 0's
-    for (uint32_t a0 = 0; a0 < n_apps; a0 += WT_CHUNK) {
-        for (uint32_t a = a0 + threadIdx.x; a < min(a0 + WT_CHUNK, n_apps); a += WT_THREADS) {
-            double inner = 0.0;
-            for (uint32_t p = 0; p < n_phases; ++p) {
-                if (!(present & (1u << p))) continue;
-                const size_t ta = (size_t)p * n_apps + a;
-                const ull t_lo = tot[2 * ta], t_hi = tot[2 * ta + 1];
-                if ((t_lo | t_hi) == 0) continue;
-                const size_t cell = ((size_t)p * n_ops + i) * n_apps + a;
-                inner = __dadd_rn(inner, __ddiv_rn(u128_to_f64_rn(hi[cell], lo[cell]), u128_to_f64_rn(t_hi, t_lo)));
+    if (n_phi != 0 && any_weight) {
+        const double d_phi = (double)n_phi;
+        const uint32_t chunks = (n_apps + WT_CHUNK - 1) / WT_CHUNK;
+        for (uint32_t c = 0; c <= chunks; ++c) {
+            if (threadIdx.x >= 32) {
+                if (c < chunks) {
+                    for (uint32_t k = threadIdx.x - 32; k < WT_CHUNK; k += WT_THREADS - 32) {
+                        const uint32_t a = c * WT_CHUNK + k;
+                        double term = 0.0;
+                        if (a < n_apps) {
+                            double inner = 0.0;
+                            for (uint32_t p = 0; p < n_phases; ++p) {
+                                if (!(mask & (1u << p))) continue;
+                                const double d = den[(size_t)p * n_apps + a];
+                                if (d == 0.0) continue;
+                                const size_t cell = ((size_t)p * n_ops + i) * n_apps + a;
+                                inner = __dadd_rn(inner, __ddiv_rn(u128_to_f64_rn(hi ? hi[cell] : 0ull, lo[cell]), d));
+                            }
+                            term = __dmul_rn(pa[a], __ddiv_rn(inner, d_phi));
+                        }
+                        s_term[c & 1][k] = term;
+                    }
+                }
+            } else if (threadIdx.x == 0 && c > 0) {
+                // (terms behind the last application are +0.0, which leaves a sum of non-negative terms as it is)
+                const double2* v = reinterpret_cast<const double2*>(s_term[(c - 1) & 1]);
+                const uint32_t n = min(WT_CHUNK, n_apps - (c - 1) * WT_CHUNK);
+                for (uint32_t k = 0; k < (n + 15) / 16 * 8; k += 8) {
+                    double2 t[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) t[u] = v[k + u];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) acc = __dadd_rn(__dadd_rn(acc, t[u].x), t[u].y);
+                }
             }
-            const double avg = __ddiv_rn(inner, d_phi);
-            const double p_a = __ddiv_rn(__ull2double_rn((ull)appw[a]), c_total);
-            s_term[a - a0] = __dmul_rn(p_a, avg);
+            __syncthreads();
         }
+    }
+    if (threadIdx.x == 0) {
+        wt[i] = acc;
+        present[i] = 0;
+        __threadfence();
+        s_last = atomicAdd(&ctl[1], 1ull) == n_ops - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!s_last) return;
+    double total = 0.0;
+    for (uint32_t i0 = 0; i0 < n_ops; i0 += WT_CHUNK) {
+        for (uint32_t k = threadIdx.x; k < WT_CHUNK; k += WT_THREADS)
+            s_term[0][k] = i0 + k < n_ops && retained[i0 + k] ? __ldcg(wt + i0 + k) : 0.0;
         __syncthreads();
         if (threadIdx.x == 0)
-            for (uint32_t a = a0; a < min(a0 + WT_CHUNK, n_apps); ++a) acc = __dadd_rn(acc, s_term[a - a0]);
+            for (uint32_t k = 0; k < min(WT_CHUNK, n_ops - i0); ++k) total = __dadd_rn(total, s_term[0][k]);
         __syncthreads();
     }
-    if (threadIdx.x == 0) wt[i] = acc;
+    if (threadIdx.x == 0) s_total = total;
+    __syncthreads();
+    for (uint32_t k = threadIdx.x; k < n_ops; k += WT_THREADS) {
+        const double v = __ldcg(wt + k);
+        h_out[k] = retained[k] && s_total > 0.0 ? __ddiv_rn(v, s_total) : 0.0;
+        h_out[n_ops + k] = v;
+    }
+    if (threadIdx.x == 0) {
+        reinterpret_cast<ull*>(h_out)[2 * (size_t)n_ops] = ctl[0];
+        ctl[1] = 0;
+    }
 }
 
-__global__ void eq3_normalise_kernel(const double* wt, const uint8_t* retained, uint32_t n_ops, double* w) {
-    __shared__ double s_total;
-    if (threadIdx.x == 0) {
-        double total = 0.0;
-        for (uint32_t i = 0; i < n_ops; ++i)
-            if (retained[i]) total = __dadd_rn(total, wt[i]);
-        s_total = total;
+// ---- launches
+cudaError_t prepare_kernels() {
+    const cudaError_t e = cudaFuncSetAttribute(eq3_local_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, LOCAL_CELLS_MAX * 8);
+    return e != cudaSuccess ? e : cudaFuncSetAttribute(eq3_local_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, LOCAL_CELLS_MAX * 8);
+}
+
+template <bool CARRY>
+cudaError_t launch_ingest(const atrex_eq3* h, const atrex_record_t* recs, ull n, cudaStream_t s) {
+    Eq3Params p;
+    p.recs = (const uint4*)recs;
+    p.n = n;
+    p.n_apps = h->n_apps; p.n_ops = h->n_ops; p.n_phases = h->n_phases;
+    p.cells = (uint32_t)h->cells;
+    p.lo = h->d_lo; p.hi = h->d_hi;
+    p.rejected = h->d_ctl;
+    const size_t cell_bytes = h->cells * 8;
+    // local: as long as every SM gets twice as many records as it has cells to add up at the end
+    if (h->cells <= LOCAL_CELLS_MAX && n >= 2ull * h->cells * h->n_sms && n >= 65536) {
+        const uint32_t threads = cell_bytes > 72 * 1024 ? 1024 : 512;
+        uint32_t per_sm = (uint32_t)(232448 / (cell_bytes + 1024));
+        if (per_sm > 2048 / threads) per_sm = 2048 / threads;
+        ull grid = n / (2 * h->cells);
+        if (grid > n / (4 * threads)) grid = n / (4 * threads);
+        if (grid > (ull)h->n_sms * per_sm) grid = (ull)h->n_sms * per_sm;
+        if (grid < 1) grid = 1;
+        return launch_chained(eq3_local_kernel<CARRY>, (uint32_t)grid, threads, cell_bytes, s, p);
     }
-    __syncthreads();
-    for (uint32_t i = threadIdx.x; i < n_ops; i += blockDim.x)
-        w[i] = (retained[i] && s_total > 0.0) ? __ddiv_rn(wt[i], s_total) : 0.0;
+    return launch_chained(eq3_direct_kernel<CARRY>, grid_for_work(n, 512, h->n_sms, 4), 512, 0, s, p);
 }
 
 }  // namespace
@@ -210,20 +326,41 @@ int atrex_eq3_create(uint32_t n_apps, uint32_t n_ops, uint32_t n_phases, const u
     atrex_eq3* h = new (std::nothrow) atrex_eq3;
     if (!h) return ATREX_ERR_NOMEM;
     h->n_apps = n_apps; h->n_ops = n_ops; h->n_phases = n_phases; h->device = device; h->cells = cells;
+    // card-hour fractions: fl(c_a / fl(sum of all))
+    ull c_sum = 0;
+    for (uint32_t a = 0; a < n_apps; ++a) c_sum += app_weights[a];
+    h->c_total = (double)c_sum;
+    double* pa = (double*)malloc((size_t)n_apps * 8);
+    if (!pa) {
+        delete h;
+        return ATREX_ERR_NOMEM;
+    }
+    for (uint32_t a = 0; a < n_apps; ++a) pa[a] = c_sum ? (double)app_weights[a] / h->c_total : 0.0;
     Guard g(device);
     cudaError_t e = cudaDeviceGetAttribute(&h->n_sms, cudaDevAttrMultiProcessorCount, device);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_appw, (size_t)n_apps * 4);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_lo, cells * 8);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_hi, cells * 8);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_tot, (size_t)n_phases * n_apps * 16);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_wt, (size_t)n_ops * 8);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_w, (size_t)n_ops * 8);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_ret, n_ops);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&h->d_rejected, 8);
-    if (e == cudaSuccess) e = cudaMemcpy(h->d_appw, app_weights, (size_t)n_apps * 4, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(h->d_lo, 0, cells * 8);
-    if (e == cudaSuccess) e = cudaMemset(h->d_hi, 0, cells * 8);
-    if (e == cudaSuccess) e = cudaMemset(h->d_rejected, 0, 8);
+    size_t o = 0;
+    auto take = [&](size_t bytes) {
+        const size_t at = o;
+        o += (bytes + 255) / 256 * 256;
+        return at;
+    };
+    const size_t o_ctl = take(16), o_present = take((size_t)n_ops * 4), o_lo = take(cells * 8), o_hi = take(cells * 8),
+                 o_den = take((size_t)n_phases * n_apps * 8), o_pa = take((size_t)n_apps * 8), o_wt = take((size_t)n_ops * 8);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&h->arena, o);
+    if (e == cudaSuccess) e = pinned_alloc((void**)&h->h_out, h->h_bytes = ((size_t)n_ops * 2 + 1) * 8 + n_ops);
+    if (e == cudaSuccess) {
+        h->d_ctl = (ull*)(h->arena + o_ctl);
+        h->d_present = (uint32_t*)(h->arena + o_present);
+        h->d_lo = (ull*)(h->arena + o_lo);
+        h->d_hi = (ull*)(h->arena + o_hi);
+        h->d_den = (double*)(h->arena + o_den);
+        h->d_pa = (double*)(h->arena + o_pa);
+        h->d_wt = (double*)(h->arena + o_wt);
+        e = cudaMemset(h->arena, 0, o_den);   // control, Phi, cells
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(h->d_pa, pa, (size_t)n_apps * 8, cudaMemcpyHostToDevice);
+    free(pa);
+    if (e == cudaSuccess) e = prepare_kernels();
     if (e != cudaSuccess) {
         cudaGetLastError();
         atrex_eq3_destroy(h);
@@ -237,8 +374,8 @@ void atrex_eq3_destroy(atrex_eq3_t* h) {
     if (!h) return;
     Guard g(h->device);
     cudaDeviceSynchronize();
-    cudaFree(h->d_appw); cudaFree(h->d_lo); cudaFree(h->d_hi); cudaFree(h->d_tot);
-    cudaFree(h->d_wt); cudaFree(h->d_w); cudaFree(h->d_ret); cudaFree(h->d_rejected);
+    cudaFree(h->arena);
+    pinned_free(h->h_out, h->h_bytes);
     delete h;
 }
 
@@ -246,10 +383,11 @@ int atrex_eq3_reset(atrex_eq3_t* h, void* stream) {
     if (!h) return ATREX_ERR_INVALID;
     Guard g(h->device);
     cudaStream_t s = (cudaStream_t)stream;
-    if (cudaMemsetAsync(h->d_lo, 0, h->cells * 8, s) != cudaSuccess || cudaMemsetAsync(h->d_hi, 0, h->cells * 8, s) != cudaSuccess ||
-        cudaMemsetAsync(h->d_rejected, 0, 8, s) != cudaSuccess)
-        return ATREX_ERR_CUDA;
+    // control, Phi, low limbs; the second limb only where wraps were counted
+    const unsigned char* end = (const unsigned char*)(h->hi_used ? h->d_hi + h->cells : h->d_lo + h->cells);
+    if (cudaMemsetAsync(h->arena, 0, end - h->arena, s) != cudaSuccess) return ATREX_ERR_CUDA;
     h->n_ingested = 0;
+    h->hi_used = false;
     return ATREX_OK;
 }
 
@@ -258,25 +396,12 @@ int atrex_eq3_ingest(atrex_eq3_t* h, const atrex_record_t* d_records, uint64_t n
     if (n == 0) return ATREX_OK;
     if (!d_records || ((uintptr_t)d_records & 15u)) return ATREX_ERR_INVALID;
     Guard g(h->device);
-    // the 32-byte aligned body as record pairs; at most one record before and one after it
-    const unsigned char* base = (const unsigned char*)d_records;
-    const uint64_t head = ((uintptr_t)base & 31u) ? 1 : 0;
-    const uint64_t n_body = n - head, n_pairs = n_body / 2;
-    const uint4* head_rec = head ? (const uint4*)base : nullptr;
-    const uint4* tail_rec = (n_body & 1) ? (const uint4*)(base + (n - 1) * 16) : nullptr;
-    ull blocks = (n_pairs + 1023) / 1024;
-    if (blocks > (ull)h->n_sms * 4) blocks = (ull)h->n_sms * 4;
-    if (blocks == 0) blocks = 1;
-    // below 2^32 records in total no cell's 64-bit sum can wrap: fire-and-forget reductions
+    // below 2^32 records in total no cell's 64-bit sum can wrap: reductions that return nothing
     const bool carry = h->n_ingested + n >= (1ull << 32);
     h->n_ingested += n;
-    if (carry)
-        eq3_ingest_kernel<true><<<(unsigned)blocks, 512, 0, (cudaStream_t)stream>>>(base + head * 16, n_pairs, head_rec, tail_rec, h->n_apps,
-                                                                                    h->n_ops, h->n_phases, h->d_lo, h->d_hi, h->d_rejected);
-    else
-        eq3_ingest_kernel<false><<<(unsigned)blocks, 512, 0, (cudaStream_t)stream>>>(base + head * 16, n_pairs, head_rec, tail_rec, h->n_apps,
-                                                                                     h->n_ops, h->n_phases, h->d_lo, h->d_hi, h->d_rejected);
-    return cudaGetLastError() == cudaSuccess ? ATREX_OK : ATREX_ERR_CUDA;
+    h->hi_used |= carry;
+    const cudaError_t e = carry ? launch_ingest<true>(h, d_records, n, (cudaStream_t)stream) : launch_ingest<false>(h, d_records, n, (cudaStream_t)stream);
+    return e == cudaSuccess ? ATREX_OK : ATREX_ERR_CUDA;
 }
 
 int atrex_eq3_finalize(atrex_eq3_t* h, const uint8_t* h_retained, double* h_w, double* h_wtilde, uint64_t* h_rejected,
@@ -284,26 +409,23 @@ int atrex_eq3_finalize(atrex_eq3_t* h, const uint8_t* h_retained, double* h_w, d
     if (!h || !h_w) return ATREX_ERR_INVALID;
     Guard g(h->device);
     cudaStream_t s = (cudaStream_t)stream;
-    uint8_t* all = nullptr;
-    if (!h_retained) {
-        all = (uint8_t*)malloc(h->n_ops);
-        if (!all) return ATREX_ERR_NOMEM;
-        memset(all, 1, h->n_ops);
-    }
-    cudaError_t e = cudaMemcpyAsync(h->d_ret, h_retained ? h_retained : all, h->n_ops, cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess && all) e = cudaStreamSynchronize(s);  // `all` is freed below
-    free(all);
-    if (e != cudaSuccess) return ATREX_ERR_CUDA;
-    const size_t pa = (size_t)h->n_phases * h->n_apps;
-    eq3_app_totals_kernel<<<(unsigned)((pa + 255) / 256), 256, 0, s>>>(h->d_lo, h->d_hi, h->n_apps, h->n_ops, h->n_phases, h->d_tot);
-    eq3_wtilde_kernel<<<h->n_ops, WT_THREADS, 0, s>>>(h->d_lo, h->d_hi, h->d_tot, h->d_appw, h->n_apps, h->n_ops, h->n_phases, h->d_wt);
-    eq3_normalise_kernel<<<1, 256, 0, s>>>(h->d_wt, h->d_ret, h->n_ops, h->d_w);
+    const uint32_t n_ops = h->n_ops;
+    // the flags are read and the results written by the kernels, in pinned memory
+    uint8_t* retained = (uint8_t*)(h->h_out + 2 * (size_t)n_ops + 1);
+    if (h_retained) memcpy(retained, h_retained, n_ops);
+    else memset(retained, 1, n_ops);
+    const ull* hi = h->hi_used ? h->d_hi : nullptr;
+    eq3_app_totals_kernel<<<dim3((h->n_apps + 31) / 32, h->n_phases), TOTAL_WARPS * 32, 0, s>>>(h->d_lo, hi, h->n_apps, n_ops, h->d_den, h->d_present);
     if (cudaGetLastError() != cudaSuccess) return ATREX_ERR_CUDA;
-    e = cudaMemcpyAsync(h_w, h->d_w, (size_t)h->n_ops * 8, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess && h_wtilde) e = cudaMemcpyAsync(h_wtilde, h->d_wt, (size_t)h->n_ops * 8, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess && h_rejected) e = cudaMemcpyAsync(h_rejected, h->d_rejected, 8, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    return e == cudaSuccess ? ATREX_OK : ATREX_ERR_CUDA;
+    const bool any_weight = h->c_total != 0.0;
+    if (launch_chained(eq3_wtilde_kernel, n_ops, WT_THREADS, 0, s, h->d_lo, hi, h->d_den, h->d_pa, h->d_present, h->n_apps, n_ops, h->n_phases,
+                       any_weight, h->d_wt, retained, h->d_ctl, h->h_out) != cudaSuccess)
+        return ATREX_ERR_CUDA;
+    if (cudaStreamSynchronize(s) != cudaSuccess) return ATREX_ERR_CUDA;
+    memcpy(h_w, h->h_out, (size_t)n_ops * 8);
+    if (h_wtilde) memcpy(h_wtilde, h->h_out + n_ops, (size_t)n_ops * 8);
+    if (h_rejected) memcpy(h_rejected, h->h_out + 2 * (size_t)n_ops, 8);
+    return ATREX_OK;
 }
 
 }  // extern "C"

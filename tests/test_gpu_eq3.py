@@ -81,3 +81,30 @@ def test_eq3_beyond_two_to_the_32_records_switches_to_counted_carries():
     ew, ewt, erej = oracle.eq3_weights(np.concatenate([x, y]), weights, n_ops, n_phases)
     assert rej == erej == 0
     assert wt.tobytes() == ewt.tobytes() and w.tobytes() == ew.tobytes()
+
+
+# cells that fit a CTA's shared memory (the last of them just) and more
+@pytest.mark.parametrize("n_apps,n_ops,n_phases", [(3, 1, 1), (100, 70, 4), (1000, 29, 1), (256, 112, 1), (128, 225, 1), (4097, 33, 2), (7000, 250, 4)])
+@pytest.mark.parametrize("n", [1, 70_001, (1 << 21) + 3, (1 << 23) + 12_345])
+@pytest.mark.parametrize("law", ["spread", "crowded"])
+def test_eq3_routes_match_the_oracle(n_apps, n_ops, n_phases, n, law):
+    import paper_2607_14541_b200 as p
+    from tracegen.layout import RECORD_DTYPE
+    rng = np.random.default_rng(n + n_apps)
+    recs = np.zeros(n, dtype=RECORD_DTYPE)
+    recs["app_id"] = rng.integers(0, n_apps + 1, n, dtype=np.uint32)          # the last application does not exist
+    recs["op_id"] = rng.integers(0, n_ops, n)
+    recs["phase"] = rng.integers(0, n_phases, n)
+    recs["duration_ns"] = rng.integers(0, 1 << 32, n, dtype=np.uint64)
+    if law == "crowded":                                                      # far more than a bin's share in one cell
+        hot = rng.random(n) < 0.6
+        recs["app_id"][hot], recs["op_id"][hot], recs["phase"][hot] = n_apps - 1, n_ops - 1, 0
+    weights = rng.integers(0, 1 << 20, n_apps).astype(np.uint32)
+    weights[0] = 1
+    ow = p.OperatorWeights(weights, n_ops, n_phases)
+    ow.ingest(to_dev(recs), n=n)
+    ow.ingest(to_dev(recs[: n // 3]), n=n // 3)
+    w, wt, rej = ow.finalize()
+    both = np.concatenate([recs, recs[: n // 3]])
+    ew, ewt, erej = oracle.eq3_weights(both, weights, n_ops, n_phases)
+    assert rej == erej and wt.tobytes() == ewt.tobytes() and w.tobytes() == ew.tobytes()
