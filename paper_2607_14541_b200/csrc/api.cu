@@ -23,7 +23,11 @@ constexpr size_t L2_TABLE_BYTES = 48ull << 20;           // a table up to this s
 constexpr uint32_t HOT_SAMPLE = 1u << 20;
 constexpr uint32_t CAND_BITS = 17;                     // candidate table of the directory build
 constexpr size_t SKETCH_BYTES = (size_t)4 << 20;        // 2^20 counters (ingest.cu SKETCH_BITS)
-constexpr size_t HOT_SCRATCH_BYTES = SKETCH_BYTES + ((size_t)12 << CAND_BITS);
+// sketch, candidate table and the first part of HotBuildScratch are cleared by every build; the sampled keys lie behind
+constexpr size_t HOT_SELECT_OFF = SKETCH_BYTES + ((size_t)12 << CAND_BITS);
+constexpr size_t HOT_COUNT_BYTES = HOT_SELECT_OFF + offsetof(HotBuildScratch, key);
+constexpr size_t HOT_SAMPLE_OFF = HOT_SELECT_OFF + (sizeof(HotBuildScratch) + 255) / 256 * 256;
+constexpr size_t HOT_SCRATCH_BYTES = HOT_SAMPLE_OFF + (size_t)HOT_SAMPLE * 8;
 constexpr uint32_t SEL_CAP = ATREX_MAX_TOPK + TOPK_CAND_CAP;
 
 size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
@@ -170,11 +174,12 @@ struct atrex_agg {
     uint32_t* d_appw = nullptr;
     ull* hot_keys = nullptr;
     ulonglong2* hot_img = nullptr;   // [n_groups][hot_slots] per-CTA directory sums not yet in the table
-    bool hot_dirty = false;          // the image rows may hold sums
+    uint32_t img_rows = 0;           // rows that hold sums
     unsigned char* staging[2] = {nullptr, nullptr};
     ull* sel = nullptr;
     atrex_entry_t* topk_out = nullptr;
     Control* h_ctl = nullptr;  // pinned mirror
+    size_t pinned_bytes = 0;
     uint32_t* hist_all = nullptr;     // [ATREX_MAX_PHASES][TOPK_BINS] first-digit counts of all phases
     ull* pick = nullptr;              // [n_phases][TOPK_PICK_MAX][4] candidates
     atrex_entry_t* h_top = nullptr;   // pinned: [n_phases][TOPK_PICK_K] the best k of each phase, then u32 [n_phases] how many
@@ -329,10 +334,11 @@ int atrex_agg_create(const atrex_agg_config_t* cfg, atrex_agg_t** out) {
         if (e == cudaSuccess) e = cudaMemset(h->ws + L.off_ctl, 0, L.off_appw - L.off_ctl);  // control, spill counts, table, work
         if (e == cudaSuccess) e = cudaMemcpy(h->d_appw, cfg->app_weights, (size_t)cfg->n_apps * 4, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemset(h->hot_keys, 0, (size_t)(L.hot_slots ? L.hot_slots : 2) * 8);
-        if (e == cudaSuccess) e = cudaMemset(h->hot_img, 0, (size_t)L.n_groups * (L.hot_slots ? L.hot_slots : 2) * 16);
-        if (e == cudaSuccess) e = cudaHostAlloc((void**)&h->h_ctl, sizeof(Control), cudaHostAllocMapped);
-        if (e == cudaSuccess)
-            e = cudaHostAlloc((void**)&h->h_top, (size_t)cfg->n_phases * (TOPK_PICK_K * sizeof(atrex_entry_t) + 4), cudaHostAllocMapped);
+        // the pinned block: every phase's best, how many there are, the control block's mirror
+        const size_t top_bytes = (size_t)cfg->n_phases * (TOPK_PICK_K * sizeof(atrex_entry_t) + 8);
+        h->pinned_bytes = top_bytes + sizeof(Control);
+        if (e == cudaSuccess) e = pinned_alloc((void**)&h->h_top, h->pinned_bytes);
+        if (e == cudaSuccess) h->h_ctl = (Control*)((unsigned char*)h->h_top + top_bytes);
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking);
         for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
             e = cudaEventCreateWithFlags(&h->ev_ready[i], cudaEventDisableTiming);
@@ -360,8 +366,7 @@ void atrex_agg_destroy(atrex_agg_t* h) {
         if (h->ev_free[i]) cudaEventDestroy(h->ev_free[i]);
     }
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
-    if (h->h_ctl) cudaFreeHost(h->h_ctl);
-    if (h->h_top) cudaFreeHost(h->h_top);
+    pinned_free(h->h_top, h->pinned_bytes);
     if (h->owns_workspace && h->ws) cudaFree(h->ws);
     delete h;
 }
@@ -373,8 +378,7 @@ int atrex_agg_reset(atrex_agg_t* h, void* stream) {
     cudaStream_t s = (cudaStream_t)stream;
     // control block, spill counts (undrained entries are discarded), keys and values
     CU(h, cudaMemsetAsync(h->ctl, 0, h->L.off_work - h->L.off_ctl, s));
-    if (h->hot_dirty) CU(h, cudaMemsetAsync(h->hot_img, 0, (size_t)h->L.n_groups * (h->L.hot_slots ? h->L.hot_slots : 2) * 16, s));
-    h->hot_dirty = false;
+    h->img_rows = 0;
     h->spill_pending = false;
     h->hot_ready = false;
     h->finalized = false;
@@ -415,6 +419,13 @@ int atrex_agg_set_work_table(atrex_agg_t* h, const atrex_work_t* rows, uint64_t 
 // drains whatever is there.
 static int drain_spill(atrex_agg* h, bool force, cudaStream_t s) {
     if (force && !h->spill_pending) return ATREX_OK;
+    if (force && h->img_rows) {
+        // results are about to be read: the directory sums kept per scatter CTA join the table (before the
+        // spilled entries do, while the frequent keys' slots are still easy to come by)
+        CU(h, launch_hot_fold(h->hot_keys, h->hot_img, h->img_rows, h->L.hot_slots, h->table_ref(), s));
+        h->launches++;
+        h->img_rows = 0;
+    }
     PartitionParams q;
     q.t = h->table_ref();
     q.spill = h->spill;
@@ -428,12 +439,6 @@ static int drain_spill(atrex_agg* h, bool force, cudaStream_t s) {
     q.seq = h->scatter_seq;
     CU(h, launch_partition(q, h->n_sms, s));
     h->launches++;
-    if (force && h->hot_dirty) {
-        // results are about to be read: the directory sums kept per scatter CTA join the table
-        CU(h, launch_hot_fold(h->hot_keys, h->hot_img, h->L.n_groups, h->L.hot_slots, h->table_ref(), s));
-        h->launches++;
-        h->hot_dirty = false;
-    }
     if (force) h->spill_pending = false;
     return ATREX_OK;
 }
@@ -460,20 +465,22 @@ static int ingest_launch(atrex_agg* h, const atrex_record_t* recs, uint64_t n, c
     if (h->L.hot_slots && !h->hot_ready) {
         HotBuildParams b;
         b.recs = (const uint4*)recs;
-        b.n_sample = (uint32_t)(n < HOT_SAMPLE ? n : HOT_SAMPLE);
-        b.stride = n / b.n_sample;
+        b.n_sample = (uint32_t)(n < HOT_SAMPLE ? n : HOT_SAMPLE) & ~(HOT_SAMPLE_RUN - 1);   // (n is at least DIRECT_RECORDS_MAX here)
+        b.stride = n / (b.n_sample / HOT_SAMPLE_RUN);
         b.n_apps = h->cfg.n_apps;
         b.n_phases = h->cfg.n_phases;
         b.hot_keys = h->hot_keys;
         b.hot_slots = h->L.hot_slots;
         b.ctl = h->ctl;
         b.sketch = (uint32_t*)h->hot_scratch;
+        b.sample = (ull*)(h->hot_scratch + HOT_SAMPLE_OFF);
+        b.scratch = (HotBuildScratch*)(h->hot_scratch + HOT_SELECT_OFF);
         b.cand_keys = (ull*)(h->hot_scratch + SKETCH_BYTES);
         b.cand_cnt = (uint32_t*)(h->hot_scratch + SKETCH_BYTES + ((size_t)8 << CAND_BITS));
         b.cand_bits = CAND_BITS;
-        CU(h, cudaMemsetAsync(h->hot_scratch, 0, HOT_SCRATCH_BYTES, s));
+        CU(h, cudaMemsetAsync(h->hot_scratch, 0, HOT_COUNT_BYTES, s));
         CU(h, launch_hot_build(b, h->n_sms, s));
-        h->launches += 3;
+        h->launches += 6;
         h->hot_ready = true;
     }
     IngestParams p;
@@ -507,8 +514,9 @@ static int ingest_launch(atrex_agg* h, const atrex_record_t* recs, uint64_t n, c
     int grid = (int)(want < 1 ? 1 : (want > (ull)h->n_sms ? (ull)h->n_sms : want));
     p.drain_above = h->L.cap / 4 * 3;
     p.seq = ++h->scatter_seq;
+    p.img_rows = h->img_rows;
     CU(h, launch_scatter(p, h->hot_ready, grid, s));
-    if (h->hot_ready) h->hot_dirty = true;
+    if (h->hot_ready && h->img_rows < (uint32_t)grid) h->img_rows = (uint32_t)grid;
     h->spill_pending = true;
     h->launches++;
     return drain_spill(h, /*force=*/false, s);

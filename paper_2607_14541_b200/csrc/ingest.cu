@@ -83,27 +83,34 @@ __device__ __forceinline__ ull limbs_drain(uint32_t a0, uint32_t a1, ull* hi_out
     return v;
 }
 
-// Adds every CTA's directory image row into the table and clears the rows.  A CTA handles 32
-// directory slots: warp w sums rows w, w + 8, ... of those slots (exact: 128-bit sum, count), the
-// eight partial sums meet in shared memory and warp 0 does one table update per slot.
-constexpr int FOLD_WARPS = 8;
+// Adds every CTA's directory image row into the table (the next launch starts the rows afresh).  A CTA handles 32
+// directory slots: warp w sums rows w, w + 16, ... of those slots (exact: 128-bit sum, count), the
+// sixteen partial sums meet in shared memory and warp 0 does one table update per slot.
+constexpr int FOLD_WARPS = 16;
 
-__global__ void __launch_bounds__(FOLD_WARPS * 32) hot_fold_kernel(const ull* hot_keys, ulonglong2* hot_img,
+__global__ void __launch_bounds__(FOLD_WARPS * 32) hot_fold_kernel(const ull* hot_keys, const ulonglong2* hot_img,
                                                                    uint32_t n_groups, uint32_t hot_slots, TableRef t) {
     __shared__ ull s_lo[FOLD_WARPS][32], s_hi[FOLD_WARPS][32], s_cnt[FOLD_WARPS][32];
     const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
     const uint32_t i = blockIdx.x * 32u + lane;
     ull lo = 0, hi = 0, count = 0;
     if (i < hot_slots) {
-        for (uint32_t g = w; g < n_groups; g += FOLD_WARPS) {
-            ulonglong2* at = hot_img + (size_t)g * hot_slots + i;
-            const ulonglong2 v = *at;
-            if ((v.x | v.y) == 0) continue;
-            const ull s = lo + v.x;
-            hi += (v.y >> HI_SHIFT) + (s < lo ? 1ull : 0ull);
-            lo = s;
-            count += v.y & COUNT_MASK;
-            *at = make_ulonglong2(0, 0);
+        constexpr uint32_t ILP = 5;     // rows in flight per lane
+        for (uint32_t g0 = w; g0 < n_groups; g0 += ILP * FOLD_WARPS) {
+            ulonglong2 v[ILP];
+#pragma unroll
+            for (uint32_t u = 0; u < ILP; ++u) {
+                const uint32_t g = g0 + u * FOLD_WARPS;
+                v[u] = g < n_groups ? hot_img[(size_t)g * hot_slots + i] : make_ulonglong2(0, 0);
+            }
+#pragma unroll
+            for (uint32_t u = 0; u < ILP; ++u) {
+                if ((v[u].x | v[u].y) == 0) continue;
+                const ull s = lo + v[u].x;
+                hi += (v[u].y >> HI_SHIFT) + (s < lo ? 1ull : 0ull);
+                lo = s;
+                count += v[u].y & COUNT_MASK;
+            }
         }
     }
     s_lo[w][lane] = lo;
@@ -490,189 +497,280 @@ __global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(PartitionP
 }
 
 // --------------------------------------------------------------------------------------
-// Hot-directory construction, three small kernels over a strided sample of the records:
-//   1. count   every sampled key bumps one of 2^20 counters chosen by its hash;
+// Hot-directory construction, small kernels over a sample of the records (runs of four neighbouring records, evenly
+// spread: a DRAM burst of 64 bytes costs the same as one record of it):
+//   1. count   every sampled key bumps one of 2^20 counters chosen by its hash; the keys are kept side by side;
 //   2. admit   sampled keys whose counter reached ADMIT_MIN are inserted, with exact counts,
 //              into a candidate table (colliding cold keys may slip in; harmless);
-//   3. select  one CTA picks the count threshold that fills the directory and installs the
-//              candidates, most frequent classes first, into 4-slot buckets.
-// Which keys end up in the directory only affects speed, never results.
+//   3. level   how many candidates have which count, and from that the count that fills the directory;
+//   4. gather  the candidates above it side by side, and how much weight each of four bucket hashes would lose;
+//   5. list    the candidates of each 4-slot bucket under the best of them;
+//   6. pick    each bucket takes its four most frequent ones.
+// Which keys end up in the directory only affects speed, never results.  Bound by latency and launches: 75 us for
+// 2^20 samples; 187 us when single records were read (twice) and one CTA did steps 3 to 6.
 constexpr uint32_t SKETCH_BITS = 20;   // as many counters as samples, so that cold keys stay below ADMIT_MIN
 constexpr uint32_t ADMIT_MIN = 3;
 constexpr uint32_t CAND_PROBES = 16;
+constexpr uint32_t SAMPLE_ILP = 4;     // samples in flight per thread
+constexpr uint32_t RUN = HOT_SAMPLE_RUN;
 
-__device__ __forceinline__ bool sample_key(const HotBuildParams& p, uint32_t j, ull* key) {
-    uint4 v = p.recs[(ull)j * p.stride];
-    uint32_t khi = v.y & 0x00FFFFFFu;
-    *key = ((ull)khi << 32) | v.z;
-    return v.x < p.n_apps && (khi >> 16) < p.n_phases;
-}
-
-// Lanes of a warp that target the same counter are combined first, so that a trace dominated
-// by one key does not serialise on one address.
-__device__ __forceinline__ void combined_count(uint32_t* counters, uint32_t index, bool active) {
-    unsigned act = __ballot_sync(0xFFFFFFFFu, active);
-    if (!active) return;
-    unsigned same = __match_any_sync(act, index);
-    if ((threadIdx.x & 31u) == (unsigned)(__ffs(same) - 1)) atomicAdd(&counters[index], (uint32_t)__popc(same));
-}
+// Counts for lanes of a warp that target the same counter are combined first, and those of a CTA in a small
+// shared-memory cache, so that a trace dominated by one key does not queue at one address.
+constexpr uint32_t CACHE = 256;
+struct CountCache {
+    uint32_t index[CACHE], count[CACHE];   // index + 1, 0 = free
+    __device__ __forceinline__ void clear() {
+        for (uint32_t i = threadIdx.x; i < CACHE; i += blockDim.x) index[i] = count[i] = 0;
+        __syncthreads();
+    }
+    __device__ __forceinline__ void add(uint32_t* counters, uint32_t at, bool active) {
+        const unsigned act = __ballot_sync(0xFFFFFFFFu, active);
+        if (!active) return;
+        const unsigned same = __match_any_sync(act, at);
+        if ((threadIdx.x & 31u) != (unsigned)(__ffs(same) - 1)) return;
+        const uint32_t n = (uint32_t)__popc(same), slot = (at * 0x9E3779B1u) >> 24;
+        static_assert(CACHE == 256, "top eight bits");
+        if (n > 1) {
+            const uint32_t owner = atomicCAS(&index[slot], 0u, at + 1u);
+            if (owner == 0 || owner == at + 1u) {
+                atomicAdd(&count[slot], n);
+                return;
+            }
+        }
+        atomicAdd(&counters[at], n);
+    }
+    __device__ __forceinline__ void flush(uint32_t* counters) {
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < CACHE; i += blockDim.x)
+            if (count[i]) atomicAdd(&counters[index[i] - 1u], count[i]);
+    }
+};
 
 __global__ void __launch_bounds__(256) hot_count_kernel(HotBuildParams p) {
+    __shared__ CountCache cache;
+    cache.clear();
+    grid_dependency_wait();
     const uint32_t stride = gridDim.x * blockDim.x;
-    const uint32_t rounds = (p.n_sample + stride - 1) / stride;  // uniform trip count: warp collectives inside
+    const uint32_t rounds = (p.n_sample + stride * SAMPLE_ILP - 1) / (stride * SAMPLE_ILP);  // uniform trip count: warp collectives inside
     for (uint32_t r = 0; r < rounds; ++r) {
-        uint32_t j = r * stride + blockIdx.x * blockDim.x + threadIdx.x;
-        ull key = 0;
-        bool ok = j < p.n_sample && sample_key(p, j, &key);
-        combined_count(p.sketch, hash32(key) >> (32 - SKETCH_BITS), ok);
+        uint4 v[SAMPLE_ILP];
+#pragma unroll
+        for (uint32_t u = 0; u < SAMPLE_ILP; ++u) {
+            const uint32_t j = (r * SAMPLE_ILP + u) * stride + blockIdx.x * blockDim.x + threadIdx.x;
+            v[u] = j < p.n_sample ? p.recs[(ull)(j / RUN) * p.stride + j % RUN] : make_uint4(0xFFFFFFFFu, 0, 0, 0);
+        }
+#pragma unroll
+        for (uint32_t u = 0; u < SAMPLE_ILP; ++u) {
+            const uint32_t j = (r * SAMPLE_ILP + u) * stride + blockIdx.x * blockDim.x + threadIdx.x;
+            const uint32_t khi = v[u].y & 0x00FFFFFFu;
+            const bool ok = j < p.n_sample && v[u].x < p.n_apps && (khi >> 16) < p.n_phases;
+            if (j < p.n_sample) p.sample[j] = ok ? ((ull)khi << 32) | v[u].z : ~0ull;
+            cache.add(p.sketch, hash32(khi & 0xFFFFu, v[u].z) >> (32 - SKETCH_BITS), ok);
+        }
     }
+    grid_dependents_launch();
+    cache.flush(p.sketch);
 }
 
 __global__ void __launch_bounds__(256) hot_admit_kernel(HotBuildParams p) {
+    __shared__ CountCache cache;
+    cache.clear();
+    grid_dependency_wait();
     const uint32_t stride = gridDim.x * blockDim.x;
-    const uint32_t rounds = (p.n_sample + stride - 1) / stride;
+    const uint32_t rounds = (p.n_sample + stride * SAMPLE_ILP - 1) / (stride * SAMPLE_ILP);
     for (uint32_t r = 0; r < rounds; ++r) {
-        uint32_t j = r * stride + blockIdx.x * blockDim.x + threadIdx.x;
-        ull key = 0;
-        bool ok = j < p.n_sample && sample_key(p, j, &key);
-        uint32_t h = hash32(key);
-        ok = ok && p.sketch[h >> (32 - SKETCH_BITS)] >= ADMIT_MIN;
-        const ull skey = ~key;
-        uint32_t s = (h * 0x9E3779B1u) >> (32 - p.cand_bits);
-        bool found = false;
-        if (ok) {
-            for (uint32_t probe = 0; probe < CAND_PROBES && !found; ++probe) {
-                ull k = ld_relaxed(&p.cand_keys[s]);
-                if (k == 0) {
-                    k = atomicCAS(&p.cand_keys[s], 0ull, skey);
-                    if (k == 0) k = skey;
-                }
-                if (k == skey)
-                    found = true;
-                else
-                    s = (s + 1) & ((1u << p.cand_bits) - 1);
-            }
+        ull key[SAMPLE_ILP];
+        uint32_t seen[SAMPLE_ILP];
+#pragma unroll
+        for (uint32_t u = 0; u < SAMPLE_ILP; ++u) {
+            const uint32_t j = (r * SAMPLE_ILP + u) * stride + blockIdx.x * blockDim.x + threadIdx.x;
+            key[u] = j < p.n_sample ? p.sample[j] : ~0ull;
         }
-        combined_count(p.cand_cnt, s, found);
+#pragma unroll
+        for (uint32_t u = 0; u < SAMPLE_ILP; ++u) seen[u] = key[u] != ~0ull ? p.sketch[hash32(key[u]) >> (32 - SKETCH_BITS)] : 0u;
+#pragma unroll
+        for (uint32_t u = 0; u < SAMPLE_ILP; ++u) {
+            const ull skey = ~key[u];
+            uint32_t s = (hash32(key[u]) * 0x9E3779B1u) >> (32 - p.cand_bits);
+            bool found = false;
+            if (seen[u] >= ADMIT_MIN) {
+                for (uint32_t probe = 0; probe < CAND_PROBES && !found; ++probe) {
+                    ull k = ld_relaxed(&p.cand_keys[s]);
+                    if (k == 0) {
+                        k = atomicCAS(&p.cand_keys[s], 0ull, skey);
+                        if (k == 0) k = skey;
+                    }
+                    if (k == skey)
+                        found = true;
+                    else
+                        s = (s + 1) & ((1u << p.cand_bits) - 1);
+                }
+            }
+            cache.add(p.cand_cnt, s, found);
+        }
+    }
+    grid_dependents_launch();
+    cache.flush(p.cand_cnt);
+}
+
+constexpr uint32_t LIST_MAX = 16;       // candidates a bucket chooses from (five on average)
+constexpr uint32_t LEVEL_THREADS = 1024;
+
+__global__ void __launch_bounds__(LEVEL_THREADS) hot_level_kernel(HotBuildParams p) {
+    __shared__ uint32_t s_hist[1024], s_warp[32];
+    __shared__ bool s_last;
+    const uint32_t t = threadIdx.x, lane = t & 31u, w = t >> 5;
+    s_hist[t] = 0;
+    __syncthreads();
+    grid_dependency_wait();
+    HotBuildScratch& x = *p.scratch;
+    const uint32_t n_cand = 1u << p.cand_bits;
+    uint32_t most = 0;
+    for (uint32_t i0 = blockIdx.x * LEVEL_THREADS; i0 < n_cand; i0 += gridDim.x * LEVEL_THREADS) {
+        const uint32_t c = p.cand_cnt[i0 + t];
+        most = max(most, c);
+        // (most counts are small: a warp's are counted by votes instead of queueing at a few bins)
+#pragma unroll
+        for (uint32_t k = ADMIT_MIN; k < ADMIT_MIN + 4; ++k) {
+            const uint32_t votes = __ballot_sync(0xFFFFFFFFu, c == k);
+            if (lane == 0 && votes) atomicAdd(&s_hist[k], (uint32_t)__popc(votes));
+        }
+        if (c != 0 && (c < ADMIT_MIN || c >= ADMIT_MIN + 4)) atomicAdd(&s_hist[min(c, 1023u)], 1u);
+    }
+    most = __reduce_max_sync(0xFFFFFFFFu, most);
+    if (lane == 0 && most) atomicMax(&x.most, most);
+    __syncthreads();
+    if (s_hist[t]) atomicAdd(&x.hist[t], s_hist[t]);
+    __syncthreads();
+    if (t == 0) {
+        __threadfence();
+        s_last = atomicAdd(&x.done, 1u) == gridDim.x - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!s_last) return;
+    // smallest threshold >= 2 whose class fits the directory with some over-subscription: thread t looks at the
+    // count 1023 - t, behind a scan over the higher ones
+    const uint32_t budget = min(p.hot_slots + p.hot_slots / 4, HOT_SELECT_MAX);
+    uint32_t incl = __ldcg(&x.hist[1023 - t]);
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+        if (lane >= (uint32_t)d) incl += o;
+    }
+    if (lane == 31) s_warp[w] = incl;
+    __syncthreads();
+    if (w == 0) {
+        uint32_t v = s_warp[lane];
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, v, d);
+            if (lane >= (uint32_t)d) v += o;
+        }
+        s_warp[lane] = v;
+    }
+    __syncthreads();
+    incl += w ? s_warp[w - 1] : 0u;
+    const int above = __syncthreads_count(t <= 1021 && incl <= budget);   // counts 1023, 1022, ... that fit
+    if (t == 0) {
+        x.threshold = 1024u - (uint32_t)above;
+        // a key holding more than 1/32 of the sample makes same-slot collisions inside a warp
+        // common: tell the scatter pass to combine equal lanes first
+        p.ctl->hot_skew = ((ull)__ldcg(&x.most) * 32u >= p.n_sample) ? 1ull : 0ull;
     }
 }
 
-constexpr uint32_t SELECT_MAX = 14336;  // candidates kept for installation (directory <= 11.6K slots, x1.25)
-constexpr uint32_t OCC_MAX = 3072;      // directory buckets (<= 11.6K / 4)
-constexpr size_t SELECT_SMEM = (size_t)SELECT_MAX * 12 + (size_t)OCC_MAX * 4;
-
-__global__ void __launch_bounds__(1024, 1) hot_select_kernel(HotBuildParams p) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    ull* c_key = reinterpret_cast<ull*>(smem_raw);                        // [SELECT_MAX]
-    uint32_t* c_cnt = reinterpret_cast<uint32_t*>(c_key + SELECT_MAX);    // [SELECT_MAX]
-    __shared__ uint32_t hist[1024];
-    __shared__ uint32_t s_thr, s_inserted, s_max, s_n;
-    const uint32_t n_cand = 1u << p.cand_bits;
-    hist[threadIdx.x] = 0;
-    for (uint32_t i = threadIdx.x; i < p.hot_slots; i += blockDim.x) p.hot_keys[i] = 0;
-    if (threadIdx.x == 0) s_inserted = s_max = s_n = 0;
-    __syncthreads();
-    // one CTA walks the candidate table: eight independent loads per thread at a time, or the scan
-    // is a chain of dependent memory round trips
-    constexpr int SCAN_ILP = 8;
-    for (uint32_t i0 = threadIdx.x; i0 < n_cand; i0 += SCAN_ILP * blockDim.x) {
-        uint32_t c[SCAN_ILP];
-#pragma unroll
-        for (int u = 0; u < SCAN_ILP; ++u) c[u] = i0 + u * blockDim.x < n_cand ? p.cand_cnt[i0 + u * blockDim.x] : 0u;
-#pragma unroll
-        for (int u = 0; u < SCAN_ILP; ++u) {
-            if (c[u] != 0) atomicAdd(&hist[min(c[u], 1023u)], 1u);
-            if (c[u] >= 1023u) atomicMax(&s_max, c[u]);
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        // smallest threshold >= 2 whose class fits the directory with some over-subscription
-        uint32_t budget = min(p.hot_slots + p.hot_slots / 4, SELECT_MAX), cum = 0, thr = 1024;
-        for (int c = 1023; c >= 2; --c) {
-            if (cum + hist[c] > budget) break;
-            cum += hist[c];
-            thr = (uint32_t)c;
-        }
-        s_thr = thr;
-        // a key holding more than 1/32 of the sample makes same-slot collisions inside a warp
-        // common: tell the scatter pass to combine equal lanes first
-        p.ctl->hot_skew = ((ull)s_max * 32u >= p.n_sample) ? 1ull : 0ull;
-    }
-    __syncthreads();
-    const uint32_t thr = s_thr;
-    // compact the selected candidates into shared memory, then install them class by class
-    for (uint32_t i0 = threadIdx.x; i0 < n_cand; i0 += SCAN_ILP * blockDim.x) {
-        uint32_t c[SCAN_ILP];
-        ull k[SCAN_ILP];
-#pragma unroll
-        for (int u = 0; u < SCAN_ILP; ++u) c[u] = i0 + u * blockDim.x < n_cand ? p.cand_cnt[i0 + u * blockDim.x] : 0u;
-#pragma unroll
-        for (int u = 0; u < SCAN_ILP; ++u) k[u] = c[u] >= thr ? p.cand_keys[i0 + u * blockDim.x] : 0ull;
-#pragma unroll
-        for (int u = 0; u < SCAN_ILP; ++u) {
-            if (c[u] >= thr) {
-                uint32_t at = atomicAdd(&s_n, 1u);
-                if (at < SELECT_MAX) {
-                    c_key[at] = k[u];
-                    c_cnt[at] = c[u];
-                }
-            }
-        }
-    }
-    __syncthreads();
-    const uint32_t n_sel = min(s_n, SELECT_MAX);
-    // pick the bucket-hash multiplier that loses the least sampled weight: a key is lost when
-    // its bucket's slots are already taken (approximated by arrival order among the keys that
-    // matter, which is close to what the class-ordered installation below does)
+// A multiplier's loss is approximated by arrival order among the keys that matter.
+__global__ void __launch_bounds__(256) hot_gather_kernel(HotBuildParams p) {
     __shared__ uint32_t s_lost[4];
-    uint32_t* occupancy = c_cnt + SELECT_MAX;  // [OCC_MAX] bucket counters behind the compact lists
-    const uint32_t n_buckets = p.hot_slots / DIR_WAYS;
     if (threadIdx.x < 4) s_lost[threadIdx.x] = 0;
-    for (uint32_t m = 0; m < 4; ++m) {
-        for (uint32_t i = threadIdx.x; i < n_buckets; i += blockDim.x) occupancy[i] = 0;
-        __syncthreads();
-        for (uint32_t i = threadIdx.x; i < n_sel; i += blockDim.x) {
-            uint32_t c = c_cnt[i];
-            if (c < 16) continue;
-            uint32_t b = dir_bucket_of_key(~c_key[i], DIR_MULTS[m], n_buckets);
-            if (atomicAdd(&occupancy[b], 1u) >= DIR_WAYS) atomicAdd(&s_lost[m], c);
+    __syncthreads();
+    grid_dependency_wait();
+    HotBuildScratch& x = *p.scratch;
+    const uint32_t thr = x.threshold, n_buckets = p.hot_slots / DIR_WAYS, lane = threadIdx.x & 31u;
+    const uint32_t i = blockIdx.x * 256 + threadIdx.x;      // (grid: one thread per candidate)
+    const uint32_t c = p.cand_cnt[i];
+    const uint32_t votes = __ballot_sync(0xFFFFFFFFu, c >= thr);
+    uint32_t base = 0;
+    if (lane == 0 && votes) base = atomicAdd(&x.n, (uint32_t)__popc(votes));
+    base = __shfl_sync(0xFFFFFFFFu, base, 0);
+    if (c >= thr) {
+        const uint32_t at = base + __popc(votes & ((1u << lane) - 1u));
+        const ull skey = p.cand_keys[i];
+        if (at < HOT_SELECT_MAX) {
+            x.key[at] = skey;
+            x.count[at] = c;
         }
-        __syncthreads();
+        if (c >= 16) {
+#pragma unroll
+            for (uint32_t m = 0; m < 4; ++m)
+                if (atomicAdd(&x.occupancy[m][dir_bucket_of_key(~skey, DIR_MULTS[m], n_buckets)], 1u) >= DIR_WAYS) atomicAdd(&s_lost[m], c);
+        }
     }
-    if (threadIdx.x == 0) {
-        uint32_t best = 0;
-        for (uint32_t m = 1; m < 4; ++m)
-            if (s_lost[m] < s_lost[best]) best = m;
-        p.ctl->dir_mult = DIR_MULTS[best];
-        s_thr = DIR_MULTS[best];  // broadcast (the threshold is already in registers)
+    grid_dependents_launch();
+    __syncthreads();
+    if (threadIdx.x < 4 && s_lost[threadIdx.x]) atomicAdd(&x.lost[threadIdx.x], s_lost[threadIdx.x]);
+}
+
+__device__ __forceinline__ uint32_t best_multiplier(const HotBuildScratch& x) {
+    uint32_t best = 0;
+#pragma unroll
+    for (uint32_t m = 1; m < 4; ++m)
+        if (x.lost[m] < x.lost[best]) best = m;
+    return DIR_MULTS[best];
+}
+
+__global__ void __launch_bounds__(256) hot_list_kernel(HotBuildParams p) {
+    grid_dependency_wait();
+    HotBuildScratch& x = *p.scratch;
+    const uint32_t i = blockIdx.x * 256 + threadIdx.x;
+    if (i < min(x.n, HOT_SELECT_MAX)) {
+        const uint32_t b = dir_bucket_of_key(~x.key[i], best_multiplier(x), p.hot_slots / DIR_WAYS);
+        const uint32_t at = atomicAdd(&x.listed[b], 1u);
+        if (at < LIST_MAX) x.list[b][at] = i;
     }
+    grid_dependents_launch();
+}
+
+__global__ void __launch_bounds__(128) hot_pick_kernel(HotBuildParams p) {
+    __shared__ uint32_t s_inserted;
+    if (threadIdx.x == 0) s_inserted = 0;
     __syncthreads();
-    const uint32_t mult = s_thr;
-    for (uint32_t i = threadIdx.x; i < n_buckets; i += blockDim.x) occupancy[i] = 0;
-    __syncthreads();
-    // install from the most to the least frequent class (counts within a class differ < 2x), so
-    // that a key can only lose its bucket to keys about as frequent as itself; a bucket's ways are
-    // handed out by its shared-memory counter
-    for (int round = 0; round < 11; ++round) {
-        uint32_t hi = round == 0 ? 0xFFFFFFFFu : (2048u >> round), lo = max(1024u >> round, thr);
-        if (lo < hi) {
-            for (uint32_t i = threadIdx.x; i < n_sel; i += blockDim.x) {
-                uint32_t c = c_cnt[i];
-                if (c >= lo && c < hi) {
-                    ull skey = c_key[i];
-                    const uint32_t b = dir_bucket_of_key(~skey, mult, n_buckets);
-                    const uint32_t way = atomicAdd(&occupancy[b], 1u);
-                    if (way < DIR_WAYS) {
-                        p.hot_keys[b * DIR_WAYS + way] = skey;
-                        atomicAdd(&s_inserted, 1u);
-                    }
+    grid_dependency_wait();
+    HotBuildScratch& x = *p.scratch;
+    const uint32_t b = blockIdx.x * 128 + threadIdx.x;
+    uint32_t inserted = 0;
+    if (b < p.hot_slots / DIR_WAYS) {
+        const uint32_t n = min(x.listed[b], LIST_MAX);
+        uint32_t top[DIR_WAYS] = {0, 0, 0, 0}, who[DIR_WAYS] = {0, 0, 0, 0};
+        for (uint32_t k = 0; k < n; ++k) {
+            uint32_t i = x.list[b][k], c = x.count[i];
+#pragma unroll
+            for (uint32_t way = 0; way < DIR_WAYS; ++way) {   // insertion into the four best
+                if (c > top[way]) {
+                    const uint32_t tc = top[way], ti = who[way];
+                    top[way] = c;
+                    who[way] = i;
+                    c = tc;
+                    i = ti;
                 }
             }
         }
-        __syncthreads();
+        ull keys[DIR_WAYS];
+#pragma unroll
+        for (uint32_t way = 0; way < DIR_WAYS; ++way) {
+            keys[way] = top[way] ? x.key[who[way]] : 0ull;
+            inserted += top[way] ? 1u : 0u;
+        }
+        ulonglong2* dst = reinterpret_cast<ulonglong2*>(p.hot_keys + b * DIR_WAYS);
+        dst[0] = make_ulonglong2(keys[0], keys[1]);
+        dst[1] = make_ulonglong2(keys[2], keys[3]);
+        if (b == 0) p.ctl->dir_mult = best_multiplier(x);
     }
-    if (threadIdx.x == 0) p.ctl->hot_n = s_inserted;
+    inserted = __reduce_add_sync(0xFFFFFFFFu, inserted);
+    if ((threadIdx.x & 31u) == 0 && inserted) atomicAdd(&s_inserted, inserted);
+    __syncthreads();
+    if (threadIdx.x == 0 && s_inserted) atomicAdd(&p.ctl->hot_n, (ull)s_inserted);
 }
 
 // --------------------------------------------------------------------------------------
@@ -695,9 +793,7 @@ cudaError_t ingest_prepare() {
     cudaError_t e = scatter_prepare();
     if (e == cudaSuccess) e = direct_prepare();
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(partition_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448 - 2048);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(hot_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SELECT_SMEM);
+    return cudaFuncSetAttribute(partition_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448 - 2048);
 }
 
 cudaError_t launch_partition(const PartitionParams& q, int n_sms, cudaStream_t stream) {
@@ -708,15 +804,20 @@ cudaError_t launch_partition(const PartitionParams& q, int n_sms, cudaStream_t s
 
 cudaError_t launch_hot_build(const HotBuildParams& p, int n_sms, cudaStream_t stream) {
     // the caller has zeroed the sketch and the candidate table on this stream
-    int grid = (int)((p.n_sample + 255) / 256);
+    int grid = (int)((p.n_sample + 256 * SAMPLE_ILP - 1) / (256 * SAMPLE_ILP));
     if (grid > n_sms * 8) grid = n_sms * 8;
     hot_count_kernel<<<grid, 256, 0, stream>>>(p);
     hot_admit_kernel<<<grid, 256, 0, stream>>>(p);
-    hot_select_kernel<<<1, 1024, SELECT_SMEM, stream>>>(p);
-    return cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
+    const uint32_t n_cand = 1u << p.cand_bits, n_buckets = p.hot_slots / DIR_WAYS;
+    if (e == cudaSuccess) e = launch_chained(hot_level_kernel, n_cand / LEVEL_THREADS, LEVEL_THREADS, 0, stream, p);
+    if (e == cudaSuccess) e = launch_chained(hot_gather_kernel, n_cand / 256, 256, 0, stream, p);
+    if (e == cudaSuccess) e = launch_chained(hot_list_kernel, (HOT_SELECT_MAX + 255) / 256, 256, 0, stream, p);
+    if (e == cudaSuccess) e = launch_chained(hot_pick_kernel, (n_buckets + 127) / 128, 128, 0, stream, p);
+    return e;
 }
 
-cudaError_t launch_hot_fold(const ull* hot_keys, ulonglong2* hot_img, uint32_t n_groups, uint32_t hot_slots,
+cudaError_t launch_hot_fold(const ull* hot_keys, const ulonglong2* hot_img, uint32_t n_groups, uint32_t hot_slots,
                             const TableRef& t, cudaStream_t stream) {
     if (hot_slots == 0) return cudaSuccess;
     hot_fold_kernel<<<(hot_slots + 31) / 32, FOLD_WARPS * 32, 0, stream>>>(hot_keys, hot_img, n_groups, hot_slots, t);

@@ -41,6 +41,7 @@ struct IngestParams {
     const ull* hot_keys;       // directory image, hot_slots entries of ~key (0 = empty)
     uint32_t hot_slots;        // multiple of 4
     uint32_t hot_buckets;      // hot_slots / 4
+    uint32_t img_rows;         // rows of hot_img that hold sums since the last fold; a CTA beyond them starts its row afresh
     ulonglong2* hot_img;       // [n_groups][hot_slots] each CTA's directory sums since the last fold, {lo, count | hi << 40}
     TableRef t;
     // spill buffers: entry i of scatter CTA g for partition p at spill + ((g * P + p) * cap + i) * 12 bytes: an 8-byte
@@ -79,17 +80,34 @@ struct PartitionParams {
     uint32_t queue_cap;
 };
 
+// Scratch of the directory build's last steps (cleared by every build up to `key`).
+constexpr uint32_t HOT_SAMPLE_RUN = 4;       // neighbouring records sampled together
+constexpr uint32_t HOT_SELECT_MAX = 14336;   // candidates kept (directory <= 11.6K slots, x1.25)
+constexpr uint32_t HOT_BUCKETS_MAX = 3072;   // directory buckets (<= 11.6K / 4)
+struct HotBuildScratch {
+    uint32_t n, most, threshold, done;
+    uint32_t lost[4];                            // sampled weight each multiplier would lose
+    uint32_t hist[1024];                         // candidates by count
+    uint32_t occupancy[4][HOT_BUCKETS_MAX];
+    uint32_t listed[HOT_BUCKETS_MAX];
+    ull key[HOT_SELECT_MAX];                     // ~key
+    uint32_t count[HOT_SELECT_MAX];
+    uint32_t list[HOT_BUCKETS_MAX][16];          // candidates of each bucket
+};
+
 struct HotBuildParams {
     const uint4* recs;
-    ull stride;
-    uint32_t n_sample;
+    ull stride;                // records from one run to the next
+    uint32_t n_sample;         // whole runs
     uint32_t n_apps, n_phases;
     ull* hot_keys;
     uint32_t hot_slots;
+    ull* sample;               // [n_sample] the sampled keys, all ones = invalid record
     uint32_t* sketch;          // [2^20] sample counters by hash
     ull* cand_keys;            // [1 << cand_bits] candidate table: ~key, 0 = empty
     uint32_t* cand_cnt;        // [1 << cand_bits] exact sample counts of the candidates
     uint32_t cand_bits;
+    HotBuildScratch* scratch;
     Control* ctl;
 };
 
@@ -174,6 +192,11 @@ inline cudaError_t launch_chained(void (*kernel)(P...), uint32_t grid, uint32_t 
     return cudaLaunchKernelEx(&c, kernel, P(args)...);
 }
 
+// Pinned host memory, visible to the device, that kernels write results to (pinned.cu).  Blocks of up to 512 KB come from
+// a pool of the process, so that creating a handle does not pay for pinning; at most eight wait there.
+cudaError_t pinned_alloc(void** out, size_t bytes);
+void pinned_free(void* block, size_t bytes);
+
 // CTAs of a grid-stride kernel: as many as the SMs hold at once (a second, partly filled wave would cost as
 // much as a full one), fewer when there is less work.  `per_sm` comes from resident_ctas, asked once.
 template <typename K>
@@ -194,7 +217,7 @@ cudaError_t scatter_prepare();
 cudaError_t launch_scatter(const IngestParams& p, bool hot, int grid, cudaStream_t stream);
 cudaError_t launch_partition(const PartitionParams& p, int n_sms, cudaStream_t stream);
 cudaError_t launch_hot_build(const HotBuildParams& p, int n_sms, cudaStream_t stream);
-cudaError_t launch_hot_fold(const ull* hot_keys, ulonglong2* hot_img, uint32_t n_groups, uint32_t hot_slots,
+cudaError_t launch_hot_fold(const ull* hot_keys, const ulonglong2* hot_img, uint32_t n_groups, uint32_t hot_slots,
                             const TableRef& t, cudaStream_t stream);
 cudaError_t launch_merge(const atrex_entry_t* in, ull n, const TableRef& t, cudaStream_t stream);
 

@@ -609,6 +609,7 @@ __global__ void __launch_bounds__(SCATTER_THREADS, 1) scatter_kernel(IngestParam
         // the end of every launch cost 59 us per launch).  hot_fold_kernel adds the rows into the table
         // before results are read.
         ulonglong2* img = p.hot_img + (size_t)blockIdx.x * L::SLOTS;
+        const bool held = blockIdx.x < p.img_rows;   // the row holds earlier launches' sums
         for (uint32_t i0 = threadIdx.x; i0 < L::SLOTS; i0 += 4 * blockDim.x) {  // four slots per thread in flight
             uint32_t cn[4], lo[4], hi[4];
             ulonglong2 o[4];
@@ -621,10 +622,10 @@ __global__ void __launch_bounds__(SCATTER_THREADS, 1) scatter_kernel(IngestParam
                 cn[u] = in ? g_acc[3 * i + 2] : 0u;
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) o[u] = (cn[u] | lo[u] | hi[u]) ? img[i0 + u * blockDim.x] : make_ulonglong2(0, 0);
+            for (int u = 0; u < 4; ++u) o[u] = held && (cn[u] | lo[u] | hi[u]) ? img[i0 + u * blockDim.x] : make_ulonglong2(0, 0);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                if ((cn[u] | lo[u] | hi[u]) == 0) continue;
+                if (i0 + u * blockDim.x >= L::SLOTS || (held && (cn[u] | lo[u] | hi[u]) == 0)) continue;
                 const ull nlo = o[u].x + ((ull)lo[u] | ((ull)hi[u] << 32));
                 img[i0 + u * blockDim.x] = make_ulonglong2(nlo, o[u].y + (ull)cn[u] + ((nlo < o[u].x ? 1ull : 0ull) << HI_SHIFT));
             }
