@@ -124,7 +124,7 @@ void compute_layout(const atrex_agg_config_t* c, size_t smem_optin, int n_sms, L
     L->off_staging[1] = o;     o += STAGING_BYTES;
     L->off_sel = o;            o += round_up((size_t)SEL_CAP * 32 * c->n_phases, ALIGN);   // one region per phase
     L->off_pick = o;           o += round_up((size_t)TOPK_PICK_MAX * 32 * c->n_phases, ALIGN);
-    L->off_hist_all = o;       o += round_up((size_t)ATREX_MAX_PHASES * TOPK_BINS * 4, ALIGN);
+    L->off_hist_all = o;       o += round_up((size_t)2 * c->n_phases * TOPK_BINS * 4, ALIGN);
     L->off_topk_out = o;       o += round_up((size_t)ATREX_MAX_TOPK * sizeof(atrex_entry_t), ALIGN);
     L->off_hot_scratch = o;    o += round_up(HOT_SCRATCH_BYTES, ALIGN);
     L->off_queue = o;          o += round_up((size_t)L->n_groups * L->queue_cap * 16, ALIGN);
@@ -145,12 +145,11 @@ struct DeviceGuard {
 
 }  // namespace
 
-// What ranking requests worked out, kept until the next finalize: the first-digit counts and, for the last k
-// asked for, every phase's answer (in pinned memory).  A phase that could not be answered that way keeps the
+// What ranking requests worked out, kept until the next finalize: for the last k asked for, every phase's answer
+// (in pinned memory).  A phase that could not be answered that way keeps the
 // selection of its last k.
 struct TopkCache {
-    ull hist_gen = 0;                       // finalize generation the counts belong to (0 = none)
-    ull pick_gen = 0;                       // ... and the answers
+    ull pick_gen = 0;                       // finalize generation the answers belong to (0 = none)
     uint32_t k = 0;                         // k of the answers
     ull sel_gen[ATREX_MAX_PHASES] = {};     // the long way, per phase
     uint32_t sel_k[ATREX_MAX_PHASES] = {};
@@ -180,10 +179,11 @@ struct atrex_agg {
     atrex_entry_t* topk_out = nullptr;
     Control* h_ctl = nullptr;  // pinned mirror
     size_t pinned_bytes = 0;
-    uint32_t* hist_all = nullptr;     // [ATREX_MAX_PHASES][TOPK_BINS] first-digit counts of all phases
+    uint32_t* hist_all = nullptr;     // [2][n_phases][TOPK_BINS] first-digit counts: the last totals pass's, and zeros for the next
+    uint32_t hist_at = 0;             // which half is the last pass's
+    ull wait_seq = 0;                 // number of the last kernel that the host waited for
     ull* pick = nullptr;              // [n_phases][TOPK_PICK_MAX][4] candidates
     atrex_entry_t* h_top = nullptr;   // pinned: [n_phases][TOPK_PICK_K] the best k of each phase, then u32 [n_phases] how many
-    bool merged = false;              // entries were folded in since reset: their phases may be any
     TopkCache topk;
     ull fin_gen = 0;                  // bumped by every successful finalize
     bool hot_ready = false;
@@ -333,12 +333,16 @@ int atrex_agg_create(const atrex_agg_config_t* cfg, atrex_agg_t** out) {
         cudaError_t e = cudaSuccess;
         if (e == cudaSuccess) e = cudaMemset(h->ws + L.off_ctl, 0, L.off_appw - L.off_ctl);  // control, spill counts, table, work
         if (e == cudaSuccess) e = cudaMemcpy(h->d_appw, cfg->app_weights, (size_t)cfg->n_apps * 4, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaMemset(h->hist_all, 0, (size_t)2 * cfg->n_phases * TOPK_BINS * 4);
         if (e == cudaSuccess) e = cudaMemset(h->hot_keys, 0, (size_t)(L.hot_slots ? L.hot_slots : 2) * 8);
         // the pinned block: every phase's best, how many there are, the control block's mirror
         const size_t top_bytes = (size_t)cfg->n_phases * (TOPK_PICK_K * sizeof(atrex_entry_t) + 8);
         h->pinned_bytes = top_bytes + sizeof(Control);
         if (e == cudaSuccess) e = pinned_alloc((void**)&h->h_top, h->pinned_bytes);
-        if (e == cudaSuccess) h->h_ctl = (Control*)((unsigned char*)h->h_top + top_bytes);
+        if (e == cudaSuccess) {
+            h->h_ctl = (Control*)((unsigned char*)h->h_top + top_bytes);
+            h->h_ctl->seq = 0;   // (the block may be another handle's former one)
+        }
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking);
         for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
             e = cudaEventCreateWithFlags(&h->ev_ready[i], cudaEventDisableTiming);
@@ -382,7 +386,6 @@ int atrex_agg_reset(atrex_agg_t* h, void* stream) {
     h->spill_pending = false;
     h->hot_ready = false;
     h->finalized = false;
-    h->merged = false;
     h->n_records = 0;
     return ATREX_OK;
 }
@@ -572,7 +575,6 @@ int atrex_agg_merge(atrex_agg_t* h, const atrex_entry_t* d_entries, uint64_t n, 
     if (!d_entries || ((uintptr_t)d_entries & 15u) != 0) return ATREX_ERR_INVALID;
     DeviceGuard guard(h->cfg.device);
     h->finalized = false;
-    h->merged = true;
     CU(h, launch_merge(d_entries, n, h->table_ref(), (cudaStream_t)stream));
     h->launches++;
     return ATREX_OK;
@@ -587,10 +589,11 @@ static int run_totals(atrex_agg* h, const uint64_t* total_lo, const uint64_t* to
         memcpy(given.hi, total_hi, sizeof(given.hi));
         given.use = 1;
     }
-    const uint32_t n_phases = h->merged ? ATREX_MAX_PHASES : h->cfg.n_phases;
-    CU(h, launch_totals(h->table_ref(), h->L.n_slots, n_phases, given, h->hist_all, h->n_sms, s));
+    const uint32_t n_phases = h->cfg.n_phases;
+    h->hist_at ^= 1u;
+    uint32_t* const half[2] = {h->hist_all, h->hist_all + (size_t)n_phases * TOPK_BINS};
+    CU(h, launch_totals(h->table_ref(), h->L.n_slots, n_phases, given, half[h->hist_at], half[h->hist_at ^ 1u], h->n_sms, s));
     h->launches++;
-    h->topk.hist_gen = 0;   // (the counts were cleared)
     return ATREX_OK;
 }
 
@@ -600,6 +603,7 @@ static FinalizeParams finalize_params(const atrex_agg* h, atrex_entry_t* out, ui
     p.n_slots = h->L.n_slots;
     p.ctl = h->ctl;
     p.mirror = h->h_ctl;
+    p.seq = 0;
     p.work = h->work_ref();
     p.peaks = h->peaks;
     p.out = out;
@@ -640,9 +644,13 @@ static int finalize_impl(atrex_agg_t* h, const atrex_hw_peaks_t* peaks, const ui
     if (rc != ATREX_OK) return rc;
     rc = run_totals(h, total_lo, total_hi, s);
     if (rc != ATREX_OK) return rc;
-    CU(h, launch_emit(finalize_params(h, d_out, out_cap), h->n_sms, s));   // (fills the mirror h_ctl)
+    FinalizeParams fin = finalize_params(h, d_out, out_cap);
+    fin.seq = ++h->wait_seq;
+    CU(h, launch_emit(fin, h->n_sms, s));   // (fills the mirror h_ctl)
     h->launches++;
-    CU(h, cudaStreamSynchronize(s));
+    const volatile ull* seq = &h->h_ctl->seq;
+    const ull want = fin.seq;
+    CU(h, wait_for_kernel([=] { return *seq == want; }, s));
     *n_out = h->h_ctl->n_out;
     rc = device_status_to_error(h->h_ctl);
     if (rc != ATREX_OK) return rc;
@@ -737,25 +745,33 @@ int atrex_agg_topk(atrex_agg_t* h, uint32_t phase, uint32_t k, atrex_entry_t* h_
     TopkCache& cache = h->topk;
     if (k <= TOPK_PICK_K) {
         // every phase's answer in one go
-        const volatile uint32_t* answered = (const uint32_t*)(h->h_top + (size_t)h->cfg.n_phases * TOPK_PICK_K);
+        ull* const answers = (ull*)(h->h_top + (size_t)h->cfg.n_phases * TOPK_PICK_K);
         if (cache.pick_gen != h->fin_gen || cache.k != k) {
             PickParams p;
             p.fin = finalize_params(h, nullptr, 0);
+            p.fin.seq = ++h->wait_seq & 0xFFFFFFFFu;
             p.n_phases = h->cfg.n_phases;
             p.k = k;
-            p.hist = h->hist_all;
+            p.hist = h->hist_all + (size_t)h->hist_at * h->cfg.n_phases * TOPK_BINS;
             p.sel = h->pick;
             p.host_top = h->h_top;
-            p.host_n = (uint32_t*)answered;
-            const bool count = cache.hist_gen != h->fin_gen;
+            p.host_n = answers;
             cache.pick_gen = 0;
-            CU(h, launch_topk_pick(p, count, h->n_sms, s));
-            h->launches += count ? 4 : 3;
-            CU(h, cudaStreamSynchronize(s));
-            cache.hist_gen = cache.pick_gen = h->fin_gen;
+            const uint32_t n_phases = p.n_phases;
+            const ull want = p.fin.seq;
+            for (uint32_t q = 0; q < n_phases; ++q) answers[q] = ~(want << 32);
+            CU(h, launch_topk_pick(p, h->n_sms, s));
+            h->launches += 3;
+            const volatile ull* a = answers;
+            CU(h, wait_for_kernel([=] {
+                for (uint32_t q = 0; q < n_phases; ++q)
+                    if (a[q] >> 32 != want) return false;
+                return true;
+            }, s));
+            cache.pick_gen = h->fin_gen;
             cache.k = k;
         }
-        const uint32_t m = answered[phase];
+        const uint32_t m = (uint32_t)((const volatile ull*)answers)[phase];
         if (m != PICK_NONE) {
             memcpy(h_out, h->h_top + (size_t)phase * TOPK_PICK_K, (size_t)m * sizeof(atrex_entry_t));
             *n_out = m;

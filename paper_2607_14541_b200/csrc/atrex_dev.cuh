@@ -60,7 +60,7 @@ struct Control {
     ull n_rejected;
     ull n_dropped;
     ull n_out;                 // entries emitted by the last finalize
-    ull pad0;
+    ull seq;                   // (mirror only) finalize whose results the mirror holds
     ull hot_n;                 // keys in the hot directory
     ull work_status;           // ST_WORK_* bits of the last work-table load
     ull hot_skew;              // 1 if one key dominates the sample: combine equal lanes per warp

@@ -12,7 +12,7 @@
 namespace atrex {
 
 constexpr int FIN_THREADS = 256;
-constexpr int TOT_THREADS = 128;
+constexpr int TOT_THREADS = 256, TOT_ILP = 6;
 
 struct SlotView {
     ull key, count, lo, hi;
@@ -34,11 +34,24 @@ __device__ __forceinline__ SlotView load_slot(const TableRef& t, ull i) {
     return v;
 }
 
+__device__ __forceinline__ uint32_t topk_first_digit(ull lo, ull hi) {
+    if ((lo | hi) == 0) return 0;
+    const int e = hi ? 128 - __clzll((long long)hi) : 64 - __clzll((long long)lo);      // 1 .. 88
+    uint32_t m;
+    if (e > 69) m = (uint32_t)(hi >> (e - 70));
+    else if (e > 64) m = (uint32_t)((hi << (70 - e)) | (lo >> (e - 6)));
+    else m = (uint32_t)(e >= 6 ? lo >> (e - 6) : lo << (6 - e));
+    return ((uint32_t)e << 5) | (m & 31u);
+}
+static_assert((88 << 5) + 31 < TOPK_BINS, "first digits fit the histogram");
+
 // ---- per-phase totals -------------------------------------------------------------------
 // Each thread keeps private per-phase 128-bit sums in its own shared-memory column; columns are added per
 // CTA and folded into accumulators in the control block with a carry-aware pair of atomics.  The last CTA
 // moves the accumulators to their place and clears them (and the emit kernel's output count), so that no
-// launch is spent on clearing; the top-k histogram is cleared on the way.
+// launch is spent on clearing.  On the way the keys are counted by the first digit of the top-k selection (per
+// phase, for topk_plan_kernel), which saves that call a pass over the table; the next pass's counters are
+// cleared here.  Bound by DRAM (566 MB: 120 us).
 __device__ __forceinline__ bool last_cta(ull* done) {
     __shared__ bool s_last;
     __syncthreads();
@@ -51,44 +64,59 @@ __device__ __forceinline__ bool last_cta(ull* done) {
     return s_last;
 }
 
+constexpr size_t totals_smem(uint32_t n_phases) { return (size_t)n_phases * (TOT_THREADS * 28 + TOPK_BINS * 4); }
+
 __global__ void __launch_bounds__(TOT_THREADS) totals_kernel(TableRef tab, ull n_slots, uint32_t n_phases, const __grid_constant__ GivenTotals given,
-                                                             uint32_t* hist) {
+                                                             uint32_t* hist, uint32_t* next_hist) {
     Control* ctl = tab.ctl;
-    __shared__ ull s_lo[ATREX_MAX_PHASES][TOT_THREADS];
-    __shared__ ull s_hi[ATREX_MAX_PHASES][TOT_THREADS];
-    __shared__ ull s_cnt[ATREX_MAX_PHASES][TOT_THREADS];
-    __shared__ uint32_t s_nk[ATREX_MAX_PHASES][TOT_THREADS];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    ull(*s_lo)[TOT_THREADS] = reinterpret_cast<ull(*)[TOT_THREADS]>(smem_raw);       // [n_phases] each
+    ull(*s_hi)[TOT_THREADS] = s_lo + n_phases;
+    ull(*s_cnt)[TOT_THREADS] = s_hi + n_phases;
+    uint32_t(*s_nk)[TOT_THREADS] = reinterpret_cast<uint32_t(*)[TOT_THREADS]>(s_cnt + n_phases);
+    uint32_t* s_hist = reinterpret_cast<uint32_t*>(s_nk + n_phases);                 // [n_phases][TOPK_BINS]
     const int t = threadIdx.x;
     for (uint32_t p = 0; p < n_phases; ++p) {
         s_lo[p][t] = 0; s_hi[p][t] = 0; s_cnt[p][t] = 0; s_nk[p][t] = 0;
     }
+    for (uint32_t i = t; i < n_phases * TOPK_BINS; i += TOT_THREADS) s_hist[i] = 0;
+    __syncthreads();
     grid_dependency_wait();
     for (uint32_t i = blockIdx.x * TOT_THREADS + t; i < n_phases * TOPK_BINS / 4; i += gridDim.x * TOT_THREADS)
-        reinterpret_cast<uint4*>(hist)[i] = make_uint4(0, 0, 0, 0);
-    // four slots per thread in flight: all key loads first, then the values of the live ones
-    constexpr int ILP = 4;
+        reinterpret_cast<uint4*>(next_hist)[i] = make_uint4(0, 0, 0, 0);
+    // six slots per thread in flight
     const ull stride = (ull)gridDim.x * blockDim.x;
-    for (ull i0 = (ull)blockIdx.x * blockDim.x + t; i0 < n_slots; i0 += stride * ILP) {
-        ull sk[ILP];
-        ulonglong2 x[ILP];
+    for (ull i0 = (ull)blockIdx.x * blockDim.x + t; i0 < n_slots; i0 += stride * TOT_ILP) {
+        ull sk[TOT_ILP];
+        ulonglong2 x[TOT_ILP];
 #pragma unroll
-        for (int u = 0; u < ILP; ++u) sk[u] = i0 + u * stride < n_slots ? tab.keys[i0 + u * stride] : 0ull;
+        for (int u = 0; u < TOT_ILP; ++u) sk[u] = i0 + u * stride < n_slots ? tab.keys[i0 + u * stride] : 0ull;
 #pragma unroll
-        for (int u = 0; u < ILP; ++u) x[u] = i0 + u * stride < n_slots ? tab.vals[i0 + u * stride] : make_ulonglong2(0, 0);  // unconditional: no wait for the keys
+        for (int u = 0; u < TOT_ILP; ++u) x[u] = i0 + u * stride < n_slots ? tab.vals[i0 + u * stride] : make_ulonglong2(0, 0);  // unconditional: no wait for the keys
 #pragma unroll
-        for (int u = 0; u < ILP; ++u) {
+        for (int u = 0; u < TOT_ILP; ++u) {
             if (sk[u] == 0) continue;
             const uint32_t p = (uint32_t)(~sk[u] >> 48) & (ATREX_MAX_PHASES - 1);
-            if (p >= n_phases) continue;
+            const ull hi = x[u].y >> HI_SHIFT;
+            if (p >= n_phases) {   // (rare: a merged entry of a phase that records of this handle cannot have)
+                const ull old = atomicAdd(&ctl->acc_lo[p], x[u].x);
+                atomicAdd(&ctl->acc_hi[p], hi + (old + x[u].x < old ? 1ull : 0ull));
+                atomicAdd(&ctl->acc_count[p], x[u].y & COUNT_MASK);
+                atomicAdd(&ctl->acc_keys[p], 1ull);
+                continue;
+            }
             const ull o = s_lo[p][t], n = o + x[u].x;
             s_lo[p][t] = n;
-            s_hi[p][t] += (x[u].y >> HI_SHIFT) + (n < o ? 1ull : 0ull);
+            s_hi[p][t] += hi + (n < o ? 1ull : 0ull);
             s_cnt[p][t] += x[u].y & COUNT_MASK;
             s_nk[p][t] += 1;
+            atomicAdd(&s_hist[p * TOPK_BINS + topk_first_digit(x[u].x, hi)], 1u);
         }
     }
     grid_dependents_launch();
     __syncthreads();
+    for (uint32_t i = t; i < n_phases * TOPK_BINS; i += TOT_THREADS)
+        if (s_hist[i] != 0) atomicAdd(&hist[i], s_hist[i]);
     const uint32_t lane = t & 31;
     for (uint32_t p = t >> 5; p < n_phases; p += TOT_THREADS / 32) {   // a warp per phase
         ull lo = 0, hi = 0, cnt = 0, nk = 0;
@@ -243,8 +271,15 @@ __global__ void __launch_bounds__(FIN_THREADS) emit_kernel(FinalizeParams p) {
     if (!last_cta(&p.ctl->emit_done)) return;
     // the host's copy of the counters and totals, straight to pinned memory
     constexpr uint32_t WORDS = offsetof(Control, acc_lo) / 8;
-    if (threadIdx.x < WORDS) reinterpret_cast<ull*>(p.mirror)[threadIdx.x] = ld_relaxed(reinterpret_cast<const ull*>(p.ctl) + threadIdx.x);
-    if (threadIdx.x == 0) p.ctl->emit_done = 0;
+    constexpr uint32_t SEQ = offsetof(Control, seq) / 8;
+    if (threadIdx.x < WORDS && threadIdx.x != SEQ)
+        reinterpret_cast<ull*>(p.mirror)[threadIdx.x] = ld_relaxed(reinterpret_cast<const ull*>(p.ctl) + threadIdx.x);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        p.ctl->emit_done = 0;
+        __threadfence_system();
+        *(volatile ull*)&p.mirror->seq = p.seq;   // the host waits for this word
+    }
 }
 
 // ---- work table ---------------------------------------------------------------------------
@@ -289,48 +324,7 @@ __global__ void __launch_bounds__(256) work_insert_kernel(const atrex_work_t* ro
 // writes the best k to pinned host memory.  Weights that span orders of magnitude leave a few dozen
 // candidates beside the winners.  (Digits on a linear scale below the phase total's highest bit put every
 // key of a flat trace into the lowest one: 26 000 candidates in one CTA's global-memory sort took 4 ms.)
-__device__ __forceinline__ uint32_t topk_first_digit(ull lo, ull hi) {
-    if ((lo | hi) == 0) return 0;
-    const int e = hi ? 128 - __clzll((long long)hi) : 64 - __clzll((long long)lo);      // 1 .. 88
-    uint32_t m;
-    if (e > 69) m = (uint32_t)(hi >> (e - 70));
-    else if (e > 64) m = (uint32_t)((hi << (70 - e)) | (lo >> (e - 6)));
-    else m = (uint32_t)(e >= 6 ? lo >> (e - 6) : lo << (6 - e));
-    return ((uint32_t)e << 5) | (m & 31u);
-}
-static_assert((88 << 5) + 31 < TOPK_BINS, "first digits fit the histogram");
-
 constexpr int PICK_THREADS = 1024;
-
-// first-digit counts of every phase
-__global__ void __launch_bounds__(PICK_THREADS) topk_count_kernel(const __grid_constant__ PickParams p) {
-    extern __shared__ uint32_t s_hist[];  // [n_phases][TOPK_BINS]
-    for (uint32_t i = threadIdx.x; i < p.n_phases * TOPK_BINS; i += PICK_THREADS) s_hist[i] = 0;
-    __syncthreads();
-    grid_dependency_wait();
-    const TableRef& tab = p.fin.t;
-    constexpr int ILP = 4;
-    const ull stride = (ull)gridDim.x * PICK_THREADS, n_slots = p.fin.n_slots;
-    for (ull i0 = (ull)blockIdx.x * PICK_THREADS + threadIdx.x; i0 < n_slots; i0 += stride * ILP) {
-        ull sk[ILP];
-        ulonglong2 x[ILP];
-#pragma unroll
-        for (int u = 0; u < ILP; ++u) {
-            const ull i = i0 + u * stride;
-            sk[u] = i < n_slots ? tab.keys[i] : 0ull;
-            x[u] = i < n_slots ? tab.vals[i] : make_ulonglong2(0, 0);  // no wait for the keys
-        }
-#pragma unroll
-        for (int u = 0; u < ILP; ++u) {
-            const uint32_t q = (uint32_t)(~sk[u] >> 48) & (ATREX_MAX_PHASES - 1);
-            if (sk[u] != 0 && q < p.n_phases) atomicAdd(&s_hist[q * TOPK_BINS + topk_first_digit(x[u].x, x[u].y >> HI_SHIFT)], 1u);
-        }
-    }
-    grid_dependents_launch();
-    __syncthreads();
-    for (uint32_t i = threadIdx.x; i < p.n_phases * TOPK_BINS; i += PICK_THREADS)
-        if (s_hist[i] != 0) atomicAdd(&p.hist[i], s_hist[i]);
-}
 
 // the digit of each phase's k-th key (one CTA per phase)
 __global__ void __launch_bounds__(PICK_THREADS) topk_plan_kernel(const __grid_constant__ PickParams p) {
@@ -421,7 +415,7 @@ __global__ void __launch_bounds__(512) topk_rank_kernel(const __grid_constant__ 
     grid_dependency_wait();
     const uint32_t q = blockIdx.x;
     if (p.fin.ctl->pick_bin[q] == PICK_NONE) {
-        if (threadIdx.x == 0) p.host_n[q] = PICK_NONE;
+        if (threadIdx.x == 0) *(volatile ull*)&p.host_n[q] = p.fin.seq << 32 | PICK_NONE;
         return;
     }
     load_phase_totals(p.fin.ctl, dT, zeroT);
@@ -469,7 +463,11 @@ __global__ void __launch_bounds__(512) topk_rank_kernel(const __grid_constant__ 
         }
         for (uint32_t i = threadIdx.x; i < min(n, p.k); i += blockDim.x) emit(i, i);
     }
-    if (threadIdx.x == 0) p.host_n[q] = min(n, p.k);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence_system();
+        *(volatile ull*)&p.host_n[q] = p.fin.seq << 32 | min(n, p.k);   // the host waits for this word
+    }
 }
 
 // ---- top-k, the long way ------------------------------------------------------------------
@@ -618,16 +616,18 @@ __global__ void __launch_bounds__(FIN_THREADS) topk_emit_kernel(FinalizeParams p
 constexpr size_t PICK_SMEM = (size_t)TOPK_PICK_MAX * 28;
 
 cudaError_t finalize_prepare() {
-    cudaError_t e = cudaFuncSetAttribute(topk_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(ATREX_MAX_PHASES * TOPK_BINS * sizeof(uint32_t)));
+    cudaError_t e = cudaFuncSetAttribute(totals_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)totals_smem(ATREX_MAX_PHASES));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(topk_rank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PICK_SMEM);
     return e;
 }
 
-cudaError_t launch_totals(const TableRef& t, ull n_slots, uint32_t n_phases, const GivenTotals& given, uint32_t* hist, int n_sms,
-                          cudaStream_t stream) {
-    static const uint32_t per_sm = resident_ctas(totals_kernel, TOT_THREADS, 0);
-    return launch_chained(totals_kernel, grid_for_work(n_slots, TOT_THREADS * 8, n_sms, per_sm), TOT_THREADS, 0, stream, t, n_slots, n_phases, given, hist);
+cudaError_t launch_totals(const TableRef& t, ull n_slots, uint32_t n_phases, const GivenTotals& given, uint32_t* hist, uint32_t* next_hist,
+                          int n_sms, cudaStream_t stream) {
+    const size_t smem = totals_smem(n_phases);
+    uint32_t per_sm = (uint32_t)(233472 / (smem + 1024));
+    if (per_sm > 4) per_sm = 4;
+    return launch_chained(totals_kernel, grid_for_work(n_slots, TOT_THREADS * TOT_ILP, n_sms, per_sm), TOT_THREADS, smem, stream, t, n_slots,
+                          n_phases, given, hist, next_hist);
 }
 
 cudaError_t launch_emit(const FinalizeParams& p, int n_sms, cudaStream_t stream) {
@@ -641,11 +641,9 @@ cudaError_t launch_work_insert(const atrex_work_t* rows, ull n, const WorkRef& w
     return cudaGetLastError();
 }
 
-cudaError_t launch_topk_pick(const PickParams& p, bool count, int n_sms, cudaStream_t stream) {
+cudaError_t launch_topk_pick(const PickParams& p, int n_sms, cudaStream_t stream) {
     static const uint32_t per_sm = resident_ctas(topk_collect_kernel, FIN_THREADS, 0);
-    cudaError_t e = cudaSuccess;
-    if (count) e = launch_chained(topk_count_kernel, grid_for_work(p.fin.n_slots, PICK_THREADS * 4, n_sms, 1), PICK_THREADS, p.n_phases * TOPK_BINS * sizeof(uint32_t), stream, p);
-    if (e == cudaSuccess) e = launch_chained(topk_plan_kernel, p.n_phases, PICK_THREADS, 0, stream, p);
+    cudaError_t e = launch_chained(topk_plan_kernel, p.n_phases, PICK_THREADS, 0, stream, p);
     if (e == cudaSuccess) e = launch_chained(topk_collect_kernel, grid_for_work(p.fin.n_slots, FIN_THREADS * 4, n_sms, per_sm), FIN_THREADS, 0, stream, p);
     if (e == cudaSuccess) e = launch_chained(topk_rank_kernel, p.n_phases, 512, PICK_SMEM, stream, p);
     return e;

@@ -1,5 +1,8 @@
 // Kernel parameter blocks and host-side launchers (internal to the library).
 #pragma once
+#include <atomic>
+#include <chrono>
+
 #include "atrex_dev.cuh"
 
 namespace atrex {
@@ -122,7 +125,8 @@ struct FinalizeParams {
     TableRef t;
     ull n_slots;
     Control* ctl;
-    Control* mirror;     // pinned host memory, filled by the emit kernel
+    Control* mirror;     // pinned host memory, filled by the emit kernel, `seq` last
+    ull seq;
     WorkRef work;
     atrex_hw_peaks_t peaks;
     atrex_entry_t* out;
@@ -141,7 +145,7 @@ struct PickParams {
     uint32_t* hist;            // [n_phases][TOPK_BINS] first-digit counts
     ull* sel;                  // [n_phases][TOPK_PICK_MAX][4]
     atrex_entry_t* host_top;   // pinned: [n_phases][TOPK_PICK_K]
-    uint32_t* host_n;          // pinned: [n_phases] entries written, PICK_NONE = not answered this way
+    ull* host_n;               // pinned: [n_phases] fin.seq << 32 | entries written (PICK_NONE: not answered this way)
 };
 
 struct TopkParams {
@@ -197,6 +201,21 @@ inline cudaError_t launch_chained(void (*kernel)(P...), uint32_t grid, uint32_t 
 cudaError_t pinned_alloc(void** out, size_t bytes);
 void pinned_free(void* block, size_t bytes);
 
+// Waits until `done()` sees what a kernel on `s` wrote to pinned memory as its last act, which the host notices
+// several microseconds before the stream counts as idle; after a millisecond, or if the kernel cannot get there,
+// by the stream itself.
+template <typename Done>
+inline cudaError_t wait_for_kernel(Done done, cudaStream_t s) {
+    const auto limit = std::chrono::steady_clock::now() + std::chrono::milliseconds(1);
+    for (uint32_t i = 1;; ++i) {
+        if (done()) {
+            std::atomic_thread_fence(std::memory_order_acquire);
+            return cudaSuccess;
+        }
+        if ((i & 63u) == 0 && std::chrono::steady_clock::now() > limit) return cudaStreamSynchronize(s);
+    }
+}
+
 // CTAs of a grid-stride kernel: as many as the SMs hold at once (a second, partly filled wave would cost as
 // much as a full one), fewer when there is less work.  `per_sm` comes from resident_ctas, asked once.
 template <typename K>
@@ -222,12 +241,12 @@ cudaError_t launch_hot_fold(const ull* hot_keys, const ulonglong2* hot_img, uint
 cudaError_t launch_merge(const atrex_entry_t* in, ull n, const TableRef& t, cudaStream_t stream);
 
 cudaError_t finalize_prepare();
-cudaError_t launch_totals(const TableRef& t, ull n_slots, uint32_t n_phases, const GivenTotals& given, uint32_t* hist, int n_sms,
+cudaError_t launch_totals(const TableRef& t, ull n_slots, uint32_t n_phases, const GivenTotals& given, uint32_t* hist, uint32_t* next_hist, int n_sms,
                           cudaStream_t stream);
 cudaError_t launch_emit(const FinalizeParams& p, int n_sms, cudaStream_t stream);
 cudaError_t launch_work_insert(const atrex_work_t* rows, ull n, const WorkRef& w, Control* ctl, int grid,
                                cudaStream_t stream);
-cudaError_t launch_topk_pick(const PickParams& p, bool count, int n_sms, cudaStream_t stream);
+cudaError_t launch_topk_pick(const PickParams& p, int n_sms, cudaStream_t stream);
 cudaError_t launch_topk_collect_all(const TopkAllParams& p, int grid, cudaStream_t stream);
 cudaError_t launch_topk_hist(const TopkParams& p, int grid, cudaStream_t stream);
 cudaError_t launch_topk_sort(ull* sel, uint32_t n_pow2, cudaStream_t stream);
