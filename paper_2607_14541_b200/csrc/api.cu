@@ -474,6 +474,7 @@ static int ingest_launch(atrex_agg* h, const atrex_record_t* recs, uint64_t n, c
         b.n_phases = h->cfg.n_phases;
         b.hot_keys = h->hot_keys;
         b.hot_slots = h->L.hot_slots;
+        b.dominated_slots = scatter_dominated_slots(h->L.lp);
         b.ctl = h->ctl;
         b.sketch = (uint32_t*)h->hot_scratch;
         b.sample = (ull*)(h->hot_scratch + HOT_SAMPLE_OFF);

@@ -54,6 +54,9 @@ constexpr uint32_t TOPK_CAND_CAP = 65536;
 constexpr uint32_t TOPK_PICK_MAX = 2048;     // candidates of a phase that one CTA ranks in shared memory
 constexpr uint32_t TOPK_PICK_K = 1024;       // ... and the largest k answered that way
 constexpr uint32_t PICK_NONE = 0xFFFFFFFFu;
+// How much of the sample the most frequent key holds: same-slot collisions inside a warp are common from 1/32 on
+// (equal lanes are then combined first); from 3/8 on the key is best taken out before anything else.
+constexpr ull SKEW_NONE = 0, SKEW_COMBINE = 1, SKEW_DOMINATED = 2;
 
 struct Control {
     ull status;
@@ -63,7 +66,8 @@ struct Control {
     ull seq;                   // (mirror only) finalize whose results the mirror holds
     ull hot_n;                 // keys in the hot directory
     ull work_status;           // ST_WORK_* bits of the last work-table load
-    ull hot_skew;              // 1 if one key dominates the sample: combine equal lanes per warp
+    ull hot_skew;              // SKEW_*: how the scatter pass deals with the most frequent key
+    ull top_key;               // the most frequent key (SKEW_DOMINATED)
     ull n_spilled;             // records routed through the spill buffers
     ull n_overflow;            // records that found their spill buffer full (slow exact path)
     ull drain_seq;             // sequence number of the last scatter launch that asked for a drain

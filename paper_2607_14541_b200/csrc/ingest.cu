@@ -651,7 +651,10 @@ __global__ void __launch_bounds__(LEVEL_THREADS) hot_level_kernel(HotBuildParams
     if (!s_last) return;
     // smallest threshold >= 2 whose class fits the directory with some over-subscription: thread t looks at the
     // count 1023 - t, behind a scan over the higher ones
-    const uint32_t budget = min(p.hot_slots + p.hot_slots / 4, HOT_SELECT_MAX);
+    const ull most_seen = __ldcg(&x.most);
+    const ull skew = most_seen * 8u >= p.n_sample * 3ull ? SKEW_DOMINATED : (most_seen * 32u >= p.n_sample ? SKEW_COMBINE : SKEW_NONE);
+    const uint32_t slots = skew == SKEW_DOMINATED ? p.dominated_slots : p.hot_slots;
+    const uint32_t budget = min(slots + slots / 4, HOT_SELECT_MAX);
     uint32_t incl = __ldcg(&x.hist[1023 - t]);
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -674,10 +677,12 @@ __global__ void __launch_bounds__(LEVEL_THREADS) hot_level_kernel(HotBuildParams
     const int above = __syncthreads_count(t <= 1021 && incl <= budget);   // counts 1023, 1022, ... that fit
     if (t == 0) {
         x.threshold = 1024u - (uint32_t)above;
-        // a key holding more than 1/32 of the sample makes same-slot collisions inside a warp
-        // common: tell the scatter pass to combine equal lanes first
-        p.ctl->hot_skew = ((ull)__ldcg(&x.most) * 32u >= p.n_sample) ? 1ull : 0ull;
+        p.ctl->hot_skew = skew;
     }
+}
+
+__device__ __forceinline__ uint32_t buckets_in_use(const HotBuildParams& p) {
+    return (p.ctl->hot_skew == SKEW_DOMINATED ? p.dominated_slots : p.hot_slots) / DIR_WAYS;
 }
 
 // A multiplier's loss is approximated by arrival order among the keys that matter.
@@ -687,7 +692,7 @@ __global__ void __launch_bounds__(256) hot_gather_kernel(HotBuildParams p) {
     __syncthreads();
     grid_dependency_wait();
     HotBuildScratch& x = *p.scratch;
-    const uint32_t thr = x.threshold, n_buckets = p.hot_slots / DIR_WAYS, lane = threadIdx.x & 31u;
+    const uint32_t thr = x.threshold, n_buckets = buckets_in_use(p), lane = threadIdx.x & 31u;
     const uint32_t i = blockIdx.x * 256 + threadIdx.x;      // (grid: one thread per candidate)
     const uint32_t c = p.cand_cnt[i];
     const uint32_t votes = __ballot_sync(0xFFFFFFFFu, c >= thr);
@@ -701,6 +706,7 @@ __global__ void __launch_bounds__(256) hot_gather_kernel(HotBuildParams p) {
             x.key[at] = skey;
             x.count[at] = c;
         }
+        if (c == x.most) p.ctl->top_key = ~skey;   // (of several equally frequent ones, any)
         if (c >= 16) {
 #pragma unroll
             for (uint32_t m = 0; m < 4; ++m)
@@ -725,7 +731,7 @@ __global__ void __launch_bounds__(256) hot_list_kernel(HotBuildParams p) {
     HotBuildScratch& x = *p.scratch;
     const uint32_t i = blockIdx.x * 256 + threadIdx.x;
     if (i < min(x.n, HOT_SELECT_MAX)) {
-        const uint32_t b = dir_bucket_of_key(~x.key[i], best_multiplier(x), p.hot_slots / DIR_WAYS);
+        const uint32_t b = dir_bucket_of_key(~x.key[i], best_multiplier(x), buckets_in_use(p));
         const uint32_t at = atomicAdd(&x.listed[b], 1u);
         if (at < LIST_MAX) x.list[b][at] = i;
     }

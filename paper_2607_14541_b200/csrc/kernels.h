@@ -30,6 +30,11 @@ constexpr uint32_t scatter_fixed_bytes(uint32_t lp) {
 }
 constexpr uint32_t scatter_hot_slots(uint32_t lp) { return ((SCATTER_SMEM_BYTES - scatter_fixed_bytes(lp)) / 21u) & ~31u; }
 
+// Where one key dominates the trace, the last part of the accumulators holds the warps' queues instead (64 records
+// each), and the directory is that much smaller.
+constexpr uint32_t SCATTER_QUEUE = 64, SCATTER_QUEUE_BYTES = 32 * SCATTER_QUEUE * 16;
+constexpr uint32_t scatter_dominated_slots(uint32_t lp) { return ((scatter_hot_slots(lp) * 12u - SCATTER_QUEUE_BYTES - 16u) / 12u) & ~31u; }
+
 struct IngestParams {
     const void* recs;          // all records of this launch (16-byte aligned) ...
     ull n_recs;
@@ -105,6 +110,7 @@ struct HotBuildParams {
     uint32_t n_apps, n_phases;
     ull* hot_keys;
     uint32_t hot_slots;
+    uint32_t dominated_slots;  // slots in use when one key dominates
     ull* sample;               // [n_sample] the sampled keys, all ones = invalid record
     uint32_t* sketch;          // [2^20] sample counters by hash
     ull* cand_keys;            // [1 << cand_bits] candidate table: ~key, 0 = empty

@@ -45,6 +45,12 @@ struct Smem {
     static constexpr uint32_t KEYS = (TAG + 4u * (NB + 1u) + 7u) & ~7u;   // ull[SLOTS + 4]  key, all ones = empty
     static constexpr uint32_t ACC = KEYS + 8u * (SLOTS + DIR_WAYS);       // {u32 lo, u32 hi, u32 count}[SLOTS + 4]
     static constexpr uint32_t TOTAL = ACC + 12u * (SLOTS + DIR_WAYS);
+    // one key dominates: fewer slots in use, the warps' queues behind them
+    static constexpr uint32_t SLOTS_DOM = scatter_dominated_slots(LP), NB_DOM = SLOTS_DOM / DIR_WAYS;
+    static constexpr uint32_t QUEUE = (ACC + 12u * SLOTS_DOM + 15u) & ~15u;   // uint4[32 warps][SCATTER_QUEUE]
+    static_assert(QUEUE + SCATTER_QUEUE_BYTES <= TOTAL, "queues");
+    template <ull SKEW>
+    static constexpr uint32_t NB_OF = SKEW == SKEW_DOMINATED ? NB_DOM : NB;
     static_assert(TOTAL <= SCATTER_SMEM_BYTES, "scatter pass shared memory");
     static_assert(SLOTS % 32 == 0, "whole buckets");
 };
@@ -187,7 +193,7 @@ __device__ __forceinline__ void spill_append(const IngestParams& p, Ctx& c, bool
 
 // One record, start to finish (the register-staged loop has no registers to spare for working on
 // two records at once).  Called by all lanes of a warp together (absent records masked by `present`).
-template <uint32_t LP, bool HOT, bool DEDUPE, bool FULL>
+template <uint32_t LP, bool HOT, ull SKEW, bool FULL>
 __device__ __forceinline__ void one_record(const IngestParams& p, Ctx& c, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3,
                                            bool present) {
     using L = Smem<LP>;
@@ -213,13 +219,13 @@ __device__ __forceinline__ void one_record(const IngestParams& p, Ctx& c, uint32
         // 8-byte key.  A wrong tag match (1 in 64 look-ups) fails the confirmation and the record takes
         // the spill path: slower, still exact.
         const uint32_t x = dir_mix(h, khi >> 16, c.mult);
-        const uint32_t b = ATREX_INDEX(__umulhi(x, L::NB), L::NB, p.t.ctl);
+        const uint32_t b = ATREX_INDEX(__umulhi(x, L::template NB_OF<SKEW>), L::template NB_OF<SKEW>, p.t.ctl);
         const uint32_t t = lds_u32(c.sb + L::TAG + b * 4u) ^ __byte_perm(x, 0, 0);   // 0 in the bytes that match
         const uint32_t m = (t - 0x01010101u) & ~t & 0x80808080u;                      // lowest flagged byte is exact
         const uint32_t at = ATREX_INDEX(b * DIR_WAYS + ((uint32_t)__clz((int)__brev(m)) >> 3), L::SLOTS + DIR_WAYS, p.t.ctl);
         bool hit = todo && m != 0 && lds_u64(c.sb + L::KEYS + at * 8u) == key;
-        if (DEDUPE) {
-            // one key dominates the trace: combine the lanes that share the first hitting lane's slot
+        if (SKEW != SKEW_NONE) {
+            // a key is frequent enough for collisions inside a warp: combine the lanes that share the first hitting lane's slot
             const unsigned hits = __ballot_sync(0xFFFFFFFFu, hit);
             if (hits != 0) {
                 const int lead = __ffs(hits) - 1;
@@ -248,7 +254,7 @@ __device__ __forceinline__ void one_record(const IngestParams& p, Ctx& c, uint32
 // registers allow it; w[r] = the record's four words).  Called by all lanes of a
 // warp together (absent records masked by `present`).  Written in stages over the R records so that
 // their shared-memory round trips overlap: all look-ups are issued before the first result is used.
-template <uint32_t LP, bool HOT, bool DEDUPE, bool FULL, int R>
+template <uint32_t LP, bool HOT, ull SKEW, bool FULL, int R>
 __device__ __forceinline__ void process(const IngestParams& p, Ctx& c, const uint32_t (&w)[R][4], bool present) {
     using L = Smem<LP>;
     uint32_t khi[R], h[R], wgt[R], x[R], tags[R];
@@ -268,7 +274,7 @@ __device__ __forceinline__ void process(const IngestParams& p, Ctx& c, const uin
             // Directory look-up: one 32-bit word per 4-slot bucket holds an 8-bit tag per slot (hash
             // bits the bucket choice does not use)
             x[r] = dir_mix(h[r], khi[r] >> 16, c.mult);
-            tags[r] = lds_u32(c.sb + L::TAG + __umulhi(x[r], L::NB) * 4u);
+            tags[r] = lds_u32(c.sb + L::TAG + __umulhi(x[r], L::template NB_OF<SKEW>) * 4u);
         }
     }
     ull prod[R];
@@ -283,7 +289,7 @@ __device__ __forceinline__ void process(const IngestParams& p, Ctx& c, const uin
             // still exact
             const uint32_t t = tags[r] ^ __byte_perm(x[r], 0, 0);                     // 0 in the bytes that match
             const uint32_t m = (t - 0x01010101u) & ~t & 0x80808080u;                  // lowest flagged byte is exact
-            at[r] = __umulhi(x[r], L::NB) * DIR_WAYS + ((uint32_t)__clz((int)__brev(m)) >> 3);
+            at[r] = __umulhi(x[r], L::template NB_OF<SKEW>) * DIR_WAYS + ((uint32_t)__clz((int)__brev(m)) >> 3);
             found[r] = ~0ull;
             if (m != 0) found[r] = lds_u64(c.sb + L::KEYS + at[r] * 8u);
         }
@@ -300,8 +306,8 @@ __device__ __forceinline__ void process(const IngestParams& p, Ctx& c, const uin
         }
         hit[r] = HOT && todo[r] && found[r] == key;
     }
-    if (HOT && DEDUPE) {
-        // one key dominates the trace: combine the lanes that share the first hitting lane's slot
+    if (HOT && SKEW != SKEW_NONE) {
+        // a key is frequent enough for collisions inside a warp: combine the lanes that share the first hitting lane's slot
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const unsigned hits = __ballot_sync(0xFFFFFFFFu, hit[r]);
@@ -345,7 +351,7 @@ __device__ __forceinline__ void process(const IngestParams& p, Ctx& c, const uin
     for (int r = 0; r < R; ++r) spill_append<LP>(p, c, todo[r], khi[r], w[r][2], prod[r], h[r]);
 }
 
-template <uint32_t LP, bool HOT, bool DEDUPE>
+template <uint32_t LP, bool HOT, ull SKEW>
 __device__ __forceinline__ void scatter_body(const IngestParams& p, Ctx& c) {
     // CTA b handles record pairs (b + k * gridDim) * 1024 + tid, k = 0, 1, ...  Three 32-byte loads
     // rotate per thread: while one is consumed the next two are in flight.  Rounds in which every
@@ -366,13 +372,13 @@ __device__ __forceinline__ void scatter_body(const IngestParams& p, Ctx& c) {
         }
     };
     auto consume_full = [&](const uint32_t (&raw)[8]) {
-        one_record<LP, HOT, DEDUPE, true>(p, c, raw[0], raw[1], raw[2], raw[3], true);
-        one_record<LP, HOT, DEDUPE, true>(p, c, raw[4], raw[5], raw[6], raw[7], true);
+        one_record<LP, HOT, SKEW, true>(p, c, raw[0], raw[1], raw[2], raw[3], true);
+        one_record<LP, HOT, SKEW, true>(p, c, raw[4], raw[5], raw[6], raw[7], true);
     };
     auto consume_tail = [&](uint32_t round, const uint32_t (&raw)[8]) {
         const bool present = round < rounds && first + (ull)round * stride < p.n_pairs;
-        one_record<LP, HOT, DEDUPE, false>(p, c, raw[0], raw[1], raw[2], raw[3], present);
-        one_record<LP, HOT, DEDUPE, false>(p, c, raw[4], raw[5], raw[6], raw[7], present);
+        one_record<LP, HOT, SKEW, false>(p, c, raw[0], raw[1], raw[2], raw[3], present);
+        one_record<LP, HOT, SKEW, false>(p, c, raw[4], raw[5], raw[6], raw[7], present);
     };
     fetch(0, bufA);
     fetch(1, bufB);
@@ -405,8 +411,102 @@ __device__ __forceinline__ void scatter_body(const IngestParams& p, Ctx& c) {
         uint4 v = make_uint4(0, 0, 0, 0);
         const bool present = threadIdx.x < p.n_single;
         if (present) v = *reinterpret_cast<const uint4*>(threadIdx.x == 0 ? p.single[0] : p.single[1]);
-        one_record<LP, HOT, DEDUPE, false>(p, c, v.x, v.y, v.z, v.w, present);
+        one_record<LP, HOT, SKEW, false>(p, c, v.x, v.y, v.z, v.w, present);
     }
+}
+
+// ---- one key dominates the trace -----------------------------------------------------------------
+// Its records are recognised before anything else is done with them and summed in registers; the others go to the
+// warp's queue in shared memory and through one_record 32 at a time, so that what is left of a warp's 32
+// records does not cost the price of 32.  Bound by DRAM once the key holds most records (90 %: 140 -> 45 warp
+// instructions per 32 records, 0.66 -> 0.37 ms per 2^27 records); the queue pays from a share of 3/8 on.
+template <uint32_t LP>
+__device__ __forceinline__ void dominated_body(const IngestParams& p, Ctx& c) {
+    using L = Smem<LP>;
+    const uint32_t lane = threadIdx.x & 31u, lt = (1u << lane) - 1u;
+    const uint32_t queue = c.sb + L::QUEUE + (threadIdx.x >> 5) * (SCATTER_QUEUE * 16u);
+    const ull top = p.t.ctl->top_key;
+    const uint32_t top_hi = (uint32_t)(top >> 32), top_lo = (uint32_t)top;
+    ull sum = 0;
+    uint32_t wraps = 0, count = 0, q = 0;
+    auto settle = [&](uint32_t n) {        // the last n records of the queue (n = 32 but for the last time)
+        __syncwarp();
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (lane < n)
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(queue + (q - n + lane) * 16u) : "memory");
+        __syncwarp();
+        q -= n;
+        one_record<LP, true, SKEW_DOMINATED, false>(p, c, v.x, v.y, v.z, v.w, lane < n);
+    };
+    auto take = [&](uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, bool present) {
+        const bool dom = present && w0 < p.n_apps && (w1 & 0x00FFFFFFu) == top_hi && w2 == top_lo;
+        const uint32_t wgt = (p.appw_in_smem != 0) ? lds_u32(c.sb + L::APPW + (w0 & (APPW_SMEM_MAX - 1u)) * 4u) : __ldg(p.app_w + (dom ? w0 : 0u));
+        const ull prod = dom ? (ull)wgt * (ull)w3 : 0ull;
+        sum += prod;
+        wraps += sum < prod ? 1u : 0u;
+        count += dom ? 1u : 0u;
+        const uint32_t others = __ballot_sync(0xFFFFFFFFu, present && !dom);
+        if (others) {
+            if (present && !dom)
+                asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(queue + (q + __popc(others & lt)) * 16u), "r"(w0), "r"(w1), "r"(w2), "r"(w3) : "memory");
+            q += __popc(others);
+            if (q >= 32) settle(32);
+        }
+    };
+    const unsigned char* body = reinterpret_cast<const unsigned char*>(p.body);
+    const uint32_t stride = gridDim.x * SCATTER_THREADS;                  // pairs per round
+    const uint32_t full_rounds = (uint32_t)(p.n_pairs / stride);
+    const uint32_t rounds = (uint32_t)((p.n_pairs + stride - 1) / stride);
+    const uint32_t first = blockIdx.x * SCATTER_THREADS + threadIdx.x;
+    uint32_t bufA[8], bufB[8];
+    auto fetch = [&](uint32_t round, uint32_t (&raw)[8]) {
+        const ull i = first + (ull)round * stride;
+        if (round < full_rounds || (round < rounds && i < p.n_pairs)) {
+            ld_stream_256(body + i * 32, raw);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) raw[j] = 0;
+        }
+    };
+    auto consume = [&](uint32_t round, const uint32_t (&raw)[8]) {
+        const bool present = round < full_rounds || (round < rounds && first + (ull)round * stride < p.n_pairs);
+        take(raw[0], raw[1], raw[2], raw[3], present);
+        take(raw[4], raw[5], raw[6], raw[7], present);
+    };
+    fetch(0, bufA);
+    for (uint32_t round = 0; round < rounds; round += 2) {
+        fetch(round + 1, bufB);
+        consume(round, bufA);
+        fetch(round + 2, bufA);
+        consume(round + 1, bufB);
+    }
+    // records that do not form an aligned pair (at most one before and one after the body)
+    if (blockIdx.x == 0 && threadIdx.x < 32) {
+        uint4 v = make_uint4(0, 0, 0, 0);
+        const bool present = threadIdx.x < p.n_single;
+        if (present) v = *reinterpret_cast<const uint4*>(threadIdx.x == 0 ? p.single[0] : p.single[1]);
+        take(v.x, v.y, v.z, v.w, present);
+    }
+    if (q) settle(q);
+    // the key's sum: lanes, warps, then one table update per CTA
+    __shared__ ull s_lo, s_hi, s_count;
+    if (threadIdx.x == 0) s_lo = s_hi = s_count = 0;
+    __syncthreads();
+    ull hi = wraps, n = count;
+#pragma unroll
+    for (int d = 16; d; d >>= 1) {
+        const ull o = __shfl_xor_sync(0xFFFFFFFFu, sum, d), s = sum + o;
+        hi += __shfl_xor_sync(0xFFFFFFFFu, hi, d) + (s < sum ? 1ull : 0ull);
+        sum = s;
+        n += __shfl_xor_sync(0xFFFFFFFFu, n, d);
+    }
+    if (lane == 0 && n) {
+        const ull old = atomicAdd(&s_lo, sum);
+        atomicAdd(&s_hi, hi + (old + sum < old ? 1ull : 0ull));
+        atomicAdd(&s_count, n);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && s_count) table_accumulate(p.t, top, hash32(top), s_lo, s_hi, s_count);
 }
 
 // ---- shared-memory record ring (ATREX_SCATTER_RING stages) ----------------------------------------
@@ -453,7 +553,7 @@ __device__ __forceinline__ uint4 lds_record(uint32_t a) {
     return v;
 }
 
-template <uint32_t LP, bool HOT, bool DEDUPE>
+template <uint32_t LP, bool HOT, ull SKEW>
 __device__ __forceinline__ void ring_body(const IngestParams& p, Ctx& c, ull* full_bar, ull* empty_bar, volatile uint32_t* abort_flag) {
     constexpr uint32_t S = SCATTER_RING_STAGES > 0 ? SCATTER_RING_STAGES : 1;
     constexpr uint32_t TILE_RECS = SCATTER_CONSUMER_WARPS * 32;
@@ -516,12 +616,12 @@ __device__ __forceinline__ void ring_body(const IngestParams& p, Ctx& c, ull* fu
         const uint32_t w[2][4] = {{r0.x, r0.y, r0.z, r0.w}, {r1.x, r1.y, r1.z, r1.w}};
         const bool full = second && first1 + TILE_RECS <= p.n_recs;     // both tiles complete (uniform)
         if (full) {
-            process<LP, HOT, DEDUPE, true, 2>(p, c, w, true);
+            process<LP, HOT, SKEW, true, 2>(p, c, w, true);
         } else {
             // ragged end: one record at a time, each with its own mask
             const uint32_t wa[1][4] = {{r0.x, r0.y, r0.z, r0.w}}, wb[1][4] = {{r1.x, r1.y, r1.z, r1.w}};
-            process<LP, HOT, DEDUPE, false, 1>(p, c, wa, p0);
-            process<LP, HOT, DEDUPE, false, 1>(p, c, wb, p1);
+            process<LP, HOT, SKEW, false, 1>(p, c, wa, p0);
+            process<LP, HOT, SKEW, false, 1>(p, c, wb, p1);
         }
     }
 }
@@ -571,16 +671,21 @@ __global__ void __launch_bounds__(SCATTER_THREADS, 1) scatter_kernel(IngestParam
     }
     __syncthreads();
 
+    const ull skew = HOT ? p.t.ctl->hot_skew : SKEW_NONE;
     if (SCATTER_RING_STAGES > 0) {
-        if (HOT && p.t.ctl->hot_skew != 0)
-            ring_body<LP, HOT, true>(p, c, s_full, s_empty, &s_abort);
+        if (HOT && skew == SKEW_DOMINATED)
+            ring_body<LP, HOT, SKEW_DOMINATED>(p, c, s_full, s_empty, &s_abort);
+        else if (HOT && skew == SKEW_COMBINE)
+            ring_body<LP, HOT, SKEW_COMBINE>(p, c, s_full, s_empty, &s_abort);
         else
-            ring_body<LP, HOT, false>(p, c, s_full, s_empty, &s_abort);
+            ring_body<LP, HOT, SKEW_NONE>(p, c, s_full, s_empty, &s_abort);
     } else {
-        if (HOT && p.t.ctl->hot_skew != 0)
-            scatter_body<LP, HOT, true>(p, c);
+        if (HOT && skew == SKEW_DOMINATED)
+            dominated_body<LP>(p, c);
+        else if (HOT && skew == SKEW_COMBINE)
+            scatter_body<LP, HOT, SKEW_COMBINE>(p, c);
         else
-            scatter_body<LP, HOT, false>(p, c);
+            scatter_body<LP, HOT, SKEW_NONE>(p, c);
     }
 
     __syncthreads();
@@ -610,13 +715,14 @@ __global__ void __launch_bounds__(SCATTER_THREADS, 1) scatter_kernel(IngestParam
         // before results are read.
         ulonglong2* img = p.hot_img + (size_t)blockIdx.x * L::SLOTS;
         const bool held = blockIdx.x < p.img_rows;   // the row holds earlier launches' sums
+        const uint32_t in_use = skew == SKEW_DOMINATED ? L::SLOTS_DOM : L::SLOTS;
         for (uint32_t i0 = threadIdx.x; i0 < L::SLOTS; i0 += 4 * blockDim.x) {  // four slots per thread in flight
             uint32_t cn[4], lo[4], hi[4];
             ulonglong2 o[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const uint32_t i = i0 + u * blockDim.x;
-                const bool in = i < L::SLOTS;
+                const bool in = i < in_use;
                 lo[u] = in ? g_acc[3 * i] : 0u;
                 hi[u] = in ? g_acc[3 * i + 1] : 0u;
                 cn[u] = in ? g_acc[3 * i + 2] : 0u;

@@ -461,3 +461,29 @@ def test_every_partition_count_with_full_range_keys(lib, max_keys, partitions, h
     assert_same_as_oracle(agg, o, 8, ks=(5,))
     st = agg.stats()
     assert st["n_spilled"] > n // 2 and st["n_drains"] >= 2 and st["n_overflow"] == 0
+
+
+@pytest.mark.parametrize("n_apps", [64, 5000])                          # weights in shared / in global memory
+@pytest.mark.parametrize("share", [0.02, 0.05, 0.34, 0.38, 0.6, 0.97, 1.0])
+def test_one_frequent_key_at_every_share(lib, share, n_apps):
+    """A key's share of the trace decides how the scatter pass treats it (like any other, lanes combined, taken
+    out before the directory): shares on both sides of the lines, products beyond 48 bits, invalid records, an
+    odd count and an unaligned start, and a second call of another law that meets the first one's directory."""
+    rng = np.random.default_rng(int(share * 100) + n_apps)
+    n = (1 << 21) + 33
+    recs = np.zeros(n, dtype=RECORD_DTYPE)
+    recs["app_id"] = rng.integers(0, n_apps + (n_apps >> 5), n)          # 3 % name an unknown application
+    recs["op_id"], recs["shape_id"], recs["phase"] = rng.integers(0, 40, n), rng.integers(0, 900, n), rng.integers(0, 2, n)
+    hot = rng.random(n) < share
+    recs["op_id"][hot], recs["shape_id"][hot], recs["phase"][hot] = 3, 0xFFFFFFFF, 1
+    recs["duration_ns"] = rng.integers(0, 1 << 28, n, dtype=np.uint32)
+    recs["duration_ns"][::1000] = 0xFFFFFFFF
+    weights = rng.integers(1, 1 << 20, n_apps).astype(np.uint32)
+    weights[::50] = 0xFFFFFFFF
+    other = recs[rng.permutation(n)[: n // 2 * 2 - 1]].copy()
+    other["op_id"] = (other["op_id"] + 1) % 40
+    both = np.concatenate([recs, other])
+    o = oracle_of(both, weights, 2)
+    agg = gpu_aggregate(lib, recs, weights, 2, max_keys=200_000, misalign=True)
+    agg.ingest(to_dev(other), n=len(other))
+    assert_same_as_oracle(agg, o, 2, ks=(3,))
