@@ -418,8 +418,8 @@ __device__ __forceinline__ void scatter_body(const IngestParams& p, Ctx& c) {
 // ---- one key dominates the trace -----------------------------------------------------------------
 // Its records are recognised before anything else is done with them and summed in registers; the others go to the
 // warp's queue in shared memory and through one_record 32 at a time, so that what is left of a warp's 32
-// records does not cost the price of 32.  Bound by DRAM once the key holds most records (90 %: 140 -> 45 warp
-// instructions per 32 records, 0.66 -> 0.37 ms per 2^27 records); the queue pays from a share of 3/8 on.
+// records does not cost the price of 32.  Bound by DRAM once the key holds most records (90 %: 140 -> 57 warp
+// instructions per 32 records, 0.66 -> 0.39 ms per 2^27 records); the queue pays from a share of 3/8 on.
 template <uint32_t LP>
 __device__ __forceinline__ void dominated_body(const IngestParams& p, Ctx& c) {
     using L = Smem<LP>;
@@ -427,8 +427,8 @@ __device__ __forceinline__ void dominated_body(const IngestParams& p, Ctx& c) {
     const uint32_t queue = c.sb + L::QUEUE + (threadIdx.x >> 5) * (SCATTER_QUEUE * 16u);
     const ull top = p.t.ctl->top_key;
     const uint32_t top_hi = (uint32_t)(top >> 32), top_lo = (uint32_t)top;
-    ull sum = 0;
-    uint32_t wraps = 0, count = 0, q = 0;
+    ull sum = 0;                           // (products of 2^48 and more take the queue, so that it cannot wrap)
+    uint32_t count = 0, q = 0;
     auto settle = [&](uint32_t n) {        // the last n records of the queue (n = 32 but for the last time)
         __syncwarp();
         uint4 v = make_uint4(0, 0, 0, 0);
@@ -439,19 +439,19 @@ __device__ __forceinline__ void dominated_body(const IngestParams& p, Ctx& c) {
         one_record<LP, true, SKEW_DOMINATED, false>(p, c, v.x, v.y, v.z, v.w, lane < n);
     };
     auto take = [&](uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, bool present) {
-        const bool dom = present && w0 < p.n_apps && (w1 & 0x00FFFFFFu) == top_hi && w2 == top_lo;
-        const uint32_t wgt = (p.appw_in_smem != 0) ? lds_u32(c.sb + L::APPW + (w0 & (APPW_SMEM_MAX - 1u)) * 4u) : __ldg(p.app_w + (dom ? w0 : 0u));
-        const ull prod = dom ? (ull)wgt * (ull)w3 : 0ull;
-        sum += prod;
-        wraps += sum < prod ? 1u : 0u;
-        count += dom ? 1u : 0u;
-        const uint32_t others = __ballot_sync(0xFFFFFFFFu, present && !dom);
-        if (others) {
-            if (present && !dom)
-                asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(queue + (q + __popc(others & lt)) * 16u), "r"(w0), "r"(w1), "r"(w2), "r"(w3) : "memory");
-            q += __popc(others);
-            if (q >= 32) settle(32);
+        const bool match = (((w1 ^ top_hi) & 0x00FFFFFFu) | (w2 ^ top_lo)) == 0u && w0 < p.n_apps && present;
+        const uint32_t wgt = (p.appw_in_smem != 0) ? lds_u32(c.sb + L::APPW + (w0 & (APPW_SMEM_MAX - 1u)) * 4u) : __ldg(p.app_w + (match ? w0 : 0u));
+        const ull prod = (ull)wgt * (ull)w3;
+        const bool dom = match && (uint32_t)(prod >> 32) < 0x10000u;
+        if (dom) {
+            sum += prod;
+            ++count;
         }
+        const uint32_t others = __ballot_sync(0xFFFFFFFFu, present && !dom);
+        if (present && !dom)
+            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(queue + (q + __popc(others & lt)) * 16u), "r"(w0), "r"(w1), "r"(w2), "r"(w3) : "memory");
+        q += __popc(others);
+        if (q >= 32) settle(32);
     };
     const unsigned char* body = reinterpret_cast<const unsigned char*>(p.body);
     const uint32_t stride = gridDim.x * SCATTER_THREADS;                  // pairs per round
@@ -459,26 +459,46 @@ __device__ __forceinline__ void dominated_body(const IngestParams& p, Ctx& c) {
     const uint32_t rounds = (uint32_t)((p.n_pairs + stride - 1) / stride);
     const uint32_t first = blockIdx.x * SCATTER_THREADS + threadIdx.x;
     uint32_t bufA[8], bufB[8];
-    auto fetch = [&](uint32_t round, uint32_t (&raw)[8]) {
+    auto fetch = [&](uint32_t round, uint32_t (&raw)[8]) {                // any round, bounds checked
         const ull i = first + (ull)round * stride;
-        if (round < full_rounds || (round < rounds && i < p.n_pairs)) {
+        if (round < rounds && i < p.n_pairs) {
             ld_stream_256(body + i * 32, raw);
         } else {
 #pragma unroll
             for (int j = 0; j < 8; ++j) raw[j] = 0;
         }
     };
-    auto consume = [&](uint32_t round, const uint32_t (&raw)[8]) {
-        const bool present = round < full_rounds || (round < rounds && first + (ull)round * stride < p.n_pairs);
+    auto consume_full = [&](const uint32_t (&raw)[8]) {
+        take(raw[0], raw[1], raw[2], raw[3], true);
+        take(raw[4], raw[5], raw[6], raw[7], true);
+    };
+    auto consume_tail = [&](uint32_t round, const uint32_t (&raw)[8]) {
+        const bool present = round < rounds && first + (ull)round * stride < p.n_pairs;
         take(raw[0], raw[1], raw[2], raw[3], present);
         take(raw[4], raw[5], raw[6], raw[7], present);
     };
     fetch(0, bufA);
-    for (uint32_t round = 0; round < rounds; round += 2) {
+    uint32_t round = 0;
+    {   // two loads alternate (a third would not fit the registers), each behind an L2 prefetch of the round after it
+        // (1 812 -> 1 559 us per 2^29 records; two rounds ahead 1 679); complete rounds need no checks
+        const unsigned char* next = body + (first + (ull)stride) * 32;
+        const uint32_t step = gridDim.x * (SCATTER_THREADS * 32u);
+        for (; round + 4 <= full_rounds; round += 2) {
+            ld_stream_256(next, bufB);
+            if ((lane & 3u) == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(next + step));
+            next += step;
+            consume_full(bufA);
+            ld_stream_256(next, bufA);
+            if ((lane & 3u) == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(next + step));
+            next += step;
+            consume_full(bufB);
+        }
+    }
+    for (; round < rounds; round += 2) {
         fetch(round + 1, bufB);
-        consume(round, bufA);
+        consume_tail(round, bufA);
         fetch(round + 2, bufA);
-        consume(round + 1, bufB);
+        consume_tail(round + 1, bufB);
     }
     // records that do not form an aligned pair (at most one before and one after the body)
     if (blockIdx.x == 0 && threadIdx.x < 32) {
@@ -492,7 +512,7 @@ __device__ __forceinline__ void dominated_body(const IngestParams& p, Ctx& c) {
     __shared__ ull s_lo, s_hi, s_count;
     if (threadIdx.x == 0) s_lo = s_hi = s_count = 0;
     __syncthreads();
-    ull hi = wraps, n = count;
+    ull hi = 0, n = count;
 #pragma unroll
     for (int d = 16; d; d >>= 1) {
         const ull o = __shfl_xor_sync(0xFFFFFFFFu, sum, d), s = sum + o;
