@@ -67,6 +67,7 @@ struct Control {
     ull hot_n;                 // keys in the hot directory
     ull work_status;           // ST_WORK_* bits of the last work-table load
     ull hot_skew;              // SKEW_*: how the scatter pass deals with the most frequent key
+    ull prefetch;              // 1: the directory holds enough of the sample for the scatter pass to prefetch records
     ull top_key;               // the most frequent key (SKEW_DOMINATED)
     ull n_spilled;             // records routed through the spill buffers
     ull n_overflow;            // records that found their spill buffer full (slow exact path)

@@ -739,13 +739,13 @@ __global__ void __launch_bounds__(256) hot_list_kernel(HotBuildParams p) {
 }
 
 __global__ void __launch_bounds__(128) hot_pick_kernel(HotBuildParams p) {
-    __shared__ uint32_t s_inserted;
-    if (threadIdx.x == 0) s_inserted = 0;
+    __shared__ uint32_t s_inserted, s_weight;
+    if (threadIdx.x == 0) s_inserted = s_weight = 0;
     __syncthreads();
     grid_dependency_wait();
     HotBuildScratch& x = *p.scratch;
     const uint32_t b = blockIdx.x * 128 + threadIdx.x;
-    uint32_t inserted = 0;
+    uint32_t inserted = 0, weight = 0;
     if (b < p.hot_slots / DIR_WAYS) {
         const uint32_t n = min(x.listed[b], LIST_MAX);
         uint32_t top[DIR_WAYS] = {0, 0, 0, 0}, who[DIR_WAYS] = {0, 0, 0, 0};
@@ -767,6 +767,7 @@ __global__ void __launch_bounds__(128) hot_pick_kernel(HotBuildParams p) {
         for (uint32_t way = 0; way < DIR_WAYS; ++way) {
             keys[way] = top[way] ? x.key[who[way]] : 0ull;
             inserted += top[way] ? 1u : 0u;
+            weight += top[way];
         }
         ulonglong2* dst = reinterpret_cast<ulonglong2*>(p.hot_keys + b * DIR_WAYS);
         dst[0] = make_ulonglong2(keys[0], keys[1]);
@@ -774,9 +775,17 @@ __global__ void __launch_bounds__(128) hot_pick_kernel(HotBuildParams p) {
         if (b == 0) p.ctl->dir_mult = best_multiplier(x);
     }
     inserted = __reduce_add_sync(0xFFFFFFFFu, inserted);
-    if ((threadIdx.x & 31u) == 0 && inserted) atomicAdd(&s_inserted, inserted);
+    weight = __reduce_add_sync(0xFFFFFFFFu, weight);
+    if ((threadIdx.x & 31u) == 0 && inserted) {
+        atomicAdd(&s_inserted, inserted);
+        atomicAdd(&s_weight, weight);
+    }
     __syncthreads();
-    if (threadIdx.x == 0 && s_inserted) atomicAdd(&p.ctl->hot_n, (ull)s_inserted);
+    if (threadIdx.x == 0 && s_inserted) {
+        atomicAdd(&p.ctl->hot_n, (ull)s_inserted);
+        const uint32_t before = atomicAdd(&x.weight, s_weight);
+        if (before * 3ull < p.n_sample && (before + s_weight) * 3ull >= p.n_sample) p.ctl->prefetch = 1;
+    }
 }
 
 // --------------------------------------------------------------------------------------

@@ -94,6 +94,7 @@ constexpr uint32_t HOT_SELECT_MAX = 14336;   // candidates kept (directory <= 11
 constexpr uint32_t HOT_BUCKETS_MAX = 3072;   // directory buckets (<= 11.6K / 4)
 struct HotBuildScratch {
     uint32_t n, most, threshold, done;
+    uint32_t weight, pad[3];                     // sampled weight in the directory
     uint32_t lost[4];                            // sampled weight each multiplier would lose
     uint32_t hist[1024];                         // candidates by count
     uint32_t occupancy[4][HOT_BUCKETS_MAX];
