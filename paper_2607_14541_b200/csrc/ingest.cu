@@ -371,6 +371,7 @@ __global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(PartitionP
     ulonglong2* const my_queue = q.queue + (size_t)blockIdx.x * q.queue_cap + (size_t)(threadIdx.x >> 5) * queue_cap_w;
     const uint32_t n_parts = 1u << q.t.lp;
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u, n_warps = blockDim.x >> 5;
+    grid_dependency_wait();
     // the spill buffers are drained lazily: unless forced, only when the scatter launch just
     // before this one found a buffer filling up
     if (!q.force && ld_relaxed(&q.t.ctl->drain_seq) != q.seq) return;
@@ -489,6 +490,7 @@ __global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(PartitionP
         for (uint32_t g = threadIdx.x; g < q.n_used; g += blockDim.x) q.spill_cnt[((ull)g << q.t.lp) + part] = 0;
         part = next;
     }
+    grid_dependents_launch();
     // the last CTA rewinds the hand-out counter for the next launch
     if (threadIdx.x == 0) {
         __threadfence();
@@ -813,8 +815,7 @@ cudaError_t ingest_prepare() {
 
 cudaError_t launch_partition(const PartitionParams& q, int n_sms, cudaStream_t stream) {
     int grid = (int)(1u << q.t.lp) < n_sms ? (int)(1u << q.t.lp) : n_sms;
-    partition_kernel<<<grid, INGEST_THREADS, (size_t)q.t.C * 20, stream>>>(q);
-    return cudaGetLastError();
+    return launch_chained(partition_kernel, (uint32_t)grid, INGEST_THREADS, (size_t)q.t.C * 20, stream, q);
 }
 
 cudaError_t launch_hot_build(const HotBuildParams& p, int n_sms, cudaStream_t stream) {

@@ -669,6 +669,7 @@ __global__ void __launch_bounds__(SCATTER_THREADS, 1) scatter_kernel(IngestParam
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
 
+    grid_dependency_wait();
     Ctx c;
     c.sb = smem_addr(smem_raw);
     c.mult = HOT ? (uint32_t)p.t.ctl->dir_mult : 1u;
@@ -709,6 +710,7 @@ __global__ void __launch_bounds__(SCATTER_THREADS, 1) scatter_kernel(IngestParam
             scatter_body<LP, HOT, SKEW_NONE>(p, c);
     }
 
+    grid_dependents_launch();
     __syncthreads();
     uint32_t spilled = 0, fullest = 0;
     bool crowded = false;
@@ -770,11 +772,8 @@ cudaError_t prepare_lp() {
 }
 
 template <uint32_t LP>
-void launch_lp(const IngestParams& p, bool hot, int grid, cudaStream_t stream) {
-    if (hot)
-        scatter_kernel<LP, true><<<grid, SCATTER_THREADS, Smem<LP>::TOTAL, stream>>>(p);
-    else
-        scatter_kernel<LP, false><<<grid, SCATTER_THREADS, Smem<LP>::TOTAL, stream>>>(p);
+cudaError_t launch_lp(const IngestParams& p, bool hot, int grid, cudaStream_t stream) {
+    return launch_chained(hot ? scatter_kernel<LP, true> : scatter_kernel<LP, false>, (uint32_t)grid, SCATTER_THREADS, Smem<LP>::TOTAL, stream, p);
 }
 
 }  // namespace
@@ -791,14 +790,13 @@ cudaError_t scatter_prepare() {
 cudaError_t launch_scatter(const IngestParams& p, bool hot, int grid, cudaStream_t stream) {
     if (hot && p.hot_slots != scatter_hot_slots(p.t.lp)) return cudaErrorInvalidValue;
     switch (p.t.lp) {
-        case 8: launch_lp<8>(p, hot, grid, stream); break;
-        case 9: launch_lp<9>(p, hot, grid, stream); break;
-        case 10: launch_lp<10>(p, hot, grid, stream); break;
-        case 11: launch_lp<11>(p, hot, grid, stream); break;
-        case 12: launch_lp<12>(p, hot, grid, stream); break;
+        case 8: return launch_lp<8>(p, hot, grid, stream);
+        case 9: return launch_lp<9>(p, hot, grid, stream);
+        case 10: return launch_lp<10>(p, hot, grid, stream);
+        case 11: return launch_lp<11>(p, hot, grid, stream);
+        case 12: return launch_lp<12>(p, hot, grid, stream);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 }  // namespace atrex
