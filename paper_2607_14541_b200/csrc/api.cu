@@ -449,10 +449,12 @@ static int drain_spill(atrex_agg* h, bool force, cudaStream_t s) {
 }
 
 static int ingest_launch(atrex_agg* h, const atrex_record_t* recs, uint64_t n, cudaStream_t s) {
-    // Small calls go straight into the table (direct.cu).  The line lies where the two-pass route's fixed
-    // costs are made up for by its higher rate: at 2^20 records for tables that L2 holds beside everything
-    // else, at 2^18 for larger ones, whose global atomics wait for DRAM.  Without the shared-memory stage only the smallest.
-    const uint64_t direct_max = h->L.hot_slots == 0 ? DIRECT_RECORDS_MAX : (h->L.n_slots * 24 > L2_TABLE_BYTES ? 1ull << 18 : 1ull << 20);
+    // Small calls go straight into the table (direct.cu).  Measured per 2^20 records: 40 to 65 us that way, 16 to 25
+    // by the two-pass route, which costs 110 to 270 us once (directory, drain, fold): made up for after 4 M records.
+    // A single call breaks even at 2^17 records once that is spent, at 2^18 where the table is larger than L2.
+    const bool small_table = h->L.n_slots * 24 <= L2_TABLE_BYTES;
+    const bool few_so_far = !h->hot_ready && h->n_records + n <= (1ull << 22);
+    const uint64_t direct_max = h->L.hot_slots == 0 ? DIRECT_RECORDS_MAX : (!few_so_far ? 1ull << 17 : (small_table ? 1ull << 22 : 1ull << 18));
     if (n <= direct_max) {
         DirectParams d;
         memset(&d, 0, sizeof(d));
