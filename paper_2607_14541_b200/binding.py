@@ -1,7 +1,9 @@
-"""ctypes binding of the C ABI declared in ``include/atrex_agg.h``.
+"""Python binding of the C ABI declared in ``include/atrex_agg.h``.
 
 Argument marshalling only: every step of the aggregation path runs in the library's CUDA
-kernels.  PyTorch appears here for device memory (workspace, output buffers) and streams.
+kernels.  The entry points stand here as ctypes functions; the methods below call those that a
+program calls often through ``_call`` (csrc/call.cpp), which takes a fraction of ctypes' time.
+PyTorch appears here for device memory (workspace, output buffers) and streams.
 There is no CPU fallback: if the shared library is missing, importing this module raises.
 """
 from __future__ import annotations
@@ -162,6 +164,22 @@ atrex_entries_bucket_by_owner = lib.atrex_entries_bucket_by_owner
 atrex_totals_combine = lib.atrex_totals_combine
 
 
+if not os.path.exists(os.path.join(_HERE, "_call.so")):
+    raise ImportError("_call.so is not built; run `python -m paper_2607_14541_b200.build`")
+from ._call import bind as _bind  # noqa: E402
+
+
+def _quick(name: str):
+    """The entry point as a callable that takes whole numbers, None and buffers."""
+    f = getattr(lib, name)
+    return _bind(C.cast(f, C.c_void_p).value, len(f.argtypes))
+
+
+_ingest, _ingest_host, _merge, _reset, _finalize, _topk, _eq3_ingest, _eq3_finalize, _eq3_reset, _score = (
+    _quick("atrex_" + n) for n in ("agg_ingest", "agg_ingest_host", "agg_merge", "agg_reset", "agg_finalize", "agg_topk",
+                                   "eq3_ingest", "eq3_finalize", "eq3_reset", "score_aggregate"))
+
+
 class AtrexError(RuntimeError):
     def __init__(self, status: int, where: str, cuda_error: int = 0):
         self.status = status
@@ -171,20 +189,16 @@ class AtrexError(RuntimeError):
         super().__init__(msg)
 
 
-def _raw_stream(torch, device: int) -> int:
-    """cudaStream_t of the device's current torch stream (the raw handle: building a Stream object for it takes
+def _raw_stream_of(torch):
+    """device -> cudaStream_t of its current torch stream (the raw handle: building a Stream object for it takes
     longer than a kernel launch)."""
     get = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-    return get(device) if get is not None else torch.cuda.current_stream(device).cuda_stream
+    return get if get is not None else (lambda device: torch.cuda.current_stream(device).cuda_stream)
 
 
 def make_peaks(peak_bw: float, peak_flops) -> atrex_hw_peaks_t:
-    pk = atrex_hw_peaks_t()
-    pk.peak_bw = float(peak_bw)
-    pf = list(peak_flops) + [1.0] * (ATREX_MAX_DTYPES - len(peak_flops))
-    for i in range(ATREX_MAX_DTYPES):
-        pk.peak_flops[i] = float(pf[i])
-    return pk
+    pf = [*peak_flops, *(1.0,) * (ATREX_MAX_DTYPES - len(peak_flops))]
+    return atrex_hw_peaks_t(peak_bw, (C.c_double * ATREX_MAX_DTYPES)(*pf[:ATREX_MAX_DTYPES]))
 
 
 class OperatorWeights:
@@ -195,20 +209,21 @@ class OperatorWeights:
         if not torch.cuda.is_available():
             raise RuntimeError("the aggregation path is CUDA-only and no CUDA device is available")
         self._torch, self.device, self.n_ops = torch, int(device), int(n_ops)
+        self._raw_stream = _raw_stream_of(torch)
         w = np.ascontiguousarray(app_weights, dtype=np.uint32)
         h = C.c_void_p()
         rc = atrex_eq3_create(int(w.shape[0]), int(n_ops), int(n_phases), w.ctypes.data, self.device, C.byref(h))
         if rc != ATREX_OK:
             raise AtrexError(rc, "atrex_eq3_create")
         self._h = h
+        self._p = h.value     # (the handle as a whole number)
 
     def _stream(self, stream=None):
-        return _raw_stream(self._torch, self.device) if stream is None else stream.cuda_stream
+        return self._raw_stream(self.device) if stream is None else stream.cuda_stream
 
     def ingest(self, records, n: int | None = None, stream=None):
-        if n is None:
-            n = records.numel() * records.element_size() // 16
-        rc = atrex_eq3_ingest(self._h, records.data_ptr(), int(n), self._stream(stream))
+        n = records.nbytes // 16 if n is None else int(n)
+        rc = _eq3_ingest(self._p, records.data_ptr(), n, self._raw_stream(self.device) if stream is None else stream.cuda_stream)
         if rc != ATREX_OK:
             raise AtrexError(rc, "atrex_eq3_ingest")
 
@@ -217,19 +232,18 @@ class OperatorWeights:
         w, wt = np.zeros(self.n_ops), np.zeros(self.n_ops)
         rej = C.c_uint64(0)
         ret = None if retained is None else np.ascontiguousarray(retained, dtype=np.uint8)
-        rc = atrex_eq3_finalize(self._h, None if ret is None else ret.ctypes.data, w.ctypes.data, wt.ctypes.data,
-                                C.byref(rej), self._stream(stream))
+        rc = _eq3_finalize(self._p, ret, w, wt, rej, self._stream(stream))
         if rc != ATREX_OK:
             raise AtrexError(rc, "atrex_eq3_finalize")
         return w, wt, int(rej.value)
 
     def reset(self, stream=None):
-        atrex_eq3_reset(self._h, self._stream(stream))
+        _eq3_reset(self._p, self._stream(stream))
 
     def close(self):
         if getattr(self, "_h", None):
             atrex_eq3_destroy(self._h)
-            self._h = None
+            self._h = self._p = None
 
     __del__ = close
 
@@ -244,9 +258,9 @@ def score_aggregate(roofline_s, unit_op, t_cand, correct, w, stream=None):
     s_agg = torch.empty(b, dtype=torch.float64, device=dev)
     s_op = torch.empty(b, n_ops, dtype=torch.float64, device=dev)
     err = torch.empty(b, dtype=torch.int64, device=dev)
-    s = _raw_stream(torch, dev.index or 0) if stream is None else stream.cuda_stream
-    rc = atrex_score_aggregate(roofline_s.data_ptr(), unit_op.data_ptr(), n, t_cand.data_ptr(), correct.data_ptr(), b,
-                               w.data_ptr(), n_ops, s_agg.data_ptr(), s_op.data_ptr(), err.data_ptr(), s)
+    s = _raw_stream_of(torch)(dev.index or 0) if stream is None else stream.cuda_stream
+    rc = _score(roofline_s.data_ptr(), unit_op.data_ptr(), n, t_cand.data_ptr(), correct.data_ptr(), b,
+                w.data_ptr(), n_ops, s_agg.data_ptr(), s_op.data_ptr(), err.data_ptr(), s)
     if rc != ATREX_OK:
         raise AtrexError(rc, "atrex_score_aggregate")
     return s_agg, s_op, err
@@ -352,6 +366,7 @@ class Aggregator:
         if not torch.cuda.is_available():
             raise RuntimeError("the aggregation path is CUDA-only and no CUDA device is available")
         self._torch = torch
+        self._raw_stream = _raw_stream_of(torch)
         self.device = int(device)
         w = np.ascontiguousarray(app_weights, dtype=np.uint32)
         cfg = atrex_agg_config_t()
@@ -372,12 +387,13 @@ class Aggregator:
         if rc != ATREX_OK:
             raise AtrexError(rc, "atrex_agg_create")
         self._h = h
+        self._p = h.value     # (the handle as a whole number)
         self.workspace_bytes = int(cfg.workspace_bytes)
 
     # -- helpers
     def _stream(self, stream=None):
         if stream is None:
-            return _raw_stream(self._torch, self.device)
+            return self._raw_stream(self.device)
         return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
     def _check(self, rc, where):
@@ -387,7 +403,7 @@ class Aggregator:
     def close(self):
         if getattr(self, "_h", None):
             atrex_agg_destroy(self._h)
-            self._h = None
+            self._h = self._p = None
             self._ws = None
 
     __del__ = close
@@ -402,13 +418,14 @@ class Aggregator:
     def ingest(self, records, n: int | None = None, stream=None):
         """``records``: CUDA uint8 tensor holding 16-byte records (or a raw device pointer with ``n``)."""
         if isinstance(records, int):
-            ptr = records
+            ptr, n = records, int(n)
         else:
-            assert records.is_cuda and records.device.index == self.device
+            assert records.get_device() == self.device          # (-1: not on a GPU)
             ptr = records.data_ptr()
-            if n is None:
-                n = records.numel() * records.element_size() // 16
-        self._check(atrex_agg_ingest(self._h, ptr, int(n), self._stream(stream)), "atrex_agg_ingest")
+            n = records.nbytes // 16 if n is None else int(n)
+        rc = _ingest(self._p, ptr, n, self._raw_stream(self.device) if stream is None else self._stream(stream))
+        if rc != ATREX_OK:
+            self._check(rc, "atrex_agg_ingest")
 
     def ingest_host(self, records, n: int | None = None, stream=None):
         """``records``: numpy array or CPU (ideally pinned) tensor of 16-byte records."""
@@ -420,13 +437,13 @@ class Aggregator:
             ptr, nb = records.data_ptr(), records.numel() * records.element_size()
         if n is None:
             n = nb // 16
-        self._check(atrex_agg_ingest_host(self._h, ptr, int(n), self._stream(stream)), "atrex_agg_ingest_host")
+        self._check(_ingest_host(self._p, ptr, int(n), self._stream(stream)), "atrex_agg_ingest_host")
 
     def merge(self, entries, n: int | None = None, stream=None):
         assert entries.is_cuda
         if n is None:
-            n = entries.numel() * entries.element_size() // 48
-        self._check(atrex_agg_merge(self._h, entries.data_ptr(), int(n), self._stream(stream)), "atrex_agg_merge")
+            n = entries.nbytes // 48
+        self._check(_merge(self._p, entries.data_ptr(), int(n), self._stream(stream)), "atrex_agg_merge")
 
     def finalize(self, peak_bw: float, peak_flops, out=None, stream=None, global_totals=None):
         """Returns (entries, n): a CUDA uint8 tensor of 48-byte entries and the entry count.
@@ -450,12 +467,12 @@ class Aggregator:
             name = "atrex_agg_finalize_with_totals"
         else:
             def call(ptr, cap):
-                return atrex_agg_finalize(self._h, C.byref(pk), ptr, cap, C.byref(n_out), self._stream(stream))
+                return _finalize(self._p, pk, ptr, cap, n_out, self._stream(stream))
             name = "atrex_agg_finalize"
         if out is None:
             self._check(call(None, 0), name)
             out = torch.empty(max(int(n_out.value), 1) * 48, dtype=torch.uint8, device=f"cuda:{self.device}")
-        cap = out.numel() * out.element_size() // 48
+        cap = out.nbytes // 48
         self._check(call(out.data_ptr(), cap), name)
         return out, int(n_out.value)
 
@@ -464,11 +481,13 @@ class Aggregator:
         return out[: n * 48].cpu().numpy().view(ENTRY_DTYPE).copy()
 
     def topk(self, phase: int, k: int, stream=None) -> np.ndarray:
-        out = np.zeros(max(k, 1), dtype=ENTRY_DTYPE)
+        out = np.empty(max(k, 1), dtype=ENTRY_DTYPE)
         n_out = C.c_uint32(0)
-        rc = atrex_agg_topk(self._h, int(phase), int(k), out.ctypes.data, C.byref(n_out), self._stream(stream))
-        self._check(rc, "atrex_agg_topk")
-        return out[: n_out.value].copy()
+        rc = _topk(self._p, int(phase), int(k), out, n_out, self._stream(stream))
+        if rc != ATREX_OK:
+            self._check(rc, "atrex_agg_topk")
+        n = n_out.value
+        return out if n == out.shape[0] else out[:n].copy()
 
     def stats(self, stream=None, check: bool = True) -> dict:
         st = atrex_stats_t()
@@ -497,7 +516,7 @@ class Aggregator:
         return out[: min(n.value, out.shape[0])].copy()
 
     def reset(self, stream=None):
-        self._check(atrex_agg_reset(self._h, self._stream(stream)), "atrex_agg_reset")
+        self._check(_reset(self._p, self._stream(stream)), "atrex_agg_reset")
 
     def launch_count(self) -> int:
         return int(atrex_agg_launch_count(self._h))

@@ -3,6 +3,7 @@ from __future__ import annotations
 
 import os
 import subprocess
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
@@ -20,8 +21,21 @@ def _stale(target: str, deps) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+CALL_SOURCE = os.path.join(CSRC, "call.cpp")
+CALL_MODULE = os.path.join(_HERE, "_call.so")
+
+
+def build_call(force: bool = False) -> str:
+    """The extension module through which the binding makes its calls."""
+    if force or _stale(CALL_MODULE, [CALL_SOURCE]):
+        subprocess.check_call([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared",
+                               "-I" + sysconfig.get_paths()["include"], "-o", CALL_MODULE, CALL_SOURCE])
+    return CALL_MODULE
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile libatrex_agg.so if it is missing or older than its sources."""
+    """Compile libatrex_agg.so (and the binding's call module) if missing or older than the sources."""
+    build_call(force=force)
     srcs = [os.path.join(CSRC, s) for s in SOURCES]
     deps = srcs + [os.path.normpath(os.path.join(CSRC, h)) for h in HEADERS]
     if force or _stale(LIB, deps):
