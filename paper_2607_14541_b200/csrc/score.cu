@@ -180,8 +180,9 @@ struct Middle {
     __device__ __forceinline__ bool clear() const { return close == 2 - (m & 1u) && ((m & 1u) || v_up - v_lo > K_APART); }
 };
 
-// Up to 32 R keys held in registers: the range of the wanted key is halved (a count over the warp each time)
-// until one key is left in it.
+// Up to 32 R keys held in registers.  Up to 32 keys, each lane counts how many are below its own (the k-th is the
+// largest that has at most k below it); above, where that would take more instructions, the range of the wanted
+// key is halved (a count over the warp each time) until one key is left in it.
 template <int R>
 __device__ __forceinline__ Middle middle_in_registers(const uint32_t* keys, uint32_t g) {
     const uint32_t lane = threadIdx.x & 31u;
@@ -201,34 +202,52 @@ __device__ __forceinline__ Middle middle_in_registers(const uint32_t* keys, uint
     d.v_lo = d.v_up = d.close = d.below = 0;
     if (d.m == 0 || d.unknown) return d;
     const uint32_t k = (d.m - 1) / 2;
-    uint32_t before = 0, through = d.m;    // keys below lo, keys up to hi
-    while (through - before > 1 && lo < hi) {
-        const uint32_t half = lo + (hi - lo) / 2 + 1;
-        uint32_t c = 0;
+    if constexpr (R == 1) {
+        uint32_t less[R] = {}, at_lo = 0, at_up = 0;
+#pragma unroll 8
+        for (uint32_t b = 0; b < g; ++b) {
+            const uint32_t y = keys[b];
 #pragma unroll
-        for (int r = 0; r < R; ++r) c += x[r] < half ? 1u : 0u;
-        c = __reduce_add_sync(FULL, c);
-        if (k < c) {
-            hi = half - 1;
-            through = c;
-        } else {
-            lo = half;
-            before = c;
+            for (int r = 0; r < R; ++r) less[r] += y < x[r] ? 1u : 0u;
         }
-    }
-    uint32_t v = ~0u;
-#pragma unroll
-    for (int r = 0; r < R; ++r) v = min(v, x[r] >= lo ? x[r] : ~0u);
-    d.v_lo = d.v_up = __reduce_min_sync(FULL, v);
-    if (!(d.m & 1u)) {
-        uint32_t leq = 0, up = ~0u;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            leq += x[r] <= d.v_lo ? 1u : 0u;
-            up = min(up, x[r] > d.v_lo ? x[r] : ~0u);
+            if (x[r] == K_ABSENT) continue;
+            at_lo = max(at_lo, less[r] <= k ? x[r] : 0u);
+            at_up = max(at_up, less[r] <= d.m / 2 ? x[r] : 0u);
         }
-        up = __reduce_min_sync(FULL, up);
-        if (__reduce_add_sync(FULL, leq) == k + 1) d.v_up = up;
+        d.v_lo = __reduce_max_sync(FULL, at_lo);
+        d.v_up = __reduce_max_sync(FULL, at_up);
+    } else {
+        uint32_t before = 0, through = d.m;    // keys below lo, keys up to hi
+        while (through - before > 1 && lo < hi) {
+            const uint32_t half = lo + (hi - lo) / 2 + 1;
+            uint32_t c = 0;
+#pragma unroll
+            for (int r = 0; r < R; ++r) c += x[r] < half ? 1u : 0u;
+            c = __reduce_add_sync(FULL, c);
+            if (k < c) {
+                hi = half - 1;
+                through = c;
+            } else {
+                lo = half;
+                before = c;
+            }
+        }
+        uint32_t v = ~0u;
+#pragma unroll
+        for (int r = 0; r < R; ++r) v = min(v, x[r] >= lo ? x[r] : ~0u);
+        d.v_lo = d.v_up = __reduce_min_sync(FULL, v);
+        if (!(d.m & 1u)) {
+            uint32_t leq = 0, up = ~0u;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                leq += x[r] <= d.v_lo ? 1u : 0u;
+                up = min(up, x[r] > d.v_lo ? x[r] : ~0u);
+            }
+            up = __reduce_min_sync(FULL, up);
+            if (__reduce_add_sync(FULL, leq) == k + 1) d.v_up = up;
+        }
     }
     uint32_t close = 0, below = 0;
 #pragma unroll
@@ -358,6 +377,70 @@ __device__ __forceinline__ uint32_t middle_slots(uint32_t* col, uint32_t& low, u
     return m;
 }
 
+// Two lanes' operator: each of the pair sorts its own column of N keys, then both walk the two columns from the
+// place where the middle begins (a binary search: `below` keys of the union lie before it).  `low` and `up`
+// are slots counted from the pair's first column, in steps of one column and 32 per row.
+template <int N>
+__device__ __forceinline__ uint32_t middle_slots_of_pair(uint32_t* col, uint32_t& low, uint32_t& up, bool& search) {
+    {
+        uint32_t v[N];
+#pragma unroll
+        for (int i = 0; i < N; ++i) v[i] = (col[32 * i] & ~K_SLOT) | (uint32_t)i;
+        sort_network<N>(v);
+#pragma unroll
+        for (int i = 0; i < N; ++i) col[32 * i] = v[i];
+    }
+    uint32_t own = 0;
+#pragma unroll
+    for (int step = 16; step; step >>= 1)
+        if (own + step <= N) own += col[32 * (own + step - 1)] < (K_ABSENT & ~K_SLOT) ? step : 0;
+    if (N == 32 && own == 31 && col[32 * 31] < (K_ABSENT & ~K_SLOT)) own = 32;
+    const uint32_t most = own ? col[32 * (own - 1)] : 0u;
+    __syncwarp();
+    const bool odd = threadIdx.x & 1u;
+    const uint32_t other = __shfl_xor_sync(FULL, own, 1), ma = odd ? other : own, mb = odd ? own : other, m = ma + mb;
+    const uint32_t highest = max(most, __shfl_xor_sync(FULL, most, 1));
+    low = up = 0;
+    search = false;
+    if (m == 0) return 0;
+    const uint32_t *a = odd ? col - 1 : col, *b = a + 1;
+    const uint32_t kl = (m - 1) / 2, t = kl > 0 ? kl - 1 : 0u;
+    uint32_t i = t > mb ? t - mb : 0u, end = min(t, ma);    // how many of the first t come from column a
+    while (i < end) {
+        const uint32_t half = (i + end) / 2;
+        if (a[32 * half] < b[32 * (t - half - 1)]) i = half + 1;
+        else end = half;
+    }
+    uint32_t j = t - i;
+    uint32_t x = i < ma ? a[32 * i] : K_ABSENT, y = j < mb ? b[32 * j] : K_ABSENT;
+    uint32_t slot = 0;
+    auto next = [&] {                                        // the next key of the union; K_ABSENT behind the last one
+        const bool from_a = x <= y;
+        const uint32_t k = from_a ? x : y;
+        slot = 32 * (k & K_SLOT) + (from_a ? 0u : 1u);
+        if (from_a) {
+            ++i;
+            x = i < ma ? a[32 * i] : K_ABSENT;
+        } else {
+            ++j;
+            y = j < mb ? b[32 * j] : K_ABSENT;
+        }
+        return k;
+    };
+    uint32_t before = 0;
+    if (kl > 0) before = next();
+    const uint32_t vl = next();
+    low = up = slot;
+    uint32_t vu = vl;
+    if (!(m & 1u)) {
+        vu = next();
+        up = slot;
+    }
+    const uint32_t above = m / 2 + 1 < m ? next() : K_ABSENT;
+    search = highest >= K_UNKNOWN || (kl > 0 && vl - before <= NET_APART) || (!(m & 1u) && vu - vl <= NET_APART) || above - vu <= NET_APART;
+    return m;
+}
+
 constexpr uint32_t WARP_ILP = 4;           // units per lane in flight
 __host__ __device__ __forceinline__ uint32_t padded_units(uint32_t n) { return (n + 32u * WARP_ILP - 1u) / (32u * WARP_ILP) * (32u * WARP_ILP); }
 
@@ -367,7 +450,7 @@ struct WarpLayout {   // byte offsets; from `prod` on relative to the warp's own
         uint32_t o = 0;
         roof = o;    o += 4u * padded_units(n);            // f32 rooflines, NaN outside the safe range
         group = o;   o += 8u * n_ops;                      // {first list entry (large groups), size | large << 31}
-        chunk = o;   o += 4u * ((n_ops + 31u) / 32u + 1u); // first slot of each chunk of 32 operators
+        chunk = o;   o += 4u * ((n_ops + 15u) / 16u + 1u); // first slot of each chunk of 32 (pairs: 16) operators
         place = o;   o += 2u * padded_units(n);            // slot of each unit, NO_GROUP flag
         unit_at = o; o += 2u * (slots + n);                // unit of each slot; behind the columns, the large groups' units
         warps = (o + 15u) & ~15u;
@@ -382,23 +465,27 @@ __host__ __device__ __forceinline__ uint32_t column_length(uint32_t g) { return 
 // Slots to provide: the group sizes are in device memory, so every chunk of operators gets room for groups
 // three standard deviations above the mean (units falling to operators at random); what does not fit is
 // treated as a large group.
-inline uint32_t warp_slots(uint32_t n, uint32_t n_ops) {
+inline uint32_t warp_slots(uint32_t n, uint32_t n_ops, bool pairs) {
     const double mean = (double)n / n_ops;
     double width = std::ceil(mean + 3.0 * std::sqrt(mean)) + 2.0;
-    if (mean > NET_MAX) width = 8;         // (hardly any group is small enough)
+    if (pairs) width = std::ceil(mean * 0.5 + 1.5 * std::sqrt(mean)) + 1.0;
+    if (mean > (pairs ? 2 * NET_MAX : NET_MAX)) width = 8;         // (hardly any group is small enough)
     if (width > NET_MAX) width = NET_MAX;
-    return (n_ops + 31u) / 32u * 32u * column_length((uint32_t)width);
+    const uint32_t per_chunk = pairs ? 16u : 32u;
+    return (n_ops + per_chunk - 1u) / per_chunk * 32u * column_length((uint32_t)width);
 }
 
 constexpr uint32_t NO_GROUP = 0x8000u;     // flag of a unit of an operator outside [0, n_ops)
 constexpr uint32_t SLOT_MASK = 0x7FFFu;    // (units without a group write to a slot behind all others)
 constexpr uint32_t WARP_KERNEL_THREADS = 256, WARP_KERNEL_CTAS = 3;   // per SM (80 registers a thread; four CTAs of 64 were 3 % slower)
 
+template <bool PAIRS>
 __global__ void __launch_bounds__(WARP_KERNEL_THREADS, WARP_KERNEL_CTAS)
     score_warp_kernel(const double* __restrict__ roofline_s, const uint32_t* __restrict__ unit_op, uint32_t n_units,
                       const double* __restrict__ t_cand, const uint8_t* __restrict__ correct, uint32_t n_cand,
                       const double* __restrict__ w, uint32_t n_ops, uint32_t max_slots, double* s_agg, double* s_op_out, ull* errors_out) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr uint32_t PER_CHUNK = PAIRS ? 16 : 32, LANES = PAIRS ? 2 : 1;
     const WarpLayout L(n_units, n_ops, max_slots);
     float* roof = reinterpret_cast<float*>(smem_raw + L.roof);
     uint16_t* place = reinterpret_cast<uint16_t*>(smem_raw + L.place);
@@ -420,25 +507,27 @@ __global__ void __launch_bounds__(WARP_KERNEL_THREADS, WARP_KERNEL_CTAS)
     count_groups(unit_op, n_units, n_ops, size);
     if (threadIdx.x < 32) {
         uint32_t slot = 0, large = 0;
-        for (uint32_t op0 = 0; op0 < n_ops; op0 += 32) {
-            const uint32_t op = op0 + lane, g = op < n_ops ? size[op] : 0u;
-            const bool is_large = g > NET_MAX || slot + 32 * column_length(g) > max_slots;
-            const uint32_t widest = __reduce_max_sync(FULL, is_large ? 0u : g);
+        for (uint32_t op0 = 0; op0 < n_ops; op0 += PER_CHUNK) {
+            const uint32_t op = op0 + lane;
+            const bool mine = lane < PER_CHUNK && op < n_ops;
+            const uint32_t g = mine ? size[op] : 0u, rows = (g + LANES - 1) / LANES;
+            const bool is_large = rows > NET_MAX || slot + 32 * column_length(rows) > max_slots;
+            const uint32_t widest = __reduce_max_sync(FULL, is_large ? 0u : rows);
             uint32_t incl = is_large ? g : 0u;
 #pragma unroll
             for (int d = 1; d < 32; d <<= 1) {
                 const uint32_t o = __shfl_up_sync(FULL, incl, d);
                 if (lane >= (uint32_t)d) incl += o;
             }
-            if (op < n_ops) {
+            if (mine) {
                 group[op] = is_large ? make_uint2(max_slots + large + incl - g, g | 0x80000000u) : make_uint2(0u, g);
                 size[op] = 0;
             }
-            if (lane == 0) chunk[op0 / 32] = slot;
+            if (lane == 0) chunk[op0 / PER_CHUNK] = slot;
             slot += widest ? 32 * column_length(widest) : 0u;
             large += __shfl_sync(FULL, incl, 31);
         }
-        if (lane == 0) chunk[(n_ops + 31) / 32] = slot;
+        if (lane == 0) chunk[(n_ops + PER_CHUNK - 1) / PER_CHUNK] = slot;
     }
     __syncthreads();
     for (uint32_t j = threadIdx.x; j < n_units; j += blockDim.x) {
@@ -450,14 +539,14 @@ __global__ void __launch_bounds__(WARP_KERNEL_THREADS, WARP_KERNEL_CTAS)
             if (g.y >> 31) {
                 to = g.x + i;
             } else {
-                to = chunk[op / 32] + (op & 31u) + 32 * i;
+                to = chunk[op / PER_CHUNK] + (op & (PER_CHUNK - 1)) * LANES + i % LANES + 32 * (i / LANES);
             }
             unit_at[to] = (uint16_t)j;
         }
         place[j] = (uint16_t)to;
     }
     __syncthreads();   // (the sizes lie in the first warp's block)
-    for (uint32_t i = lane; i < chunk[(n_ops + 31) / 32]; i += 32) keys[i] = K_ABSENT;   // unused slots stay absent
+    for (uint32_t i = lane; i < chunk[(n_ops + PER_CHUNK - 1) / PER_CHUNK]; i += 32) keys[i] = K_ABSENT;   // unused slots stay absent
     __syncwarp();
 
     for (uint32_t cand = blockIdx.x * n_warps + warp; cand < n_cand; cand += gridDim.x * n_warps) {
@@ -487,32 +576,41 @@ __global__ void __launch_bounds__(WARP_KERNEL_THREADS, WARP_KERNEL_CTAS)
             }
         }
         __syncwarp();
-        for (uint32_t op0 = 0; op0 < n_ops; op0 += 32) {
-            const uint32_t op = op0 + lane;
+        for (uint32_t op0 = 0; op0 < n_ops; op0 += PER_CHUNK) {
+            const uint32_t op = op0 + lane / LANES;
             const uint2 g = op < n_ops ? group[op] : make_uint2(0, 0);
             const bool is_large = g.y >> 31;
-            const uint32_t first_slot = chunk[op0 / 32] + lane, length = (chunk[op0 / 32 + 1] - chunk[op0 / 32]) / 32;
-            uint32_t* col = keys + first_slot;
+            const uint32_t at = chunk[op0 / PER_CHUNK], first_slot = at + lane / LANES * LANES, length = (chunk[op0 / PER_CHUNK + 1] - at) / 32;
+            uint32_t* col = keys + at + lane;
             uint32_t low = 0, up = 0, m = 0;
             bool search = false;
-            if (length == 8) m = middle_slots<8>(col, low, up, search);
-            else if (length == 16) m = middle_slots<16>(col, low, up, search);
-            else if (length == 20) m = middle_slots<20>(col, low, up, search);
-            else if (length == 24) m = middle_slots<24>(col, low, up, search);
-            else if (length == 28) m = middle_slots<28>(col, low, up, search);
-            else if (length == 32) m = middle_slots<32>(col, low, up, search);
+            auto middle = [&](auto n) {
+                if constexpr (PAIRS) {
+                    m = middle_slots_of_pair<n.value>(col, low, up, search);
+                } else {
+                    m = middle_slots<n.value>(col, low, up, search);
+                    low *= 32;
+                    up *= 32;
+                }
+            };
+            if (length == 8) middle(std::integral_constant<int, 8>());
+            else if (length == 16) middle(std::integral_constant<int, 16>());
+            else if (length == 20) middle(std::integral_constant<int, 20>());
+            else if (length == 24) middle(std::integral_constant<int, 24>());
+            else if (length == 28) middle(std::integral_constant<int, 28>());
+            else if (length == 32) middle(std::integral_constant<int, 32>());
             double s = 0.0;
             if (m != 0 && !search) {
-                const uint32_t ju = unit_at[first_slot + 32 * up], jl = unit_at[first_slot + 32 * low];
+                const uint32_t ju = unit_at[first_slot + up], jl = unit_at[first_slot + low];
                 s = __ddiv_rn(__ldg(roofline_s + ju), __ldg(t + ju));
                 if (!(m & 1u)) s = __dmul_rn(__dadd_rn(__ddiv_rn(__ldg(roofline_s + jl), __ldg(t + jl)), s), 0.5);
             }
-            for (uint32_t todo = __ballot_sync(FULL, search || is_large); todo; todo &= todo - 1) {
+            for (uint32_t todo = __ballot_sync(FULL, (search || is_large) && lane % LANES == 0); todo; todo &= todo - 1) {
                 const uint32_t src = __ffs(todo) - 1;
                 const uint32_t first = __shfl_sync(FULL, is_large ? g.x : first_slot, src), packed = __shfl_sync(FULL, g.y, src);
                 const uint32_t n = packed & 0x7FFFFFFFu, stride = packed >> 31 ? 1u : 32u;
                 auto key_at = [=](uint32_t a) {
-                    const uint32_t j = unit_at[first + a * stride];
+                    const uint32_t j = unit_at[first + (stride == 1 ? a : a % LANES + 32 * (a / LANES))];
                     return exact_key(__ldg(roofline_s + j), __ldg(t + j), __ldg(ok + j) != 0);
                 };
                 uint32_t usable = 0;
@@ -554,7 +652,7 @@ __global__ void __launch_bounds__(WARP_KERNEL_THREADS, WARP_KERNEL_CTAS)
                 }
                 if (lane == src) s = median_of_keys(k_lo, (usable & 1u) ? k_lo : k_hi, usable & 1u);
             }
-            if (op < n_ops) {
+            if (op < n_ops && lane % LANES == 0) {
                 prod[op] = __dmul_rn(w[op], s);
                 if (s_op_out) s_op_out[(size_t)cand * n_ops + op] = s;
             }
@@ -851,7 +949,8 @@ extern "C" int atrex_score_aggregate(const double* d_roofline_s, const uint32_t*
         std::lock_guard<std::mutex> hold(g_score_lock);
         if (g_score_sms[attr.device] == 0) {
             int v = 0;
-            if (cudaFuncSetAttribute(score_warp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SCORE_SMEM_MAX) != cudaSuccess ||
+            if (cudaFuncSetAttribute(score_warp_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SCORE_SMEM_MAX) != cudaSuccess ||
+                cudaFuncSetAttribute(score_warp_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SCORE_SMEM_MAX) != cudaSuccess ||
                 cudaFuncSetAttribute(score_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SCORE_SMEM_MAX) != cudaSuccess ||
                 cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, attr.device) != cudaSuccess) {
                 cudaGetLastError();
@@ -863,20 +962,34 @@ extern "C" int atrex_score_aggregate(const double* d_roofline_s, const uint32_t*
     }
     const uint32_t n = (uint32_t)n_units, b = (uint32_t)n_candidates;
     ull* errors = reinterpret_cast<ull*>(d_errors);
-    // One candidate per warp pays once there are candidates enough for several warps on every SM, and as
-    // long as an SM's shared memory holds 16 warps' keys; otherwise a CTA works on each candidate.
-    const uint32_t slots = warp_slots(n, n_ops);
+    // One candidate per warp pays once a few warps on every SM have one; a CTA per candidate is quicker for fewer, by
+    // its shorter chain.  Where most groups are too large for the lanes' columns, the warps search them one by
+    // one: later (three rounds of CTAs), and only for small candidates.  A lane to an operator up to a mean group of
+    // 24, two above (8 000 candidates: 440 units in 14 operators 70 -> 29 us, 1 000 units in 25 operators 181 -> 62;
+    // 440 units in 27 operators 31, by pairs 42).
+    const bool pairs = n > 24u * n_ops;
+    const uint32_t slots = warp_slots(n, n_ops, pairs);
     const WarpLayout wl(n, n_ops, slots);
-    const size_t warp_smem = wl.warps + (size_t)wl.warp_bytes * (WARP_KERNEL_THREADS / 32);
-    if (b >= (uint32_t)n_sms * 16u && slots + n < SLOT_MASK && warp_smem * 2 <= SM_SMEM - 2048) {
-        const uint32_t fit = (uint32_t)(SM_SMEM / (warp_smem + 1024)), per_sm = fit < WARP_KERNEL_CTAS ? fit : WARP_KERNEL_CTAS;
-        const uint32_t warps = WARP_KERNEL_THREADS / 32, want = (b + warps - 1) / warps, most = (uint32_t)n_sms * per_sm;
-        score_warp_kernel<<<want < most ? want : most, WARP_KERNEL_THREADS, warp_smem, (cudaStream_t)stream>>>(
+    const bool sorted = n <= 48u * n_ops;
+    uint32_t warps = 0, per_sm = 0;    // the split of an SM's shared memory that holds most warps
+    for (uint32_t c = WARP_KERNEL_CTAS; c >= 1; --c) {
+        const size_t room = SM_SMEM / c - 1024 < (size_t)SCORE_SMEM_MAX ? SM_SMEM / c - 1024 : (size_t)SCORE_SMEM_MAX;
+        uint32_t k = room > wl.warps ? (uint32_t)((room - wl.warps) / wl.warp_bytes) : 0u;
+        if (k > WARP_KERNEL_THREADS / 32) k = WARP_KERNEL_THREADS / 32;
+        if (k * c > warps * per_sm) warps = k, per_sm = c;
+    }
+    const uint32_t sms = (uint32_t)n_sms, held = warps * per_sm;
+    const bool enough = sorted ? b >= 4u * sms && b >= n && held >= (pairs ? 6u : 12u) : b >= 16u * sms && held >= 16 && (n <= 72u * n_ops || n <= 768);
+    if (enough && slots + n < SLOT_MASK) {
+        const uint32_t want = (b + warps - 1) / warps, most = (uint32_t)n_sms * per_sm;
+        const size_t warp_smem = wl.warps + (size_t)wl.warp_bytes * warps;
+        auto* kernel = pairs ? score_warp_kernel<true> : score_warp_kernel<false>;
+        kernel<<<want < most ? want : most, warps * 32, warp_smem, (cudaStream_t)stream>>>(
             d_roofline_s, d_unit_op, n, d_t_cand, d_correct, b, d_w, n_ops, slots, d_s_agg, d_s_op, errors);
     } else {
         const uint32_t threads = n <= 4096 ? 256u : (n <= 13000 ? 512u : 1024u);
         const size_t smem = CtaLayout(n, n_ops, threads).total;
-        uint32_t per_sm = (uint32_t)(SM_SMEM / (smem + 2560));
+        per_sm = (uint32_t)(SM_SMEM / (smem + 2560));
         if (per_sm > 1024u / threads) per_sm = 1024u / threads;   // (64 registers a thread)
         if (per_sm < 1) per_sm = 1;
         const uint32_t most = (uint32_t)n_sms * per_sm;

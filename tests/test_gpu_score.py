@@ -63,10 +63,11 @@ def test_score_limits():
 
 # group sizes at the edges of the lane-sorted columns, the register searches and the shared-memory search
 EDGE_GROUPS = {"lanes": [1, 2, 7, 8, 9, 15, 16, 17, 20, 24, 25, 28, 31, 32, 0, 5], "mixed": [32, 33, 3, 64, 65, 1, 128, 129, 0, 40],
-               "wide": [255, 256, 257, 600, 31, 33], "many": [3, 0, 9, 1] * 40}
+               "wide": [255, 256, 257, 600, 31, 33], "many": [3, 0, 9, 1] * 40,
+               "pairs": [33, 63, 64, 65, 40, 31, 1, 0, 2, 47, 48, 49, 56, 24, 25, 35, 60, 3, 32, 16, 130, 17]}
 
 
-@pytest.mark.parametrize("batch", [3, 2500])       # one candidate per CTA, one per warp
+@pytest.mark.parametrize("batch", [3, 700, 2500])  # one candidate per CTA (small CTAs at 700 and up to 1 024 units), one per warp
 @pytest.mark.parametrize("groups", sorted(EDGE_GROUPS))
 def test_score_parity_at_group_size_edges(groups, batch):
     sizes = EDGE_GROUPS[groups]
