@@ -136,12 +136,13 @@ void compute_layout(const atrex_agg_config_t* c, size_t smem_optin, int n_sms, L
 
 struct DeviceGuard {
     int prev = -1;
+    bool switched = false;
     explicit DeviceGuard(int dev) {
         if (cudaGetDevice(&prev) != cudaSuccess) prev = -1;
-        if (prev != dev) cudaSetDevice(dev);
+        if (prev != dev) switched = cudaSetDevice(dev) == cudaSuccess;
     }
     ~DeviceGuard() {
-        if (prev >= 0) cudaSetDevice(prev);
+        if (switched && prev >= 0) cudaSetDevice(prev);
     }
 };
 

@@ -44,7 +44,8 @@ struct atrex_eq3 {
     uint32_t* d_present = nullptr;   // [n_ops] bit phi: operator i has time in phase phi (cleared by every finalize)
     ull* d_ctl = nullptr;         // [0] rejected, [1] finalize: operators done
     size_t h_bytes = 0;
-    double* h_out = nullptr;      // pinned: w [n_ops], wtilde [n_ops], rejected; then the retained flags [n_ops]
+    double* h_out = nullptr;      // pinned: w [n_ops], wtilde [n_ops], rejected, number of the finalize; then the retained flags [n_ops]
+    ull n_finalized = 0;
     size_t cells = 0;
     double c_total = 0.0;
     bool hi_used = false;
@@ -55,12 +56,13 @@ namespace {
 
 struct Guard {
     int prev = -1;
+    bool switched = false;
     explicit Guard(int dev) {
         if (cudaGetDevice(&prev) != cudaSuccess) prev = -1;
-        if (prev != dev) cudaSetDevice(dev);
+        if (prev != dev) switched = cudaSetDevice(dev) == cudaSuccess;
     }
     ~Guard() {
-        if (prev >= 0) cudaSetDevice(prev);
+        if (prev >= 0 && switched) cudaSetDevice(prev);
     }
 };
 
@@ -204,7 +206,7 @@ constexpr uint32_t WT_CHUNK = 960;    // two terms per computing thread
 
 __global__ void __launch_bounds__(WT_THREADS) eq3_wtilde_kernel(const ull* lo, const ull* hi, const double* den, const double* pa, uint32_t* present,
                                                                 uint32_t n_apps, uint32_t n_ops, uint32_t n_phases, bool any_weight, double* wt,
-                                                                const uint8_t* retained, ull* ctl, double* h_out) {
+                                                                const uint8_t* retained, ull* ctl, double* h_out, ull seq) {
     __shared__ __align__(16) double s_term[2][WT_CHUNK];
     __shared__ double s_total;
     __shared__ bool s_last;
@@ -275,9 +277,13 @@ __global__ void __launch_bounds__(WT_THREADS) eq3_wtilde_kernel(const ull* lo, c
         h_out[k] = retained[k] && s_total > 0.0 ? __ddiv_rn(v, s_total) : 0.0;
         h_out[n_ops + k] = v;
     }
+    __threadfence_system();
+    __syncthreads();
     if (threadIdx.x == 0) {
         reinterpret_cast<ull*>(h_out)[2 * (size_t)n_ops] = ctl[0];
         ctl[1] = 0;
+        __threadfence_system();
+        reinterpret_cast<volatile ull*>(h_out)[2 * (size_t)n_ops + 1] = seq;   // the host waits for this word
     }
 }
 
@@ -347,7 +353,7 @@ int atrex_eq3_create(uint32_t n_apps, uint32_t n_ops, uint32_t n_phases, const u
     const size_t o_ctl = take(16), o_present = take((size_t)n_ops * 4), o_lo = take(cells * 8), o_hi = take(cells * 8),
                  o_den = take((size_t)n_phases * n_apps * 8), o_pa = take((size_t)n_apps * 8), o_wt = take((size_t)n_ops * 8);
     if (e == cudaSuccess) e = cudaMalloc((void**)&h->arena, o);
-    if (e == cudaSuccess) e = pinned_alloc((void**)&h->h_out, h->h_bytes = ((size_t)n_ops * 2 + 1) * 8 + n_ops);
+    if (e == cudaSuccess) e = pinned_alloc((void**)&h->h_out, h->h_bytes = ((size_t)n_ops * 2 + 2) * 8 + n_ops);
     if (e == cudaSuccess) {
         h->d_ctl = (ull*)(h->arena + o_ctl);
         h->d_present = (uint32_t*)(h->arena + o_present);
@@ -411,17 +417,20 @@ int atrex_eq3_finalize(atrex_eq3_t* h, const uint8_t* h_retained, double* h_w, d
     cudaStream_t s = (cudaStream_t)stream;
     const uint32_t n_ops = h->n_ops;
     // the flags are read and the results written by the kernels, in pinned memory
-    uint8_t* retained = (uint8_t*)(h->h_out + 2 * (size_t)n_ops + 1);
+    uint8_t* retained = (uint8_t*)(h->h_out + 2 * (size_t)n_ops + 2);
     if (h_retained) memcpy(retained, h_retained, n_ops);
     else memset(retained, 1, n_ops);
     const ull* hi = h->hi_used ? h->d_hi : nullptr;
+    const volatile ull* done = (const volatile ull*)h->h_out + 2 * (size_t)n_ops + 1;
+    const ull seq = ++h->n_finalized;
+    *(volatile ull*)done = 0;    // (a block from the pool holds whatever its last owner left)
     eq3_app_totals_kernel<<<dim3((h->n_apps + 31) / 32, h->n_phases), TOTAL_WARPS * 32, 0, s>>>(h->d_lo, hi, h->n_apps, n_ops, h->d_den, h->d_present);
     if (cudaGetLastError() != cudaSuccess) return ATREX_ERR_CUDA;
     const bool any_weight = h->c_total != 0.0;
     if (launch_chained(eq3_wtilde_kernel, n_ops, WT_THREADS, 0, s, h->d_lo, hi, h->d_den, h->d_pa, h->d_present, h->n_apps, n_ops, h->n_phases,
-                       any_weight, h->d_wt, retained, h->d_ctl, h->h_out) != cudaSuccess)
+                       any_weight, h->d_wt, retained, h->d_ctl, h->h_out, seq) != cudaSuccess)
         return ATREX_ERR_CUDA;
-    if (cudaStreamSynchronize(s) != cudaSuccess) return ATREX_ERR_CUDA;
+    if (wait_for_kernel([=] { return *done == seq; }, s) != cudaSuccess) return ATREX_ERR_CUDA;
     memcpy(h_w, h->h_out, (size_t)n_ops * 8);
     if (h_wtilde) memcpy(h_wtilde, h->h_out + n_ops, (size_t)n_ops * 8);
     if (h_rejected) memcpy(h_rejected, h->h_out + 2 * (size_t)n_ops, 8);

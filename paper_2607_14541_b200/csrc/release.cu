@@ -431,7 +431,8 @@ constexpr uint32_t TILE_CAP = 6144;         // ... and has at most this many ite
 constexpr uint32_t TILE_LOCAL_BINS = 4096, TILE_THREADS = 512;
 constexpr uint32_t TILE_CLASH_MAX = 24;     // larger local bins send the tile to the comparison network
 constexpr size_t TILE_SMEM = (size_t)TILE_CAP * 8 + TILE_LOCAL_BINS * 4;    // three CTAs per SM
-constexpr uint32_t SMALL_SORT_MAX = 4096;   // up to here one CTA does everything
+constexpr uint32_t COUNT_SORT_MAX = 8192;   // up to here one kernel ranks every key by counting
+constexpr int REPORT_SLOTS = 32;
 
 struct BinCtl {                  // at the start of the scratch, cleared by every call (with the bins behind it)
     ull counter;                 // items (entries of the phase)
@@ -446,7 +447,23 @@ static_assert(sizeof(BinCtl) == 128, "half of the control block");
 
 struct BinReport {               // in pinned host memory, written by the kernels
     ull overflow, counter, total_lo, total_hi, n_keep, covered_lo, covered_hi, too_large;
+    ull done;                    // the call's last kernel is through
+    ull pad[7];
 };
+// CTAs of a call's last kernel that are through, by the call's report slot; back at 0 after the last one
+__device__ uint32_t g_finished[REPORT_SLOTS];
+
+// The last act of every CTA of a call's last kernel (all of its threads): the last CTA tells the host, which
+// notices that several microseconds before the stream counts as idle.
+__device__ __forceinline__ void finish_call(BinReport* report, uint32_t slot) {
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    __threadfence();
+    if (atomicInc(&g_finished[slot], gridDim.x - 1) == gridDim.x - 1) {
+        __threadfence_system();
+        *(volatile ull*)&report->done = 1;
+    }
+}
 
 struct BinSort {                 // what the kernels share
     BinCtl* ctl;
@@ -464,6 +481,7 @@ struct BinSort {                 // what the kernels share
     uint32_t n;                  // upper bound of the item count
     uint32_t bits;
     bool ranking;
+    uint32_t slot;               // the report's number
 };
 
 __device__ __forceinline__ uint32_t item_count(const BinSort& b) { return b.ranking ? (uint32_t)b.ctl->counter : b.n; }
@@ -919,10 +937,11 @@ __global__ void __launch_bounds__(TILE_THREADS) bin_tile_kernel(const BinSort b,
     __shared__ ull s_sum[2];
     __shared__ uint32_t s_range[2];
     grid_dependency_wait();
-    if (b.ctl->overflow) return;
-    const uint32_t first = b.tile_start[blockIdx.x], n = b.tile_start[blockIdx.x + 1] - first;
+    const bool overflow = b.ctl->overflow;
+    const uint32_t first = overflow ? 0u : b.tile_start[blockIdx.x], n = overflow ? 0u : b.tile_start[blockIdx.x + 1] - first;
     if (n == 0) {
-        if (b.ranking && threadIdx.x < 2) b.tile_sum[2 * blockIdx.x + threadIdx.x] = 0;
+        if (!b.ranking) finish_call(b.report, b.slot);
+        else if (!overflow && threadIdx.x < 2) b.tile_sum[2 * blockIdx.x + threadIdx.x] = 0;
         return;
     }
     uint32_t top = 0, ntop = 0;
@@ -945,7 +964,10 @@ __global__ void __launch_bounds__(TILE_THREADS) bin_tile_kernel(const BinSort b,
     if (threadIdx.x < 2) s_sum[threadIdx.x] = 0;
     ulonglong2 sum = make_ulonglong2(0, 0);
     gather_tile(b.entries, s_item, n, out, first, out_cap, sum);
-    if (!b.ranking) return;
+    if (!b.ranking) {
+        finish_call(b.report, b.slot);
+        return;
+    }
     for (uint32_t i = threadIdx.x; i < n; i += TILE_THREADS) {   // rows that are not wanted: their order is kept for the shares
         if (first + i < out_cap) continue;
         const uint32_t at = (uint32_t)s_item[i];
@@ -964,52 +986,68 @@ __global__ void __launch_bounds__(TILE_THREADS) bin_tile_kernel(const BinSort b,
     if (threadIdx.x < 2) b.tile_sum[2 * blockIdx.x + threadIdx.x] = s_sum[threadIdx.x];
 }
 
-// Key order of up to SMALL_SORT_MAX entries, all of it in one CTA.
-__global__ void __launch_bounds__(1024) small_sort_kernel(const atrex_entry_t* entries, uint32_t n, atrex_entry_t* out, BinReport* report) {
+// Key order of up to COUNT_SORT_MAX entries in one kernel: an entry's place is the number of keys before its own.
+// Every CTA reads all keys (32 bytes of L2 each: 1 us of an SM's bandwidth for 4 096) and places 32 U entries, a
+// lane each (U of them), every warp counting over its own sixteenth of the keys.  Bound by latency: 4 096 entries
+// in 9 us (sorted by one CTA in shared memory: 16), the call 15 us, 8 000 entries 24 (binned sort: 37).  (Keys read
+// once per cluster of eight and handed round through distributed shared memory: slower, 4 096 remote stores into
+// each SM take 10 us.)
+constexpr uint32_t COUNT_THREADS = 512, COUNT_LOADS = 8;
+template <uint32_t U>
+__global__ void __launch_bounds__(COUNT_THREADS) count_sort_kernel(const atrex_entry_t* entries, uint32_t n, atrex_entry_t* out, BinReport* report, uint32_t slot) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    ull* s_item = reinterpret_cast<ull*>(smem_raw);
-    uint32_t* s_local = reinterpret_cast<uint32_t*>(s_item + TILE_CAP);
-    __shared__ ull s_part[32];
-    __shared__ BinCtl s_ctl;
-    ull key[SMALL_SORT_MAX / 1024];
-    ull mp = 0, mo = 0, ms = 0;
+    ull* s_key = reinterpret_cast<ull*>(smem_raw);   // [n, rounded up to an even number]
+    __shared__ uint32_t s_place[32 * U];
+    const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5, base = blockIdx.x * 32 * U;
+    for (uint32_t i = threadIdx.x; i < 32 * U; i += COUNT_THREADS) s_place[i] = 0;
     grid_dependency_wait();
+    for (uint32_t i0 = threadIdx.x; i0 < n; i0 += COUNT_LOADS * COUNT_THREADS) {
+        ull key[COUNT_LOADS];
 #pragma unroll
-    for (uint32_t u = 0; u < SMALL_SORT_MAX / 1024; ++u) {
-        const uint32_t i = threadIdx.x + u * 1024;
-        key[u] = i < n ? entries[i].key : 0ull;
-    }
+        for (uint32_t u = 0; u < COUNT_LOADS; ++u) key[u] = i0 + u * COUNT_THREADS < n ? entries[i0 + u * COUNT_THREADS].key : 0ull;
 #pragma unroll
-    for (uint32_t u = 0; u < SMALL_SORT_MAX / 1024; ++u) {
-        mp = max_ull(mp, key[u] >> 48);
-        mo = max_ull(mo, (key[u] >> 32) & 0xFFFFu);
-        ms = max_ull(ms, key[u] & 0xFFFFFFFFull);
+        for (uint32_t u = 0; u < COUNT_LOADS; ++u)
+            if (i0 + u * COUNT_THREADS < n) s_key[i0 + u * COUNT_THREADS] = key[u];
     }
-    mp = block_reduce(mp, max_ull, s_part);
-    mo = block_reduce(mo, max_ull, s_part);
-    ms = block_reduce(ms, max_ull, s_part);
-    if (threadIdx.x == 0) {
-        s_ctl.max_phase = mp;
-        s_ctl.max_op = mo;
-        s_ctl.max_shape = ms;
-    }
+    if (threadIdx.x == 0 && (n & 1u)) s_key[n] = ~0ull;   // (before nothing)
+    grid_dependents_launch();
     __syncthreads();
-    const KeyRadix radix(&s_ctl);
-    const ull span = (s_ctl.max_phase + 1) * radix.ops * radix.shapes - 1;
-    const int len = 64 - __clzll((long long)span), shift = len > 32 ? len - 32 : 0;
-    sort_tile(entries, false, n, 0u, (uint32_t)(span >> shift), [&](uint32_t i) {
-        ull k = key[0];
+    ull mine[U];
+    uint32_t before[U];
 #pragma unroll
-        for (uint32_t u = 1; u < SMALL_SORT_MAX / 1024; ++u) k = i / 1024 == u ? key[u] : k;
-        return radix.word(k) >> shift << 32 | i;
-    }, s_item, s_local);
-    ulonglong2 unused = make_ulonglong2(0, 0);
-    gather_tile(entries, s_item, n, out, 0, n, unused);
-    __syncthreads();
-    if (threadIdx.x == 0) {   // the host waits for this word
-        __threadfence_system();
-        *(volatile ull*)&report->counter = 1;
+    for (uint32_t u = 0; u < U; ++u) {
+        mine[u] = base + u * 32 + lane < n ? s_key[base + u * 32 + lane] : 0ull;
+        before[u] = 0;
     }
+    // equal keys keep their input order: those at lower positions count too
+    const uint32_t per = ((n + COUNT_THREADS / 32 - 1) / (COUNT_THREADS / 32) + 1) & ~1u, first = min((n + 1) & ~1u, w * per), end = min((n + 1) & ~1u, first + per);
+    const uint32_t own = min(max(base, first), end), behind = min(max(base + 32 * U, first), end);   // (all of these are even)
+    const ulonglong2* pair = reinterpret_cast<const ulonglong2*>(s_key);
+#pragma unroll 8
+    for (uint32_t i = first / 2; i < own / 2; ++i) {
+        const ulonglong2 key = pair[i];
+#pragma unroll
+        for (uint32_t u = 0; u < U; ++u) before[u] += (key.x <= mine[u] ? 1u : 0u) + (key.y <= mine[u] ? 1u : 0u);
+    }
+    for (uint32_t i = own; i < behind; ++i) {
+        const ull key = s_key[i];
+#pragma unroll
+        for (uint32_t u = 0; u < U; ++u) before[u] += key < mine[u] || (key == mine[u] && i < base + u * 32 + lane) ? 1u : 0u;
+    }
+#pragma unroll 8
+    for (uint32_t i = behind / 2; i < end / 2; ++i) {
+        const ulonglong2 key = pair[i];
+#pragma unroll
+        for (uint32_t u = 0; u < U; ++u) before[u] += (key.x < mine[u] ? 1u : 0u) + (key.y < mine[u] ? 1u : 0u);
+    }
+#pragma unroll
+    for (uint32_t u = 0; u < U; ++u)
+        if (before[u]) atomicAdd(&s_place[u * 32 + lane], before[u]);
+    __syncthreads();
+    const ull* src = reinterpret_cast<const ull*>(entries + base);
+    ull* dst = reinterpret_cast<ull*>(out);
+    for (uint32_t x = threadIdx.x; x < min(32 * U, n - base) * 6; x += COUNT_THREADS) dst[(size_t)s_place[x / 6] * 6 + x % 6] = src[x];
+    finish_call(report, slot);
 }
 
 // 6. (ranking) exclusive scan of the tiles' weighted times, and the sum the coverage cut needs: the smallest
@@ -1063,7 +1101,10 @@ __global__ void __launch_bounds__(SCAN_BLOCK) bin_tile_scan_kernel(const BinSort
 __global__ void __launch_bounds__(SCAN_BLOCK) bin_share_kernel(const BinSort b, const atrex_entry_t* ranked, double* cum, uint32_t out_cap) {
     __shared__ ull warp_tot[32][2];
     grid_dependency_wait();
-    if (b.ctl->overflow) return;
+    if (b.ctl->overflow) {
+        finish_call(b.report, b.slot);
+        return;
+    }
     const uint32_t first = b.tile_start[blockIdx.x], end = b.tile_start[blockIdx.x + 1];
     const ull total_lo = b.ctl->total_lo, total_hi = b.ctl->total_hi, need_lo = b.ctl->need_lo, need_hi = b.ctl->need_hi;
     const double total = u128_to_f64_rn(total_hi, total_lo);
@@ -1086,12 +1127,14 @@ __global__ void __launch_bounds__(SCAN_BLOCK) bin_share_kernel(const BinSort b, 
                 b.report->n_keep = (ull)r + 1;
                 b.report->covered_lo = lo;
                 b.report->covered_hi = hi;
+                __threadfence_system();
             }
             if (r < out_cap) cum[r] = (total_lo | total_hi) ? __ddiv_rn(u128_to_f64_rn(hi, lo), total) : 0.0;
         }
         add128(run_lo, run_hi, blo, bhi);
         __syncthreads();  // warp_tot is reused by the next round
     }
+    finish_call(b.report, b.slot);
 }
 
 // ---- host side
@@ -1166,7 +1209,7 @@ int prepare_sort_kernels(int* n_sms) {
             cudaFuncSetAttribute(bin_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 << BIN_BITS_MAX) != cudaSuccess ||
             cudaFuncSetAttribute(bin_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(4 * CURSORS_MAX + (2 << BIN_BITS_MAX))) != cudaSuccess ||
             cudaFuncSetAttribute(bin_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(small_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM) != cudaSuccess ||
+            cudaFuncSetAttribute(count_sort_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(COUNT_SORT_MAX * 8)) != cudaSuccess ||
             cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
             cudaGetLastError();
             return ATREX_ERR_CUDA;
@@ -1218,9 +1261,15 @@ public:
     ReportSlot(const ReportSlot&) = delete;
     ReportSlot& operator=(const ReportSlot&) = delete;
     BinReport* get() const { return slot_ < 0 ? nullptr : pool() + slot_; }
+    uint32_t number() const { return (uint32_t)slot_; }
+    // waits for the call's last kernel (finish_call)
+    cudaError_t wait(cudaStream_t s) const {
+        const volatile ull* done = &get()->done;
+        return wait_for_kernel([=] { return *done != 0; }, s);
+    }
 
 private:
-    static constexpr int SLOTS = 32;
+    static constexpr int SLOTS = REPORT_SLOTS;
     static std::mutex& lock() { static std::mutex m; return m; }
     static std::condition_variable& freed() { static std::condition_variable c; return c; }
     static BinReport*& pool() { static BinReport* p = nullptr; return p; }
@@ -1229,12 +1278,13 @@ private:
 };
 
 // The scratch as the binned sort uses it.
-BinSort carve_bins(void* base, const atrex_entry_t* entries, uint64_t n, bool ranking, BinReport* report) {
+BinSort carve_bins(void* base, const atrex_entry_t* entries, uint64_t n, bool ranking, const ReportSlot& slot) {
     unsigned char* p = (unsigned char*)base;
     const uint64_t tiles = (n + TILE_STEP - 1) / TILE_STEP;
     BinSort b;
     b.ctl = (BinCtl*)p;
-    b.report = report;
+    b.report = slot.get();
+    b.slot = slot.number();
     b.entries = entries;
     b.n = (uint32_t)n;
     b.ranking = ranking;
@@ -1300,21 +1350,23 @@ extern "C" int atrex_entries_sort_by_key(const atrex_entry_t* d_entries, uint64_
     const uint32_t m = (uint32_t)n;
     int n_sms = 0;
     if (prepare_sort_kernels(&n_sms) != ATREX_OK) return ATREX_ERR_CUDA;
-    if (n <= SMALL_SORT_MAX) {
+    if (n <= COUNT_SORT_MAX) {   // (above, counting takes longer than the binned sort's launches)
         ReportSlot report;
         if (!report.get()) return ATREX_ERR_NOMEM;
-        if (launch_chained(small_sort_kernel, 1, 1024, TILE_SMEM, s, d_entries, m, d_out, report.get()) != cudaSuccess) return ATREX_ERR_CUDA;
-        const volatile ull* done = &report.get()->counter;
-        return wait_for_kernel([=] { return *done != 0; }, s) == cudaSuccess ? ATREX_OK : ATREX_ERR_CUDA;
+        const uint32_t per_cta = n <= 4096 ? 32 : 64, grid = (m + per_cta - 1) / per_cta;
+        auto* kernel = n <= 4096 ? count_sort_kernel<1> : count_sort_kernel<2>;
+        if (launch_chained(kernel, grid, COUNT_THREADS, (size_t)(m + 1) / 2 * 16, s, d_entries, m, d_out, report.get(), report.number()) != cudaSuccess)
+            return ATREX_ERR_CUDA;
+        return report.wait(s) == cudaSuccess ? ATREX_OK : ATREX_ERR_CUDA;
     }
     {
         ReportSlot report;
         if (!report.get()) return ATREX_ERR_NOMEM;
-        const BinSort b = carve_bins(d_scratch, d_entries, n, false, report.get());
+        const BinSort b = carve_bins(d_scratch, d_entries, n, false, report);
         if (cudaMemsetAsync(b.ctl, 0, sizeof(BinCtl) + (4ull << b.bits), s) != cudaSuccess) return ATREX_ERR_CUDA;
         const uint32_t want = (m + 4 * BIN_THREADS - 1) / (4 * BIN_THREADS), most = 4u * (uint32_t)n_sms;
         if (launch_chained(bin_keys_kernel, want < most ? want : most, BIN_THREADS, 0, s, b) != cudaSuccess ||
-            launch_bins(b, d_out, n, n_sms, s) != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
+            launch_bins(b, d_out, n, n_sms, s) != cudaSuccess || report.wait(s) != cudaSuccess)
             return ATREX_ERR_CUDA;
         if (!((volatile BinReport*)report.get())->overflow) return ATREX_OK;
     }
@@ -1356,7 +1408,7 @@ extern "C" int atrex_entries_rank(const atrex_entry_t* d_entries, uint64_t n, ui
     {
         ReportSlot slot;
         if (!slot.get()) return ATREX_ERR_NOMEM;
-        const BinSort b = carve_bins(d_scratch, d_entries, n, true, slot.get());
+        const BinSort b = carve_bins(d_scratch, d_entries, n, true, slot);
         if (cudaMemsetAsync(b.ctl, 0, sizeof(BinCtl) + (4ull << b.bits), s) != cudaSuccess) return ATREX_ERR_CUDA;
         const uint32_t want = ((uint32_t)n + 4 * BIN_THREADS - 1) / (4 * BIN_THREADS), most = 4u * (uint32_t)n_sms;
         const uint32_t tiles = ((uint32_t)n + TILE_STEP - 1) / TILE_STEP, cap = (uint32_t)(out_cap < n ? out_cap : n);
@@ -1364,7 +1416,7 @@ extern "C" int atrex_entries_rank(const atrex_entry_t* d_entries, uint64_t n, ui
             launch_bins(b, d_ranked, cap, n_sms, s) != cudaSuccess ||
             launch_chained(bin_tile_scan_kernel, 1, SCAN_BLOCK, 0, s, b, coverage_ppm) != cudaSuccess ||
             launch_chained(bin_share_kernel, tiles, SCAN_BLOCK, 0, s, b, d_ranked, d_cum_share, cap) != cudaSuccess ||
-            cudaStreamSynchronize(s) != cudaSuccess)
+            slot.wait(s) != cudaSuccess)
             return ATREX_ERR_CUDA;
         const volatile BinReport* r = slot.get();
         if (r->too_large || !r->overflow) {

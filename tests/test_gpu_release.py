@@ -247,3 +247,13 @@ def test_binned_sort_at_its_edges(lib, n, shape):
     assert host(lib.sort_entries_by_key(d, n), oracle.ENTRY_DTYPE).tobytes() == oracle.sort_by_key(e).tobytes()
     check_rank(lib, e, d, n, (0, 7), ppms=(0, 500_000, 1_000_000))
     check_rank(lib, e, d, n, (0,), ppms=(900_000,), out_cap=n // 2)
+
+
+@pytest.mark.parametrize("n", [33, 257, 4_096, 4_097, 8_192, 8_193])
+def test_equal_keys_keep_their_order(lib, n):
+    """A list put together from several shards holds a key more than once: same order as in the input."""
+    rng = np.random.default_rng(n)
+    e = np.zeros(n, dtype=oracle.ENTRY_DTYPE)
+    e["key"] = rng.integers(0, max(2, n // 5), n).astype(np.uint64) << np.uint64(30)
+    e["count"] = np.arange(n)
+    assert host(lib.sort_entries_by_key(dev(e), n), oracle.ENTRY_DTYPE).tobytes() == e[np.argsort(e["key"], kind="stable")].tobytes()
