@@ -428,9 +428,10 @@ constexpr uint32_t SHARE_THREADS = 1024;     // counting and moving: one CTA per
 constexpr uint32_t CURSORS_MAX = 1u << 14;
 constexpr uint32_t TILE_STEP = 2048;        // a tile is the bins that start in one such window of positions
 constexpr uint32_t TILE_CAP = 6144;         // ... and has at most this many items
-constexpr uint32_t TILE_LOCAL_BINS = 4096, TILE_THREADS = 512;
-constexpr uint32_t TILE_CLASH_MAX = 24;     // larger local bins send the tile to the comparison network
-constexpr size_t TILE_SMEM = (size_t)TILE_CAP * 8 + TILE_LOCAL_BINS * 4;    // three CTAs per SM
+constexpr uint32_t TILE_LOCAL_BINS = 4096, TILE_THREADS = 512, TILE_HELD = 5, GATHER_LOADS = 6;
+constexpr uint32_t TILE_CLASH_MAX = 24;     // larger local bins are crowded: some are sorted by a warp or the CTA each,
+constexpr uint32_t TILE_CROWDED = 32;       // more of them, or larger ones, send the tile to the comparison network
+constexpr size_t TILE_SMEM = (size_t)TILE_CAP * 8 + TILE_LOCAL_BINS * 4;    // (what it leaves of two CTAs is L1 for the gather)
 constexpr uint32_t COUNT_SORT_MAX = 8192;   // up to here one kernel ranks every key by counting
 constexpr int REPORT_SLOTS = 32;
 
@@ -482,6 +483,7 @@ struct BinSort {                 // what the kernels share
     uint32_t bits;
     bool ranking;
     uint32_t slot;               // the report's number
+    uint32_t turns;              // parts of the cursors that step 4 serves one after the other
 };
 
 __device__ __forceinline__ uint32_t item_count(const BinSort& b) { return b.ranking ? (uint32_t)b.ctl->counter : b.n; }
@@ -753,7 +755,8 @@ __global__ void __launch_bounds__(1024) bin_scan_kernel(const BinSort b) {
 // 4. items to their tiles (or bins, where there are more tiles than a CTA can keep cursors for), in any order
 //    within: the CTA counts its share once more, reserves a range at each cursor with one global atomic, and
 //    writes.  Cursors per tile make for runs twice as long as cursors per bin, which keeps the partly written
-//    sectors of all CTAs within L2 (16.3 M items: 456 -> 190 us).
+//    sectors of all CTAs within L2.  From 2 048 cursors on those would take 40 MB and more: the CTAs go over their
+//    shares twice, for one half of the cursors each time (15 M items: 396 -> 300 us; three and four times: the same).
 __global__ void __launch_bounds__(SHARE_THREADS) bin_scatter_kernel(const BinSort b) {
     extern __shared__ __align__(16) uint32_t s_cursor[];                       // [n_cursors]
     uint16_t* s_place = reinterpret_cast<uint16_t*>(s_cursor + b.n_cursors);   // [1 << bits]
@@ -771,21 +774,26 @@ __global__ void __launch_bounds__(SHARE_THREADS) bin_scatter_kernel(const BinSor
     for (uint32_t i = threadIdx.x; i < b.n_cursors; i += SHARE_THREADS)
         if (s_cursor[i]) s_cursor[i] = atomicAdd(&b.cursors[i], s_cursor[i]);
     __syncthreads();
-    for (uint32_t i0 = first + threadIdx.x; i0 < end; i0 += 4 * SHARE_THREADS) {
-        ull w[4];
-        uint32_t idx[4];
+    const uint32_t span = (b.n_cursors + b.turns - 1) / b.turns;
+    for (uint32_t turn = 0; turn < b.turns; ++turn) {
+        for (uint32_t i0 = first + threadIdx.x; i0 < end; i0 += 4 * SHARE_THREADS) {
+            ull w[4];
+            uint32_t idx[4];
 #pragma unroll
-        for (uint32_t u = 0; u < 4; ++u) {
-            const uint32_t i = i0 + u * SHARE_THREADS;
-            w[u] = i < end ? b.words[i] : 0ull;
-            idx[u] = b.ranking && i < end ? b.idx[i] : i;
-        }
+            for (uint32_t u = 0; u < 4; ++u) {
+                const uint32_t i = i0 + u * SHARE_THREADS;
+                w[u] = i < end ? b.words[i] : 0ull;
+                idx[u] = b.ranking && i < end ? b.idx[i] : i;
+            }
 #pragma unroll
-        for (uint32_t u = 0; u < 4; ++u) {
-            if (i0 + u * SHARE_THREADS >= end) continue;
-            if (!b.ranking) w[u] = radix.word(w[u]);
-            const uint32_t pos = atomicAdd(&s_cursor[s_place[range.bin(w[u])]], 1u);
-            b.items[pos] = range.item(w[u], idx[u]);
+            for (uint32_t u = 0; u < 4; ++u) {
+                if (i0 + u * SHARE_THREADS >= end) continue;
+                if (!b.ranking) w[u] = radix.word(w[u]);
+                const uint32_t to = s_place[range.bin(w[u])];
+                if (to - turn * span >= span) continue;
+                const uint32_t pos = atomicAdd(&s_cursor[to], 1u);
+                b.items[pos] = range.item(w[u], idx[u]);
+            }
         }
     }
 }
@@ -802,23 +810,109 @@ __device__ __forceinline__ bool item_less(const atrex_entry_t* entries, bool ran
     return x < y;               // equal keys keep their input order
 }
 
-// Sorts n <= TILE_CAP items whose leading bits lie in [low, high] into s_item.  `load(i)` gives item i (twice).  Each item goes to one of 4 096 local bins of equal width -- less than one item per bin, so that
-// a thread puts a bin in order by insertion; crowded local bins (words that cluster) send the whole tile
-// through a bitonic network instead, with absent items behind the last one.
-template <typename Load>
-__device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ranking, uint32_t n, uint32_t low, uint32_t high, Load load, ull* s_item,
+// Every comparator of this form of the bitonic network puts the smaller element at the lower position, so that
+// positions at or beyond n can be left out (whole CTA).
+template <typename Less, typename Swap>
+__device__ __forceinline__ void bitonic(uint32_t n, Less less, Swap swap) {
+    const int bits = n > 1 ? 32 - __clz((int)(n - 1)) : 0;
+    for (int k = 1; k <= bits; ++k) {
+        for (int j = k - 1; j >= 0; --j) {
+            for (uint32_t t = threadIdx.x; t < 1u << (bits - 1); t += blockDim.x) {
+                const uint32_t lo = (t >> j) << (j + 1) | (t & ((1u << j) - 1u)), in = (1u << k) - 1u;
+                const uint32_t hi = j == k - 1 ? (lo | in) - (lo & in) : lo + (1u << j);
+                if (hi < n && less(hi, lo)) swap(hi, lo);
+            }
+            __syncthreads();
+        }
+    }
+}
+
+// A crowded local bin of n items in order: the network over copies of their entries' weights and
+// keys in shared memory (whole CTA).  (3.2 M entries of two phases, some 800 of each at the clamp of their weights:
+// the network over the whole tile, reading entries at every comparison, took that one tile 110 us, longer than
+// all others together.)
+__device__ __noinline__ void sort_crowded_bin(const atrex_entry_t* entries, bool ranking, ull* s_item, uint32_t n, ull* s_key, ull* s_lo, ull* s_hi) {
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
+        const atrex_entry_t* e = entries + (uint32_t)s_item[i];
+        s_key[i] = e->key;
+        s_lo[i] = ranking ? e->wt_lo : 0ull;
+        s_hi[i] = ranking ? e->wt_hi : 0ull;
+    }
+    __syncthreads();
+    bitonic(n, [&](uint32_t a, uint32_t b) {
+        const ull x = s_item[a], y = s_item[b];
+        if ((x ^ y) >> 32) return x < y;
+        if (s_hi[a] != s_hi[b]) return s_hi[a] > s_hi[b];
+        if (s_lo[a] != s_lo[b]) return s_lo[a] > s_lo[b];
+        if (s_key[a] != s_key[b]) return s_key[a] < s_key[b];
+        return x < y;           // equal keys keep their input order
+    }, [&](uint32_t a, uint32_t b) {
+        ull x = s_item[a]; s_item[a] = s_item[b]; s_item[b] = x;
+        x = s_key[a]; s_key[a] = s_key[b]; s_key[b] = x;
+        x = s_lo[a]; s_lo[a] = s_lo[b]; s_lo[b] = x;
+        x = s_hi[a]; s_hi[a] = s_hi[b]; s_hi[b] = x;
+    });
+}
+
+// A crowded local bin of up to 64 items by one warp: every lane counts the items before its own two.
+__device__ __forceinline__ void sort_small_bin(const atrex_entry_t* entries, bool ranking, ull* s_item, uint32_t n) {
+    const uint32_t lane = threadIdx.x & 31u;
+    ull item[2], hi[2], lo[2], key[2];
+    uint32_t before[2] = {0, 0};
+#pragma unroll
+    for (uint32_t u = 0; u < 2; ++u) {
+        const bool in = u * 32 + lane < n;
+        item[u] = in ? s_item[u * 32 + lane] : ~0ull;
+        const atrex_entry_t* e = entries + (in ? (uint32_t)item[u] : 0u);
+        hi[u] = in && ranking ? e->wt_hi : 0ull;
+        lo[u] = in && ranking ? e->wt_lo : 0ull;
+        key[u] = in ? e->key : 0ull;
+    }
+#pragma unroll
+    for (uint32_t v = 0; v < 2; ++v) {
+        for (uint32_t j = 0; j < 32 && v * 32 + j < n; ++j) {
+            const ull y = __shfl_sync(FULL, item[v], j), y_hi = __shfl_sync(FULL, hi[v], j), y_lo = __shfl_sync(FULL, lo[v], j),
+                      y_key = __shfl_sync(FULL, key[v], j);
+#pragma unroll
+            for (uint32_t u = 0; u < 2; ++u) {
+                bool less = y < item[u];            // equal keys keep their input order
+                if (!((y ^ item[u]) >> 32)) {
+                    if (y_key != key[u]) less = y_key < key[u];
+                    if (y_lo != lo[u]) less = y_lo > lo[u];
+                    if (y_hi != hi[u]) less = y_hi > hi[u];
+                }
+                before[u] += less ? 1u : 0u;
+            }
+        }
+    }
+    __syncwarp();
+#pragma unroll
+    for (uint32_t u = 0; u < 2; ++u)
+        if (u * 32 + lane < n) s_item[before[u]] = item[u];
+}
+
+// Sorts n <= TILE_CAP items whose leading bits lie in [low, high] into s_item.  `each(f)` calls f with each of
+// this thread's items (twice).  Each item goes to one of 4 096 local bins of equal width -- less than one item per bin, so that
+// a thread puts a bin in order by insertion; a few crowded local bins (hundreds of equal weights, say) go
+// through a bitonic network each, many of them send the whole tile through a bitonic network, with absent items behind the last one.
+template <typename Each>
+__device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ranking, uint32_t n, uint32_t low, uint32_t high, Each each, ull* s_item,
                                           uint32_t* s_local) {
     __shared__ uint32_t s_warp[32];
-    __shared__ uint32_t s_crowded;
+    __shared__ uint32_t s_crowded, s_bin[TILE_CROWDED];
     const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
     const int len = 32 - __clz((int)(high - low));
     const int shift = len > 12 ? len - 12 : 0;
     for (uint32_t i = threadIdx.x; i < TILE_LOCAL_BINS; i += blockDim.x) s_local[i] = 0;
     if (threadIdx.x == 0) s_crowded = 0;
     __syncthreads();
-    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
-        if (atomicAdd(&s_local[((uint32_t)(load(i) >> 32) - low) >> shift], 1u) >= TILE_CLASH_MAX) s_crowded = 1;
-    }
+    each([&](ull item) {
+        const uint32_t d = ((uint32_t)(item >> 32) - low) >> shift;
+        if (atomicAdd(&s_local[d], 1u) == TILE_CLASH_MAX) {
+            const uint32_t at = atomicAdd(&s_crowded, 1u);
+            if (at < TILE_CROWDED) s_bin[at] = d;
+        }
+    });
     __syncthreads();
     // exclusive scan of the local bins: each thread a run of them
     const uint32_t per = TILE_LOCAL_BINS / blockDim.x, first = threadIdx.x * per;
@@ -849,15 +943,26 @@ __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ran
         at += c;
     }
     __syncthreads();
-    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
-        const ull item = load(i);
-        s_item[atomicAdd(&s_local[((uint32_t)(item >> 32) - low) >> shift], 1u)] = item;
-    }
+    each([&](ull item) { s_item[atomicAdd(&s_local[((uint32_t)(item >> 32) - low) >> shift], 1u)] = item; });
     __syncthreads();
-    if (!s_crowded) {
-        // (a bin's cursor now stands at its end, its predecessor's at its start)
+    // (a bin's cursor now stands at its end, its predecessor's at its start)
+    const uint32_t crowded = s_crowded;
+    const uint32_t room = (TILE_CAP - n) / 3;    // (behind the items there is room for so many copies)
+    bool by_bins = crowded <= TILE_CROWDED;
+    for (uint32_t k = 0; by_bins && k < crowded; ++k) by_bins = s_local[s_bin[k]] - (s_bin[k] ? s_local[s_bin[k] - 1] : 0u) <= room;
+    if (by_bins) {
+        for (uint32_t k = w; k < crowded; k += n_warps) {
+            const uint32_t d = s_bin[k], b0 = d ? s_local[d - 1] : 0u;
+            if (s_local[d] - b0 <= 64) sort_small_bin(entries, ranking, s_item + b0, s_local[d] - b0);
+        }
+        for (uint32_t k = 0; k < crowded; ++k) {     // (the same for every thread)
+            const uint32_t d = s_bin[k], b0 = d ? s_local[d - 1] : 0u;
+            if (s_local[d] - b0 <= 64) continue;
+            sort_crowded_bin(entries, ranking, s_item + b0, s_local[d] - b0, s_item + n, s_item + n + room, s_item + n + 2 * room);
+        }
         for (uint32_t d = threadIdx.x; d < TILE_LOCAL_BINS; d += blockDim.x) {
             const uint32_t b0 = d ? s_local[d - 1] : 0u, b1 = s_local[d];
+            if (b1 - b0 > TILE_CLASH_MAX) continue;
             for (uint32_t i = b0 + 1; i < b1; ++i) {
                 const ull item = s_item[i];
                 uint32_t j = i;
@@ -869,24 +974,8 @@ __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ran
             }
         }
     } else {
-        // every comparator of this form of the network puts the smaller item at the lower position, so that
-        // positions at or beyond n can be left out
-        uint32_t pow2 = 2;
-        while (pow2 < n) pow2 <<= 1;
-        for (uint32_t k = 2; k <= pow2; k <<= 1) {
-            for (uint32_t j = k >> 1; j; j >>= 1) {
-                for (uint32_t t = threadIdx.x; t < pow2 / 2; t += blockDim.x) {
-                    const uint32_t lo = (t / j) * 2 * j + (t & (j - 1));
-                    const uint32_t hi = j == k >> 1 ? (lo | (k - 1)) - (lo & (k - 1)) : lo + j;
-                    if (hi < n && item_less(entries, ranking, s_item[hi], s_item[lo])) {
-                        const ull x = s_item[lo];
-                        s_item[lo] = s_item[hi];
-                        s_item[hi] = x;
-                    }
-                }
-                __syncthreads();
-            }
-        }
+        bitonic(n, [&](uint32_t a, uint32_t b) { return item_less(entries, ranking, s_item[a], s_item[b]); },
+                [&](uint32_t a, uint32_t b) { const ull x = s_item[a]; s_item[a] = s_item[b]; s_item[b] = x; });
     }
     __syncthreads();
 }
@@ -901,15 +990,15 @@ __device__ __forceinline__ void gather_tile(const atrex_entry_t* entries, const 
     if ((((uintptr_t)entries | (uintptr_t)out) & 15u) == 0) {
         const ulonglong2* src = reinterpret_cast<const ulonglong2*>(entries);
         ulonglong2* dst = reinterpret_cast<ulonglong2*>(out + first);
-        for (uint32_t i = threadIdx.x; i < rows * 3; i += 4 * blockDim.x) {
-            ulonglong2 v[4];
+        for (uint32_t i = threadIdx.x; i < rows * 3; i += GATHER_LOADS * blockDim.x) {
+            ulonglong2 v[GATHER_LOADS];
 #pragma unroll
-            for (uint32_t u = 0; u < 4; ++u) {
+            for (uint32_t u = 0; u < GATHER_LOADS; ++u) {
                 const uint32_t x = i + u * blockDim.x;
                 if (x < rows * 3) v[u] = __ldg(src + (size_t)(uint32_t)s_item[x / 3] * 3 + x % 3);
             }
 #pragma unroll
-            for (uint32_t u = 0; u < 4; ++u)
+            for (uint32_t u = 0; u < GATHER_LOADS; ++u)
             {
                 const uint32_t x = i + u * blockDim.x;
                 if (x >= rows * 3) continue;
@@ -938,18 +1027,34 @@ __global__ void __launch_bounds__(TILE_THREADS) bin_tile_kernel(const BinSort b,
     __shared__ uint32_t s_range[2];
     grid_dependency_wait();
     const bool overflow = b.ctl->overflow;
-    const uint32_t first = overflow ? 0u : b.tile_start[blockIdx.x], n = overflow ? 0u : b.tile_start[blockIdx.x + 1] - first;
+    // the last tile first: at both ends of a ranking the words lie uneven, which takes a tile twice as long
+    const uint32_t n_tiles = (item_count(b) + TILE_STEP - 1) / TILE_STEP;
+    const uint32_t tile = blockIdx.x >= n_tiles ? blockIdx.x : (blockIdx.x ? blockIdx.x - 1 : n_tiles - 1);
+    const uint32_t first = overflow ? 0u : b.tile_start[tile], n = overflow ? 0u : b.tile_start[tile + 1] - first;
     if (n == 0) {
         if (!b.ranking) finish_call(b.report, b.slot);
-        else if (!overflow && threadIdx.x < 2) b.tile_sum[2 * blockIdx.x + threadIdx.x] = 0;
+        else if (!overflow && threadIdx.x < 2) b.tile_sum[2 * tile + threadIdx.x] = 0;
         return;
     }
+    // the items are read once, all of a thread's at a time (a tile rarely has more than TILE_HELD per thread)
+    ull held[TILE_HELD];
+#pragma unroll
+    for (uint32_t u = 0; u < TILE_HELD; ++u) {
+        const uint32_t i = u * TILE_THREADS + threadIdx.x;
+        held[u] = i < n ? __ldcs(b.items + first + i) : 0ull;
+    }
+    auto each = [&](auto f) {
+#pragma unroll
+        for (uint32_t u = 0; u < TILE_HELD; ++u)
+            if (u * TILE_THREADS + threadIdx.x < n) f(held[u]);
+        for (uint32_t i = TILE_HELD * TILE_THREADS + threadIdx.x; i < n; i += TILE_THREADS) f(b.items[first + i]);
+    };
     uint32_t top = 0, ntop = 0;
-    for (uint32_t i = threadIdx.x; i < n; i += TILE_THREADS) {
-        const uint32_t w = (uint32_t)(b.items[first + i] >> 32);
+    each([&](ull item) {
+        const uint32_t w = (uint32_t)(item >> 32);
         top = max(top, w);
         ntop = max(ntop, ~w);
-    }
+    });
     if (threadIdx.x == 0) s_range[0] = s_range[1] = 0;
     __syncthreads();
     top = __reduce_max_sync(FULL, top);
@@ -959,7 +1064,7 @@ __global__ void __launch_bounds__(TILE_THREADS) bin_tile_kernel(const BinSort b,
         atomicMax(&s_range[1], top);
     }
     __syncthreads();
-    sort_tile(b.entries, b.ranking, n, ~s_range[0], s_range[1], [&](uint32_t i) { return b.items[first + i]; }, s_item, s_local);
+    sort_tile(b.entries, b.ranking, n, ~s_range[0], s_range[1], each, s_item, s_local);
     grid_dependents_launch();
     if (threadIdx.x < 2) s_sum[threadIdx.x] = 0;
     ulonglong2 sum = make_ulonglong2(0, 0);
@@ -983,7 +1088,7 @@ __global__ void __launch_bounds__(TILE_THREADS) bin_tile_kernel(const BinSort b,
     }
     if ((threadIdx.x & 31) == 0 && (sum.x | sum.y)) atomic_add128(&s_sum[0], &s_sum[1], sum.x, sum.y);
     __syncthreads();
-    if (threadIdx.x < 2) b.tile_sum[2 * blockIdx.x + threadIdx.x] = s_sum[threadIdx.x];
+    if (threadIdx.x < 2) b.tile_sum[2 * tile + threadIdx.x] = s_sum[threadIdx.x];
 }
 
 // Key order of up to COUNT_SORT_MAX entries in one kernel: an entry's place is the number of keys before its own.
@@ -1294,6 +1399,7 @@ BinSort carve_bins(void* base, const atrex_entry_t* entries, uint64_t n, bool ra
     p += sizeof(BinCtl);
     b.by_tile = tiles <= CURSORS_MAX;
     b.n_cursors = b.by_tile ? (uint32_t)tiles : 1u << b.bits;
+    b.turns = b.n_cursors >= 2048 ? 2 : 1;
     b.bins = (uint32_t*)p;       p += 4ull << b.bits;
     b.cursors = (uint32_t*)p;    p += 4ull * ((b.n_cursors + 3) & ~3u);
     b.tile_sum = (ull*)p;        p += tiles * 16;
