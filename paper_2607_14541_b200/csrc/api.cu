@@ -732,6 +732,7 @@ static int select_phase(atrex_agg_t* h, uint32_t q, uint32_t k, cudaStream_t s) 
     CU(h, cudaMemsetAsync(h->ctl->sel_count_all, 0, sizeof(h->ctl->sel_count_all), s));
     CU(h, cudaMemsetAsync(h->sel + (size_t)q * SEL_CAP * 4, 0, (size_t)n_pow2 * 32, s));   // (the sort wants zeros behind the candidates)
     CU(h, launch_topk_collect_all(all, h->scan_grid(h->L.n_slots, 256 * 4), s));
+    CU(h, cudaMemsetAsync(h->ctl->sel_count_all, 0, sizeof(h->ctl->sel_count_all), s));
     CU(h, launch_topk_sort(h->sel + (size_t)q * SEL_CAP * 4, n_pow2, s));
     h->launches += 2;
     cache.sel_gen[q] = h->fin_gen;
@@ -767,7 +768,7 @@ int atrex_agg_topk(atrex_agg_t* h, uint32_t phase, uint32_t k, atrex_entry_t* h_
             const ull want = p.fin.seq;
             for (uint32_t q = 0; q < n_phases; ++q) answers[q] = ~(want << 32);
             CU(h, launch_topk_pick(p, h->n_sms, s));
-            h->launches += 3;
+            h->launches += 2;
             const volatile ull* a = answers;
             CU(h, wait_for_kernel([=] {
                 for (uint32_t q = 0; q < n_phases; ++q)

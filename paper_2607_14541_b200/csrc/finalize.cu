@@ -319,61 +319,81 @@ __global__ void __launch_bounds__(256) work_insert_kernel(const atrex_work_t* ro
 
 // ---- top-k, the usual way -----------------------------------------------------------------
 // All phases at once, without a word from the host in between: a first digit on a logarithmic scale (bit
-// length and the five bits below the leading one: 3 % steps) is counted per phase; one CTA per phase finds
-// the digit of its k-th key; the keys at or above it are collected; one CTA per phase ranks them exactly and
+// length and the five bits below the leading one: 3 % steps) is counted per phase; the digit of each
+// phase's k-th key is found; the keys at or above it are collected; one CTA per phase ranks them exactly and
 // writes the best k to pinned host memory.  Weights that span orders of magnitude leave a few dozen
 // candidates beside the winners.  (Digits on a linear scale below the phase total's highest bit put every
 // key of a flat trace into the lowest one: 26 000 candidates in one CTA's global-memory sort took 4 ms.)
-constexpr int PICK_THREADS = 1024;
+//
+// Every collecting CTA finds the digits for itself, a quarter of a phase's bins to a warp at a time: a
+// microsecond, where a kernel of its own before this one cost four.
+constexpr uint32_t QUARTER = TOPK_BINS / 4;
 
-// the digit of each phase's k-th key (one CTA per phase)
-__global__ void __launch_bounds__(PICK_THREADS) topk_plan_kernel(const __grid_constant__ PickParams p) {
-    __shared__ uint32_t s_warp[32];
-    grid_dependency_wait();
-    const uint32_t q = blockIdx.x, t = threadIdx.x, lane = t & 31u, w = t >> 5;
-    // thread t holds the four bins below TOPK_BINS - 4 t, highest first
-    const uint4 v = reinterpret_cast<const uint4*>(p.hist + (size_t)q * TOPK_BINS)[TOPK_BINS / 4 - 1 - t];
-    const uint32_t c[4] = {v.w, v.z, v.y, v.x};
-    const uint32_t own = c[0] + c[1] + c[2] + c[3];
-    uint32_t incl = own;
+// Keys in one quarter of phase q's bins, quarter 0 the highest (one warp); v[u] = lane's four bins of step u, the
+// highest bins in step 0 and lane 0.
+__device__ __forceinline__ uint32_t load_quarter(const PickParams& p, uint32_t q, uint32_t quarter, uint4 (&v)[8]) {
+    const uint4* hist = reinterpret_cast<const uint4*>(p.hist + (size_t)q * TOPK_BINS) + (TOPK_BINS - quarter * QUARTER) / 4 - 1 - (threadIdx.x & 31u);
+    uint32_t sum = 0;
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, incl, d);
-        if (lane >= (uint32_t)d) incl += o;
-    }
-    if (lane == 31) s_warp[w] = incl;
-    __syncthreads();
-    if (w == 0) {
-        uint32_t s = s_warp[lane];
+    for (int u = 0; u < 8; ++u) v[u] = *(hist - 32 * u);
 #pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, s, d);
-            if (lane >= (uint32_t)d) s += o;
+    for (int u = 0; u < 8; ++u) sum += v[u].x + v[u].y + v[u].z + v[u].w;
+    return __reduce_add_sync(0xFFFFFFFFu, sum);
+}
+
+// the digit of phase q's k-th key, which lies in this quarter, `above` keys in higher ones (one warp)
+__device__ __forceinline__ uint32_t digit_in_quarter(const PickParams& p, uint32_t q, uint32_t quarter, uint32_t above) {
+    const uint32_t lane = threadIdx.x & 31u;
+    uint4 v[8];
+    load_quarter(p, q, quarter, v);
+    uint32_t found = PICK_NONE;
+#pragma unroll
+    for (uint32_t u = 0; u < 8; ++u) {
+        const uint32_t own = v[u].x + v[u].y + v[u].z + v[u].w, all = __reduce_add_sync(0xFFFFFFFFu, own);
+        if (above < p.k && above + all >= p.k) {
+            uint32_t incl = own;
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+                if (lane >= (uint32_t)d) incl += o;
+            }
+            const uint32_t src = __ffs(__ballot_sync(0xFFFFFFFFu, above + incl >= p.k)) - 1;
+            uint32_t at = above + incl - own + v[u].w, digit = TOPK_BINS - 1 - quarter * QUARTER - 4 * (32 * u + lane);
+            if (at < p.k) { at += v[u].z; --digit; }
+            if (at < p.k) { at += v[u].y; --digit; }
+            if (at < p.k) { at += v[u].x; --digit; }
+            found = __shfl_sync(0xFFFFFFFFu, at <= TOPK_PICK_MAX ? digit : PICK_NONE, src);
         }
-        s_warp[lane] = s;
+        above += all;
     }
-    __syncthreads();
-    const uint32_t all = s_warp[31];
-    uint32_t above = incl - own + (w ? s_warp[w - 1] : 0u);
-    if (t == 0) {
-        p.fin.ctl->sel_count_all[q] = 0;
-        if (all <= p.k) p.fin.ctl->pick_bin[q] = all <= TOPK_PICK_MAX ? 0u : PICK_NONE;
-    }
-    if (all > p.k && above < p.k) {
-#pragma unroll
-        for (uint32_t u = 0; u < 4; ++u) {
-            if (above < p.k && above + c[u] >= p.k)
-                p.fin.ctl->pick_bin[q] = above + c[u] <= TOPK_PICK_MAX ? TOPK_BINS - 1 - (4 * t + u) : PICK_NONE;
-            above += c[u];
-        }
-    }
+    return found;
 }
 
 // the keys at or above that digit
 __global__ void __launch_bounds__(FIN_THREADS) topk_collect_kernel(const __grid_constant__ PickParams p) {
-    __shared__ uint32_t s_bin[ATREX_MAX_PHASES];
+    __shared__ uint32_t s_bin[ATREX_MAX_PHASES], s_sum[4 * ATREX_MAX_PHASES];
+    static_assert(FIN_THREADS / 32 >= ATREX_MAX_PHASES, "a warp per phase");
     grid_dependency_wait();
-    if (threadIdx.x < ATREX_MAX_PHASES) s_bin[threadIdx.x] = threadIdx.x < p.n_phases ? p.fin.ctl->pick_bin[threadIdx.x] : PICK_NONE;
+    const uint32_t warp = threadIdx.x >> 5;
+    for (uint32_t i = warp; i < 4 * p.n_phases; i += FIN_THREADS / 32) {
+        uint4 v[8];
+        const uint32_t sum = load_quarter(p, i / 4, i % 4, v);
+        if ((threadIdx.x & 31u) == 0) s_sum[i] = sum;
+    }
+    __syncthreads();
+    if (warp < ATREX_MAX_PHASES) {
+        uint32_t digit = PICK_NONE;
+        if (warp < p.n_phases) {
+            uint32_t above = 0, quarter = 0;
+            while (quarter < 4 && above + s_sum[4 * warp + quarter] < p.k) above += s_sum[4 * warp + quarter++];
+            if (quarter < 4) digit = digit_in_quarter(p, warp, quarter, above);
+            else digit = above <= TOPK_PICK_MAX ? 0u : PICK_NONE;              // fewer than k keys: all of them
+        }
+        if ((threadIdx.x & 31u) == 0) {
+            s_bin[warp] = digit;
+            if (blockIdx.x == 0) p.fin.ctl->pick_bin[warp] = digit;
+        }
+    }
     __syncthreads();
     const TableRef& tab = p.fin.t;
     constexpr int ILP = 4;
@@ -465,6 +485,7 @@ __global__ void __launch_bounds__(512) topk_rank_kernel(const __grid_constant__ 
     }
     __syncthreads();
     if (threadIdx.x == 0) {
+        p.fin.ctl->sel_count_all[q] = 0;   // (for the next request)
         __threadfence_system();
         *(volatile ull*)&p.host_n[q] = p.fin.seq << 32 | min(n, p.k);   // the host waits for this word
     }
@@ -643,8 +664,7 @@ cudaError_t launch_work_insert(const atrex_work_t* rows, ull n, const WorkRef& w
 
 cudaError_t launch_topk_pick(const PickParams& p, int n_sms, cudaStream_t stream) {
     static const uint32_t per_sm = resident_ctas(topk_collect_kernel, FIN_THREADS, 0);
-    cudaError_t e = launch_chained(topk_plan_kernel, p.n_phases, PICK_THREADS, 0, stream, p);
-    if (e == cudaSuccess) e = launch_chained(topk_collect_kernel, grid_for_work(p.fin.n_slots, FIN_THREADS * 4, n_sms, per_sm), FIN_THREADS, 0, stream, p);
+    cudaError_t e = launch_chained(topk_collect_kernel, grid_for_work(p.fin.n_slots, FIN_THREADS * 4, n_sms, per_sm), FIN_THREADS, 0, stream, p);
     if (e == cudaSuccess) e = launch_chained(topk_rank_kernel, p.n_phases, 512, PICK_SMEM, stream, p);
     return e;
 }
