@@ -164,7 +164,8 @@ __global__ void __launch_bounds__(TOTAL_WARPS * 32) eq3_app_totals_kernel(const 
                                                                           uint32_t* present) {
     __shared__ ull s_lo[TOTAL_WARPS][32], s_hi[TOTAL_WARPS][32];
     grid_dependency_wait();
-    const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5, app = blockIdx.x * 32 + lane, phase = blockIdx.y;
+    const uint32_t per_phase = (n_apps + 31) / 32, phase = blockIdx.x / per_phase;
+    const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5, app = blockIdx.x % per_phase * 32 + lane;
     ull t_lo = 0, t_hi = 0;
     for (uint32_t i0 = w; i0 < n_ops; i0 += 4 * TOTAL_WARPS) {
         ull x[4], y[4];
@@ -424,8 +425,9 @@ int atrex_eq3_finalize(atrex_eq3_t* h, const uint8_t* h_retained, double* h_w, d
     const volatile ull* done = (const volatile ull*)h->h_out + 2 * (size_t)n_ops + 1;
     const ull seq = ++h->n_finalized;
     *(volatile ull*)done = 0;    // (a block from the pool holds whatever its last owner left)
-    eq3_app_totals_kernel<<<dim3((h->n_apps + 31) / 32, h->n_phases), TOTAL_WARPS * 32, 0, s>>>(h->d_lo, hi, h->n_apps, n_ops, h->d_den, h->d_present);
-    if (cudaGetLastError() != cudaSuccess) return ATREX_ERR_CUDA;
+    if (launch_chained(eq3_app_totals_kernel, (h->n_apps + 31) / 32 * h->n_phases, TOTAL_WARPS * 32, 0, s, h->d_lo, hi, h->n_apps, n_ops, h->d_den,
+                       h->d_present) != cudaSuccess)
+        return ATREX_ERR_CUDA;
     const bool any_weight = h->c_total != 0.0;
     if (launch_chained(eq3_wtilde_kernel, n_ops, WT_THREADS, 0, s, h->d_lo, hi, h->d_den, h->d_pa, h->d_present, h->n_apps, n_ops, h->n_phases,
                        any_weight, h->d_wt, retained, h->d_ctl, h->h_out, seq) != cudaSuccess)

@@ -546,6 +546,14 @@ __device__ __forceinline__ T block_reduce(T v, T (*op)(T, T), T* s_part) {   // 
 }
 __device__ __forceinline__ ull max_ull(ull a, ull b) { return a > b ? a : b; }
 
+// 0. the control block and the bins behind it cleared (a kernel in the chain: a memset breaks it, 3 us each side)
+__global__ void __launch_bounds__(BIN_THREADS) bin_clear_kernel(uint4* at, uint32_t n) {
+    grid_dependency_wait();
+    const uint32_t i = blockIdx.x * BIN_THREADS + threadIdx.x;
+    if (i < n) at[i] = make_uint4(0, 0, 0, 0);
+    grid_dependents_launch();
+}
+
 // 1a. (key order) the keys side by side, and the largest value of each field
 __global__ void __launch_bounds__(BIN_THREADS) bin_keys_kernel(const BinSort b) {
     __shared__ ull s_part[32];
@@ -1413,6 +1421,11 @@ BinSort carve_bins(void* base, const atrex_entry_t* entries, uint64_t n, bool ra
 // (what it needs beyond the pairs is less than the radix sort's digit counts, as long as there are a few tiles)
 static_assert(sizeof(BinCtl) + (4u << 5) + 4u * 4u + 16u * 3u + 4u * 4u + 256u <= sizeof(ReleaseCtl) + 1024u + 1024u + 256u, "smallest case");
 
+cudaError_t launch_clear(const BinSort& b, cudaStream_t s) {
+    const uint32_t n = (uint32_t)((sizeof(BinCtl) + (4ull << b.bits)) / 16);
+    return launch_chained(bin_clear_kernel, (n + BIN_THREADS - 1) / BIN_THREADS, BIN_THREADS, 0, s, (uint4*)b.ctl, n);
+}
+
 // Steps 2 to 5, behind the kernel that made the words.
 cudaError_t launch_bins(const BinSort& b, atrex_entry_t* out, uint64_t out_cap, int n_sms, cudaStream_t s) {
     const uint32_t bytes = 4u << b.bits, tiles = (b.n + TILE_STEP - 1) / TILE_STEP;
@@ -1469,7 +1482,7 @@ extern "C" int atrex_entries_sort_by_key(const atrex_entry_t* d_entries, uint64_
         ReportSlot report;
         if (!report.get()) return ATREX_ERR_NOMEM;
         const BinSort b = carve_bins(d_scratch, d_entries, n, false, report);
-        if (cudaMemsetAsync(b.ctl, 0, sizeof(BinCtl) + (4ull << b.bits), s) != cudaSuccess) return ATREX_ERR_CUDA;
+        if (launch_clear(b, s) != cudaSuccess) return ATREX_ERR_CUDA;
         const uint32_t want = (m + 4 * BIN_THREADS - 1) / (4 * BIN_THREADS), most = 4u * (uint32_t)n_sms;
         if (launch_chained(bin_keys_kernel, want < most ? want : most, BIN_THREADS, 0, s, b) != cudaSuccess ||
             launch_bins(b, d_out, n, n_sms, s) != cudaSuccess || report.wait(s) != cudaSuccess)
@@ -1515,7 +1528,7 @@ extern "C" int atrex_entries_rank(const atrex_entry_t* d_entries, uint64_t n, ui
         ReportSlot slot;
         if (!slot.get()) return ATREX_ERR_NOMEM;
         const BinSort b = carve_bins(d_scratch, d_entries, n, true, slot);
-        if (cudaMemsetAsync(b.ctl, 0, sizeof(BinCtl) + (4ull << b.bits), s) != cudaSuccess) return ATREX_ERR_CUDA;
+        if (launch_clear(b, s) != cudaSuccess) return ATREX_ERR_CUDA;
         const uint32_t want = ((uint32_t)n + 4 * BIN_THREADS - 1) / (4 * BIN_THREADS), most = 4u * (uint32_t)n_sms;
         const uint32_t tiles = ((uint32_t)n + TILE_STEP - 1) / TILE_STEP, cap = (uint32_t)(out_cap < n ? out_cap : n);
         if (launch_chained(bin_phase_kernel, want < most ? want : most, BIN_THREADS, 0, s, b, phase) != cudaSuccess ||
