@@ -441,6 +441,12 @@ __device__ __forceinline__ uint32_t middle_slots_of_pair(uint32_t* col, uint32_t
     return m;
 }
 
+template <bool PAIRS, int N>
+__device__ __forceinline__ uint32_t middle_of(uint32_t* col, uint32_t& low, uint32_t& up, bool& search) {
+    if constexpr (PAIRS) return middle_slots_of_pair<N>(col, low, up, search);
+    else return middle_slots<N>(col, low, up, search);
+}
+
 constexpr uint32_t WARP_ILP = 4;           // units per lane in flight
 __host__ __device__ __forceinline__ uint32_t padded_units(uint32_t n) { return (n + 32u * WARP_ILP - 1u) / (32u * WARP_ILP) * (32u * WARP_ILP); }
 
@@ -584,24 +590,15 @@ __global__ void __launch_bounds__(WARP_KERNEL_THREADS, WARP_KERNEL_CTAS)
             uint32_t* col = keys + at + lane;
             uint32_t low = 0, up = 0, m = 0;
             bool search = false;
-            auto middle = [&](auto n) {
-                if constexpr (PAIRS) {
-                    m = middle_slots_of_pair<n.value>(col, low, up, search);
-                } else {
-                    m = middle_slots<n.value>(col, low, up, search);
-                    low *= 32;
-                    up *= 32;
-                }
-            };
-            if (length == 8) middle(std::integral_constant<int, 8>());
-            else if (length == 16) middle(std::integral_constant<int, 16>());
-            else if (length == 20) middle(std::integral_constant<int, 20>());
-            else if (length == 24) middle(std::integral_constant<int, 24>());
-            else if (length == 28) middle(std::integral_constant<int, 28>());
-            else if (length == 32) middle(std::integral_constant<int, 32>());
+            if (length == 8) m = middle_of<PAIRS, 8>(col, low, up, search);
+            else if (length == 16) m = middle_of<PAIRS, 16>(col, low, up, search);
+            else if (length == 20) m = middle_of<PAIRS, 20>(col, low, up, search);
+            else if (length == 24) m = middle_of<PAIRS, 24>(col, low, up, search);
+            else if (length == 28) m = middle_of<PAIRS, 28>(col, low, up, search);
+            else if (length == 32) m = middle_of<PAIRS, 32>(col, low, up, search);
             double s = 0.0;
             if (m != 0 && !search) {
-                const uint32_t ju = unit_at[first_slot + up], jl = unit_at[first_slot + low];
+                const uint32_t ju = unit_at[first_slot + (PAIRS ? up : 32 * up)], jl = unit_at[first_slot + (PAIRS ? low : 32 * low)];
                 s = __ddiv_rn(__ldg(roofline_s + ju), __ldg(t + ju));
                 if (!(m & 1u)) s = __dmul_rn(__dadd_rn(__ddiv_rn(__ldg(roofline_s + jl), __ldg(t + jl)), s), 0.5);
             }
@@ -610,7 +607,7 @@ __global__ void __launch_bounds__(WARP_KERNEL_THREADS, WARP_KERNEL_CTAS)
                 const uint32_t first = __shfl_sync(FULL, is_large ? g.x : first_slot, src), packed = __shfl_sync(FULL, g.y, src);
                 const uint32_t n = packed & 0x7FFFFFFFu, stride = packed >> 31 ? 1u : 32u;
                 auto key_at = [=](uint32_t a) {
-                    const uint32_t j = unit_at[first + (stride == 1 ? a : a % LANES + 32 * (a / LANES))];
+                    const uint32_t j = unit_at[first + (PAIRS && stride != 1 ? a % LANES + 32 * (a / LANES) : a * stride)];
                     return exact_key(__ldg(roofline_s + j), __ldg(t + j), __ldg(ok + j) != 0);
                 };
                 uint32_t usable = 0;
