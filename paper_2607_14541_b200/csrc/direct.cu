@@ -86,7 +86,8 @@ __global__ void __launch_bounds__(RECORDS_THREADS) direct_records_kernel(DirectP
 }
 
 // Four slots of the shared table to the key table at once: their key look-ups, then their returning adds,
-// are in flight together.
+// are in flight together.  (The counts added without waiting for the low words' answers, the rare carries by adds of
+// their own: 2^20 records over 4 096 keys 5 us slower.)
 __device__ __forceinline__ void flush_slots(const TableRef& t, const ull (&key)[4], const uint32_t (&h)[4], const ull (&v)[4],
                                             const uint32_t (&count)[4]) {
     ull idx[4], found[4], old[4];
