@@ -1,9 +1,7 @@
 // Kernel parameter blocks and host-side launchers (internal to the library).
 #pragma once
-#include <atomic>
-#include <chrono>
-
 #include "atrex_dev.cuh"
+#include "host_wait.h"
 
 namespace atrex {
 
@@ -207,21 +205,6 @@ inline cudaError_t launch_chained(void (*kernel)(P...), uint32_t grid, uint32_t 
 // a pool of the process, so that creating a handle does not pay for pinning; at most eight wait there.
 cudaError_t pinned_alloc(void** out, size_t bytes);
 void pinned_free(void* block, size_t bytes);
-
-// Waits until `done()` sees what a kernel on `s` wrote to pinned memory as its last act, which the host notices
-// several microseconds before the stream counts as idle; after a millisecond, or if the kernel cannot get there,
-// by the stream itself.
-template <typename Done>
-inline cudaError_t wait_for_kernel(Done done, cudaStream_t s) {
-    const auto limit = std::chrono::steady_clock::now() + std::chrono::milliseconds(1);
-    for (uint32_t i = 1;; ++i) {
-        if (done()) {
-            std::atomic_thread_fence(std::memory_order_acquire);
-            return cudaSuccess;
-        }
-        if ((i & 63u) == 0 && std::chrono::steady_clock::now() > limit) return cudaStreamSynchronize(s);
-    }
-}
 
 // CTAs of a grid-stride kernel: as many as the SMs hold at once (a second, partly filled wave would cost as
 // much as a full one), fewer when there is less work.  `per_sm` comes from resident_ctas, asked once.

@@ -13,7 +13,6 @@
 //
 // The running sum is an exact 128-bit prefix sum in rank order (sums of tiles or blocks, a scan of those, a
 // local scan), rounded once per row when the share is formed.
-#include <condition_variable>
 #include <cstring>
 #include <mutex>
 
@@ -433,7 +432,6 @@ constexpr uint32_t TILE_CLASH_MAX = 24;     // larger local bins are crowded: so
 constexpr uint32_t TILE_CROWDED = 32;       // more of them, or larger ones, send the tile to the comparison network
 constexpr size_t TILE_SMEM = (size_t)TILE_CAP * 8 + TILE_LOCAL_BINS * 4;    // (what it leaves of two CTAs is L1 for the gather)
 constexpr uint32_t COUNT_SORT_MAX = 8192;   // up to here one kernel ranks every key by counting
-constexpr int REPORT_SLOTS = 32;
 
 struct BinCtl {                  // at the start of the scratch, cleared by every call (with the bins behind it)
     ull counter;                 // items (entries of the phase)
@@ -446,11 +444,6 @@ struct BinCtl {                  // at the start of the scratch, cleared by ever
 };
 static_assert(sizeof(BinCtl) == 128, "half of the control block");
 
-struct BinReport {               // in pinned host memory, written by the kernels
-    ull overflow, counter, total_lo, total_hi, n_keep, covered_lo, covered_hi, too_large;
-    ull done;                    // the call's last kernel is through
-    ull pad[7];
-};
 // CTAs of a call's last kernel that are through, by the call's report slot; back at 0 after the last one
 __device__ uint32_t g_finished[REPORT_SLOTS];
 
@@ -1350,46 +1343,6 @@ int sort_by_word(const Scratch& sc, int cur, uint32_t m, ull differing_bits, cud
     return cur;
 }
 
-// Reports from the device: a few pinned slots for the whole process, handed out per call (a call that finds
-// none free waits for one; calls are milliseconds at most).
-class ReportSlot {
-public:
-    ReportSlot() {
-        std::unique_lock<std::mutex> hold(lock());
-        if (pool() == nullptr && cudaHostAlloc((void**)&pool(), SLOTS * sizeof(BinReport), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
-            cudaGetLastError();
-            return;
-        }
-        freed().wait(hold, [] { return used() != FULL; });
-        slot_ = __builtin_ctz(~used());
-        used() |= 1u << slot_;
-        memset((void*)get(), 0, sizeof(BinReport));
-    }
-    ~ReportSlot() {
-        if (slot_ < 0) return;
-        std::lock_guard<std::mutex> hold(lock());
-        used() &= ~(1u << slot_);
-        freed().notify_one();
-    }
-    ReportSlot(const ReportSlot&) = delete;
-    ReportSlot& operator=(const ReportSlot&) = delete;
-    BinReport* get() const { return slot_ < 0 ? nullptr : pool() + slot_; }
-    uint32_t number() const { return (uint32_t)slot_; }
-    // waits for the call's last kernel (finish_call)
-    cudaError_t wait(cudaStream_t s) const {
-        const volatile ull* done = &get()->done;
-        return wait_for_kernel([=] { return *done != 0; }, s);
-    }
-
-private:
-    static constexpr int SLOTS = REPORT_SLOTS;
-    static std::mutex& lock() { static std::mutex m; return m; }
-    static std::condition_variable& freed() { static std::condition_variable c; return c; }
-    static BinReport*& pool() { static BinReport* p = nullptr; return p; }
-    static uint32_t& used() { static uint32_t u = 0; return u; }
-    int slot_ = -1;
-};
-
 // The scratch as the binned sort uses it.
 BinSort carve_bins(void* base, const atrex_entry_t* entries, uint64_t n, bool ranking, const ReportSlot& slot) {
     unsigned char* p = (unsigned char*)base;
@@ -1470,22 +1423,22 @@ extern "C" int atrex_entries_sort_by_key(const atrex_entry_t* d_entries, uint64_
     int n_sms = 0;
     if (prepare_sort_kernels(&n_sms) != ATREX_OK) return ATREX_ERR_CUDA;
     if (n <= COUNT_SORT_MAX) {   // (above, counting takes longer than the binned sort's launches)
-        ReportSlot report;
+        ReportSlot report(s);
         if (!report.get()) return ATREX_ERR_NOMEM;
         const uint32_t per_cta = n <= 4096 ? 32 : 64, grid = (m + per_cta - 1) / per_cta;
         auto* kernel = n <= 4096 ? count_sort_kernel<1> : count_sort_kernel<2>;
         if (launch_chained(kernel, grid, COUNT_THREADS, (size_t)(m + 1) / 2 * 16, s, d_entries, m, d_out, report.get(), report.number()) != cudaSuccess)
             return ATREX_ERR_CUDA;
-        return report.wait(s) == cudaSuccess ? ATREX_OK : ATREX_ERR_CUDA;
+        return report.wait() == cudaSuccess ? ATREX_OK : ATREX_ERR_CUDA;
     }
     {
-        ReportSlot report;
+        ReportSlot report(s);
         if (!report.get()) return ATREX_ERR_NOMEM;
         const BinSort b = carve_bins(d_scratch, d_entries, n, false, report);
         if (launch_clear(b, s) != cudaSuccess) return ATREX_ERR_CUDA;
         const uint32_t want = (m + 4 * BIN_THREADS - 1) / (4 * BIN_THREADS), most = 4u * (uint32_t)n_sms;
         if (launch_chained(bin_keys_kernel, want < most ? want : most, BIN_THREADS, 0, s, b) != cudaSuccess ||
-            launch_bins(b, d_out, n, n_sms, s) != cudaSuccess || report.wait(s) != cudaSuccess)
+            launch_bins(b, d_out, n, n_sms, s) != cudaSuccess || report.wait() != cudaSuccess)
             return ATREX_ERR_CUDA;
         if (!((volatile BinReport*)report.get())->overflow) return ATREX_OK;
     }
@@ -1525,7 +1478,7 @@ extern "C" int atrex_entries_rank(const atrex_entry_t* d_entries, uint64_t n, ui
     int n_sms = 0;
     if (prepare_sort_kernels(&n_sms) != ATREX_OK) return ATREX_ERR_CUDA;
     {
-        ReportSlot slot;
+        ReportSlot slot(s);
         if (!slot.get()) return ATREX_ERR_NOMEM;
         const BinSort b = carve_bins(d_scratch, d_entries, n, true, slot);
         if (launch_clear(b, s) != cudaSuccess) return ATREX_ERR_CUDA;
@@ -1535,7 +1488,7 @@ extern "C" int atrex_entries_rank(const atrex_entry_t* d_entries, uint64_t n, ui
             launch_bins(b, d_ranked, cap, n_sms, s) != cudaSuccess ||
             launch_chained(bin_tile_scan_kernel, 1, SCAN_BLOCK, 0, s, b, coverage_ppm) != cudaSuccess ||
             launch_chained(bin_share_kernel, tiles, SCAN_BLOCK, 0, s, b, d_ranked, d_cum_share, cap) != cudaSuccess ||
-            slot.wait(s) != cudaSuccess)
+            slot.wait() != cudaSuccess)
             return ATREX_ERR_CUDA;
         const volatile BinReport* r = slot.get();
         if (r->too_large || !r->overflow) {
