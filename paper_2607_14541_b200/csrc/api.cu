@@ -473,13 +473,13 @@ static int ingest_launch(atrex_agg* h, const atrex_record_t* recs, uint64_t n, c
     if (h->L.hot_slots && !h->hot_ready) {
         HotBuildParams b;
         b.recs = (const uint4*)recs;
-        // A record of the sample costs the build 70 ps (2^20: 80 us), a poorer choice the scatter pass up to 4 % where
+        // A record of the sample costs the build 85 ps (2^20: 95 us), a poorer choice the scatter pass up to 4 % where
         // many keys compete: one of 256 records, or one for 16 provisioned keys, whichever is more, from 2^18 on
         // (2^26 records over 2^19 keys 757 -> 729 us with 2^18; 2^30 over 2^24 keys 11.8 ms with 2^20, 12.0 with 2^18)
         ull sample = n / 256 > h->cfg.max_keys / 16 ? n / 256 : h->cfg.max_keys / 16;
         sample = pow2_at_least(sample < HOT_SAMPLE / 4 ? HOT_SAMPLE / 4 : (sample < HOT_SAMPLE ? sample : HOT_SAMPLE));
-        b.n_sample = (uint32_t)(n < sample ? n : sample) & ~(HOT_SAMPLE_RUN - 1);   // (n is at least DIRECT_RECORDS_MAX here)
-        b.stride = n / (b.n_sample / HOT_SAMPLE_RUN);
+        b.n_sample = (uint32_t)(n < sample ? n : sample);
+        b.stride = n / b.n_sample;
         b.n_apps = h->cfg.n_apps;
         b.n_phases = h->cfg.n_phases;
         b.hot_keys = h->hot_keys;

@@ -499,8 +499,12 @@ __global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(PartitionP
 }
 
 // --------------------------------------------------------------------------------------
-// Hot-directory construction, small kernels over a sample of the records (runs of four neighbouring records, evenly
-// spread: a DRAM burst of 64 bytes costs the same as one record of it):
+// Hot-directory construction, small kernels over a sample of the records: one out of every `stride`, at a place in
+// its stretch that a hash chooses.  Traces have neighbours that are alike (a kernel launched in a loop) and patterns
+// that repeat (services taking turns), so records sampled side by side, or at a fixed distance, would show a key far
+// more or less often than it occurs.  (Sampled four neighbours at a time, a trace whose keys come four times in a
+// row lost 40 % of the keys that hold an eighth of it to keys that come once; single records lose 1 %, and cost 5 us
+// more for 2^18 samples, 15 for 2^20.)
 //   1. count   every sampled key bumps one of 2^20 counters chosen by its hash; the keys are kept side by side;
 //   2. admit   sampled keys whose counter reached ADMIT_MIN are inserted, with exact counts,
 //              into a candidate table (colliding cold keys may slip in; harmless);
@@ -508,13 +512,18 @@ __global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(PartitionP
 //   4. gather  the candidates above it side by side, and how much weight each of four bucket hashes would lose;
 //   5. list    the candidates of each 4-slot bucket under the best of them;
 //   6. pick    each bucket takes its four most frequent ones.
-// Which keys end up in the directory only affects speed, never results.  Bound by latency and launches: 75 us for
+// Which keys end up in the directory only affects speed, never results.  Bound by latency and launches: 90 us for
 // 2^20 samples; 187 us when single records were read (twice) and one CTA did steps 3 to 6.
 constexpr uint32_t SKETCH_BITS = 20;   // as many counters as samples, so that cold keys stay below ADMIT_MIN
 constexpr uint32_t ADMIT_MIN = 3;
 constexpr uint32_t CAND_PROBES = 16;
 constexpr uint32_t SAMPLE_ILP = 4;     // samples in flight per thread
-constexpr uint32_t RUN = HOT_SAMPLE_RUN;
+
+__device__ __forceinline__ ull sample_at(const HotBuildParams& p, uint32_t j) {
+    uint32_t h = j * HASH_A;
+    h = (h ^ (h >> 15)) * HASH_C;
+    return (ull)j * p.stride + __umulhi(h, (uint32_t)p.stride);
+}
 
 // Counts for lanes of a warp that target the same counter are combined first, and those of a CTA in a small
 // shared-memory cache, so that a trace dominated by one key does not queue at one address.
@@ -559,7 +568,7 @@ __global__ void __launch_bounds__(256) hot_count_kernel(HotBuildParams p) {
 #pragma unroll
         for (uint32_t u = 0; u < SAMPLE_ILP; ++u) {
             const uint32_t j = (r * SAMPLE_ILP + u) * stride + blockIdx.x * blockDim.x + threadIdx.x;
-            v[u] = j < p.n_sample ? p.recs[(ull)(j / RUN) * p.stride + j % RUN] : make_uint4(0xFFFFFFFFu, 0, 0, 0);
+            v[u] = j < p.n_sample ? p.recs[sample_at(p, j)] : make_uint4(0xFFFFFFFFu, 0, 0, 0);
         }
 #pragma unroll
         for (uint32_t u = 0; u < SAMPLE_ILP; ++u) {

@@ -87,7 +87,6 @@ struct PartitionParams {
 };
 
 // Scratch of the directory build's last steps (cleared by every build up to `key`).
-constexpr uint32_t HOT_SAMPLE_RUN = 4;       // neighbouring records sampled together
 constexpr uint32_t HOT_SELECT_MAX = 14336;   // candidates kept (directory <= 11.6K slots, x1.25)
 constexpr uint32_t HOT_BUCKETS_MAX = 3072;   // directory buckets (<= 11.6K / 4)
 struct HotBuildScratch {
@@ -104,8 +103,8 @@ struct HotBuildScratch {
 
 struct HotBuildParams {
     const uint4* recs;
-    ull stride;                // records from one run to the next
-    uint32_t n_sample;         // whole runs
+    ull stride;                // records per sampled one (below 2^32)
+    uint32_t n_sample;         // n_sample * stride <= records of the call
     uint32_t n_apps, n_phases;
     ull* hot_keys;
     uint32_t hot_slots;
