@@ -28,7 +28,8 @@ constexpr size_t HOT_SELECT_OFF = SKETCH_BYTES + ((size_t)12 << CAND_BITS);
 constexpr size_t HOT_COUNT_BYTES = HOT_SELECT_OFF + offsetof(HotBuildScratch, key);
 constexpr size_t HOT_SAMPLE_OFF = HOT_SELECT_OFF + (sizeof(HotBuildScratch) + 255) / 256 * 256;
 constexpr size_t HOT_SCRATCH_BYTES = HOT_SAMPLE_OFF + (size_t)HOT_SAMPLE * 8;
-constexpr uint32_t SEL_CAP = ATREX_MAX_TOPK + TOPK_CAND_CAP;
+constexpr uint32_t SEL_CAP = ATREX_MAX_TOPK;           // items of a phase that the long way to the top-k sorts
+static_assert((SEL_CAP & (SEL_CAP - 1)) == 0 && SEL_CAP >= TOPK_PICK_MAX, "a power of two");
 
 size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -48,7 +49,7 @@ ull pow2_at_least(ull x) {
 }
 
 struct Layout {
-    size_t off_ctl, off_keys, off_vals, off_work, off_appw, off_hot, off_staging[2], off_sel, off_pick, off_topk_out, off_hist_all,
+    size_t off_ctl, off_keys, off_vals, off_work, off_appw, off_hot, off_staging[2], off_sel, off_pick, off_topk_out, off_hist_all, off_hist_next,
         off_spill_cnt, off_spill, off_hot_scratch, off_queue, off_hot_img, total;
     ull n_slots, work_slots;
     uint32_t lp, C;              // partitions = 1 << lp, slots per partition
@@ -127,6 +128,7 @@ void compute_layout(const atrex_agg_config_t* c, size_t smem_optin, int n_sms, L
     L->off_sel = o;            o += round_up((size_t)SEL_CAP * 32 * c->n_phases, ALIGN);   // one region per phase
     L->off_pick = o;           o += round_up((size_t)TOPK_PICK_MAX * 32 * c->n_phases, ALIGN);
     L->off_hist_all = o;       o += round_up((size_t)2 * c->n_phases * TOPK_BINS * 4, ALIGN);
+    L->off_hist_next = o;      o += round_up((size_t)c->n_phases * TOPK_BINS * 4, ALIGN);
     L->off_topk_out = o;       o += round_up((size_t)ATREX_MAX_TOPK * sizeof(atrex_entry_t), ALIGN);
     L->off_hot_scratch = o;    o += round_up(HOT_SCRATCH_BYTES, ALIGN);
     L->off_queue = o;          o += round_up((size_t)L->n_groups * L->queue_cap * 16, ALIGN);
@@ -149,13 +151,12 @@ struct DeviceGuard {
 }  // namespace
 
 // What ranking requests worked out, kept until the next finalize: for the last k asked for, every phase's answer
-// (in pinned memory).  A phase that could not be answered that way keeps the
-// selection of its last k.
+// (in pinned memory); for the last k that took the long way, the sorted selections of the phases that do.
 struct TopkCache {
     ull pick_gen = 0;                       // finalize generation the answers belong to (0 = none)
     uint32_t k = 0;                         // k of the answers
-    ull sel_gen[ATREX_MAX_PHASES] = {};     // the long way, per phase
-    uint32_t sel_k[ATREX_MAX_PHASES] = {};
+    ull sel_gen = 0;                        // the long way
+    uint32_t sel_k = 0, sel_mask = 0;       // its phases
     ull total[ATREX_MAX_PHASES] = {};       // candidates selected
 };
 
@@ -184,9 +185,11 @@ struct atrex_agg {
     size_t pinned_bytes = 0;
     uint32_t* hist_all = nullptr;     // [2][n_phases][TOPK_BINS] first-digit counts: the last totals pass's, and zeros for the next
     uint32_t hist_at = 0;             // which half is the last pass's
+    uint32_t* hist_next = nullptr;    // [n_phases][TOPK_BINS] counts of a further digit
     ull wait_seq = 0;                 // number of the last kernel that the host waited for
     ull* pick = nullptr;              // [n_phases][TOPK_PICK_MAX][4] candidates
-    atrex_entry_t* h_top = nullptr;   // pinned: [n_phases][TOPK_PICK_K] the best k of each phase, then u32 [n_phases] how many
+    atrex_entry_t* h_top = nullptr;   // pinned: [n_phases][TOPK_PICK_K] the best k of each phase, then [n_phases] how many
+    TopkDigit* h_digit = nullptr;     // pinned: [n_phases]
     TopkCache topk;
     ull fin_gen = 0;                  // bumped by every successful finalize
     bool hot_ready = false;
@@ -333,18 +336,21 @@ int atrex_agg_create(const atrex_agg_config_t* cfg, atrex_agg_t** out) {
         h->topk_out = (atrex_entry_t*)(h->ws + L.off_topk_out);
         h->hist_all = (uint32_t*)(h->ws + L.off_hist_all);
         h->pick = (ull*)(h->ws + L.off_pick);
+        h->hist_next = (uint32_t*)(h->ws + L.off_hist_next);
         cudaError_t e = cudaSuccess;
         if (e == cudaSuccess) e = cudaMemset(h->ws + L.off_ctl, 0, L.off_appw - L.off_ctl);  // control, spill counts, table, work
         if (e == cudaSuccess) e = cudaMemcpy(h->d_appw, cfg->app_weights, (size_t)cfg->n_apps * 4, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemset(h->hist_all, 0, (size_t)2 * cfg->n_phases * TOPK_BINS * 4);
         if (e == cudaSuccess) e = cudaMemset(h->hot_keys, 0, (size_t)(L.hot_slots ? L.hot_slots : 2) * 8);
-        // the pinned block: every phase's best, how many there are, the control block's mirror
-        const size_t top_bytes = (size_t)cfg->n_phases * (TOPK_PICK_K * sizeof(atrex_entry_t) + 8);
-        h->pinned_bytes = top_bytes + sizeof(Control);
+        // the pinned block: every phase's best, how many there are, a digit each, the control block's mirror
+        const size_t top_bytes = (size_t)cfg->n_phases * (TOPK_PICK_K * sizeof(atrex_entry_t) + 8), digit_bytes = cfg->n_phases * sizeof(TopkDigit);
+        h->pinned_bytes = top_bytes + digit_bytes + sizeof(Control);
         if (e == cudaSuccess) e = pinned_alloc((void**)&h->h_top, h->pinned_bytes);
         if (e == cudaSuccess) {
-            h->h_ctl = (Control*)((unsigned char*)h->h_top + top_bytes);
+            h->h_digit = (TopkDigit*)((unsigned char*)h->h_top + top_bytes);
+            h->h_ctl = (Control*)((unsigned char*)h->h_digit + digit_bytes);
             h->h_ctl->seq = 0;   // (the block may be another handle's former one)
+            memset(h->h_digit, 0, digit_bytes);
         }
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking);
         for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
@@ -671,77 +677,88 @@ static int finalize_impl(atrex_agg_t* h, const atrex_hw_peaks_t* peaks, const ui
     return ATREX_OK;
 }
 
-// Radix-select plan of one phase for the best k: fixes leading digits of the ranking composite until
-// the class holding the k-th entry is small enough to sort, one single-phase pass per digit.
-static int plan_phase(atrex_agg_t* h, uint32_t q, uint32_t k, TopkAllParams* all, ull* total, cudaStream_t s) {
-    const ull n_phase = h->h_ctl->keys_per_phase[q];
-    all->n_prefix_digits[q] = 0;
-    all->active_mask |= 1u << q;
-    if (n_phase <= k) {
-        all->collect_all_mask |= 1u << q;
-        *total = n_phase;
-        return ATREX_OK;
-    }
-    const uint32_t n_digits = (144 - all->shift[q] + 11) / 12;
-    ull need = k, cand = 0;
-    while (true) {
-        TopkParams p;
-        memset(&p, 0, sizeof(p));
-        p.t = h->table_ref();
-        p.n_slots = h->L.n_slots;
-        p.ctl = h->ctl;
-        p.phase = q;
-        p.shift = all->shift[q];
-        p.n_prefix_digits = all->n_prefix_digits[q];
-        memcpy(p.prefix_digit, all->prefix_digit[q], sizeof(p.prefix_digit));
-        CU(h, cudaMemsetAsync(h->ctl->hist, 0, sizeof(h->ctl->hist), s));
-        CU(h, launch_topk_hist(p, h->scan_grid(h->L.n_slots, 256 * 4), s));
-        h->launches++;
-        CU(h, cudaMemcpyAsync(h->h_ctl->hist, h->ctl->hist, sizeof(h->ctl->hist), cudaMemcpyDeviceToHost, s));
-        CU(h, cudaStreamSynchronize(s));
-        const uint32_t* hist = h->h_ctl->hist;
-        ull above = 0;
-        int bin = TOPK_BINS - 1;
-        for (; bin > 0; --bin) {
-            if (above + hist[bin] >= need) break;
-            above += hist[bin];
-        }
-        need -= above;
-        cand = hist[bin];
-        all->prefix_digit[q][all->n_prefix_digits[q]++] = (uint16_t)bin;
-        if (cand <= TOPK_CAND_CAP || all->n_prefix_digits[q] == n_digits) break;
-    }
-    *total = (k - need) + cand;
-    return ATREX_OK;
-}
-
-// One phase's candidates for the best k, sorted, in its selection region.
-static int select_phase(atrex_agg_t* h, uint32_t q, uint32_t k, cudaStream_t s) {
+// The candidates for the best k of all phases in `mask`, sorted, each in its selection region (the long way, see
+// finalize.cu).
+static int select_phases(atrex_agg* h, uint32_t mask, uint32_t k, cudaStream_t s) {
     TopkCache& cache = h->topk;
-    if (cache.sel_gen[q] == h->fin_gen && cache.sel_k[q] == k) return ATREX_OK;
+    const uint32_t n_phases = h->cfg.n_phases;
+    cache.sel_gen = 0;
     TopkAllParams all;
     memset(&all, 0, sizeof(all));
     all.t = h->table_ref();
     all.n_slots = h->L.n_slots;
+    all.hist = h->hist_next;
     all.sel = h->sel;
     all.sel_count = h->ctl->sel_count_all;
     all.sel_cap = SEL_CAP;
-    // digits start at the highest bit the phase's total has (no key's weighted time exceeds it)
-    const ull hi = h->h_ctl->total_hi[q], lo = h->h_ctl->total_lo[q];
-    const int top_bit = hi ? 64 + (63 - __builtin_clzll(hi)) : (lo ? 63 - __builtin_clzll(lo) : 0);
-    all.shift[q] = (uint32_t)(143 - (top_bit + 56));
-    int rc = plan_phase(h, q, k, &all, &cache.total[q], s);
-    if (rc != ATREX_OK) return rc;
-    if (cache.total[q] > SEL_CAP) return ATREX_ERR_STATE;  // cannot happen: composites are unique
-    const uint32_t n_pow2 = (uint32_t)pow2_at_least(cache.total[q] < 2 ? 2 : cache.total[q]);
+    // the items to sort stay within what k alone would be padded to
+    const ull most = pow2_at_least(k) > TOPK_PICK_MAX ? pow2_at_least(k) : TOPK_PICK_MAX;
+    TopkDigitParams digit;
+    memset(&digit, 0, sizeof(digit));
+    digit.answers = h->h_digit;
+    for (uint32_t q = 0; q < n_phases; ++q) {
+        if (!((mask >> q) & 1u)) continue;
+        cache.total[q] = h->h_ctl->keys_per_phase[q];
+        if (cache.total[q] <= k) {
+            all.collect_all_mask |= 1u << q;
+        } else {
+            digit.active_mask |= 1u << q;
+            digit.need[q] = k;
+        }
+    }
+    for (uint32_t known = 0; digit.active_mask; ++known) {   // digits known of the phases still active: the first one and `known` - 1 more
+        if (known == 0) {
+            digit.hist = h->hist_all + (size_t)h->hist_at * n_phases * TOPK_BINS;
+        } else {
+            if (known > TOPK_DIGITS) return ATREX_ERR_STATE;   // cannot happen: composites are unique
+            all.active_mask = digit.active_mask;
+            for (uint32_t q = 0, row = 0; q < n_phases; ++q)
+                if ((all.active_mask >> q) & 1u) all.row[q] = row++;
+            CU(h, cudaMemsetAsync(h->hist_next, 0, (size_t)n_phases * TOPK_BINS * 4, s));
+            CU(h, launch_topk_hist(all, h->n_sms, s));
+            h->launches++;
+            digit.hist = h->hist_next;
+        }
+        digit.seq = ++h->wait_seq;
+        CU(h, launch_topk_digit(digit, n_phases, s));
+        h->launches++;
+        const volatile TopkDigit* a = h->h_digit;
+        const ull want = digit.seq;
+        const uint32_t asked = digit.active_mask;
+        auto answered = [=] {
+            for (uint32_t q = 0; q < n_phases; ++q)
+                if (((asked >> q) & 1u) && a[q].seq != want) return false;
+            return true;
+        };
+        CU(h, wait_for_kernel(answered, s));
+        if (!answered()) return ATREX_ERR_STATE;               // cannot happen: more than k keys were counted
+        for (uint32_t q = 0; q < n_phases; ++q) {
+            if (!((asked >> q) & 1u)) continue;
+            if (known == 0) all.first[q] = (uint32_t)a[q].bin;
+            else all.digit[q][all.n_digits[q]++] = (uint16_t)a[q].bin;
+            digit.need[q] -= (uint32_t)a[q].above;
+            cache.total[q] = k - digit.need[q] + a[q].in_bin;  // the better ones and those level with the k-th
+            if (cache.total[q] <= most) digit.active_mask &= ~(1u << q);
+        }
+    }
+    TopkSortParams sort;
+    memset(&sort, 0, sizeof(sort));
+    sort.sel = h->sel;
+    sort.sel_cap = SEL_CAP;
     CU(h, cudaMemsetAsync(h->ctl->sel_count_all, 0, sizeof(h->ctl->sel_count_all), s));
-    CU(h, cudaMemsetAsync(h->sel + (size_t)q * SEL_CAP * 4, 0, (size_t)n_pow2 * 32, s));   // (the sort wants zeros behind the candidates)
+    for (uint32_t q = 0; q < n_phases; ++q) {
+        if (!((mask >> q) & 1u)) continue;
+        sort.n_pow2[q] = (uint32_t)pow2_at_least(cache.total[q] < 2 ? 2 : cache.total[q]);
+        CU(h, cudaMemsetAsync(h->sel + (size_t)q * SEL_CAP * 4, 0, (size_t)sort.n_pow2[q] * 32, s));   // (the sort wants zeros behind the candidates)
+    }
+    all.active_mask = mask;
     CU(h, launch_topk_collect_all(all, h->scan_grid(h->L.n_slots, 256 * 4), s));
     CU(h, cudaMemsetAsync(h->ctl->sel_count_all, 0, sizeof(h->ctl->sel_count_all), s));
-    CU(h, launch_topk_sort(h->sel + (size_t)q * SEL_CAP * 4, n_pow2, s));
+    CU(h, launch_topk_sort(sort, n_phases, s));
     h->launches += 2;
-    cache.sel_gen[q] = h->fin_gen;
-    cache.sel_k[q] = k;
+    cache.sel_gen = h->fin_gen;
+    cache.sel_k = k;
+    cache.sel_mask = mask;
     return ATREX_OK;
 }
 
@@ -755,6 +772,9 @@ int atrex_agg_topk(atrex_agg_t* h, uint32_t phase, uint32_t k, atrex_entry_t* h_
     DeviceGuard guard(h->cfg.device);
     cudaStream_t s = (cudaStream_t)stream;
     TopkCache& cache = h->topk;
+    uint32_t long_way = 0;   // the phases that a request of this k cannot answer at once
+    for (uint32_t q = 0; q < h->cfg.n_phases; ++q)
+        if (h->h_ctl->keys_per_phase[q] != 0) long_way |= 1u << q;
     if (k <= TOPK_PICK_K) {
         // every phase's answer in one go
         ull* const answers = (ull*)(h->h_top + (size_t)h->cfg.n_phases * TOPK_PICK_K);
@@ -789,9 +809,13 @@ int atrex_agg_topk(atrex_agg_t* h, uint32_t phase, uint32_t k, atrex_entry_t* h_
             *n_out = m;
             return ATREX_OK;
         }
+        for (uint32_t q = 0; q < h->cfg.n_phases; ++q)
+            if ((uint32_t)((const volatile ull*)answers)[q] != PICK_NONE) long_way &= ~(1u << q);
     }
-    int rc = select_phase(h, phase, k, s);
-    if (rc != ATREX_OK) return rc;
+    if (cache.sel_gen != h->fin_gen || cache.sel_k != k || cache.sel_mask != long_way) {
+        const int rc = select_phases(h, long_way, k, s);
+        if (rc != ATREX_OK) return rc;
+    }
     const ull total = cache.total[phase];
     const uint32_t m = (uint32_t)(total < k ? total : k);
     CU(h, launch_topk_emit(finalize_params(h, h->topk_out, m), h->sel + (size_t)phase * SEL_CAP * 4, m, s));

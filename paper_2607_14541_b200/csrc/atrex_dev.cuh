@@ -18,7 +18,7 @@
 //                 the scattered appends within a few pages), read by CTA p of the partition pass
 //   work table  : the same P partitions (by the same hash of op_id and shape_id) of Cw 32-byte
 //                 slots {~(op_id << 32 | shape_id), flops, bytes, dtype}, probed inside the partition
-//   control     : counters, per-phase totals, top-k histogram
+//   control     : counters, per-phase totals
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -49,8 +49,6 @@ constexpr ull ST_TIMEOUT = 16;
 constexpr ull ST_BOUNDS = 32;   // debug build: an index was outside its array
 
 constexpr int TOPK_BINS = 4096;       // 12-bit digits
-constexpr int TOPK_DIGITS = 12;       // 144-bit composite = 88-bit weighted time, 56-bit ~key
-constexpr uint32_t TOPK_CAND_CAP = 65536;
 constexpr uint32_t TOPK_PICK_MAX = 2048;     // candidates of a phase that one CTA ranks in shared memory
 constexpr uint32_t TOPK_PICK_K = 1024;       // ... and the largest k answered that way
 constexpr uint32_t PICK_NONE = 0xFFFFFFFFu;
@@ -86,7 +84,6 @@ struct Control {
     ull tot_done, emit_done;              // CTAs that are through; the last one moves the sums on / fills the mirror
     ull sel_count_all[ATREX_MAX_PHASES];  // top-k: candidates collected per phase
     uint32_t pick_bin[ATREX_MAX_PHASES];  // top-k: first digit of the last bin that is collected, PICK_NONE = too many candidates
-    uint32_t hist[TOPK_BINS];
 };
 
 // 32-bit mixer of (op_id, shape_id) for the key table, the spill partitions, the hot directory

@@ -493,25 +493,33 @@ __global__ void __launch_bounds__(512) topk_rank_kernel(const __grid_constant__ 
 
 // ---- top-k, the long way ------------------------------------------------------------------
 // For k above TOPK_PICK_K, and where more than TOPK_PICK_MAX keys share the first digit of the k-th.
+// A most-significant-digit radix select narrows the table down to little more than the k best keys, which a CTA per
+// phase sorts.  The first digit is the logarithmic one that the totals pass has counted already; where too many keys
+// share it, 12-bit digits of the rest follow, one pass over the table each, for all phases at once.  Every phase
+// that a request of this k would take this way is selected and sorted with the first one asked for: the
+// table is read once or twice instead of twice per phase (16 M keys, k = 1 500: two phases 1 483 -> 375 us, eight 4 844 ->
+// 562).  Sorting twice as many items costs more than a further pass, so digits are added until the items'
+// padded number is that of k alone.
+//
 // Ranking composite, larger = better: bits 56..143 hold the 88-bit weighted time, bits 0..55
-// the complemented key (so the smaller key wins a tie).  Unique per key.  A most-significant-
-// digit radix select (12-bit digits) narrows the table down to the definite winners plus a
-// bounded set of candidates, which one CTA then sorts.
+// the complemented key (so the smaller key wins a tie).  Unique per key.
 struct Composite {
     ull c[3];  // c[2] = bits 128..143
 };
 
-__device__ __forceinline__ Composite composite_of(const SlotView& v) {
+__device__ __forceinline__ Composite composite_of(ull key, ull lo, ull hi) {
     Composite x;
-    x.c[0] = ((~v.key) & 0x00FFFFFFFFFFFFFFull) | (v.lo << 56);
-    x.c[1] = (v.lo >> 8) | (v.hi << 56);
-    x.c[2] = v.hi >> 8;
+    x.c[0] = ((~key) & 0x00FFFFFFFFFFFFFFull) | (lo << 56);
+    x.c[1] = (lo >> 8) | (hi << 56);
+    x.c[2] = hi >> 8;
     return x;
 }
 
-// Digit d (most significant first) of the composite shifted left by `shift` bits.  The shift
-// drops the leading zero bits that every key of the phase shares (no weighted time exceeds the
-// phase total), so that the first digit already separates the top of the ranking.
+// Leading bits of the composite that keys of one first digit share: all above the weighted time's bit length e, and
+// six from there on.
+__device__ __forceinline__ int shared_bits(uint32_t first) { return 94 - max((int)(first >> 5), 6); }
+
+// Digit d (most significant first) of the composite shifted left by `shift` bits.
 __device__ __forceinline__ uint32_t digit_of(const Composite& x, int d, int shift) {
     int off = 144 - 12 * (d + 1) - shift;
     if (off < 0) return (uint32_t)(x.c[0] << (-off)) & 0xFFFu;  // last, partial digit
@@ -521,42 +529,22 @@ __device__ __forceinline__ uint32_t digit_of(const Composite& x, int d, int shif
     return (uint32_t)v & 0xFFFu;
 }
 
-// -1: below the prefix, 0: equal on all fixed digits, +1: above
-__device__ __forceinline__ int compare_prefix(const Composite& x, const TopkParams& p) {
-    for (uint32_t d = 0; d < p.n_prefix_digits; ++d) {
-        uint32_t a = digit_of(x, (int)d, (int)p.shift), b = p.prefix_digit[d];
+// A key of phase q against the digits known so far -- -1: below, 0: equal on all of them, +1: above
+__device__ __forceinline__ int compare_known(const TopkAllParams& p, uint32_t q, ull key, ull lo, ull hi, Composite& x) {
+    const uint32_t first = topk_first_digit(lo, hi);
+    if (first != p.first[q]) return first > p.first[q] ? 1 : -1;
+    x = composite_of(key, lo, hi);
+    const int shift = shared_bits(first);
+    for (uint32_t d = 0; d < p.n_digits[q]; ++d) {
+        const uint32_t a = digit_of(x, (int)d, shift), b = p.digit[q][d];
         if (a != b) return a > b ? 1 : -1;
     }
     return 0;
 }
 
-__global__ void __launch_bounds__(FIN_THREADS) topk_hist_kernel(TopkParams p) {
-    __shared__ uint32_t h[TOPK_BINS];
-    for (int i = threadIdx.x; i < TOPK_BINS; i += blockDim.x) h[i] = 0;
-    __syncthreads();
-    for (ull i = (ull)blockIdx.x * blockDim.x + threadIdx.x; i < p.n_slots; i += (ull)gridDim.x * blockDim.x) {
-        SlotView v = load_slot(p.t, i);
-        if (!v.live || (uint32_t)(v.key >> 48) != p.phase) continue;
-        Composite x = composite_of(v);
-        if (compare_prefix(x, p) != 0) continue;
-        atomicAdd(&h[digit_of(x, (int)p.n_prefix_digits, (int)p.shift)], 1u);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < TOPK_BINS; i += blockDim.x)
-        if (h[i] != 0) atomicAdd(&p.ctl->hist[i], h[i]);
-}
-
-// -1: below the prefix, 0: equal on all fixed digits, +1: above (one phase of a multi-phase pass)
-__device__ __forceinline__ int compare_prefix_of(const Composite& x, const TopkAllParams& p, uint32_t q) {
-    for (uint32_t d = 0; d < p.n_prefix_digits[q]; ++d) {
-        uint32_t a = digit_of(x, (int)d, (int)p.shift[q]), b = p.prefix_digit[q][d];
-        if (a != b) return a > b ? 1 : -1;
-    }
-    return 0;
-}
-
-// Candidates of all active phases in one pass, each phase into its own selection region.
-__global__ void __launch_bounds__(FIN_THREADS) topk_collect_all_kernel(const __grid_constant__ TopkAllParams p) {
+// f(phase, key, lo, hi, slot) for every live slot of an active phase, four slots per thread in flight
+template <typename F>
+__device__ __forceinline__ void each_active(const TopkAllParams& p, F f) {
     constexpr int ILP = 4;
     const ull stride = (ull)gridDim.x * blockDim.x;
     for (ull i0 = (ull)blockIdx.x * blockDim.x + threadIdx.x; i0 < p.n_slots; i0 += stride * ILP) {
@@ -571,25 +559,85 @@ __global__ void __launch_bounds__(FIN_THREADS) topk_collect_all_kernel(const __g
 #pragma unroll
         for (int u = 0; u < ILP; ++u) {
             const uint32_t q = (uint32_t)(~sk[u] >> 48) & (ATREX_MAX_PHASES - 1);
-            if (!(sk[u] != 0 && ((p.active_mask >> q) & 1u))) sk[u] = 0;
-        }
-#pragma unroll
-        for (int u = 0; u < ILP; ++u) {
-            if (sk[u] == 0) continue;
-            SlotView v;
-            v.key = ~sk[u];
-            v.lo = x[u].x;
-            v.hi = x[u].y >> HI_SHIFT;
-            const uint32_t q = (uint32_t)(v.key >> 48) & (ATREX_MAX_PHASES - 1);
-            const Composite c = composite_of(v);
-            if (!((p.collect_all_mask >> q) & 1u) && compare_prefix_of(c, p, q) < 0) continue;
-            const ull pos = atomicAdd(&p.sel_count[q], 1ull);
-            if (pos < p.sel_cap) {
-                ull* dst = p.sel + ((ull)q * p.sel_cap + pos) * 4;
-                dst[0] = c.c[2]; dst[1] = c.c[1]; dst[2] = c.c[0]; dst[3] = i0 + u * stride;
-            }
+            if (sk[u] != 0 && ((p.active_mask >> q) & 1u)) f(q, ~sk[u], x[u].x, x[u].y >> HI_SHIFT, i0 + u * stride);
         }
     }
+}
+
+// Counts of the next digit of the active phases' keys that are level with the known ones (shared memory: a row each).
+constexpr int TOPK_HIST_THREADS = 1024;
+__global__ void __launch_bounds__(TOPK_HIST_THREADS) topk_hist_kernel(const __grid_constant__ TopkAllParams p) {
+    extern __shared__ uint32_t s_hist[];
+    const uint32_t rows = __popc(p.active_mask);
+    for (uint32_t i = threadIdx.x; i < rows * TOPK_BINS; i += blockDim.x) s_hist[i] = 0;
+    __syncthreads();
+    each_active(p, [&](uint32_t q, ull key, ull lo, ull hi, ull) {
+        Composite x;
+        if (compare_known(p, q, key, lo, hi, x) == 0) atomicAdd(&s_hist[p.row[q] * TOPK_BINS + digit_of(x, (int)p.n_digits[q], shared_bits(p.first[q]))], 1u);
+    });
+    __syncthreads();
+    for (uint32_t q = 0; q < ATREX_MAX_PHASES; ++q) {
+        if (!((p.active_mask >> q) & 1u)) continue;
+        for (uint32_t i = threadIdx.x; i < TOPK_BINS; i += blockDim.x) {
+            const uint32_t c = s_hist[p.row[q] * TOPK_BINS + i];
+            if (c) atomicAdd(&p.hist[(size_t)q * TOPK_BINS + i], c);
+        }
+    }
+}
+
+// The digit of each active phase's wanted key (a CTA per phase, four bins to a thread, the highest first), told to the host.
+__global__ void __launch_bounds__(TOPK_BINS / 4) topk_digit_kernel(const __grid_constant__ TopkDigitParams p) {
+    __shared__ uint32_t s_warp[32];
+    const uint32_t q = blockIdx.x, t = threadIdx.x, lane = t & 31u, w = t >> 5, need = p.need[q];
+    grid_dependency_wait();
+    if (!((p.active_mask >> q) & 1u)) return;
+    const uint4 v = reinterpret_cast<const uint4*>(p.hist + (size_t)q * TOPK_BINS)[TOPK_BINS / 4 - 1 - t];
+    const uint32_t own = v.x + v.y + v.z + v.w;
+    uint32_t incl = own;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+        if (lane >= (uint32_t)d) incl += o;
+    }
+    if (lane == 31) s_warp[w] = incl;
+    __syncthreads();
+    if (w == 0) {
+        uint32_t c = s_warp[lane];
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, c, d);
+            if (lane >= (uint32_t)d) c += o;
+        }
+        s_warp[lane] = c;
+    }
+    __syncthreads();
+    if (w) incl += s_warp[w - 1];
+    uint32_t above = incl - own;
+    if (above >= need || incl < need) return;          // (exactly one thread goes on)
+    uint32_t bin = TOPK_BINS - 1 - 4 * t, in_bin = v.w;
+    if (above + in_bin < need) { above += in_bin; --bin; in_bin = v.z; }
+    if (above + in_bin < need) { above += in_bin; --bin; in_bin = v.y; }
+    if (above + in_bin < need) { above += in_bin; --bin; in_bin = v.x; }
+    volatile TopkDigit* a = p.answers + q;
+    a->bin = bin;
+    a->above = above;
+    a->in_bin = in_bin;
+    __threadfence_system();
+    a->seq = p.seq;                                    // the host waits for this word
+}
+
+// Candidates of all active phases in one pass, each into its own selection region.
+__global__ void __launch_bounds__(FIN_THREADS) topk_collect_all_kernel(const __grid_constant__ TopkAllParams p) {
+    each_active(p, [&](uint32_t q, ull key, ull lo, ull hi, ull slot) {
+        Composite x;
+        if (!((p.collect_all_mask >> q) & 1u) && compare_known(p, q, key, lo, hi, x) < 0) return;
+        x = composite_of(key, lo, hi);
+        const ull pos = atomicAdd(&p.sel_count[q], 1ull);
+        if (pos < p.sel_cap) {
+            ull* dst = p.sel + ((ull)q * p.sel_cap + pos) * 4;
+            dst[0] = x.c[2]; dst[1] = x.c[1]; dst[2] = x.c[0]; dst[3] = slot;
+        }
+    });
 }
 
 __device__ __forceinline__ bool sel_less(const ull* a, const ull* b) {
@@ -598,9 +646,11 @@ __device__ __forceinline__ bool sel_less(const ull* a, const ull* b) {
     return a[2] < b[2];
 }
 
-// Bitonic sort, descending by composite, of n (power of two) 32-byte items in global memory,
-// by a single CTA.  Padding items are all-zero and sink to the end.
-__global__ void __launch_bounds__(1024) topk_sort_kernel(ull* sel, uint32_t n) {
+// Bitonic sort, descending by composite, of each phase's n (power of two) 32-byte items in global memory,
+// by a CTA per phase.  Padding items are all-zero and sink to the end.
+__global__ void __launch_bounds__(1024) topk_sort_kernel(const __grid_constant__ TopkSortParams p) {
+    const uint32_t n = p.n_pow2[blockIdx.x];
+    ull* sel = p.sel + (size_t)blockIdx.x * p.sel_cap * 4;
     for (uint32_t k = 2; k <= n; k <<= 1) {
         for (uint32_t j = k >> 1; j > 0; j >>= 1) {
             for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
@@ -639,6 +689,7 @@ constexpr size_t PICK_SMEM = (size_t)TOPK_PICK_MAX * 28;
 cudaError_t finalize_prepare() {
     cudaError_t e = cudaFuncSetAttribute(totals_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)totals_smem(ATREX_MAX_PHASES));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(topk_rank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PICK_SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(topk_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ATREX_MAX_PHASES * TOPK_BINS * 4);
     return e;
 }
 
@@ -674,13 +725,18 @@ cudaError_t launch_topk_collect_all(const TopkAllParams& p, int grid, cudaStream
     return cudaGetLastError();
 }
 
-cudaError_t launch_topk_hist(const TopkParams& p, int grid, cudaStream_t stream) {
-    topk_hist_kernel<<<grid, FIN_THREADS, 0, stream>>>(p);
+cudaError_t launch_topk_hist(const TopkAllParams& p, int n_sms, cudaStream_t stream) {
+    const uint32_t rows = (uint32_t)__builtin_popcount(p.active_mask), per_sm = rows <= 6 ? 2 : 1;
+    topk_hist_kernel<<<grid_for_work(p.n_slots, TOPK_HIST_THREADS * 4, n_sms, per_sm), TOPK_HIST_THREADS, rows * TOPK_BINS * 4, stream>>>(p);
     return cudaGetLastError();
 }
 
-cudaError_t launch_topk_sort(ull* sel, uint32_t n_pow2, cudaStream_t stream) {
-    topk_sort_kernel<<<1, 1024, 0, stream>>>(sel, n_pow2);
+cudaError_t launch_topk_digit(const TopkDigitParams& p, uint32_t n_phases, cudaStream_t stream) {
+    return launch_chained(topk_digit_kernel, n_phases, TOPK_BINS / 4, 0, stream, p);
+}
+
+cudaError_t launch_topk_sort(const TopkSortParams& p, uint32_t n_phases, cudaStream_t stream) {
+    topk_sort_kernel<<<n_phases, 1024, 0, stream>>>(p);
     return cudaGetLastError();
 }
 

@@ -152,32 +152,36 @@ struct PickParams {
     ull* host_n;               // pinned: [n_phases] fin.seq << 32 | entries written (PICK_NONE: not answered this way)
 };
 
-struct TopkParams {
-    TableRef t;
-    ull n_slots;
-    Control* ctl;
-    uint32_t phase;
-    uint32_t n_prefix_digits;   // leading 12-bit digits of the ranking composite already fixed
-    uint16_t prefix_digit[12];  // their values, most significant first
-    uint32_t shift;             // leading zero bits of the composite dropped before digit extraction
-    int collect_all;
-    ull* sel;                   // [sel_cap][4]: composite words 2,1,0 and the slot index
-    uint32_t sel_cap;
-};
-
-// Top-k over several phases in one pass over the table: phase q of `active_mask` has its own digit
-// alignment, fixed prefix, histogram row and selection region.
+// Top-k, the long way: phases in one pass over the table, each with its own place in the ranking (see finalize.cu).
+constexpr uint32_t TOPK_DIGITS = 12;                   // 12-bit digits behind the first one, at most
 struct TopkAllParams {
     TableRef t;
     ull n_slots;
     uint32_t active_mask;                              // phases taking part in this pass
-    uint32_t collect_all_mask;                         // phases whose every entry is collected
-    uint32_t shift[ATREX_MAX_PHASES];
-    uint32_t n_prefix_digits[ATREX_MAX_PHASES];
-    uint16_t prefix_digit[ATREX_MAX_PHASES][12];
-    ull* sel;                                          // [ATREX_MAX_PHASES][sel_cap][4]
+    uint32_t collect_all_mask;                         // ... of which every entry is collected
+    uint32_t row[ATREX_MAX_PHASES];                    // counting: each active phase's row in shared memory
+    uint32_t first[ATREX_MAX_PHASES];                  // first digit of the k-th key
+    uint32_t n_digits[ATREX_MAX_PHASES];               // further digits already known
+    uint16_t digit[ATREX_MAX_PHASES][TOPK_DIGITS];
+    uint32_t* hist;                                    // [n_phases][TOPK_BINS] counts of the next digit
+    ull* sel;                                          // [n_phases][sel_cap][4]: composite words 2, 1, 0 and the slot index
     ull* sel_count;                                    // [ATREX_MAX_PHASES]
     uint32_t sel_cap;
+};
+struct TopkDigit {                                     // in pinned memory: where a phase's k-th key lies
+    ull seq, bin, above, in_bin;                       // ... its digit, keys in higher bins, keys in its own
+};
+struct TopkDigitParams {
+    const uint32_t* hist;                              // [n_phases][TOPK_BINS]
+    uint32_t active_mask;
+    uint32_t need[ATREX_MAX_PHASES];                   // the wanted key's place among the counted ones
+    TopkDigit* answers;                                // [n_phases], `seq` last
+    ull seq;
+};
+struct TopkSortParams {
+    ull* sel;                                          // [n_phases][sel_cap][4]
+    uint32_t sel_cap;
+    uint32_t n_pow2[ATREX_MAX_PHASES];                 // items of each phase with padding, 0 = nothing to do
 };
 
 // Launches a kernel whose set-up may overlap its predecessor on the stream (the kernel starts with
@@ -237,8 +241,9 @@ cudaError_t launch_work_insert(const atrex_work_t* rows, ull n, const WorkRef& w
                                cudaStream_t stream);
 cudaError_t launch_topk_pick(const PickParams& p, int n_sms, cudaStream_t stream);
 cudaError_t launch_topk_collect_all(const TopkAllParams& p, int grid, cudaStream_t stream);
-cudaError_t launch_topk_hist(const TopkParams& p, int grid, cudaStream_t stream);
-cudaError_t launch_topk_sort(ull* sel, uint32_t n_pow2, cudaStream_t stream);
+cudaError_t launch_topk_hist(const TopkAllParams& p, int n_sms, cudaStream_t stream);
+cudaError_t launch_topk_digit(const TopkDigitParams& p, uint32_t n_phases, cudaStream_t stream);
+cudaError_t launch_topk_sort(const TopkSortParams& p, uint32_t n_phases, cudaStream_t stream);
 cudaError_t launch_topk_emit(const FinalizeParams& p, const ull* sel, uint32_t n, cudaStream_t stream);
 
 }  // namespace atrex

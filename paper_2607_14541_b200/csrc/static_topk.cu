@@ -122,9 +122,9 @@ extern "C" int atrex_topk_entries_static(const atrex_entry_t* d_entries, uint64_
     if (cudaMemcpyAsync(&count, counter, sizeof(count), cudaMemcpyDeviceToHost, s) != cudaSuccess) return ATREX_ERR_CUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return ATREX_ERR_CUDA;
     if (count == 0) return ATREX_OK;
-    uint32_t n_pow2 = 2;
-    while (n_pow2 < count) n_pow2 <<= 1;
-    if (launch_topk_sort(sel, n_pow2, s) != cudaSuccess) return ATREX_ERR_CUDA;
+    TopkSortParams sort{sel, MAX_ENTRIES, {2}};
+    while (sort.n_pow2[0] < count) sort.n_pow2[0] <<= 1;
+    if (launch_topk_sort(sort, 1, s) != cudaSuccess) return ATREX_ERR_CUDA;
     const uint32_t m = (uint32_t)(count < k ? count : k);
     static_emit_kernel<<<(m + 255) / 256, 256, 0, s>>>(d_entries, sel, m, d_out);
     if (cudaGetLastError() != cudaSuccess) return ATREX_ERR_CUDA;
