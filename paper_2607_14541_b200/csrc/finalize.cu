@@ -12,7 +12,7 @@
 namespace atrex {
 
 constexpr int FIN_THREADS = 256;
-constexpr int TOT_THREADS = 256, TOT_ILP = 6;
+constexpr uint32_t TOT_ILP = 6;
 
 struct SlotView {
     ull key, count, lo, hi;
@@ -43,15 +43,17 @@ __device__ __forceinline__ uint32_t topk_first_digit(ull lo, ull hi) {
     else m = (uint32_t)(e >= 6 ? lo >> (e - 6) : lo << (6 - e));
     return ((uint32_t)e << 5) | (m & 31u);
 }
-static_assert((88 << 5) + 31 < TOPK_BINS, "first digits fit the histogram");
+constexpr uint32_t FIRST_BINS = (88 << 5) + 32;
+static_assert(FIRST_BINS <= TOPK_BINS && FIRST_BINS % 4 == 0, "first digits fit the histogram");
 
 // ---- per-phase totals -------------------------------------------------------------------
 // Each thread keeps private per-phase 128-bit sums in its own shared-memory column; columns are added per
 // CTA and folded into accumulators in the control block with a carry-aware pair of atomics.  The last CTA
 // moves the accumulators to their place and clears them (and the emit kernel's output count), so that no
 // launch is spent on clearing.  On the way the keys are counted by the first digit of the top-k selection (per
-// phase, for topk_plan_kernel), which saves that call a pass over the table; the next pass's counters are
-// cleared here.  Bound by DRAM (566 MB: 120 us).
+// phase, for the top-k), which saves that call a pass over the table; the next pass's counters are
+// cleared here.  Bound by DRAM (566 MB: 120 us), given 512 threads per SM or more: shared memory holds that many up to eight
+// phases (16 M keys, whole finalize: five phases 650 -> 569 us, eight 650 -> 582; with one CTA of 256 threads before).
 __device__ __forceinline__ bool last_cta(ull* done) {
     __shared__ bool s_last;
     __syncthreads();
@@ -64,29 +66,32 @@ __device__ __forceinline__ bool last_cta(ull* done) {
     return s_last;
 }
 
-constexpr size_t totals_smem(uint32_t n_phases) { return (size_t)n_phases * (TOT_THREADS * 28 + TOPK_BINS * 4); }
+constexpr uint32_t TOT_THREADS = 256, TOT_WIDE_FROM = 7;       // (from seven phases on one CTA per SM, of twice as many threads)
+constexpr uint32_t totals_threads(uint32_t n_phases) { return n_phases < TOT_WIDE_FROM ? TOT_THREADS : 2 * TOT_THREADS; }
+constexpr size_t totals_smem(uint32_t n_phases) { return (size_t)n_phases * (totals_threads(n_phases) * 28 + FIRST_BINS * 4); }
 
-__global__ void __launch_bounds__(TOT_THREADS) totals_kernel(TableRef tab, ull n_slots, uint32_t n_phases, const __grid_constant__ GivenTotals given,
+template <uint32_t THREADS>
+__global__ void __launch_bounds__(THREADS) totals_kernel(TableRef tab, ull n_slots, uint32_t n_phases, const __grid_constant__ GivenTotals given,
                                                              uint32_t* hist, uint32_t* next_hist) {
     Control* ctl = tab.ctl;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    ull(*s_lo)[TOT_THREADS] = reinterpret_cast<ull(*)[TOT_THREADS]>(smem_raw);       // [n_phases] each
-    ull(*s_hi)[TOT_THREADS] = s_lo + n_phases;
-    ull(*s_cnt)[TOT_THREADS] = s_hi + n_phases;
-    uint32_t(*s_nk)[TOT_THREADS] = reinterpret_cast<uint32_t(*)[TOT_THREADS]>(s_cnt + n_phases);
-    uint32_t* s_hist = reinterpret_cast<uint32_t*>(s_nk + n_phases);                 // [n_phases][TOPK_BINS]
-    const int t = threadIdx.x;
-    for (uint32_t p = 0; p < n_phases; ++p) {
-        s_lo[p][t] = 0; s_hi[p][t] = 0; s_cnt[p][t] = 0; s_nk[p][t] = 0;
+    const uint32_t t = threadIdx.x;
+    ull* s_lo = reinterpret_cast<ull*>(smem_raw);                                    // [n_phases][THREADS] each
+    ull* s_hi = s_lo + n_phases * THREADS;
+    ull* s_cnt = s_hi + n_phases * THREADS;
+    uint32_t* s_nk = reinterpret_cast<uint32_t*>(s_cnt + n_phases * THREADS);
+    uint32_t* s_hist = s_nk + n_phases * THREADS;                                    // [n_phases][FIRST_BINS]
+    for (uint32_t i = t; i < n_phases * THREADS; i += THREADS) {
+        s_lo[i] = 0; s_hi[i] = 0; s_cnt[i] = 0; s_nk[i] = 0;
     }
-    for (uint32_t i = t; i < n_phases * TOPK_BINS; i += TOT_THREADS) s_hist[i] = 0;
+    for (uint32_t i = t; i < n_phases * FIRST_BINS; i += THREADS) s_hist[i] = 0;
     __syncthreads();
     grid_dependency_wait();
-    for (uint32_t i = blockIdx.x * TOT_THREADS + t; i < n_phases * TOPK_BINS / 4; i += gridDim.x * TOT_THREADS)
+    for (uint32_t i = blockIdx.x * THREADS + t; i < n_phases * TOPK_BINS / 4; i += gridDim.x * THREADS)
         reinterpret_cast<uint4*>(next_hist)[i] = make_uint4(0, 0, 0, 0);
     // six slots per thread in flight
-    const ull stride = (ull)gridDim.x * blockDim.x;
-    for (ull i0 = (ull)blockIdx.x * blockDim.x + t; i0 < n_slots; i0 += stride * TOT_ILP) {
+    const ull stride = (ull)gridDim.x * THREADS;
+    for (ull i0 = (ull)blockIdx.x * THREADS + t; i0 < n_slots; i0 += stride * TOT_ILP) {
         ull sk[TOT_ILP];
         ulonglong2 x[TOT_ILP];
 #pragma unroll
@@ -105,27 +110,29 @@ __global__ void __launch_bounds__(TOT_THREADS) totals_kernel(TableRef tab, ull n
                 atomicAdd(&ctl->acc_keys[p], 1ull);
                 continue;
             }
-            const ull o = s_lo[p][t], n = o + x[u].x;
-            s_lo[p][t] = n;
-            s_hi[p][t] += hi + (n < o ? 1ull : 0ull);
-            s_cnt[p][t] += x[u].y & COUNT_MASK;
-            s_nk[p][t] += 1;
-            atomicAdd(&s_hist[p * TOPK_BINS + topk_first_digit(x[u].x, hi)], 1u);
+            const uint32_t at = p * THREADS + t;
+            const ull o = s_lo[at], n = o + x[u].x;
+            s_lo[at] = n;
+            s_hi[at] += hi + (n < o ? 1ull : 0ull);
+            s_cnt[at] += x[u].y & COUNT_MASK;
+            s_nk[at] += 1;
+            atomicAdd(&s_hist[p * FIRST_BINS + topk_first_digit(x[u].x, hi)], 1u);
         }
     }
     grid_dependents_launch();
     __syncthreads();
-    for (uint32_t i = t; i < n_phases * TOPK_BINS; i += TOT_THREADS)
-        if (s_hist[i] != 0) atomicAdd(&hist[i], s_hist[i]);
+    for (uint32_t p = 0; p < n_phases; ++p)
+        for (uint32_t i = t; i < FIRST_BINS; i += THREADS)
+            if (s_hist[p * FIRST_BINS + i] != 0) atomicAdd(&hist[p * TOPK_BINS + i], s_hist[p * FIRST_BINS + i]);
     const uint32_t lane = t & 31;
-    for (uint32_t p = t >> 5; p < n_phases; p += TOT_THREADS / 32) {   // a warp per phase
+    for (uint32_t p = t >> 5; p < n_phases; p += THREADS / 32) {   // a warp per phase
         ull lo = 0, hi = 0, cnt = 0, nk = 0;
-        for (int j = lane; j < TOT_THREADS; j += 32) {
-            const ull n = lo + s_lo[p][j];
-            hi += s_hi[p][j] + (n < lo ? 1ull : 0ull);
+        for (uint32_t j = p * THREADS + lane; j < (p + 1) * THREADS; j += 32) {
+            const ull n = lo + s_lo[j];
+            hi += s_hi[j] + (n < lo ? 1ull : 0ull);
             lo = n;
-            cnt += s_cnt[p][j];
-            nk += s_nk[p][j];
+            cnt += s_cnt[j];
+            nk += s_nk[j];
         }
 #pragma unroll
         for (int d = 16; d; d >>= 1) {
@@ -687,7 +694,8 @@ __global__ void __launch_bounds__(FIN_THREADS) topk_emit_kernel(FinalizeParams p
 constexpr size_t PICK_SMEM = (size_t)TOPK_PICK_MAX * 28;
 
 cudaError_t finalize_prepare() {
-    cudaError_t e = cudaFuncSetAttribute(totals_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)totals_smem(ATREX_MAX_PHASES));
+    cudaError_t e = cudaFuncSetAttribute(totals_kernel<TOT_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)totals_smem(TOT_WIDE_FROM - 1));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(totals_kernel<2 * TOT_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)totals_smem(ATREX_MAX_PHASES));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(topk_rank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PICK_SMEM);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(topk_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ATREX_MAX_PHASES * TOPK_BINS * 4);
     return e;
@@ -696,9 +704,11 @@ cudaError_t finalize_prepare() {
 cudaError_t launch_totals(const TableRef& t, ull n_slots, uint32_t n_phases, const GivenTotals& given, uint32_t* hist, uint32_t* next_hist,
                           int n_sms, cudaStream_t stream) {
     const size_t smem = totals_smem(n_phases);
+    const uint32_t threads = totals_threads(n_phases);
     uint32_t per_sm = (uint32_t)(233472 / (smem + 1024));
     if (per_sm > 4) per_sm = 4;
-    return launch_chained(totals_kernel, grid_for_work(n_slots, TOT_THREADS * TOT_ILP, n_sms, per_sm), TOT_THREADS, smem, stream, t, n_slots,
+    auto* kernel = threads == TOT_THREADS ? totals_kernel<TOT_THREADS> : totals_kernel<2 * TOT_THREADS>;
+    return launch_chained(kernel, grid_for_work(n_slots, threads * TOT_ILP, n_sms, per_sm), threads, smem, stream, t, n_slots,
                           n_phases, given, hist, next_hist);
 }
 
