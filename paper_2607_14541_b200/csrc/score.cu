@@ -897,6 +897,38 @@ __global__ void __launch_bounds__(1024)
     }
 }
 
+// One candidate per warp (true) or per CTA (false); `held`: candidates an SM holds at once by warps.  A CTA has the shorter
+// chain, a warp the smaller sum of work, so the warps win once every SM has several candidates, and the sooner the better
+// the operators fill a warp's lanes.  Device times in us, warps / CTAs, on both sides of each line:
+//   up to 500 units     4 candidates per SM and one per unit (groups up to 48), 16 per SM beyond: 450 units in 16 operators, 660
+//                       candidates 7.8 / 11.1; 300 in 12, 450 candidates 9.4 / 8.6
+//   groups up to 30     8 per SM, and one per unit, 1.4 from 1 500 units on, where fewer warps fit an SM: 1 000 units in 35
+//                       operators, 900 candidates 22.0 / 22.0, 2 000 25.0 / 37.2; 2 000 units in 83, 1 500 candidates 58 / 43
+//   up to 50            5 per SM (8 from 44 on): two lanes an operator are full, and a CTA's warps search every group: 1 400 units
+//                       in 35 operators, 600 candidates 27.5 / 27.9, 1 500 36.0 / 44.0
+//   beyond              16 per SM up to a mean of 64, with fewer units the more groups are then too large for two lanes: 800 units
+//                       in 15 operators, 2 400 candidates 18 / 34; 1 000 in 17, 2 400 candidates 48 / 39, 3 500 41 / 57; 2 000 in
+//                       31, 2 400 candidates 157 / 67
+bool by_warps(uint32_t n, uint32_t n_ops, uint32_t b, uint32_t sms, uint32_t held) {
+    if (held < (n <= 24 * n_ops ? 12u : 6u)) return false;
+    if (n <= 500) return n <= 48 * n_ops ? b >= 4 * sms && b >= n : b >= 16 * sms;
+    const bool enough = b * 10ull >= n * (n <= 1500 ? 10ull : 14ull);
+    if (n <= 30 * n_ops) return b >= 8 * sms && enough;
+    if (n <= 50 * n_ops) return b >= (n <= 44 * n_ops ? 5 : 8) * sms && (n <= 2200 || enough);
+    if (n <= 700) return b >= 16 * sms;
+    return b >= 16 * sms && n <= 64 * n_ops && (ull)n * (n - 44 * n_ops) <= (b < 20 * sms ? 14000ull : 19000ull) * n_ops;
+}
+
+// Threads of a CTA that holds one candidate.  Where there are more candidates than the SMs hold at 256 threads (four CTAs
+// each, by registers), smaller CTAs take all of them at once (700 units in 28 operators: 600 candidates 16.6 us at 256 threads,
+// 11.0 at 192, 900 18.9, 13.8 at 128).  Larger groups need the warps (19 operators of 36: 825 candidates 16.9, 18.2 at 128).
+uint32_t cta_threads(uint32_t n, uint32_t n_ops, uint32_t b, uint32_t sms) {
+    if (n > 4096) return n <= 13000 ? 512u : 1024u;
+    if (n > 1400 || b <= 4 * sms) return 256u;
+    if (b <= 5 * sms) return n <= 36 * n_ops ? 192u : 256u;
+    return n <= 30 * n_ops && (n <= 800 || b <= 8 * sms) ? 128u : 256u;
+}
+
 constexpr int SCORE_MAX_DEVICES = 64;
 std::mutex g_score_lock;
 int g_score_sms[SCORE_MAX_DEVICES];   // per device: its SM count, once the kernels' shared-memory limit has been raised there
@@ -959,15 +991,11 @@ extern "C" int atrex_score_aggregate(const double* d_roofline_s, const uint32_t*
     }
     const uint32_t n = (uint32_t)n_units, b = (uint32_t)n_candidates;
     ull* errors = reinterpret_cast<ull*>(d_errors);
-    // One candidate per warp pays once a few warps on every SM have one; a CTA per candidate is quicker for fewer, by
-    // its shorter chain.  Where most groups are too large for the lanes' columns, the warps search them one by
-    // one: later (three rounds of CTAs), and only for small candidates.  A lane to an operator up to a mean group of
-    // 24, two above (8 000 candidates: 440 units in 14 operators 70 -> 29 us, 1 000 units in 25 operators 181 -> 62;
-    // 440 units in 27 operators 31, by pairs 42).
+    // A lane to an operator up to a mean group of 24, two above (8 000 candidates: 440 units in 14 operators 70 -> 29 us,
+    // 1 000 units in 25 operators 181 -> 62; 440 units in 27 operators 31, by pairs 42).
     const bool pairs = n > 24u * n_ops;
     const uint32_t slots = warp_slots(n, n_ops, pairs);
     const WarpLayout wl(n, n_ops, slots);
-    const bool sorted = n <= 48u * n_ops;
     uint32_t warps = 0, per_sm = 0;    // the split of an SM's shared memory that holds most warps
     for (uint32_t c = WARP_KERNEL_CTAS; c >= 1; --c) {
         const size_t room = SM_SMEM / c - 1024 < (size_t)SCORE_SMEM_MAX ? SM_SMEM / c - 1024 : (size_t)SCORE_SMEM_MAX;
@@ -976,15 +1004,14 @@ extern "C" int atrex_score_aggregate(const double* d_roofline_s, const uint32_t*
         if (k * c > warps * per_sm) warps = k, per_sm = c;
     }
     const uint32_t sms = (uint32_t)n_sms, held = warps * per_sm;
-    const bool enough = sorted ? b >= 4u * sms && b >= n && held >= (pairs ? 6u : 12u) : b >= 16u * sms && held >= 16 && (n <= 72u * n_ops || n <= 768);
-    if (enough && slots + n < SLOT_MASK) {
+    if (by_warps(n, n_ops, b, sms, held) && slots + n < SLOT_MASK) {
         const uint32_t want = (b + warps - 1) / warps, most = (uint32_t)n_sms * per_sm;
         const size_t warp_smem = wl.warps + (size_t)wl.warp_bytes * warps;
         auto* kernel = pairs ? score_warp_kernel<true> : score_warp_kernel<false>;
         kernel<<<want < most ? want : most, warps * 32, warp_smem, (cudaStream_t)stream>>>(
             d_roofline_s, d_unit_op, n, d_t_cand, d_correct, b, d_w, n_ops, slots, d_s_agg, d_s_op, errors);
     } else {
-        const uint32_t threads = n <= 4096 ? 256u : (n <= 13000 ? 512u : 1024u);
+        const uint32_t threads = cta_threads(n, n_ops, b, sms);
         const size_t smem = CtaLayout(n, n_ops, threads).total;
         per_sm = (uint32_t)(SM_SMEM / (smem + 2560));
         if (per_sm > 1024u / threads) per_sm = 1024u / threads;   // (64 registers a thread)

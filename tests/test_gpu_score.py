@@ -87,3 +87,21 @@ def test_score_parity_at_group_size_edges(groups, batch):
     assert got[0].tobytes() == exp[0].tobytes()
     assert got[1].tobytes() == exp[1].tobytes()
     assert np.array_equal(got[2], exp[2])
+
+
+@pytest.mark.parametrize("batch", [592, 593, 740, 741, 1_184, 1_185])
+@pytest.mark.parametrize("n_units,n_ops", [(700, 28), (800, 22), (801, 27), (1_400, 56), (1_401, 40), (500, 10), (501, 16)])
+def test_score_parity_where_the_kernels_change(n_units, n_ops, batch):
+    """Candidates on both sides of what the SMs hold at once (CTAs of 256, 192 and 128 threads, one candidate per warp)."""
+    rng = np.random.default_rng(n_units + batch)
+    unit_op = rng.integers(0, n_ops + 1, n_units).astype(np.uint32)       # one operator in n_ops + 1 is out of range
+    roof = np.exp(rng.uniform(np.log(1e-6), np.log(1e-1), n_units))
+    t = roof[None, :] / rng.uniform(0.01, 1.02, (batch, n_units))
+    t[0::5] = roof / np.round(rng.uniform(0.1, 1.0, n_units), 1)          # ties
+    ok = rng.random((batch, n_units)) < 0.8
+    w = rng.dirichlet(np.ones(n_ops))
+    exp = oracle.score_candidates(roof, unit_op, t, ok, w)
+    got = run_gpu(roof, unit_op, t, ok, w)
+    assert got[0].tobytes() == exp[0].tobytes()
+    assert got[1].tobytes() == exp[1].tobytes()
+    assert np.array_equal(got[2], exp[2])
