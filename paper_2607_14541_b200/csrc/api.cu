@@ -459,6 +459,10 @@ static int ingest_launch(atrex_agg* h, const atrex_record_t* recs, uint64_t n, c
     // Small calls go straight into the table (direct.cu).  Measured per 2^20 records: 40 to 65 us that way, 16 to 25
     // by the two-pass route, which costs 110 to 270 us once (directory, drain, fold): made up for after 4 M records.
     // A single call breaks even at 2^17 records once that is spent, at 2^18 where the table is larger than L2.
+    // The records so far are those of earlier calls: a call's own pieces are not counted against it, so that every piece
+    // of a first host call (2^22 records) goes direct where the table stays in L2.  The link takes 290 us for 2^20 records
+    // and hides either route but for the last piece's: counting the pieces takes 25 to 75 us longer at 6 M records, -46
+    // to +6 at 12.6 M, 0 to 23 at 20 M, 2 to 150 at 40 M (4 096 to 2^20 keys, uniform, Zipf, one dominant key).
     const bool small_table = h->L.n_slots * 24 <= L2_TABLE_BYTES;
     const bool few_so_far = !h->hot_ready && h->n_records + n <= (1ull << 22);
     const uint64_t direct_max = h->L.hot_slots == 0 ? DIRECT_RECORDS_MAX : (!few_so_far ? 1ull << 17 : (small_table ? 1ull << 22 : 1ull << 18));

@@ -42,3 +42,23 @@ def test_small_calls_match_the_oracle(n, law):
     assert got.tobytes() == o.finalize(PEAK_BW, PEAK_FLOPS).tobytes()
     st = agg.stats()
     assert st["n_valid"] + st["n_rejected"] == 2 * n and st["n_rejected"] == 2 * int((recs["app_id"] >= 8).sum())
+
+
+def test_a_first_host_call_goes_direct_whatever_its_size():
+    """Into a table that stays in L2, every piece of a host call takes one direct launch (the rule looks at the records of
+    earlier calls); the next device call, with more than 2^22 records before it, takes the two-pass route."""
+    import torch
+    import paper_2607_14541_b200 as p
+    weights = np.arange(1, 9, dtype=np.uint32)
+    n, later = (1 << 22) + 5, 1 << 18
+    recs = trace(n + later, "few", 11)
+    host = torch.from_numpy(recs[:n].view(np.uint8).reshape(-1)).pin_memory()
+    agg = p.Aggregator(weights, 3, 4096)
+    before = agg.launch_count()
+    agg.ingest_host(host, n=n)
+    assert agg.launch_count() - before == 2 and agg.stats()["hot_slots"] == 0
+    agg.ingest(torch.from_numpy(recs[n:].view(np.uint8).reshape(-1)).cuda(), n=later)
+    assert agg.stats()["hot_slots"] > 0
+    o = oracle.Oracle(weights, 3)
+    o.ingest(recs, threads=4)
+    assert sorted_by_key(agg.finalize_numpy(PEAK_BW, PEAK_FLOPS)).tobytes() == o.finalize(PEAK_BW, PEAK_FLOPS).tobytes()
