@@ -443,7 +443,6 @@ static int drain_spill(atrex_agg* h, bool force, cudaStream_t s) {
     q.spill = h->spill;
     q.spill_cnt = h->spill_cnt;
     q.n_groups = h->L.n_groups;
-    q.n_used = h->L.n_groups;
     q.cap = h->L.cap;
     q.queue = h->queue;
     q.queue_cap = h->L.queue_cap;
@@ -526,7 +525,6 @@ static int ingest_launch(atrex_agg* h, const atrex_record_t* recs, uint64_t n, c
     p.app_w = h->d_appw;
     p.hot_keys = h->hot_keys;
     p.hot_slots = h->L.hot_slots;
-    p.hot_buckets = h->L.hot_slots / 4;
     p.hot_img = h->hot_img;
     p.t = h->table_ref();
     p.spill = h->spill;

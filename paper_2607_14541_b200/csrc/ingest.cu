@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(PartitionP
         }
         __syncthreads();
         uint32_t local_total = 0;
-        for (uint32_t g = threadIdx.x; g < q.n_used; g += blockDim.x) local_total += q.spill_cnt[((ull)g << q.t.lp) + part];
+        for (uint32_t g = threadIdx.x; g < q.n_groups; g += blockDim.x) local_total += q.spill_cnt[((ull)g << q.t.lp) + part];
         local_total = __reduce_add_sync(0xFFFFFFFFu, local_total);
         if (lane == 0 && local_total) atomicAdd(&s_total, local_total);
 
@@ -427,14 +427,14 @@ __global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(PartitionP
 
         const uint32_t part_bits = part << (32 - q.t.lp), hmask = 0xFFFFFFFFu >> q.t.lp;
         uint32_t qn_w = 0;  // entries in this warp's queue segment (warp-uniform)
-        for (uint32_t g = warp; g < q.n_used; g += n_warps) {
+        for (uint32_t g = warp; g < q.n_groups; g += n_warps) {
             const ull sb = ((ull)g << q.t.lp) + part;
             const uint32_t n_e = q.spill_cnt[sb];
             const unsigned char* buf = q.spill + sb * q.cap * SPILL_ENTRY_BYTES;
             // Short-distance L2 prefetch, a fixed window of 256 entries per warp (a longer reach gets
             // evicted before use: all warps of all CTAs together must stay well inside L2): the head of
             // this warp's next sub-buffer now, and inside the loop the lines two batches ahead.
-            if (g + n_warps < q.n_used) prefetch_entries(q, ((ull)(g + n_warps) << q.t.lp) + part, lane);
+            if (g + n_warps < q.n_groups) prefetch_entries(q, ((ull)(g + n_warps) << q.t.lp) + part, lane);
             for (uint32_t e0 = 0; e0 < n_e; e0 += 128) {
                 if (lane < 12 && (e0 + 256u) * SPILL_ENTRY_BYTES + lane * 128u < n_e * SPILL_ENTRY_BYTES)
                     prefetch_l2(buf + (e0 + 256u) * SPILL_ENTRY_BYTES + lane * 128u);
@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(PartitionP
             if (next < n_parts) {
                 const unsigned char* nk = reinterpret_cast<const unsigned char*>(q.t.keys + (ull)next * C);
                 for (uint32_t off = threadIdx.x * 128u; off < C * 8u; off += blockDim.x * 128u) prefetch_l2(nk + off);
-                if (warp < q.n_used) prefetch_entries(q, ((ull)warp << q.t.lp) + next, lane);
+                if (warp < q.n_groups) prefetch_entries(q, ((ull)warp << q.t.lp) + next, lane);
             }
         }
         // read-modify-write of the touched slots, four per thread in flight (the loads miss L1 by
@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(PartitionP
             }
         }
         // this partition's buffers are empty again
-        for (uint32_t g = threadIdx.x; g < q.n_used; g += blockDim.x) q.spill_cnt[((ull)g << q.t.lp) + part] = 0;
+        for (uint32_t g = threadIdx.x; g < q.n_groups; g += blockDim.x) q.spill_cnt[((ull)g << q.t.lp) + part] = 0;
         part = next;
     }
     grid_dependents_launch();

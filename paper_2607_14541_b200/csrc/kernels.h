@@ -46,7 +46,6 @@ struct IngestParams {
     const uint32_t* app_w;     // device copy of the card-hour weights
     const ull* hot_keys;       // directory image, hot_slots entries of ~key (0 = empty)
     uint32_t hot_slots;        // multiple of 4
-    uint32_t hot_buckets;      // hot_slots / 4
     uint32_t img_rows;         // rows of hot_img that hold sums since the last fold; a CTA beyond them starts its row afresh
     ulonglong2* hot_img;       // [n_groups][hot_slots] each CTA's directory sums since the last fold, {lo, count | hi << 40}
     TableRef t;
@@ -77,8 +76,7 @@ struct PartitionParams {
     TableRef t;
     const unsigned char* spill;
     uint32_t* spill_cnt;
-    uint32_t n_groups;         // row pitch G
-    uint32_t n_used;           // scatter CTAs whose buffers are read (<= G)
+    uint32_t n_groups;         // scatter CTAs whose buffers are read
     uint32_t cap;
     uint32_t force;            // 1: drain unconditionally; 0: only if the scatter launch `seq` asked for it
     ull seq;
