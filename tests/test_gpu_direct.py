@@ -56,9 +56,9 @@ def test_a_first_host_call_goes_direct_whatever_its_size():
     agg = p.Aggregator(weights, 3, 4096)
     before = agg.launch_count()
     agg.ingest_host(host, n=n)
-    assert agg.launch_count() - before == 2 and agg.stats()["hot_slots"] == 0
+    assert agg.launch_count() - before == 2 and len(agg.hot_directory()) == 0
     agg.ingest(torch.from_numpy(recs[n:].view(np.uint8).reshape(-1)).cuda(), n=later)
-    assert agg.stats()["hot_slots"] > 0
+    assert len(agg.hot_directory()) > 0
     o = oracle.Oracle(weights, 3)
     o.ingest(recs, threads=4)
     assert sorted_by_key(agg.finalize_numpy(PEAK_BW, PEAK_FLOPS)).tobytes() == o.finalize(PEAK_BW, PEAK_FLOPS).tobytes()
