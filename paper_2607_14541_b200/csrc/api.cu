@@ -57,6 +57,7 @@ struct Layout {
     uint32_t n_groups, cap;      // spill buffers: [P][n_groups][cap] entries
     ull sub_launch;              // records per scatter + partition launch pair
     uint32_t hot_slots;
+    ShortFormat fmt;           // short spill entries and directory words
     uint32_t queue_cap;        // deferred entries per CTA in the partition pass
     bool appw_in_smem;
 };
@@ -75,7 +76,9 @@ void compute_layout(const atrex_agg_config_t* c, size_t smem_optin, int n_sms, L
     // tail of its load, not for the mean: with m = max_keys / P keys expected, the keys of one
     // (operator, shape) -- up to n_phases of them -- always fall together, which bounds the standard
     // deviation by sqrt(n_phases * m); six of those plus a constant, and never less than 1.3 m (2 m for small tables).
-    const uint32_t c_max = (uint32_t)((smem_optin - 2048) / 20) & ~127u;
+    L->appw_in_smem = c->n_apps <= APPW_SMEM_MAX;
+    const bool with_weights = L->appw_in_smem && SCATTER_RING_STAGES == 0;   // (the partition pass multiplies short entries)
+    const uint32_t c_max = (uint32_t)((smem_optin - 2048 - (with_weights ? 4 * c->n_apps : 0)) / 20) & ~31u;
     auto slots_for = [&](uint32_t lp) -> ull {
         const ull m = (c->max_keys + (1ull << lp) - 1) >> lp;
         // two slots per key where the smallest number of partitions allows it (probes mostly end at the first
@@ -110,9 +113,26 @@ void compute_layout(const atrex_agg_config_t* c, size_t smem_optin, int n_sms, L
     // work table: same partitions as the key table, 1.5 slots per row plus slack for uneven partitions
     L->Cw = c->max_work_rows ? (uint32_t)((((c->max_work_rows * 3 / 2) >> L->lp) + 64 + 31) / 32 * 32) : 0;
     L->work_slots = (ull)L->Cw << L->lp;
-    L->appw_in_smem = c->n_apps <= APPW_SMEM_MAX;
     L->hot_slots = scatter_hot_slots(L->lp);   // what the scatter pass's shared memory holds for this partition count
     if (c->flags & ATREX_FLAG_NO_HOT_DIRECTORY) L->hot_slots = 0;
+    // Short spill entries: phases and applications take what they need, the operators all that a directory word has left
+    // as long as durations keep 20 bits (2 % of log-normal durations around 50 us are longer and take two entries), and
+    // eight bits in any case; below 16 bits of duration an entry of 12 bytes would be no worse.
+    const auto bits_for = [](uint32_t n) {
+        uint32_t b = 0;
+        while (b < 32 && (1u << b) < n) ++b;
+        return b;
+    };
+    L->fmt = ShortFormat{0, 0, 0, 0};
+    if (with_weights) {
+        const uint32_t phase_bits = bits_for(c->n_phases), app_bits = bits_for(c->n_apps);
+        for (uint32_t op_bits = DIR_ID_BITS - 1 - phase_bits; op_bits >= 8; --op_bits) {
+            const uint32_t low = 63 - (32 - L->lp) - phase_bits - op_bits, dur_bits = (low < 32 ? low : 32) - app_bits;
+            L->fmt = ShortFormat{phase_bits + op_bits, op_bits, app_bits, dur_bits < 31 ? dur_bits : 31};
+            if (dur_bits >= 20) break;
+        }
+        if (L->fmt.dur_bits < 16) L->fmt = ShortFormat{0, 0, 0, 0};
+    }
     size_t o = 0;
     // (control block, spill counts and table are neighbours: a reset clears them in one piece)
     L->off_ctl = o;            o += round_up(sizeof(Control), ALIGN);
@@ -444,6 +464,10 @@ static int drain_spill(atrex_agg* h, bool force, cudaStream_t s) {
     q.spill_cnt = h->spill_cnt;
     q.n_groups = h->L.n_groups;
     q.cap = h->L.cap;
+    q.short_cap = h->L.cap / 2 * 3;
+    q.fmt = h->L.fmt;
+    q.n_apps = h->cfg.n_apps;
+    q.app_w = h->d_appw;
     q.queue = h->queue;
     q.queue_cap = h->L.queue_cap;
     q.force = force ? 1u : 0u;
@@ -492,8 +516,12 @@ static int ingest_launch(atrex_agg* h, const atrex_record_t* recs, uint64_t n, c
         b.n_apps = h->cfg.n_apps;
         b.n_phases = h->cfg.n_phases;
         b.hot_keys = h->hot_keys;
+        b.op_bits = h->L.fmt.dur_bits ? h->L.fmt.op_bits : 0;
         b.hot_slots = h->L.hot_slots;
-        b.dominated_slots = scatter_dominated_slots(h->L.lp);
+        for (int words = 0; words < 2; ++words) {
+            b.slots[words][0] = scatter_slots(h->L.lp, words != 0);
+            b.slots[words][1] = scatter_dominated_slots(h->L.lp, words != 0);
+        }
         b.ctl = h->ctl;
         b.sketch = (uint32_t*)h->hot_scratch;
         b.sample = (ull*)(h->hot_scratch + HOT_SAMPLE_OFF);
@@ -523,6 +551,7 @@ static int ingest_launch(atrex_agg* h, const atrex_record_t* recs, uint64_t n, c
     p.phase_lim = h->cfg.n_phases << 16;
     p.appw_in_smem = h->L.appw_in_smem ? 1u : 0u;
     p.app_w = h->d_appw;
+    p.fmt = h->L.fmt;
     p.hot_keys = h->hot_keys;
     p.hot_slots = h->L.hot_slots;
     p.hot_img = h->hot_img;
@@ -535,6 +564,8 @@ static int ingest_launch(atrex_agg* h, const atrex_record_t* recs, uint64_t n, c
     ull want = (p.n_pairs + pairs_per_cta_iter - 1) / pairs_per_cta_iter;
     int grid = (int)(want < 1 ? 1 : (want > (ull)h->n_sms ? (ull)h->n_sms : want));
     p.drain_above = h->L.cap / 4 * 3;
+    p.short_cap = h->L.cap / 2 * 3;       // (the same bytes)
+    p.short_drain_above = p.short_cap / 4 * 3;
     p.seq = ++h->scatter_seq;
     p.img_rows = h->img_rows;
     CU(h, launch_scatter(p, h->hot_ready, grid, s));
@@ -865,7 +896,7 @@ int atrex_agg_stats(atrex_agg_t* h, atrex_stats_t* out, void* stream) {
     out->n_spilled = c->n_spilled;
     out->n_overflow = c->n_overflow;
     out->max_spill_fill = c->max_fill;
-    out->spill_cap = h->L.cap;
+    out->spill_cap = c->words ? h->L.cap / 2 * 3 : h->L.cap;
     out->n_drains = c->n_drains;
     return device_status_to_error(c);
 }

@@ -13,7 +13,8 @@
 //                 keys and per-launch accumulators fit in one SM's shared memory: the
 //                 aggregation pass owns a partition per CTA and needs no global atomics.
 //   spill bufs  : [G][P][cap] 12-byte entries -- an 8-byte word {weighted duration, operator}
-//                 and a 4-byte word {phase, low hash bits} -- and [G][P] counts,
+//                 and a 4-byte word {phase, low hash bits} -- or [G][P][3/2 cap] short ones of 8 bytes
+//                 (ShortFormat below), and [G][P] counts,
 //                 written by CTA g of the scatter pass (its buffers are contiguous, which keeps
 //                 the scattered appends within a few pages), read by CTA p of the partition pass
 //   work table  : the same P partitions (by the same hash of op_id and shape_id) of Cw 32-byte
@@ -66,6 +67,7 @@ struct Control {
     ull work_status;           // ST_WORK_* bits of the last work-table load
     ull hot_skew;              // SKEW_*: how the scatter pass deals with the most frequent key
     ull prefetch;              // 1: the directory holds enough of the sample for the scatter pass to prefetch records
+    ull words;                 // 1: the directory is in its words form (every operator of the sample fits)
     ull top_key;               // the most frequent key (SKEW_DOMINATED)
     ull n_spilled;             // records routed through the spill buffers
     ull n_overflow;            // records that found their spill buffer full (slow exact path)
@@ -145,6 +147,20 @@ constexpr uint32_t SPILL_ENTRY_BYTES = 12;
 __device__ __forceinline__ ull ckey_of_spill(ull a, uint32_t b, uint32_t part, uint32_t lp) {
     return ckey_of(((b >> 24) << 16) | (uint32_t)(a >> 48), (part << (32 - lp)) | (b & (0xFFFFFFFFu >> lp)));
 }
+
+// A short entry (8 bytes), where phase and operator fit `id_bits` together and the weights the kernels' shared memory:
+// from the top bit on
+//   continuation (1) | phase << op_bits | operator (id_bits) | hash bits below the partition's (32 - lp) | application | duration
+// with the last two, `app_bits` and `dur_bits` wide, at the bottom of the low word (what lies between is zero).  A longer
+// duration's rest follows as a continuation, which adds to the time and not to the count.
+struct ShortFormat {
+    uint32_t id_bits, op_bits, app_bits, dur_bits;   // dur_bits = 0: no short entries
+    __host__ __device__ __forceinline__ uint32_t shift() const { return 1u + id_bits; }
+    __device__ __forceinline__ uint32_t dur_mask() const { return (1u << dur_bits) - 1u; }
+    __device__ __forceinline__ uint32_t app_mask() const { return (1u << app_bits) - 1u; }
+};
+constexpr uint32_t SHORT_ENTRY_BYTES = 8;
+constexpr uint32_t SHORT_CONTINUATION = 0x80000000u;   // in the high word
 
 __device__ __forceinline__ ull pack_key(uint32_t phase, uint32_t op, uint32_t shape) {
     return ((ull)phase << 48) | ((ull)op << 32) | (ull)shape;

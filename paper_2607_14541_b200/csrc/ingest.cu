@@ -5,7 +5,7 @@
 // the L2's atomic rate, not by bandwidth, so the hot path avoids global atomics altogether:
 //
 // Pass 1  SCATTER  (scatter.cu) accumulates the records of hot keys in a shared-memory directory
-//   and appends every other record as a 12-byte entry to the CTA's private buffer of the key's
+//   and appends every other record as an entry of 8 or 12 bytes to the CTA's private buffer of the key's
 //   partition.
 //
 // Pass 2  PARTITION  (persistent CTAs, one partition at a time each).  Runs lazily: only when a
@@ -26,7 +26,6 @@
 namespace atrex {
 
 constexpr int INGEST_THREADS = 1024;
-constexpr uint32_t DIR_WAYS = 4;                   // slots per hot-directory bucket (32 bytes of keys)
 constexpr uint32_t NEW_KEY_FLAG = 0x80000000u;     // partition pass: slot claimed in this launch
 
 __device__ __forceinline__ uint32_t dir_bucket_of_key(ull key, uint32_t mult, uint32_t n_buckets) {
@@ -67,10 +66,10 @@ __device__ __forceinline__ ull atoms_cas64(uint32_t a, ull expected, ull desired
 // Shared-memory accumulation uses native 32-bit atomics only (64-bit shared atomics are
 // compare-and-swap loops).  A slot's weighted time is kept in two limbs: the returning add on
 // the low limb tells the adder whether it wrapped, and the adder then adds the carry, with the
-// value's high word, to the high limb (part_accumulate).  One add raises the high limb by at most 2^21 (a warp's
-// combined 32 records of < 2^48 each), so the adder that takes it across 2^30 drains both
-// limbs; the adds that can slip in before its exchange (one per thread of the CTA) stay below
-// 2^31, so the high limb never wraps.
+// value's high word, to the high limb (part_accumulate).  One add raises the high limb by at most 2^16, or 2^23 for a
+// warp's combined 128 entries of < 2^48 each, so the adder that takes it across 2^30 drains both
+// limbs; the adds that can slip in before its exchange (one per thread of the CTA, at most one of them
+// per warp combined) stay below 2^31, so the high limb never wraps.
 constexpr uint32_t DRAIN_BIT = 0x40000000u;
 
 __device__ __forceinline__ ull limbs_drain(uint32_t a0, uint32_t a1, ull* hi_out) {
@@ -148,8 +147,14 @@ __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefe
 // empty), acc {u32 low limb, u32 count | NEW_KEY_FLAG}[C], a1 u32[C] (high limb).
 struct PartSmem {
     uint32_t keys, acc, a1;
+    uint32_t weights;          // short entries: u32[n_apps]
 };
 
+__device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
+    uint32_t v;
+    asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
 __device__ __forceinline__ uint4 lds_v4u32(uint32_t a) {
     uint4 v;
     asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a));
@@ -161,7 +166,7 @@ __device__ __forceinline__ uint4 lds_v4u32(uint32_t a) {
 // the key's slot, or PROBE_FAILED when the partition has no room.
 constexpr uint32_t PROBE_FAILED = 0xFFFFFFFFu;
 
-__device__ __forceinline__ uint32_t probe_general(const PartSmem& m, ull skey, uint32_t slot, uint32_t advance, bool busy,
+__device__ __forceinline__ uint32_t probe_general(const PartSmem& m, ull skey, uint32_t slot, uint32_t advance, bool busy, uint32_t count,
                                                   uint32_t C, Control* ctl) {
     uint32_t steps = 0;
     while (__any_sync(0xFFFFFFFFu, busy)) {
@@ -188,7 +193,7 @@ __device__ __forceinline__ uint32_t probe_general(const PartSmem& m, ull skey, u
                 busy = false;
                 slot = PROBE_FAILED;
                 atomicOr(&ctl->status, ST_TABLE_FULL);
-                atomicAdd(&ctl->n_dropped, 1ull);
+                atomicAdd(&ctl->n_dropped, (ull)count);
             }
         }
     }
@@ -205,14 +210,14 @@ __device__ __noinline__ void part_drain_slot(uint32_t acc, uint32_t a1, ulonglon
     if (hi) atomicAdd(vp + 1, hi << HI_SHIFT);
 }
 
-// One entry's product (vlo + 2^32 vhi, vhi < 2^16) and count into its slot's limbs: a returning add on
+// One entry's product (vlo + 2^32 vhi, vhi < 2^16; combined entries: 2^23) and count (0: a continuation) into its slot's limbs: a returning add on
 // the low limb, whose wrap is the carry; the high limb is touched only when there is something to add.
-__device__ __forceinline__ void part_accumulate(const PartSmem& m, uint32_t slot, uint32_t vlo, uint32_t vhi,
+__device__ __forceinline__ void part_accumulate(const PartSmem& m, uint32_t slot, uint32_t vlo, uint32_t vhi, uint32_t count,
                                                 ulonglong2* vals_of_partition, uint32_t C, Control* ctl) {
     slot = ATREX_INDEX(slot, C, ctl);
     const uint32_t acc = m.acc + slot * 8;
     const uint32_t o0 = atoms_add(acc, vlo);
-    reds_add(acc + 4, 1u);
+    reds_add(acc + 4, count);
     const uint32_t x = vhi + ((o0 + vlo < o0) ? 1u : 0u);
     if (x != 0) {
         const uint32_t o1 = atoms_add(m.a1 + slot * 4, x);
@@ -220,10 +225,18 @@ __device__ __forceinline__ void part_accumulate(const PartSmem& m, uint32_t slot
     }
 }
 
-// The first 256 entries (24 lines) of sub-buffer `sb` towards L2, as far as it holds that many.
+// Where the entries are: their size, their buffers' pitch.
+__device__ __forceinline__ const unsigned char* entries_of(const PartitionParams& q, ull sb) {
+    return q.spill + sb * q.cap * SPILL_ENTRY_BYTES;     // (a buffer of short entries takes as many bytes)
+}
+template <bool SHORT>
+constexpr uint32_t ENTRY_BYTES = SHORT ? SHORT_ENTRY_BYTES : SPILL_ENTRY_BYTES;
+
+// The first 256 entries (24 or 16 lines) of sub-buffer `sb` towards L2, as far as it holds that many.
+template <bool SHORT>
 __device__ __forceinline__ void prefetch_entries(const PartitionParams& q, ull sb, uint32_t lane) {
-    const uint32_t bytes = q.spill_cnt[sb] * SPILL_ENTRY_BYTES;
-    if (lane < 24 && lane * 128u < bytes) prefetch_l2(q.spill + sb * q.cap * SPILL_ENTRY_BYTES + lane * 128u);
+    const uint32_t bytes = q.spill_cnt[sb] * ENTRY_BYTES<SHORT>;
+    if (lane < 2u * ENTRY_BYTES<SHORT> && lane * 128u < bytes) prefetch_l2(entries_of(q, sb) + lane * 128u);
 }
 
 // Settles a warp's queued entries, one per lane and round, by the general probe.  Other warps may
@@ -234,21 +247,48 @@ __device__ __noinline__ void settle_queue(const TableRef t, const PartSmem m, co
                                           ull base, uint32_t lane);
 
 // A queued entry: {key, product}; bit 63 of the product word says that the key's first pair was full
-// of other keys when the entry was looked up, so its probe may start at the second pair.
-constexpr ull QUEUED_SKIP_FIRST = 1ull << 63;
+// of other keys when the entry was looked up, so its probe may start at the second pair; bit 62 that it is a continuation.
+constexpr ull QUEUED_SKIP_FIRST = 1ull << 63, QUEUED_CONTINUATION = 1ull << 62;
 
-// One batch of 128 entries of a sub-buffer, four consecutive ones (48 bytes) per lane.  FULL: the
+// One batch of 128 entries of a sub-buffer, four consecutive ones (48 bytes; 32 if short) per lane.  FULL: the
 // batch is complete (no masks).  Keys are handled as their two 32-bit halves (kh: mark, phase,
 // operator; kl: hash).  Entry state is bit sets per lane -- `open` (present, slot not known yet), `hit`
 // (slot known), `room` (the first pair of the probe sequence had a free slot when it was read).
 // part_bits = the partition's index in the hash's top bits, hmask = the hash bits below them.
-template <bool FULL>
+template <bool SHORT, bool CROWDED, bool FULL>
 __device__ __forceinline__ void stream_batch(const PartitionParams& q, const PartSmem& m, const unsigned char* src,
                                              uint32_t part_bits, uint32_t hmask, uint32_t e0, uint32_t n_e, uint32_t C, ull base,
                                              ulonglong2* my_queue, uint32_t queue_cap_w, uint32_t& qn_w, uint32_t lane) {
     uint32_t kh[4], kl[4], vlo[4], vhi[4], slot[4];
-    uint32_t open = 0;
-    {
+    uint32_t open = 0, extra = 0;    // extra: continuations
+    if (SHORT) {
+        const uint32_t e = e0 + 4u * lane;
+        uint32_t w[8];
+        if (FULL || e < n_e) {       // (a buffer's capacity is a multiple of 16: a lane that holds any entry may read all 32 bytes)
+            asm volatile("ld.global.L1::no_allocate.L2::evict_first.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                         : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
+                         : "l"(src + (size_t)e * SHORT_ENTRY_BYTES));
+            open = FULL ? 0xFu : (0xFu >> (4u - min(n_e - e, 4u)));
+        } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) w[j] = 0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t lo = w[2 * u], hi = w[2 * u + 1];
+            const uint32_t id = (hi & ~SHORT_CONTINUATION) >> (31u - q.fmt.id_bits), phase = id >> q.fmt.op_bits;
+            kh[u] = (0x80000000u | id) + phase * (0x10000u - (1u << q.fmt.op_bits));    // phase << 16 | operator
+            kl[u] = part_bits | (__funnelshift_l(lo, hi, 1u + q.fmt.id_bits) >> q.t.lp);
+            const uint32_t more = hi >> 31;
+            const uint32_t dur = (lo & q.fmt.dur_mask()) << (more ? q.fmt.dur_bits : 0u);
+            const uint32_t app = ATREX_INDEX((lo >> q.fmt.dur_bits) & q.fmt.app_mask(), q.n_apps, q.t.ctl);
+            const ull v = (ull)lds_u32(m.weights + app * 4u) * dur;
+            extra |= more << u;
+            vlo[u] = (uint32_t)v;
+            vhi[u] = (uint32_t)(v >> 32);
+            slot[u] = local_of(kl[u], phase, C) & ~1u;
+        }
+    } else {
         // the lane's entries e, e + 1, e + 2, e + 3 (e a multiple of 4) as twelve words; in an even
         // entry the 8-byte word comes first, in an odd one last.  A buffer's capacity is a multiple
         // of 4, so a lane that holds any entry may read all 48 bytes.
@@ -324,14 +364,37 @@ __device__ __forceinline__ void stream_batch(const PartitionParams& q, const Par
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             if (open & (1u << u)) {
-                const ull v = vlo[u] | ((ull)vhi[u] << 32) | ((room >> u) & 1u ? 0ull : QUEUED_SKIP_FIRST);
+                const ull v = vlo[u] | ((ull)vhi[u] << 32) | ((room >> u) & 1u ? 0ull : QUEUED_SKIP_FIRST) |
+                              (SHORT && ((extra >> u) & 1u) ? QUEUED_CONTINUATION : 0ull);
                 my_queue[ATREX_INDEX(qbase + before[u], queue_cap_w, q.t.ctl)] = make_ulonglong2(((ull)kh[u] << 32) | kl[u], v);
             }
         }
     }
+    // (a crowded partition: where a quarter of the lanes' first entries share a slot, the batch's entries of that slot are
+    // summed first)
+    for (int turn = 0; CROWDED && turn < 4; ++turn) {
+        const uint32_t hits = __ballot_sync(0xFFFFFFFFu, hit & 1u);
+        if (hits == 0) break;
+        const int lead = __ffs(hits) - 1;
+        const uint32_t shared_slot = __shfl_sync(0xFFFFFFFFu, slot[0], lead);
+        if (__popc(__ballot_sync(0xFFFFFFFFu, (hit & 1u) != 0 && slot[0] == shared_slot)) < 8) break;
+        ull sum = 0;         // < 2^50
+        uint32_t count = 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if ((hit & (1u << u)) != 0 && slot[u] == shared_slot) {
+                sum += (ull)vlo[u] | ((ull)vhi[u] << 32);
+                count += SHORT ? ~(extra >> u) & 1u : 1u;
+                hit &= ~(1u << u);
+            }
+        }
+        const ull all = (ull)__reduce_add_sync(0xFFFFFFFFu, (uint32_t)sum & 0x1FFFFFFu) + ((ull)__reduce_add_sync(0xFFFFFFFFu, (uint32_t)(sum >> 25)) << 25);
+        count = __reduce_add_sync(0xFFFFFFFFu, count);
+        if (lane == (uint32_t)lead) part_accumulate(m, shared_slot, (uint32_t)all, (uint32_t)(all >> 32), count, q.t.vals + base, C, q.t.ctl);
+    }
 #pragma unroll
     for (int u = 0; u < 4; ++u)
-        if (hit & (1u << u)) part_accumulate(m, slot[u], vlo[u], vhi[u], q.t.vals + base, C, q.t.ctl);
+        if (hit & (1u << u)) part_accumulate(m, slot[u], vlo[u], vhi[u], SHORT ? ~(extra >> u) & 1u : 1u, q.t.vals + base, C, q.t.ctl);
 }
 
 __device__ __noinline__ void settle_queue(const TableRef t, const PartSmem m, const ulonglong2* my_queue, uint32_t qn_w, uint32_t C,
@@ -347,15 +410,61 @@ __device__ __noinline__ void settle_queue(const TableRef t, const PartSmem m, co
             start += advance;
             if (start >= C) start -= C;
         }
-        const uint32_t found = probe_general(m, ent.x, start, advance, serving, C, t.ctl);
+        const uint32_t count = ent.y & QUEUED_CONTINUATION ? 0u : 1u;
+        const uint32_t found = probe_general(m, ent.x, start, advance, serving, count, C, t.ctl);
         if (serving && found != PROBE_FAILED)
-            part_accumulate(m, found, (uint32_t)ent.y, (uint32_t)(ent.y >> 32) & 0xFFFFu, t.vals + base, C, t.ctl);
+            part_accumulate(m, found, (uint32_t)ent.y, (uint32_t)(ent.y >> 32) & 0xFFFFu, count, t.vals + base, C, t.ctl);
     }
     __syncwarp();   // the queue may be overwritten from here on
 }
 
-__global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(PartitionParams q) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+// A warp's share of a partition's entries: sub-buffers warp, warp + n_warps, ...  Returns how many wait in its queue.
+template <bool SHORT, bool CROWDED>
+__device__ __forceinline__ uint32_t stream_share(const PartitionParams& q, const PartSmem& m, uint32_t part, ulonglong2* my_queue, uint32_t queue_cap_w,
+                                                 uint32_t warp, uint32_t n_warps, uint32_t lane) {
+    const uint32_t C = q.t.C;
+    const ull base = (ull)part * C;
+    const uint32_t part_bits = part << (32 - q.t.lp), hmask = 0xFFFFFFFFu >> q.t.lp;
+    uint32_t qn_w = 0;  // entries in this warp's queue segment (warp-uniform)
+    for (uint32_t g = warp; g < q.n_groups; g += n_warps) {
+        const ull sb = ((ull)g << q.t.lp) + part;
+        const uint32_t n_e = q.spill_cnt[sb];
+        const unsigned char* buf = entries_of(q, sb);
+        // Short-distance L2 prefetch, a fixed window of 256 entries per warp (a longer reach gets
+        // evicted before use: all warps of all CTAs together must stay well inside L2): the head of
+        // this warp's next sub-buffer now, and inside the loop the lines two batches ahead.
+        if (g + n_warps < q.n_groups) prefetch_entries<SHORT>(q, ((ull)(g + n_warps) << q.t.lp) + part, lane);
+        for (uint32_t e0 = 0; e0 < n_e; e0 += 128) {
+            if (lane < ENTRY_BYTES<SHORT> && (e0 + 256u) * ENTRY_BYTES<SHORT> + lane * 128u < n_e * ENTRY_BYTES<SHORT>)
+                prefetch_l2(buf + (e0 + 256u) * ENTRY_BYTES<SHORT> + lane * 128u);
+            if (qn_w + 128u > queue_cap_w) {   // (warp-uniform) the next batch might not fit the queue
+                settle_queue(q.t, m, my_queue, qn_w, C, base, lane);
+                qn_w = 0;
+            }
+            if (e0 + 128u <= n_e)
+                stream_batch<SHORT, CROWDED, true>(q, m, buf, part_bits, hmask, e0, n_e, C, base, my_queue, queue_cap_w, qn_w, lane);
+            else
+                stream_batch<SHORT, CROWDED, false>(q, m, buf, part_bits, hmask, e0, n_e, C, base, my_queue, queue_cap_w, qn_w, lane);
+        }
+    }
+    return qn_w;
+}
+
+// A frequent key that found no place in the scatter pass's directory fills its partition, and the lanes queue at its
+// limbs.  Whether a quarter of a partition's entries are alike shows in the first ones of a warp's share (2^27 records over
+// 1 024 keys, 4 of them in such partitions: drain 240 -> 55 us).
+__device__ __forceinline__ bool looks_crowded(const PartitionParams& q, uint32_t part, uint32_t warp, uint32_t lane) {
+    if (warp >= q.n_groups) return false;
+    const ull sb = ((ull)warp << q.t.lp) + part;
+    const uint32_t n = q.spill_cnt[sb];
+    const uint32_t hi = lane < n ? *reinterpret_cast<const uint32_t*>(entries_of(q, sb) + lane * SHORT_ENTRY_BYTES + 4) & ~SHORT_CONTINUATION : ~lane;
+    const uint32_t common = __shfl_sync(0xFFFFFFFFu, hi, 0), other = __shfl_sync(0xFFFFFFFFu, hi, 1);
+    return __popc(__ballot_sync(0xFFFFFFFFu, hi == common)) >= 8 || __popc(__ballot_sync(0xFFFFFFFFu, hi == other)) >= 8;
+}
+
+// What a CTA of the partition pass does, for either kind of entries.
+template <bool SHORT>
+__device__ __forceinline__ void partition_cta(const PartitionParams& q, unsigned char* smem_raw) {
     const uint32_t C = q.t.C;
     ull* s_keys = reinterpret_cast<ull*>(smem_raw);
     uint2* s_acc = reinterpret_cast<uint2*>(s_keys + C);      // {low limb, count | NEW_KEY_FLAG}
@@ -364,6 +473,7 @@ __global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(PartitionP
     m.keys = smem_addr(s_keys);
     m.acc = smem_addr(s_acc);
     m.a1 = smem_addr(s_a1);
+    m.weights = smem_addr(s_a1 + C);
     __shared__ uint32_t s_total;
     // each warp owns a segment of the CTA's queue: no shared counter, and a warp can settle its own
     // leftovers as soon as its share of the stream is through
@@ -371,12 +481,8 @@ __global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(PartitionP
     ulonglong2* const my_queue = q.queue + (size_t)blockIdx.x * q.queue_cap + (size_t)(threadIdx.x >> 5) * queue_cap_w;
     const uint32_t n_parts = 1u << q.t.lp;
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u, n_warps = blockDim.x >> 5;
-    grid_dependency_wait();
-    // the spill buffers are drained lazily: unless forced, only when the scatter launch just
-    // before this one found a buffer filling up
-    if (!q.force && ld_relaxed(&q.t.ctl->drain_seq) != q.seq) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&q.t.ctl->n_drains, 1ull);
-
+    if (SHORT)
+        for (uint32_t i = threadIdx.x; i < q.n_apps; i += blockDim.x) (s_a1 + C)[i] = q.app_w[i];
     // Partitions are handed out by a counter (their entry counts differ by a few per cent, and a static
     // split leaves the kernel waiting for its slowest CTA); a CTA always holds its next partition as
     // well, so that it can pull that one's keys and entries towards L2 early.
@@ -425,29 +531,8 @@ __global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(PartitionP
         }
         __syncthreads();
 
-        const uint32_t part_bits = part << (32 - q.t.lp), hmask = 0xFFFFFFFFu >> q.t.lp;
-        uint32_t qn_w = 0;  // entries in this warp's queue segment (warp-uniform)
-        for (uint32_t g = warp; g < q.n_groups; g += n_warps) {
-            const ull sb = ((ull)g << q.t.lp) + part;
-            const uint32_t n_e = q.spill_cnt[sb];
-            const unsigned char* buf = q.spill + sb * q.cap * SPILL_ENTRY_BYTES;
-            // Short-distance L2 prefetch, a fixed window of 256 entries per warp (a longer reach gets
-            // evicted before use: all warps of all CTAs together must stay well inside L2): the head of
-            // this warp's next sub-buffer now, and inside the loop the lines two batches ahead.
-            if (g + n_warps < q.n_groups) prefetch_entries(q, ((ull)(g + n_warps) << q.t.lp) + part, lane);
-            for (uint32_t e0 = 0; e0 < n_e; e0 += 128) {
-                if (lane < 12 && (e0 + 256u) * SPILL_ENTRY_BYTES + lane * 128u < n_e * SPILL_ENTRY_BYTES)
-                    prefetch_l2(buf + (e0 + 256u) * SPILL_ENTRY_BYTES + lane * 128u);
-                if (qn_w + 128u > queue_cap_w) {   // (warp-uniform) the next batch might not fit the queue
-                    settle_queue(q.t, m, my_queue, qn_w, C, base, lane);
-                    qn_w = 0;
-                }
-                if (e0 + 128u <= n_e)
-                    stream_batch<true>(q, m, buf, part_bits, hmask, e0, n_e, C, base, my_queue, queue_cap_w, qn_w, lane);
-                else
-                    stream_batch<false>(q, m, buf, part_bits, hmask, e0, n_e, C, base, my_queue, queue_cap_w, qn_w, lane);
-            }
-        }
+        const uint32_t qn_w = SHORT && looks_crowded(q, part, warp, lane) ? stream_share<SHORT, true>(q, m, part, my_queue, queue_cap_w, warp, n_warps, lane)
+                                                                          : stream_share<SHORT, false>(q, m, part, my_queue, queue_cap_w, warp, n_warps, lane);
         settle_queue(q.t, m, my_queue, qn_w, C, base, lane);
         __syncthreads();
         {   // while the deltas are written back, pull the next partition's keys and each warp's
@@ -455,7 +540,7 @@ __global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(PartitionP
             if (next < n_parts) {
                 const unsigned char* nk = reinterpret_cast<const unsigned char*>(q.t.keys + (ull)next * C);
                 for (uint32_t off = threadIdx.x * 128u; off < C * 8u; off += blockDim.x * 128u) prefetch_l2(nk + off);
-                if (warp < q.n_groups) prefetch_entries(q, ((ull)warp << q.t.lp) + next, lane);
+                if (warp < q.n_groups) prefetch_entries<SHORT>(q, ((ull)warp << q.t.lp) + next, lane);
             }
         }
         // read-modify-write of the touched slots, four per thread in flight (the loads miss L1 by
@@ -490,6 +575,19 @@ __global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(PartitionP
         for (uint32_t g = threadIdx.x; g < q.n_groups; g += blockDim.x) q.spill_cnt[((ull)g << q.t.lp) + part] = 0;
         part = next;
     }
+}
+
+__global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(PartitionParams q) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    grid_dependency_wait();
+    // the spill buffers are drained lazily: unless forced, only when the scatter launch just
+    // before this one found a buffer filling up
+    if (!q.force && ld_relaxed(&q.t.ctl->drain_seq) != q.seq) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&q.t.ctl->n_drains, 1ull);
+    if (q.t.ctl->words != 0)
+        partition_cta<true>(q, smem_raw);
+    else
+        partition_cta<false>(q, smem_raw);
     grid_dependents_launch();
     // the last CTA rewinds the hand-out counter for the next launch
     if (threadIdx.x == 0) {
@@ -510,8 +608,8 @@ __global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(PartitionP
 //              into a candidate table (colliding cold keys may slip in; harmless);
 //   3. level   how many candidates have which count, and from that the count that fills the directory;
 //   4. gather  the candidates above it side by side, and how much weight each of four bucket hashes would lose;
-//   5. list    the candidates of each 4-slot bucket under the best of them;
-//   6. pick    each bucket takes its four most frequent ones.
+//   5. list    the candidates of each bucket (two slots or four, see scatter.cu) under the best of them;
+//   6. pick    each bucket takes its most frequent ones.
 // Which keys end up in the directory only affects speed, never results.  Bound by latency and launches: 90 us for
 // 2^20 samples; 187 us when single records were read (twice) and one CTA did steps 3 to 6.
 constexpr uint32_t SKETCH_BITS = 20;   // as many counters as samples, so that cold keys stay below ADMIT_MIN
@@ -563,6 +661,7 @@ __global__ void __launch_bounds__(256) hot_count_kernel(HotBuildParams p) {
     grid_dependency_wait();
     const uint32_t stride = gridDim.x * blockDim.x;
     const uint32_t rounds = (p.n_sample + stride * SAMPLE_ILP - 1) / (stride * SAMPLE_ILP);  // uniform trip count: warp collectives inside
+    uint32_t max_op = 0;
     for (uint32_t r = 0; r < rounds; ++r) {
         uint4 v[SAMPLE_ILP];
 #pragma unroll
@@ -576,9 +675,12 @@ __global__ void __launch_bounds__(256) hot_count_kernel(HotBuildParams p) {
             const uint32_t khi = v[u].y & 0x00FFFFFFu;
             const bool ok = j < p.n_sample && v[u].x < p.n_apps && (khi >> 16) < p.n_phases;
             if (j < p.n_sample) p.sample[j] = ok ? ((ull)khi << 32) | v[u].z : ~0ull;
+            if (ok) max_op = max(max_op, khi & 0xFFFFu);
             cache.add(p.sketch, hash32(khi & 0xFFFFu, v[u].z) >> (32 - SKETCH_BITS), ok);
         }
     }
+    max_op = __reduce_max_sync(0xFFFFFFFFu, max_op);
+    if ((threadIdx.x & 31u) == 0 && max_op >> p.op_bits) atomicMax(&p.scratch->max_op, max_op);   // (only what does not fit is told)
     grid_dependents_launch();
     cache.flush(p.sketch);
 }
@@ -624,6 +726,10 @@ __global__ void __launch_bounds__(256) hot_admit_kernel(HotBuildParams p) {
     cache.flush(p.cand_cnt);
 }
 
+// The words form's two-way buckets lose 5 % of 4 096 equally frequent keys, the tags form's four-way ones 2.4 %: there the
+// tags hold more (2^27 records 835 us either way).  Below, neither loses much and words are faster (2 048 keys: 734
+// against 802 us); above, words hold as many or more (12 288 keys: 1 052 against 1 082; 32 768: 1 378 against 1 808).
+constexpr uint32_t TAGS_FROM = 3000, TAGS_TO = 5000;
 constexpr uint32_t LIST_MAX = 16;       // candidates a bucket chooses from (five on average)
 constexpr uint32_t LEVEL_THREADS = 1024;
 
@@ -660,12 +766,13 @@ __global__ void __launch_bounds__(LEVEL_THREADS) hot_level_kernel(HotBuildParams
     }
     __syncthreads();
     if (!s_last) return;
-    // smallest threshold >= 2 whose class fits the directory with some over-subscription: thread t looks at the
-    // count 1023 - t, behind a scan over the higher ones
+    // smallest threshold >= 2 whose class fits the directory with some over-subscription (a bucket of two ways fills
+    // less evenly than one of four): thread t looks at the count 1023 - t, behind a scan over the higher ones
     const ull most_seen = __ldcg(&x.most);
     const ull skew = most_seen * 8u >= p.n_sample * 3ull ? SKEW_DOMINATED : (most_seen * 32u >= p.n_sample ? SKEW_COMBINE : SKEW_NONE);
-    const uint32_t slots = skew == SKEW_DOMINATED ? p.dominated_slots : p.hot_slots;
-    const uint32_t budget = min(slots + slots / 4, HOT_SELECT_MAX);
+    const bool words = p.op_bits != 0 && __ldcg(&x.max_op) == 0;
+    const uint32_t slots = p.slots[words][skew == SKEW_DOMINATED];
+    const uint32_t budget = min(words ? 2 * slots : slots + slots / 4, HOT_SELECT_MAX);
     uint32_t incl = __ldcg(&x.hist[1023 - t]);
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -686,14 +793,21 @@ __global__ void __launch_bounds__(LEVEL_THREADS) hot_level_kernel(HotBuildParams
     __syncthreads();
     incl += w ? s_warp[w - 1] : 0u;
     const int above = __syncthreads_count(t <= 1021 && incl <= budget);   // counts 1023, 1022, ... that fit
-    if (t == 0) {
+    if (above == 0 ? t == 0 : t == (uint32_t)above - 1u) {
+        const uint32_t selected = above ? incl : 0u;
         x.threshold = 1024u - (uint32_t)above;
         p.ctl->hot_skew = skew;
+        p.ctl->words = words && !(selected > TAGS_FROM && selected <= TAGS_TO) ? 1 : 0;
     }
 }
 
-__device__ __forceinline__ uint32_t buckets_in_use(const HotBuildParams& p) {
-    return (p.ctl->hot_skew == SKEW_DOMINATED ? p.dominated_slots : p.hot_slots) / DIR_WAYS;
+struct Buckets {
+    uint32_t n, ways;
+};
+__device__ __forceinline__ Buckets buckets_in_use(const HotBuildParams& p) {
+    const bool words = p.ctl->words != 0;
+    const uint32_t ways = words ? WORD_WAYS : TAG_WAYS;
+    return {p.slots[words][p.ctl->hot_skew == SKEW_DOMINATED] / ways, ways};
 }
 
 // A multiplier's loss is approximated by arrival order among the keys that matter.
@@ -703,7 +817,8 @@ __global__ void __launch_bounds__(256) hot_gather_kernel(HotBuildParams p) {
     __syncthreads();
     grid_dependency_wait();
     HotBuildScratch& x = *p.scratch;
-    const uint32_t thr = x.threshold, n_buckets = buckets_in_use(p), lane = threadIdx.x & 31u;
+    const Buckets buckets = buckets_in_use(p);
+    const uint32_t thr = x.threshold, lane = threadIdx.x & 31u;
     const uint32_t i = blockIdx.x * 256 + threadIdx.x;      // (grid: one thread per candidate)
     const uint32_t c = p.cand_cnt[i];
     const uint32_t votes = __ballot_sync(0xFFFFFFFFu, c >= thr);
@@ -721,7 +836,7 @@ __global__ void __launch_bounds__(256) hot_gather_kernel(HotBuildParams p) {
         if (c >= 16) {
 #pragma unroll
             for (uint32_t m = 0; m < 4; ++m)
-                if (atomicAdd(&x.occupancy[m][dir_bucket_of_key(~skey, DIR_MULTS[m], n_buckets)], 1u) >= DIR_WAYS) atomicAdd(&s_lost[m], c);
+                if (atomicAdd(&x.occupancy[m][dir_bucket_of_key(~skey, DIR_MULTS[m], buckets.n)], 1u) >= buckets.ways) atomicAdd(&s_lost[m], c);
         }
     }
     grid_dependents_launch();
@@ -742,7 +857,7 @@ __global__ void __launch_bounds__(256) hot_list_kernel(HotBuildParams p) {
     HotBuildScratch& x = *p.scratch;
     const uint32_t i = blockIdx.x * 256 + threadIdx.x;
     if (i < min(x.n, HOT_SELECT_MAX)) {
-        const uint32_t b = dir_bucket_of_key(~x.key[i], best_multiplier(x), buckets_in_use(p));
+        const uint32_t b = dir_bucket_of_key(~x.key[i], best_multiplier(x), buckets_in_use(p).n);
         const uint32_t at = atomicAdd(&x.listed[b], 1u);
         if (at < LIST_MAX) x.list[b][at] = i;
     }
@@ -755,15 +870,15 @@ __global__ void __launch_bounds__(128) hot_pick_kernel(HotBuildParams p) {
     __syncthreads();
     grid_dependency_wait();
     HotBuildScratch& x = *p.scratch;
-    const uint32_t b = blockIdx.x * 128 + threadIdx.x;
+    const uint32_t b = blockIdx.x * 128 + threadIdx.x, ways = buckets_in_use(p).ways;
     uint32_t inserted = 0, weight = 0;
-    if (b < p.hot_slots / DIR_WAYS) {
+    if (b < p.hot_slots / ways) {        // (the whole image: buckets that are not in use have nothing listed)
         const uint32_t n = min(x.listed[b], LIST_MAX);
-        uint32_t top[DIR_WAYS] = {0, 0, 0, 0}, who[DIR_WAYS] = {0, 0, 0, 0};
+        uint32_t top[TAG_WAYS] = {0, 0, 0, 0}, who[TAG_WAYS] = {0, 0, 0, 0};
         for (uint32_t k = 0; k < n; ++k) {
             uint32_t i = x.list[b][k], c = x.count[i];
 #pragma unroll
-            for (uint32_t way = 0; way < DIR_WAYS; ++way) {   // insertion into the four best
+            for (uint32_t way = 0; way < TAG_WAYS; ++way) {   // insertion into the four best
                 if (c > top[way]) {
                     const uint32_t tc = top[way], ti = who[way];
                     top[way] = c;
@@ -773,16 +888,17 @@ __global__ void __launch_bounds__(128) hot_pick_kernel(HotBuildParams p) {
                 }
             }
         }
-        ull keys[DIR_WAYS];
+        ull keys[TAG_WAYS];
 #pragma unroll
-        for (uint32_t way = 0; way < DIR_WAYS; ++way) {
-            keys[way] = top[way] ? x.key[who[way]] : 0ull;
-            inserted += top[way] ? 1u : 0u;
-            weight += top[way];
+        for (uint32_t way = 0; way < TAG_WAYS; ++way) {
+            const bool taken = way < ways && top[way] != 0;
+            keys[way] = taken ? x.key[who[way]] : 0ull;
+            inserted += taken ? 1u : 0u;
+            weight += taken ? top[way] : 0u;
         }
-        ulonglong2* dst = reinterpret_cast<ulonglong2*>(p.hot_keys + b * DIR_WAYS);
+        ulonglong2* dst = reinterpret_cast<ulonglong2*>(p.hot_keys + b * ways);
         dst[0] = make_ulonglong2(keys[0], keys[1]);
-        dst[1] = make_ulonglong2(keys[2], keys[3]);
+        if (ways == TAG_WAYS) dst[1] = make_ulonglong2(keys[2], keys[3]);
         if (b == 0) p.ctl->dir_mult = best_multiplier(x);
     }
     inserted = __reduce_add_sync(0xFFFFFFFFu, inserted);
@@ -824,7 +940,7 @@ cudaError_t ingest_prepare() {
 
 cudaError_t launch_partition(const PartitionParams& q, int n_sms, cudaStream_t stream) {
     int grid = (int)(1u << q.t.lp) < n_sms ? (int)(1u << q.t.lp) : n_sms;
-    return launch_chained(partition_kernel, (uint32_t)grid, INGEST_THREADS, (size_t)q.t.C * 20, stream, q);
+    return launch_chained(partition_kernel, (uint32_t)grid, INGEST_THREADS, partition_smem_bytes(q.t.C, q.n_apps, q.fmt.dur_bits != 0), stream, q);
 }
 
 cudaError_t launch_hot_build(const HotBuildParams& p, int n_sms, cudaStream_t stream) {
@@ -834,7 +950,7 @@ cudaError_t launch_hot_build(const HotBuildParams& p, int n_sms, cudaStream_t st
     hot_count_kernel<<<grid, 256, 0, stream>>>(p);
     hot_admit_kernel<<<grid, 256, 0, stream>>>(p);
     cudaError_t e = cudaGetLastError();
-    const uint32_t n_cand = 1u << p.cand_bits, n_buckets = p.hot_slots / DIR_WAYS;
+    const uint32_t n_cand = 1u << p.cand_bits, n_buckets = p.hot_slots / WORD_WAYS;
     if (e == cudaSuccess) e = launch_chained(hot_level_kernel, n_cand / LEVEL_THREADS, LEVEL_THREADS, 0, stream, p);
     if (e == cudaSuccess) e = launch_chained(hot_gather_kernel, n_cand / 256, 256, 0, stream, p);
     if (e == cudaSuccess) e = launch_chained(hot_list_kernel, (HOT_SELECT_MAX + 255) / 256, 256, 0, stream, p);

@@ -16,8 +16,9 @@ namespace atrex {
 
 // Shared memory of the scatter pass (dynamic, one CTA per SM) and what fits in it.  Per partition a
 // cursor word, 16 KB of card-hour weights, the record ring if there
-// is one, then the hot directory: a tag byte, an 8-byte key and 12 bytes of accumulators per slot, in
-// whole 4-way buckets.
+// is one, then the hot directory, in one of two forms (scatter.cu says which and why):
+//   words  a 32-bit word that identifies the key inside its bucket and 12 bytes of accumulators per slot, 2-way buckets
+//   tags   a tag byte, an 8-byte key and 12 bytes of accumulators per slot, 4-way buckets
 constexpr uint32_t APPW_SMEM_MAX = 4096;
 constexpr uint32_t SCATTER_SMEM_BYTES = 232448 - 1024;
 constexpr uint32_t SCATTER_RING_STAGES = ATREX_SCATTER_RING;
@@ -26,12 +27,17 @@ constexpr uint32_t SCATTER_RING_TILE = SCATTER_CONSUMER_WARPS * 32 * 16;   // on
 constexpr uint32_t scatter_fixed_bytes(uint32_t lp) {
     return (4u << lp) + 4u * APPW_SMEM_MAX + SCATTER_RING_STAGES * SCATTER_RING_TILE + 128u;
 }
-constexpr uint32_t scatter_hot_slots(uint32_t lp) { return ((SCATTER_SMEM_BYTES - scatter_fixed_bytes(lp)) / 21u) & ~31u; }
+constexpr uint32_t WORD_WAYS = 2, TAG_WAYS = 4;
+constexpr uint32_t scatter_slots(uint32_t lp, bool words) { return ((SCATTER_SMEM_BYTES - scatter_fixed_bytes(lp)) / (words ? 16u : 21u)) & ~31u; }
+constexpr uint32_t scatter_hot_slots(uint32_t lp) { return scatter_slots(lp, true); }   // of the directory image, either form
+// A word holds the top bits of what the bucket hash leaves over and, below them, phase and operator.  All ones there mark
+// an empty slot, so that those two have one bit less.
+constexpr uint32_t DIR_ID_BITS = 12, DIR_ID_MASK = (1u << DIR_ID_BITS) - 1u;
 
 // Where one key dominates the trace, the last part of the accumulators holds the warps' queues instead (64 records
 // each), and the directory is that much smaller.
 constexpr uint32_t SCATTER_QUEUE = 64, SCATTER_QUEUE_BYTES = 32 * SCATTER_QUEUE * 16;
-constexpr uint32_t scatter_dominated_slots(uint32_t lp) { return ((scatter_hot_slots(lp) * 12u - SCATTER_QUEUE_BYTES - 16u) / 12u) & ~31u; }
+constexpr uint32_t scatter_dominated_slots(uint32_t lp, bool words) { return ((scatter_slots(lp, words) * 12u - SCATTER_QUEUE_BYTES - 16u) / 12u) & ~31u; }
 
 struct IngestParams {
     const void* recs;          // all records of this launch (16-byte aligned) ...
@@ -44,18 +50,21 @@ struct IngestParams {
     uint32_t phase_lim;        // n_phases << 16: bound of (phase << 16 | op_id)
     uint32_t appw_in_smem;
     const uint32_t* app_w;     // device copy of the card-hour weights
+    ShortFormat fmt;           // short spill entries; operators below 2^fmt.op_bits fit a directory word
     const ull* hot_keys;       // directory image, hot_slots entries of ~key (0 = empty)
     uint32_t hot_slots;        // multiple of 4
     uint32_t img_rows;         // rows of hot_img that hold sums since the last fold; a CTA beyond them starts its row afresh
     ulonglong2* hot_img;       // [n_groups][hot_slots] each CTA's directory sums since the last fold, {lo, count | hi << 40}
     TableRef t;
     // spill buffers: entry i of scatter CTA g for partition p at spill + ((g * P + p) * cap + i) * 12 bytes: an 8-byte
-    // word {product, operator} and a 4-byte word {phase, low hash bits}, the 8-byte word at the 8-byte aligned end
+    // word {product, operator} and a 4-byte word {phase, low hash bits}, the 8-byte word at the 8-byte aligned end;
+    // short entries (ShortFormat) at spill + ((g * P + p) * short_cap + i) * 8 bytes
     unsigned char* spill;
     uint32_t* spill_cnt;       // [n_groups][P]
     uint32_t n_groups;         // G, row pitch of the buffers (= CTAs of the widest scatter launch)
     uint32_t cap;              // entries per (partition, CTA) buffer, a multiple of 32 (whole 128-byte lines)
     uint32_t drain_above;      // ask for a drain when a buffer holds more entries than this
+    uint32_t short_cap, short_drain_above;   // the same in short entries
     ull seq;                   // sequence number of this launch
 };
 
@@ -77,7 +86,10 @@ struct PartitionParams {
     const unsigned char* spill;
     uint32_t* spill_cnt;
     uint32_t n_groups;         // scatter CTAs whose buffers are read
-    uint32_t cap;
+    uint32_t cap, short_cap;
+    ShortFormat fmt;
+    uint32_t n_apps;
+    const uint32_t* app_w;     // card-hour weights (short entries)
     uint32_t force;            // 1: drain unconditionally; 0: only if the scatter launch `seq` asked for it
     ull seq;
     ulonglong2* queue;         // [gridDim][queue_cap] entries whose first look failed, settled after the partition's stream
@@ -85,11 +97,13 @@ struct PartitionParams {
 };
 
 // Scratch of the directory build's last steps (cleared by every build up to `key`).
-constexpr uint32_t HOT_SELECT_MAX = 14336;   // candidates kept (directory <= 11.6K slots, x1.25)
-constexpr uint32_t HOT_BUCKETS_MAX = 3072;   // directory buckets (<= 11.6K / 4)
+constexpr uint32_t HOT_SELECT_MAX = 27648;   // candidates kept (see hot_level_kernel)
+constexpr uint32_t HOT_BUCKETS_MAX = 6912;   // directory buckets
+static_assert(scatter_slots(8, true) / WORD_WAYS <= HOT_BUCKETS_MAX && scatter_slots(8, false) / TAG_WAYS <= HOT_BUCKETS_MAX &&
+              scatter_slots(8, true) * 2 <= HOT_SELECT_MAX, "directory build scratch");
 struct HotBuildScratch {
     uint32_t n, most, threshold, done;
-    uint32_t weight, pad[3];                     // sampled weight in the directory
+    uint32_t weight, max_op, pad[2];             // sampled weight in the directory, largest operator sampled
     uint32_t lost[4];                            // sampled weight each multiplier would lose
     uint32_t hist[1024];                         // candidates by count
     uint32_t occupancy[4][HOT_BUCKETS_MAX];
@@ -104,9 +118,10 @@ struct HotBuildParams {
     ull stride;                // records per sampled one (below 2^32)
     uint32_t n_sample;         // n_sample * stride <= records of the call
     uint32_t n_apps, n_phases;
+    uint32_t op_bits;          // operators below 2^op_bits fit a directory word (0: that form is not used)
     ull* hot_keys;
-    uint32_t hot_slots;
-    uint32_t dominated_slots;  // slots in use when one key dominates
+    uint32_t hot_slots;        // of the image
+    uint32_t slots[2][2];      // slots in use by [words][one key dominates]
     ull* sample;               // [n_sample] the sampled keys, all ones = invalid record
     uint32_t* sketch;          // [2^20] sample counters by hash
     ull* cand_keys;            // [1 << cand_bits] candidate table: ~key, 0 = empty
@@ -226,6 +241,7 @@ cudaError_t launch_direct(DirectParams p, int n_sms, cudaStream_t stream);
 cudaError_t scatter_prepare();
 cudaError_t launch_scatter(const IngestParams& p, bool hot, int grid, cudaStream_t stream);
 cudaError_t launch_partition(const PartitionParams& p, int n_sms, cudaStream_t stream);
+inline size_t partition_smem_bytes(uint32_t C, uint32_t n_apps, bool short_entries) { return (size_t)C * 20 + (short_entries ? (size_t)n_apps * 4 : 0); }
 cudaError_t launch_hot_build(const HotBuildParams& p, int n_sms, cudaStream_t stream);
 cudaError_t launch_hot_fold(const ull* hot_keys, const ulonglong2* hot_img, uint32_t n_groups, uint32_t hot_slots,
                             const TableRef& t, cudaStream_t stream);

@@ -5,9 +5,17 @@
 // validates, packs the key and multiplies the application's card-hour weight by the duration.
 //   * Keys found in the shared-memory HOT DIRECTORY (the most frequent keys of a sample of the
 //     trace, identical in every CTA, read-only during the pass) are accumulated on the spot with
-//     32-bit shared-memory atomics in limbs with explicit carries.
-//   * Every other record becomes a 12-byte entry {product, operator, phase, hash bits} appended to
-//     the CTA's private buffer of the key's partition (see spill_append).
+//     32-bit shared-memory atomics in limbs with explicit carries.  It comes in two forms:
+//       words  a key's phase and operator, if they fit 11 bits together, and what its bucket leaves over of the bucket
+//              hash (a bijection of the shape) make one 32-bit word that identifies it inside the bucket: one 8-byte
+//              load looks at both slots of a bucket and settles the look-up.  16 bytes a slot instead of 21 hold a third more
+//              keys, and what is left of a record fits a short entry (2^27 records, 50 % spilled: 820 -> 655 us; 67 %
+//              spilled 970 -> 700; 27 % 690 -> 560; 1 024 keys, none spilled: 690 -> 550).
+//       tags   operators of any size: a tag byte per slot of a 4-way bucket, the slot whose tag matches confirmed
+//              against its 8-byte key.  Chosen by the directory build where a sampled operator does not fit a word.
+//   * Every other record becomes an entry appended to the CTA's private buffer of the key's partition: with the words
+//     form a short one of 8 bytes {phase, operator, hash bits, application, duration} (short_append), with the tags form,
+//     or without a directory, one of 12 bytes {product, operator, phase, hash bits} (spill_append).
 // At the end the CTA adds its directory accumulators to its own row of a directory image
 // ([CTA][slot], plain coalesced read-modify-writes; hot_fold_kernel adds the rows into the table
 // before results are read) and stores its per-partition cursors: the buffers persist across launches
@@ -30,30 +38,41 @@ namespace {
 #endif
 constexpr int SCATTER_THREADS = ATREX_SCATTER_THREADS;
 constexpr uint32_t NO_SLOT = 0xFFFFFFFFu;
-constexpr uint32_t DIR_WAYS = 4;
+// the directory's form
+constexpr int DIR_NONE = 0, DIR_TAGS = 1, DIR_WORDS = 2;
 
 // Shared-memory map of the scatter pass for 2^LP partitions (byte offsets into the dynamic shared memory).
-template <uint32_t LP>
+template <uint32_t LP, int DIR>
 struct Smem {
     static constexpr uint32_t P = 1u << LP;
-    static constexpr uint32_t SLOTS = scatter_hot_slots(LP);   // directory slots, whole 4-way buckets
-    static constexpr uint32_t NB = SLOTS / DIR_WAYS;
+    static constexpr bool W = DIR == DIR_WORDS;
+    static constexpr uint32_t WAYS = W ? WORD_WAYS : TAG_WAYS;
+    static constexpr uint32_t SLOTS = scatter_slots(LP, W);     // directory slots, whole buckets
+    static constexpr uint32_t NB = SLOTS / WAYS;
     static constexpr uint32_t RING = 0;                         // record ring: SCATTER_RING_STAGES tiles
     static constexpr uint32_t CUR = RING + SCATTER_RING_STAGES * SCATTER_RING_TILE;   // u32[P]  entries appended to this CTA's buffer of each partition
     static constexpr uint32_t APPW = CUR + 4u * P;              // u32[APPW_SMEM_MAX]  card-hour weights
-    static constexpr uint32_t TAG = APPW + 4u * APPW_SMEM_MAX;  // u32[NB + 1]  four 8-bit tags per bucket (+ one pad bucket)
+    static constexpr uint32_t LONG = APPW + 4u * APPW_SMEM_MAX;    // words: records that took two short entries (and a pad word)
+    static constexpr uint32_t WORDS = LONG + 8u;                // ... u32[SLOTS]
+    static constexpr uint32_t TAG = LONG;                       // tags: u32[NB + 1]  four 8-bit tags per bucket (+ one pad bucket)
     static constexpr uint32_t KEYS = (TAG + 4u * (NB + 1u) + 7u) & ~7u;   // ull[SLOTS + 4]  key, all ones = empty
-    static constexpr uint32_t ACC = KEYS + 8u * (SLOTS + DIR_WAYS);       // {u32 lo, u32 hi, u32 count}[SLOTS + 4]
-    static constexpr uint32_t TOTAL = ACC + 12u * (SLOTS + DIR_WAYS);
+    static constexpr uint32_t PAD = W ? 0u : TAG_WAYS;          // (a look-up without a match reads the slot behind its bucket)
+    static constexpr uint32_t ACC = W ? WORDS + 4u * SLOTS : KEYS + 8u * (SLOTS + PAD);   // {u32 lo, u32 hi, u32 count}[SLOTS + PAD]
+    static constexpr uint32_t TOTAL = ACC + 12u * (SLOTS + PAD);
     // one key dominates: fewer slots in use, the warps' queues behind them
-    static constexpr uint32_t SLOTS_DOM = scatter_dominated_slots(LP), NB_DOM = SLOTS_DOM / DIR_WAYS;
+    static constexpr uint32_t SLOTS_DOM = scatter_dominated_slots(LP, W), NB_DOM = SLOTS_DOM / WAYS;
     static constexpr uint32_t QUEUE = (ACC + 12u * SLOTS_DOM + 15u) & ~15u;   // uint4[32 warps][SCATTER_QUEUE]
     static_assert(QUEUE + SCATTER_QUEUE_BYTES <= TOTAL, "queues");
     template <ull SKEW>
     static constexpr uint32_t NB_OF = SKEW == SKEW_DOMINATED ? NB_DOM : NB;
     static_assert(TOTAL <= SCATTER_SMEM_BYTES, "scatter pass shared memory");
     static_assert(SLOTS % 32 == 0, "whole buckets");
+    // The products hash x buckets of a bucket's hashes differ by multiples of the number of buckets in their low words,
+    // so with at least 2^DIR_ID_BITS buckets the bits that a word keeps of it tell them apart.
+    static_assert(!W || SCATTER_RING_STAGES != 0 || NB_DOM >= 1u << DIR_ID_BITS, "words identify keys");
 };
+template <uint32_t LP>
+constexpr uint32_t smem_total() { return Smem<LP, DIR_WORDS>::TOTAL > Smem<LP, DIR_TAGS>::TOTAL ? Smem<LP, DIR_WORDS>::TOTAL : Smem<LP, DIR_TAGS>::TOTAL; }
 
 __device__ __forceinline__ void ld_stream_256(const void* p, uint32_t (&w)[8]) {
     asm volatile("ld.global.L1::no_allocate.L2::evict_first.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
@@ -61,11 +80,16 @@ __device__ __forceinline__ void ld_stream_256(const void* p, uint32_t (&w)[8]) {
                  : "l"(p));
 }
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-// Loads of the directory's tags and keys and of the weights: these arrays are read-only during the
+// Loads of the directory's words, tags and keys and of the weights: these arrays are read-only during the
 // pass, so the loads are not volatile and the compiler may overlap the look-ups of several records.
 __device__ __forceinline__ uint32_t lds_u32(uint32_t a) {
     uint32_t v;
     asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a));
+    return v;
+}
+__device__ __forceinline__ uint2 lds_v2u32(uint32_t a) {
+    uint2 v;
+    asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
     return v;
 }
 __device__ __forceinline__ ull lds_u64(uint32_t a) {
@@ -118,7 +142,8 @@ __device__ __noinline__ void drain_slot(TableRef t, uint32_t acc, ull key, uint3
 
 // (rare) A record that cannot take the limb route: straight to the table with full 64-bit adds.
 __device__ __noinline__ void table_route(TableRef t, ull key, uint32_t h, ull prod) { table_accumulate(t, key, h, prod, 0, 1); }
-// (rare) An invalid record is counted; a valid one whose product has bits at or above 2^48 goes to the table.
+// (rare) An invalid record is counted; a valid one whose product has bits at or above 2^48, or whose operator does not
+// fit, goes to the table.
 __device__ __noinline__ void rare_record(TableRef t, bool valid, ull key, uint32_t h, ull prod) {
     if (valid)
         table_accumulate(t, key, h, prod, 0, 1);
@@ -129,10 +154,10 @@ __device__ __noinline__ void rare_record(TableRef t, bool valid, ull key, uint32
 // Add (count, v) to a directory slot, v < 2^53, count <= 32.  Most products fit 32 bits and most
 // low-limb adds do not wrap: the high limb is then left alone (one returning atomic and one reduction
 // per hit instead of two and one).
-template <uint32_t LP>
+template <uint32_t LP, int DIR>
 __device__ __forceinline__ void dir_add(const IngestParams& p, const Ctx& c, uint32_t slot, ull v, uint32_t count, ull key,
                                         uint32_t h) {
-    const uint32_t acc = c.sb + Smem<LP>::ACC + ATREX_INDEX(slot, Smem<LP>::SLOTS, p.t.ctl) * 12u;
+    const uint32_t acc = c.sb + Smem<LP, DIR>::ACC + ATREX_INDEX(slot, (Smem<LP, DIR>::SLOTS), p.t.ctl) * 12u;
     const uint32_t v0 = (uint32_t)v;
     const uint32_t o0 = atoms_add(acc, v0);
     reds_add(acc + 8, count);
@@ -143,10 +168,8 @@ __device__ __forceinline__ void dir_add(const IngestParams& p, const Ctx& c, uin
     }
 }
 
-// (rare) The buffer is full: the ticket is handed back and the record takes the exact slow path.
-template <uint32_t LP>
-__device__ __noinline__ void spill_overflow(TableRef t, uint32_t cw, ull key, ull prod, uint32_t h) {
-    reds_add(cw, 0xFFFFFFFFu);
+// (rare) The buffer is full: the ticket has been handed back, the record takes the exact slow path.
+__device__ __noinline__ void count_overflow(TableRef t, ull key, ull prod, uint32_t h) {
     table_accumulate(t, key, h, prod, 0, 1);
     atomicAdd(&t.ctl->n_overflow, 1ull);
 }
@@ -159,8 +182,8 @@ template <uint32_t LP>
 __device__ __forceinline__ void spill_append(const IngestParams& p, Ctx& c, bool todo, uint32_t khi, uint32_t shape, ull prod,
                                              uint32_t h) {
     if (!todo) return;
-    const uint32_t part = ATREX_INDEX(h >> (32 - LP), Smem<LP>::P, p.t.ctl);
-    const uint32_t cw = c.sb + Smem<LP>::CUR + part * 4u;
+    const uint32_t part = ATREX_INDEX(h >> (32 - LP), 1u << LP, p.t.ctl);
+    const uint32_t cw = c.sb + Smem<LP, DIR_NONE>::CUR + part * 4u;     // (the same in either form)
     const uint32_t tk = atoms_add(cw, 1u);
     if (tk < p.cap) {
         // Entry tk occupies bytes [12 tk, 12 tk + 12) of the buffer; its 8-byte word sits at whichever
@@ -187,16 +210,49 @@ __device__ __forceinline__ void spill_append(const IngestParams& p, Ctx& c, bool
             if ((off & 127u) - 96u < 12u) asm volatile("prefetch.global.L2 [%0+64];" ::"l"(at));
         }
     } else {
-        spill_overflow<LP>(p.t, cw, ((ull)khi << 32) | shape, prod, h);
+        reds_add(cw, 0xFFFFFFFFu);
+        count_overflow(p.t, ((ull)khi << 32) | shape, prod, h);
     }
+}
+
+// The same as a short entry (ShortFormat), in one store; a duration that does not fit takes a second entry behind it.
+template <uint32_t LP>
+__device__ __forceinline__ void short_append(const IngestParams& p, Ctx& c, bool todo, uint32_t khi, uint32_t app, uint32_t shape,
+                                             uint32_t dur, ull prod, uint32_t h) {
+    if (!todo) return;
+    const uint32_t part = ATREX_INDEX(h >> (32 - LP), 1u << LP, p.t.ctl);
+    const uint32_t cw = c.sb + Smem<LP, DIR_WORDS>::CUR + part * 4u;
+    const uint32_t rest = dur >> p.fmt.dur_bits, n = rest ? 2u : 1u;
+    const uint32_t tk = atoms_add(cw, n);
+    if (tk + n <= p.short_cap) {
+        const uint32_t hash = h << LP, id = ((khi >> 16) << p.fmt.op_bits) + (khi & 0xFFFFu);
+        const uint32_t hi = (id << (31u - p.fmt.id_bits)) | (hash >> (1u + p.fmt.id_bits));
+        const uint32_t lo = (hash << (31u - p.fmt.id_bits)) | (app << p.fmt.dur_bits);
+        unsigned char* at = c.my_spill + (part * p.short_cap + ATREX_INDEX(tk, p.short_cap, p.t.ctl)) * SHORT_ENTRY_BYTES;
+        asm volatile("st.global.L2::cache_hint.v2.u32 [%0], {%1, %2}, %3;" ::"l"(at), "r"(lo | (dur & p.fmt.dur_mask())), "r"(hi), "l"(c.keep) : "memory");
+        // three entries before the buffer reaches its next line (four, where this one takes two places), as above
+        if ((tk & 15u) - (14u - n) < n) asm volatile("prefetch.global.L2 [%0+64];" ::"l"(at));
+        if (rest) {
+            reds_add(c.sb + Smem<LP, DIR_WORDS>::LONG, 1u);
+            asm volatile("st.global.L2::cache_hint.v2.u32 [%0+8], {%1, %2}, %3;" ::"l"(at), "r"(lo | rest), "r"(hi | SHORT_CONTINUATION), "l"(c.keep) : "memory");
+        }
+    } else {
+        reds_add(cw, 0u - n);
+        count_overflow(p.t, ((ull)khi << 32) | shape, prod, h);
+    }
+}
+
+// A directory slot's word (words form): the bits that the bucket leaves over of hash x buckets, phase and operator.
+__device__ __forceinline__ uint32_t dir_word(uint32_t product_lo, uint32_t khi, uint32_t op_bits) {
+    return (product_lo & ~DIR_ID_MASK) | (((khi >> 16) << op_bits) + (khi & 0xFFFFu));
 }
 
 // One record, start to finish (the register-staged loop has no registers to spare for working on
 // two records at once).  Called by all lanes of a warp together (absent records masked by `present`).
-template <uint32_t LP, bool HOT, ull SKEW, bool FULL>
+template <uint32_t LP, int DIR, ull SKEW, bool FULL>
 __device__ __forceinline__ void one_record(const IngestParams& p, Ctx& c, uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3,
                                            bool present) {
-    using L = Smem<LP>;
+    using L = Smem<LP, DIR>;
     const uint32_t khi = w1 & 0x00FFFFFFu;                  // phase << 16 | op_id: the key's high word
     bool ok = w0 < p.n_apps && khi < p.phase_lim;
     if (!FULL) ok = ok && present;
@@ -210,20 +266,33 @@ __device__ __forceinline__ void one_record(const IngestParams& p, Ctx& c, uint32
     // < 2^20, durations < 2^28).  Anything larger is still exact: straight to the table.  That and
     // the count of invalid records share one rarely taken branch (two separate ones cost the
     // configurations whose records mostly hit the directory 4-9 %).
-    const bool todo_in = ok && (uint32_t)(prod >> 32) < 0x10000u;
+    bool todo_in = ok && (uint32_t)(prod >> 32) < 0x10000u;
+    // (words form: an operator that no sampled record had may not fit a word and a short entry)
+    if (DIR == DIR_WORDS) todo_in = todo_in && ((khi & 0xFFFFu) >> p.fmt.op_bits) == 0u;
     bool todo = todo_in;
     if ((FULL || present) && !todo_in) rare_record(p.t, ok, key, h, prod);
-    if (HOT) {
-        // Directory look-up: one 32-bit word per 4-slot bucket holds an 8-bit tag per slot (hash bits
-        // the bucket choice does not use); the lowest slot whose tag matches is confirmed against the
-        // 8-byte key.  A wrong tag match (1 in 64 look-ups) fails the confirmation and the record takes
-        // the spill path: slower, still exact.
+    if (DIR != DIR_NONE) {
         const uint32_t x = dir_mix(h, khi >> 16, c.mult);
-        const uint32_t b = ATREX_INDEX(__umulhi(x, L::template NB_OF<SKEW>), L::template NB_OF<SKEW>, p.t.ctl);
-        const uint32_t t = lds_u32(c.sb + L::TAG + b * 4u) ^ __byte_perm(x, 0, 0);   // 0 in the bytes that match
-        const uint32_t m = (t - 0x01010101u) & ~t & 0x80808080u;                      // lowest flagged byte is exact
-        const uint32_t at = ATREX_INDEX(b * DIR_WAYS + ((uint32_t)__clz((int)__brev(m)) >> 3), L::SLOTS + DIR_WAYS, p.t.ctl);
-        bool hit = todo && m != 0 && lds_u64(c.sb + L::KEYS + at * 8u) == key;
+        uint32_t at;
+        bool hit;
+        if (DIR == DIR_WORDS) {
+            const ull product = (ull)x * L::template NB_OF<SKEW>;
+            const uint32_t b = ATREX_INDEX((uint32_t)(product >> 32), L::template NB_OF<SKEW>, p.t.ctl);
+            const uint32_t word = dir_word((uint32_t)product, khi, p.fmt.op_bits);
+            const uint2 w = lds_v2u32(c.sb + L::WORDS + b * 8u);
+            const bool second = w.y == word;
+            at = b * 2u + (second ? 1u : 0u);
+            hit = todo && (w.x == word || second);
+        } else {
+            // One 32-bit word per 4-slot bucket holds an 8-bit tag per slot (hash bits the bucket choice does not
+            // use); the lowest slot whose tag matches is confirmed against the 8-byte key.  A wrong tag match (1 in
+            // 64 look-ups) fails the confirmation and the record takes the spill path: slower, still exact.
+            const uint32_t b = ATREX_INDEX(__umulhi(x, L::template NB_OF<SKEW>), L::template NB_OF<SKEW>, p.t.ctl);
+            const uint32_t t = lds_u32(c.sb + L::TAG + b * 4u) ^ __byte_perm(x, 0, 0);   // 0 in the bytes that match
+            const uint32_t m = (t - 0x01010101u) & ~t & 0x80808080u;                      // lowest flagged byte is exact
+            at = ATREX_INDEX(b * TAG_WAYS + ((uint32_t)__clz((int)__brev(m)) >> 3), L::SLOTS + TAG_WAYS, p.t.ctl);
+            hit = todo && m != 0 && lds_u64(c.sb + L::KEYS + at * 8u) == key;
+        }
         if (SKEW != SKEW_NONE) {
             // a key is frequent enough for collisions inside a warp: combine the lanes that share the first hitting lane's slot
             const unsigned hits = __ballot_sync(0xFFFFFFFFu, hit);
@@ -236,27 +305,30 @@ __device__ __forceinline__ void one_record(const IngestParams& p, Ctx& c, uint32
                     const uint32_t s_lo = __reduce_add_sync(same, (uint32_t)prod & 0xFFFFFFu);
                     const uint32_t s_hi = __reduce_add_sync(same, (uint32_t)(prod >> 24));
                     if ((threadIdx.x & 31u) == (unsigned)lead)
-                        dir_add<LP>(p, c, ls, (ull)s_lo + ((ull)s_hi << 24), (uint32_t)__popc(same), key, h);
+                        dir_add<LP, DIR>(p, c, ls, (ull)s_lo + ((ull)s_hi << 24), (uint32_t)__popc(same), key, h);
                     hit = false;
                     todo = false;
                 }
             }
         }
         if (hit) {
-            dir_add<LP>(p, c, at, prod, 1u, key, h);
+            dir_add<LP, DIR>(p, c, at, prod, 1u, key, h);
             todo = false;
         }
     }
-    spill_append<LP>(p, c, todo, khi, w2, prod, h);
+    if (DIR == DIR_WORDS)
+        short_append<LP>(p, c, todo, khi, w0, w2, w3, prod, h);
+    else
+        spill_append<LP>(p, c, todo, khi, w2, prod, h);
 }
 
 // The same for R records per lane at once (used with the shared-memory record ring, where the
 // registers allow it; w[r] = the record's four words).  Called by all lanes of a
 // warp together (absent records masked by `present`).  Written in stages over the R records so that
 // their shared-memory round trips overlap: all look-ups are issued before the first result is used.
-template <uint32_t LP, bool HOT, ull SKEW, bool FULL, int R>
+template <uint32_t LP, int DIR, ull SKEW, bool FULL, int R>
 __device__ __forceinline__ void process(const IngestParams& p, Ctx& c, const uint32_t (&w)[R][4], bool present) {
-    using L = Smem<LP>;
+    using L = Smem<LP, DIR>;
     uint32_t khi[R], h[R], wgt[R], x[R], tags[R];
     bool todo[R];
 #pragma unroll
@@ -270,7 +342,7 @@ __device__ __forceinline__ void process(const IngestParams& p, Ctx& c, const uin
         // some other weight, which is not used), else from global memory
         wgt[r] = (p.appw_in_smem != 0) ? lds_u32(c.sb + L::APPW + (w[r][0] & (APPW_SMEM_MAX - 1u)) * 4u) : __ldg(p.app_w + (ok ? w[r][0] : 0u));
         h[r] = hash32(khi[r] & 0xFFFFu, w[r][2]);
-        if (HOT) {
+        if (DIR != DIR_NONE) {
             // Directory look-up: one 32-bit word per 4-slot bucket holds an 8-bit tag per slot (hash
             // bits the bucket choice does not use)
             x[r] = dir_mix(h[r], khi[r] >> 16, c.mult);
@@ -283,13 +355,13 @@ __device__ __forceinline__ void process(const IngestParams& p, Ctx& c, const uin
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         prod[r] = (ull)wgt[r] * (ull)w[r][3];
-        if (HOT) {
+        if (DIR != DIR_NONE) {
             // the lowest slot whose tag matches is confirmed against the 8-byte key; a wrong tag match
             // (1 in 64 look-ups) fails the confirmation and the record takes the spill path: slower,
             // still exact
             const uint32_t t = tags[r] ^ __byte_perm(x[r], 0, 0);                     // 0 in the bytes that match
             const uint32_t m = (t - 0x01010101u) & ~t & 0x80808080u;                  // lowest flagged byte is exact
-            at[r] = __umulhi(x[r], L::template NB_OF<SKEW>) * DIR_WAYS + ((uint32_t)__clz((int)__brev(m)) >> 3);
+            at[r] = __umulhi(x[r], L::template NB_OF<SKEW>) * TAG_WAYS + ((uint32_t)__clz((int)__brev(m)) >> 3);
             found[r] = ~0ull;
             if (m != 0) found[r] = lds_u64(c.sb + L::KEYS + at[r] * 8u);
         }
@@ -304,9 +376,9 @@ __device__ __forceinline__ void process(const IngestParams& p, Ctx& c, const uin
             table_route(p.t, key, h[r], prod[r]);
             todo[r] = false;
         }
-        hit[r] = HOT && todo[r] && found[r] == key;
+        hit[r] = DIR != DIR_NONE && todo[r] && found[r] == key;
     }
-    if (HOT && SKEW != SKEW_NONE) {
+    if (DIR != DIR_NONE && SKEW != SKEW_NONE) {
         // a key is frequent enough for collisions inside a warp: combine the lanes that share the first hitting lane's slot
 #pragma unroll
         for (int r = 0; r < R; ++r) {
@@ -320,13 +392,13 @@ __device__ __forceinline__ void process(const IngestParams& p, Ctx& c, const uin
                 const uint32_t s_lo = __reduce_add_sync(same, (uint32_t)prod[r] & 0xFFFFFFu);
                 const uint32_t s_hi = __reduce_add_sync(same, (uint32_t)(prod[r] >> 24));
                 if ((threadIdx.x & 31u) == (unsigned)lead)
-                    dir_add<LP>(p, c, ls, (ull)s_lo + ((ull)s_hi << 24), (uint32_t)__popc(same), ((ull)khi[r] << 32) | w[r][2], h[r]);
+                    dir_add<LP, DIR>(p, c, ls, (ull)s_lo + ((ull)s_hi << 24), (uint32_t)__popc(same), ((ull)khi[r] << 32) | w[r][2], h[r]);
                 hit[r] = false;
                 todo[r] = false;
             }
         }
     }
-    if (HOT) {
+    if (DIR != DIR_NONE) {
         // hits: the returning low-limb adds of all R records first, then the rest
         uint32_t o0[R];
 #pragma unroll
@@ -351,7 +423,7 @@ __device__ __forceinline__ void process(const IngestParams& p, Ctx& c, const uin
     for (int r = 0; r < R; ++r) spill_append<LP>(p, c, todo[r], khi[r], w[r][2], prod[r], h[r]);
 }
 
-template <uint32_t LP, bool HOT, ull SKEW>
+template <uint32_t LP, int DIR, ull SKEW>
 __device__ __forceinline__ void scatter_body(const IngestParams& p, Ctx& c) {
     // CTA b handles record pairs (b + k * gridDim) * 1024 + tid, k = 0, 1, ...  Two 32-byte loads
     // alternate per thread: while one is consumed the next is in flight.  Rounds in which every
@@ -372,13 +444,13 @@ __device__ __forceinline__ void scatter_body(const IngestParams& p, Ctx& c) {
         }
     };
     auto consume_full = [&](const uint32_t (&raw)[8]) {
-        one_record<LP, HOT, SKEW, true>(p, c, raw[0], raw[1], raw[2], raw[3], true);
-        one_record<LP, HOT, SKEW, true>(p, c, raw[4], raw[5], raw[6], raw[7], true);
+        one_record<LP, DIR, SKEW, true>(p, c, raw[0], raw[1], raw[2], raw[3], true);
+        one_record<LP, DIR, SKEW, true>(p, c, raw[4], raw[5], raw[6], raw[7], true);
     };
     auto consume_tail = [&](uint32_t round, const uint32_t (&raw)[8]) {
         const bool present = round < rounds && first + (ull)round * stride < p.n_pairs;
-        one_record<LP, HOT, SKEW, false>(p, c, raw[0], raw[1], raw[2], raw[3], present);
-        one_record<LP, HOT, SKEW, false>(p, c, raw[4], raw[5], raw[6], raw[7], present);
+        one_record<LP, DIR, SKEW, false>(p, c, raw[0], raw[1], raw[2], raw[3], present);
+        one_record<LP, DIR, SKEW, false>(p, c, raw[4], raw[5], raw[6], raw[7], present);
     };
     fetch(0, bufA);
     uint32_t round = 0;
@@ -389,7 +461,7 @@ __device__ __forceinline__ void scatter_body(const IngestParams& p, Ctx& c) {
         // Each load goes out behind an L2 prefetch of the round after it -- where a third of the sample or more is in
         // the directory: the lines of a trace that mostly spills need the L2 more (52 % spilled: 856 -> 832 us
         // per 2^27 records with the prefetch, 75 %: 1 003 -> 1 026).
-        const bool ahead = (threadIdx.x & 3u) == 0 && HOT && p.t.ctl->prefetch != 0;
+        const bool ahead = (threadIdx.x & 3u) == 0 && DIR != DIR_NONE && p.t.ctl->prefetch != 0;
         for (; round + 4 <= full_rounds; round += 2) {
             ld_stream_256(next, bufB);
             if (ahead) asm volatile("prefetch.global.L2 [%0];" ::"l"(next + step));
@@ -412,7 +484,7 @@ __device__ __forceinline__ void scatter_body(const IngestParams& p, Ctx& c) {
         uint4 v = make_uint4(0, 0, 0, 0);
         const bool present = threadIdx.x < p.n_single;
         if (present) v = *reinterpret_cast<const uint4*>(threadIdx.x == 0 ? p.single[0] : p.single[1]);
-        one_record<LP, HOT, SKEW, false>(p, c, v.x, v.y, v.z, v.w, present);
+        one_record<LP, DIR, SKEW, false>(p, c, v.x, v.y, v.z, v.w, present);
     }
 }
 
@@ -421,9 +493,9 @@ __device__ __forceinline__ void scatter_body(const IngestParams& p, Ctx& c) {
 // warp's queue in shared memory and through one_record 32 at a time, so that what is left of a warp's 32
 // records does not cost the price of 32.  Bound by DRAM once the key holds most records (90 %: 140 -> 57 warp
 // instructions per 32 records, 0.66 -> 0.39 ms per 2^27 records); the queue pays from a share of 3/8 on.
-template <uint32_t LP>
+template <uint32_t LP, int DIR>
 __device__ __forceinline__ void dominated_body(const IngestParams& p, Ctx& c) {
-    using L = Smem<LP>;
+    using L = Smem<LP, DIR>;
     const uint32_t lane = threadIdx.x & 31u, lt = (1u << lane) - 1u;
     const uint32_t queue = c.sb + L::QUEUE + (threadIdx.x >> 5) * (SCATTER_QUEUE * 16u);
     const ull top = p.t.ctl->top_key;
@@ -437,7 +509,7 @@ __device__ __forceinline__ void dominated_body(const IngestParams& p, Ctx& c) {
             asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(queue + (q - n + lane) * 16u) : "memory");
         __syncwarp();
         q -= n;
-        one_record<LP, true, SKEW_DOMINATED, false>(p, c, v.x, v.y, v.z, v.w, lane < n);
+        one_record<LP, DIR, SKEW_DOMINATED, false>(p, c, v.x, v.y, v.z, v.w, lane < n);
     };
     auto take = [&](uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, bool present) {
         const bool match = (((w1 ^ top_hi) & 0x00FFFFFFu) | (w2 ^ top_lo)) == 0u && w0 < p.n_apps && present;
@@ -574,7 +646,7 @@ __device__ __forceinline__ uint4 lds_record(uint32_t a) {
     return v;
 }
 
-template <uint32_t LP, bool HOT, ull SKEW>
+template <uint32_t LP, int DIR, ull SKEW>
 __device__ __forceinline__ void ring_body(const IngestParams& p, Ctx& c, ull* full_bar, ull* empty_bar, volatile uint32_t* abort_flag) {
     constexpr uint32_t S = SCATTER_RING_STAGES > 0 ? SCATTER_RING_STAGES : 1;
     constexpr uint32_t TILE_RECS = SCATTER_CONSUMER_WARPS * 32;
@@ -600,7 +672,7 @@ __device__ __forceinline__ void ring_body(const IngestParams& p, Ctx& c, ull* fu
                 const ull first = T * TILE_RECS;
                 const uint32_t n_here = (uint32_t)(p.n_recs - first < TILE_RECS ? p.n_recs - first : TILE_RECS);
                 mbar_expect_tx(fb + s * 8, n_here * 16u);
-                bulk_load(c.sb + Smem<LP>::RING + s * SCATTER_RING_TILE, recs + first * 16, n_here * 16u, fb + s * 8, policy);
+                bulk_load(c.sb + Smem<LP, DIR>::RING + s * SCATTER_RING_TILE, recs + first * 16, n_here * 16u, fb + s * 8, policy);
             }
             if (*abort_flag) {
                 // leaving early: give the copies still in flight a (bounded) chance to land first
@@ -627,8 +699,8 @@ __device__ __forceinline__ void ring_body(const IngestParams& p, Ctx& c, ull* fu
         const ull first0 = ((ull)k * gridDim.x + blockIdx.x) * TILE_RECS, first1 = first0 + (ull)gridDim.x * TILE_RECS;
         const bool p0 = first0 + threadIdx.x < p.n_recs, p1 = second && first1 + threadIdx.x < p.n_recs;
         uint4 r0 = make_uint4(0, 0, 0, 0), r1 = make_uint4(0, 0, 0, 0);
-        if (p0) r0 = lds_record(c.sb + Smem<LP>::RING + s0 * SCATTER_RING_TILE + lane_off);
-        if (p1) r1 = lds_record(c.sb + Smem<LP>::RING + s1 * SCATTER_RING_TILE + lane_off);
+        if (p0) r0 = lds_record(c.sb + Smem<LP, DIR>::RING + s0 * SCATTER_RING_TILE + lane_off);
+        if (p1) r1 = lds_record(c.sb + Smem<LP, DIR>::RING + s1 * SCATTER_RING_TILE + lane_off);
         __syncwarp();
         if ((threadIdx.x & 31u) == 0) {   // the warp has its records in registers: hand the stages back
             mbar_arrive(eb + s0 * 8);
@@ -637,12 +709,113 @@ __device__ __forceinline__ void ring_body(const IngestParams& p, Ctx& c, ull* fu
         const uint32_t w[2][4] = {{r0.x, r0.y, r0.z, r0.w}, {r1.x, r1.y, r1.z, r1.w}};
         const bool full = second && first1 + TILE_RECS <= p.n_recs;     // both tiles complete (uniform)
         if (full) {
-            process<LP, HOT, SKEW, true, 2>(p, c, w, true);
+            process<LP, DIR, SKEW, true, 2>(p, c, w, true);
         } else {
             // ragged end: one record at a time, each with its own mask
             const uint32_t wa[1][4] = {{r0.x, r0.y, r0.z, r0.w}}, wb[1][4] = {{r1.x, r1.y, r1.z, r1.w}};
-            process<LP, HOT, SKEW, false, 1>(p, c, wa, p0);
-            process<LP, HOT, SKEW, false, 1>(p, c, wb, p1);
+            process<LP, DIR, SKEW, false, 1>(p, c, wa, p0);
+            process<LP, DIR, SKEW, false, 1>(p, c, wb, p1);
+        }
+    }
+}
+
+struct RingBars {
+    ull *full, *empty;
+    volatile uint32_t* abort_flag;
+};
+
+// What a CTA does with the directory in the form DIR: loads it, goes through its records, stores cursors and sums.
+template <uint32_t LP, int DIR>
+__device__ __forceinline__ void scatter_cta(const IngestParams& p, Ctx& c, unsigned char* smem_raw, const RingBars& ring) {
+    using L = Smem<LP, DIR>;
+    uint32_t* g_cursor = reinterpret_cast<uint32_t*>(smem_raw + L::CUR);
+    uint32_t* g_acc = reinterpret_cast<uint32_t*>(smem_raw + L::ACC);
+    const ull skew = DIR != DIR_NONE ? p.t.ctl->hot_skew : SKEW_NONE;
+    if (DIR == DIR_WORDS && threadIdx.x == 0) *reinterpret_cast<uint32_t*>(smem_raw + L::LONG) = 0;
+    if (DIR != DIR_NONE) {
+        for (uint32_t i = threadIdx.x; i < L::SLOTS + L::PAD; i += blockDim.x) {
+            const ull image = i < L::SLOTS ? p.hot_keys[i] : 0ull;   // ~key, 0 = empty
+            const uint32_t khi = (uint32_t)(~image >> 32), x = dir_mix(hash32(~image), (khi >> 16) & 0xFFu, c.mult);
+            if (DIR == DIR_WORDS) {
+                const uint32_t left = x * (skew == SKEW_DOMINATED ? L::NB_DOM : L::NB);
+                reinterpret_cast<uint32_t*>(smem_raw + L::WORDS)[i] = image ? dir_word(left, khi, p.fmt.op_bits) : DIR_ID_MASK;
+            } else {
+                reinterpret_cast<ull*>(smem_raw + L::KEYS)[i] = ~image;
+                (smem_raw + L::TAG)[i] = image ? (unsigned char)(x & 0xFFu) : 0;
+            }
+            g_acc[3 * i] = 0;
+            g_acc[3 * i + 1] = 0;
+            g_acc[3 * i + 2] = 0;
+        }
+    }
+    __syncthreads();
+
+    if (SCATTER_RING_STAGES > 0) {
+        if (DIR != DIR_NONE && skew == SKEW_DOMINATED)
+            ring_body<LP, DIR, SKEW_DOMINATED>(p, c, ring.full, ring.empty, ring.abort_flag);
+        else if (DIR != DIR_NONE && skew == SKEW_COMBINE)
+            ring_body<LP, DIR, SKEW_COMBINE>(p, c, ring.full, ring.empty, ring.abort_flag);
+        else
+            ring_body<LP, DIR, SKEW_NONE>(p, c, ring.full, ring.empty, ring.abort_flag);
+    } else {
+        if (DIR != DIR_NONE && skew == SKEW_DOMINATED)
+            dominated_body<LP, DIR>(p, c);
+        else if (DIR != DIR_NONE && skew == SKEW_COMBINE)
+            scatter_body<LP, DIR, SKEW_COMBINE>(p, c);
+        else
+            scatter_body<LP, DIR, SKEW_NONE>(p, c);
+    }
+
+    grid_dependents_launch();
+    __syncthreads();
+    const uint32_t cap = DIR == DIR_WORDS ? p.short_cap : p.cap, drain_above = DIR == DIR_WORDS ? p.short_drain_above : p.drain_above;
+    uint32_t spilled = 0, fullest = 0;
+    bool crowded = false;
+    if (DIR == DIR_WORDS && threadIdx.x == 0) spilled = 0u - *reinterpret_cast<const uint32_t*>(smem_raw + L::LONG);   // (records, not entries)
+    for (uint32_t i = threadIdx.x; i < L::P; i += blockDim.x) {
+        const size_t at = ((size_t)blockIdx.x << LP) + i;
+        const uint32_t before = p.spill_cnt[at], n = min(g_cursor[i], cap);
+        p.spill_cnt[at] = n;
+        spilled += n - before;
+        crowded |= n > drain_above;
+        fullest = max(fullest, n);
+    }
+    fullest = __reduce_max_sync(0xFFFFFFFFu, fullest);
+    spilled = __reduce_add_sync(0xFFFFFFFFu, spilled);
+    crowded = __any_sync(0xFFFFFFFFu, crowded);
+    if ((threadIdx.x & 31u) == 0) {
+        if (spilled) atomicAdd(&p.t.ctl->n_spilled, (ull)(long long)(int32_t)spilled);   // (the first warp's may be negative)
+        // a buffer is filling up: have the partition pass that follows this launch drain them
+        if (crowded) atomicMax(&p.t.ctl->drain_seq, p.seq);
+        atomicMax(&p.t.ctl->max_fill, (ull)fullest);
+    }
+    if (DIR != DIR_NONE) {
+        // This launch's directory sums go to the CTA's own row of the directory image: plain coalesced
+        // read-modify-writes, no atomics (148 CTAs adding the same few thousand keys into the table at
+        // the end of every launch cost 59 us per launch).  hot_fold_kernel adds the rows into the table
+        // before results are read.
+        ulonglong2* img = p.hot_img + (size_t)blockIdx.x * p.hot_slots;
+        const bool held = blockIdx.x < p.img_rows;   // the row holds earlier launches' sums
+        const uint32_t in_use = skew == SKEW_DOMINATED ? L::SLOTS_DOM : L::SLOTS;
+        for (uint32_t i0 = threadIdx.x; i0 < p.hot_slots; i0 += 4 * blockDim.x) {  // four slots per thread in flight
+            uint32_t cn[4], lo[4], hi[4];
+            ulonglong2 o[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const uint32_t i = i0 + u * blockDim.x;
+                const bool in = i < in_use;
+                lo[u] = in ? g_acc[3 * i] : 0u;
+                hi[u] = in ? g_acc[3 * i + 1] : 0u;
+                cn[u] = in ? g_acc[3 * i + 2] : 0u;
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) o[u] = held && (cn[u] | lo[u] | hi[u]) ? img[i0 + u * blockDim.x] : make_ulonglong2(0, 0);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (i0 + u * blockDim.x >= p.hot_slots || (held && (cn[u] | lo[u] | hi[u]) == 0)) continue;
+                const ull nlo = o[u].x + ((ull)lo[u] | ((ull)hi[u] << 32));
+                img[i0 + u * blockDim.x] = make_ulonglong2(nlo, o[u].y + (ull)cn[u] + ((nlo < o[u].x ? 1ull : 0ull) << HI_SHIFT));
+            }
         }
     }
 }
@@ -650,12 +823,9 @@ __device__ __forceinline__ void ring_body(const IngestParams& p, Ctx& c, ull* fu
 template <uint32_t LP, bool HOT>
 __global__ void __launch_bounds__(SCATTER_THREADS, 1) scatter_kernel(IngestParams p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    using L = Smem<LP>;
+    using L = Smem<LP, DIR_NONE>;                  // (what is used of it here is the same in every form)
     uint32_t* g_cursor = reinterpret_cast<uint32_t*>(smem_raw + L::CUR);
     uint32_t* g_appw = reinterpret_cast<uint32_t*>(smem_raw + L::APPW);
-    uint32_t* g_tag = reinterpret_cast<uint32_t*>(smem_raw + L::TAG);
-    ull* g_keys = reinterpret_cast<ull*>(smem_raw + L::KEYS);
-    uint32_t* g_acc = reinterpret_cast<uint32_t*>(smem_raw + L::ACC);
 
     __shared__ __align__(8) ull s_full[SCATTER_RING_STAGES ? SCATTER_RING_STAGES : 1], s_empty[SCATTER_RING_STAGES ? SCATTER_RING_STAGES : 1];
     __shared__ uint32_t s_abort;
@@ -673,93 +843,20 @@ __global__ void __launch_bounds__(SCATTER_THREADS, 1) scatter_kernel(IngestParam
     Ctx c;
     c.sb = smem_addr(smem_raw);
     c.mult = HOT ? (uint32_t)p.t.ctl->dir_mult : 1u;
-    c.my_spill = p.spill + ((size_t)blockIdx.x << LP) * p.cap * SPILL_ENTRY_BYTES;
+    c.my_spill = p.spill + ((size_t)blockIdx.x << LP) * p.cap * SPILL_ENTRY_BYTES;   // (as many bytes as short_cap short entries)
     asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(c.keep));
 
     // The buffers persist across launches until the partition pass drains them: resume the cursors.
     for (uint32_t i = threadIdx.x; i < L::P; i += blockDim.x) g_cursor[i] = p.spill_cnt[((size_t)blockIdx.x << LP) + i];
     if (p.appw_in_smem != 0)
         for (uint32_t i = threadIdx.x; i < p.n_apps; i += blockDim.x) g_appw[i] = p.app_w[i];
-    if (HOT) {
-        for (uint32_t i = threadIdx.x; i < L::SLOTS + DIR_WAYS; i += blockDim.x) {
-            const ull image = i < L::SLOTS ? p.hot_keys[i] : 0ull;   // ~key, 0 = empty
-            g_keys[i] = ~image;
-            reinterpret_cast<unsigned char*>(g_tag)[i] =
-                image ? (unsigned char)(dir_mix(hash32(~image), (uint32_t)(~image >> 48) & 0xFFu, c.mult) & 0xFFu) : 0;
-            g_acc[3 * i] = 0;
-            g_acc[3 * i + 1] = 0;
-            g_acc[3 * i + 2] = 0;
-        }
-    }
-    __syncthreads();
-
-    const ull skew = HOT ? p.t.ctl->hot_skew : SKEW_NONE;
-    if (SCATTER_RING_STAGES > 0) {
-        if (HOT && skew == SKEW_DOMINATED)
-            ring_body<LP, HOT, SKEW_DOMINATED>(p, c, s_full, s_empty, &s_abort);
-        else if (HOT && skew == SKEW_COMBINE)
-            ring_body<LP, HOT, SKEW_COMBINE>(p, c, s_full, s_empty, &s_abort);
-        else
-            ring_body<LP, HOT, SKEW_NONE>(p, c, s_full, s_empty, &s_abort);
-    } else {
-        if (HOT && skew == SKEW_DOMINATED)
-            dominated_body<LP>(p, c);
-        else if (HOT && skew == SKEW_COMBINE)
-            scatter_body<LP, HOT, SKEW_COMBINE>(p, c);
-        else
-            scatter_body<LP, HOT, SKEW_NONE>(p, c);
-    }
-
-    grid_dependents_launch();
-    __syncthreads();
-    uint32_t spilled = 0, fullest = 0;
-    bool crowded = false;
-    for (uint32_t i = threadIdx.x; i < L::P; i += blockDim.x) {
-        const size_t at = ((size_t)blockIdx.x << LP) + i;
-        const uint32_t before = p.spill_cnt[at], n = min(g_cursor[i], p.cap);
-        p.spill_cnt[at] = n;
-        spilled += n - before;
-        crowded |= n > p.drain_above;
-        fullest = max(fullest, n);
-    }
-    fullest = __reduce_max_sync(0xFFFFFFFFu, fullest);
-    spilled = __reduce_add_sync(0xFFFFFFFFu, spilled);
-    crowded = __any_sync(0xFFFFFFFFu, crowded);
-    if ((threadIdx.x & 31u) == 0) {
-        if (spilled) atomicAdd(&p.t.ctl->n_spilled, (ull)spilled);
-        // a buffer is filling up: have the partition pass that follows this launch drain them
-        if (crowded) atomicMax(&p.t.ctl->drain_seq, p.seq);
-        atomicMax(&p.t.ctl->max_fill, (ull)fullest);
-    }
-    if (HOT) {
-        // This launch's directory sums go to the CTA's own row of the directory image: plain coalesced
-        // read-modify-writes, no atomics (148 CTAs adding the same few thousand keys into the table at
-        // the end of every launch cost 59 us per launch).  hot_fold_kernel adds the rows into the table
-        // before results are read.
-        ulonglong2* img = p.hot_img + (size_t)blockIdx.x * L::SLOTS;
-        const bool held = blockIdx.x < p.img_rows;   // the row holds earlier launches' sums
-        const uint32_t in_use = skew == SKEW_DOMINATED ? L::SLOTS_DOM : L::SLOTS;
-        for (uint32_t i0 = threadIdx.x; i0 < L::SLOTS; i0 += 4 * blockDim.x) {  // four slots per thread in flight
-            uint32_t cn[4], lo[4], hi[4];
-            ulonglong2 o[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const uint32_t i = i0 + u * blockDim.x;
-                const bool in = i < in_use;
-                lo[u] = in ? g_acc[3 * i] : 0u;
-                hi[u] = in ? g_acc[3 * i + 1] : 0u;
-                cn[u] = in ? g_acc[3 * i + 2] : 0u;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) o[u] = held && (cn[u] | lo[u] | hi[u]) ? img[i0 + u * blockDim.x] : make_ulonglong2(0, 0);
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (i0 + u * blockDim.x >= L::SLOTS || (held && (cn[u] | lo[u] | hi[u]) == 0)) continue;
-                const ull nlo = o[u].x + ((ull)lo[u] | ((ull)hi[u] << 32));
-                img[i0 + u * blockDim.x] = make_ulonglong2(nlo, o[u].y + (ull)cn[u] + ((nlo < o[u].x ? 1ull : 0ull) << HI_SHIFT));
-            }
-        }
-    }
+    const RingBars ring = {s_full, s_empty, &s_abort};
+    if (!HOT)
+        scatter_cta<LP, DIR_NONE>(p, c, smem_raw, ring);
+    else if (SCATTER_RING_STAGES == 0 && p.t.ctl->words != 0)
+        scatter_cta<LP, DIR_WORDS>(p, c, smem_raw, ring);
+    else
+        scatter_cta<LP, DIR_TAGS>(p, c, smem_raw, ring);
 }
 
 template <uint32_t LP>
@@ -773,7 +870,7 @@ cudaError_t prepare_lp() {
 
 template <uint32_t LP>
 cudaError_t launch_lp(const IngestParams& p, bool hot, int grid, cudaStream_t stream) {
-    return launch_chained(hot ? scatter_kernel<LP, true> : scatter_kernel<LP, false>, (uint32_t)grid, SCATTER_THREADS, Smem<LP>::TOTAL, stream, p);
+    return launch_chained(hot ? scatter_kernel<LP, true> : scatter_kernel<LP, false>, (uint32_t)grid, SCATTER_THREADS, smem_total<LP>(), stream, p);
 }
 
 }  // namespace

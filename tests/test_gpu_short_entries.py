@@ -1,0 +1,74 @@
+"""Short spill entries (8 bytes) and the directory's words form against the oracle: bit for bit, at the edges of their fields."""
+import numpy as np
+import pytest
+
+import oracle
+from tests.helpers import sorted_by_key
+from tracegen.layout import RECORD_DTYPE
+
+pytestmark = pytest.mark.gpu
+PEAK_BW, PEAK_FLOPS = 8e12, [1e15] * 8
+
+
+def check(agg, o):
+    assert sorted_by_key(agg.finalize_numpy(PEAK_BW, PEAK_FLOPS)).tobytes() == o.finalize(PEAK_BW, PEAK_FLOPS).tobytes()
+
+
+def ingest(agg, recs, start=0):
+    import torch
+    agg.ingest(torch.from_numpy(recs[start:].view(np.uint8).reshape(-1)).cuda(), n=len(recs) - start)
+
+
+@pytest.mark.parametrize("max_keys", [2_000_000, 4_000_000, 9_000_000, 18_000_000, 1 << 25])      # 256 ... 4 096 partitions
+@pytest.mark.parametrize("n_apps,n_phases,n_ops", [(1, 1, 1), (4, 2, 64), (4096, 2, 65), (300, 3, 128), (4096, 4, 256), (17, 8, 256), (4097, 2, 64)])
+def test_every_field_at_its_edges(max_keys, n_apps, n_phases, n_ops):
+    """Durations on both sides of every power of two (the longer ones take a second entry, from 2^16 to 2^31 on), the first
+    and last application, phase and operator, shapes at the ends of their range, and three records whose operator is
+    larger than any that a sample is likely to see."""
+    import paper_2607_14541_b200 as p
+    rng = np.random.default_rng(max_keys + n_apps)
+    n, pool = 400_003, 60_000
+    recs = np.zeros(n, dtype=RECORD_DTYPE)
+    shapes = rng.integers(0, 1 << 32, pool, dtype=np.uint64).astype(np.uint32)
+    shapes[:4] = (0, 1, 0x80000000, 0xFFFFFFFF)
+    pick = np.where(rng.random(n) < 0.3, rng.integers(0, 300, n), rng.integers(0, pool, n))
+    recs["shape_id"], recs["op_id"] = shapes[pick], pick % n_ops
+    recs["app_id"] = np.where(rng.random(n) < 0.2, n_apps - 1, rng.integers(0, n_apps + 1, n))      # one in n_apps + 1 does not exist
+    recs["phase"] = rng.integers(0, n_phases, n)
+    edge = (np.uint64(1) << rng.integers(0, 33, n, dtype=np.uint64)) - rng.integers(0, 2, n, dtype=np.uint64)
+    recs["duration_ns"] = np.minimum(edge, 0xFFFFFFFF).astype(np.uint32)
+    recs["op_id"][[777, 200_000, n - 1]] = (n_ops, 0x0FFF, 0xFFFF)
+    weights = rng.integers(0, 1 << 20, n_apps).astype(np.uint32)
+    weights[-1] = 0xFFFFFFFF
+    agg = p.Aggregator(weights, n_phases, max_keys)
+    o = oracle.Oracle(weights, n_phases)
+    for part in np.array_split(recs, [280_000]):                   # the second call meets the first one's keys, drained once
+        ingest(agg, part)
+        o.ingest(part, threads=4)
+        check(agg, o)
+    st = agg.stats()
+    assert st["n_dropped"] == 0 and st["n_spilled"] <= st["n_valid"] and st["n_valid"] + st["n_rejected"] == n
+
+
+@pytest.mark.parametrize("n_keys", [1, 3, 40])
+def test_crowded_partitions_and_full_buffers(n_keys):
+    """A second call whose records all go to a few keys that the directory does not hold: the partition pass sums equal
+    entries first, and the buffers of one or two entries a record run over into the exact slow path."""
+    import paper_2607_14541_b200 as p
+    rng = np.random.default_rng(n_keys)
+    n = (1 << 22) + 4096
+    recs = np.zeros(n + (1 << 20), dtype=RECORD_DTYPE)
+    recs["app_id"] = rng.integers(0, 3, len(recs))
+    recs["op_id"], recs["shape_id"] = rng.integers(0, 5, len(recs)), rng.integers(0, 8_000, len(recs))
+    recs["duration_ns"] = rng.choice(np.array([7, 0x00FFFFFF, 0x0FFFFFFF, 0xFFFFFFFF], dtype=np.uint32), len(recs))
+    late = recs[n:]
+    late["op_id"], late["shape_id"] = 6, 100_000 + rng.integers(0, n_keys, len(late))
+    weights = np.array([1, 0xFFFF, 77], dtype=np.uint32)
+    agg = p.Aggregator(weights, 1, 60_000)
+    o = oracle.Oracle(weights, 1)
+    o.ingest(recs, threads=8)
+    ingest(agg, recs[:n])
+    ingest(agg, recs, n)
+    check(agg, o)
+    st = agg.stats()
+    assert st["n_valid"] == len(recs) and (st["n_overflow"] > 0) == (n_keys < 40)
