@@ -123,15 +123,22 @@ void compute_layout(const atrex_agg_config_t* c, size_t smem_optin, int n_sms, L
         while (b < 32 && (1u << b) < n) ++b;
         return b;
     };
-    L->fmt = ShortFormat{0, 0, 0, 0};
+    memset(&L->fmt, 0, sizeof(L->fmt));
     if (with_weights) {
-        const uint32_t phase_bits = bits_for(c->n_phases), app_bits = bits_for(c->n_apps);
-        for (uint32_t op_bits = DIR_ID_BITS - 1 - phase_bits; op_bits >= 8; --op_bits) {
-            const uint32_t low = 63 - (32 - L->lp) - phase_bits - op_bits, dur_bits = (low < 32 ? low : 32) - app_bits;
-            L->fmt = ShortFormat{phase_bits + op_bits, op_bits, app_bits, dur_bits < 31 ? dur_bits : 31};
-            if (dur_bits >= 20) break;
+        ShortFormat& f = L->fmt;
+        f.phase_bits = bits_for(c->n_phases);
+        f.app_bits = bits_for(c->n_apps);
+        const uint32_t in_high = L->lp - 1 < DIR_ID_BITS - 1 ? L->lp - 1 : DIR_ID_BITS - 1;
+        uint32_t op_bits = DIR_ID_BITS - 1 - f.phase_bits, rest_bits = 0;
+        for (;; --op_bits) {
+            rest_bits = f.phase_bits + op_bits > in_high ? f.phase_bits + op_bits - in_high : 0;
+            f.dur_bits = 32 - rest_bits - f.app_bits;
+            if (f.dur_bits >= 20 || op_bits == 8) break;
         }
-        if (L->fmt.dur_bits < 16) L->fmt = ShortFormat{0, 0, 0, 0};
+        f.rest_shift = rest_bits ? 32 - rest_bits : 31;
+        f.rest_mask = rest_bits ? ~0u << f.rest_shift : 0u;
+        if (f.dur_bits > 31) f.dur_bits = 31;
+        f.max_ops = 1u << op_bits;
     }
     size_t o = 0;
     // (control block, spill counts and table are neighbours: a reset clears them in one piece)
@@ -466,6 +473,8 @@ static int drain_spill(atrex_agg* h, bool force, cudaStream_t s) {
     q.cap = h->L.cap;
     q.short_cap = h->L.cap / 2 * 3;
     q.fmt = h->L.fmt;
+    // (a record that does not fit goes to the table by itself, ten to forty times slower)
+    q.misfit_max = (uint32_t)(h->n_records / 256 < (1u << 18) ? 1u << 18 : (h->n_records / 256 < 0xFFFFFFFFull ? h->n_records / 256 : 0xFFFFFFFFull));
     q.n_apps = h->cfg.n_apps;
     q.app_w = h->d_appw;
     q.queue = h->queue;
@@ -516,7 +525,7 @@ static int ingest_launch(atrex_agg* h, const atrex_record_t* recs, uint64_t n, c
         b.n_apps = h->cfg.n_apps;
         b.n_phases = h->cfg.n_phases;
         b.hot_keys = h->hot_keys;
-        b.op_bits = h->L.fmt.dur_bits ? h->L.fmt.op_bits : 0;
+        b.max_ops = h->L.fmt.max_ops;
         b.hot_slots = h->L.hot_slots;
         for (int words = 0; words < 2; ++words) {
             b.slots[words][0] = scatter_slots(h->L.lp, words != 0);
@@ -896,7 +905,7 @@ int atrex_agg_stats(atrex_agg_t* h, atrex_stats_t* out, void* stream) {
     out->n_spilled = c->n_spilled;
     out->n_overflow = c->n_overflow;
     out->max_spill_fill = c->max_fill;
-    out->spill_cap = c->words ? h->L.cap / 2 * 3 : h->L.cap;
+    out->spill_cap = c->form == FORM_SHORT ? h->L.cap / 2 * 3 : h->L.cap;
     out->n_drains = c->n_drains;
     return device_status_to_error(c);
 }

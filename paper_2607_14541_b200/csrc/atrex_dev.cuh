@@ -57,6 +57,11 @@ constexpr uint32_t PICK_NONE = 0xFFFFFFFFu;
 // (equal lanes are then combined first); from 3/8 on the key is best taken out before anything else.
 constexpr ull SKEW_NONE = 0, SKEW_COMBINE = 1, SKEW_DOMINATED = 2;
 
+// The spill entries' form and with it the directory's, chosen by the directory build (0, after a reset: 12-byte entries and
+// the directory's tags form, if there is one).
+constexpr ull FORM_LONG = 0, FORM_SHORT = 1;
+constexpr ull FORM_LONG_ONLY = 2;   // 12-byte entries and no more directory (too many records did not fit its words)
+
 struct Control {
     ull status;
     ull n_rejected;
@@ -67,7 +72,9 @@ struct Control {
     ull work_status;           // ST_WORK_* bits of the last work-table load
     ull hot_skew;              // SKEW_*: how the scatter pass deals with the most frequent key
     ull prefetch;              // 1: the directory holds enough of the sample for the scatter pass to prefetch records
-    ull words;                 // 1: the directory is in its words form (every operator of the sample fits)
+    ull form;                  // FORM_*: of the spill entries and the directory
+    ull n_misfit;              // records whose operator does not fit that form
+    ull rests;                 // 1: short entries since the last drain hold identities with a rest
     ull top_key;               // the most frequent key (SKEW_DOMINATED)
     ull n_spilled;             // records routed through the spill buffers
     ull n_overflow;            // records that found their spill buffer full (slow exact path)
@@ -131,7 +138,7 @@ __device__ __forceinline__ uint32_t dir_bucket(uint32_t h, uint32_t phase, uint3
     return __umulhi(dir_mix(h, phase, mult), n_buckets);
 }
 
-// The partition pass's own form of a key, unique inside a partition: bit 63 set (so that 0 can mean
+// The partition pass's form of a key where entries are long, unique inside a partition: bit 63 set (so that 0 can mean
 // an empty slot), phase << 16 | operator in bits 32..55, the 32-bit hash below.
 constexpr ull CKEY_MARK = 1ull << 63;
 __device__ __forceinline__ ull ckey_of(uint32_t khi24, uint32_t h) { return CKEY_MARK | ((ull)khi24 << 32) | h; }
@@ -148,17 +155,22 @@ __device__ __forceinline__ ull ckey_of_spill(ull a, uint32_t b, uint32_t part, u
     return ckey_of(((b >> 24) << 16) | (uint32_t)(a >> 48), (part << (32 - lp)) | (b & (0xFFFFFFFFu >> lp)));
 }
 
-// A short entry (8 bytes), where phase and operator fit `id_bits` together and the weights the kernels' shared memory:
-// from the top bit on
-//   continuation (1) | phase << op_bits | operator (id_bits) | hash bits below the partition's (32 - lp) | application | duration
-// with the last two, `app_bits` and `dur_bits` wide, at the bottom of the low word (what lies between is zero).  A longer
-// duration's rest follows as a continuation, which adds to the time and not to the count.
+// A short entry (8 bytes), where the application fits `app_bits` and phase and operator the DIR_ID_BITS - 1 of a directory
+// word; identity = operator << phase_bits | phase.
+//   high word  continuation (1) | hash bits below the partition's (32 - lp) | low lp - 1 bits of the identity
+//   low word   the rest of the identity | application | duration (dur_bits)
+// A longer duration's rest follows as a continuation, which adds to the time and not to the count.  As long as no operator
+// among the entries is so large that its identity has a rest, the high word alone identifies a key in its partition.
 struct ShortFormat {
-    uint32_t id_bits, op_bits, app_bits, dur_bits;   // dur_bits = 0: no short entries
-    __host__ __device__ __forceinline__ uint32_t shift() const { return 1u + id_bits; }
-    __device__ __forceinline__ uint32_t dur_mask() const { return (1u << dur_bits) - 1u; }
-    __device__ __forceinline__ uint32_t app_mask() const { return (1u << app_bits) - 1u; }
+    uint32_t phase_bits, app_bits, dur_bits;   // dur_bits = 0: no short entries
+    uint32_t rest_shift, rest_mask;            // the identity's rest in the low word
+    uint32_t max_ops;                          // operators that fit
+    __host__ __device__ __forceinline__ uint32_t dur_mask() const { return (1u << dur_bits) - 1u; }
+    __host__ __device__ __forceinline__ uint32_t app_mask() const { return (1u << app_bits) - 1u; }
 };
+// A directory word holds the top bits of what the bucket hash leaves over and, below them, phase and operator.  All ones
+// there mark an empty slot, so that those two have one bit less, in short entries too.
+constexpr uint32_t DIR_ID_BITS = 12, DIR_ID_MASK = (1u << DIR_ID_BITS) - 1u;
 constexpr uint32_t SHORT_ENTRY_BYTES = 8;
 constexpr uint32_t SHORT_CONTINUATION = 0x80000000u;   // in the high word
 
@@ -208,8 +220,8 @@ constexpr ull NO_INDEX = ~0ull;
 
 __device__ __forceinline__ uint32_t part_of(uint32_t h, uint32_t lp) { return h >> (32 - lp); }  // lp >= 1
 
-// Probe sequence of a key inside its partition (double hashing over slot pairs): it starts at the
-// pair holding local_of() and moves on by one of eight strides chosen by other hash bits; inside a
+// Probe sequence of a key inside its partition (double hashing over slot pairs): it starts at
+// first_pair() and moves on by one of eight strides chosen by other hash bits; inside a
 // pair the even slot comes first.  The strides are coprime to the number of pairs, so the sequence
 // visits every pair once.  Every prober -- this file's global-memory path and the partition pass's
 // shared-memory path -- follows the same order, and a key sits at the first slot of its sequence
@@ -217,12 +229,16 @@ __device__ __forceinline__ uint32_t part_of(uint32_t h, uint32_t lp) { return h 
 // here (up to 0.7) made the slowest of a warp's probes several times the average, do not form.
 // The phase, which the partition choice ignores, is mixed into the start so that the phases of one
 // (operator, shape) do not pile up on the same pair.
-__device__ __forceinline__ uint32_t local_of(uint32_t h, uint32_t phase, uint32_t C) {
-    return __umulhi((h ^ (phase * 0x9E3779B9u)) * 0x85EBCA6Bu, C);
+//
+// Both come from the key's window: the 20 hash bits below the partition's, at the top of a word.  (Those a short entry
+// holds side by side: the partition pass gets at them with a shift and a mask.)
+constexpr uint32_t WINDOW_BITS = 20, WINDOW_MASK = ~0u << (32 - WINDOW_BITS);
+__device__ __forceinline__ uint32_t window_of(uint32_t h, uint32_t lp) { return (h << lp) & WINDOW_MASK; }
+__device__ __forceinline__ uint32_t first_pair(uint32_t window, uint32_t phase, uint32_t C) {
+    return __umulhi(window + phase * 0x9E3779B9u, C) & ~1u;
 }
-__device__ __forceinline__ uint32_t stride_index(uint32_t h) { return (h >> 3) & 7u; }
-__device__ __forceinline__ uint32_t stride_of(const TableRef& t, uint32_t index) {
-    return (uint32_t)(t.strides >> (8 * index)) & 0xFFu;
+__device__ __forceinline__ uint32_t pair_stride(const TableRef& t, uint32_t window) {      // in slots
+    return 2u * ((uint32_t)(t.strides >> (8 * ((window >> (32 - WINDOW_BITS)) & 7u))) & 0xFFu);
 }
 
 // Find (or claim) the slot of `key` directly in HBM.  Returns NO_INDEX when the key's
@@ -231,8 +247,8 @@ __device__ __forceinline__ uint32_t stride_of(const TableRef& t, uint32_t index)
 __device__ __forceinline__ ull find_or_claim(const TableRef& t, ull key, uint32_t h) {
     const ull skey = ~key;
     const ull base = (ull)part_of(h, t.lp) * t.C;
-    uint32_t s = local_of(h, (uint32_t)(key >> 48), t.C) & ~1u;
-    const uint32_t advance = 2u * stride_of(t, stride_index(h));
+    const uint32_t window = window_of(h, t.lp), advance = pair_stride(t, window);
+    uint32_t s = first_pair(window, (uint32_t)(key >> 48), t.C);
     for (uint32_t probe = 0; probe < t.C; ++probe) {
         ull* kp = t.keys + ATREX_INDEX(base + s, (ull)t.C << t.lp, t.ctl);
         ull k = ld_relaxed(kp);

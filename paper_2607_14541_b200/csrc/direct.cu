@@ -93,7 +93,7 @@ __device__ __forceinline__ void flush_slots(const TableRef& t, const ull (&key)[
     ull idx[4], found[4], old[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-        idx[u] = (ull)part_of(h[u], t.lp) * t.C + (local_of(h[u], (uint32_t)(key[u] >> 48), t.C) & ~1u);
+        idx[u] = (ull)part_of(h[u], t.lp) * t.C + first_pair(window_of(h[u], t.lp), (uint32_t)(key[u] >> 48), t.C);
         found[u] = count[u] ? ld_relaxed(t.keys + ATREX_INDEX(idx[u], (ull)t.C << t.lp, t.ctl)) : 0ull;
     }
 #pragma unroll

@@ -165,8 +165,9 @@ __global__ void __launch_bounds__(THREADS) totals_kernel(TableRef tab, ull n_slo
 // linear probing the longest of a warp's 32 probe sequences -- which is what the warp waits for --
 // was several times the average.
 __device__ __forceinline__ uint32_t work_stride(const WorkRef& w, uint32_t h) {
-    return (uint32_t)(w.strides >> (8 * stride_index(h))) & 0xFFu;
+    return (uint32_t)(w.strides >> (8 * ((h >> 3) & 7u))) & 0xFFu;
 }
+__device__ __forceinline__ uint32_t work_start(const WorkRef& w, uint32_t h) { return __umulhi(h * 0x85EBCA6Bu, w.Cw); }
 __device__ __forceinline__ double roofline_time(const WorkRef& w, const atrex_hw_peaks_t& pk, ull key) {
     const double qnan = __longlong_as_double(0x7FF8000000000000ll);
     if (w.table == nullptr) return qnan;
@@ -174,7 +175,7 @@ __device__ __forceinline__ double roofline_time(const WorkRef& w, const atrex_hw
     ull skey = ~pair;
     const uint32_t h = hash32(pair);
     const WorkSlot* part = w.table + (ull)part_of(h, w.lp) * w.Cw;
-    uint32_t s = local_of(h, 0u, w.Cw);
+    uint32_t s = work_start(w, h);
     const uint32_t advance = work_stride(w, h);
     for (uint32_t probe = 0; probe < w.Cw; ++probe) {
         const WorkSlot* e = part + s;
@@ -301,7 +302,7 @@ __global__ void __launch_bounds__(256) work_insert_kernel(const atrex_work_t* ro
         ull skey = ~pair;
         const uint32_t h = hash32(pair);
         WorkSlot* part = w.table + (ull)part_of(h, w.lp) * w.Cw;
-        uint32_t s = local_of(h, 0u, w.Cw);
+        uint32_t s = work_start(w, h);
         const uint32_t advance = work_stride(w, h);
         bool done = false;
         for (uint32_t probe = 0; probe < w.Cw && !done; ++probe) {

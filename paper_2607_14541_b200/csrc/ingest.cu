@@ -36,9 +36,9 @@ __constant__ uint32_t DIR_MULTS[4] = {0xC2B2AE35u, 0x27D4EB2Fu, 0x165667B1u, 0x9
 // Shared memory is addressed explicitly through 32-bit shared-window addresses in the hot
 // loops: one integer add per access instead of generic 64-bit pointer arithmetic.
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ ulonglong2 lds_v2u64(uint32_t a) {
-    ulonglong2 v;
-    asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"(a));
+__device__ __forceinline__ uint2 lds_v2u32(uint32_t a) {
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a));
     return v;
 }
 __device__ __forceinline__ uint32_t atoms_add(uint32_t a, uint32_t v) {
@@ -55,6 +55,11 @@ __device__ __forceinline__ void reds_or(uint32_t a, uint32_t v) {
 __device__ __forceinline__ uint32_t atoms_exch(uint32_t a, uint32_t v) {
     uint32_t o;
     asm volatile("atom.shared.exch.b32 %0, [%1], %2;" : "=r"(o) : "r"(a), "r"(v) : "memory");
+    return o;
+}
+__device__ __forceinline__ uint32_t atoms_cas32(uint32_t a, uint32_t expected, uint32_t desired) {
+    uint32_t o;
+    asm volatile("atom.shared.cas.b32 %0, [%1], %2, %3;" : "=r"(o) : "r"(a), "r"(expected), "r"(desired) : "memory");
     return o;
 }
 __device__ __forceinline__ ull atoms_cas64(uint32_t a, ull expected, ull desired) {
@@ -143,8 +148,8 @@ __global__ void __launch_bounds__(FOLD_WARPS * 32) hot_fold_kernel(const ull* ho
 // when the segment could not take another batch); then write the deltas back.
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
-// Shared-window addresses of the partition pass's arrays: keys ull[C] (the pass's own key form, 0 =
-// empty), acc {u32 low limb, u32 count | NEW_KEY_FLAG}[C], a1 u32[C] (high limb).
+// Shared-window addresses of the partition pass's arrays: keys[C] (in the form of the entries, 0 = empty; ull, or
+// u32 where entries are tight), acc {u32 low limb, u32 count | NEW_KEY_FLAG}[C], a1 u32[C] (high limb).
 struct PartSmem {
     uint32_t keys, acc, a1;
     uint32_t weights;          // short entries: u32[n_apps]
@@ -161,27 +166,98 @@ __device__ __forceinline__ uint4 lds_v4u32(uint32_t a) {
     return v;
 }
 
+// FORM_TIGHT: short entries of whose identities none has a rest.
+constexpr ull FORM_TIGHT = FORM_LONG_ONLY + 1;
+
+// The keys as the pass holds them.  Long entries: ckey_of.  Short ones: the words of an entry without its payload, bit 63
+// set; tight ones the high word alone.  Keys that such an entry cannot have (operators that do not fit) are in the table
+// too: they take their slots as something that no entry's key equals.
+template <ull FORM>
+struct FormKey {
+    uint32_t hi, lo;           // tight: lo = 0
+};
+template <ull FORM>
+constexpr uint32_t KEY_BYTES = FORM == FORM_TIGHT ? 4 : 8;
+template <ull FORM>
+constexpr uint32_t ENTRY_BYTES = FORM == FORM_LONG ? SPILL_ENTRY_BYTES : SHORT_ENTRY_BYTES;
+template <ull FORM>
+__device__ __forceinline__ FormKey<FORM> form_key(const PartitionParams& q, ull key) {
+    if (FORM == FORM_LONG) {
+        const ull c = ckey_of_key(key);
+        return {(uint32_t)(c >> 32), (uint32_t)c};
+    }
+    const uint32_t khi = (uint32_t)(key >> 32), op = khi & 0xFFFFu, phase = (khi >> 16) & 0xFFu, h = hash32(op, (uint32_t)key);
+    if (op >= q.fmt.max_ops || phase >> q.fmt.phase_bits != 0 || (FORM == FORM_TIGHT && (op << q.fmt.phase_bits) >> (q.t.lp - 1u) != 0)) return {1u, FORM == FORM_TIGHT ? 0u : h};
+    const uint32_t id = (op << q.fmt.phase_bits) | phase, in_high = (1u << (q.t.lp - 1u)) - 1u;
+    return {SHORT_CONTINUATION | ((h << q.t.lp) >> 1) | (id & in_high), FORM == FORM_TIGHT ? 0u : (id >> (q.t.lp - 1u)) << q.fmt.rest_shift};
+}
+template <ull FORM>
+__device__ __forceinline__ ull key_of_form(const PartitionParams& q, FormKey<FORM> k, uint32_t part) {
+    if (FORM == FORM_LONG) return key_of_ckey(((ull)k.hi << 32) | k.lo);
+    const uint32_t rest = FORM == FORM_TIGHT ? 0u : (k.lo & q.fmt.rest_mask) >> q.fmt.rest_shift;
+    const uint32_t id = (k.hi & ((1u << (q.t.lp - 1u)) - 1u)) | (rest << (q.t.lp - 1u)), op = id >> q.fmt.phase_bits;
+    const uint32_t h = (part << (32 - q.t.lp)) | ((k.hi << 1) >> q.t.lp);
+    return pack_key(id & ((1u << q.fmt.phase_bits) - 1u), op, shape_of_hash(h, op));
+}
+template <ull FORM>
+__device__ __forceinline__ uint32_t window_of_form(const PartitionParams& q, FormKey<FORM> k) {
+    return FORM == FORM_LONG ? window_of(k.lo, q.t.lp) : (k.hi << 1) & WINDOW_MASK;
+}
+template <ull FORM>
+__device__ __forceinline__ uint32_t phase_of_form(const PartitionParams& q, FormKey<FORM> k) {
+    return FORM == FORM_LONG ? (k.hi >> 16) & 0xFFu : k.hi & ((1u << q.fmt.phase_bits) - 1u);
+}
+
+// What a look at a pair of slots (the even one at `slot`) sees.
+struct PairLook {
+    bool first, second;            // the key is there
+    bool first_free, second_free;
+};
+template <ull FORM>
+__device__ __forceinline__ PairLook look_at(const PartSmem& m, uint32_t slot, FormKey<FORM> k) {
+    if (FORM == FORM_TIGHT) {
+        const uint2 v = lds_v2u32(m.keys + slot * 4u);
+        return {v.x == k.hi, v.y == k.hi, v.x == 0, v.y == 0};
+    }
+    const uint4 v = lds_v4u32(m.keys + slot * 8u);
+    return {v.x == k.lo && v.y == k.hi, v.z == k.lo && v.w == k.hi, v.y == 0, v.w == 0};
+}
+// Claims a free slot.  True: the key is there now (its own claim, noted for the write-back, or another lane's).
+template <ull FORM>
+__device__ __forceinline__ bool claim(const PartSmem& m, uint32_t slot, FormKey<FORM> k) {
+    bool mine, there;
+    if (FORM == FORM_TIGHT) {
+        const uint32_t old = atoms_cas32(m.keys + slot * 4u, 0u, k.hi);
+        mine = old == 0;
+        there = mine || old == k.hi;
+    } else {
+        const ull skey = ((ull)k.hi << 32) | k.lo, old = atoms_cas64(m.keys + slot * 8u, 0ull, skey);
+        mine = old == 0;
+        there = mine || old == skey;
+    }
+    if (mine) reds_or(m.acc + slot * 8u + 4u, NEW_KEY_FLAG);
+    return there;
+}
+
 // General probe, one entry per lane (busy = this lane has one): walks the key's probe sequence from
 // the pair at `slot`, claims the first free slot if the key is not there.  Warp-convergent.  Returns
 // the key's slot, or PROBE_FAILED when the partition has no room.
 constexpr uint32_t PROBE_FAILED = 0xFFFFFFFFu;
 
-__device__ __forceinline__ uint32_t probe_general(const PartSmem& m, ull skey, uint32_t slot, uint32_t advance, bool busy, uint32_t count,
+template <ull FORM>
+__device__ __forceinline__ uint32_t probe_general(const PartSmem& m, FormKey<FORM> key, uint32_t slot, uint32_t advance, bool busy, uint32_t count,
                                                   uint32_t C, Control* ctl) {
     uint32_t steps = 0;
     while (__any_sync(0xFFFFFFFFu, busy)) {
         if (busy) {
-            const ulonglong2 kk = lds_v2u64(m.keys + ATREX_INDEX(slot, C - 1u, ctl) * 8);
-            const bool hit1 = kk.y == skey;
-            if (kk.x == skey || hit1) {
-                slot += hit1 ? 1u : 0u;
+            const PairLook look = look_at(m, ATREX_INDEX(slot, C - 1u, ctl), key);
+            if (look.first || look.second) {
+                slot += look.second ? 1u : 0u;
                 busy = false;
-            } else if (kk.x == 0 || kk.y == 0) {
+            } else if (look.first_free || look.second_free) {
                 // claim the first empty slot of the pair; a lost race re-reads the pair
-                const uint32_t at = slot + (kk.x == 0 ? 0u : 1u);
-                const ull old = atoms_cas64(m.keys + at * 8, 0ull, skey);
-                if (old == 0) reds_or(m.acc + at * 8 + 4, NEW_KEY_FLAG);
-                if (old == 0 || old == skey) {
+                const uint32_t at = slot + (look.first_free ? 0u : 1u);
+                if (claim(m, at, key)) {
                     slot = at;
                     busy = false;
                 }
@@ -225,43 +301,40 @@ __device__ __forceinline__ void part_accumulate(const PartSmem& m, uint32_t slot
     }
 }
 
-// Where the entries are: their size, their buffers' pitch.
+// Where a sub-buffer's entries are.
 __device__ __forceinline__ const unsigned char* entries_of(const PartitionParams& q, ull sb) {
     return q.spill + sb * q.cap * SPILL_ENTRY_BYTES;     // (a buffer of short entries takes as many bytes)
 }
-template <bool SHORT>
-constexpr uint32_t ENTRY_BYTES = SHORT ? SHORT_ENTRY_BYTES : SPILL_ENTRY_BYTES;
-
 // The first 256 entries (24 or 16 lines) of sub-buffer `sb` towards L2, as far as it holds that many.
-template <bool SHORT>
+template <ull FORM>
 __device__ __forceinline__ void prefetch_entries(const PartitionParams& q, ull sb, uint32_t lane) {
-    const uint32_t bytes = q.spill_cnt[sb] * ENTRY_BYTES<SHORT>;
-    if (lane < 2u * ENTRY_BYTES<SHORT> && lane * 128u < bytes) prefetch_l2(entries_of(q, sb) + lane * 128u);
+    const uint32_t bytes = q.spill_cnt[sb] * ENTRY_BYTES<FORM>;
+    if (lane < 2u * ENTRY_BYTES<FORM> && lane * 128u < bytes) prefetch_l2(entries_of(q, sb) + lane * 128u);
 }
 
 // Settles a warp's queued entries, one per lane and round, by the general probe.  Other warps may
 // still be streaming: the probe copes with keys that appear meanwhile.  Called once the warp's share of
 // the partition's stream is through, and before a batch that might not fit the queue (a crowded
 // partition of new keys).  Not inlined: it runs a few times per partition and warp.
-__device__ __noinline__ void settle_queue(const TableRef t, const PartSmem m, const ulonglong2* my_queue, uint32_t qn_w, uint32_t C,
-                                          ull base, uint32_t lane);
+template <ull FORM>
+__device__ __noinline__ void settle_queue(const PartitionParams& q, const PartSmem m, const ulonglong2* my_queue, uint32_t qn_w, ull base, uint32_t lane);
 
 // A queued entry: {key, product}; bit 63 of the product word says that the key's first pair was full
 // of other keys when the entry was looked up, so its probe may start at the second pair; bit 62 that it is a continuation.
 constexpr ull QUEUED_SKIP_FIRST = 1ull << 63, QUEUED_CONTINUATION = 1ull << 62;
 
 // One batch of 128 entries of a sub-buffer, four consecutive ones (48 bytes; 32 if short) per lane.  FULL: the
-// batch is complete (no masks).  Keys are handled as their two 32-bit halves (kh: mark, phase,
-// operator; kl: hash).  Entry state is bit sets per lane -- `open` (present, slot not known yet), `hit`
+// batch is complete (no masks).  Entry state is bit sets per lane -- `open` (present, slot not known yet), `hit`
 // (slot known), `room` (the first pair of the probe sequence had a free slot when it was read).
-// part_bits = the partition's index in the hash's top bits, hmask = the hash bits below them.
-template <bool SHORT, bool CROWDED, bool FULL>
+template <ull FORM, bool CROWDED, bool FULL>
 __device__ __forceinline__ void stream_batch(const PartitionParams& q, const PartSmem& m, const unsigned char* src,
-                                             uint32_t part_bits, uint32_t hmask, uint32_t e0, uint32_t n_e, uint32_t C, ull base,
+                                             uint32_t part, uint32_t e0, uint32_t n_e, uint32_t C, ull base,
                                              ulonglong2* my_queue, uint32_t queue_cap_w, uint32_t& qn_w, uint32_t lane) {
-    uint32_t kh[4], kl[4], vlo[4], vhi[4], slot[4];
+    FormKey<FORM> key[4];
+    uint32_t vlo[4], vhi[4], slot[4];
     uint32_t open = 0, extra = 0;    // extra: continuations
-    if (SHORT) {
+    if (FORM != FORM_LONG) {
+        const ShortFormat& f = q.fmt;
         const uint32_t e = e0 + 4u * lane;
         uint32_t w[8];
         if (FULL || e < n_e) {       // (a buffer's capacity is a multiple of 16: a lane that holds any entry may read all 32 bytes)
@@ -276,17 +349,16 @@ __device__ __forceinline__ void stream_batch(const PartitionParams& q, const Par
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const uint32_t lo = w[2 * u], hi = w[2 * u + 1];
-            const uint32_t id = (hi & ~SHORT_CONTINUATION) >> (31u - q.fmt.id_bits), phase = id >> q.fmt.op_bits;
-            kh[u] = (0x80000000u | id) + phase * (0x10000u - (1u << q.fmt.op_bits));    // phase << 16 | operator
-            kl[u] = part_bits | (__funnelshift_l(lo, hi, 1u + q.fmt.id_bits) >> q.t.lp);
+            key[u].hi = hi | SHORT_CONTINUATION;
+            key[u].lo = FORM == FORM_TIGHT ? 0u : lo & f.rest_mask;
             const uint32_t more = hi >> 31;
-            const uint32_t dur = (lo & q.fmt.dur_mask()) << (more ? q.fmt.dur_bits : 0u);
-            const uint32_t app = ATREX_INDEX((lo >> q.fmt.dur_bits) & q.fmt.app_mask(), q.n_apps, q.t.ctl);
+            const uint32_t dur = (lo & f.dur_mask()) << (more ? f.dur_bits : 0u);
+            const uint32_t app = ATREX_INDEX((lo >> f.dur_bits) & f.app_mask(), q.n_apps, q.t.ctl);
             const ull v = (ull)lds_u32(m.weights + app * 4u) * dur;
             extra |= more << u;
             vlo[u] = (uint32_t)v;
             vhi[u] = (uint32_t)(v >> 32);
-            slot[u] = local_of(kl[u], phase, C) & ~1u;
+            slot[u] = first_pair(window_of_form(q, key[u]), phase_of_form(q, key[u]), C);
         }
     } else {
         // the lane's entries e, e + 1, e + 2, e + 3 (e a multiple of 4) as twelve words; in an even
@@ -307,11 +379,11 @@ __device__ __forceinline__ void stream_batch(const PartitionParams& q, const Par
         const uint32_t b[4] = {w[0].z, w[0].w, w[2].x, w[2].y};
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            kh[u] = 0x80000000u | ((b[u] >> 8) & 0x00FF0000u) | (ahi[u] >> 16);
-            kl[u] = part_bits | (b[u] & hmask);
+            key[u].hi = 0x80000000u | ((b[u] >> 8) & 0x00FF0000u) | (ahi[u] >> 16);
+            key[u].lo = (part << (32 - q.t.lp)) | (b[u] & (0xFFFFFFFFu >> q.t.lp));
             vlo[u] = alo[u];
             vhi[u] = ahi[u] & 0xFFFFu;
-            slot[u] = local_of(kl[u], b[u] >> 24, C) & ~1u;  // first pair of the probe sequence
+            slot[u] = first_pair(window_of_form(q, key[u]), b[u] >> 24, C);
         }
     }
     // First look, straight-line for all four entries: most keys sit in the first pair of slots of
@@ -319,13 +391,11 @@ __device__ __forceinline__ void stream_batch(const PartitionParams& q, const Par
     uint32_t hit = 0, room = 0, even_taken = 0;
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-        const uint4 kk = lds_v4u32(m.keys + ATREX_INDEX(slot[u], C - 1u, q.t.ctl) * 8);
-        const bool h0 = kk.x == kl[u] && kk.y == kh[u];
-        const bool h1 = kk.z == kl[u] && kk.w == kh[u];
-        if (h1) slot[u] |= 1u;
-        if (h0 || h1) hit |= 1u << u;
-        if (kk.w == 0) room |= 1u << u;
-        if (kk.y != 0) even_taken |= 1u << u;
+        const PairLook look = look_at(m, ATREX_INDEX(slot[u], C - 1u, q.t.ctl), key[u]);
+        if (look.second) slot[u] |= 1u;
+        if (look.first || look.second) hit |= 1u << u;
+        if (look.second_free) room |= 1u << u;
+        if (!look.first_free) even_taken |= 1u << u;
     }
     hit &= open;     // (an absent entry is a well-formed key too)
     open &= ~hit;
@@ -336,10 +406,7 @@ __device__ __forceinline__ void stream_batch(const PartitionParams& q, const Par
         for (int u = 0; u < 4; ++u) {
             if (open & room & (1u << u)) {
                 const uint32_t at = slot[u] + ((even_taken >> u) & 1u);
-                const ull skey = ((ull)kh[u] << 32) | kl[u];
-                const ull old = atoms_cas64(m.keys + at * 8, 0ull, skey);
-                if (old == 0) reds_or(m.acc + at * 8 + 4, NEW_KEY_FLAG);
-                if (old == 0 || old == skey) {
+                if (claim(m, at, key[u])) {
                     slot[u] = at;
                     hit |= 1u << u;
                     open &= ~(1u << u);
@@ -365,8 +432,8 @@ __device__ __forceinline__ void stream_batch(const PartitionParams& q, const Par
         for (int u = 0; u < 4; ++u) {
             if (open & (1u << u)) {
                 const ull v = vlo[u] | ((ull)vhi[u] << 32) | ((room >> u) & 1u ? 0ull : QUEUED_SKIP_FIRST) |
-                              (SHORT && ((extra >> u) & 1u) ? QUEUED_CONTINUATION : 0ull);
-                my_queue[ATREX_INDEX(qbase + before[u], queue_cap_w, q.t.ctl)] = make_ulonglong2(((ull)kh[u] << 32) | kl[u], v);
+                              (FORM != FORM_LONG && ((extra >> u) & 1u) ? QUEUED_CONTINUATION : 0ull);
+                my_queue[ATREX_INDEX(qbase + before[u], queue_cap_w, q.t.ctl)] = make_ulonglong2(((ull)key[u].hi << 32) | key[u].lo, v);
             }
         }
     }
@@ -384,7 +451,7 @@ __device__ __forceinline__ void stream_batch(const PartitionParams& q, const Par
         for (int u = 0; u < 4; ++u) {
             if ((hit & (1u << u)) != 0 && slot[u] == shared_slot) {
                 sum += (ull)vlo[u] | ((ull)vhi[u] << 32);
-                count += SHORT ? ~(extra >> u) & 1u : 1u;
+                count += FORM != FORM_LONG ? ~(extra >> u) & 1u : 1u;
                 hit &= ~(1u << u);
             }
         }
@@ -394,37 +461,37 @@ __device__ __forceinline__ void stream_batch(const PartitionParams& q, const Par
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u)
-        if (hit & (1u << u)) part_accumulate(m, slot[u], vlo[u], vhi[u], SHORT ? ~(extra >> u) & 1u : 1u, q.t.vals + base, C, q.t.ctl);
+        if (hit & (1u << u)) part_accumulate(m, slot[u], vlo[u], vhi[u], FORM != FORM_LONG ? ~(extra >> u) & 1u : 1u, q.t.vals + base, C, q.t.ctl);
 }
 
-__device__ __noinline__ void settle_queue(const TableRef t, const PartSmem m, const ulonglong2* my_queue, uint32_t qn_w, uint32_t C,
-                                          ull base, uint32_t lane) {
+template <ull FORM>
+__device__ __noinline__ void settle_queue(const PartitionParams& q, const PartSmem m, const ulonglong2* my_queue, uint32_t qn_w, ull base, uint32_t lane) {
+    const uint32_t C = q.t.C;
     __syncwarp();   // the queue was written by other lanes of this warp
     for (uint32_t i0 = 0; i0 < qn_w; i0 += 32u) {
         const bool serving = i0 + lane < qn_w;
         const ulonglong2 ent = serving ? __ldcg(my_queue + i0 + lane) : make_ulonglong2(0, 0);
-        const uint32_t hh = (uint32_t)ent.x;
-        const uint32_t advance = 2u * stride_of(t, stride_index(hh));
-        uint32_t start = local_of(hh, ckey_phase(ent.x), C) & ~1u;
+        const FormKey<FORM> key = {(uint32_t)(ent.x >> 32), (uint32_t)ent.x};
+        const uint32_t window = window_of_form(q, key), advance = pair_stride(q.t, window);
+        uint32_t start = first_pair(window, phase_of_form(q, key), C);
         if (ent.y & QUEUED_SKIP_FIRST) {
             start += advance;
             if (start >= C) start -= C;
         }
         const uint32_t count = ent.y & QUEUED_CONTINUATION ? 0u : 1u;
-        const uint32_t found = probe_general(m, ent.x, start, advance, serving, count, C, t.ctl);
+        const uint32_t found = probe_general(m, key, start, advance, serving, count, C, q.t.ctl);
         if (serving && found != PROBE_FAILED)
-            part_accumulate(m, found, (uint32_t)ent.y, (uint32_t)(ent.y >> 32) & 0xFFFFu, count, t.vals + base, C, t.ctl);
+            part_accumulate(m, found, (uint32_t)ent.y, (uint32_t)(ent.y >> 32) & 0xFFFFu, count, q.t.vals + base, C, q.t.ctl);
     }
     __syncwarp();   // the queue may be overwritten from here on
 }
 
 // A warp's share of a partition's entries: sub-buffers warp, warp + n_warps, ...  Returns how many wait in its queue.
-template <bool SHORT, bool CROWDED>
+template <ull FORM, bool CROWDED>
 __device__ __forceinline__ uint32_t stream_share(const PartitionParams& q, const PartSmem& m, uint32_t part, ulonglong2* my_queue, uint32_t queue_cap_w,
                                                  uint32_t warp, uint32_t n_warps, uint32_t lane) {
     const uint32_t C = q.t.C;
     const ull base = (ull)part * C;
-    const uint32_t part_bits = part << (32 - q.t.lp), hmask = 0xFFFFFFFFu >> q.t.lp;
     uint32_t qn_w = 0;  // entries in this warp's queue segment (warp-uniform)
     for (uint32_t g = warp; g < q.n_groups; g += n_warps) {
         const ull sb = ((ull)g << q.t.lp) + part;
@@ -433,18 +500,18 @@ __device__ __forceinline__ uint32_t stream_share(const PartitionParams& q, const
         // Short-distance L2 prefetch, a fixed window of 256 entries per warp (a longer reach gets
         // evicted before use: all warps of all CTAs together must stay well inside L2): the head of
         // this warp's next sub-buffer now, and inside the loop the lines two batches ahead.
-        if (g + n_warps < q.n_groups) prefetch_entries<SHORT>(q, ((ull)(g + n_warps) << q.t.lp) + part, lane);
+        if (g + n_warps < q.n_groups) prefetch_entries<FORM>(q, ((ull)(g + n_warps) << q.t.lp) + part, lane);
         for (uint32_t e0 = 0; e0 < n_e; e0 += 128) {
-            if (lane < ENTRY_BYTES<SHORT> && (e0 + 256u) * ENTRY_BYTES<SHORT> + lane * 128u < n_e * ENTRY_BYTES<SHORT>)
-                prefetch_l2(buf + (e0 + 256u) * ENTRY_BYTES<SHORT> + lane * 128u);
+            if (lane < ENTRY_BYTES<FORM> && (e0 + 256u) * ENTRY_BYTES<FORM> + lane * 128u < n_e * ENTRY_BYTES<FORM>)
+                prefetch_l2(buf + (e0 + 256u) * ENTRY_BYTES<FORM> + lane * 128u);
             if (qn_w + 128u > queue_cap_w) {   // (warp-uniform) the next batch might not fit the queue
-                settle_queue(q.t, m, my_queue, qn_w, C, base, lane);
+                settle_queue<FORM>(q, m, my_queue, qn_w, base, lane);
                 qn_w = 0;
             }
             if (e0 + 128u <= n_e)
-                stream_batch<SHORT, CROWDED, true>(q, m, buf, part_bits, hmask, e0, n_e, C, base, my_queue, queue_cap_w, qn_w, lane);
+                stream_batch<FORM, CROWDED, true>(q, m, buf, part, e0, n_e, C, base, my_queue, queue_cap_w, qn_w, lane);
             else
-                stream_batch<SHORT, CROWDED, false>(q, m, buf, part_bits, hmask, e0, n_e, C, base, my_queue, queue_cap_w, qn_w, lane);
+                stream_batch<FORM, CROWDED, false>(q, m, buf, part, e0, n_e, C, base, my_queue, queue_cap_w, qn_w, lane);
         }
     }
     return qn_w;
@@ -462,15 +529,14 @@ __device__ __forceinline__ bool looks_crowded(const PartitionParams& q, uint32_t
     return __popc(__ballot_sync(0xFFFFFFFFu, hi == common)) >= 8 || __popc(__ballot_sync(0xFFFFFFFFu, hi == other)) >= 8;
 }
 
-// What a CTA of the partition pass does, for either kind of entries.
-template <bool SHORT>
+// What a CTA of the partition pass does, for each form of the entries.
+template <ull FORM>
 __device__ __forceinline__ void partition_cta(const PartitionParams& q, unsigned char* smem_raw) {
     const uint32_t C = q.t.C;
-    ull* s_keys = reinterpret_cast<ull*>(smem_raw);
-    uint2* s_acc = reinterpret_cast<uint2*>(s_keys + C);      // {low limb, count | NEW_KEY_FLAG}
+    uint2* s_acc = reinterpret_cast<uint2*>(smem_raw + C * KEY_BYTES<FORM>);   // {low limb, count | NEW_KEY_FLAG}
     uint32_t* s_a1 = reinterpret_cast<uint32_t*>(s_acc + C);  // high limb
     PartSmem m;
-    m.keys = smem_addr(s_keys);
+    m.keys = smem_addr(smem_raw);
     m.acc = smem_addr(s_acc);
     m.a1 = smem_addr(s_a1);
     m.weights = smem_addr(s_a1 + C);
@@ -481,23 +547,20 @@ __device__ __forceinline__ void partition_cta(const PartitionParams& q, unsigned
     ulonglong2* const my_queue = q.queue + (size_t)blockIdx.x * q.queue_cap + (size_t)(threadIdx.x >> 5) * queue_cap_w;
     const uint32_t n_parts = 1u << q.t.lp;
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u, n_warps = blockDim.x >> 5;
-    if (SHORT)
+    if (FORM != FORM_LONG)
         for (uint32_t i = threadIdx.x; i < q.n_apps; i += blockDim.x) (s_a1 + C)[i] = q.app_w[i];
     // Partitions are handed out by a counter (their entry counts differ by a few per cent, and a static
-    // split leaves the kernel waiting for its slowest CTA); a CTA always holds its next partition as
-    // well, so that it can pull that one's keys and entries towards L2 early.
+    // split leaves the kernel waiting for its slowest CTA).  A CTA draws its next one when its entries are through, early
+    // enough to pull that one's keys and entries towards L2 during the write-back; drawn any earlier, the CTAs that
+    // start first hold two of what little is left of 256 partitions (53 M entries: 730 us, three partitions at most CTAs' ends).
     __shared__ uint32_t s_next;
-    if (blockIdx.x >= n_parts) return;                             // (never: at least 256 partitions)
-    if (threadIdx.x == 0) s_next = (uint32_t)atomicAdd(&q.t.ctl->part_cursor, 1ull);
-    uint32_t part = blockIdx.x;                                     // the first round is the static one
+    const auto draw = [&] {
+        if (threadIdx.x == 0) s_next = gridDim.x + (uint32_t)atomicAdd(&q.t.ctl->part_cursor, 1ull);   // (the first round is the static one)
+    };
+    uint32_t part = blockIdx.x;
     while (part < n_parts) {
-        __syncthreads();  // s_next is set; the previous partition's write-back has finished reading shared memory
-        const uint32_t next = gridDim.x + s_next;                   // the counter starts at 0: partitions >= gridDim
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            s_total = 0;
-            s_next = (uint32_t)atomicAdd(&q.t.ctl->part_cursor, 1ull);
-        }
+        __syncthreads();  // the previous partition's write-back has finished reading shared memory
+        if (threadIdx.x == 0) s_total = 0;
         __syncthreads();
         uint32_t local_total = 0;
         for (uint32_t g = threadIdx.x; g < q.n_groups; g += blockDim.x) local_total += q.spill_cnt[((ull)g << q.t.lp) + part];
@@ -506,7 +569,9 @@ __device__ __forceinline__ void partition_cta(const PartitionParams& q, unsigned
 
         __syncthreads();
         if (s_total == 0) {  // nothing was spilled to this partition (uniform)
-            part = next;
+            draw();
+            __syncthreads();
+            part = s_next;
             continue;
         }
 
@@ -519,7 +584,9 @@ __device__ __forceinline__ void partition_cta(const PartitionParams& q, unsigned
             for (int u = 0; u < 4; ++u) {
                 const uint32_t i = i0 + u * blockDim.x;
                 if (i < C) {
-                    s_keys[i] = k[u] == 0 ? 0ull : ckey_of_key(~k[u]);   // the table stores complemented keys, 0 = empty
+                    const FormKey<FORM> f = k[u] == 0 ? FormKey<FORM>{0u, 0u} : form_key<FORM>(q, ~k[u]);   // the table stores complemented keys, 0 = empty
+                    if (FORM == FORM_TIGHT) reinterpret_cast<uint32_t*>(smem_raw)[i] = f.hi;
+                    else reinterpret_cast<uint2*>(smem_raw)[i] = make_uint2(f.lo, f.hi);
                     s_acc[i] = make_uint2(0, 0);
                     s_a1[i] = 0;
                 }
@@ -531,16 +598,19 @@ __device__ __forceinline__ void partition_cta(const PartitionParams& q, unsigned
         }
         __syncthreads();
 
-        const uint32_t qn_w = SHORT && looks_crowded(q, part, warp, lane) ? stream_share<SHORT, true>(q, m, part, my_queue, queue_cap_w, warp, n_warps, lane)
-                                                                          : stream_share<SHORT, false>(q, m, part, my_queue, queue_cap_w, warp, n_warps, lane);
-        settle_queue(q.t, m, my_queue, qn_w, C, base, lane);
+        const uint32_t qn_w = FORM != FORM_LONG && looks_crowded(q, part, warp, lane)
+                                  ? stream_share<FORM, FORM != FORM_LONG>(q, m, part, my_queue, queue_cap_w, warp, n_warps, lane)
+                                  : stream_share<FORM, false>(q, m, part, my_queue, queue_cap_w, warp, n_warps, lane);
+        draw();
+        settle_queue<FORM>(q, m, my_queue, qn_w, base, lane);
         __syncthreads();
+        const uint32_t next = s_next;
         {   // while the deltas are written back, pull the next partition's keys and each warp's
             // first sub-buffer towards L2 (used within microseconds, so they are still there)
             if (next < n_parts) {
                 const unsigned char* nk = reinterpret_cast<const unsigned char*>(q.t.keys + (ull)next * C);
                 for (uint32_t off = threadIdx.x * 128u; off < C * 8u; off += blockDim.x * 128u) prefetch_l2(nk + off);
-                if (warp < q.n_groups) prefetch_entries<SHORT>(q, ((ull)warp << q.t.lp) + next, lane);
+                if (warp < q.n_groups) prefetch_entries<FORM>(q, ((ull)warp << q.t.lp) + next, lane);
             }
         }
         // read-modify-write of the touched slots, four per thread in flight (the loads miss L1 by
@@ -568,7 +638,12 @@ __device__ __forceinline__ void partition_cta(const PartitionParams& q, unsigned
                 const ull nlo = old[u].x + ((ull)c[u].x | ((ull)s_a1[i] << 32));
                 const ull cnthi = old[u].y + (ull)(c[u].y & ~NEW_KEY_FLAG) + ((nlo < old[u].x ? 1ull : 0ull) << HI_SHIFT);
                 q.t.vals[base + i] = make_ulonglong2(nlo, cnthi);
-                if (c[u].y & NEW_KEY_FLAG) q.t.keys[base + i] = ~key_of_ckey(s_keys[i]);
+                if (c[u].y & NEW_KEY_FLAG) {
+                    FormKey<FORM> f = {0u, 0u};
+                    if (FORM == FORM_TIGHT) f.hi = reinterpret_cast<const uint32_t*>(smem_raw)[i];
+                    else f = {reinterpret_cast<const uint2*>(smem_raw)[i].y, reinterpret_cast<const uint2*>(smem_raw)[i].x};
+                    q.t.keys[base + i] = ~key_of_form<FORM>(q, f, part);
+                }
             }
         }
         // this partition's buffers are empty again
@@ -577,22 +652,34 @@ __device__ __forceinline__ void partition_cta(const PartitionParams& q, unsigned
     }
 }
 
-__global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(PartitionParams q) {
+__global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(const __grid_constant__ PartitionParams q) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     grid_dependency_wait();
     // the spill buffers are drained lazily: unless forced, only when the scatter launch just
     // before this one found a buffer filling up
-    if (!q.force && ld_relaxed(&q.t.ctl->drain_seq) != q.seq) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&q.t.ctl->n_drains, 1ull);
-    if (q.t.ctl->words != 0)
-        partition_cta<true>(q, smem_raw);
+    Control* const ctl = q.t.ctl;
+    const bool misfits = ld_relaxed(&ctl->n_misfit) > q.misfit_max;
+    if (!q.force && !misfits && ld_relaxed(&ctl->drain_seq) != q.seq) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&ctl->n_drains, 1ull);
+    const ull form = ld_relaxed(&ctl->form);
+    if (form != FORM_SHORT)
+        partition_cta<FORM_LONG>(q, smem_raw);
+    else if (ld_relaxed(&ctl->rests) != 0)
+        partition_cta<FORM_SHORT>(q, smem_raw);
     else
-        partition_cta<false>(q, smem_raw);
+        partition_cta<FORM_TIGHT>(q, smem_raw);
     grid_dependents_launch();
-    // the last CTA rewinds the hand-out counter for the next launch
+    // The last CTA rewinds the hand-out counter for the next launch.  Where many records did not fit the form of the
+    // entries, the next ones are long (the buffers are empty now).
     if (threadIdx.x == 0) {
         __threadfence();
-        if (atomicAdd(&q.t.ctl->part_done, 1ull) == gridDim.x - 1) q.t.ctl->part_cursor = q.t.ctl->part_done = 0;
+        if (atomicAdd(&ctl->part_done, 1ull) == gridDim.x - 1) {
+            ctl->part_cursor = ctl->part_done = ctl->rests = 0;
+            if (misfits) {
+                ctl->form = FORM_LONG_ONLY;
+                ctl->n_misfit = 0;
+            }
+        }
     }
 }
 
@@ -680,7 +767,7 @@ __global__ void __launch_bounds__(256) hot_count_kernel(HotBuildParams p) {
         }
     }
     max_op = __reduce_max_sync(0xFFFFFFFFu, max_op);
-    if ((threadIdx.x & 31u) == 0 && max_op >> p.op_bits) atomicMax(&p.scratch->max_op, max_op);   // (only what does not fit is told)
+    if ((threadIdx.x & 31u) == 0 && max_op >= p.max_ops) atomicMax(&p.scratch->max_op, max_op);   // (only what does not fit is told)
     grid_dependents_launch();
     cache.flush(p.sketch);
 }
@@ -726,10 +813,12 @@ __global__ void __launch_bounds__(256) hot_admit_kernel(HotBuildParams p) {
     cache.flush(p.cand_cnt);
 }
 
-// The words form's two-way buckets lose 5 % of 4 096 equally frequent keys, the tags form's four-way ones 2.4 %: there the
-// tags hold more (2^27 records 835 us either way).  Below, neither loses much and words are faster (2 048 keys: 734
-// against 802 us); above, words hold as many or more (12 288 keys: 1 052 against 1 082; 32 768: 1 378 against 1 808).
-constexpr uint32_t TAGS_FROM = 3000, TAGS_TO = 5000;
+// The words form's two-way buckets lose 5 % of 4 096 equally frequent keys and 9 % of 6 144, the tags form's four-way ones
+// 2 and 6 %.  Words are faster where some keys are more frequent than others, which the buckets keep (2^27 records,
+// Zipf(1.1) over 6 144 keys: 791 us against 884), and where keys are equally frequent but fewer (2 048: 740 against 809,
+// 4 096: 811 against 860) or more (12 288: 1 056 against 1 082, 32 768: 1 357 against 1 808).  Between, tags hold more
+// (6 144: 909 against 940, 6 880: 933 against 966), and from TAGS_PART on where such keys hold only a part of the trace.
+constexpr uint32_t TAGS_PART = 3500, TAGS_FROM = 5500, TAGS_TO = 7500, EVEN = 4;
 constexpr uint32_t LIST_MAX = 16;       // candidates a bucket chooses from (five on average)
 constexpr uint32_t LEVEL_THREADS = 1024;
 
@@ -770,10 +859,11 @@ __global__ void __launch_bounds__(LEVEL_THREADS) hot_level_kernel(HotBuildParams
     // less evenly than one of four): thread t looks at the count 1023 - t, behind a scan over the higher ones
     const ull most_seen = __ldcg(&x.most);
     const ull skew = most_seen * 8u >= p.n_sample * 3ull ? SKEW_DOMINATED : (most_seen * 32u >= p.n_sample ? SKEW_COMBINE : SKEW_NONE);
-    const bool words = p.op_bits != 0 && __ldcg(&x.max_op) == 0;
+    const bool words = p.max_ops != 0 && __ldcg(&x.max_op) == 0;
     const uint32_t slots = p.slots[words][skew == SKEW_DOMINATED];
     const uint32_t budget = min(words ? 2 * slots : slots + slots / 4, HOT_SELECT_MAX);
-    uint32_t incl = __ldcg(&x.hist[1023 - t]);
+    const uint32_t mine = __ldcg(&x.hist[1023 - t]);
+    uint32_t incl = mine;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
         const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, incl, d);
@@ -793,11 +883,19 @@ __global__ void __launch_bounds__(LEVEL_THREADS) hot_level_kernel(HotBuildParams
     __syncthreads();
     incl += w ? s_warp[w - 1] : 0u;
     const int above = __syncthreads_count(t <= 1021 && incl <= budget);   // counts 1023, 1022, ... that fit
+    __shared__ uint32_t s_weight;                                          // of the sample, in the selected candidates
+    if (t == 0) s_weight = 0;
+    __syncthreads();
+    const uint32_t weight = __reduce_add_sync(0xFFFFFFFFu, t < (uint32_t)above ? mine * (1023u - t) : 0u);
+    if (lane == 0 && weight) atomicAdd(&s_weight, weight);
+    __syncthreads();
     if (above == 0 ? t == 0 : t == (uint32_t)above - 1u) {
         const uint32_t selected = above ? incl : 0u;
         x.threshold = 1024u - (uint32_t)above;
         p.ctl->hot_skew = skew;
-        p.ctl->words = words && !(selected > TAGS_FROM && selected <= TAGS_TO) ? 1 : 0;
+        const bool even = most_seen * selected < (ull)EVEN * s_weight;
+        const bool tags = even && selected > (s_weight < p.n_sample / 2 ? TAGS_PART : TAGS_FROM) && selected <= TAGS_TO;
+        p.ctl->form = words && !tags ? FORM_SHORT : FORM_LONG;
     }
 }
 
@@ -805,12 +903,13 @@ struct Buckets {
     uint32_t n, ways;
 };
 __device__ __forceinline__ Buckets buckets_in_use(const HotBuildParams& p) {
-    const bool words = p.ctl->words != 0;
+    const bool words = p.ctl->form != FORM_LONG;
     const uint32_t ways = words ? WORD_WAYS : TAG_WAYS;
     return {p.slots[words][p.ctl->hot_skew == SKEW_DOMINATED] / ways, ways};
 }
 
-// A multiplier's loss is approximated by arrival order among the keys that matter.
+// A multiplier's loss is approximated by arrival order among the keys that matter: those that hold 1/4096 of the sample.
+// (A key of that size that finds no slot fills its partition, and the partition pass waits for the CTA that has it.)
 __global__ void __launch_bounds__(256) hot_gather_kernel(HotBuildParams p) {
     __shared__ uint32_t s_lost[4];
     if (threadIdx.x < 4) s_lost[threadIdx.x] = 0;
@@ -833,7 +932,7 @@ __global__ void __launch_bounds__(256) hot_gather_kernel(HotBuildParams p) {
             x.count[at] = c;
         }
         if (c == x.most) p.ctl->top_key = ~skey;   // (of several equally frequent ones, any)
-        if (c >= 16) {
+        if (c >= max(p.n_sample >> 12, 16u)) {
 #pragma unroll
             for (uint32_t m = 0; m < 4; ++m)
                 if (atomicAdd(&x.occupancy[m][dir_bucket_of_key(~skey, DIR_MULTS[m], buckets.n)], 1u) >= buckets.ways) atomicAdd(&s_lost[m], c);

@@ -30,9 +30,6 @@ constexpr uint32_t scatter_fixed_bytes(uint32_t lp) {
 constexpr uint32_t WORD_WAYS = 2, TAG_WAYS = 4;
 constexpr uint32_t scatter_slots(uint32_t lp, bool words) { return ((SCATTER_SMEM_BYTES - scatter_fixed_bytes(lp)) / (words ? 16u : 21u)) & ~31u; }
 constexpr uint32_t scatter_hot_slots(uint32_t lp) { return scatter_slots(lp, true); }   // of the directory image, either form
-// A word holds the top bits of what the bucket hash leaves over and, below them, phase and operator.  All ones there mark
-// an empty slot, so that those two have one bit less.
-constexpr uint32_t DIR_ID_BITS = 12, DIR_ID_MASK = (1u << DIR_ID_BITS) - 1u;
 
 // Where one key dominates the trace, the last part of the accumulators holds the warps' queues instead (64 records
 // each), and the directory is that much smaller.
@@ -50,7 +47,7 @@ struct IngestParams {
     uint32_t phase_lim;        // n_phases << 16: bound of (phase << 16 | op_id)
     uint32_t appw_in_smem;
     const uint32_t* app_w;     // device copy of the card-hour weights
-    ShortFormat fmt;           // short spill entries; operators below 2^fmt.op_bits fit a directory word
+    ShortFormat fmt;           // short spill entries and directory words
     const ull* hot_keys;       // directory image, hot_slots entries of ~key (0 = empty)
     uint32_t hot_slots;        // multiple of 4
     uint32_t img_rows;         // rows of hot_img that hold sums since the last fold; a CTA beyond them starts its row afresh
@@ -87,7 +84,8 @@ struct PartitionParams {
     uint32_t* spill_cnt;
     uint32_t n_groups;         // scatter CTAs whose buffers are read
     uint32_t cap, short_cap;
-    ShortFormat fmt;
+    ShortFormat fmt;           // as in IngestParams
+    uint32_t misfit_max;       // more records than this that do not fit: drain, and long entries from here on
     uint32_t n_apps;
     const uint32_t* app_w;     // card-hour weights (short entries)
     uint32_t force;            // 1: drain unconditionally; 0: only if the scatter launch `seq` asked for it
@@ -118,7 +116,7 @@ struct HotBuildParams {
     ull stride;                // records per sampled one (below 2^32)
     uint32_t n_sample;         // n_sample * stride <= records of the call
     uint32_t n_apps, n_phases;
-    uint32_t op_bits;          // operators below 2^op_bits fit a directory word (0: that form is not used)
+    uint32_t max_ops;          // as in ShortFormat (0: no short entries)
     ull* hot_keys;
     uint32_t hot_slots;        // of the image
     uint32_t slots[2][2];      // slots in use by [words][one key dominates]

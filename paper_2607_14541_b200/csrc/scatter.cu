@@ -52,7 +52,8 @@ struct Smem {
     static constexpr uint32_t RING = 0;                         // record ring: SCATTER_RING_STAGES tiles
     static constexpr uint32_t CUR = RING + SCATTER_RING_STAGES * SCATTER_RING_TILE;   // u32[P]  entries appended to this CTA's buffer of each partition
     static constexpr uint32_t APPW = CUR + 4u * P;              // u32[APPW_SMEM_MAX]  card-hour weights
-    static constexpr uint32_t LONG = APPW + 4u * APPW_SMEM_MAX;    // words: records that took two short entries (and a pad word)
+    static constexpr uint32_t LONG = APPW + 4u * APPW_SMEM_MAX;    // words: records that took two short entries
+    static constexpr uint32_t RESTS = LONG + 4u;                // ... whether an entry's identity has a rest
     static constexpr uint32_t WORDS = LONG + 8u;                // ... u32[SLOTS]
     static constexpr uint32_t TAG = LONG;                       // tags: u32[NB + 1]  four 8-bit tags per bucket (+ one pad bucket)
     static constexpr uint32_t KEYS = (TAG + 4u * (NB + 1u) + 7u) & ~7u;   // ull[SLOTS + 4]  key, all ones = empty
@@ -144,10 +145,12 @@ __device__ __noinline__ void drain_slot(TableRef t, uint32_t acc, ull key, uint3
 __device__ __noinline__ void table_route(TableRef t, ull key, uint32_t h, ull prod) { table_accumulate(t, key, h, prod, 0, 1); }
 // (rare) An invalid record is counted; a valid one whose product has bits at or above 2^48, or whose operator does not
 // fit, goes to the table.
+template <bool COUNT_MISFITS>
 __device__ __noinline__ void rare_record(TableRef t, bool valid, ull key, uint32_t h, ull prod) {
-    if (valid)
+    if (valid) {
         table_accumulate(t, key, h, prod, 0, 1);
-    else
+        if (COUNT_MISFITS && (uint32_t)(prod >> 32) < 0x10000u) atomicAdd(&t.ctl->n_misfit, 1ull);
+    } else
         atomicAdd(&t.ctl->n_rejected, 1ull);
 }
 
@@ -215,25 +218,30 @@ __device__ __forceinline__ void spill_append(const IngestParams& p, Ctx& c, bool
     }
 }
 
+// Operator and phase as directory words and short entries hold them (see ShortFormat).
+__device__ __forceinline__ uint32_t identity(uint32_t khi, uint32_t phase_bits) { return ((khi & 0xFFFFu) << phase_bits) + (khi >> 16); }
+
 // The same as a short entry (ShortFormat), in one store; a duration that does not fit takes a second entry behind it.
-template <uint32_t LP>
+template <uint32_t LP, int DIR>
 __device__ __forceinline__ void short_append(const IngestParams& p, Ctx& c, bool todo, uint32_t khi, uint32_t app, uint32_t shape,
                                              uint32_t dur, ull prod, uint32_t h) {
     if (!todo) return;
     const uint32_t part = ATREX_INDEX(h >> (32 - LP), 1u << LP, p.t.ctl);
-    const uint32_t cw = c.sb + Smem<LP, DIR_WORDS>::CUR + part * 4u;
-    const uint32_t rest = dur >> p.fmt.dur_bits, n = rest ? 2u : 1u;
+    const uint32_t cw = c.sb + Smem<LP, DIR>::CUR + part * 4u;
+    const ShortFormat& f = p.fmt;
+    const uint32_t rest = dur >> f.dur_bits, n = rest ? 2u : 1u;
     const uint32_t tk = atoms_add(cw, n);
     if (tk + n <= p.short_cap) {
-        const uint32_t hash = h << LP, id = ((khi >> 16) << p.fmt.op_bits) + (khi & 0xFFFFu);
-        const uint32_t hi = (id << (31u - p.fmt.id_bits)) | (hash >> (1u + p.fmt.id_bits));
-        const uint32_t lo = (hash << (31u - p.fmt.id_bits)) | (app << p.fmt.dur_bits);
+        const uint32_t id = identity(khi, f.phase_bits);
+        const uint32_t hi = ((h << (LP - 1u)) & 0x7FFFFFFFu) | (id & ((1u << (LP - 1u)) - 1u));
+        const uint32_t id_rest = id >> (LP - 1u), lo = (id_rest << f.rest_shift) | (app << f.dur_bits);
+        if (LP - 1u < DIR_ID_BITS - 1u && id_rest) asm volatile("st.shared.u32 [%0], 1;" ::"r"(c.sb + Smem<LP, DIR>::RESTS) : "memory");
         unsigned char* at = c.my_spill + (part * p.short_cap + ATREX_INDEX(tk, p.short_cap, p.t.ctl)) * SHORT_ENTRY_BYTES;
-        asm volatile("st.global.L2::cache_hint.v2.u32 [%0], {%1, %2}, %3;" ::"l"(at), "r"(lo | (dur & p.fmt.dur_mask())), "r"(hi), "l"(c.keep) : "memory");
+        asm volatile("st.global.L2::cache_hint.v2.u32 [%0], {%1, %2}, %3;" ::"l"(at), "r"(lo | (dur & f.dur_mask())), "r"(hi), "l"(c.keep) : "memory");
         // three entries before the buffer reaches its next line (four, where this one takes two places), as above
         if ((tk & 15u) - (14u - n) < n) asm volatile("prefetch.global.L2 [%0+64];" ::"l"(at));
         if (rest) {
-            reds_add(c.sb + Smem<LP, DIR_WORDS>::LONG, 1u);
+            reds_add(c.sb + Smem<LP, DIR>::LONG, 1u);
             asm volatile("st.global.L2::cache_hint.v2.u32 [%0+8], {%1, %2}, %3;" ::"l"(at), "r"(lo | rest), "r"(hi | SHORT_CONTINUATION), "l"(c.keep) : "memory");
         }
     } else {
@@ -243,8 +251,8 @@ __device__ __forceinline__ void short_append(const IngestParams& p, Ctx& c, bool
 }
 
 // A directory slot's word (words form): the bits that the bucket leaves over of hash x buckets, phase and operator.
-__device__ __forceinline__ uint32_t dir_word(uint32_t product_lo, uint32_t khi, uint32_t op_bits) {
-    return (product_lo & ~DIR_ID_MASK) | (((khi >> 16) << op_bits) + (khi & 0xFFFFu));
+__device__ __forceinline__ uint32_t dir_word(uint32_t product_lo, uint32_t khi, uint32_t phase_bits) {
+    return (product_lo & ~DIR_ID_MASK) | identity(khi, phase_bits);
 }
 
 // One record, start to finish (the register-staged loop has no registers to spare for working on
@@ -268,17 +276,17 @@ __device__ __forceinline__ void one_record(const IngestParams& p, Ctx& c, uint32
     // configurations whose records mostly hit the directory 4-9 %).
     bool todo_in = ok && (uint32_t)(prod >> 32) < 0x10000u;
     // (words form: an operator that no sampled record had may not fit a word and a short entry)
-    if (DIR == DIR_WORDS) todo_in = todo_in && ((khi & 0xFFFFu) >> p.fmt.op_bits) == 0u;
+    if (L::W) todo_in = todo_in && (khi & 0xFFFFu) < p.fmt.max_ops;
     bool todo = todo_in;
-    if ((FULL || present) && !todo_in) rare_record(p.t, ok, key, h, prod);
+    if ((FULL || present) && !todo_in) rare_record<L::W>(p.t, ok, key, h, prod);
     if (DIR != DIR_NONE) {
         const uint32_t x = dir_mix(h, khi >> 16, c.mult);
         uint32_t at;
         bool hit;
-        if (DIR == DIR_WORDS) {
+        if (L::W) {
             const ull product = (ull)x * L::template NB_OF<SKEW>;
             const uint32_t b = ATREX_INDEX((uint32_t)(product >> 32), L::template NB_OF<SKEW>, p.t.ctl);
-            const uint32_t word = dir_word((uint32_t)product, khi, p.fmt.op_bits);
+            const uint32_t word = dir_word((uint32_t)product, khi, p.fmt.phase_bits);
             const uint2 w = lds_v2u32(c.sb + L::WORDS + b * 8u);
             const bool second = w.y == word;
             at = b * 2u + (second ? 1u : 0u);
@@ -316,8 +324,8 @@ __device__ __forceinline__ void one_record(const IngestParams& p, Ctx& c, uint32
             todo = false;
         }
     }
-    if (DIR == DIR_WORDS)
-        short_append<LP>(p, c, todo, khi, w0, w2, w3, prod, h);
+    if (L::W)
+        short_append<LP, DIR>(p, c, todo, khi, w0, w2, w3, prod, h);
     else
         spill_append<LP>(p, c, todo, khi, w2, prod, h);
 }
@@ -724,21 +732,21 @@ struct RingBars {
     volatile uint32_t* abort_flag;
 };
 
-// What a CTA does with the directory in the form DIR: loads it, goes through its records, stores cursors and sums.
+// What a CTA does with the directory in the form DIR (empty: nothing is in it): loads it, goes through its records, stores cursors and sums.
 template <uint32_t LP, int DIR>
-__device__ __forceinline__ void scatter_cta(const IngestParams& p, Ctx& c, unsigned char* smem_raw, const RingBars& ring) {
+__device__ __forceinline__ void scatter_cta(const IngestParams& p, Ctx& c, unsigned char* smem_raw, const RingBars& ring, bool empty) {
     using L = Smem<LP, DIR>;
     uint32_t* g_cursor = reinterpret_cast<uint32_t*>(smem_raw + L::CUR);
     uint32_t* g_acc = reinterpret_cast<uint32_t*>(smem_raw + L::ACC);
     const ull skew = DIR != DIR_NONE ? p.t.ctl->hot_skew : SKEW_NONE;
-    if (DIR == DIR_WORDS && threadIdx.x == 0) *reinterpret_cast<uint32_t*>(smem_raw + L::LONG) = 0;
+    if (L::W && threadIdx.x < 2) reinterpret_cast<uint32_t*>(smem_raw + L::LONG)[threadIdx.x] = 0;
     if (DIR != DIR_NONE) {
         for (uint32_t i = threadIdx.x; i < L::SLOTS + L::PAD; i += blockDim.x) {
-            const ull image = i < L::SLOTS ? p.hot_keys[i] : 0ull;   // ~key, 0 = empty
+            const ull image = i < L::SLOTS && !empty ? p.hot_keys[i] : 0ull;   // ~key, 0 = empty
             const uint32_t khi = (uint32_t)(~image >> 32), x = dir_mix(hash32(~image), (khi >> 16) & 0xFFu, c.mult);
-            if (DIR == DIR_WORDS) {
+            if (L::W) {
                 const uint32_t left = x * (skew == SKEW_DOMINATED ? L::NB_DOM : L::NB);
-                reinterpret_cast<uint32_t*>(smem_raw + L::WORDS)[i] = image ? dir_word(left, khi, p.fmt.op_bits) : DIR_ID_MASK;
+                reinterpret_cast<uint32_t*>(smem_raw + L::WORDS)[i] = image ? dir_word(left, khi & 0x00FFFFFFu, p.fmt.phase_bits) : DIR_ID_MASK;
             } else {
                 reinterpret_cast<ull*>(smem_raw + L::KEYS)[i] = ~image;
                 (smem_raw + L::TAG)[i] = image ? (unsigned char)(x & 0xFFu) : 0;
@@ -768,10 +776,13 @@ __device__ __forceinline__ void scatter_cta(const IngestParams& p, Ctx& c, unsig
 
     grid_dependents_launch();
     __syncthreads();
-    const uint32_t cap = DIR == DIR_WORDS ? p.short_cap : p.cap, drain_above = DIR == DIR_WORDS ? p.short_drain_above : p.drain_above;
+    const uint32_t cap = L::W ? p.short_cap : p.cap, drain_above = L::W ? p.short_drain_above : p.drain_above;
     uint32_t spilled = 0, fullest = 0;
     bool crowded = false;
-    if (DIR == DIR_WORDS && threadIdx.x == 0) spilled = 0u - *reinterpret_cast<const uint32_t*>(smem_raw + L::LONG);   // (records, not entries)
+    if (L::W && threadIdx.x == 0) {
+        spilled = 0u - *reinterpret_cast<const uint32_t*>(smem_raw + L::LONG);      // (records, not entries)
+        if (*reinterpret_cast<const uint32_t*>(smem_raw + L::RESTS)) p.t.ctl->rests = 1;
+    }
     for (uint32_t i = threadIdx.x; i < L::P; i += blockDim.x) {
         const size_t at = ((size_t)blockIdx.x << LP) + i;
         const uint32_t before = p.spill_cnt[at], n = min(g_cursor[i], cap);
@@ -851,12 +862,13 @@ __global__ void __launch_bounds__(SCATTER_THREADS, 1) scatter_kernel(IngestParam
     if (p.appw_in_smem != 0)
         for (uint32_t i = threadIdx.x; i < p.n_apps; i += blockDim.x) g_appw[i] = p.app_w[i];
     const RingBars ring = {s_full, s_empty, &s_abort};
+    const ull form = HOT ? p.t.ctl->form : FORM_LONG_ONLY;
     if (!HOT)
-        scatter_cta<LP, DIR_NONE>(p, c, smem_raw, ring);
-    else if (SCATTER_RING_STAGES == 0 && p.t.ctl->words != 0)
-        scatter_cta<LP, DIR_WORDS>(p, c, smem_raw, ring);
+        scatter_cta<LP, DIR_NONE>(p, c, smem_raw, ring, true);
+    else if (SCATTER_RING_STAGES == 0 && form == FORM_SHORT)
+        scatter_cta<LP, DIR_WORDS>(p, c, smem_raw, ring, false);
     else
-        scatter_cta<LP, DIR_TAGS>(p, c, smem_raw, ring);
+        scatter_cta<LP, DIR_TAGS>(p, c, smem_raw, ring, form == FORM_LONG_ONLY);
 }
 
 template <uint32_t LP>

@@ -72,3 +72,28 @@ def test_crowded_partitions_and_full_buffers(n_keys):
     check(agg, o)
     st = agg.stats()
     assert st["n_valid"] == len(recs) and (st["n_overflow"] > 0) == (n_keys < 40)
+
+
+def test_operators_that_no_longer_fit():
+    """Records whose operator the sampled ones did not announce go to the table one by one until there are many; the
+    entries are long from then on, the directory's sums so far are kept."""
+    import paper_2607_14541_b200 as p
+    rng = np.random.default_rng(5)
+    n, part = 3 << 20, 1 << 20
+    recs = np.zeros(n, dtype=RECORD_DTYPE)
+    recs["app_id"], recs["phase"] = rng.integers(0, 9, n), rng.integers(0, 2, n)
+    recs["op_id"], recs["shape_id"] = rng.integers(0, 100, n), rng.integers(0, 1000, n)
+    recs["duration_ns"] = rng.integers(0, 1 << 32, n, dtype=np.uint64).astype(np.uint32)
+    recs["op_id"][part:] += np.where(rng.random(n - part) < 0.5, 5000, 0).astype(np.uint16)
+    weights = rng.integers(0, 1 << 16, 9).astype(np.uint32)
+    agg = p.Aggregator(weights, 2, 3_000_000)
+    o = oracle.Oracle(weights, 2)
+    for at in range(0, n, part):
+        ingest(agg, recs[at: at + part])
+        o.ingest(recs[at: at + part], threads=4)
+    drains, cap = agg.stats()["n_drains"], agg.stats()["spill_cap"]
+    check(agg, o)
+    assert drains >= 2 and agg.stats()["n_valid"] == n
+    agg.reset()                                                   # short entries again
+    ingest(agg, recs[:part])
+    assert agg.stats()["spill_cap"] == cap // 2 * 3
