@@ -49,7 +49,7 @@ ull pow2_at_least(ull x) {
 }
 
 struct Layout {
-    size_t off_ctl, off_keys, off_vals, off_work, off_appw, off_hot, off_staging[2], off_sel, off_pick, off_topk_out, off_hist_all, off_hist_next,
+    size_t off_ctl, off_keys, off_vals, off_work, off_appw, off_hot, off_hot_words, off_staging[2], off_sel, off_pick, off_topk_out, off_hist_all, off_hist_next,
         off_spill_cnt, off_spill, off_hot_scratch, off_queue, off_hot_img, total;
     ull n_slots, work_slots;
     uint32_t lp, C;              // partitions = 1 << lp, slots per partition
@@ -149,6 +149,7 @@ void compute_layout(const atrex_agg_config_t* c, size_t smem_optin, int n_sms, L
     L->off_work = o;           o += round_up(L->work_slots * sizeof(WorkSlot), ALIGN);
     L->off_appw = o;           o += round_up((size_t)c->n_apps * 4, ALIGN);
     L->off_hot = o;            o += round_up((size_t)(L->hot_slots ? L->hot_slots : 2) * 8, ALIGN);
+    L->off_hot_words = o;      o += round_up((size_t)(L->hot_slots ? L->hot_slots : 2) * 4, ALIGN);
     L->off_hot_img = o;        o += round_up((size_t)L->n_groups * (L->hot_slots ? L->hot_slots : 2) * 16, ALIGN);
     L->off_staging[0] = o;     o += STAGING_BYTES;
     L->off_staging[1] = o;     o += STAGING_BYTES;
@@ -208,7 +209,9 @@ struct atrex_agg {
     unsigned char* staging[2] = {nullptr, nullptr};
     ull* sel = nullptr;
     atrex_entry_t* topk_out = nullptr;
-    Control* h_ctl = nullptr;  // pinned mirror
+    Control* h_ctl = nullptr;  // pinned: the host's copy of the control block
+    ulonglong2* h_told = nullptr;     // pinned: [CONTROL_WORDS] as the last finalize's kernel tells them
+    ulonglong2* h_top_told = nullptr;    // pinned: [n_phases][TOPK_TOLD_K][6] ... the best few of each phase
     size_t pinned_bytes = 0;
     uint32_t* hist_all = nullptr;     // [2][n_phases][TOPK_BINS] first-digit counts: the last totals pass's, and zeros for the next
     uint32_t hist_at = 0;             // which half is the last pass's
@@ -369,14 +372,17 @@ int atrex_agg_create(const atrex_agg_config_t* cfg, atrex_agg_t** out) {
         if (e == cudaSuccess) e = cudaMemcpy(h->d_appw, cfg->app_weights, (size_t)cfg->n_apps * 4, cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemset(h->hist_all, 0, (size_t)2 * cfg->n_phases * TOPK_BINS * 4);
         if (e == cudaSuccess) e = cudaMemset(h->hot_keys, 0, (size_t)(L.hot_slots ? L.hot_slots : 2) * 8);
-        // the pinned block: every phase's best, how many there are, a digit each, the control block's mirror
+        // the pinned block: what kernels tell with stamps, every phase's best, how many there are, a digit each, the control block's copy
         const size_t top_bytes = (size_t)cfg->n_phases * (TOPK_PICK_K * sizeof(atrex_entry_t) + 8), digit_bytes = cfg->n_phases * sizeof(TopkDigit);
-        h->pinned_bytes = top_bytes + digit_bytes + sizeof(Control);
-        if (e == cudaSuccess) e = pinned_alloc((void**)&h->h_top, h->pinned_bytes);
+        const size_t told_bytes = CONTROL_WORDS * 16 + (size_t)cfg->n_phases * TOPK_TOLD_K * 96;
+        h->pinned_bytes = told_bytes + top_bytes + digit_bytes + sizeof(Control);
+        if (e == cudaSuccess) e = pinned_alloc((void**)&h->h_told, h->pinned_bytes);
         if (e == cudaSuccess) {
+            memset(h->h_told, 0, told_bytes);        // (the block may be another handle's former one: no stamp of its may be left)
+            h->h_top_told = h->h_told + CONTROL_WORDS;
+            h->h_top = (atrex_entry_t*)((unsigned char*)h->h_told + told_bytes);
             h->h_digit = (TopkDigit*)((unsigned char*)h->h_top + top_bytes);
             h->h_ctl = (Control*)((unsigned char*)h->h_digit + digit_bytes);
-            h->h_ctl->seq = 0;   // (the block may be another handle's former one)
             memset(h->h_digit, 0, digit_bytes);
         }
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking);
@@ -406,7 +412,7 @@ void atrex_agg_destroy(atrex_agg_t* h) {
         if (h->ev_free[i]) cudaEventDestroy(h->ev_free[i]);
     }
     if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
-    pinned_free(h->h_top, h->pinned_bytes);
+    pinned_free(h->h_told, h->pinned_bytes);
     if (h->owns_workspace && h->ws) cudaFree(h->ws);
     delete h;
 }
@@ -527,6 +533,8 @@ static int ingest_launch(atrex_agg* h, const atrex_record_t* recs, uint64_t n, c
         b.hot_keys = h->hot_keys;
         b.max_ops = h->L.fmt.max_ops;
         b.hot_slots = h->L.hot_slots;
+        b.hot_words = (uint32_t*)(h->ws + h->L.off_hot_words);
+        b.phase_bits = h->L.fmt.phase_bits;
         for (int words = 0; words < 2; ++words) {
             b.slots[words][0] = scatter_slots(h->L.lp, words != 0);
             b.slots[words][1] = scatter_dominated_slots(h->L.lp, words != 0);
@@ -563,6 +571,7 @@ static int ingest_launch(atrex_agg* h, const atrex_record_t* recs, uint64_t n, c
     p.fmt = h->L.fmt;
     p.hot_keys = h->hot_keys;
     p.hot_slots = h->L.hot_slots;
+    p.hot_words = (const uint4*)(h->ws + h->L.off_hot_words);
     p.hot_img = h->hot_img;
     p.t = h->table_ref();
     p.spill = h->spill;
@@ -639,7 +648,7 @@ int atrex_agg_merge(atrex_agg_t* h, const atrex_entry_t* d_entries, uint64_t n, 
     return ATREX_OK;
 }
 
-static int run_totals(atrex_agg* h, const uint64_t* total_lo, const uint64_t* total_hi, cudaStream_t s) {
+static GivenTotals given_totals(const uint64_t* total_lo, const uint64_t* total_hi) {
     GivenTotals given;
     memset(&given, 0, sizeof(given));
     if (total_lo) {
@@ -648,10 +657,14 @@ static int run_totals(atrex_agg* h, const uint64_t* total_lo, const uint64_t* to
         memcpy(given.hi, total_hi, sizeof(given.hi));
         given.use = 1;
     }
-    const uint32_t n_phases = h->cfg.n_phases;
+    return given;
+}
+
+static uint32_t* hist_half(atrex_agg* h, uint32_t which) { return h->hist_all + (size_t)which * h->cfg.n_phases * TOPK_BINS; }
+
+static int run_totals(atrex_agg* h, const GivenTotals& given, cudaStream_t s) {
     h->hist_at ^= 1u;
-    uint32_t* const half[2] = {h->hist_all, h->hist_all + (size_t)n_phases * TOPK_BINS};
-    CU(h, launch_totals(h->table_ref(), h->L.n_slots, n_phases, given, half[h->hist_at], half[h->hist_at ^ 1u], h->n_sms, s));
+    CU(h, launch_totals(h->table_ref(), h->L.n_slots, h->cfg.n_phases, given, hist_half(h, h->hist_at), hist_half(h, h->hist_at ^ 1u), h->n_sms, s));
     h->launches++;
     return ATREX_OK;
 }
@@ -661,8 +674,8 @@ static FinalizeParams finalize_params(const atrex_agg* h, atrex_entry_t* out, ui
     p.t = h->table_ref();
     p.n_slots = h->L.n_slots;
     p.ctl = h->ctl;
-    p.mirror = h->h_ctl;
-    p.seq = 0;
+    p.told = h->h_told;
+    p.stamp = 0;
     p.work = h->work_ref();
     p.peaks = h->peaks;
     p.out = out;
@@ -673,6 +686,17 @@ static FinalizeParams finalize_params(const atrex_agg* h, atrex_entry_t* out, ui
 static int finalize_impl(atrex_agg_t* h, const atrex_hw_peaks_t* peaks, const uint64_t* total_lo,
                          const uint64_t* total_hi, atrex_entry_t* d_out, uint64_t out_cap, uint64_t* n_out,
                          void* stream);
+
+// Words that a kernel tells (finalize.cu): whether all of them have arrived, and what they say.
+static bool all_told(const ulonglong2* words, uint32_t n, uint32_t stamp) {
+    const volatile ull* half = (const volatile ull*)words;
+    for (uint32_t i = 2 * n; i-- > 0;)
+        if (half[i] >> 32 != stamp) return false;
+    return true;
+}
+static void take_told(const ulonglong2* words, uint32_t n, void* out) {
+    for (uint32_t i = 0; i < n; ++i) ((ull*)out)[i] = (uint32_t)words[i].x | words[i].y << 32;
+}
 
 int atrex_agg_finalize(atrex_agg_t* h, const atrex_hw_peaks_t* peaks, atrex_entry_t* d_out, uint64_t out_cap,
                        uint64_t* n_out, void* stream) {
@@ -701,15 +725,25 @@ static int finalize_impl(atrex_agg_t* h, const atrex_hw_peaks_t* peaks, const ui
     h->peaks = *peaks;
     int rc = drain_spill(h, /*force=*/true, s);
     if (rc != ATREX_OK) return rc;
-    rc = run_totals(h, total_lo, total_hi, s);
-    if (rc != ATREX_OK) return rc;
+    const GivenTotals given = given_totals(total_lo, total_hi);
     FinalizeParams fin = finalize_params(h, d_out, out_cap);
-    fin.seq = ++h->wait_seq;
-    CU(h, launch_emit(fin, h->n_sms, s));   // (fills the mirror h_ctl)
+    // (the last kernel tells the control block)
+    if (finalize_is_small(h->L.n_slots)) {
+        fin.stamp = (uint32_t)++h->wait_seq;
+        h->hist_at ^= 1u;
+        CU(h, launch_finalize_small(fin, h->cfg.n_phases, given, hist_half(h, h->hist_at), hist_half(h, h->hist_at ^ 1u), s));
+    } else {
+        rc = run_totals(h, given, s);
+        if (rc != ATREX_OK) return rc;
+        fin.stamp = (uint32_t)++h->wait_seq;
+        CU(h, launch_emit(fin, h->n_sms, s));
+    }
     h->launches++;
-    const volatile ull* seq = &h->h_ctl->seq;
-    const ull want = fin.seq;
-    CU(h, wait_for_kernel([=] { return *seq == want; }, s));
+    const ulonglong2* const told = h->h_told;
+    const uint32_t stamp = fin.stamp;
+    CU(h, wait_for_kernel([=] { return all_told(told, CONTROL_WORDS, stamp); }, s));
+    if (!all_told(told, CONTROL_WORDS, stamp)) return ATREX_ERR_STATE;   // (cannot happen: the stream is idle)
+    take_told(told, CONTROL_WORDS, h->h_ctl);
     *n_out = h->h_ctl->n_out;
     rc = device_status_to_error(h->h_ctl);
     if (rc != ATREX_OK) return rc;
@@ -823,25 +857,31 @@ int atrex_agg_topk(atrex_agg_t* h, uint32_t phase, uint32_t k, atrex_entry_t* h_
         if (cache.pick_gen != h->fin_gen || cache.k != k) {
             PickParams p;
             p.fin = finalize_params(h, nullptr, 0);
-            p.fin.seq = ++h->wait_seq & 0xFFFFFFFFu;
+            p.fin.stamp = (uint32_t)++h->wait_seq;
             p.n_phases = h->cfg.n_phases;
             p.k = k;
             p.hist = h->hist_all + (size_t)h->hist_at * h->cfg.n_phases * TOPK_BINS;
             p.sel = h->pick;
             p.host_top = h->h_top;
+            p.host_told = h->h_top_told;
             p.host_n = answers;
             cache.pick_gen = 0;
             const uint32_t n_phases = p.n_phases;
-            const ull want = p.fin.seq;
-            for (uint32_t q = 0; q < n_phases; ++q) answers[q] = ~(want << 32);
+            const uint32_t stamp = p.fin.stamp;
+            for (uint32_t q = 0; q < n_phases; ++q) answers[q] = (ull)~stamp << 32;
             CU(h, launch_topk_pick(p, h->n_sms, s));
-            h->launches += 2;
+            h->launches += finalize_is_small(h->L.n_slots) ? 1 : 2;
             const volatile ull* a = answers;
-            CU(h, wait_for_kernel([=] {
+            const ulonglong2* const rows = k <= TOPK_TOLD_K ? h->h_top_told : nullptr;
+            const auto answered = [=] {
                 for (uint32_t q = 0; q < n_phases; ++q)
-                    if (a[q] >> 32 != want) return false;
+                    if (a[q] >> 32 != stamp || (rows && (uint32_t)a[q] != PICK_NONE && !all_told(rows + (size_t)q * TOPK_TOLD_K * 6, (uint32_t)a[q] * 6, stamp))) return false;
                 return true;
-            }, s));
+            };
+            CU(h, wait_for_kernel(answered, s));
+            if (!answered()) return ATREX_ERR_STATE;                     // (cannot happen: the stream is idle)
+            for (uint32_t q = 0; rows && q < n_phases; ++q)
+                if ((uint32_t)a[q] != PICK_NONE) take_told(rows + (size_t)q * TOPK_TOLD_K * 6, (uint32_t)a[q] * 6, h->h_top + (size_t)q * TOPK_PICK_K);
             cache.pick_gen = h->fin_gen;
             cache.k = k;
         }
@@ -885,7 +925,7 @@ int atrex_agg_stats(atrex_agg_t* h, atrex_stats_t* out, void* stream) {
     cudaStream_t s = (cudaStream_t)stream;
     int rc = drain_spill(h, /*force=*/true, s);
     if (rc != ATREX_OK) return rc;
-    rc = run_totals(h, nullptr, nullptr, s);
+    rc = run_totals(h, given_totals(nullptr, nullptr), s);
     if (rc != ATREX_OK) return rc;
     CU(h, cudaMemcpyAsync(h->h_ctl, h->ctl, offsetof(Control, acc_lo), cudaMemcpyDeviceToHost, s));
     CU(h, cudaStreamSynchronize(s));

@@ -21,6 +21,7 @@
 //                 slots {~(op_id << 32 | shape_id), flops, bytes, dtype}, probed inside the partition
 //   control     : counters, per-phase totals
 #pragma once
+#include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -52,6 +53,7 @@ constexpr ull ST_BOUNDS = 32;   // debug build: an index was outside its array
 constexpr int TOPK_BINS = 4096;       // 12-bit digits
 constexpr uint32_t TOPK_PICK_MAX = 2048;     // candidates of a phase that one CTA ranks in shared memory
 constexpr uint32_t TOPK_PICK_K = 1024;       // ... and the largest k answered that way
+constexpr uint32_t TOPK_TOLD_K = 128;        // ... of these with stamps (12 of 96 KB more pinned memory per phase)
 constexpr uint32_t PICK_NONE = 0xFFFFFFFFu;
 // How much of the sample the most frequent key holds: same-slot collisions inside a warp are common from 1/32 on
 // (equal lanes are then combined first); from 3/8 on the key is best taken out before anything else.
@@ -67,7 +69,6 @@ struct Control {
     ull n_rejected;
     ull n_dropped;
     ull n_out;                 // entries emitted by the last finalize
-    ull seq;                   // (mirror only) finalize whose results the mirror holds
     ull hot_n;                 // keys in the hot directory
     ull work_status;           // ST_WORK_* bits of the last work-table load
     ull hot_skew;              // SKEW_*: how the scatter pass deals with the most frequent key
@@ -88,12 +89,14 @@ struct Control {
     ull total_hi[ATREX_MAX_PHASES];
     ull keys_per_phase[ATREX_MAX_PHASES];
     ull count_per_phase[ATREX_MAX_PHASES];
-    // ---- up to here mirrored in pinned host memory by every finalize
+    // ---- up to here told to the host by every finalize
     ull acc_lo[ATREX_MAX_PHASES], acc_hi[ATREX_MAX_PHASES], acc_keys[ATREX_MAX_PHASES], acc_count[ATREX_MAX_PHASES];   // totals pass: sums so far
     ull tot_done, emit_done;              // CTAs that are through; the last one moves the sums on / fills the mirror
     ull sel_count_all[ATREX_MAX_PHASES];  // top-k: candidates collected per phase
     uint32_t pick_bin[ATREX_MAX_PHASES];  // top-k: first digit of the last bin that is collected, PICK_NONE = too many candidates
 };
+
+constexpr uint32_t CONTROL_WORDS = offsetof(Control, acc_lo) / 8;   // what the host gets to see
 
 // 32-bit mixer of (op_id, shape_id) for the key table, the spill partitions, the hot directory
 // and the work table: two multiplicative hashes of the two words, folded and multiplied once
@@ -171,6 +174,12 @@ struct ShortFormat {
 // A directory word holds the top bits of what the bucket hash leaves over and, below them, phase and operator.  All ones
 // there mark an empty slot, so that those two have one bit less, in short entries too.
 constexpr uint32_t DIR_ID_BITS = 12, DIR_ID_MASK = (1u << DIR_ID_BITS) - 1u;
+// Operator and phase as directory words and short entries hold them; khi = phase << 16 | operator.
+__device__ __forceinline__ uint32_t identity(uint32_t khi, uint32_t phase_bits) { return ((khi & 0xFFFFu) << phase_bits) + (khi >> 16); }
+// A directory slot's word (words form): the bits that the bucket leaves over of hash x buckets, phase and operator.
+__device__ __forceinline__ uint32_t dir_word(uint32_t product_lo, uint32_t khi, uint32_t phase_bits) {
+    return (product_lo & ~DIR_ID_MASK) | identity(khi, phase_bits);
+}
 constexpr uint32_t SHORT_ENTRY_BYTES = 8;
 constexpr uint32_t SHORT_CONTINUATION = 0x80000000u;   // in the high word
 

@@ -12,6 +12,14 @@
 namespace atrex {
 
 constexpr int FIN_THREADS = 256;
+
+// A word for the host in pinned memory: both halves carry the stamp of the answer they belong to and are stored whole, so
+// that the host sees for itself what has arrived.  (A flag behind the words has to wait for a fence of the system first, which is
+// a round trip over the link: 2 us of an answer.)
+__device__ __forceinline__ void tell(ulonglong2* to, ull word, uint32_t stamp) {
+    const ull mark = (ull)stamp << 32;
+    asm volatile("st.volatile.global.v2.u64 [%0], {%1, %2};" ::"l"(to), "l"(mark | (uint32_t)word), "l"(mark | (word >> 32)) : "memory");
+}
 constexpr uint32_t TOT_ILP = 6;
 
 struct SlotView {
@@ -212,6 +220,23 @@ __device__ __forceinline__ void store_entry(atrex_entry_t* dst, const atrex_entr
     q[2] = make_ulonglong2((ull)__double_as_longlong(e.phase_weight), (ull)__double_as_longlong(e.roofline_s));
 }
 
+// Row `row` of phase q's best, for the host.
+__device__ __forceinline__ void tell_row(const PickParams& p, uint32_t q, uint32_t row, const atrex_entry_t& e) {
+    if (p.k > TOPK_TOLD_K) {
+        store_entry(p.host_top + (size_t)q * TOPK_PICK_K + row, e);
+        return;
+    }
+    ulonglong2* to = p.host_told + ((size_t)q * TOPK_TOLD_K + row) * 6;
+    const ull words[6] = {e.key, e.count, e.wt_lo, e.wt_hi, (ull)__double_as_longlong(e.phase_weight), (ull)__double_as_longlong(e.roofline_s)};
+#pragma unroll
+    for (int i = 0; i < 6; ++i) tell(to + i, words[i], p.fin.stamp);
+}
+// ... and how many rows there are, PICK_NONE: not answered this way (one thread; all rows stored before)
+__device__ __forceinline__ void tell_count(const PickParams& p, uint32_t q, uint32_t n) {
+    if (p.k > TOPK_TOLD_K) __threadfence_system();      // (rows without stamps)
+    *(volatile ull*)&p.host_n[q] = (ull)p.fin.stamp << 32 | n;   // the host waits for this word
+}
+
 __device__ __forceinline__ void load_phase_totals(const Control* ctl, double* dT, bool* zeroT) {
     if (threadIdx.x < ATREX_MAX_PHASES) {
         ull lo = ctl->total_lo[threadIdx.x], hi = ctl->total_hi[threadIdx.x];
@@ -278,16 +303,8 @@ __global__ void __launch_bounds__(FIN_THREADS) emit_kernel(FinalizeParams p) {
     grid_dependents_launch();
     if (!last_cta(&p.ctl->emit_done)) return;
     // the host's copy of the counters and totals, straight to pinned memory
-    constexpr uint32_t WORDS = offsetof(Control, acc_lo) / 8;
-    constexpr uint32_t SEQ = offsetof(Control, seq) / 8;
-    if (threadIdx.x < WORDS && threadIdx.x != SEQ)
-        reinterpret_cast<ull*>(p.mirror)[threadIdx.x] = ld_relaxed(reinterpret_cast<const ull*>(p.ctl) + threadIdx.x);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        p.ctl->emit_done = 0;
-        __threadfence_system();
-        *(volatile ull*)&p.mirror->seq = p.seq;   // the host waits for this word
-    }
+    if (threadIdx.x < CONTROL_WORDS) tell(p.told + threadIdx.x, ld_relaxed(reinterpret_cast<const ull*>(p.ctl) + threadIdx.x), p.stamp);
+    if (threadIdx.x == 0) p.ctl->emit_done = 0;
 }
 
 // ---- work table ---------------------------------------------------------------------------
@@ -377,13 +394,10 @@ __device__ __forceinline__ uint32_t digit_in_quarter(const PickParams& p, uint32
     return found;
 }
 
-// the keys at or above that digit
-__global__ void __launch_bounds__(FIN_THREADS) topk_collect_kernel(const __grid_constant__ PickParams p) {
-    __shared__ uint32_t s_bin[ATREX_MAX_PHASES], s_sum[4 * ATREX_MAX_PHASES];
-    static_assert(FIN_THREADS / 32 >= ATREX_MAX_PHASES, "a warp per phase");
-    grid_dependency_wait();
+// the digit of every phase's k-th key (all threads of a CTA; PICK_NONE: too many keys to rank this way)
+__device__ __forceinline__ void find_digits(const PickParams& p, uint32_t* s_bin, uint32_t* s_sum) {
     const uint32_t warp = threadIdx.x >> 5;
-    for (uint32_t i = warp; i < 4 * p.n_phases; i += FIN_THREADS / 32) {
+    for (uint32_t i = warp; i < 4 * p.n_phases; i += blockDim.x / 32) {
         uint4 v[8];
         const uint32_t sum = load_quarter(p, i / 4, i % 4, v);
         if ((threadIdx.x & 31u) == 0) s_sum[i] = sum;
@@ -397,12 +411,18 @@ __global__ void __launch_bounds__(FIN_THREADS) topk_collect_kernel(const __grid_
             if (quarter < 4) digit = digit_in_quarter(p, warp, quarter, above);
             else digit = above <= TOPK_PICK_MAX ? 0u : PICK_NONE;              // fewer than k keys: all of them
         }
-        if ((threadIdx.x & 31u) == 0) {
-            s_bin[warp] = digit;
-            if (blockIdx.x == 0) p.fin.ctl->pick_bin[warp] = digit;
-        }
+        if ((threadIdx.x & 31u) == 0) s_bin[warp] = digit;
     }
     __syncthreads();
+}
+
+// the keys at or above that digit
+__global__ void __launch_bounds__(FIN_THREADS) topk_collect_kernel(const __grid_constant__ PickParams p) {
+    __shared__ uint32_t s_bin[ATREX_MAX_PHASES], s_sum[4 * ATREX_MAX_PHASES];
+    static_assert(FIN_THREADS / 32 >= ATREX_MAX_PHASES, "a warp per phase");
+    grid_dependency_wait();
+    find_digits(p, s_bin, s_sum);
+    if (blockIdx.x == 0 && threadIdx.x < ATREX_MAX_PHASES) p.fin.ctl->pick_bin[threadIdx.x] = s_bin[threadIdx.x];
     const TableRef& tab = p.fin.t;
     constexpr int ILP = 4;
     const ull stride = (ull)gridDim.x * FIN_THREADS, n_slots = p.fin.n_slots;
@@ -431,6 +451,39 @@ __global__ void __launch_bounds__(FIN_THREADS) topk_collect_kernel(const __grid_
     grid_dependents_launch();
 }
 
+// n candidates ranked: before(a, b) compares two of them, swap(a, b) exchanges them, emit(row, a) takes one of the best k
+// (all threads of a CTA)
+template <typename Before, typename Swap, typename Emit>
+__device__ __forceinline__ void rank_candidates(uint32_t n, uint32_t best, Before before, Swap swap, Emit emit) {
+    if (n <= 512) {     // every candidate counts those before it
+        if (threadIdx.x < n) {
+            uint32_t row = 0;
+            for (uint32_t j = 0; j < n; ++j) row += before(j, threadIdx.x) ? 1u : 0u;
+            if (row < best) emit(row, threadIdx.x);
+        }
+        return;
+    }
+    // bitonic network over positions 0 .. n - 1 (every comparator puts the better one first, so that
+    // positions beyond n can be left out)
+    for (uint32_t k = 2; k / 2 < n; k <<= 1) {
+        for (uint32_t j = k >> 1; j; j >>= 1) {
+            for (uint32_t t = threadIdx.x; t < n; t += blockDim.x) {
+                const uint32_t lo = (t / j) * 2 * j + (t & (j - 1));
+                const uint32_t hi = j == k >> 1 ? (lo | (k - 1)) - (lo & (k - 1)) : lo + j;
+                if (hi < n && before(hi, lo)) swap(lo, hi);
+            }
+            __syncthreads();
+        }
+    }
+    for (uint32_t i = threadIdx.x; i < min(n, best); i += blockDim.x) emit(i, i);
+}
+template <typename T>
+__device__ __forceinline__ void exchange(T& a, T& b) {
+    const T x = a;
+    a = b;
+    b = x;
+}
+
 // the candidates of each phase ranked: weighted time descending, key ascending (one CTA per phase)
 __global__ void __launch_bounds__(512) topk_rank_kernel(const __grid_constant__ PickParams p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -443,7 +496,7 @@ __global__ void __launch_bounds__(512) topk_rank_kernel(const __grid_constant__ 
     grid_dependency_wait();
     const uint32_t q = blockIdx.x;
     if (p.fin.ctl->pick_bin[q] == PICK_NONE) {
-        if (threadIdx.x == 0) *(volatile ull*)&p.host_n[q] = p.fin.seq << 32 | PICK_NONE;
+        if (threadIdx.x == 0) tell_count(p, q, PICK_NONE);
         return;
     }
     load_phase_totals(p.fin.ctl, dT, zeroT);
@@ -463,39 +516,18 @@ __global__ void __launch_bounds__(512) topk_rank_kernel(const __grid_constant__ 
     };
     auto emit = [&](uint32_t row, uint32_t i) {
         const SlotView v = load_slot(p.fin.t, s_at[i]);
-        store_entry(p.host_top + (size_t)q * TOPK_PICK_K + row, make_entry(v, dT, zeroT, p.fin));
+        tell_row(p, q, row, make_entry(v, dT, zeroT, p.fin));
     };
-    if (n <= 512) {     // every candidate counts those before it
-        if (threadIdx.x < n) {
-            uint32_t row = 0;
-            for (uint32_t j = 0; j < n; ++j) row += before(j, threadIdx.x) ? 1u : 0u;
-            if (row < p.k) emit(row, threadIdx.x);
-        }
-    } else {
-        // bitonic network over positions 0 .. n - 1 (every comparator puts the better one first, so that
-        // positions beyond n can be left out)
-        for (uint32_t k = 2; k / 2 < n; k <<= 1) {
-            for (uint32_t j = k >> 1; j; j >>= 1) {
-                for (uint32_t t = threadIdx.x; t < n; t += blockDim.x) {
-                    const uint32_t lo = (t / j) * 2 * j + (t & (j - 1));
-                    const uint32_t hi = j == k >> 1 ? (lo | (k - 1)) - (lo & (k - 1)) : lo + j;
-                    if (hi < n && before(hi, lo)) {
-                        ull x = s_hi[lo]; s_hi[lo] = s_hi[hi]; s_hi[hi] = x;
-                        x = s_lo[lo]; s_lo[lo] = s_lo[hi]; s_lo[hi] = x;
-                        x = s_key[lo]; s_key[lo] = s_key[hi]; s_key[hi] = x;
-                        const uint32_t y = s_at[lo]; s_at[lo] = s_at[hi]; s_at[hi] = y;
-                    }
-                }
-                __syncthreads();
-            }
-        }
-        for (uint32_t i = threadIdx.x; i < min(n, p.k); i += blockDim.x) emit(i, i);
-    }
+    rank_candidates(n, p.k, before, [&](uint32_t a, uint32_t b) {
+        exchange(s_hi[a], s_hi[b]);
+        exchange(s_lo[a], s_lo[b]);
+        exchange(s_key[a], s_key[b]);
+        exchange(s_at[a], s_at[b]);
+    }, emit);
     __syncthreads();
     if (threadIdx.x == 0) {
         p.fin.ctl->sel_count_all[q] = 0;   // (for the next request)
-        __threadfence_system();
-        *(volatile ull*)&p.host_n[q] = p.fin.seq << 32 | min(n, p.k);   // the host waits for this word
+        tell_count(p, q, min(n, p.k));
     }
 }
 
@@ -694,10 +726,317 @@ __global__ void __launch_bounds__(FIN_THREADS) topk_emit_kernel(FinalizeParams p
 // ---- launchers ----------------------------------------------------------------------------
 constexpr size_t PICK_SMEM = (size_t)TOPK_PICK_MAX * 28;
 
+// ---- small tables --------------------------------------------------------------------------
+// Up to 65 536 slots (some 25 000 keys) one cluster of 8 or 16 CTAs, four slots to a thread, does in one launch what takes
+// two above, and keeps the table in registers in between: the CTAs' sums and counts meet through distributed shared memory and
+// cluster barriers, where kernels of many CTAs pay for atomics to one address, a fence and a word counted per CTA, and the
+// next launch.  Latency-bound: SMALL_FIGURES
+constexpr uint32_t SMALL_THREADS = 1024, SMALL_ILP = 4, SMALL_CTA_SLOTS = SMALL_THREADS * SMALL_ILP, SMALL_CTAS_MAX = 16;
+constexpr uint32_t SMALL_PIECES = 7;                     // a phase's sums: weighted time in four pieces of 22 bits, count in two of 20, keys
+constexpr uint32_t SMALL_SUMS = ATREX_MAX_PHASES * SMALL_PIECES;
+constexpr size_t FINALIZE_SMALL_SMEM = SMALL_CTA_SLOTS * 24;
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ uint32_t remote_addr(const void* p, uint32_t rank) {   // of the same variable in another CTA of the cluster
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+    return a;
+}
+__device__ __forceinline__ ull remote_u64(const ull* p, uint32_t rank) {
+    ull v;
+    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(remote_addr(p, rank)) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t remote_u32(const uint32_t* p, uint32_t rank) {
+    uint32_t v;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(remote_addr(p, rank)) : "memory");
+    return v;
+}
+__device__ __forceinline__ ull warp_sum(ull v) {
+#pragma unroll
+    for (int d = 16; d; d >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, d);
+    return v;
+}
+
+__global__ void __launch_bounds__(SMALL_THREADS) finalize_small_kernel(const __grid_constant__ FinalizeParams p, uint32_t n_phases,
+                                                                       const __grid_constant__ GivenTotals given, uint32_t* hist, uint32_t* next_hist) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    ulonglong2* const q_val = reinterpret_cast<ulonglong2*>(smem_raw);              // [SMALL_CTA_SLOTS] the CTA's live slots side by side
+    ull* const q_key = reinterpret_cast<ull*>(q_val + SMALL_CTA_SLOTS);
+    __shared__ uint32_t s_warp[32][SMALL_SUMS], s_warp_live[32], s_live, s_base;
+    __shared__ ull s_cta[SMALL_SUMS], s_all[SMALL_SUMS], s_word[CONTROL_WORDS];
+    __shared__ double dT[ATREX_MAX_PHASES];
+    __shared__ bool zeroT[ATREX_MAX_PHASES];
+    const uint32_t t = threadIdx.x, lane = t & 31u, w = t >> 5, rank = cluster_rank(), ctas = gridDim.x;
+    Control* const ctl = p.ctl;
+    for (uint32_t i = t; i < 32 * SMALL_SUMS; i += SMALL_THREADS) (&s_warp[0][0])[i] = 0;
+    grid_dependency_wait();
+    ull sk[SMALL_ILP];
+    ulonglong2 x[SMALL_ILP];
+#pragma unroll
+    for (uint32_t u = 0; u < SMALL_ILP; ++u) {
+        const uint32_t i = (rank * SMALL_ILP + u) * SMALL_THREADS + t;
+        sk[u] = i < p.n_slots ? p.t.keys[i] : 0ull;
+        x[u] = i < p.n_slots ? p.t.vals[i] : make_ulonglong2(0, 0);
+    }
+    if (rank == 0 && t < CONTROL_WORDS) s_word[t] = ld_relaxed(reinterpret_cast<const ull*>(ctl) + t);   // for the host, who is told by the first CTA
+    for (uint32_t i = rank * SMALL_THREADS + t; i < n_phases * TOPK_BINS / 4; i += ctas * SMALL_THREADS)
+        reinterpret_cast<uint4*>(next_hist)[i] = make_uint4(0, 0, 0, 0);
+    // The live slots side by side: a table is hardly ever fuller than a half and often emptier than an eighth, and what follows
+    // is a few hundred instructions a warp.
+    uint32_t live = 0, at[SMALL_ILP];
+#pragma unroll
+    for (uint32_t u = 0; u < SMALL_ILP; ++u) {
+        const uint32_t votes = __ballot_sync(0xFFFFFFFFu, sk[u] != 0);
+        at[u] = live + __popc(votes & ((1u << lane) - 1u));
+        live += __popc(votes);
+    }
+    if (lane == 0) s_warp_live[w] = live;
+    __syncthreads();
+    uint32_t incl = s_warp_live[lane];
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t o = __shfl_up_sync(0xFFFFFFFFu, incl, d);
+        if (lane >= (uint32_t)d) incl += o;
+    }
+    const uint32_t n_live = __shfl_sync(0xFFFFFFFFu, incl, 31), mine = __shfl_sync(0xFFFFFFFFu, incl, w) - live;
+    if (t == 0) s_live = n_live;
+#pragma unroll
+    for (uint32_t u = 0; u < SMALL_ILP; ++u) {
+        if (sk[u] == 0) continue;
+        q_key[mine + at[u]] = ~sk[u];
+        q_val[mine + at[u]] = x[u];
+    }
+    __syncthreads();
+    double roofline[SMALL_ILP];
+    if (w * 32 < n_live) {
+        bool beyond = false;            // (a merged entry of a phase that records of this handle cannot have)
+#pragma unroll
+        for (uint32_t u = 0; u < SMALL_ILP; ++u) {
+            const uint32_t j = u * SMALL_THREADS + t;
+            if (j >= n_live) continue;
+            const uint32_t q = (uint32_t)(q_key[j] >> 48) & (ATREX_MAX_PHASES - 1);
+            if (q < n_phases) atomicAdd(&hist[q * TOPK_BINS + topk_first_digit(q_val[j].x, q_val[j].y >> HI_SHIFT)], 1u);
+            else beyond = true;
+        }
+        const uint32_t phases = __any_sync(0xFFFFFFFFu, beyond) ? ATREX_MAX_PHASES : n_phases;
+        for (uint32_t q = 0; q < phases; ++q) {
+            uint32_t c[SMALL_PIECES] = {0, 0, 0, 0, 0, 0, 0};
+#pragma unroll
+            for (uint32_t u = 0; u < SMALL_ILP; ++u) {
+                const uint32_t j = u * SMALL_THREADS + t;
+                if (j >= n_live || ((uint32_t)(q_key[j] >> 48) & (ATREX_MAX_PHASES - 1)) != q) continue;
+                const ull lo = q_val[j].x, hi = q_val[j].y >> HI_SHIFT, n = q_val[j].y & COUNT_MASK;
+                c[0] += (uint32_t)lo & 0x3FFFFFu;
+                c[1] += (uint32_t)(lo >> 22) & 0x3FFFFFu;
+                c[2] += (uint32_t)(lo >> 44) | ((uint32_t)hi & 3u) << 20;
+                c[3] += (uint32_t)(hi >> 2);
+                c[4] += (uint32_t)n & 0xFFFFFu;
+                c[5] += (uint32_t)(n >> 20);
+                c[6] += 1;
+            }
+            __syncwarp();
+#pragma unroll
+            for (uint32_t j = 0; j < SMALL_PIECES; ++j) {
+                const uint32_t sum = __reduce_add_sync(0xFFFFFFFFu, c[j]);       // (128 slots: below 2^29)
+                if (lane == j) s_warp[w][q * SMALL_PIECES + j] = sum;
+            }
+        }
+    }
+    __syncthreads();
+    for (uint32_t i = w; i < SMALL_SUMS; i += SMALL_THREADS / 32) {
+        const ull sum = warp_sum(s_warp[lane][i]);
+        if (lane == 0) s_cta[i] = sum;
+    }
+    __syncthreads();
+    cluster_arrive();
+    // (the roofline times need no totals: their look-ups overlap the barrier)
+#pragma unroll
+    for (uint32_t u = 0; u < SMALL_ILP; ++u) {
+        const uint32_t j = u * SMALL_THREADS + t;
+        roofline[u] = j < n_live ? roofline_time(p.work, p.peaks, q_key[j]) : 0.0;
+    }
+    __syncwarp();
+    cluster_wait();
+    for (uint32_t i = w; i <= SMALL_SUMS; i += SMALL_THREADS / 32) {
+        if (i < SMALL_SUMS) {
+            const ull sum = warp_sum(lane < ctas ? remote_u64(&s_cta[i], lane) : 0ull);
+            if (lane == 0) s_all[i] = sum;
+        } else {
+            const uint32_t n = lane < ctas ? remote_u32(&s_live, lane) : 0u;
+            const uint32_t before = __reduce_add_sync(0xFFFFFFFFu, lane < rank ? n : 0u), all = __reduce_add_sync(0xFFFFFFFFu, n);
+            if (lane == 0) {
+                s_base = before;
+                if (rank == 0) s_word[offsetof(Control, n_out) / 8] = ctl->n_out = all;
+            }
+        }
+    }
+    __syncthreads();
+    if (t < ATREX_MAX_PHASES) {
+        const ull* c = s_all + t * SMALL_PIECES;
+        ull lo = c[0], hi = c[3] << 2;
+        const ull add[2] = {c[1] << 22, c[2] << 44};
+        hi += (c[1] >> 42) + (c[2] >> 20);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            lo += add[j];
+            hi += lo < add[j] ? 1ull : 0ull;
+        }
+        if (given.use) {
+            lo = given.lo[t];
+            hi = given.hi[t];
+        }
+        dT[t] = u128_to_f64_rn(hi, lo);
+        zeroT[t] = (lo | hi) == 0;
+        if (rank == 0) {
+            s_word[offsetof(Control, total_lo) / 8 + t] = ctl->total_lo[t] = lo;
+            s_word[offsetof(Control, total_hi) / 8 + t] = ctl->total_hi[t] = hi;
+            s_word[offsetof(Control, count_per_phase) / 8 + t] = ctl->count_per_phase[t] = c[4] + (c[5] << 20);
+            s_word[offsetof(Control, keys_per_phase) / 8 + t] = ctl->keys_per_phase[t] = c[6];
+        }
+    }
+    __syncthreads();
+    grid_dependents_launch();
+#pragma unroll
+    for (uint32_t u = 0; u < SMALL_ILP; ++u) {
+        const uint32_t j = u * SMALL_THREADS + t;
+        const ull pos = s_base + j;
+        if (j >= n_live || pos >= p.out_cap) continue;
+        const ulonglong2 y = q_val[j];
+        atrex_entry_t e;
+        e.key = q_key[j];
+        e.count = y.y & COUNT_MASK;
+        e.wt_lo = y.x;
+        e.wt_hi = y.y >> HI_SHIFT;
+        const uint32_t q = (uint32_t)(e.key >> 48) & (ATREX_MAX_PHASES - 1);
+        e.phase_weight = zeroT[q] ? 0.0 : __ddiv_rn(u128_to_f64_rn(e.wt_hi, e.wt_lo), dT[q]);
+        e.roofline_s = roofline[u];
+        store_entry(p.out + pos, e);
+    }
+    __syncthreads();
+    if (t == 0) __threadfence();
+    cluster_arrive();                   // (no CTA leaves while another reads its shared memory, and the host is told last)
+    cluster_wait();
+    if (rank == 0 && t < CONTROL_WORDS) tell(p.told + t, s_word[t], p.stamp);
+}
+
+// Top-k of every phase of a small table in one launch: every CTA finds the digits and lists its candidates in shared
+// memory, CTA q gathers those of phase q and ranks them.
+struct SmallPick {
+    ull key[SMALL_CTA_SLOTS], lo[SMALL_CTA_SLOTS], cnthi[SMALL_CTA_SLOTS];            // this CTA's candidates
+    ull g_key[TOPK_PICK_MAX], g_lo[TOPK_PICK_MAX], g_cnthi[TOPK_PICK_MAX];            // this phase's
+};
+__global__ void __launch_bounds__(SMALL_THREADS) topk_small_kernel(const __grid_constant__ PickParams p) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    SmallPick& s = *reinterpret_cast<SmallPick*>(smem_raw);
+    __shared__ uint32_t s_bin[ATREX_MAX_PHASES], s_sum[4 * ATREX_MAX_PHASES], s_n, s_gathered;
+    __shared__ double dT[ATREX_MAX_PHASES];
+    __shared__ bool zeroT[ATREX_MAX_PHASES];
+    const uint32_t t = threadIdx.x, lane = t & 31u, w = t >> 5, rank = cluster_rank(), ctas = gridDim.x;
+    if (t == 0) s_n = s_gathered = 0;
+    grid_dependency_wait();
+    ull sk[SMALL_ILP];
+    ulonglong2 x[SMALL_ILP];
+#pragma unroll
+    for (uint32_t u = 0; u < SMALL_ILP; ++u) {
+        const uint32_t i = (rank * SMALL_ILP + u) * SMALL_THREADS + t;
+        sk[u] = i < p.fin.n_slots ? p.fin.t.keys[i] : 0ull;
+        x[u] = i < p.fin.n_slots ? p.fin.t.vals[i] : make_ulonglong2(0, 0);
+    }
+    find_digits(p, s_bin, s_sum);
+#pragma unroll
+    for (uint32_t u = 0; u < SMALL_ILP; ++u) {
+        if (sk[u] == 0) continue;
+        const uint32_t q = (uint32_t)(~sk[u] >> 48) & (ATREX_MAX_PHASES - 1);
+        if (topk_first_digit(x[u].x, x[u].y >> HI_SHIFT) < s_bin[q]) continue;      // (PICK_NONE: never)
+        const uint32_t at = atomicAdd(&s_n, 1u);
+        s.key[at] = ~sk[u];
+        s.lo[at] = x[u].x;
+        s.cnthi[at] = x[u].y;
+    }
+    __syncthreads();
+    cluster_arrive();
+    cluster_wait();
+    const bool ranks = rank < p.n_phases && s_bin[rank] != PICK_NONE;
+    if (ranks) {
+        for (uint32_t r = w; r < ctas; r += SMALL_THREADS / 32) {
+            const uint32_t n = remote_u32(&s_n, r);
+            for (uint32_t i = lane; i < n; i += 32) {
+                const ull key = remote_u64(&s.key[i], r);
+                if (((uint32_t)(key >> 48) & (ATREX_MAX_PHASES - 1)) != rank) continue;
+                const uint32_t at = atomicAdd(&s_gathered, 1u);
+                if (at >= TOPK_PICK_MAX) continue;                               // (cannot happen: the digits were chosen so)
+                s.g_key[at] = key;
+                s.g_lo[at] = remote_u64(&s.lo[i], r);
+                s.g_cnthi[at] = remote_u64(&s.cnthi[i], r);
+            }
+        }
+        load_phase_totals(p.fin.ctl, dT, zeroT);      // (a barrier of the CTA)
+    }
+    cluster_arrive();                 // nobody reads anybody's shared memory any more
+    if (ranks) {
+        const uint32_t n = min(s_gathered, TOPK_PICK_MAX);
+        const auto before = [&](uint32_t a, uint32_t b) {
+            const ull ha = s.g_cnthi[a] >> HI_SHIFT, hb = s.g_cnthi[b] >> HI_SHIFT;
+            if (ha != hb) return ha > hb;
+            if (s.g_lo[a] != s.g_lo[b]) return s.g_lo[a] > s.g_lo[b];
+            return s.g_key[a] < s.g_key[b];
+        };
+        const auto swap = [&](uint32_t a, uint32_t b) {
+            exchange(s.g_key[a], s.g_key[b]);
+            exchange(s.g_lo[a], s.g_lo[b]);
+            exchange(s.g_cnthi[a], s.g_cnthi[b]);
+        };
+        rank_candidates(n, p.k, before, swap, [&](uint32_t row, uint32_t i) {
+            SlotView v;
+            v.key = s.g_key[i];
+            v.live = true;
+            v.lo = s.g_lo[i];
+            v.count = s.g_cnthi[i] & COUNT_MASK;
+            v.hi = s.g_cnthi[i] >> HI_SHIFT;
+            tell_row(p, rank, row, make_entry(v, dT, zeroT, p.fin));
+        });
+    }
+    __syncthreads();
+    if (t == 0 && rank < p.n_phases) tell_count(p, rank, ranks ? min(min(s_gathered, TOPK_PICK_MAX), p.k) : PICK_NONE);
+    cluster_wait();
+}
+
+uint32_t small_ctas(ull n_slots) { return n_slots <= 8 * SMALL_CTA_SLOTS ? 8u : 16u; }
+
+// One cluster, set up while its predecessor on the stream is still running (see launch_chained).
+template <typename... P, typename... A>
+cudaError_t launch_cluster(void (*kernel)(P...), uint32_t ctas, size_t smem, cudaStream_t stream, const A&... args) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(ctas);
+    c.blockDim = dim3(SMALL_THREADS);
+    c.dynamicSmemBytes = smem;
+    c.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = ctas;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = attr;
+    c.numAttrs = 2;
+    return cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+
 cudaError_t finalize_prepare() {
     cudaError_t e = cudaFuncSetAttribute(totals_kernel<TOT_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)totals_smem(TOT_WIDE_FROM - 1));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(totals_kernel<2 * TOT_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)totals_smem(ATREX_MAX_PHASES));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(topk_rank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PICK_SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(finalize_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FINALIZE_SMALL_SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(finalize_small_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(topk_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmallPick));
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(topk_small_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(topk_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ATREX_MAX_PHASES * TOPK_BINS * 4);
     return e;
 }
@@ -724,7 +1063,14 @@ cudaError_t launch_work_insert(const atrex_work_t* rows, ull n, const WorkRef& w
     return cudaGetLastError();
 }
 
+bool finalize_is_small(ull n_slots) { return n_slots <= (ull)SMALL_CTAS_MAX * SMALL_CTA_SLOTS; }
+
+cudaError_t launch_finalize_small(const FinalizeParams& p, uint32_t n_phases, const GivenTotals& given, uint32_t* hist, uint32_t* next_hist, cudaStream_t stream) {
+    return launch_cluster(finalize_small_kernel, small_ctas(p.n_slots), FINALIZE_SMALL_SMEM, stream, p, n_phases, given, hist, next_hist);
+}
+
 cudaError_t launch_topk_pick(const PickParams& p, int n_sms, cudaStream_t stream) {
+    if (finalize_is_small(p.fin.n_slots)) return launch_cluster(topk_small_kernel, small_ctas(p.fin.n_slots), sizeof(SmallPick), stream, p);
     static const uint32_t per_sm = resident_ctas(topk_collect_kernel, FIN_THREADS, 0);
     cudaError_t e = launch_chained(topk_collect_kernel, grid_for_work(p.fin.n_slots, FIN_THREADS * 4, n_sms, per_sm), FIN_THREADS, 0, stream, p);
     if (e == cudaSuccess) e = launch_chained(topk_rank_kernel, p.n_phases, 512, PICK_SMEM, stream, p);

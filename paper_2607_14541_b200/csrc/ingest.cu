@@ -969,7 +969,9 @@ __global__ void __launch_bounds__(128) hot_pick_kernel(HotBuildParams p) {
     __syncthreads();
     grid_dependency_wait();
     HotBuildScratch& x = *p.scratch;
-    const uint32_t b = blockIdx.x * 128 + threadIdx.x, ways = buckets_in_use(p).ways;
+    const uint32_t b = blockIdx.x * 128 + threadIdx.x;
+    const Buckets buckets = buckets_in_use(p);
+    const uint32_t ways = buckets.ways, mult = best_multiplier(x);
     uint32_t inserted = 0, weight = 0;
     if (b < p.hot_slots / ways) {        // (the whole image: buckets that are not in use have nothing listed)
         const uint32_t n = min(x.listed[b], LIST_MAX);
@@ -997,8 +999,19 @@ __global__ void __launch_bounds__(128) hot_pick_kernel(HotBuildParams p) {
         }
         ulonglong2* dst = reinterpret_cast<ulonglong2*>(p.hot_keys + b * ways);
         dst[0] = make_ulonglong2(keys[0], keys[1]);
-        if (ways == TAG_WAYS) dst[1] = make_ulonglong2(keys[2], keys[3]);
-        if (b == 0) p.ctl->dir_mult = best_multiplier(x);
+        if (ways == TAG_WAYS) {
+            dst[1] = make_ulonglong2(keys[2], keys[3]);
+        } else {   // (worked out here once and not by every CTA of every scatter launch)
+            uint32_t word[WORD_WAYS];
+#pragma unroll
+            for (uint32_t way = 0; way < WORD_WAYS; ++way) {
+                const uint32_t khi = (uint32_t)(~keys[way] >> 32) & 0x00FFFFFFu;
+                const uint32_t left = dir_mix(hash32(~keys[way]), khi >> 16, mult) * buckets.n;
+                word[way] = keys[way] ? dir_word(left, khi, p.phase_bits) : DIR_ID_MASK;
+            }
+            reinterpret_cast<uint2*>(p.hot_words)[b] = make_uint2(word[0], word[1]);
+        }
+        if (b == 0) p.ctl->dir_mult = mult;
     }
     inserted = __reduce_add_sync(0xFFFFFFFFu, inserted);
     weight = __reduce_add_sync(0xFFFFFFFFu, weight);

@@ -50,6 +50,7 @@ struct IngestParams {
     ShortFormat fmt;           // short spill entries and directory words
     const ull* hot_keys;       // directory image, hot_slots entries of ~key (0 = empty)
     uint32_t hot_slots;        // multiple of 4
+    const uint4* hot_words;    // the slots' words (words form)
     uint32_t img_rows;         // rows of hot_img that hold sums since the last fold; a CTA beyond them starts its row afresh
     ulonglong2* hot_img;       // [n_groups][hot_slots] each CTA's directory sums since the last fold, {lo, count | hi << 40}
     TableRef t;
@@ -119,6 +120,8 @@ struct HotBuildParams {
     uint32_t max_ops;          // as in ShortFormat (0: no short entries)
     ull* hot_keys;
     uint32_t hot_slots;        // of the image
+    uint32_t* hot_words;       // [hot_slots] (words form)
+    uint32_t phase_bits;       // as in ShortFormat
     uint32_t slots[2][2];      // slots in use by [words][one key dominates]
     ull* sample;               // [n_sample] the sampled keys, all ones = invalid record
     uint32_t* sketch;          // [2^20] sample counters by hash
@@ -140,8 +143,8 @@ struct FinalizeParams {
     TableRef t;
     ull n_slots;
     Control* ctl;
-    Control* mirror;     // pinned host memory, filled by the emit kernel, `seq` last
-    ull seq;
+    ulonglong2* told;    // pinned: the control block's first CONTROL_WORDS words for the host, each with the stamp
+    uint32_t stamp;
     WorkRef work;
     atrex_hw_peaks_t peaks;
     atrex_entry_t* out;
@@ -159,8 +162,9 @@ struct PickParams {
     uint32_t n_phases, k;
     uint32_t* hist;            // [n_phases][TOPK_BINS] first-digit counts
     ull* sel;                  // [n_phases][TOPK_PICK_MAX][4]
-    atrex_entry_t* host_top;   // pinned: [n_phases][TOPK_PICK_K]
-    ull* host_n;               // pinned: [n_phases] fin.seq << 32 | entries written (PICK_NONE: not answered this way)
+    atrex_entry_t* host_top;   // pinned: [n_phases][TOPK_PICK_K] (k > TOPK_TOLD_K)
+    ulonglong2* host_told;     // pinned: [n_phases][TOPK_TOLD_K][6] rows with stamps (smaller k)
+    ull* host_n;               // pinned: [n_phases] fin.stamp << 32 | entries written (PICK_NONE: not answered this way)
 };
 
 // Top-k, the long way: phases in one pass over the table, each with its own place in the ranking (see finalize.cu).
@@ -249,6 +253,9 @@ cudaError_t finalize_prepare();
 cudaError_t launch_totals(const TableRef& t, ull n_slots, uint32_t n_phases, const GivenTotals& given, uint32_t* hist, uint32_t* next_hist, int n_sms,
                           cudaStream_t stream);
 cudaError_t launch_emit(const FinalizeParams& p, int n_sms, cudaStream_t stream);
+bool finalize_is_small(ull n_slots);       // totals and entries in one launch
+cudaError_t launch_finalize_small(const FinalizeParams& p, uint32_t n_phases, const GivenTotals& given, uint32_t* hist, uint32_t* next_hist,
+                                  cudaStream_t stream);
 cudaError_t launch_work_insert(const atrex_work_t* rows, ull n, const WorkRef& w, Control* ctl, int grid,
                                cudaStream_t stream);
 cudaError_t launch_topk_pick(const PickParams& p, int n_sms, cudaStream_t stream);

@@ -54,7 +54,7 @@ struct Smem {
     static constexpr uint32_t APPW = CUR + 4u * P;              // u32[APPW_SMEM_MAX]  card-hour weights
     static constexpr uint32_t LONG = APPW + 4u * APPW_SMEM_MAX;    // words: records that took two short entries
     static constexpr uint32_t RESTS = LONG + 4u;                // ... whether an entry's identity has a rest
-    static constexpr uint32_t WORDS = LONG + 8u;                // ... u32[SLOTS]
+    static constexpr uint32_t WORDS = LONG + 16u;               // ... u32[SLOTS]
     static constexpr uint32_t TAG = LONG;                       // tags: u32[NB + 1]  four 8-bit tags per bucket (+ one pad bucket)
     static constexpr uint32_t KEYS = (TAG + 4u * (NB + 1u) + 7u) & ~7u;   // ull[SLOTS + 4]  key, all ones = empty
     static constexpr uint32_t PAD = W ? 0u : TAG_WAYS;          // (a look-up without a match reads the slot behind its bucket)
@@ -218,9 +218,6 @@ __device__ __forceinline__ void spill_append(const IngestParams& p, Ctx& c, bool
     }
 }
 
-// Operator and phase as directory words and short entries hold them (see ShortFormat).
-__device__ __forceinline__ uint32_t identity(uint32_t khi, uint32_t phase_bits) { return ((khi & 0xFFFFu) << phase_bits) + (khi >> 16); }
-
 // The same as a short entry (ShortFormat), in one store; a duration that does not fit takes a second entry behind it.
 template <uint32_t LP, int DIR>
 __device__ __forceinline__ void short_append(const IngestParams& p, Ctx& c, bool todo, uint32_t khi, uint32_t app, uint32_t shape,
@@ -248,11 +245,6 @@ __device__ __forceinline__ void short_append(const IngestParams& p, Ctx& c, bool
         reds_add(cw, 0u - n);
         count_overflow(p.t, ((ull)khi << 32) | shape, prod, h);
     }
-}
-
-// A directory slot's word (words form): the bits that the bucket leaves over of hash x buckets, phase and operator.
-__device__ __forceinline__ uint32_t dir_word(uint32_t product_lo, uint32_t khi, uint32_t phase_bits) {
-    return (product_lo & ~DIR_ID_MASK) | identity(khi, phase_bits);
 }
 
 // One record, start to finish (the register-staged loop has no registers to spare for working on
@@ -740,17 +732,14 @@ __device__ __forceinline__ void scatter_cta(const IngestParams& p, Ctx& c, unsig
     uint32_t* g_acc = reinterpret_cast<uint32_t*>(smem_raw + L::ACC);
     const ull skew = DIR != DIR_NONE ? p.t.ctl->hot_skew : SKEW_NONE;
     if (L::W && threadIdx.x < 2) reinterpret_cast<uint32_t*>(smem_raw + L::LONG)[threadIdx.x] = 0;
-    if (DIR != DIR_NONE) {
+    if (L::W) {
+        for (uint32_t i = threadIdx.x; i < L::SLOTS / 4; i += blockDim.x) reinterpret_cast<uint4*>(smem_raw + L::WORDS)[i] = p.hot_words[i];
+        for (uint32_t i = threadIdx.x; i < L::SLOTS * 3 / 4; i += blockDim.x) reinterpret_cast<uint4*>(g_acc)[i] = make_uint4(0, 0, 0, 0);
+    } else if (DIR != DIR_NONE) {
         for (uint32_t i = threadIdx.x; i < L::SLOTS + L::PAD; i += blockDim.x) {
             const ull image = i < L::SLOTS && !empty ? p.hot_keys[i] : 0ull;   // ~key, 0 = empty
-            const uint32_t khi = (uint32_t)(~image >> 32), x = dir_mix(hash32(~image), (khi >> 16) & 0xFFu, c.mult);
-            if (L::W) {
-                const uint32_t left = x * (skew == SKEW_DOMINATED ? L::NB_DOM : L::NB);
-                reinterpret_cast<uint32_t*>(smem_raw + L::WORDS)[i] = image ? dir_word(left, khi & 0x00FFFFFFu, p.fmt.phase_bits) : DIR_ID_MASK;
-            } else {
-                reinterpret_cast<ull*>(smem_raw + L::KEYS)[i] = ~image;
-                (smem_raw + L::TAG)[i] = image ? (unsigned char)(x & 0xFFu) : 0;
-            }
+            reinterpret_cast<ull*>(smem_raw + L::KEYS)[i] = ~image;
+            (smem_raw + L::TAG)[i] = image ? (unsigned char)(dir_mix(hash32(~image), (uint32_t)(~image >> 48) & 0xFFu, c.mult) & 0xFFu) : 0;
             g_acc[3 * i] = 0;
             g_acc[3 * i + 1] = 0;
             g_acc[3 * i + 2] = 0;
