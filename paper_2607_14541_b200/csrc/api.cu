@@ -146,7 +146,7 @@ void compute_layout(const atrex_agg_config_t* c, size_t smem_optin, int n_sms, L
     L->off_spill_cnt = o;      o += round_up(((size_t)L->n_groups << L->lp) * 4, ALIGN);
     L->off_keys = o;           o += round_up(L->n_slots * 8, ALIGN);
     L->off_vals = o;           o += round_up(L->n_slots * 16, ALIGN);
-    L->off_work = o;           o += round_up(L->work_slots * sizeof(WorkSlot), ALIGN);
+    L->off_work = o;           o += round_up(L->work_slots * WORK_SLOT_BYTES, ALIGN);
     L->off_appw = o;           o += round_up((size_t)c->n_apps * 4, ALIGN);
     L->off_hot = o;            o += round_up((size_t)(L->hot_slots ? L->hot_slots : 2) * 8, ALIGN);
     L->off_hot_words = o;      o += round_up((size_t)(L->hot_slots ? L->hot_slots : 2) * 4, ALIGN);
@@ -201,7 +201,7 @@ struct atrex_agg {
     unsigned char* spill = nullptr;
     ulonglong2* queue = nullptr;
     unsigned char* hot_scratch = nullptr;
-    WorkSlot* work = nullptr;
+    ull* work = nullptr;      // keys, the rows behind them
     uint32_t* d_appw = nullptr;
     ull* hot_keys = nullptr;
     ulonglong2* hot_img = nullptr;   // [n_groups][hot_slots] per-CTA directory sums not yet in the table
@@ -258,7 +258,8 @@ struct atrex_agg {
     }
     WorkRef work_ref() const {
         WorkRef w;
-        w.table = L.work_slots ? work : nullptr;
+        w.keys = L.work_slots ? work : nullptr;
+        w.rows = (double2*)(work + L.work_slots);
         w.lp = L.lp;
         w.Cw = L.Cw;
         w.strides = work_strides;
@@ -348,7 +349,7 @@ int atrex_agg_create(const atrex_agg_config_t* cfg, atrex_agg_t** out) {
         }
         const Layout& L = h->L;
         h->key_strides = atrex_agg::strides_for(L.C / 2);   // in slot pairs
-        h->work_strides = atrex_agg::strides_for(L.Cw ? L.Cw : 1);
+        h->work_strides = atrex_agg::strides_for(L.Cw ? L.Cw / WORK_WAYS : 1);
         h->ctl = (Control*)(h->ws + L.off_ctl);
         h->keys = (ull*)(h->ws + L.off_keys);
         h->vals = (ulonglong2*)(h->ws + L.off_vals);
@@ -356,7 +357,7 @@ int atrex_agg_create(const atrex_agg_config_t* cfg, atrex_agg_t** out) {
         h->spill = h->ws + L.off_spill;
         h->queue = (ulonglong2*)(h->ws + L.off_queue);
         h->hot_scratch = h->ws + L.off_hot_scratch;
-        h->work = (WorkSlot*)(h->ws + L.off_work);
+        h->work = (ull*)(h->ws + L.off_work);
         h->d_appw = (uint32_t*)(h->ws + L.off_appw);
         h->hot_keys = (ull*)(h->ws + L.off_hot);
         h->hot_img = (ulonglong2*)(h->ws + L.off_hot_img);
@@ -438,7 +439,7 @@ int atrex_agg_set_work_table(atrex_agg_t* h, const atrex_work_t* rows, uint64_t 
     DeviceGuard guard(h->cfg.device);
     cudaStream_t s = (cudaStream_t)stream;
     if (h->L.work_slots == 0) return ATREX_OK;
-    CU(h, cudaMemsetAsync(h->work, 0, h->L.work_slots * sizeof(WorkSlot), s));
+    CU(h, cudaMemsetAsync(h->work, 0, h->L.work_slots * sizeof(ull), s));
     CU(h, cudaMemsetAsync(&h->ctl->work_status, 0, sizeof(ull), s));
     const uint64_t per_piece = STAGING_BYTES / sizeof(atrex_work_t);
     for (uint64_t off = 0; off < n; off += per_piece) {
@@ -452,7 +453,7 @@ int atrex_agg_set_work_table(atrex_agg_t* h, const atrex_work_t* rows, uint64_t 
     CU(h, cudaStreamSynchronize(s));
     h->finalized = false;
     if (h->h_ctl->work_status != 0) {
-        CU(h, cudaMemsetAsync(h->work, 0, h->L.work_slots * sizeof(WorkSlot), s));
+        CU(h, cudaMemsetAsync(h->work, 0, h->L.work_slots * sizeof(ull), s));
         CU(h, cudaStreamSynchronize(s));
         return ATREX_ERR_INVALID;
     }

@@ -17,8 +17,10 @@
 //                 (ShortFormat below), and [G][P] counts,
 //                 written by CTA g of the scatter pass (its buffers are contiguous, which keeps
 //                 the scattered appends within a few pages), read by CTA p of the partition pass
-//   work table  : the same P partitions (by the same hash of op_id and shape_id) of Cw 32-byte
-//                 slots {~(op_id << 32 | shape_id), flops, bytes, dtype}, probed inside the partition
+//   work table  : the same P partitions (by the same hash of op_id and shape_id) of Cw slots, structure of arrays:
+//                   keys[P*Cw]  used (bit 63) | dtype << 48 | op_id << 32 | shape_id, in buckets of four
+//                   rows[P*Cw]  {flops, bytes} as binary64
+//                 probed inside the partition
 //   control     : counters, per-phase totals
 #pragma once
 #include <cstddef>
@@ -31,13 +33,10 @@ namespace atrex {
 
 typedef unsigned long long ull;
 
-struct WorkSlot {
-    ull skey;      // ~(op_id << 32 | shape_id), 0 = EMPTY
-    ull flops;
-    ull bytes;
-    ull dtype;
-};
-static_assert(sizeof(WorkSlot) == 32, "one slot per 32-byte sector");
+// A key of the work table: the pair with its data type above it, 0 = EMPTY
+constexpr ull WORK_USED = 1ull << 63;
+constexpr uint32_t WORK_WAYS = 4;             // keys to a bucket: one 32-byte sector
+constexpr uint32_t WORK_SLOT_BYTES = 8 + 16;  // key; flops and bytes
 
 constexpr ull COUNT_MASK = (1ull << 40) - 1;
 constexpr int HI_SHIFT = 40;

@@ -169,33 +169,54 @@ __global__ void __launch_bounds__(THREADS) totals_kernel(TableRef tab, ull n_slo
 }
 
 // ---- per-key results ----------------------------------------------------------------------
-// The work table is probed by double hashing (strides coprime to the partition's slot count): with
-// linear probing the longest of a warp's 32 probe sequences -- which is what the warp waits for --
-// was several times the average.
+// The work table is probed a bucket of four keys at a time (one 32-byte load), from bucket to bucket by double hashing
+// (strides coprime to the partition's bucket count): the longest of a warp's 32 probe sequences is what the warp waits for.
+// Slot by slot it was eight loads; with linear probing several times that.  Buckets fill from the first way on.
+constexpr ull WORK_PAIR = 0x0000FFFFFFFFFFFFull;
 __device__ __forceinline__ uint32_t work_stride(const WorkRef& w, uint32_t h) {
     return (uint32_t)(w.strides >> (8 * ((h >> 3) & 7u))) & 0xFFu;
 }
-__device__ __forceinline__ uint32_t work_start(const WorkRef& w, uint32_t h) { return __umulhi(h * 0x85EBCA6Bu, w.Cw); }
+__device__ __forceinline__ uint32_t work_start(const WorkRef& w, uint32_t h) { return __umulhi(h * 0x85EBCA6Bu, w.Cw / WORK_WAYS); }
+__device__ __forceinline__ uint32_t work_next(const WorkRef& w, uint32_t bucket, uint32_t advance) {
+    bucket += advance;
+    while (bucket >= w.Cw / WORK_WAYS) bucket -= w.Cw / WORK_WAYS;    // (a small table's stride may be longer than the table)
+    return bucket;
+}
+struct WorkKeys {
+    ull k[WORK_WAYS];
+};
+__device__ __forceinline__ WorkKeys load_work_keys(const ull* bucket) {
+    WorkKeys x;
+    asm("ld.global.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(x.k[0]), "=l"(x.k[1]), "=l"(x.k[2]), "=l"(x.k[3]) : "l"(bucket));
+    return x;
+}
+// The way that holds `pair`, WORK_WAYS if none does; `dtype` is set where one does.
+__device__ __forceinline__ uint32_t work_way(const WorkKeys& x, ull pair, uint32_t& dtype) {
+    uint32_t way = WORK_WAYS;
+#pragma unroll
+    for (uint32_t i = 0; i < WORK_WAYS; ++i) {
+        if (((x.k[i] ^ (WORK_USED | pair)) & (WORK_USED | WORK_PAIR)) != 0) continue;
+        way = i;
+        dtype = (uint32_t)(x.k[i] >> 48) & (ATREX_MAX_DTYPES - 1);
+    }
+    return way;
+}
+__device__ __forceinline__ double roofline_of(const double2& work, uint32_t dtype, const atrex_hw_peaks_t& pk) {
+    return fmax(__ddiv_rn(work.x, pk.peak_flops[dtype]), __ddiv_rn(work.y, pk.peak_bw));
+}
 __device__ __forceinline__ double roofline_time(const WorkRef& w, const atrex_hw_peaks_t& pk, ull key) {
     const double qnan = __longlong_as_double(0x7FF8000000000000ll);
-    if (w.table == nullptr) return qnan;
-    ull pair = key & 0x0000FFFFFFFFFFFFull;
-    ull skey = ~pair;
-    const uint32_t h = hash32(pair);
-    const WorkSlot* part = w.table + (ull)part_of(h, w.lp) * w.Cw;
-    uint32_t s = work_start(w, h);
-    const uint32_t advance = work_stride(w, h);
-    for (uint32_t probe = 0; probe < w.Cw; ++probe) {
-        const WorkSlot* e = part + s;
-        ull k = e->skey;
-        if (k == skey) {
-            double t_compute = __ddiv_rn(__ull2double_rn(e->flops), pk.peak_flops[e->dtype & (ATREX_MAX_DTYPES - 1)]);
-            double t_memory = __ddiv_rn(__ull2double_rn(e->bytes), pk.peak_bw);
-            return fmax(t_compute, t_memory);
-        }
-        if (k == 0) break;
-        s += advance;
-        if (s >= w.Cw) s -= w.Cw;
+    if (w.keys == nullptr) return qnan;
+    const uint32_t h = hash32(key & WORK_PAIR), first = part_of(h, w.lp) * w.Cw, advance = work_stride(w, h);
+    uint32_t bucket = work_start(w, h);
+    for (uint32_t probe = 0; probe < w.Cw / WORK_WAYS; ++probe) {
+        const uint32_t at = first + bucket * WORK_WAYS;
+        const WorkKeys x = load_work_keys(w.keys + at);
+        uint32_t dtype = 0;
+        const uint32_t way = work_way(x, key & WORK_PAIR, dtype);
+        if (way != WORK_WAYS) return roofline_of(w.rows[at + way], dtype, pk);
+        if (x.k[WORK_WAYS - 1] == 0) break;
+        bucket = work_next(w, bucket, advance);
     }
     return qnan;
 }
@@ -248,57 +269,116 @@ __device__ __forceinline__ void load_phase_totals(const Control* ctl, double* dT
 
 // Each warp looks at 128 slots per round (four coalesced rows), queues the live ones in shared
 // memory and then works through the queue with all lanes busy: at a table load of a third, the
-// divisions and the work-table probe run on full warps instead of one lane in three.
+// divisions and the work-table probe run on full warps instead of one lane in three.  A lane probes for two
+// entries side by side (four need more registers than four CTAs per SM have, and three CTAs are slower), and the entries
+// go out through shared memory in whole lines.  Bound by latency and instructions at half occupancy (3.1 M keys
+// of 5.8 M slots: 121 -> 97 us, DRAM 45 %; 15 M of 23.6 M: 540 -> 475; one entry at a time over the same buckets 155, four
+// 113; five CTAs of 48 registers: 2 % more on the whole refresh).
 constexpr int EMIT_ILP = 4;
+constexpr int EMIT_PROBES = 2;
 constexpr int EMIT_WARPS = FIN_THREADS / 32;
 
-__global__ void __launch_bounds__(FIN_THREADS) emit_kernel(FinalizeParams p) {
+__global__ void __launch_bounds__(FIN_THREADS) emit_kernel(const __grid_constant__ FinalizeParams p) {
     __shared__ double dT[ATREX_MAX_PHASES];
     __shared__ bool zeroT[ATREX_MAX_PHASES];
     __shared__ ull q_key[EMIT_WARPS][32 * EMIT_ILP];
     __shared__ ulonglong2 q_val[EMIT_WARPS][32 * EMIT_ILP];
+    __shared__ ulonglong2 s_out[EMIT_WARPS][32 * 3];
     grid_dependency_wait();
     load_phase_totals(p.ctl, dT, zeroT);
     const unsigned lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
     const ull stride = (ull)gridDim.x * blockDim.x;
     const ull rounds = (p.n_slots + stride * EMIT_ILP - 1) / (stride * EMIT_ILP);  // uniform: warps stay converged
     for (ull r = 0; r < rounds; ++r) {
-        ull sk[EMIT_ILP];
-        ulonglong2 xv[EMIT_ILP];
-#pragma unroll
-        for (int u = 0; u < EMIT_ILP; ++u) {
-            const ull i = (r * EMIT_ILP + u) * stride + (ull)blockIdx.x * blockDim.x + threadIdx.x;
-            sk[u] = i < p.n_slots ? p.t.keys[i] : 0ull;
-            xv[u] = i < p.n_slots ? p.t.vals[i] : make_ulonglong2(0, 0);  // with the key, not after it
-        }
         uint32_t total = 0;
+        {
+            ull sk[EMIT_ILP];
+            ulonglong2 xv[EMIT_ILP];
 #pragma unroll
-        for (int u = 0; u < EMIT_ILP; ++u) {
-            const unsigned live = __ballot_sync(0xFFFFFFFFu, sk[u] != 0);
-            if (sk[u] != 0) {
-                const uint32_t at = total + __popc(live & ((1u << lane) - 1u));
-                q_key[w][at] = ~sk[u];
-                q_val[w][at] = xv[u];
+            for (int u = 0; u < EMIT_ILP; ++u) {
+                const ull i = (r * EMIT_ILP + u) * stride + (ull)blockIdx.x * blockDim.x + threadIdx.x;
+                sk[u] = i < p.n_slots ? p.t.keys[i] : 0ull;
+                xv[u] = i < p.n_slots ? p.t.vals[i] : make_ulonglong2(0, 0);  // with the key, not after it
             }
-            total += __popc(live);
+#pragma unroll
+            for (int u = 0; u < EMIT_ILP; ++u) {
+                const unsigned live = __ballot_sync(0xFFFFFFFFu, sk[u] != 0);
+                if (sk[u] != 0) {
+                    const uint32_t at = total + __popc(live & ((1u << lane) - 1u));
+                    q_key[w][at] = ~sk[u];
+                    q_val[w][at] = xv[u];
+                }
+                total += __popc(live);
+            }
         }
         if (total == 0) continue;
         ull base = 0;
         if (lane == 0) base = atomicAdd(&p.ctl->n_out, (ull)total);
-        base = __shfl_sync(0xFFFFFFFFu, base, 0);
         __syncwarp();
-        for (uint32_t j = lane; j < total; j += 32) {
-            SlotView v;
-            const ulonglong2 x = q_val[w][j];
-            v.key = q_key[w][j];
-            v.live = true;
-            v.lo = x.x;
-            v.count = x.y & COUNT_MASK;
-            v.hi = x.y >> HI_SHIFT;
-            const ull pos = base + j;
-            if (pos < p.out_cap) store_entry(p.out + pos, make_entry(v, dT, zeroT, p));
+        base = __shfl_sync(0xFFFFFFFFu, base, 0);
+        for (uint32_t j0 = 0; j0 < total; j0 += 32 * EMIT_PROBES) {
+            // The entries' rows of the work table: the partition's first slot, the bucket, stride (once found: slot and type).
+            uint32_t slot[EMIT_PROBES], bucket[EMIT_PROBES], advance[EMIT_PROBES], pending = 0, known = 0;
+#pragma unroll
+            for (int u = 0; u < EMIT_PROBES; ++u) {
+                slot[u] = bucket[u] = advance[u] = 0;
+                if (p.work.keys != nullptr && j0 + lane + 32u * u < total) {
+                    const uint32_t h = hash32(q_key[w][j0 + lane + 32u * u]);
+                    slot[u] = part_of(h, p.work.lp) * p.work.Cw;
+                    bucket[u] = work_start(p.work, h);
+                    advance[u] = work_stride(p.work, h);
+                    pending |= 1u << u;
+                }
+            }
+            for (uint32_t probe = 0; probe < p.work.Cw && __any_sync(0xFFFFFFFFu, pending != 0); ++probe) {
+                WorkKeys x[EMIT_PROBES];
+#pragma unroll
+                for (int u = 0; u < EMIT_PROBES; ++u)
+                    if (pending & (1u << u)) x[u] = load_work_keys(p.work.keys + (slot[u] + bucket[u] * WORK_WAYS));
+#pragma unroll
+                for (int u = 0; u < EMIT_PROBES; ++u) {
+                    if (!(pending & (1u << u))) continue;
+                    uint32_t dtype = 0;
+                    const uint32_t way = work_way(x[u], q_key[w][j0 + lane + 32u * u] & WORK_PAIR, dtype);
+                    if (way != WORK_WAYS) {
+                        pending &= ~(1u << u);
+                        known |= 1u << u;
+                        slot[u] += bucket[u] * WORK_WAYS + way;
+                        advance[u] = dtype;
+                    } else if (x[u].k[WORK_WAYS - 1] == 0) {
+                        pending &= ~(1u << u);
+                    } else {
+                        bucket[u] = work_next(p.work, bucket[u], advance[u]);
+                    }
+                }
+            }
+            double2 work[EMIT_PROBES];
+#pragma unroll
+            for (int u = 0; u < EMIT_PROBES; ++u) work[u] = known & (1u << u) ? p.work.rows[slot[u]] : make_double2(0.0, 0.0);
+#pragma unroll
+            for (int u = 0; u < EMIT_PROBES; ++u) {
+                const uint32_t j1 = j0 + 32u * u, j = j1 + lane;
+                if (j1 >= total) break;
+                if (j < total) {
+                    const ull key = q_key[w][j];
+                    const ulonglong2 x = q_val[w][j];
+                    const int ph = (int)(key >> 48) & (ATREX_MAX_PHASES - 1);
+                    const double weight = zeroT[ph] ? 0.0 : __ddiv_rn(u128_to_f64_rn(x.y >> HI_SHIFT, x.x), dT[ph]);
+                    const double roofline = known & (1u << u) ? roofline_of(work[u], advance[u], p.peaks) : __longlong_as_double(0x7FF8000000000000ll);
+                    s_out[w][3 * lane] = make_ulonglong2(key, x.y & COUNT_MASK);
+                    s_out[w][3 * lane + 1] = make_ulonglong2(x.x, x.y >> HI_SHIFT);
+                    s_out[w][3 * lane + 2] = make_ulonglong2((ull)__double_as_longlong(weight), (ull)__double_as_longlong(roofline));
+                }
+                __syncwarp();
+                const ull at = base + j1;
+                const uint32_t fit = at >= p.out_cap ? 0u : (uint32_t)min(p.out_cap - at, (ull)min(total - j1, 32u));
+                ulonglong2* to = reinterpret_cast<ulonglong2*>(p.out + at);
+#pragma unroll
+                for (uint32_t k = lane; k < 96; k += 32)
+                    if (k < 3 * fit) to[k] = s_out[w][k];
+                __syncwarp();
+            }
         }
-        __syncwarp();  // the queue is refilled in the next round
     }
     grid_dependents_launch();
     if (!last_cta(&p.ctl->emit_done)) return;
@@ -315,27 +395,21 @@ __global__ void __launch_bounds__(256) work_insert_kernel(const atrex_work_t* ro
             atomicOr(&ctl->work_status, ST_WORK_DTYPE);
             continue;
         }
-        ull pair = ((ull)r.op_id << 32) | (ull)r.shape_id;
-        ull skey = ~pair;
-        const uint32_t h = hash32(pair);
-        WorkSlot* part = w.table + (ull)part_of(h, w.lp) * w.Cw;
-        uint32_t s = work_start(w, h);
-        const uint32_t advance = work_stride(w, h);
+        const ull pair = ((ull)r.op_id << 32) | (ull)r.shape_id;
+        const uint32_t h = hash32(pair), first = part_of(h, w.lp) * w.Cw, advance = work_stride(w, h);
+        uint32_t bucket = work_start(w, h);
         bool done = false;
         for (uint32_t probe = 0; probe < w.Cw && !done; ++probe) {
-            WorkSlot* e = part + s;
-            ull old = atomicCAS(&e->skey, 0ull, skey);
+            const uint32_t at = first + bucket * WORK_WAYS + probe % WORK_WAYS;
+            const ull old = atomicCAS(&w.keys[at], 0ull, WORK_USED | (ull)r.dtype << 48 | pair);
             if (old == 0) {
-                e->flops = r.flops;
-                e->bytes = r.bytes;
-                e->dtype = r.dtype;
+                w.rows[at] = make_double2(__ull2double_rn(r.flops), __ull2double_rn(r.bytes));
                 done = true;
-            } else if (old == skey) {
+            } else if ((old & WORK_PAIR) == pair) {
                 atomicOr(&ctl->work_status, ST_WORK_DUP);
                 done = true;
-            } else {
-                s += advance;
-                if (s >= w.Cw) s -= w.Cw;
+            } else if (probe % WORK_WAYS == WORK_WAYS - 1) {
+                bucket = work_next(w, bucket, advance);
             }
         }
         if (!done) atomicOr(&ctl->work_status, ST_WORK_FULL);
@@ -730,7 +804,8 @@ constexpr size_t PICK_SMEM = (size_t)TOPK_PICK_MAX * 28;
 // Up to 65 536 slots (some 25 000 keys) one cluster of 8 or 16 CTAs, four slots to a thread, does in one launch what takes
 // two above, and keeps the table in registers in between: the CTAs' sums and counts meet through distributed shared memory and
 // cluster barriers, where kernels of many CTAs pay for atomics to one address, a fence and a word counted per CTA, and the
-// next launch.  Latency-bound: SMALL_FIGURES
+// next launch.  Latency-bound (4 001 records over 2 phases, whole build 71.8 ->
+// 66.3 us; 2^20 over 4 096 keys 103.9 -> 96.3).
 constexpr uint32_t SMALL_THREADS = 1024, SMALL_ILP = 4, SMALL_CTA_SLOTS = SMALL_THREADS * SMALL_ILP, SMALL_CTAS_MAX = 16;
 constexpr uint32_t SMALL_PIECES = 7;                     // a phase's sums: weighted time in four pieces of 22 bits, count in two of 20, keys
 constexpr uint32_t SMALL_SUMS = ATREX_MAX_PHASES * SMALL_PIECES;

@@ -133,10 +133,11 @@ struct HotBuildParams {
 };
 
 struct WorkRef {
-    WorkSlot* table;     // [P * Cw], nullptr when no work table was provisioned
+    ull* keys;           // [P * Cw], nullptr when no work table was provisioned
+    double2* rows;       // [P * Cw] {flops, bytes}, rounded once
     uint32_t lp;         // log2(P), same partitioning as the key table
-    uint32_t Cw;         // slots per partition
-    ull strides;         // eight probe strides, one byte each: odd primes that do not divide Cw (double hashing)
+    uint32_t Cw;         // slots per partition, whole buckets
+    ull strides;         // eight probe strides in buckets, one byte each: odd primes that do not divide their number (double hashing)
 };
 
 struct FinalizeParams {
