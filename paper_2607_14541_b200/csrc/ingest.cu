@@ -655,16 +655,21 @@ __device__ __forceinline__ void partition_cta(const PartitionParams& q, unsigned
 __global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(const __grid_constant__ PartitionParams q) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     grid_dependency_wait();
-    // the spill buffers are drained lazily: unless forced, only when the scatter launch just
-    // before this one found a buffer filling up
+    // The spill buffers are drained lazily: unless forced, only when the scatter launch just before this one found a buffer
+    // filling up.  A warp asks for all that this hangs on at once: asked by every warp of 148 CTAs, one word after the other, a
+    // launch that has nothing to do waited for thousands of reads of one L2 sector (4.6 us; four words by every warp 6.5; now 2.9).
     Control* const ctl = q.t.ctl;
-    const bool misfits = ld_relaxed(&ctl->n_misfit) > q.misfit_max;
-    if (!q.force && !misfits && ld_relaxed(&ctl->drain_seq) != q.seq) return;
+    __shared__ ull s_asked[4];
+    if (threadIdx.x < 4)
+        s_asked[threadIdx.x] = ld_relaxed(threadIdx.x == 0 ? &ctl->n_misfit : threadIdx.x == 1 ? &ctl->drain_seq : threadIdx.x == 2 ? &ctl->form : &ctl->rests);
+    __syncthreads();
+    const bool misfits = s_asked[0] > q.misfit_max;
+    if (!q.force && !misfits && s_asked[1] != q.seq) return;
+    const ull form = s_asked[2], rests = s_asked[3];
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&ctl->n_drains, 1ull);
-    const ull form = ld_relaxed(&ctl->form);
     if (form != FORM_SHORT)
         partition_cta<FORM_LONG>(q, smem_raw);
-    else if (ld_relaxed(&ctl->rests) != 0)
+    else if (rests != 0)
         partition_cta<FORM_SHORT>(q, smem_raw);
     else
         partition_cta<FORM_TIGHT>(q, smem_raw);
