@@ -533,6 +533,7 @@ static int ingest_launch(atrex_agg* h, const atrex_record_t* recs, uint64_t n, c
         b.n_phases = h->cfg.n_phases;
         b.hot_keys = h->hot_keys;
         b.max_ops = h->L.fmt.max_ops;
+        b.dur_mask = h->L.fmt.dur_mask();
         b.hot_slots = h->L.hot_slots;
         b.hot_words = (uint32_t*)(h->ws + h->L.off_hot_words);
         b.phase_bits = h->L.fmt.phase_bits;

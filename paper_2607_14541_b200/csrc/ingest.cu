@@ -753,7 +753,7 @@ __global__ void __launch_bounds__(256) hot_count_kernel(HotBuildParams p) {
     grid_dependency_wait();
     const uint32_t stride = gridDim.x * blockDim.x;
     const uint32_t rounds = (p.n_sample + stride * SAMPLE_ILP - 1) / (stride * SAMPLE_ILP);  // uniform trip count: warp collectives inside
-    uint32_t max_op = 0;
+    uint32_t max_op = 0, n_long = 0;
     for (uint32_t r = 0; r < rounds; ++r) {
         uint4 v[SAMPLE_ILP];
 #pragma unroll
@@ -768,11 +768,14 @@ __global__ void __launch_bounds__(256) hot_count_kernel(HotBuildParams p) {
             const bool ok = j < p.n_sample && v[u].x < p.n_apps && (khi >> 16) < p.n_phases;
             if (j < p.n_sample) p.sample[j] = ok ? ((ull)khi << 32) | v[u].z : ~0ull;
             if (ok) max_op = max(max_op, khi & 0xFFFFu);
+            if (ok && v[u].w > p.dur_mask) ++n_long;
             cache.add(p.sketch, hash32(khi & 0xFFFFu, v[u].z) >> (32 - SKETCH_BITS), ok);
         }
     }
     max_op = __reduce_max_sync(0xFFFFFFFFu, max_op);
     if ((threadIdx.x & 31u) == 0 && max_op >= p.max_ops) atomicMax(&p.scratch->max_op, max_op);   // (only what does not fit is told)
+    n_long = __reduce_add_sync(0xFFFFFFFFu, n_long);
+    if ((threadIdx.x & 31u) == 0 && n_long > rounds * SAMPLE_ILP * 8u) atomicAdd(&p.scratch->n_long, n_long);   // (a quarter of the warp's or more)
     grid_dependents_launch();
     cache.flush(p.sketch);
 }
@@ -864,7 +867,11 @@ __global__ void __launch_bounds__(LEVEL_THREADS) hot_level_kernel(HotBuildParams
     // less evenly than one of four): thread t looks at the count 1023 - t, behind a scan over the higher ones
     const ull most_seen = __ldcg(&x.most);
     const ull skew = most_seen * 8u >= p.n_sample * 3ull ? SKEW_DOMINATED : (most_seen * 32u >= p.n_sample ? SKEW_COMBINE : SKEW_NONE);
-    const bool words = p.max_ops != 0 && __ldcg(&x.max_op) == 0;
+    // (Two short entries are longer than a long one.  Where one key dominates, few records look into the directory and the words
+    // form's look-ups do not make up for them from three quarters of such durations on: 2^28 records, 10 % spilled, all of
+    // them so long, whole build 1 591 -> 1 400 us, the drain 510 -> 328 of it.)
+    const bool mostly_long = __ldcg(&x.n_long) >= p.n_sample / 4 * 3;
+    const bool words = p.max_ops != 0 && __ldcg(&x.max_op) == 0 && !(skew == SKEW_DOMINATED && mostly_long);
     const uint32_t slots = p.slots[words][skew == SKEW_DOMINATED];
     const uint32_t budget = min(words ? 2 * slots : slots + slots / 4, HOT_SELECT_MAX);
     const uint32_t mine = __ldcg(&x.hist[1023 - t]);

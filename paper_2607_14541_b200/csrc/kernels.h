@@ -102,7 +102,7 @@ static_assert(scatter_slots(8, true) / WORD_WAYS <= HOT_BUCKETS_MAX && scatter_s
               scatter_slots(8, true) * 2 <= HOT_SELECT_MAX, "directory build scratch");
 struct HotBuildScratch {
     uint32_t n, most, threshold, done;
-    uint32_t weight, max_op, pad[2];             // sampled weight in the directory, largest operator sampled
+    uint32_t weight, max_op, n_long, pad;        // sampled weight in the directory, largest operator, durations of two short entries
     uint32_t lost[4];                            // sampled weight each multiplier would lose
     uint32_t hist[1024];                         // candidates by count
     uint32_t occupancy[4][HOT_BUCKETS_MAX];
@@ -117,7 +117,7 @@ struct HotBuildParams {
     ull stride;                // records per sampled one (below 2^32)
     uint32_t n_sample;         // n_sample * stride <= records of the call
     uint32_t n_apps, n_phases;
-    uint32_t max_ops;          // as in ShortFormat (0: no short entries)
+    uint32_t max_ops, dur_mask;   // as in ShortFormat (max_ops 0: no short entries)
     ull* hot_keys;
     uint32_t hot_slots;        // of the image
     uint32_t* hot_words;       // [hot_slots] (words form)

@@ -97,3 +97,27 @@ def test_operators_that_no_longer_fit():
     agg.reset()                                                   # short entries again
     ingest(agg, recs[:part])
     assert agg.stats()["spill_cap"] == cap // 2 * 3
+
+
+@pytest.mark.parametrize("hot", [0.0, 0.9])
+@pytest.mark.parametrize("long_share", [0.7, 0.8, 1.0])
+def test_durations_that_mostly_take_two_entries(long_share, hot):
+    """Around the share of long durations from which the entries beside a dominant key are long ones (64 applications:
+    26 bits or fewer fit a short entry)."""
+    import paper_2607_14541_b200 as p
+    rng = np.random.default_rng(int(long_share * 10 + hot * 100))
+    n = 1_000_003
+    recs = np.zeros(n, dtype=RECORD_DTYPE)
+    recs["app_id"], recs["op_id"] = rng.integers(0, 64, n), rng.integers(0, 64, n)
+    recs["phase"], recs["shape_id"] = rng.integers(0, 2, n), rng.integers(0, 8_192, n)
+    cold = rng.random(n) >= hot
+    for field in ("op_id", "phase", "shape_id"):
+        recs[field] *= cold
+    recs["duration_ns"] = np.where(rng.random(n) < long_share, (1 << 28) - 1, 50_000)
+    weights = np.full(64, (1 << 20) - 1, dtype=np.uint32)
+    agg = p.Aggregator(weights, 2, 2_000_000)
+    o = oracle.Oracle(weights, 2)
+    for _ in range(2):
+        ingest(agg, recs)
+        o.ingest(recs, threads=4)
+    check(agg, o)
