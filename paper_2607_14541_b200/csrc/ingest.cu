@@ -342,6 +342,10 @@ __device__ __forceinline__ void stream_batch(const PartitionParams& q, const Par
                          : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
                          : "l"(src + (size_t)e * SHORT_ENTRY_BYTES));
             open = FULL ? 0xFu : (0xFu >> (4u - min(n_e - e, 4u)));
+            // (what lies behind the last entry may be anything: no application is to be read from it)
+#pragma unroll
+            for (int u = 1; u < 4; ++u)
+                if (!FULL && (open & (1u << u)) == 0) w[2 * u] = 0;
         } else {
 #pragma unroll
             for (int j = 0; j < 8; ++j) w[j] = 0;

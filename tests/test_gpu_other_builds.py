@@ -30,6 +30,18 @@ def test_parity_cases_under_the_bounds_checked_build():
     assert " passed" in run.stdout
 
 
+def test_short_entries_under_the_bounds_checked_build():
+    import importlib.util
+    spec = importlib.util.spec_from_file_location("atrex_build", os.path.join(ROOT, "paper_2607_14541_b200", "build.py"))
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    env = dict(os.environ, ATREX_AGG_LIBRARY=mod.build_checked())
+    run = subprocess.run([sys.executable, "-m", "pytest", "tests/test_gpu_short_entries.py", "-x", "-q"],
+                         cwd=ROOT, env=env, capture_output=True, text=True, timeout=1200)
+    assert run.returncode == 0, run.stdout[-3000:] + run.stderr[-2000:]
+    assert " passed" in run.stdout
+
+
 @pytest.mark.parametrize("variant", ["ring4"])
 def test_parity_cases_under_the_scatter_variants(variant):
     """The scatter pass's build-time variant -- the shared-memory record ring filled by bulk asynchronous

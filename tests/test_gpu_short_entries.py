@@ -121,3 +121,33 @@ def test_durations_that_mostly_take_two_entries(long_share, hot):
         ingest(agg, recs)
         o.ingest(recs, threads=4)
     check(agg, o)
+
+
+@pytest.mark.parametrize("n_apps,n_ops,max_keys", [(3, 9, 60_000), (300, 64, 60_000), (1_025, 256, 300_000), (2_500, 200, 4_000_000)])
+def test_what_lies_behind_the_last_entry_is_not_looked_at(n_apps, n_ops, max_keys, monkeypatch):
+    """Ragged buffers in a workspace of all ones, and in one that held the long entries of an earlier trace: where the number of
+    applications is no power of two, an application field read from there names none (the bounds-checked build
+    would say so)."""
+    import torch
+    import paper_2607_14541_b200 as p
+    rng = np.random.default_rng(n_apps)
+    weights = rng.integers(0, 1 << 20, n_apps).astype(np.uint32)
+    empty = torch.empty
+    with monkeypatch.context() as m:
+        m.setattr(torch, "empty", lambda *args, **kw: empty(*args, **kw).fill_(0xFF))
+        agg = p.Aggregator(weights, 2, max_keys)
+    # (fewer records of a small table go straight into it)
+    least = (1 << 22) + 1 if max_keys < 1_000_000 else 270_000
+    for wide in (0, 1, 0):                                         # operators of any size: long entries
+        n = least + 2 * int(rng.integers(0, 5_000))
+        recs = np.zeros(n, dtype=RECORD_DTYPE)
+        recs["app_id"], recs["phase"] = rng.integers(0, n_apps, n), rng.integers(0, 2, n)
+        recs["op_id"], recs["shape_id"] = rng.integers(0, n_ops, n) + 60_000 * wide, rng.integers(0, max_keys // (3 * n_ops), n)
+        recs["duration_ns"] = rng.integers(0, 1 << 32, n, dtype=np.uint64).astype(np.uint32)
+        o = oracle.Oracle(weights, 2)
+        o.ingest(recs, threads=8)
+        agg.reset()
+        ingest(agg, recs)
+        check(agg, o)
+        st = agg.stats()
+        assert 0 < st["n_spilled"] and st["n_valid"] == n
