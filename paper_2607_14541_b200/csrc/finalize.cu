@@ -904,8 +904,15 @@ __device__ __forceinline__ uint32_t cluster_rank() {
     asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// (the aligned forms are for whole warps: lanes that took different ways come together first)
+__device__ __forceinline__ void cluster_arrive() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 __device__ __forceinline__ uint32_t remote_addr(const void* p, uint32_t rank) {   // of the same variable in another CTA of the cluster
     uint32_t a;
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
@@ -1025,7 +1032,6 @@ __global__ void __launch_bounds__(SMALL_THREADS) finalize_small_kernel(const __g
         const uint32_t j = u * SMALL_THREADS + t;
         roofline[u] = j < n_live ? roofline_time(p.work, p.peaks, q_key[j]) : 0.0;
     }
-    __syncwarp();
     cluster_wait();
     for (uint32_t i = w; i <= SMALL_SUMS; i += SMALL_THREADS / 32) {
         if (i < SMALL_SUMS) {
