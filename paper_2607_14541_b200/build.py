@@ -59,8 +59,9 @@ def build_checked(force: bool = False) -> str:
     return DEBUG_LIB
 
 
-# the scatter pass's build-time variant that the test-suite runs the parity cases under
-VARIANTS = {"ring4": ["-DATREX_SCATTER_RING=4"]}
+# the build-time variant that the test-suite runs the parity cases under: the scatter pass's record ring, and no clusters
+# (small tables by the kernels of the large ones, as where a cluster does not fit)
+VARIANTS = {"ring4": ["-DATREX_SCATTER_RING=4", "-DATREX_SMALL_CLUSTERS=0"]}
 
 
 def variant_path(name: str) -> str:

@@ -224,6 +224,7 @@ struct atrex_agg {
     ull fin_gen = 0;                  // bumped by every successful finalize
     bool hot_ready = false;
     bool finalized = false;
+    bool one_cluster = false;     // finalize and top-k of this (small) table: a launch of one cluster each
     bool spill_pending = false;   // entries may sit in the spill buffers
     ull scatter_seq = 0;          // sequence number of the last scatter launch
     atrex_hw_peaks_t peaks;
@@ -393,6 +394,7 @@ int atrex_agg_create(const atrex_agg_config_t* cfg, atrex_agg_t** out) {
         }
         if (e == cudaSuccess) e = ingest_prepare();
         if (e == cudaSuccess) e = finalize_prepare();
+        if (e == cudaSuccess) h->one_cluster = finalize_in_one_cluster(L.n_slots);
         if (e == cudaSuccess) e = cudaDeviceSynchronize();
         if (e != cudaSuccess) { h->last_cuda_error = (int)e; rc = ATREX_ERR_CUDA; break; }
     } while (0);
@@ -730,7 +732,7 @@ static int finalize_impl(atrex_agg_t* h, const atrex_hw_peaks_t* peaks, const ui
     const GivenTotals given = given_totals(total_lo, total_hi);
     FinalizeParams fin = finalize_params(h, d_out, out_cap);
     // (the last kernel tells the control block)
-    if (finalize_is_small(h->L.n_slots)) {
+    if (h->one_cluster) {
         fin.stamp = (uint32_t)++h->wait_seq;
         h->hist_at ^= 1u;
         CU(h, launch_finalize_small(fin, h->cfg.n_phases, given, hist_half(h, h->hist_at), hist_half(h, h->hist_at ^ 1u), s));
@@ -871,8 +873,8 @@ int atrex_agg_topk(atrex_agg_t* h, uint32_t phase, uint32_t k, atrex_entry_t* h_
             const uint32_t n_phases = p.n_phases;
             const uint32_t stamp = p.fin.stamp;
             for (uint32_t q = 0; q < n_phases; ++q) answers[q] = (ull)~stamp << 32;
-            CU(h, launch_topk_pick(p, h->n_sms, s));
-            h->launches += finalize_is_small(h->L.n_slots) ? 1 : 2;
+            CU(h, launch_topk_pick(p, h->one_cluster, h->n_sms, s));
+            h->launches += h->one_cluster ? 1 : 2;
             const volatile ull* a = answers;
             const ulonglong2* const rows = k <= TOPK_TOLD_K ? h->h_top_told : nullptr;
             const auto answered = [=] {

@@ -1180,23 +1180,39 @@ __global__ void __launch_bounds__(SMALL_THREADS) topk_small_kernel(const __grid_
 
 uint32_t small_ctas(ull n_slots) { return n_slots <= 8 * SMALL_CTA_SLOTS ? 8u : 16u; }
 
-// One cluster, set up while its predecessor on the stream is still running (see launch_chained).
+// A launch of one cluster, set up while its predecessor on the stream is still running (see launch_chained).
+struct ClusterLaunch {
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t config = {};
+    ClusterLaunch(uint32_t ctas, size_t smem, cudaStream_t stream) {
+        config.gridDim = dim3(ctas);
+        config.blockDim = dim3(SMALL_THREADS);
+        config.dynamicSmemBytes = smem;
+        config.stream = stream;
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = ctas;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[1].val.programmaticStreamSerializationAllowed = 1;
+        config.attrs = attr;
+        config.numAttrs = 2;
+    }
+    ClusterLaunch(const ClusterLaunch&) = delete;
+    ClusterLaunch& operator=(const ClusterLaunch&) = delete;
+};
+
 template <typename... P, typename... A>
 cudaError_t launch_cluster(void (*kernel)(P...), uint32_t ctas, size_t smem, cudaStream_t stream, const A&... args) {
-    cudaLaunchConfig_t c = {};
-    c.gridDim = dim3(ctas);
-    c.blockDim = dim3(SMALL_THREADS);
-    c.dynamicSmemBytes = smem;
-    c.stream = stream;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = ctas;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    c.attrs = attr;
-    c.numAttrs = 2;
-    return cudaLaunchKernelEx(&c, kernel, P(args)...);
+    ClusterLaunch launch(ctas, smem, stream);
+    return cudaLaunchKernelEx(&launch.config, kernel, P(args)...);
+}
+template <typename... P>
+bool cluster_fits(void (*kernel)(P...), uint32_t ctas, size_t smem) {
+    ClusterLaunch launch(ctas, smem, nullptr);
+    int n = 0;
+    const bool fits = cudaOccupancyMaxActiveClusters(&n, kernel, &launch.config) == cudaSuccess && n > 0;
+    if (!fits) cudaGetLastError();
+    return fits;
 }
 
 cudaError_t finalize_prepare() {
@@ -1233,14 +1249,22 @@ cudaError_t launch_work_insert(const atrex_work_t* rows, ull n, const WorkRef& w
     return cudaGetLastError();
 }
 
-bool finalize_is_small(ull n_slots) { return n_slots <= (ull)SMALL_CTAS_MAX * SMALL_CTA_SLOTS; }
+#ifndef ATREX_SMALL_CLUSTERS
+#define ATREX_SMALL_CLUSTERS 1
+#endif
+// Small tables go through one cluster where the process has the SMs for it in one place; a share of the GPU (some of its
+// SMs only) may not, and 16 CTAs are more than every GPU promises.
+bool finalize_in_one_cluster(ull n_slots) {
+    if (!ATREX_SMALL_CLUSTERS || n_slots > (ull)SMALL_CTAS_MAX * SMALL_CTA_SLOTS) return false;
+    return cluster_fits(finalize_small_kernel, small_ctas(n_slots), FINALIZE_SMALL_SMEM) && cluster_fits(topk_small_kernel, small_ctas(n_slots), sizeof(SmallPick));
+}
 
 cudaError_t launch_finalize_small(const FinalizeParams& p, uint32_t n_phases, const GivenTotals& given, uint32_t* hist, uint32_t* next_hist, cudaStream_t stream) {
     return launch_cluster(finalize_small_kernel, small_ctas(p.n_slots), FINALIZE_SMALL_SMEM, stream, p, n_phases, given, hist, next_hist);
 }
 
-cudaError_t launch_topk_pick(const PickParams& p, int n_sms, cudaStream_t stream) {
-    if (finalize_is_small(p.fin.n_slots)) return launch_cluster(topk_small_kernel, small_ctas(p.fin.n_slots), sizeof(SmallPick), stream, p);
+cudaError_t launch_topk_pick(const PickParams& p, bool one_cluster, int n_sms, cudaStream_t stream) {
+    if (one_cluster) return launch_cluster(topk_small_kernel, small_ctas(p.fin.n_slots), sizeof(SmallPick), stream, p);
     static const uint32_t per_sm = resident_ctas(topk_collect_kernel, FIN_THREADS, 0);
     cudaError_t e = launch_chained(topk_collect_kernel, grid_for_work(p.fin.n_slots, FIN_THREADS * 4, n_sms, per_sm), FIN_THREADS, 0, stream, p);
     if (e == cudaSuccess) e = launch_chained(topk_rank_kernel, p.n_phases, RANK_THREADS, PICK_SMEM, stream, p);

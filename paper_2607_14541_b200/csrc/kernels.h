@@ -254,12 +254,12 @@ cudaError_t finalize_prepare();
 cudaError_t launch_totals(const TableRef& t, ull n_slots, uint32_t n_phases, const GivenTotals& given, uint32_t* hist, uint32_t* next_hist, int n_sms,
                           cudaStream_t stream);
 cudaError_t launch_emit(const FinalizeParams& p, int n_sms, cudaStream_t stream);
-bool finalize_is_small(ull n_slots);       // totals and entries in one launch
+bool finalize_in_one_cluster(ull n_slots);       // totals and entries in one launch, the best k in another (asked after finalize_prepare)
 cudaError_t launch_finalize_small(const FinalizeParams& p, uint32_t n_phases, const GivenTotals& given, uint32_t* hist, uint32_t* next_hist,
                                   cudaStream_t stream);
 cudaError_t launch_work_insert(const atrex_work_t* rows, ull n, const WorkRef& w, Control* ctl, int grid,
                                cudaStream_t stream);
-cudaError_t launch_topk_pick(const PickParams& p, int n_sms, cudaStream_t stream);
+cudaError_t launch_topk_pick(const PickParams& p, bool one_cluster, int n_sms, cudaStream_t stream);
 cudaError_t launch_topk_collect_all(const TopkAllParams& p, int grid, cudaStream_t stream);
 cudaError_t launch_topk_hist(const TopkAllParams& p, int n_sms, cudaStream_t stream);
 cudaError_t launch_topk_digit(const TopkDigitParams& p, uint32_t n_phases, cudaStream_t stream);

@@ -60,6 +60,23 @@ def test_parity_cases_under_the_scatter_variants(variant):
     assert " passed" in run.stdout
 
 
+def test_small_tables_where_no_cluster_fits():
+    """Entries and rankings of small tables by the kernels that large ones take (the variant has no clusters)."""
+    import importlib.util
+    spec = importlib.util.spec_from_file_location("atrex_build", os.path.join(ROOT, "paper_2607_14541_b200", "build.py"))
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    env = dict(os.environ, ATREX_AGG_LIBRARY=mod.build_variant_if_stale("ring4", mod.VARIANTS["ring4"]))
+    count = ("import numpy as np, paper_2607_14541_b200 as p; a = p.Aggregator(np.ones(1, dtype=np.uint32), 1, 4096); b = a.launch_count(); "
+             "a.finalize(1e12, [1e12] * 8); print(a.launch_count() - b)")
+    probe = subprocess.run([sys.executable, "-c", count], cwd=ROOT, env=env, capture_output=True, text=True, timeout=300)
+    assert probe.returncode == 0 and probe.stdout.strip() == "4", probe.stderr[-2000:]        # (two calls; a cluster takes one launch each)
+    run = subprocess.run([sys.executable, "-m", "pytest", "tests/test_gpu_topk_ranks.py", "tests/test_gpu_emit.py", "-x", "-q"],
+                         cwd=ROOT, env=env, capture_output=True, text=True, timeout=1200)
+    assert run.returncode == 0, run.stdout[-3000:] + run.stderr[-2000:]
+    assert " passed" in run.stdout
+
+
 def test_the_regular_build_has_no_checks():
     import paper_2607_14541_b200 as p
     assert p.atrex_build_has_bounds_checks() == 0 or os.environ.get("ATREX_AGG_LIBRARY")
