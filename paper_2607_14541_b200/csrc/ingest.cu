@@ -779,7 +779,7 @@ __global__ void __launch_bounds__(256) hot_count_kernel(HotBuildParams p) {
     max_op = __reduce_max_sync(0xFFFFFFFFu, max_op);
     if ((threadIdx.x & 31u) == 0 && max_op >= p.max_ops) atomicMax(&p.scratch->max_op, max_op);   // (only what does not fit is told)
     n_long = __reduce_add_sync(0xFFFFFFFFu, n_long);
-    if ((threadIdx.x & 31u) == 0 && n_long > rounds * SAMPLE_ILP * 8u) atomicAdd(&p.scratch->n_long, n_long);   // (a quarter of the warp's or more)
+    if ((threadIdx.x & 31u) == 0 && n_long > rounds * SAMPLE_ILP * 4u) atomicAdd(&p.scratch->n_long, n_long);   // (an eighth of the warp's or more)
     grid_dependents_launch();
     cache.flush(p.sketch);
 }
@@ -831,6 +831,21 @@ __global__ void __launch_bounds__(256) hot_admit_kernel(HotBuildParams p) {
 // 4 096: 811 against 860) or more (12 288: 1 056 against 1 082, 32 768: 1 357 against 1 808).  Between, tags hold more
 // (6 144: 909 against 940, 6 880: 933 against 966), and from TAGS_PART on where such keys hold only a part of the trace.
 constexpr uint32_t TAGS_PART = 3500, TAGS_FROM = 5500, TAGS_TO = 7500, EVEN = 4;
+// A duration that takes two short entries makes 16 bytes of a record, a long entry has 12.  Whole builds of 2^27 records, long
+// entries and then short ones at a share of such durations of 0, 0.2, 0.5 and 1:
+//   4 M keys Zipf(0.8), 75 % spilled     1 970   1 793 1 982 2 298 2 741 us       (short ones are faster until 0.18)
+//   8 M keys Zipf(1.1), 50 %             2 045   1 848 1 956 2 215 2 554          (0.30)
+//   35 % on one key, the rest over 2 M   1 885   1 719 1 850 2 122 2 701          (0.25)
+//   90 % on one key                        728     729   752   781   760          (0.05)
+//   12 288 equally frequent keys         1 065   1 022 1 096 1 225 1 178          (0.15)
+//   4 096 equally frequent keys            855     786   809   842   891          (0.75)
+//   32 768 equally frequent keys         1 690   1 292 1 390 1 564 1 948          (0.65)
+//   0.5 M equally frequent keys          2 390   1 786 2 014 2 384 3 114          (0.50)
+//   0.5 M keys Zipf(1.2), 27 %           1 095     947 1 011 1 100 1 219          (0.46)
+// So entries are long from a quarter on, and from 7/16 on where the keys that the directory may hold have five eighths of the
+// sample and where keys are equally frequent.  A trace of 2^20 records takes as long either way (192 us and
+// 196, 285 and 296; of 2^24: 437 and 536), and how it goes on cannot be told from it.
+constexpr ull FORM_MATTERS = 1u << 20;
 constexpr uint32_t LIST_MAX = 16;       // candidates a bucket chooses from (five on average)
 constexpr uint32_t LEVEL_THREADS = 1024;
 
@@ -871,13 +886,7 @@ __global__ void __launch_bounds__(LEVEL_THREADS) hot_level_kernel(HotBuildParams
     // less evenly than one of four): thread t looks at the count 1023 - t, behind a scan over the higher ones
     const ull most_seen = __ldcg(&x.most);
     const ull skew = most_seen * 8u >= p.n_sample * 3ull ? SKEW_DOMINATED : (most_seen * 32u >= p.n_sample ? SKEW_COMBINE : SKEW_NONE);
-    // (Two short entries are longer than a long one.  Where one key dominates, few records look into the directory and the words
-    // form's look-ups do not make up for them from three quarters of such durations on: 2^28 records, 10 % spilled, all of
-    // them so long, whole build 1 591 -> 1 400 us, the drain 510 -> 328 of it.)
-    const bool mostly_long = __ldcg(&x.n_long) >= p.n_sample / 4 * 3;
-    const bool words = p.max_ops != 0 && __ldcg(&x.max_op) == 0 && !(skew == SKEW_DOMINATED && mostly_long);
-    const uint32_t slots = p.slots[words][skew == SKEW_DOMINATED];
-    const uint32_t budget = min(words ? 2 * slots : slots + slots / 4, HOT_SELECT_MAX);
+    const bool fits = p.max_ops != 0 && __ldcg(&x.max_op) == 0;     // short entries and words can hold what was sampled
     const uint32_t mine = __ldcg(&x.hist[1023 - t]);
     uint32_t incl = mine;
 #pragma unroll
@@ -898,20 +907,30 @@ __global__ void __launch_bounds__(LEVEL_THREADS) hot_level_kernel(HotBuildParams
     }
     __syncthreads();
     incl += w ? s_warp[w - 1] : 0u;
-    const int above = __syncthreads_count(t <= 1021 && incl <= budget);   // counts 1023, 1022, ... that fit
-    __shared__ uint32_t s_weight;                                          // of the sample, in the selected candidates
-    if (t == 0) s_weight = 0;
+    auto selection = [&](bool words) {                                     // counts 1023, 1022, ... that fit
+        const uint32_t slots = p.slots[words][skew == SKEW_DOMINATED];
+        const uint32_t budget = min(words ? 2 * slots : slots + slots / 4, HOT_SELECT_MAX);
+        return (uint32_t)__syncthreads_count(t <= 1021 && incl <= budget);
+    };
+    uint32_t above = selection(fits);
+    __shared__ uint32_t s_weight, s_selected;                              // of the sample, in the selected candidates; how many they are
+    if (t == 0) s_weight = s_selected = 0;
     __syncthreads();
-    const uint32_t weight = __reduce_add_sync(0xFFFFFFFFu, t < (uint32_t)above ? mine * (1023u - t) : 0u);
+    const uint32_t weight = __reduce_add_sync(0xFFFFFFFFu, t < above ? mine * (1023u - t) : 0u);
     if (lane == 0 && weight) atomicAdd(&s_weight, weight);
+    if (t + 1u == above) s_selected = incl;
     __syncthreads();
-    if (above == 0 ? t == 0 : t == (uint32_t)above - 1u) {
-        const uint32_t selected = above ? incl : 0u;
-        x.threshold = 1024u - (uint32_t)above;
+    const bool even = most_seen * s_selected < (ull)EVEN * s_weight;
+    const bool tags = even && s_selected > (s_weight < p.n_sample / 2 ? TAGS_PART : TAGS_FROM) && s_selected <= TAGS_TO;
+    const bool often_hit = s_weight / 5 >= p.n_sample / 8;
+    const ull long_from = skew != SKEW_DOMINATED && (often_hit || even) ? p.n_sample / 16 * 7 : p.n_sample / 4;
+    const bool often_long = __ldcg(&x.n_long) >= long_from && (skew == SKEW_DOMINATED || p.n_sample * p.stride > FORM_MATTERS);
+    const bool words = fits && !often_long && !tags;
+    if (fits && often_long) above = selection(false);
+    if (t == 0) {
+        x.threshold = 1024u - above;
         p.ctl->hot_skew = skew;
-        const bool even = most_seen * selected < (ull)EVEN * s_weight;
-        const bool tags = even && selected > (s_weight < p.n_sample / 2 ? TAGS_PART : TAGS_FROM) && selected <= TAGS_TO;
-        p.ctl->form = words && !tags ? FORM_SHORT : FORM_LONG;
+        p.ctl->form = words ? FORM_SHORT : FORM_LONG;
     }
 }
 

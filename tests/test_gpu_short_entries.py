@@ -151,3 +151,24 @@ def test_what_lies_behind_the_last_entry_is_not_looked_at(n_apps, n_ops, max_key
         check(agg, o)
         st = agg.stats()
         assert 0 < st["n_spilled"] and st["n_valid"] == n
+
+
+@pytest.mark.parametrize("hot", [0.0, 0.4, 0.9])
+@pytest.mark.parametrize("long_share,is_short", [(0.0, True), (0.1, True), (0.6, False), (1.0, False)])
+def test_entries_are_long_where_many_durations_take_two(long_share, is_short, hot):
+    """The form of the entries, as the capacity of a buffer tells it, whatever the share of the most frequent key."""
+    import paper_2607_14541_b200 as p
+    rng = np.random.default_rng(int(long_share * 10 + hot * 100))
+    n = 1_400_003                                                  # (below 2^20 it does not matter)
+    recs = np.zeros(n, dtype=RECORD_DTYPE)
+    recs["app_id"], recs["op_id"] = rng.integers(0, 64, n), rng.integers(0, 64, n)
+    recs["phase"], recs["shape_id"] = rng.integers(0, 2, n), rng.integers(0, 8_192, n)
+    cold = rng.random(n) >= hot
+    for field in ("op_id", "phase", "shape_id"):
+        recs[field] *= cold
+    recs["duration_ns"] = np.where(rng.random(n) < long_share, (1 << 28) - 1, 50_000)
+    agg = p.Aggregator(np.full(64, 7, dtype=np.uint32), 2, 2_000_000)
+    cap = agg.stats()["spill_cap"]
+    ingest(agg, recs)
+    st = agg.stats()
+    assert st["spill_cap"] == (cap // 2 * 3 if is_short else cap) and st["n_spilled"] > 0
