@@ -493,10 +493,22 @@ __device__ __forceinline__ void scatter_body(const IngestParams& p, Ctx& c) {
 // warp's queue in shared memory and through one_record 32 at a time, so that what is left of a warp's 32
 // records does not cost the price of 32.  Bound by DRAM once the key holds most records (90 %: 140 -> 57 warp
 // instructions per 32 records, 0.66 -> 0.39 ms per 2^27 records); the queue pays from a share of 3/8 on.
+// The lane's number and the mask of the lanes below it are read where they are needed: kept in registers they pushed
+// the loop's own values out to memory, beside five other bodies in one kernel (tags form, 2^29 records of two-entry durations:
+// ingest 1 801 -> 1 690 us; words form, whole build 2 431 -> 2 409; tables of 2^21 to 2^25 keys: 1 to 8 % in the tags form).
+__device__ __forceinline__ uint32_t lane_id() {
+    uint32_t v;
+    asm("mov.u32 %0, %%laneid;" : "=r"(v));
+    return v;
+}
+__device__ __forceinline__ uint32_t lanes_below() {
+    uint32_t v;
+    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(v));
+    return v;
+}
 template <uint32_t LP, int DIR>
 __device__ __forceinline__ void dominated_body(const IngestParams& p, Ctx& c) {
     using L = Smem<LP, DIR>;
-    const uint32_t lane = threadIdx.x & 31u, lt = (1u << lane) - 1u;
     const uint32_t queue = c.sb + L::QUEUE + (threadIdx.x >> 5) * (SCATTER_QUEUE * 16u);
     const ull top = p.t.ctl->top_key;
     const uint32_t top_hi = (uint32_t)(top >> 32), top_lo = (uint32_t)top;
@@ -505,11 +517,11 @@ __device__ __forceinline__ void dominated_body(const IngestParams& p, Ctx& c) {
     auto settle = [&](uint32_t n) {        // the last n records of the queue (n = 32 but for the last time)
         __syncwarp();
         uint4 v = make_uint4(0, 0, 0, 0);
-        if (lane < n)
-            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(queue + (q - n + lane) * 16u) : "memory");
+        if (lane_id() < n)
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(queue + (q - n + lane_id()) * 16u) : "memory");
         __syncwarp();
         q -= n;
-        one_record<LP, DIR, SKEW_DOMINATED, false>(p, c, v.x, v.y, v.z, v.w, lane < n);
+        one_record<LP, DIR, SKEW_DOMINATED, false>(p, c, v.x, v.y, v.z, v.w, lane_id() < n);
     };
     auto take = [&](uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, bool present) {
         const bool match = (((w1 ^ top_hi) & 0x00FFFFFFu) | (w2 ^ top_lo)) == 0u && w0 < p.n_apps && present;
@@ -522,7 +534,7 @@ __device__ __forceinline__ void dominated_body(const IngestParams& p, Ctx& c) {
         }
         const uint32_t others = __ballot_sync(0xFFFFFFFFu, present && !dom);
         if (present && !dom)
-            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(queue + (q + __popc(others & lt)) * 16u), "r"(w0), "r"(w1), "r"(w2), "r"(w3) : "memory");
+            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(queue + (q + __popc(others & lanes_below())) * 16u), "r"(w0), "r"(w1), "r"(w2), "r"(w3) : "memory");
         q += __popc(others);
         if (q >= 32) settle(32);
     };
@@ -558,11 +570,11 @@ __device__ __forceinline__ void dominated_body(const IngestParams& p, Ctx& c) {
         const uint32_t step = gridDim.x * (SCATTER_THREADS * 32u);
         for (; round + 4 <= full_rounds; round += 2) {
             ld_stream_256(next, bufB);
-            if ((lane & 3u) == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(next + step));
+            if ((threadIdx.x & 3u) == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(next + step));
             next += step;
             consume_full(bufA);
             ld_stream_256(next, bufA);
-            if ((lane & 3u) == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(next + step));
+            if ((threadIdx.x & 3u) == 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(next + step));
             next += step;
             consume_full(bufB);
         }
@@ -593,7 +605,7 @@ __device__ __forceinline__ void dominated_body(const IngestParams& p, Ctx& c) {
         sum = s;
         n += __shfl_xor_sync(0xFFFFFFFFu, n, d);
     }
-    if (lane == 0 && n) {
+    if (lane_id() == 0 && n) {
         const ull old = atomicAdd(&s_lo, sum);
         atomicAdd(&s_hi, hi + (old + sum < old ? 1ull : 0ull));
         atomicAdd(&s_count, n);
