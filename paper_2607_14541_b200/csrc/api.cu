@@ -223,6 +223,9 @@ struct atrex_agg {
     TopkCache topk;
     ull fin_gen = 0;                  // bumped by every successful finalize
     bool hot_ready = false;
+    ull* h_long = nullptr;        // pinned: the trace whose entries had to become long, as the partition pass tells it
+    ull trace = 1;                // number of this trace: one more with every reset
+    bool long_only = false;       // ... its entries have, and the directory was built anew for them
     bool finalized = false;
     bool one_cluster = false;     // finalize and top-k of this (small) table: a launch of one cluster each
     bool spill_pending = false;   // entries may sit in the spill buffers
@@ -377,7 +380,7 @@ int atrex_agg_create(const atrex_agg_config_t* cfg, atrex_agg_t** out) {
         // the pinned block: what kernels tell with stamps, every phase's best, how many there are, a digit each, the control block's copy
         const size_t top_bytes = (size_t)cfg->n_phases * (TOPK_PICK_K * sizeof(atrex_entry_t) + 8), digit_bytes = cfg->n_phases * sizeof(TopkDigit);
         const size_t told_bytes = CONTROL_WORDS * 16 + (size_t)cfg->n_phases * TOPK_TOLD_K * 96;
-        h->pinned_bytes = told_bytes + top_bytes + digit_bytes + sizeof(Control);
+        h->pinned_bytes = told_bytes + top_bytes + digit_bytes + sizeof(Control) + 8;
         if (e == cudaSuccess) e = pinned_alloc((void**)&h->h_told, h->pinned_bytes);
         if (e == cudaSuccess) {
             memset(h->h_told, 0, told_bytes);        // (the block may be another handle's former one: no stamp of its may be left)
@@ -386,6 +389,8 @@ int atrex_agg_create(const atrex_agg_config_t* cfg, atrex_agg_t** out) {
             h->h_digit = (TopkDigit*)((unsigned char*)h->h_top + top_bytes);
             h->h_ctl = (Control*)((unsigned char*)h->h_digit + digit_bytes);
             memset(h->h_digit, 0, digit_bytes);
+            h->h_long = (ull*)(h->h_ctl + 1);
+            *h->h_long = 0;
         }
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->copy_stream, cudaStreamNonBlocking);
         for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
@@ -430,6 +435,8 @@ int atrex_agg_reset(atrex_agg_t* h, void* stream) {
     h->img_rows = 0;
     h->spill_pending = false;
     h->hot_ready = false;
+    h->long_only = false;
+    ++h->trace;
     h->finalized = false;
     h->n_records = 0;
     return ATREX_OK;
@@ -462,17 +469,25 @@ int atrex_agg_set_work_table(atrex_agg_t* h, const atrex_work_t* rows, uint64_t 
     return ATREX_OK;
 }
 
+// The directory sums kept per scatter CTA join the table.
+static int fold_directory(atrex_agg* h, cudaStream_t s) {
+    if (h->img_rows == 0) return ATREX_OK;
+    CU(h, launch_hot_fold(h->hot_keys, h->hot_img, h->img_rows, h->L.hot_slots, h->table_ref(), s));
+    h->launches++;
+    h->img_rows = 0;
+    return ATREX_OK;
+}
+
 // Partition pass over the spill buffers.  Unforced, the kernel exits at once unless the scatter
 // launch just before it saw a buffer more than 3/4 full; forced (before results are read), it
 // drains whatever is there.
 static int drain_spill(atrex_agg* h, bool force, cudaStream_t s) {
     if (force && !h->spill_pending) return ATREX_OK;
-    if (force && h->img_rows) {
-        // results are about to be read: the directory sums kept per scatter CTA join the table (before the
-        // spilled entries do, while the frequent keys' slots are still easy to come by)
-        CU(h, launch_hot_fold(h->hot_keys, h->hot_img, h->img_rows, h->L.hot_slots, h->table_ref(), s));
-        h->launches++;
-        h->img_rows = 0;
+    if (force) {
+        // results are about to be read (the directory's sums before the spilled entries, while the frequent keys' slots are
+        // still easy to come by)
+        const int rc = fold_directory(h, s);
+        if (rc != ATREX_OK) return rc;
     }
     PartitionParams q;
     q.t = h->table_ref();
@@ -490,6 +505,8 @@ static int drain_spill(atrex_agg* h, bool force, cudaStream_t s) {
     q.queue_cap = h->L.queue_cap;
     q.force = force ? 1u : 0u;
     q.seq = h->scatter_seq;
+    q.told_long = h->h_long;
+    q.trace = h->trace;
     CU(h, launch_partition(q, h->n_sms, s));
     h->launches++;
     if (force) h->spill_pending = false;
@@ -520,6 +537,15 @@ static int ingest_launch(atrex_agg* h, const atrex_record_t* recs, uint64_t n, c
         h->launches++;
         return ATREX_OK;
     }
+    // Where the entries had to become long, the directory has been empty since: the first call that hears of it builds
+    // another, in the form that holds operators of any size, from its own records.  (2^27-record calls, from the second on half of
+    // the records with operators that the first did not have: FIGURES)
+    if (h->hot_ready && !h->long_only && *(const volatile ull*)h->h_long == h->trace) {
+        const int rc = fold_directory(h, s);
+        if (rc != ATREX_OK) return rc;
+        h->hot_ready = false;
+        h->long_only = true;
+    }
     // hot directory from a sample of the first call after create/reset that takes the two-pass route
     if (h->L.hot_slots && !h->hot_ready) {
         HotBuildParams b;
@@ -534,7 +560,7 @@ static int ingest_launch(atrex_agg* h, const atrex_record_t* recs, uint64_t n, c
         b.n_apps = h->cfg.n_apps;
         b.n_phases = h->cfg.n_phases;
         b.hot_keys = h->hot_keys;
-        b.max_ops = h->L.fmt.max_ops;
+        b.max_ops = h->long_only ? 0 : h->L.fmt.max_ops;
         b.dur_mask = h->L.fmt.dur_mask();
         b.hot_slots = h->L.hot_slots;
         b.hot_words = (uint32_t*)(h->ws + h->L.off_hot_words);
@@ -962,7 +988,9 @@ int atrex_agg_hot_directory(atrex_agg_t* h, uint64_t* h_keys, uint32_t cap, uint
     cudaStream_t s = (cudaStream_t)stream;
     ull* image = (ull*)malloc((size_t)h->L.hot_slots * 8);
     if (!image) return ATREX_ERR_NOMEM;
+    ull form = FORM_LONG;
     cudaError_t e = cudaMemcpyAsync(image, h->hot_keys, (size_t)h->L.hot_slots * 8, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&form, &h->ctl->form, sizeof(form), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
         free(image);
@@ -970,7 +998,7 @@ int atrex_agg_hot_directory(atrex_agg_t* h, uint64_t* h_keys, uint32_t cap, uint
         return ATREX_ERR_CUDA;
     }
     uint32_t n = 0;
-    for (uint32_t i = 0; i < h->L.hot_slots; ++i) {
+    for (uint32_t i = 0; form != FORM_LONG_ONLY && i < h->L.hot_slots; ++i) {
         if (image[i] == 0) continue;
         if (n < cap) h_keys[n] = ~image[i];
         ++n;

@@ -61,7 +61,7 @@ constexpr ull SKEW_NONE = 0, SKEW_COMBINE = 1, SKEW_DOMINATED = 2;
 // The spill entries' form and with it the directory's, chosen by the directory build (0, after a reset: 12-byte entries and
 // the directory's tags form, if there is one).
 constexpr ull FORM_LONG = 0, FORM_SHORT = 1;
-constexpr ull FORM_LONG_ONLY = 2;   // 12-byte entries and no more directory (too many records did not fit its words)
+constexpr ull FORM_LONG_ONLY = 2;   // 12-byte entries and an empty directory (too many records did not fit its words), until another is built
 
 struct Control {
     ull status;

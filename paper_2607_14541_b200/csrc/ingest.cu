@@ -679,14 +679,16 @@ __global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(const __gr
         partition_cta<FORM_TIGHT>(q, smem_raw);
     grid_dependents_launch();
     // The last CTA rewinds the hand-out counter for the next launch.  Where many records did not fit the form of the
-    // entries, the next ones are long (the buffers are empty now).
+    // entries, the next ones are long (the buffers are empty now); the directory stays empty until the host, which is told,
+    // has another built.
     if (threadIdx.x == 0) {
         __threadfence();
         if (atomicAdd(&ctl->part_done, 1ull) == gridDim.x - 1) {
             ctl->part_cursor = ctl->part_done = ctl->rests = 0;
             if (misfits) {
                 ctl->form = FORM_LONG_ONLY;
-                ctl->n_misfit = 0;
+                ctl->n_misfit = ctl->hot_n = 0;
+                *(volatile ull*)q.told_long = q.trace;
             }
         }
     }
@@ -930,6 +932,7 @@ __global__ void __launch_bounds__(LEVEL_THREADS) hot_level_kernel(HotBuildParams
     if (t == 0) {
         x.threshold = 1024u - above;
         p.ctl->hot_skew = skew;
+        p.ctl->hot_n = p.ctl->prefetch = 0;     // (hot_pick_kernel adds up)
         p.ctl->form = words ? FORM_SHORT : FORM_LONG;
     }
 }

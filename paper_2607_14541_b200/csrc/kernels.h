@@ -93,6 +93,8 @@ struct PartitionParams {
     ull seq;
     ulonglong2* queue;         // [gridDim][queue_cap] entries whose first look failed, settled after the partition's stream
     uint32_t queue_cap;
+    ull* told_long;            // pinned: `trace`, once its entries had to become long
+    ull trace;
 };
 
 // Scratch of the directory build's last steps (cleared by every build up to `key`).

@@ -172,3 +172,37 @@ def test_entries_are_long_where_many_durations_take_two(long_share, is_short, ho
     ingest(agg, recs)
     st = agg.stats()
     assert st["spill_cap"] == (cap // 2 * 3 if is_short else cap) and st["n_spilled"] > 0
+
+
+def test_a_directory_is_built_anew_where_operators_no_longer_fit():
+    """500 keys hold most of the trace.  When half of its records turn to operators that do not fit, the directory is given up;
+    the call after that finds one for the records as they are now, and a reset starts afresh."""
+    import torch
+    import paper_2607_14541_b200 as p
+    rng = np.random.default_rng(11)
+    part = (1 << 20) + 5
+    recs = np.zeros(4 * part, dtype=RECORD_DTYPE)
+    recs["app_id"], recs["phase"] = rng.integers(0, 9, len(recs)), rng.integers(0, 2, len(recs))
+    recs["op_id"] = rng.integers(0, 5, len(recs))
+    recs["shape_id"] = np.where(rng.random(len(recs)) < 0.9, rng.integers(0, 50, len(recs)), rng.integers(50, 100_000, len(recs)))
+    recs["duration_ns"] = rng.integers(0, 1 << 20, len(recs))
+    recs["op_id"][part:] += np.where(rng.random(len(recs) - part) < 0.5, 5_000, 0).astype(np.uint16)
+    weights = rng.integers(0, 1 << 16, 9).astype(np.uint32)
+    agg = p.Aggregator(weights, 2, 3_000_000)
+    for _ in range(2):
+        o = oracle.Oracle(weights, 2)
+        held, spilled = [], [0]
+        for at in range(0, len(recs), part):
+            ingest(agg, recs[at: at + part])
+            o.ingest(recs[at: at + part], threads=4)
+            torch.cuda.synchronize()
+            held.append(agg.hot_directory() >> np.uint64(32) & np.uint64(0xFFFF))
+            st = agg.stats()
+            spilled.append(st["n_spilled"])
+            assert st["hot_slots"] == len(held[-1]) and st["max_spill_fill"] <= st["spill_cap"]
+        check(agg, o)
+        assert len(held[0]) >= 490 and held[0].max() < 5
+        assert len(held[1]) == 0
+        assert all((h < 5).sum() >= 490 and (h >= 5_000).sum() >= 490 for h in held[2:])
+        assert spilled[4] - spilled[3] < 0.2 * part
+        agg.reset()
