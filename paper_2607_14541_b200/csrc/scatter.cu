@@ -54,6 +54,7 @@ struct Smem {
     static constexpr uint32_t APPW = CUR + 4u * P;              // u32[APPW_SMEM_MAX]  card-hour weights
     static constexpr uint32_t LONG = APPW + 4u * APPW_SMEM_MAX;    // words: records that took two short entries
     static constexpr uint32_t RESTS = LONG + 4u;                // ... whether an entry's identity has a rest
+    static constexpr uint32_t MISFITS = LONG + 8u;              // ... records whose operator does not fit
     static constexpr uint32_t WORDS = LONG + 16u;               // ... u32[SLOTS]
     static constexpr uint32_t TAG = LONG;                       // tags: u32[NB + 1]  four 8-bit tags per bucket (+ one pad bucket)
     static constexpr uint32_t KEYS = (TAG + 4u * (NB + 1u) + 7u) & ~7u;   // ull[SLOTS + 4]  key, all ones = empty
@@ -144,12 +145,13 @@ __device__ __noinline__ void drain_slot(TableRef t, uint32_t acc, ull key, uint3
 // (rare) A record that cannot take the limb route: straight to the table with full 64-bit adds.
 __device__ __noinline__ void table_route(TableRef t, ull key, uint32_t h, ull prod) { table_accumulate(t, key, h, prod, 0, 1); }
 // (rare) An invalid record is counted; a valid one whose product has bits at or above 2^48, or whose operator does not
-// fit, goes to the table.
+// fit, goes to the table.  Those are counted in shared memory: there may be many, and a counter of the whole GPU takes
+// no more than one and a half in a nanosecond.
 template <bool COUNT_MISFITS>
-__device__ __noinline__ void rare_record(TableRef t, bool valid, ull key, uint32_t h, ull prod) {
+__device__ __noinline__ void rare_record(TableRef t, bool valid, ull key, uint32_t h, ull prod, uint32_t misfits) {
     if (valid) {
         table_accumulate(t, key, h, prod, 0, 1);
-        if (COUNT_MISFITS && (uint32_t)(prod >> 32) < 0x10000u) atomicAdd(&t.ctl->n_misfit, 1ull);
+        if (COUNT_MISFITS && (uint32_t)(prod >> 32) < 0x10000u) reds_add(misfits, 1u);
     } else
         atomicAdd(&t.ctl->n_rejected, 1ull);
 }
@@ -270,7 +272,7 @@ __device__ __forceinline__ void one_record(const IngestParams& p, Ctx& c, uint32
     // (words form: an operator that no sampled record had may not fit a word and a short entry)
     if (L::W) todo_in = todo_in && (khi & 0xFFFFu) < p.fmt.max_ops;
     bool todo = todo_in;
-    if ((FULL || present) && !todo_in) rare_record<L::W>(p.t, ok, key, h, prod);
+    if ((FULL || present) && !todo_in) rare_record<L::W>(p.t, ok, key, h, prod, c.sb + L::MISFITS);
     if (DIR != DIR_NONE) {
         const uint32_t x = dir_mix(h, khi >> 16, c.mult);
         uint32_t at;
@@ -743,7 +745,7 @@ __device__ __forceinline__ void scatter_cta(const IngestParams& p, Ctx& c, unsig
     uint32_t* g_cursor = reinterpret_cast<uint32_t*>(smem_raw + L::CUR);
     uint32_t* g_acc = reinterpret_cast<uint32_t*>(smem_raw + L::ACC);
     const ull skew = DIR != DIR_NONE ? p.t.ctl->hot_skew : SKEW_NONE;
-    if (L::W && threadIdx.x < 2) reinterpret_cast<uint32_t*>(smem_raw + L::LONG)[threadIdx.x] = 0;
+    if (L::W && threadIdx.x < 3) reinterpret_cast<uint32_t*>(smem_raw + L::LONG)[threadIdx.x] = 0;
     if (L::W) {
         for (uint32_t i = threadIdx.x; i < L::SLOTS / 4; i += blockDim.x) reinterpret_cast<uint4*>(smem_raw + L::WORDS)[i] = p.hot_words[i];
         for (uint32_t i = threadIdx.x; i < L::SLOTS * 3 / 4; i += blockDim.x) reinterpret_cast<uint4*>(g_acc)[i] = make_uint4(0, 0, 0, 0);
@@ -783,6 +785,8 @@ __device__ __forceinline__ void scatter_cta(const IngestParams& p, Ctx& c, unsig
     if (L::W && threadIdx.x == 0) {
         spilled = 0u - *reinterpret_cast<const uint32_t*>(smem_raw + L::LONG);      // (records, not entries)
         if (*reinterpret_cast<const uint32_t*>(smem_raw + L::RESTS)) p.t.ctl->rests = 1;
+        const uint32_t misfits = *reinterpret_cast<const uint32_t*>(smem_raw + L::MISFITS);
+        if (misfits) atomicAdd(&p.t.ctl->n_misfit, (ull)misfits);
     }
     for (uint32_t i = threadIdx.x; i < L::P; i += blockDim.x) {
         const size_t at = ((size_t)blockIdx.x << LP) + i;
