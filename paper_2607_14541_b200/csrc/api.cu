@@ -96,9 +96,12 @@ void compute_layout(const atrex_agg_config_t* c, size_t smem_optin, int n_sms, L
     L->n_slots = (ull)L->C << L->lp;
     L->n_groups = (uint32_t)n_sms;
     L->sub_launch = c->max_keys >= (1ull << 21) ? (1ull << 27) : (c->max_keys >= (1ull << 16) ? (1ull << 25) : (1ull << 24));
-    // room for 4.5 launches' worth of entries if every record spilled; a drain is requested when a
-    // buffer passes 3/4 of that, which leaves more than one full launch of headroom.  At the bench
-    // workload (half of the records spill) four launches accumulate between drains.
+    // room for 4.5 launches' worth of long entries if every record spilled, 6.75 of short ones; a drain is requested when a
+    // buffer passes 3/4 of that, which leaves 1.1 and 1.7 full launches of headroom.  A short entry's record takes two where its
+    // duration is long: a launch that is mostly such asks from 5/8 on, which leaves room for two entries a record.  (Only
+    // where short durations turn into long ones from one launch to the next may a buffer still run over: exact, but
+    // record by record.)  At the bench workload (half of the records spill) four or five launches
+    // accumulate between drains.
     ull per_buf = (L->sub_launch * 9 / 2) / (((ull)n_sms) << L->lp);
     if (per_buf < 64) per_buf = 64;
     if (per_buf > 32768) per_buf = 32768;   // the scatter pass counts a buffer's entries in 16 bits, with headroom
@@ -616,6 +619,7 @@ static int ingest_launch(atrex_agg* h, const atrex_record_t* recs, uint64_t n, c
     p.drain_above = h->L.cap / 4 * 3;
     p.short_cap = h->L.cap / 2 * 3;       // (the same bytes)
     p.short_drain_above = p.short_cap / 4 * 3;
+    p.long_drain_above = p.short_cap / 8 * 5;
     p.seq = ++h->scatter_seq;
     p.img_rows = h->img_rows;
     CU(h, launch_scatter(p, h->hot_ready, grid, s));

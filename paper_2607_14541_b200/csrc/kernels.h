@@ -62,7 +62,8 @@ struct IngestParams {
     uint32_t n_groups;         // G, row pitch of the buffers (= CTAs of the widest scatter launch)
     uint32_t cap;              // entries per (partition, CTA) buffer, a multiple of 32 (whole 128-byte lines)
     uint32_t drain_above;      // ask for a drain when a buffer holds more entries than this
-    uint32_t short_cap, short_drain_above;   // the same in short entries
+    uint32_t short_cap, short_drain_above;   // the same in short entries ...
+    uint32_t long_drain_above;               // ... of which many records take two
     ull seq;                   // sequence number of this launch
 };
 

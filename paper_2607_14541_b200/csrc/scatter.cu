@@ -779,7 +779,10 @@ __device__ __forceinline__ void scatter_cta(const IngestParams& p, Ctx& c, unsig
 
     grid_dependents_launch();
     __syncthreads();
-    const uint32_t cap = L::W ? p.short_cap : p.cap, drain_above = L::W ? p.short_drain_above : p.drain_above;
+    const uint32_t cap = L::W ? p.short_cap : p.cap;
+    uint32_t drain_above = L::W ? p.short_drain_above : p.drain_above;
+    // (where three eighths of the launch's records took two entries, the next launch may bring two entries for each of its)
+    if (L::W && (ull)*reinterpret_cast<const uint32_t*>(smem_raw + L::LONG) * gridDim.x >= p.n_pairs / 4 * 3) drain_above = p.long_drain_above;
     uint32_t spilled = 0, fullest = 0;
     bool crowded = false;
     if (L::W && threadIdx.x == 0) {

@@ -206,3 +206,32 @@ def test_a_directory_is_built_anew_where_operators_no_longer_fit():
         assert all((h < 5).sum() >= 490 and (h >= 5_000).sum() >= 490 for h in held[2:])
         assert spilled[4] - spilled[3] < 0.2 * part
         agg.reset()
+
+
+def test_buffers_have_room_for_two_entries_a_record():
+    """Equally frequent keys, the first call's durations short, all others long, in calls of unequal size that leave the buffers
+    just below the line that short durations are drained at: the full launch that follows must find room."""
+    import torch
+    import paper_2607_14541_b200 as p
+    rng = np.random.default_rng(5)
+    n, n_keys = 1 << 25, 500_000                                   # (records of one launch of such a table)
+    recs = np.zeros(n, dtype=RECORD_DTYPE)
+    recs["app_id"], recs["shape_id"] = rng.integers(0, 64, n), rng.integers(0, n_keys, n)
+    recs["op_id"] = recs["shape_id"] % 7
+    recs["duration_ns"] = (1 << 28) - 1
+    few = recs[: (1 << 22) + 64].copy()                          # (fewer go straight into the table)
+    few["duration_ns"] = 50_000
+    weights = np.arange(1, 65, dtype=np.uint32)
+    agg = p.Aggregator(weights, 2, 1_000_000)
+    o = oracle.Oracle(weights, 2)
+    cap = agg.stats()["spill_cap"]
+    ingest(agg, few)
+    o.ingest(few, threads=8)
+    on_gpu = torch.from_numpy(recs.view(np.uint8).reshape(-1)).cuda()
+    for part in (n, n, n // 8, n):
+        agg.ingest(on_gpu, n=part)
+        o.ingest(recs[:part], threads=8)
+    st = agg.stats()
+    assert st["spill_cap"] == cap // 2 * 3 and st["n_spilled"] > 0.9 * st["n_valid"]
+    assert st["n_overflow"] == 0
+    check(agg, o)
