@@ -128,8 +128,9 @@ typedef struct {
                                              only, the most that one thread block's table held */
     uint64_t n_spilled;                   /* records that went through the partition spill buffers */
     uint64_t n_overflow;                  /* records that found their spill buffer full (slow exact path) */
-    uint64_t max_spill_fill;              /* fullest spill buffer seen since reset, in entries */
-    uint64_t spill_cap;                   /* capacity of one spill buffer, in entries */
+    uint64_t max_spill_fill;              /* fullest spill buffer seen since reset, in entries of the form in use now: 8 or
+                                             12 bytes (a record takes one, or two of 8 bytes where its duration is long) */
+    uint64_t spill_cap;                   /* capacity of one spill buffer, in the same entries */
     uint64_t n_drains;                    /* partition passes that ran since reset */
 } atrex_stats_t;
 

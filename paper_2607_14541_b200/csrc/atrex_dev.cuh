@@ -79,7 +79,7 @@ struct Control {
     ull n_spilled;             // records routed through the spill buffers
     ull n_overflow;            // records that found their spill buffer full (slow exact path)
     ull drain_seq;             // sequence number of the last scatter launch that asked for a drain
-    ull max_fill;              // fullest spill buffer seen since reset (entries)
+    ull max_fill;              // fullest spill buffer seen since reset (entries of the present form)
     ull n_drains;              // partition passes that actually ran
     ull dir_mult;              // multiplier of the hot directory's bucket hash chosen at build time
     ull part_cursor;           // partition pass: next partition to hand out (zeroed before each launch)

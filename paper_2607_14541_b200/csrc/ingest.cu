@@ -688,6 +688,7 @@ __global__ void __launch_bounds__(INGEST_THREADS, 1) partition_kernel(const __gr
             if (misfits) {
                 ctl->form = FORM_LONG_ONLY;
                 ctl->n_misfit = ctl->hot_n = 0;
+                ctl->max_fill = (ctl->max_fill * SHORT_ENTRY_BYTES + SPILL_ENTRY_BYTES - 1) / SPILL_ENTRY_BYTES;   // (in entries: as many bytes)
                 *(volatile ull*)q.told_long = q.trace;
             }
         }

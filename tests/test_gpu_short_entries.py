@@ -235,3 +235,28 @@ def test_buffers_have_room_for_two_entries_a_record():
     assert st["spill_cap"] == cap // 2 * 3 and st["n_spilled"] > 0.9 * st["n_valid"]
     assert st["n_overflow"] == 0
     check(agg, o)
+
+
+def test_fill_and_capacity_are_told_in_the_same_entries():
+    """Buffers that ran over with short entries, whose capacity counts long ones after operators that do not fit."""
+    import paper_2607_14541_b200 as p
+    rng = np.random.default_rng(6)
+    first, crowd, wide = (1 << 22) + 1, 1 << 20, 600_000
+    recs = np.zeros(first + crowd + wide, dtype=RECORD_DTYPE)
+    recs["op_id"], recs["shape_id"] = rng.integers(0, 5, len(recs)), rng.integers(0, 50_000, len(recs))
+    recs["duration_ns"] = 1_000
+    recs["op_id"][first: first + crowd], recs["shape_id"][first: first + crowd] = 6, 77_777
+    recs["op_id"][first + crowd:] += 5_000
+    weights = np.array([3], dtype=np.uint32)
+    agg = p.Aggregator(weights, 1, 300_000)
+    o = oracle.Oracle(weights, 1)
+    o.ingest(recs, threads=8)
+    cap = agg.stats()["spill_cap"]
+    ingest(agg, recs[:first])
+    ingest(agg, recs[first: first + crowd])
+    st = agg.stats()
+    assert st["spill_cap"] == st["max_spill_fill"] == cap // 2 * 3 and st["n_overflow"] > 0
+    ingest(agg, recs, first + crowd)
+    st = agg.stats()
+    assert st["spill_cap"] == st["max_spill_fill"] == cap
+    check(agg, o)
