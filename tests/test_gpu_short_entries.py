@@ -260,3 +260,26 @@ def test_fill_and_capacity_are_told_in_the_same_entries():
     st = agg.stats()
     assert st["spill_cap"] == st["max_spill_fill"] == cap
     check(agg, o)
+
+
+def test_the_largest_table_filled():
+    """As many keys as the largest table is provisioned for, those of an (operator, shape) in all eight phases, with the weights of
+    4 096 applications beside a partition's slots in shared memory (the least slots a key can have): none is dropped."""
+    import torch
+    import paper_2607_14541_b200 as p
+    n, phases = 1 << 25, 8
+    key = torch.arange(n, device="cuda")
+    pair = key // phases
+    recs = torch.empty(n, 4, dtype=torch.int32, device="cuda")
+    recs[:, 0] = key % 4096
+    recs[:, 1] = pair % 200 | (key % phases) << 16
+    recs[:, 2] = pair // 200 * 2654435761 % (1 << 31)
+    recs[:, 3] = 1_000
+    agg = p.Aggregator(np.full(4096, 5, dtype=np.uint32), phases, n)
+    for half in (recs[: n // 3], recs[n // 3:], recs):              # new keys beside old ones, then all of them found again
+        agg.ingest(half)
+        agg.stats()
+    st = agg.stats()
+    assert st["n_keys"] == n and st["n_dropped"] == 0 and st["keys_per_phase"][:phases] == [n // phases] * phases
+    assert st["table_slots"] < 1.31 * n
+    assert st["totals"][:phases] == [2 * n // phases * 5 * 1_000] * phases
