@@ -71,8 +71,9 @@ bool config_ok(const atrex_agg_config_t* c) {
 }
 
 void compute_layout(const atrex_agg_config_t* c, size_t smem_optin, int n_sms, Layout* L) {
-    // Partition geometry: one partition's keys + per-launch accumulators (20 B per slot) must fit one
-    // SM's shared memory.  A key can only live in its hash partition, so a partition is sized for the
+    // Partition geometry: one partition's keys + per-launch accumulators (20 B per slot) and, where entries may be
+    // short, the applications' weights must fit one SM's shared memory (10 688 slots beside 4 096 weights and not 11 488:
+    // 2^30 records over 16 M keys, whole build +0.5 %).  A key can only live in its hash partition, so a partition is sized for the
     // tail of its load, not for the mean: with m = max_keys / P keys expected, the keys of one
     // (operator, shape) -- up to n_phases of them -- always fall together, which bounds the standard
     // deviation by sqrt(n_phases * m); six of those plus a constant, and never less than 1.3 m (2 m for small tables).

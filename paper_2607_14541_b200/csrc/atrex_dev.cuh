@@ -234,7 +234,7 @@ __device__ __forceinline__ uint32_t part_of(uint32_t h, uint32_t lp) { return h 
 // visits every pair once.  Every prober -- this file's global-memory path and the partition pass's
 // shared-memory path -- follows the same order, and a key sits at the first slot of its sequence
 // that was free when it arrived.  Clusters of linear probing, which at the load factors reached
-// here (up to 0.7) made the slowest of a warp's probes several times the average, do not form.
+// here (up to 0.77: 2^25 keys beside the weights of 4 096 applications) made the slowest of a warp's probes several times the average, do not form.
 // The phase, which the partition choice ignores, is mixed into the start so that the phases of one
 // (operator, shape) do not pile up on the same pair.
 //

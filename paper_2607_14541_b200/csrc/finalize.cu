@@ -60,7 +60,7 @@ static_assert(FIRST_BINS <= TOPK_BINS && FIRST_BINS % 4 == 0, "first digits fit 
 // moves the accumulators to their place and clears them (and the emit kernel's output count), so that no
 // launch is spent on clearing.  On the way the keys are counted by the first digit of the top-k selection (per
 // phase, for the top-k), which saves that call a pass over the table; the next pass's counters are
-// cleared here.  Bound by DRAM (566 MB: 120 us), given 512 threads per SM or more: shared memory holds that many up to eight
+// cleared here.  Bound by DRAM (525 MB: 91 us), given 512 threads per SM or more: shared memory holds that many up to eight
 // phases (16 M keys, whole finalize: five phases 650 -> 569 us, eight 650 -> 582; with one CTA of 256 threads before).
 __device__ __forceinline__ bool last_cta(ull* done) {
     __shared__ bool s_last;
@@ -272,7 +272,7 @@ __device__ __forceinline__ void load_phase_totals(const Control* ctl, double* dT
 // divisions and the work-table probe run on full warps instead of one lane in three.  A lane probes for two
 // entries side by side (four need more registers than four CTAs per SM have, and three CTAs are slower), and the entries
 // go out through shared memory in whole lines.  Bound by latency and instructions at half occupancy (3.1 M keys
-// of 5.8 M slots: 121 -> 97 us, DRAM 45 %; 15 M of 23.6 M: 540 -> 475; one entry at a time over the same buckets 155, four
+// of 5.8 M slots: 121 -> 97 us, DRAM 45 %; 15 M of 21.9 M: 540 -> 475; one entry at a time over the same buckets 155, four
 // 113; five CTAs of 48 registers: 2 % more on the whole refresh).
 constexpr int EMIT_ILP = 4;
 constexpr int EMIT_PROBES = 2;

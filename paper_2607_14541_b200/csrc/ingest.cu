@@ -138,10 +138,10 @@ __global__ void __launch_bounds__(FOLD_WARPS * 32) hot_fold_kernel(const ull* ho
 
 // --------------------------------------------------------------------------------------
 // Pass 2: a CTA aggregates one partition at a time entirely in shared memory.  CTAs are
-// persistent and take partitions blockIdx.x, blockIdx.x + gridDim.x, ...; while one partition
-// is processed, the next one's keys and spill entries are pulled into L2.  Per partition: copy the
-// keys in, each in the pass's own 64-bit form (phase, operator, 32-bit hash: unique inside a
-// partition, and what a spill entry carries); stream the entries of all scatter CTAs, four per lane,
+// persistent; each begins with partition blockIdx.x and draws its further ones from a counter, early enough that
+// their keys and first entries are pulled into L2 during the write-back.  Per partition: copy the
+// keys in, each in the form that the entries carry it in (FormKey below: 32 or 64 bits, unique inside a
+// partition); stream the entries of all scatter CTAs, four per lane,
 // and settle each with one look at the first pair of its probe sequence (hit, or a new key with room
 // there); entries that need more than that wait in the warp's segment of a per-CTA queue in global
 // memory and are settled, 32 per round, once the warp's share of the stream is through (or earlier,
@@ -833,6 +833,8 @@ __global__ void __launch_bounds__(256) hot_admit_kernel(HotBuildParams p) {
 // Zipf(1.1) over 6 144 keys: 791 us against 884), and where keys are equally frequent but fewer (2 048: 740 against 809,
 // 4 096: 811 against 860) or more (12 288: 1 056 against 1 082, 32 768: 1 357 against 1 808).  Between, tags hold more
 // (6 144: 909 against 940, 6 880: 933 against 966), and from TAGS_PART on where such keys hold only a part of the trace.
+// (These lines were measured while the scatter kernel spilled registers; without, words take 898 us against 935 at 6 144 keys
+// and 1 550 against 1 730 where they hold 45 %.)
 constexpr uint32_t TAGS_PART = 3500, TAGS_FROM = 5500, TAGS_TO = 7500, EVEN = 4;
 // A duration that takes two short entries makes 16 bytes of a record, a long entry has 12.  Whole builds of 2^27 records, long
 // entries and then short ones at a share of such durations of 0, 0.2, 0.5 and 1:
