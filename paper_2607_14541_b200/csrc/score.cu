@@ -11,9 +11,10 @@
 // the result has one bit pattern.
 //
 // Where a unit goes when units are grouped by operator is the same for every candidate, so a CTA works
-// that out once and then goes through its candidates.  Two kernels:
+// that out once and then goes through its candidates.  Three kernels:
 //   score_warp_kernel  one candidate per warp, no barriers: many candidates of few units
 //   score_cta_kernel   one candidate per CTA: few candidates, or more units than a warp should hold
+//   score_bins_kernel  one candidate per CTA, no grouping: operators of 64 units and more
 // The kernel before these (one candidate per CTA, grouping redone for every candidate, exact scores ranked
 // against each other) was bound by its barriers and shared-memory atomics: 65 536 candidates x 440 units x
 // 30 operators in 594 us, 1 000 x 12 001 units x 7 operators in 1 179 us.
@@ -897,6 +898,280 @@ __global__ void __launch_bounds__(1024)
     }
 }
 
+// ---- one candidate per CTA, large groups ------------------------------------------------------------
+// No order is made of an operator's units: while their keys are formed, each bumps one of its operator's counters by
+// the key's range, a warp finds the range that holds the middle, and the few units in it (or as close to it as
+// keys may err) are ranked by their exact scores.  Every step but the finding is spread over the whole CTA, and units stay
+// where they are, so that nothing is worked out about the grouping.  Where the middle's range holds too many units it is
+// cut again; what stays too many (ties) is searched among them.  Bound by latency at 48 warps per SM (loads, shared-memory
+// atomics, barriers: 40 % of the issue slots).  1 000 candidates x 12 001 units x 7 operators: 145 us by score_cta_kernel, 78;
+// with the next loads issued before a thread's units are worked on 116 (spills); strides not known at compile time 86.
+constexpr uint32_t NEAR_MAX = 32;             // units near an operator's middle that one warp ranks, a lane each
+constexpr uint32_t BINS_LOW = (127u - 7u) << 23, BINS_LOG_SPAN = 26;   // first cut: scores from 2^-7 to 2, what lies outside in the end bins
+constexpr uint32_t CUTS_MAX = 6;              // (each narrows the range 32-fold or more)
+constexpr uint32_t NOWHERE = 0xFFFFFFFFu;     // no key is as close above it
+
+struct BinsLayout {
+    uint32_t prod, window, state, bins, listed, list, spare, op, total;
+    __host__ __device__ BinsLayout(uint32_t n, uint32_t n_ops, uint32_t log_bins, uint32_t threads) {
+        uint32_t o = (4u * n + 15u) & ~15u;          // (keys first)
+        state = o;   o += 16u * n_ops;               // {lowest key of the middle's range, usable units below it, usable units, how to go on}
+        bins = o;    o += n_ops << (log_bins + 1u);  // two counters to a word
+        window = o;  o += 8u * (n_ops + 1u);                // {from, span}: units whose keys are near the middle; or {from, shift} of the next cut
+        prod = o;    o += 8u * n_ops;                // w * S
+        listed = o;  o += 4u * n_ops;
+        list = o;    o += 2u * NEAR_MAX * n_ops;     // units near the middle
+        spare = o = (o + 15u) & ~15u;  o += threads / 32u * 4u * SELECT_BINS;
+        op = o;      o += n;
+        total = (o + 15u) & ~15u;
+    }
+};
+// Counters per operator: a quarter of the mean group, so that the middle's range holds about ten units of an even distribution.
+inline uint32_t log_bins_for(uint32_t n, uint32_t n_ops) {
+    uint32_t b = 6;
+    while (b < 10 && (4u * n_ops << b) < n) ++b;
+    return b;
+}
+constexpr uint32_t GO_NONE = 0, GO_RANK = 1, GO_CUT = 2, GO_SEARCH = 3, GO_SEARCH_ALL = 4;
+
+// The counter (of 2 W per lane, W words) that holds the k-th counted unit; `incl`, `own`: units up to and in this lane's counters.
+struct Bin {
+    uint32_t at, before, n;
+};
+__device__ __forceinline__ Bin find_bin(const uint32_t* words, uint32_t W, uint32_t incl, uint32_t own, uint32_t k) {
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t src = __ffs(__ballot_sync(FULL, incl > k)) - 1, base = __shfl_sync(FULL, incl - own, src);
+    if (W == 1) {
+        const uint32_t word = words[src], first = word & 0xFFFFu;
+        return base + first > k ? Bin{2 * src, base, first} : Bin{2 * src + 1, base + first, word >> 16};
+    }
+    uint32_t c = 0;
+    if (lane < 2 * W) {
+        const uint32_t word = words[src * W + lane / 2];
+        c = lane & 1u ? word >> 16 : word & 0xFFFFu;
+    }
+    uint32_t upto = c;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const uint32_t o = __shfl_up_sync(FULL, upto, d);
+        if (lane >= (uint32_t)d) upto += o;
+    }
+    const uint32_t in = __ffs(__ballot_sync(FULL, base + upto > k)) - 1;
+    return {src * 2 * W + in, base + __shfl_sync(FULL, upto - c, in), __shfl_sync(FULL, c, in)};
+}
+
+constexpr int bins_ctas(int threads) { return threads == 1024 ? 1 : 1536 / threads; }   // per SM, by registers
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, bins_ctas(THREADS))
+    score_bins_kernel(const double* __restrict__ roofline_s, const uint32_t* __restrict__ unit_op, uint32_t n_units,
+                      const double* __restrict__ t_cand, const uint8_t* __restrict__ correct, uint32_t n_cand,
+                      const double* __restrict__ w, uint32_t n_ops, uint32_t log_bins, double* s_agg, double* s_op_out, ull* errors_out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ uint32_t s_errors[2];
+    constexpr uint32_t U = 4;                                            // units of a thread in flight
+    __shared__ uint32_t s_cut;                                           // round of cuts that is still wanted
+    const BinsLayout L(n_units, n_ops, log_bins, THREADS);
+    uint32_t* keys = reinterpret_cast<uint32_t*>(smem_raw);
+    uint4* state = reinterpret_cast<uint4*>(smem_raw + L.state);
+    uint32_t* bins = reinterpret_cast<uint32_t*>(smem_raw + L.bins);
+    uint2* window = reinterpret_cast<uint2*>(smem_raw + L.window);
+    double* prod = reinterpret_cast<double*>(smem_raw + L.prod);
+    uint32_t* listed = reinterpret_cast<uint32_t*>(smem_raw + L.listed);
+    uint16_t* list = reinterpret_cast<uint16_t*>(smem_raw + L.list);
+    uint8_t* ops = smem_raw + L.op;                                      // n_ops: none
+    uint32_t* spare = reinterpret_cast<uint32_t*>(smem_raw + L.spare) + (threadIdx.x >> 5) * SELECT_BINS;
+    const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u, n_warps = THREADS / 32;
+    const uint32_t n_bins = 1u << log_bins, op_words = n_bins / 2, W = op_words / 32, first_shift = BINS_LOG_SPAN - log_bins;
+    for (uint32_t j = threadIdx.x; j < n_units; j += THREADS) {
+        const uint32_t op = unit_op[j];
+        ops[j] = (uint8_t)min(op, n_ops);
+    }
+    for (uint32_t i = threadIdx.x; i < n_ops * op_words; i += THREADS) bins[i] = 0;
+    for (uint32_t i = threadIdx.x; i < n_ops; i += THREADS) {
+        listed[i] = 0;
+        state[i].w = GO_NONE;
+    }
+    if (threadIdx.x == 0) {
+        s_errors[0] = s_errors[1] = s_cut = 0;
+        window[n_ops] = make_uint2(NOWHERE, 0);                          // (units without an operator)
+    }
+    __syncthreads();
+    auto count_in = [&](uint32_t op, uint32_t bin) { atomicAdd(&bins[op * op_words + bin / 2], 1u << (bin % 2 * 16)); };
+
+    uint32_t turn = 0;
+    for (uint32_t cand = blockIdx.x; cand < n_cand; cand += gridDim.x, turn ^= 1u) {
+        const double* t = t_cand + (size_t)cand * n_units;
+        const uint8_t* ok = correct + (size_t)cand * n_units;
+        if (cand + gridDim.x < n_cand) {   // the CTA's next candidate starts towards L2
+            const size_t ahead = (size_t)gridDim.x * n_units;
+            for (uint32_t o = threadIdx.x * 16u; o < n_units; o += THREADS * 16u) asm volatile("prefetch.global.L2 [%0];" ::"l"(t + ahead + o));
+            for (uint32_t o = threadIdx.x * 128u; o < n_units; o += THREADS * 128u) asm volatile("prefetch.global.L2 [%0];" ::"l"(ok + ahead + o));
+        }
+        // 1. approximate keys, counted by operator and range
+        uint32_t errors = 0;
+        auto some_units = [&](uint32_t j0, auto inside) {                // units j0, j0 + THREADS, ...
+            double tj[U], rj[U];
+            uint32_t okj[U];
+#pragma unroll
+            for (uint32_t u = 0; u < U; ++u) {
+                if (!inside(u)) continue;
+                tj[u] = __ldg(t + j0 + u * THREADS);
+                okj[u] = __ldg(ok + j0 + u * THREADS);
+                rj[u] = __ldg(roofline_s + j0 + u * THREADS);
+            }
+#pragma unroll
+            for (uint32_t u = 0; u < U; ++u) {
+                if (!inside(u)) continue;
+                const uint32_t op = ops[j0 + u * THREADS];
+                const uint32_t key = approx_key(approx_roofline(rj[u]), roofline_s + j0 + u * THREADS, tj[u], (okj[u] != 0) & (op != n_ops), errors);
+                keys[j0 + u * THREADS] = key;
+                if (key < K_UNKNOWN)
+                    count_in(op, min(n_bins - 1, (uint32_t)max((int)(key - BINS_LOW), 0) >> first_shift));
+                else if (key == K_UNKNOWN)
+                    state[op].w = GO_SEARCH_ALL;
+            }
+        };
+        uint32_t j0 = threadIdx.x;
+        for (; j0 + (U - 1) * THREADS < n_units; j0 += U * THREADS) some_units(j0, [](uint32_t) { return true; });
+        some_units(j0, [&](uint32_t u) { return j0 + u * THREADS < n_units; });
+        errors = __reduce_add_sync(FULL, errors);
+        if (lane == 0 && errors) atomicAdd(&s_errors[turn], errors);
+        __syncthreads();
+        // 2. the range of each operator's middle; once more inside it where it holds too many
+        for (uint32_t round = 1;; ++round) {
+            for (uint32_t op = warp; op < n_ops; op += n_warps) {
+                uint4 st = state[op];
+                if (round > 1 && st.w != GO_CUT) continue;
+                uint32_t* words = bins + op * op_words;
+                uint32_t own = 0;
+                for (uint32_t i = 0; i < W; ++i) own += (words[lane * W + i] & 0xFFFFu) + (words[lane * W + i] >> 16);
+                uint32_t incl = own;
+#pragma unroll
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint32_t o = __shfl_up_sync(FULL, incl, d);
+                    if (lane >= (uint32_t)d) incl += o;
+                }
+                uint32_t base = BINS_LOW, shift = first_shift, below = 0, m = __shfl_sync(FULL, incl, 31);
+                if (round > 1) {
+                    const uint2 cut = window[op];
+                    base = cut.x;
+                    shift = cut.y;
+                    below = st.y;
+                    m = st.z;
+                }
+                uint2 win = make_uint2(NOWHERE, 0);
+                if (st.w != GO_SEARCH_ALL) {
+                    st = make_uint4(0, 0, m, GO_NONE);
+                    if (m != 0) {
+                        const Bin low = find_bin(words, W, incl, own, (m - 1) / 2 - below);
+                        Bin up = low;
+                        if (!(m & 1u) && m / 2 - below >= low.before + low.n) up = find_bin(words, W, incl, own, m / 2 - below);
+                        uint32_t from = base + (low.at << shift), to = base + ((up.at + 1) << shift) - 1;
+                        if (round == 1 && low.at == 0) from = 0;
+                        if (round == 1 && up.at == n_bins - 1) to = K_UNKNOWN - 1;
+                        to = min(to, K_UNKNOWN - 1);
+                        st.x = from;
+                        st.y = below + low.before;
+                        const uint32_t in = up.before + up.n - low.before;
+                        st.w = in <= NEAR_MAX ? GO_RANK : (shift == 0 || round == CUTS_MAX ? GO_SEARCH : GO_CUT);
+                        if (st.w == GO_CUT) {
+                            const int len = 32 - __clz((int)(to - from));
+                            win = make_uint2(from, len > (int)log_bins ? len - log_bins : 0u);
+                        } else {
+                            const uint32_t first = from > K_APART ? from - K_APART : 0u;
+                            win = make_uint2(first, min(to + K_APART, K_UNKNOWN - 1) - first);
+                        }
+                    }
+                }
+                __syncwarp();
+                for (uint32_t i = lane; i < op_words; i += 32) words[i] = 0;
+                if (lane == 0) {
+                    state[op] = st;
+                    window[op] = win;
+                    if (st.w == GO_CUT) s_cut = round;
+                }
+            }
+            __syncthreads();
+            if (s_cut != round) break;
+            for (uint32_t j = threadIdx.x; j < n_units; j += THREADS) {
+                const uint32_t key = keys[j];
+                if (key >= K_UNKNOWN) continue;
+                const uint32_t op = ops[j];
+                if (state[op].w != GO_CUT) continue;
+                const uint2 cut = window[op];
+                const uint32_t bin = (key - cut.x) >> cut.y;
+                if (key >= cut.x && bin < n_bins) count_in(op, bin);
+            }
+            __syncthreads();
+        }
+        // 3. the units near the middles
+#pragma unroll 4
+        for (uint32_t j = threadIdx.x; j < n_units; j += THREADS) {
+            const uint32_t key = keys[j], op = ops[j];
+            const uint2 win = window[op];
+            if (key - win.x > win.y) continue;                           // (nothing is near K_UNKNOWN or above)
+            const uint32_t at = atomicAdd(&listed[op], 1u);
+            if (at < NEAR_MAX) list[op * NEAR_MAX + at] = (uint16_t)j;
+        }
+        __syncthreads();
+        // 4. Eq. 5 by their exact scores, and the products of Eq. 6
+        if (threadIdx.x == 0) s_cut = 0;
+        for (uint32_t op = warp; op < n_ops; op += n_warps) {
+            const uint4 st = state[op];
+            const uint32_t n = listed[op], m = st.z;
+            double s = 0.0;
+            if (st.w == GO_RANK && n <= NEAR_MAX) {
+                const uint32_t j = lane < n ? list[op * NEAR_MAX + lane] : 0u;
+                const ull x = lane < n ? exact_key(__ldg(roofline_s + j), __ldg(t + j), true) : ~0ull;
+                const uint32_t below = st.y - __popc(__ballot_sync(FULL, lane < n && keys[j] < st.x));   // units that are not listed
+                uint32_t less = 0, leq = 0;
+                for (uint32_t i = 0; i < n; ++i) {
+                    const ull y = __shfl_sync(FULL, x, i);
+                    less += y < x ? 1u : 0u;
+                    leq += y <= x ? 1u : 0u;
+                }
+                const uint32_t kl = (m - 1) / 2 - below, ku = m / 2 - below;
+                const ull k_lo = __shfl_sync(FULL, x, __ffs(__ballot_sync(FULL, lane < n && less <= kl && kl < leq)) - 1);
+                const ull k_hi = __shfl_sync(FULL, x, __ffs(__ballot_sync(FULL, lane < n && less <= ku && ku < leq)) - 1);
+                s = median_of_keys(k_lo, k_hi, m & 1u);
+            } else if (st.w != GO_NONE) {
+                // too many units alike, or units whose keys say nothing: exact scores of those near the middle, or of all
+                const bool all = st.w == GO_SEARCH_ALL;
+                const uint2 win = window[op];
+                auto key_at = [=](uint32_t j) {
+                    const uint32_t key = keys[j];
+                    const bool in = ops[j] == op && (all ? key != K_ABSENT : key < K_UNKNOWN && key - win.x <= win.y);
+                    return in ? exact_key(__ldg(roofline_s + j), __ldg(t + j), true) : ~0ull;
+                };
+                uint32_t counted = 0;      // all: the usable units; else the listed ones below the middle's range
+                for (uint32_t j = lane; j < n_units; j += 32)
+                    if (ops[j] == op) counted += all ? (keys[j] != K_ABSENT ? 1u : 0u) : (keys[j] - win.x <= win.y && keys[j] < st.x ? 1u : 0u);
+                counted = __reduce_add_sync(FULL, counted);
+                const uint32_t usable = all ? counted : m, below = all ? 0u : st.y - counted;
+                ull k_lo, k_hi;
+                warp_select<ull>(key_at, n_units, (usable - 1) / 2 - below, spare, &k_lo, &k_hi);
+                s = median_of_keys(k_lo, (usable & 1u) ? k_lo : k_hi, usable & 1u);
+            }
+            __syncwarp();
+            if (lane == 0) {
+                listed[op] = 0;
+                state[op].w = GO_NONE;
+                prod[op] = __dmul_rn(w[op], s);
+                if (s_op_out) s_op_out[(size_t)cand * n_ops + op] = s;
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {   // (the others go on to the next candidate: nothing of this is touched before two more barriers)
+            double agg = 0.0;     // Eq. 6 in operator order
+#pragma unroll 4
+            for (uint32_t i = 0; i < n_ops; ++i) agg = __dadd_rn(agg, prod[i]);
+            s_agg[cand] = agg;
+            if (errors_out) errors_out[cand] = s_errors[turn];
+            s_errors[turn] = 0;
+        }
+    }
+}
+
 // One candidate per warp (true) or per CTA (false); `held`: candidates an SM holds at once by warps.  A CTA has the shorter
 // chain, a warp the smaller sum of work, so the warps win once every SM has several candidates, and the sooner the better
 // the operators fill a warp's lanes.  Device times in us, warps / CTAs, on both sides of each line:
@@ -906,9 +1181,8 @@ __global__ void __launch_bounds__(1024)
 //                       operators, 900 candidates 22.0 / 22.0, 2 000 25.0 / 37.2; 2 000 units in 83, 1 500 candidates 58 / 43
 //   up to 50            5 per SM (8 from 44 on): two lanes an operator are full, and a CTA's warps search every group: 1 400 units
 //                       in 35 operators, 600 candidates 27.5 / 27.9, 1 500 36.0 / 44.0
-//   beyond              16 per SM up to a mean of 64, with fewer units the more groups are then too large for two lanes: 800 units
-//                       in 15 operators, 2 400 candidates 18 / 34; 1 000 in 17, 2 400 candidates 48 / 39, 3 500 41 / 57; 2 000 in
-//                       31, 2 400 candidates 157 / 67
+//   beyond (up to 64)   16 per SM, with fewer units the more groups are then too large for two lanes: 800 units
+//                       in 15 operators, 2 400 candidates 18 / 34; 1 000 in 17, 2 400 candidates 48 / 39, 3 500 41 / 57
 bool by_warps(uint32_t n, uint32_t n_ops, uint32_t b, uint32_t sms, uint32_t held) {
     if (held < (n <= 24 * n_ops ? 12u : 6u)) return false;
     if (n <= 500) return n <= 48 * n_ops ? b >= 4 * sms && b >= n : b >= 16 * sms;
@@ -916,7 +1190,7 @@ bool by_warps(uint32_t n, uint32_t n_ops, uint32_t b, uint32_t sms, uint32_t hel
     if (n <= 30 * n_ops) return b >= 8 * sms && enough;
     if (n <= 50 * n_ops) return b >= (n <= 44 * n_ops ? 5 : 8) * sms && (n <= 2200 || enough);
     if (n <= 700) return b >= 16 * sms;
-    return b >= 16 * sms && n <= 64 * n_ops && (ull)n * (n - 44 * n_ops) <= (b < 20 * sms ? 14000ull : 19000ull) * n_ops;
+    return b >= 16 * sms && (ull)n * (n - 44 * n_ops) <= (b < 20 * sms ? 14000ull : 19000ull) * n_ops;
 }
 
 // Threads of a CTA that holds one candidate.  Where there are more candidates than the SMs hold at 256 threads (four CTAs
@@ -927,6 +1201,26 @@ uint32_t cta_threads(uint32_t n, uint32_t n_ops, uint32_t b, uint32_t sms) {
     if (n > 1400 || b <= 4 * sms) return 256u;
     if (b <= 5 * sms) return n <= 36 * n_ops ? 192u : 256u;
     return n <= 30 * n_ops && (n <= 800 || b <= 8 * sms) ? 128u : 256u;
+}
+
+// One candidate per CTA by counting (score_bins_kernel), from groups of 64 units on in the mean: there it is the fastest for
+// every number of candidates (us, counting / the better of the other two: 6 000 units in 90 operators, 600 candidates 60 / 69,
+// 5 000 387 / 421; 700 in 10, 1 500 22.5 / 26.6; 12 001 in 7, 1 000 78 / 145), below, its two steps of a warp per operator
+// outweigh what it saves (6 000 in 150, 500 candidates 73 / 78; 8 000 in 200, 3 000 487 / 438; 3 000 in 300, 5 000 950 / 226).
+constexpr uint32_t BINS_GROUP_MIN = 64;
+constexpr uint32_t BINS_OPS_MAX = 255;        // (a unit's operator is kept in a byte, n_ops where it has none)
+
+// Its threads.  A candidate's latency falls with the threads as long as SMs would idle; with several candidates per SM, CTAs
+// that are large enough to cover the loads and no larger, as fewer warps wait while an operator's warp works (us at 128 / 256 /
+// 512 / 1 024 threads: 700 units in 4 operators, 100 candidates 12.6 / 12.6 / 12.1 / 12.2, 5 000 37 / 41 / 61 / 121;
+// 3 000 in 15, 300 candidates 30 / 21.5 / 17.7 / 22.8, 5 000 121 / 120 / 129 / 188; 6 000 in 4, 100 candidates 22.9 / 18.6 / 14.6
+// / 13.2, 5 000 175 / 141 / 148 / 219).  Where shared memory holds one or two CTAs an SM, or the operators are many, the largest
+// (16 000 in 80, 1 500 candidates 560 / 321 / 218 / 203; 12 000 in 181 741 / 412 / 267 / 254, in 4 179 / 119 / 98 / 108).
+uint32_t bins_threads(uint32_t n, uint32_t n_ops, uint32_t b, uint32_t sms) {
+    if (b <= sms) return n > 3000 ? 1024u : n > 1000 ? 512u : 256u;
+    if (n > 14000 || (n > 9000 && n_ops > 100)) return 1024u;
+    if (n > 4000 || (n > 2000 && b <= 3 * sms)) return 512u;
+    return n > 1000 || b <= 4 * sms ? 256u : 128u;
 }
 
 constexpr int SCORE_MAX_DEVICES = 64;
@@ -978,7 +1272,11 @@ extern "C" int atrex_score_aggregate(const double* d_roofline_s, const uint32_t*
         std::lock_guard<std::mutex> hold(g_score_lock);
         if (g_score_sms[attr.device] == 0) {
             int v = 0;
-            if (cudaFuncSetAttribute(score_warp_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SCORE_SMEM_MAX) != cudaSuccess ||
+            if (cudaFuncSetAttribute(score_bins_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, SCORE_SMEM_MAX) != cudaSuccess ||
+                cudaFuncSetAttribute(score_bins_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, SCORE_SMEM_MAX) != cudaSuccess ||
+                cudaFuncSetAttribute(score_bins_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, SCORE_SMEM_MAX) != cudaSuccess ||
+                cudaFuncSetAttribute(score_bins_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, SCORE_SMEM_MAX) != cudaSuccess ||
+                cudaFuncSetAttribute(score_warp_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SCORE_SMEM_MAX) != cudaSuccess ||
                 cudaFuncSetAttribute(score_warp_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SCORE_SMEM_MAX) != cudaSuccess ||
                 cudaFuncSetAttribute(score_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SCORE_SMEM_MAX) != cudaSuccess ||
                 cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, attr.device) != cudaSuccess) {
@@ -1004,7 +1302,16 @@ extern "C" int atrex_score_aggregate(const double* d_roofline_s, const uint32_t*
         if (k * c > warps * per_sm) warps = k, per_sm = c;
     }
     const uint32_t sms = (uint32_t)n_sms, held = warps * per_sm;
-    if (by_warps(n, n_ops, b, sms, held) && slots + n < SLOT_MASK) {
+    if (n >= BINS_GROUP_MIN * n_ops && n_ops <= BINS_OPS_MAX) {
+        const uint32_t threads = bins_threads(n, n_ops, b, sms), log_bins = log_bins_for(n, n_ops);
+        const size_t smem = BinsLayout(n, n_ops, log_bins, threads).total;
+        auto* kernel = threads == 128 ? score_bins_kernel<128> : threads == 256 ? score_bins_kernel<256> : threads == 512 ? score_bins_kernel<512> : score_bins_kernel<1024>;
+        per_sm = (uint32_t)(SM_SMEM / (smem + 1024 + 16));
+        if (per_sm > (uint32_t)bins_ctas((int)threads)) per_sm = (uint32_t)bins_ctas((int)threads);
+        if (per_sm < 1) per_sm = 1;
+        kernel<<<b < sms * per_sm ? b : sms * per_sm, threads, smem, (cudaStream_t)stream>>>(
+            d_roofline_s, d_unit_op, n, d_t_cand, d_correct, b, d_w, n_ops, log_bins, d_s_agg, d_s_op, errors);
+    } else if (by_warps(n, n_ops, b, sms, held) && slots + n < SLOT_MASK) {
         const uint32_t want = (b + warps - 1) / warps, most = (uint32_t)n_sms * per_sm;
         const size_t warp_smem = wl.warps + (size_t)wl.warp_bytes * warps;
         auto* kernel = pairs ? score_warp_kernel<true> : score_warp_kernel<false>;

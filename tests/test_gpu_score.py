@@ -105,3 +105,36 @@ def test_score_parity_where_the_kernels_change(n_units, n_ops, batch):
     assert got[0].tobytes() == exp[0].tobytes()
     assert got[1].tobytes() == exp[1].tobytes()
     assert np.array_equal(got[2], exp[2])
+
+
+# operators counted by range: sizes around every line of its dispatch, groups that end in the first, the last and a crowded range
+@pytest.mark.parametrize("n_units,n_ops,batch", [
+    (64, 1, 3), (127, 2, 150), (128, 2, 150), (1000, 15, 149), (1001, 15, 149), (1000, 3, 600), (2001, 2, 300), (3000, 40, 20), (3001, 40, 20),
+    (4001, 5, 460), (9001, 101, 150), (14_001, 7, 149), (16_320, 255, 2), (16_384, 256, 2), (16_384, 1, 150)])
+@pytest.mark.parametrize("law", ["even", "uneven", "two values", "far apart", "close"])
+def test_score_parity_by_counting(n_units, n_ops, batch, law):
+    rng = np.random.default_rng(n_units + n_ops + len(law))
+    unit_op = rng.integers(0, n_ops + 1, n_units).astype(np.uint32)       # one operator in n_ops + 1 is out of range
+    if law == "uneven":
+        unit_op[: n_units // 2] = n_ops - 1
+    roof = np.exp(rng.uniform(np.log(1e-6), np.log(1e-1), n_units))
+    batch = min(batch, 3_000_000 // n_units)
+    score = rng.uniform(0.01, 1.02, (batch, n_units))
+    if law == "two values":                                               # the middles lie in different ranges, or among ties
+        score = np.where(rng.random((batch, n_units)) < 0.5, 0.01, 0.9)
+    if law == "far apart":                                                # mostly outside the first cut's range
+        score = np.exp2(rng.uniform(-50, 40, (batch, n_units)))
+    if law == "close":
+        score = 0.3 * (1 + rng.integers(0, 1 << 12, (batch, n_units)) * 2.0 ** -34)
+    t = roof[None, :] / score
+    if law == "far apart":
+        t[:, ::501] *= 2.0 ** -300                                        # outside binary32
+    t[0::7, ::9] = 0.0
+    ok = rng.random((batch, n_units)) < 0.8
+    ok[-1] = unit_op[None, :] == 0                                        # an operator or none with anything correct
+    w = rng.dirichlet(np.ones(n_ops))
+    exp = oracle.score_candidates(roof, unit_op, t, ok, w)
+    got = run_gpu(roof, unit_op, t, ok, w)
+    assert got[0].tobytes() == exp[0].tobytes()
+    assert got[1].tobytes() == exp[1].tobytes()
+    assert np.array_equal(got[2], exp[2])
