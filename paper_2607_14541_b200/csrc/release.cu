@@ -426,10 +426,12 @@ constexpr uint32_t BIN_BITS_MAX = 14, BIN_THREADS = 512;
 constexpr uint32_t SHARE_THREADS = 1024;     // counting and moving: one CTA per SM, for long runs
 constexpr uint32_t CURSORS_MAX = 1u << 14;
 constexpr uint32_t TILE_STEP = 2048;        // a tile is the bins that start in one such window of positions
+constexpr uint32_t TILE_GROUP = 64;         // tiles whose weighted times are summed
 constexpr uint32_t TILE_CAP = 6144;         // ... and has at most this many items
 constexpr uint32_t TILE_LOCAL_BINS = 4096, TILE_THREADS = 512, TILE_HELD = 5, GATHER_LOADS = 6;
 constexpr uint32_t TILE_CLASH_MAX = 24;     // larger local bins are crowded: some are sorted by a warp or the CTA each,
-constexpr uint32_t TILE_CROWDED = 32;       // more of them, or larger ones, send the tile to the comparison network
+constexpr uint32_t TILE_CROWDED = 32;       // more of them send the tile to the comparison network
+constexpr uint32_t TILE_SMALL_CROWD = 64;   // sorted by a warp
 constexpr size_t TILE_SMEM = (size_t)TILE_CAP * 8 + TILE_LOCAL_BINS * 4;    // (what it leaves of two CTAs is L1 for the gather)
 constexpr uint32_t COUNT_SORT_MAX = 8192;   // up to here one kernel ranks every key by counting
 
@@ -463,15 +465,16 @@ struct BinSort {                 // what the kernels share
     BinCtl* ctl;
     BinReport* report;
     const atrex_entry_t* entries;
-    ull* words;                  // [n] raw words: keys (key order), words (ranking)
-    uint32_t* idx;               // [n] (ranking) entry of each word, later the entries' order
-    ull* items;                  // [n] in bin order: leading 32 bits of the word's place in the range, then the entry
+    ull* words;                  // [n] raw words: keys (key order), words (ranking); (ranking) later low words of the ranked weighted times
+    uint32_t* idx;               // [n] (ranking) entry of each word
+    ull* items;                  // [n] in bin order: leading 32 bits of the word's place in the range, then the entry; later the high words
     uint32_t* bins;              // [1 << bits] counts, then each bin's cursor number
     uint32_t* cursors;           // [n_cursors] where the next item of a tile (by_tile) or bin goes
     uint32_t* tile_start;        // [tiles + 1]
     uint32_t n_cursors;
     bool by_tile;                // items of a tile lie in any order, not bin by bin
-    ull* tile_sum;               // [tiles][2]
+    ulonglong2* tile_sum;        // (ranking) [tiles] weighted time
+    ulonglong2* group_sum;       // (ranking) ... of TILE_GROUP tiles
     uint32_t n;                  // upper bound of the item count
     uint32_t bits;
     bool ranking;
@@ -539,7 +542,7 @@ __device__ __forceinline__ T block_reduce(T v, T (*op)(T, T), T* s_part) {   // 
 }
 __device__ __forceinline__ ull max_ull(ull a, ull b) { return a > b ? a : b; }
 
-// 0. the control block and the bins behind it cleared (a kernel in the chain: a memset breaks it, 3 us each side)
+// 0. the control block, the sums of groups of tiles and the bins behind it cleared (a kernel in the chain: a memset breaks it, 3 us each side)
 __global__ void __launch_bounds__(BIN_THREADS) bin_clear_kernel(uint4* at, uint32_t n) {
     grid_dependency_wait();
     const uint32_t i = blockIdx.x * BIN_THREADS + threadIdx.x;
@@ -577,7 +580,9 @@ __global__ void __launch_bounds__(BIN_THREADS) bin_keys_kernel(const BinSort b) 
     }
 }
 
-// 1b. (ranking) the phase's entries: words and indices side by side in any order, word range, exact total
+// 1b. (ranking) the phase's entries: words and indices side by side in any order, word range, exact total.  Bound by the entries' DRAM
+//     reads, 4.4 TB/s (weights asked for once the phase was known: 3.1 M entries 38 us, now 34; 15 M 154, now 130; the next round's lines
+//     prefetched into L2 as well: 40 and 140).
 __global__ void __launch_bounds__(BIN_THREADS) bin_phase_kernel(const BinSort b, uint32_t phase) {
     constexpr uint32_t PER = 4;
     __shared__ ull s_part[32];
@@ -588,10 +593,13 @@ __global__ void __launch_bounds__(BIN_THREADS) bin_phase_kernel(const BinSort b,
     for (uint32_t t0 = blockIdx.x * (BIN_THREADS * PER); t0 < b.n; t0 += gridDim.x * (BIN_THREADS * PER)) {
         bool mine[PER];
         uint32_t place[PER], run = 0;
+        ull lo[PER], hi[PER];
 #pragma unroll
-        for (uint32_t u = 0; u < PER; ++u) {
+        for (uint32_t u = 0; u < PER; ++u) {   // (the weights are asked for with the keys: the lines are the same, mostly)
             const uint32_t i = t0 + u * BIN_THREADS + threadIdx.x;
             mine[u] = i < b.n && (uint32_t)(b.entries[i].key >> 48) == phase;
+            lo[u] = i < b.n ? b.entries[i].wt_lo : 0ull;
+            hi[u] = i < b.n ? b.entries[i].wt_hi : 0ull;
         }
 #pragma unroll
         for (uint32_t u = 0; u < PER; ++u) {
@@ -617,12 +625,12 @@ __global__ void __launch_bounds__(BIN_THREADS) bin_phase_kernel(const BinSort b,
         for (uint32_t u = 0; u < PER; ++u) {
             if (!mine[u]) continue;
             const uint32_t i = t0 + u * BIN_THREADS + threadIdx.x, pos = s_base + s_warp[w] + place[u];
-            const ull lo = b.entries[i].wt_lo, hi = b.entries[i].wt_hi, word = rank_word(lo, hi);
+            const ull word = rank_word(lo[u], hi[u]);
             b.words[pos] = word;
             b.idx[pos] = i;
             top = max_ull(top, word);
             ntop = max_ull(ntop, ~word);
-            add128(sum_lo, sum_hi, lo, hi);
+            add128(sum_lo, sum_hi, lo[u], hi[u]);
         }
         __syncthreads();   // s_warp and s_base are reused
     }
@@ -680,13 +688,26 @@ __global__ void __launch_bounds__(SHARE_THREADS) bin_count_kernel(const BinSort 
 }
 
 // 3. where each bin and each tile starts; a bin that no tile can hold ends the attempt (one CTA)
-__global__ void __launch_bounds__(1024) bin_scan_kernel(const BinSort b) {
+//    (ranking) and the sum that the coverage cut needs: the smallest k with 10^6 * prefix_k >= ppm * T, i.e.
+//    prefix_k >= ceil(ppm * T / 10^6)
+__global__ void __launch_bounds__(1024) bin_scan_kernel(const BinSort b, uint32_t coverage_ppm) {
     __shared__ uint32_t s_warp[32];
     __shared__ uint32_t s_max;
     grid_dependency_wait();
     const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5, m = item_count(b);
     const uint32_t n_bins = 1u << b.bits, per = (n_bins + 1023) / 1024, first = threadIdx.x * per;
     if (threadIdx.x == 0) s_max = 0;
+    if (b.ranking && threadIdx.x == 1023) {       // (while the others wait for the bins)
+        BinReport* r = b.report;
+        BinCtl* ctl = b.ctl;
+        r->counter = ctl->counter;
+        r->total_lo = ctl->total_lo;
+        r->total_hi = ctl->total_hi;
+        const unsigned __int128 total = ((unsigned __int128)ctl->total_hi << 64) | ctl->total_lo;
+        const unsigned __int128 need = ((unsigned __int128)coverage_ppm * total + 999999u) / 1000000u;   // (not asked for, where that wraps)
+        ctl->need_lo = (ull)need;
+        ctl->need_hi = (ull)(need >> 64);
+    }
     __syncthreads();
     uint32_t c[1u << (BIN_BITS_MAX - 10)];
     uint32_t sum = 0, most = 0;
@@ -748,8 +769,10 @@ __global__ void __launch_bounds__(1024) bin_scan_kernel(const BinSort b) {
         if (b.by_tile) b.cursors[0] = 0;
         for (uint32_t j = m / TILE_STEP + 1; j <= n_tiles; ++j) b.tile_start[j] = m;
         const bool overflow = s_max + TILE_STEP > TILE_CAP;
-        b.ctl->overflow = overflow;
         b.report->overflow = overflow;
+        const bool too_large = b.ranking && (b.ctl->total_hi >> 44) != 0;      // T * 10^6 must fit 128 bits
+        b.report->too_large = too_large;
+        b.ctl->overflow = overflow || too_large;
     }
 }
 
@@ -828,31 +851,122 @@ __device__ __forceinline__ void bitonic(uint32_t n, Less less, Swap swap) {
     }
 }
 
-// A crowded local bin of n items in order: the network over copies of their entries' weights and
-// keys in shared memory (whole CTA).  (3.2 M entries of two phases, some 800 of each at the clamp of their weights:
-// the network over the whole tile, reading entries at every comparison, took that one tile 110 us, longer than
-// all others together.)
-__device__ __noinline__ void sort_crowded_bin(const atrex_entry_t* entries, bool ranking, ull* s_item, uint32_t n, ull* s_key, ull* s_lo, ull* s_hi) {
-    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) {
-        const atrex_entry_t* e = entries + (uint32_t)s_item[i];
-        s_key[i] = e->key;
-        s_lo[i] = ranking ? e->wt_lo : 0ull;
-        s_hi[i] = ranking ? e->wt_hi : 0ull;
+// A crowded local bin, the n items at s_item[b0], in order (whole CTA).  They are cut into bins once more, between the
+// smallest and the largest of what their leading bits left out -- the weighted times' 57 bits, or the keys where those are all
+// alike --, bins that are still crowded again, and so on.  Items that nothing tells apart but their entries' order, and more than CROWD_MAX, go
+// through the network, which reads entries at every comparison.  `s_bins`: CROWD_BINS + CROWD_MAX / 2 words.  (1.6 M rows, 1 600
+// of them at the clamp of their weights: the tile that held those went through a network as a whole, kernel 90 us, now 75 with the weighted
+// times written for the shares; 7.5 M rows, 7 500 of them: 572, now 367)
+constexpr uint32_t CROWD_BINS = 2048, CROWD_MAX = 4096, CROWD_CLASH_MAX = 64, CROWD_SEGMENTS = 32;
+__device__ __noinline__ void sort_crowded_bin(const atrex_entry_t* entries, bool ranking, ull* s_item, uint32_t b0, uint32_t n, uint32_t* s_bins) {
+    __shared__ ull s_range[2];
+    __shared__ uint32_t s_warp[32], s_segments, s_from[CROWD_SEGMENTS], s_size[CROWD_SEGMENTS];
+    uint16_t* s_list = reinterpret_cast<uint16_t*>(s_bins + CROWD_BINS);
+    const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
+    auto by_network = [&](uint32_t from, uint32_t size) {
+        bitonic(size, [&](uint32_t a, uint32_t b) { return item_less(entries, ranking, s_item[from + a], s_item[from + b]); },
+                [&](uint32_t a, uint32_t b) { const ull x = s_item[from + a]; s_item[from + a] = s_item[from + b]; s_item[from + b] = x; });
+    };
+    if (threadIdx.x == 0) {
+        s_segments = 1;
+        s_from[0] = b0;
+        s_size[0] = n;
     }
     __syncthreads();
-    bitonic(n, [&](uint32_t a, uint32_t b) {
-        const ull x = s_item[a], y = s_item[b];
-        if ((x ^ y) >> 32) return x < y;
-        if (s_hi[a] != s_hi[b]) return s_hi[a] > s_hi[b];
-        if (s_lo[a] != s_lo[b]) return s_lo[a] > s_lo[b];
-        if (s_key[a] != s_key[b]) return s_key[a] < s_key[b];
-        return x < y;           // equal keys keep their input order
-    }, [&](uint32_t a, uint32_t b) {
-        ull x = s_item[a]; s_item[a] = s_item[b]; s_item[b] = x;
-        x = s_key[a]; s_key[a] = s_key[b]; s_key[b] = x;
-        x = s_lo[a]; s_lo[a] = s_lo[b]; s_lo[b] = x;
-        x = s_hi[a]; s_hi[a] = s_hi[b]; s_hi[b] = x;
-    });
+    for (uint32_t k = 0; k < min(s_segments, CROWD_SEGMENTS); ++k) {       // (the same for every thread)
+        const uint32_t from = s_from[k], size = s_size[k];
+        ull* item = s_item + from;
+        const atrex_entry_t* one = entries + (uint32_t)item[0];
+        bool differ = false;
+        for (uint32_t i = threadIdx.x; ranking && i < size; i += TILE_THREADS) {
+            const atrex_entry_t* e = entries + (uint32_t)item[i];
+            differ |= e->wt_lo != one->wt_lo || e->wt_hi != one->wt_hi;
+        }
+        const bool by_key = __syncthreads_or(differ) == 0;
+        auto word = [&](uint32_t i) {
+            const atrex_entry_t* e = entries + (uint32_t)item[i];
+            return by_key ? e->key : rank_word(e->wt_lo, e->wt_hi);
+        };
+        if (threadIdx.x < 2) s_range[threadIdx.x] = 0;
+        for (uint32_t i = threadIdx.x; i < CROWD_BINS; i += TILE_THREADS) s_bins[i] = 0;
+        __syncthreads();
+        ull top = 0, ntop = 0;
+        for (uint32_t i = threadIdx.x; i < size; i += TILE_THREADS) {
+            const ull x = word(i);
+            top = max_ull(top, x);
+            ntop = max_ull(ntop, ~x);
+        }
+#pragma unroll
+        for (int d = 16; d; d >>= 1) {
+            top = max_ull(top, __shfl_xor_sync(FULL, top, d));
+            ntop = max_ull(ntop, __shfl_xor_sync(FULL, ntop, d));
+        }
+        if (lane == 0) {
+            atomicMax(&s_range[0], top);
+            atomicMax(&s_range[1], ntop);
+        }
+        __syncthreads();
+        const ull low = ~s_range[1];
+        if (s_range[0] == low || size > CROWD_MAX) {
+            by_network(from, size);
+            continue;
+        }
+        const int len = 64 - __clzll((long long)(s_range[0] - low)), shift = len > 11 ? len - 11 : 0;
+        static_assert(CROWD_BINS == 1u << 11, "bits of a bin");
+        auto bin_of = [&](uint32_t i) { return (uint32_t)((word(i) - low) >> shift); };
+        for (uint32_t i = threadIdx.x; i < size; i += TILE_THREADS) atomicAdd(&s_bins[bin_of(i)], 1u);
+        __syncthreads();
+        constexpr uint32_t PER = CROWD_BINS / TILE_THREADS;
+        uint32_t c[PER], sum = 0;
+#pragma unroll
+        for (uint32_t u = 0; u < PER; ++u) sum += c[u] = s_bins[threadIdx.x * PER + u];
+        uint32_t incl = sum;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t o = __shfl_up_sync(FULL, incl, d);
+            if (lane >= (uint32_t)d) incl += o;
+        }
+        if (lane == 31) s_warp[w] = incl;
+        __syncthreads();
+        uint32_t at = incl - sum;
+        for (uint32_t j = 0; j < w; ++j) at += s_warp[j];
+#pragma unroll
+        for (uint32_t u = 0; u < PER; ++u) {
+            s_bins[threadIdx.x * PER + u] = at;
+            if (c[u] > CROWD_CLASH_MAX) {
+                const uint32_t next = atomicAdd(&s_segments, 1u);
+                if (next < CROWD_SEGMENTS) {
+                    s_from[next] = from + at;
+                    s_size[next] = c[u];
+                }
+            }
+            at += c[u];
+        }
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < size; i += TILE_THREADS) s_list[atomicAdd(&s_bins[bin_of(i)], 1u)] = (uint16_t)i;
+        __syncthreads();
+        // a bin's counter now stands at its end; every item's place in its bin, and all items there (they are held for a moment)
+        ull held[CROWD_MAX / TILE_THREADS];
+        uint32_t place[CROWD_MAX / TILE_THREADS];
+#pragma unroll
+        for (uint32_t u = 0; u < CROWD_MAX / TILE_THREADS; ++u) {
+            const uint32_t at = u * TILE_THREADS + threadIdx.x;
+            if (at >= size) continue;
+            const uint32_t i = s_list[at], d = bin_of(i), begin = d ? s_bins[d - 1] : 0u, end = s_bins[d];
+            held[u] = item[i];
+            place[u] = at;                               // (in a bin that is still crowded: for now)
+            if (end - begin <= CROWD_CLASH_MAX) {
+                place[u] = begin;
+                for (uint32_t j = begin; j < end; ++j) place[u] += j != at && item_less(entries, ranking, item[s_list[j]], held[u]) ? 1u : 0u;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (uint32_t u = 0; u < CROWD_MAX / TILE_THREADS; ++u)
+            if (u * TILE_THREADS + threadIdx.x < size) item[place[u]] = held[u];
+        __syncthreads();
+    }
+    if (s_segments > CROWD_SEGMENTS) by_network(b0, n);
 }
 
 // A crowded local bin of up to 64 items by one warp: every lane counts the items before its own two.
@@ -894,13 +1008,14 @@ __device__ __forceinline__ void sort_small_bin(const atrex_entry_t* entries, boo
 
 // Sorts n <= TILE_CAP items whose leading bits lie in [low, high] into s_item.  `each(f)` calls f with each of
 // this thread's items (twice).  Each item goes to one of 4 096 local bins of equal width -- less than one item per bin, so that
-// a thread puts a bin in order by insertion; a few crowded local bins (hundreds of equal weights, say) go
-// through a bitonic network each, many of them send the whole tile through a bitonic network, with absent items behind the last one.
+// a thread puts a bin in order by insertion; a few crowded local bins (hundreds of equal weights, say) are
+// sorted on their own, many of them send the whole tile through a bitonic network, with absent items behind the last one.
+// (Every item's place counted by a thread of its own instead: 3.1 M entries 107.5 -> 111 us.)
 template <typename Each>
 __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ranking, uint32_t n, uint32_t low, uint32_t high, Each each, ull* s_item,
                                           uint32_t* s_local) {
     __shared__ uint32_t s_warp[32];
-    __shared__ uint32_t s_crowded, s_bin[TILE_CROWDED];
+    __shared__ uint32_t s_crowded, s_bin[TILE_CROWDED], s_begin[TILE_CROWDED], s_size[TILE_CROWDED];
     const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
     const int len = 32 - __clz((int)(high - low));
     const int shift = len > 12 ? len - 12 : 0;
@@ -948,18 +1063,14 @@ __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ran
     __syncthreads();
     // (a bin's cursor now stands at its end, its predecessor's at its start)
     const uint32_t crowded = s_crowded;
-    const uint32_t room = (TILE_CAP - n) / 3;    // (behind the items there is room for so many copies)
-    bool by_bins = crowded <= TILE_CROWDED;
-    for (uint32_t k = 0; by_bins && k < crowded; ++k) by_bins = s_local[s_bin[k]] - (s_bin[k] ? s_local[s_bin[k] - 1] : 0u) <= room;
-    if (by_bins) {
+    if (crowded <= TILE_CROWDED) {
         for (uint32_t k = w; k < crowded; k += n_warps) {
-            const uint32_t d = s_bin[k], b0 = d ? s_local[d - 1] : 0u;
-            if (s_local[d] - b0 <= 64) sort_small_bin(entries, ranking, s_item + b0, s_local[d] - b0);
-        }
-        for (uint32_t k = 0; k < crowded; ++k) {     // (the same for every thread)
-            const uint32_t d = s_bin[k], b0 = d ? s_local[d - 1] : 0u;
-            if (s_local[d] - b0 <= 64) continue;
-            sort_crowded_bin(entries, ranking, s_item + b0, s_local[d] - b0, s_item + n, s_item + n + room, s_item + n + 2 * room);
+            const uint32_t d = s_bin[k], b0 = d ? s_local[d - 1] : 0u, size = s_local[d] - b0;
+            if (size <= TILE_SMALL_CROWD) sort_small_bin(entries, ranking, s_item + b0, size);
+            if (lane == 0) {
+                s_begin[k] = b0;
+                s_size[k] = size;
+            }
         }
         for (uint32_t d = threadIdx.x; d < TILE_LOCAL_BINS; d += blockDim.x) {
             const uint32_t b0 = d ? s_local[d - 1] : 0u, b1 = s_local[d];
@@ -974,6 +1085,9 @@ __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ran
                 s_item[j] = item;
             }
         }
+        __syncthreads();
+        for (uint32_t k = 0; k < crowded; ++k)           // (the same for every thread; the local bins are not needed any more)
+            if (s_size[k] > TILE_SMALL_CROWD) sort_crowded_bin(entries, ranking, s_item, s_begin[k], s_size[k], s_local);
     } else {
         bitonic(n, [&](uint32_t a, uint32_t b) { return item_less(entries, ranking, s_item[a], s_item[b]); },
                 [&](uint32_t a, uint32_t b) { const ull x = s_item[a]; s_item[a] = s_item[b]; s_item[b] = x; });
@@ -984,9 +1098,10 @@ __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ran
 // Entries of the sorted items to out[first .. first + n), as far as out_cap: three lanes to an entry, so that
 // the stores are contiguous and an entry's read is three 16-byte pieces of one or two lines (8-byte pieces
 // where a caller's buffer is only 8-byte aligned).
-// (`sum`: 128-bit sum of the weighted times this thread copied)
+// (each(row, lo, hi): the weighted time of a row)
+template <typename Weight>
 __device__ __forceinline__ void gather_tile(const atrex_entry_t* entries, const ull* s_item, uint32_t n, atrex_entry_t* out, uint32_t first,
-                                            uint32_t out_cap, ulonglong2& sum) {
+                                            uint32_t out_cap, Weight each) {
     const uint32_t rows = first < out_cap ? min(n, out_cap - first) : 0u;
     if ((((uintptr_t)entries | (uintptr_t)out) & 15u) == 0) {
         const ulonglong2* src = reinterpret_cast<const ulonglong2*>(entries);
@@ -1004,17 +1119,17 @@ __device__ __forceinline__ void gather_tile(const atrex_entry_t* entries, const 
                 const uint32_t x = i + u * blockDim.x;
                 if (x >= rows * 3) continue;
                 __stcs(dst + x, v[u]);
-                if (x % 3 == 1) add128(sum.x, sum.y, v[u].x, v[u].y);
+                if (x % 3 == 1) each(x / 3, v[u].x, v[u].y);
             }
         }
     } else {
         const ull* src = reinterpret_cast<const ull*>(entries);
         ull* dst = reinterpret_cast<ull*>(out + first);
         for (uint32_t i = threadIdx.x; i < rows * 6; i += blockDim.x) {
-            const ull v = src[(size_t)(uint32_t)s_item[i / 6] * 6 + i % 6];
+            const size_t at = (size_t)(uint32_t)s_item[i / 6] * 6 + i % 6;
+            const ull v = src[at];
             dst[i] = v;
-            if (i % 6 == 2) add128(sum.x, sum.y, v, 0ull);
-            if (i % 6 == 3) sum.y += v;
+            if (i % 6 == 2) each(i / 6, v, src[at + 1]);
         }
     }
 }
@@ -1034,7 +1149,7 @@ __global__ void __launch_bounds__(TILE_THREADS) bin_tile_kernel(const BinSort b,
     const uint32_t first = overflow ? 0u : b.tile_start[tile], n = overflow ? 0u : b.tile_start[tile + 1] - first;
     if (n == 0) {
         if (!b.ranking) finish_call(b.report, b.slot);
-        else if (!overflow && threadIdx.x < 2) b.tile_sum[2 * tile + threadIdx.x] = 0;
+        else if (!overflow && threadIdx.x == 0) b.tile_sum[tile] = make_ulonglong2(0, 0);
         return;
     }
     // the items are read once, all of a thread's at a time (a tile rarely has more than TILE_HELD per thread)
@@ -1069,17 +1184,23 @@ __global__ void __launch_bounds__(TILE_THREADS) bin_tile_kernel(const BinSort b,
     grid_dependents_launch();
     if (threadIdx.x < 2) s_sum[threadIdx.x] = 0;
     ulonglong2 sum = make_ulonglong2(0, 0);
-    gather_tile(b.entries, s_item, n, out, first, out_cap, sum);
     if (!b.ranking) {
+        gather_tile(b.entries, s_item, n, out, first, out_cap, [](uint32_t, ull, ull) {});
         finish_call(b.report, b.slot);
         return;
     }
-    for (uint32_t i = threadIdx.x; i < n; i += TILE_THREADS) {   // rows that are not wanted: their order is kept for the shares
+    // (the shares read a row's weighted time where the words were and where the items were, which this CTA alone read: the ranked
+    // rows themselves would have to come from memory once more)
+    auto weight = [&](uint32_t row, ull lo, ull hi) {
+        add128(sum.x, sum.y, lo, hi);
+        b.words[first + row] = lo;
+        b.items[first + row] = hi;
+    };
+    gather_tile(b.entries, s_item, n, out, first, out_cap, weight);
+    for (uint32_t i = threadIdx.x; i < n; i += TILE_THREADS) {   // rows that are not wanted
         if (first + i < out_cap) continue;
-        const uint32_t at = (uint32_t)s_item[i];
-        const atrex_entry_t* e = b.entries + at;
-        add128(sum.x, sum.y, e->wt_lo, e->wt_hi);
-        b.idx[first + i] = at;
+        const atrex_entry_t* e = b.entries + (uint32_t)s_item[i];
+        weight(i, e->wt_lo, e->wt_hi);
     }
     __syncthreads();   // s_sum is cleared
 #pragma unroll
@@ -1089,7 +1210,106 @@ __global__ void __launch_bounds__(TILE_THREADS) bin_tile_kernel(const BinSort b,
     }
     if ((threadIdx.x & 31) == 0 && (sum.x | sum.y)) atomic_add128(&s_sum[0], &s_sum[1], sum.x, sum.y);
     __syncthreads();
-    if (threadIdx.x < 2) b.tile_sum[2 * tile + threadIdx.x] = s_sum[threadIdx.x];
+    if (threadIdx.x == 0) {
+        b.tile_sum[tile] = make_ulonglong2(s_sum[0], s_sum[1]);
+        ull* group = reinterpret_cast<ull*>(b.group_sum + tile / TILE_GROUP);
+        atomic_add128(group, group + 1, s_sum[0], s_sum[1]);
+    }
+}
+
+// 6. (ranking) running share of each row, and the row at the coverage cut.  A CTA takes a run of tiles and adds up for itself what lies
+//    before it, group by group and then tile by tile (a scan of the tiles in a launch of its own took 11 us).  A thread takes four rows
+//    one behind the other, so that one scan over the warp serves 128 of them; the shares go out through shared memory, side by side.
+//    Bound by latency and instructions (a row's share is sixty): with the scan of the tiles, 1.6 M rows 46 us while a lane took
+//    a row, every 1 024 rows three barriers, and the ranked rows were read back; now 26 behind the tiles.  7.5 M rows 155, now 88.
+constexpr uint32_t CUM_THREADS = 512, CUM_ROWS = 4, CUM_CTAS = 2;
+__global__ void __launch_bounds__(CUM_THREADS, CUM_CTAS) bin_share_kernel(const BinSort b, double* cum, uint32_t out_cap) {
+    __shared__ ulonglong2 s_part[CUM_THREADS / 32];
+    __shared__ double s_cum[CUM_THREADS * CUM_ROWS];
+    grid_dependency_wait();
+    const ull total_lo = b.ctl->total_lo, total_hi = b.ctl->total_hi, need_lo = b.ctl->need_lo, need_hi = b.ctl->need_hi, overflow = b.ctl->overflow;
+    const uint32_t n_tiles = (item_count(b) + TILE_STEP - 1) / TILE_STEP, run = (n_tiles + gridDim.x - 1) / gridDim.x;
+    const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5, tile = min(n_tiles, blockIdx.x * run), group = tile / TILE_GROUP;
+    if (overflow) {
+        finish_call(b.report, b.slot);
+        return;
+    }
+    const uint32_t first = b.tile_start[tile], end = b.tile_start[min(n_tiles, tile + run)];
+    const double total = u128_to_f64_rn(total_hi, total_lo);
+    // sums of the warps (in each one's last lane): of those before this one, and of all
+    auto all_warps = [&](ull lo, ull hi, ull& before_lo, ull& before_hi, ull& all_lo, ull& all_hi) {
+        if (lane == 31) s_part[w] = make_ulonglong2(lo, hi);
+        __syncthreads();
+        const ulonglong2 v = lane < CUM_THREADS / 32 ? s_part[lane] : make_ulonglong2(0, 0);
+        before_lo = lane < w ? v.x : 0ull, before_hi = lane < w ? v.y : 0ull, all_lo = v.x, all_hi = v.y;
+#pragma unroll
+        for (int d = 16; d; d >>= 1) {
+            const ull olo = __shfl_xor_sync(FULL, before_lo, d), ohi = __shfl_xor_sync(FULL, before_hi, d);
+            add128(before_lo, before_hi, olo, ohi);
+            const ull alo = __shfl_xor_sync(FULL, all_lo, d), ahi = __shfl_xor_sync(FULL, all_hi, d);
+            add128(all_lo, all_hi, alo, ahi);
+        }
+    };
+    ull run_lo = 0, run_hi = 0;
+    if (first < end) {
+        ull lo = 0, hi = 0, unused_lo, unused_hi;
+        for (uint32_t g = threadIdx.x; g < group; g += CUM_THREADS) add128(lo, hi, b.group_sum[g].x, b.group_sum[g].y);
+        for (uint32_t t = group * TILE_GROUP + threadIdx.x; t < tile; t += CUM_THREADS) add128(lo, hi, b.tile_sum[t].x, b.tile_sum[t].y);
+#pragma unroll
+        for (int d = 16; d; d >>= 1) {
+            const ull olo = __shfl_xor_sync(FULL, lo, d), ohi = __shfl_xor_sync(FULL, hi, d);
+            add128(lo, hi, olo, ohi);
+        }
+        all_warps(lo, hi, unused_lo, unused_hi, run_lo, run_hi);
+        __syncthreads();
+    }
+    for (uint32_t base = first; base < end; base += CUM_ROWS * CUM_THREADS) {
+        const uint32_t r0 = base + threadIdx.x * CUM_ROWS;
+        ull lo[CUM_ROWS], hi[CUM_ROWS];
+#pragma unroll
+        for (uint32_t u = 0; u < CUM_ROWS; ++u) {
+            lo[u] = hi[u] = 0;
+            if (r0 + u < end) {
+                lo[u] = b.words[r0 + u];
+                hi[u] = b.items[r0 + u];
+            }
+        }
+        ull own_lo = 0, own_hi = 0;
+#pragma unroll
+        for (uint32_t u = 0; u < CUM_ROWS; ++u) add128(own_lo, own_hi, lo[u], hi[u]);
+        ull at_lo = own_lo, at_hi = own_hi;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const ull olo = __shfl_up_sync(FULL, at_lo, d), ohi = __shfl_up_sync(FULL, at_hi, d);
+            if (lane >= (uint32_t)d) add128(at_lo, at_hi, olo, ohi);
+        }
+        ull before_lo, before_hi, all_lo, all_hi;
+        all_warps(at_lo, at_hi, before_lo, before_hi, all_lo, all_hi);
+        add128(at_lo, at_hi, before_lo, before_hi);
+        add128(at_lo, at_hi, run_lo, run_hi);                    // up to and with this thread's rows
+        const bool reaches = (need_lo | need_hi) && !less128(at_lo, at_hi, need_lo, need_hi);
+        at_hi -= own_hi + (at_lo < own_lo ? 1ull : 0ull);        // up to them
+        at_lo -= own_lo;
+        const bool cut_here = reaches && less128(at_lo, at_hi, need_lo, need_hi);
+        add128(run_lo, run_hi, all_lo, all_hi);
+#pragma unroll
+        for (uint32_t u = 0; u < CUM_ROWS; ++u) {
+            const ull ex_lo = at_lo, ex_hi = at_hi;
+            add128(at_lo, at_hi, lo[u], hi[u]);                  // inclusive prefix of the whole list
+            if (cut_here && r0 + u < end && less128(ex_lo, ex_hi, need_lo, need_hi) && !less128(at_lo, at_hi, need_lo, need_hi)) {
+                b.report->n_keep = (ull)r0 + u + 1;
+                b.report->covered_lo = at_lo;
+                b.report->covered_hi = at_hi;
+                __threadfence_system();
+            }
+            s_cum[threadIdx.x * CUM_ROWS + u] = (total_lo | total_hi) ? __ddiv_rn(u128_to_f64_rn(at_hi, at_lo), total) : 0.0;
+        }
+        __syncthreads();                                         // (s_part may be written again, too)
+        const uint32_t rows = min(end, out_cap) > base ? min(min(end, out_cap) - base, CUM_ROWS * CUM_THREADS) : 0u;
+        for (uint32_t i = threadIdx.x; i < rows; i += CUM_THREADS) cum[base + i] = s_cum[i];
+        __syncthreads();
+    }
+    finish_call(b.report, b.slot);
 }
 
 // Key order of up to COUNT_SORT_MAX entries in one kernel: an entry's place is the number of keys before its own.
@@ -1154,93 +1374,6 @@ __global__ void __launch_bounds__(COUNT_THREADS) count_sort_kernel(const atrex_e
     ull* dst = reinterpret_cast<ull*>(out);
     for (uint32_t x = threadIdx.x; x < min(32 * U, n - base) * 6; x += COUNT_THREADS) dst[(size_t)s_place[x / 6] * 6 + x % 6] = src[x];
     finish_call(report, slot);
-}
-
-// 6. (ranking) exclusive scan of the tiles' weighted times, and the sum the coverage cut needs: the smallest
-//    k with 10^6 * prefix_k >= ppm * T, i.e. prefix_k >= ceil(ppm * T / 10^6) (one CTA)
-__global__ void __launch_bounds__(SCAN_BLOCK) bin_tile_scan_kernel(const BinSort b, uint32_t coverage_ppm) {
-    __shared__ ull warp_tot[32][2];
-    grid_dependency_wait();
-    if (threadIdx.x == 0) {
-        BinReport* r = b.report;
-        BinCtl* c = b.ctl;
-        r->counter = c->counter;
-        r->total_lo = c->total_lo;
-        r->total_hi = c->total_hi;
-        r->too_large = (c->total_hi >> 44) != 0;           // T * 10^6 must fit 128 bits
-        r->n_keep = r->covered_lo = r->covered_hi = 0;
-        if ((c->total_hi >> 44) != 0) {
-            c->overflow = 1;
-        } else {
-            const unsigned __int128 total = ((unsigned __int128)c->total_hi << 64) | c->total_lo;
-            const unsigned __int128 need = ((unsigned __int128)coverage_ppm * total + 999999u) / 1000000u;
-            c->need_lo = (ull)need;
-            c->need_hi = (ull)(need >> 64);
-        }
-    }
-    __syncthreads();
-    if (b.ctl->overflow) return;
-    const uint32_t n_tiles = (item_count(b) + TILE_STEP - 1) / TILE_STEP;
-    ull run_lo = 0, run_hi = 0;
-    for (uint32_t base = 0; base < n_tiles; base += SCAN_BLOCK) {
-        const uint32_t t = base + threadIdx.x;
-        ull lo = 0, hi = 0;
-        if (t < n_tiles) {
-            lo = b.tile_sum[2 * t];
-            hi = b.tile_sum[2 * t + 1];
-        }
-        const ull own_lo = lo, own_hi = hi;
-        ull blo, bhi;
-        block_scan128(lo, hi, warp_tot, blo, bhi);
-        if (t < n_tiles) {
-            ull elo = lo - own_lo, ehi = hi - own_hi - (lo < own_lo ? 1ull : 0ull);   // exclusive
-            add128(elo, ehi, run_lo, run_hi);
-            b.tile_sum[2 * t] = elo;
-            b.tile_sum[2 * t + 1] = ehi;
-        }
-        add128(run_lo, run_hi, blo, bhi);
-        __syncthreads();  // warp_tot is reused by the next round
-    }
-}
-
-// 7. (ranking) running share of each row, and the row at the coverage cut
-__global__ void __launch_bounds__(SCAN_BLOCK) bin_share_kernel(const BinSort b, const atrex_entry_t* ranked, double* cum, uint32_t out_cap) {
-    __shared__ ull warp_tot[32][2];
-    grid_dependency_wait();
-    if (b.ctl->overflow) {
-        finish_call(b.report, b.slot);
-        return;
-    }
-    const uint32_t first = b.tile_start[blockIdx.x], end = b.tile_start[blockIdx.x + 1];
-    const ull total_lo = b.ctl->total_lo, total_hi = b.ctl->total_hi, need_lo = b.ctl->need_lo, need_hi = b.ctl->need_hi;
-    const double total = u128_to_f64_rn(total_hi, total_lo);
-    ull run_lo = b.tile_sum[2 * blockIdx.x], run_hi = b.tile_sum[2 * blockIdx.x + 1];
-    for (uint32_t base = first; base < end; base += SCAN_BLOCK) {
-        const uint32_t r = base + threadIdx.x;
-        ull lo = 0, hi = 0;
-        if (r < end) {
-            const atrex_entry_t* e = r < out_cap ? ranked + r : b.entries + b.idx[r];
-            lo = e->wt_lo;
-            hi = e->wt_hi;
-        }
-        const ull own_lo = lo, own_hi = hi;
-        ull blo, bhi;
-        block_scan128(lo, hi, warp_tot, blo, bhi);
-        if (r < end) {
-            add128(lo, hi, run_lo, run_hi);   // inclusive prefix of the whole list
-            const ull ex_lo = lo - own_lo, ex_hi = hi - own_hi - (lo < own_lo ? 1ull : 0ull);
-            if ((need_lo | need_hi) && less128(ex_lo, ex_hi, need_lo, need_hi) && !less128(lo, hi, need_lo, need_hi)) {
-                b.report->n_keep = (ull)r + 1;
-                b.report->covered_lo = lo;
-                b.report->covered_hi = hi;
-                __threadfence_system();
-            }
-            if (r < out_cap) cum[r] = (total_lo | total_hi) ? __ddiv_rn(u128_to_f64_rn(hi, lo), total) : 0.0;
-        }
-        add128(run_lo, run_hi, blo, bhi);
-        __syncthreads();  // warp_tot is reused by the next round
-    }
-    finish_call(b.report, b.slot);
 }
 
 // ---- host side
@@ -1343,6 +1476,8 @@ int sort_by_word(const Scratch& sc, int cur, uint32_t m, ull differing_bits, cud
     return cur;
 }
 
+inline uint64_t group_bytes(uint64_t tiles, bool ranking) { return ranking ? (tiles + TILE_GROUP - 1) / TILE_GROUP * 16 : 0; }
+
 // The scratch as the binned sort uses it.
 BinSort carve_bins(void* base, const atrex_entry_t* entries, uint64_t n, bool ranking, const ReportSlot& slot) {
     unsigned char* p = (unsigned char*)base;
@@ -1358,12 +1493,13 @@ BinSort carve_bins(void* base, const atrex_entry_t* entries, uint64_t n, bool ra
     b.bits = 4;
     while (b.bits < BIN_BITS_MAX && ((b.bits < 12 ? 256ull : 1024ull) << b.bits) < n) ++b.bits;
     p += sizeof(BinCtl);
+    b.group_sum = (ulonglong2*)p; p += group_bytes(tiles, ranking);
     b.by_tile = tiles <= CURSORS_MAX;
     b.n_cursors = b.by_tile ? (uint32_t)tiles : 1u << b.bits;
     b.turns = b.n_cursors >= 2048 ? 2 : 1;
     b.bins = (uint32_t*)p;       p += 4ull << b.bits;
     b.cursors = (uint32_t*)p;    p += 4ull * ((b.n_cursors + 3) & ~3u);
-    b.tile_sum = (ull*)p;        p += tiles * 16;
+    b.tile_sum = (ulonglong2*)p; p += tiles * 16;
     b.tile_start = (uint32_t*)p; p += (tiles + 1) * 4;
     p = (unsigned char*)base + align256(p - (unsigned char*)base);
     b.words = (ull*)p;           p += align256(n * 8);
@@ -1372,20 +1508,20 @@ BinSort carve_bins(void* base, const atrex_entry_t* entries, uint64_t n, bool ra
     return b;
 }
 // (what it needs beyond the pairs is less than the radix sort's digit counts, as long as there are a few tiles)
-static_assert(sizeof(BinCtl) + (4u << 5) + 4u * 4u + 16u * 3u + 4u * 4u + 256u <= sizeof(ReleaseCtl) + 1024u + 1024u + 256u, "smallest case");
+static_assert(sizeof(BinCtl) + 16u + (4u << 5) + 4u * 4u + 16u * 3u + 4u * 4u + 256u <= sizeof(ReleaseCtl) + 1024u + 1024u + 256u, "smallest case");
 
 cudaError_t launch_clear(const BinSort& b, cudaStream_t s) {
-    const uint32_t n = (uint32_t)((sizeof(BinCtl) + (4ull << b.bits)) / 16);
+    const uint32_t n = (uint32_t)((sizeof(BinCtl) + group_bytes((b.n + TILE_STEP - 1) / TILE_STEP, b.ranking) + (4ull << b.bits)) / 16);
     return launch_chained(bin_clear_kernel, (n + BIN_THREADS - 1) / BIN_THREADS, BIN_THREADS, 0, s, (uint4*)b.ctl, n);
 }
 
 // Steps 2 to 5, behind the kernel that made the words.
-cudaError_t launch_bins(const BinSort& b, atrex_entry_t* out, uint64_t out_cap, int n_sms, cudaStream_t s) {
+cudaError_t launch_bins(const BinSort& b, uint32_t coverage_ppm, atrex_entry_t* out, uint64_t out_cap, int n_sms, cudaStream_t s) {
     const uint32_t bytes = 4u << b.bits, tiles = (b.n + TILE_STEP - 1) / TILE_STEP;
     uint32_t grid = (b.n + 4095) / 4096;
     if (grid > (uint32_t)n_sms) grid = (uint32_t)n_sms;
     cudaError_t e = launch_chained(bin_count_kernel, grid, SHARE_THREADS, bytes, s, b);
-    if (e == cudaSuccess) e = launch_chained(bin_scan_kernel, 1, 1024, 0, s, b);
+    if (e == cudaSuccess) e = launch_chained(bin_scan_kernel, 1, 1024, 0, s, b, coverage_ppm);
     if (e == cudaSuccess) e = launch_chained(bin_scatter_kernel, grid, SHARE_THREADS, b.n_cursors * 4 + (2u << b.bits), s, b);
     if (e == cudaSuccess) e = launch_chained(bin_tile_kernel, tiles, TILE_THREADS, TILE_SMEM, s, b, out, (uint32_t)(out_cap < b.n ? out_cap : b.n));
     return e;
@@ -1438,7 +1574,7 @@ extern "C" int atrex_entries_sort_by_key(const atrex_entry_t* d_entries, uint64_
         if (launch_clear(b, s) != cudaSuccess) return ATREX_ERR_CUDA;
         const uint32_t want = (m + 4 * BIN_THREADS - 1) / (4 * BIN_THREADS), most = 4u * (uint32_t)n_sms;
         if (launch_chained(bin_keys_kernel, want < most ? want : most, BIN_THREADS, 0, s, b) != cudaSuccess ||
-            launch_bins(b, d_out, n, n_sms, s) != cudaSuccess || report.wait() != cudaSuccess)
+            launch_bins(b, 0, d_out, n, n_sms, s) != cudaSuccess || report.wait() != cudaSuccess)
             return ATREX_ERR_CUDA;
         if (!((volatile BinReport*)report.get())->overflow) return ATREX_OK;
     }
@@ -1485,9 +1621,8 @@ extern "C" int atrex_entries_rank(const atrex_entry_t* d_entries, uint64_t n, ui
         const uint32_t want = ((uint32_t)n + 4 * BIN_THREADS - 1) / (4 * BIN_THREADS), most = 4u * (uint32_t)n_sms;
         const uint32_t tiles = ((uint32_t)n + TILE_STEP - 1) / TILE_STEP, cap = (uint32_t)(out_cap < n ? out_cap : n);
         if (launch_chained(bin_phase_kernel, want < most ? want : most, BIN_THREADS, 0, s, b, phase) != cudaSuccess ||
-            launch_bins(b, d_ranked, cap, n_sms, s) != cudaSuccess ||
-            launch_chained(bin_tile_scan_kernel, 1, SCAN_BLOCK, 0, s, b, coverage_ppm) != cudaSuccess ||
-            launch_chained(bin_share_kernel, tiles, SCAN_BLOCK, 0, s, b, d_ranked, d_cum_share, cap) != cudaSuccess ||
+            launch_bins(b, coverage_ppm, d_ranked, cap, n_sms, s) != cudaSuccess ||
+            launch_chained(bin_share_kernel, tiles < CUM_CTAS * (uint32_t)n_sms ? tiles : CUM_CTAS * (uint32_t)n_sms, CUM_THREADS, 0, s, b, d_cum_share, cap) != cudaSuccess ||
             slot.wait() != cudaSuccess)
             return ATREX_ERR_CUDA;
         const volatile BinReport* r = slot.get();

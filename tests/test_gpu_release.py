@@ -257,3 +257,38 @@ def test_equal_keys_keep_their_order(lib, n):
     e["key"] = rng.integers(0, max(2, n // 5), n).astype(np.uint64) << np.uint64(30)
     e["count"] = np.arange(n)
     assert host(lib.sort_entries_by_key(dev(e), n), oracle.ENTRY_DTYPE).tobytes() == e[np.argsort(e["key"], kind="stable")].tobytes()
+
+
+@pytest.mark.parametrize("n", [3_000, 9_001, 40_000, 700_001])
+@pytest.mark.parametrize("crowd", ["alike", "close", "alike and close", "alike, equal keys", "steps"])
+def test_crowded_weights(lib, n, crowd):
+    """Hundreds to thousands of weights in one place of a wide scale: equal ones (their keys decide, or the input order), some that only
+    the last bits tell apart, both, and many values of a hundred equal ones each."""
+    rng = np.random.default_rng(n + len(crowd))
+    e = np.zeros(n, dtype=oracle.ENTRY_DTYPE)
+    e["key"] = rng.permutation(np.arange(n, dtype=np.uint64) * np.uint64(977))
+    e["count"] = np.arange(n)
+    wt = np.exp2(rng.normal(40, 5, n).clip(5, 59)).astype(np.uint64)
+    m = min(n, 2_900)
+    at = rng.permutation(n)[:m]
+    if crowd == "close":
+        wt[at] = np.uint64(1 << 60) + rng.integers(0, 1 << 20, m).astype(np.uint64)
+    elif crowd == "steps":
+        wt[at] = np.uint64(1 << 60) + (rng.integers(0, 29, m).astype(np.uint64) << np.uint64(9))
+    else:
+        wt[at] = np.uint64(1 << 60)
+    if crowd == "alike and close":
+        wt[at[::3]] += rng.integers(0, 1 << 45, len(at[::3])).astype(np.uint64)
+    if crowd == "alike, equal keys":
+        e["key"][at[: m // 2]] = 977
+    e["wt_lo"] = wt
+    d = dev(e)
+    for phase, ppm, cap in [(0, 0, None), (0, 900_000, n // 2)]:
+        got_r, got_c, got_res = lib.rank_entries(d, n, phase, ppm, out_cap=cap)
+        order = np.lexsort((np.arange(n), e["key"], ~e["wt_lo"]))           # weight descending, key ascending, input order
+        rows = len(host(got_c, np.float64))
+        assert host(got_r, lib.ENTRY_DTYPE).tobytes() == e[order][:rows].tobytes()
+        if crowd != "alike, equal keys":
+            exp_r, exp_c, exp_res = oracle.rank_phase(e, phase, ppm, out_cap=cap)
+            assert got_res == exp_res and host(got_c, np.float64).tobytes() == exp_c.tobytes()
+            assert host(got_r, lib.ENTRY_DTYPE).tobytes() == exp_r.tobytes()
