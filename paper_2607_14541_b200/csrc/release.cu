@@ -425,13 +425,19 @@ __global__ void __launch_bounds__(SCAN_BLOCK) rank_emit_kernel(const atrex_entry
 constexpr uint32_t BIN_BITS_MAX = 14, BIN_THREADS = 512;
 constexpr uint32_t SHARE_THREADS = 1024;     // counting and moving: one CTA per SM, for long runs
 constexpr uint32_t CURSORS_MAX = 1u << 14;
-constexpr uint32_t TILE_STEP = 2048;        // a tile is the bins that start in one such window of positions
+// A tile is the bins that start in one window of 2^log_step positions: 2 048, or 512 where a list is so short that larger tiles would
+// leave SMs without one and make every phase of a tile's sort longer (tile kernel, key order of 10 000 entries 12.7 -> 7.9 us, 150 000
+// 13.5 -> 9.3, 250 000 13.2 -> 15.4; one phase of two, 75 000 entries 27.9 -> 12.7, 250 000 25.5 -> 14.0, 400 000 no change in all).
+constexpr uint32_t TILE_LOG_STEP = 11, SMALL_LOG_STEP = 9;
+constexpr uint64_t SMALL_LIST_MAX = 150000, SMALL_RANKING_MAX = 300000;
 constexpr uint32_t TILE_GROUP = 64;         // tiles whose weighted times are summed
 constexpr uint32_t TILE_CAP = 6144;         // ... and has at most this many items
-constexpr uint32_t TILE_LOCAL_BINS = 4096, TILE_THREADS = 512, TILE_HELD = 5, GATHER_LOADS = 6;
+constexpr uint32_t TILE_LOCAL_BINS = 4096, SMALL_LOCAL_BINS = 1024, TILE_THREADS = 512, TILE_HELD = 5, GATHER_LOADS = 6;
 constexpr uint32_t TILE_CLASH_MAX = 24;     // larger local bins are crowded: some are sorted by a warp or the CTA each,
+constexpr uint32_t TILE_TIES = 8;           // from so many on, half of them alike in their leading bits, a local bin counts as crowded, too
 constexpr uint32_t TILE_CROWDED = 32;       // more of them send the tile to the comparison network
-constexpr uint32_t TILE_SMALL_CROWD = 64;   // sorted by a warp
+constexpr uint32_t TILE_SMALL_CROWD = 64;   // sorted by a warp each, side by side, which takes 12 us; the whole CTA takes 4 for one,
+constexpr uint32_t TILE_CROWDED_FEW = 3;    // so that so many are sorted one after the other
 constexpr size_t TILE_SMEM = (size_t)TILE_CAP * 8 + TILE_LOCAL_BINS * 4;    // (what it leaves of two CTAs is L1 for the gather)
 constexpr uint32_t COUNT_SORT_MAX = 8192;   // up to here one kernel ranks every key by counting
 
@@ -472,6 +478,7 @@ struct BinSort {                 // what the kernels share
     uint32_t* cursors;           // [n_cursors] where the next item of a tile (by_tile) or bin goes
     uint32_t* tile_start;        // [tiles + 1]
     uint32_t n_cursors;
+    uint32_t log_step;           // a tile's window of positions
     bool by_tile;                // items of a tile lie in any order, not bin by bin
     ulonglong2* tile_sum;        // (ranking) [tiles] weighted time
     ulonglong2* group_sum;       // (ranking) ... of TILE_GROUP tiles
@@ -482,6 +489,7 @@ struct BinSort {                 // what the kernels share
     uint32_t turns;              // parts of the cursors that step 4 serves one after the other
 };
 
+__host__ __device__ __forceinline__ uint32_t tiles_of(const BinSort& b, uint32_t items) { return (uint32_t)(((uint64_t)items + (1u << b.log_step) - 1) >> b.log_step); }
 __device__ __forceinline__ uint32_t item_count(const BinSort& b) { return b.ranking ? (uint32_t)b.ctl->counter : b.n; }
 
 __device__ __forceinline__ ull rank_word(ull lo, ull hi) {
@@ -749,16 +757,16 @@ __global__ void __launch_bounds__(1024) bin_scan_kernel(const BinSort b, uint32_
     }
     __syncthreads();
     uint32_t at = incl - sum + (w ? s_warp[w - 1] : 0u);
-    // tile j starts at the first bin start at or beyond j * TILE_STEP (tile 0 at 0)
-    const uint32_t n_tiles = (b.n + TILE_STEP - 1) / TILE_STEP;
+    // tile j starts at the first bin start at or beyond j * 2^log_step (tile 0 at 0)
+    const uint32_t n_tiles = tiles_of(b, b.n);
 #pragma unroll
     for (uint32_t u = 0; u < 1u << (BIN_BITS_MAX - 10); ++u) {
         if (u >= per || first + u >= n_bins) continue;
         // (a bin belongs to the tile whose window it starts in)
-        b.bins[first + u] = b.by_tile ? at / TILE_STEP : first + u;
+        b.bins[first + u] = b.by_tile ? at >> b.log_step : first + u;
         if (!b.by_tile) b.cursors[first + u] = at;
         const uint32_t next = at + c[u];
-        for (uint32_t j = at / TILE_STEP + 1; j <= next / TILE_STEP; ++j) {
+        for (uint32_t j = (at >> b.log_step) + 1; j <= next >> b.log_step; ++j) {
             b.tile_start[j] = next;
             if (b.by_tile && j < b.n_cursors) b.cursors[j] = next;
         }
@@ -767,8 +775,8 @@ __global__ void __launch_bounds__(1024) bin_scan_kernel(const BinSort b, uint32_
     if (threadIdx.x == 0) {
         b.tile_start[0] = 0;
         if (b.by_tile) b.cursors[0] = 0;
-        for (uint32_t j = m / TILE_STEP + 1; j <= n_tiles; ++j) b.tile_start[j] = m;
-        const bool overflow = s_max + TILE_STEP > TILE_CAP;
+        for (uint32_t j = (m >> b.log_step) + 1; j <= n_tiles; ++j) b.tile_start[j] = m;
+        const bool overflow = s_max + (1u << b.log_step) > TILE_CAP;
         b.report->overflow = overflow;
         const bool too_large = b.ranking && (b.ctl->total_hi >> 44) != 0;      // T * 10^6 must fit 128 bits
         b.report->too_large = too_large;
@@ -1007,19 +1015,21 @@ __device__ __forceinline__ void sort_small_bin(const atrex_entry_t* entries, boo
 }
 
 // Sorts n <= TILE_CAP items whose leading bits lie in [low, high] into s_item.  `each(f)` calls f with each of
-// this thread's items (twice).  Each item goes to one of 4 096 local bins of equal width -- less than one item per bin, so that
+// this thread's items (twice).  Each item goes to one of twice as many local bins of equal width as a tile usually has items -- less than one item per bin, so that
 // a thread puts a bin in order by insertion; a few crowded local bins (hundreds of equal weights, say) are
 // sorted on their own, many of them send the whole tile through a bitonic network, with absent items behind the last one.
 // (Every item's place counted by a thread of its own instead: 3.1 M entries 107.5 -> 111 us.)
-template <typename Each>
+template <uint32_t LOCAL_BINS, typename Each>
 __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ranking, uint32_t n, uint32_t low, uint32_t high, Each each, ull* s_item,
                                           uint32_t* s_local) {
     __shared__ uint32_t s_warp[32];
     __shared__ uint32_t s_crowded, s_bin[TILE_CROWDED], s_begin[TILE_CROWDED], s_size[TILE_CROWDED];
     const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
     const int len = 32 - __clz((int)(high - low));
-    const int shift = len > 12 ? len - 12 : 0;
-    for (uint32_t i = threadIdx.x; i < TILE_LOCAL_BINS; i += blockDim.x) s_local[i] = 0;
+    constexpr int BITS = LOCAL_BINS == 4096 ? 12 : 10;
+    static_assert(LOCAL_BINS == 1u << BITS, "bits of a local bin");
+    const int shift = len > BITS ? len - BITS : 0;
+    for (uint32_t i = threadIdx.x; i < LOCAL_BINS; i += blockDim.x) s_local[i] = 0;
     if (threadIdx.x == 0) s_crowded = 0;
     __syncthreads();
     each([&](ull item) {
@@ -1031,7 +1041,7 @@ __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ran
     });
     __syncthreads();
     // exclusive scan of the local bins: each thread a run of them
-    const uint32_t per = TILE_LOCAL_BINS / blockDim.x, first = threadIdx.x * per;
+    const uint32_t per = LOCAL_BINS / blockDim.x, first = threadIdx.x * per;
     uint32_t sum = 0;
     for (uint32_t u = 0; u < per; ++u) sum += s_local[first + u];
     uint32_t incl = sum;
@@ -1064,17 +1074,28 @@ __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ran
     // (a bin's cursor now stands at its end, its predecessor's at its start)
     const uint32_t crowded = s_crowded;
     if (crowded <= TILE_CROWDED) {
+        const uint32_t by_warp = crowded > TILE_CROWDED_FEW ? TILE_SMALL_CROWD : 0u;
         for (uint32_t k = w; k < crowded; k += n_warps) {
             const uint32_t d = s_bin[k], b0 = d ? s_local[d - 1] : 0u, size = s_local[d] - b0;
-            if (size <= TILE_SMALL_CROWD) sort_small_bin(entries, ranking, s_item + b0, size);
+            if (size <= by_warp) sort_small_bin(entries, ranking, s_item + b0, size);
             if (lane == 0) {
                 s_begin[k] = b0;
                 s_size[k] = size;
             }
         }
-        for (uint32_t d = threadIdx.x; d < TILE_LOCAL_BINS; d += blockDim.x) {
+        for (uint32_t d = threadIdx.x; d < LOCAL_BINS; d += blockDim.x) {
             const uint32_t b0 = d ? s_local[d - 1] : 0u, b1 = s_local[d];
             if (b1 - b0 > TILE_CLASH_MAX) continue;
+            if (b1 - b0 >= TILE_TIES) {                  // leading bits alike: every comparison would read two entries
+                uint32_t ties = 0;
+                for (uint32_t i = b0 + 1; i < b1; ++i) ties += (s_item[i] ^ s_item[b0]) >> 32 ? 0u : 1u;
+                const uint32_t k = ties < TILE_TIES / 2 ? TILE_CROWDED : atomicAdd(&s_crowded, 1u);
+                if (k < TILE_CROWDED) {
+                    s_begin[k] = b0;
+                    s_size[k] = b1 - b0;
+                    continue;
+                }
+            }
             for (uint32_t i = b0 + 1; i < b1; ++i) {
                 const ull item = s_item[i];
                 uint32_t j = i;
@@ -1086,8 +1107,8 @@ __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ran
             }
         }
         __syncthreads();
-        for (uint32_t k = 0; k < crowded; ++k)           // (the same for every thread; the local bins are not needed any more)
-            if (s_size[k] > TILE_SMALL_CROWD) sort_crowded_bin(entries, ranking, s_item, s_begin[k], s_size[k], s_local);
+        for (uint32_t k = 0; k < min(s_crowded, TILE_CROWDED); ++k)      // (the same for every thread; the local bins are not needed any more)
+            if (k >= crowded || s_size[k] > by_warp) sort_crowded_bin(entries, ranking, s_item, s_begin[k], s_size[k], s_local);
     } else {
         bitonic(n, [&](uint32_t a, uint32_t b) { return item_less(entries, ranking, s_item[a], s_item[b]); },
                 [&](uint32_t a, uint32_t b) { const ull x = s_item[a]; s_item[a] = s_item[b]; s_item[b] = x; });
@@ -1135,6 +1156,7 @@ __device__ __forceinline__ void gather_tile(const atrex_entry_t* entries, const 
 }
 
 // 5. a tile's items in order, their entries gathered; (ranking) the tile's weighted time, and the order itself
+template <uint32_t LOCAL_BINS>
 __global__ void __launch_bounds__(TILE_THREADS) bin_tile_kernel(const BinSort b, atrex_entry_t* out, uint32_t out_cap) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     ull* s_item = reinterpret_cast<ull*>(smem_raw);
@@ -1144,7 +1166,7 @@ __global__ void __launch_bounds__(TILE_THREADS) bin_tile_kernel(const BinSort b,
     grid_dependency_wait();
     const bool overflow = b.ctl->overflow;
     // the last tile first: at both ends of a ranking the words lie uneven, which takes a tile twice as long
-    const uint32_t n_tiles = (item_count(b) + TILE_STEP - 1) / TILE_STEP;
+    const uint32_t n_tiles = tiles_of(b, item_count(b));
     const uint32_t tile = blockIdx.x >= n_tiles ? blockIdx.x : (blockIdx.x ? blockIdx.x - 1 : n_tiles - 1);
     const uint32_t first = overflow ? 0u : b.tile_start[tile], n = overflow ? 0u : b.tile_start[tile + 1] - first;
     if (n == 0) {
@@ -1180,7 +1202,7 @@ __global__ void __launch_bounds__(TILE_THREADS) bin_tile_kernel(const BinSort b,
         atomicMax(&s_range[1], top);
     }
     __syncthreads();
-    sort_tile(b.entries, b.ranking, n, ~s_range[0], s_range[1], each, s_item, s_local);
+    sort_tile<LOCAL_BINS>(b.entries, b.ranking, n, ~s_range[0], s_range[1], each, s_item, s_local);
     grid_dependents_launch();
     if (threadIdx.x < 2) s_sum[threadIdx.x] = 0;
     ulonglong2 sum = make_ulonglong2(0, 0);
@@ -1228,7 +1250,7 @@ __global__ void __launch_bounds__(CUM_THREADS, CUM_CTAS) bin_share_kernel(const 
     __shared__ double s_cum[CUM_THREADS * CUM_ROWS];
     grid_dependency_wait();
     const ull total_lo = b.ctl->total_lo, total_hi = b.ctl->total_hi, need_lo = b.ctl->need_lo, need_hi = b.ctl->need_hi, overflow = b.ctl->overflow;
-    const uint32_t n_tiles = (item_count(b) + TILE_STEP - 1) / TILE_STEP, run = (n_tiles + gridDim.x - 1) / gridDim.x;
+    const uint32_t n_tiles = tiles_of(b, item_count(b)), run = (n_tiles + gridDim.x - 1) / gridDim.x;
     const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5, tile = min(n_tiles, blockIdx.x * run), group = tile / TILE_GROUP;
     if (overflow) {
         finish_call(b.report, b.slot);
@@ -1447,7 +1469,8 @@ int prepare_sort_kernels(int* n_sms) {
         if (cudaFuncSetAttribute(radix_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCATTER_SMEM) != cudaSuccess ||
             cudaFuncSetAttribute(bin_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 << BIN_BITS_MAX) != cudaSuccess ||
             cudaFuncSetAttribute(bin_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(4 * CURSORS_MAX + (2 << BIN_BITS_MAX))) != cudaSuccess ||
-            cudaFuncSetAttribute(bin_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM) != cudaSuccess ||
+            cudaFuncSetAttribute(bin_tile_kernel<TILE_LOCAL_BINS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM) != cudaSuccess ||
+            cudaFuncSetAttribute(bin_tile_kernel<SMALL_LOCAL_BINS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM) != cudaSuccess ||
             cudaFuncSetAttribute(count_sort_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(COUNT_SORT_MAX * 8)) != cudaSuccess ||
             cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
             cudaGetLastError();
@@ -1481,17 +1504,19 @@ inline uint64_t group_bytes(uint64_t tiles, bool ranking) { return ranking ? (ti
 // The scratch as the binned sort uses it.
 BinSort carve_bins(void* base, const atrex_entry_t* entries, uint64_t n, bool ranking, const ReportSlot& slot) {
     unsigned char* p = (unsigned char*)base;
-    const uint64_t tiles = (n + TILE_STEP - 1) / TILE_STEP;
     BinSort b;
+    b.log_step = n <= (ranking ? SMALL_RANKING_MAX : SMALL_LIST_MAX) ? SMALL_LOG_STEP : TILE_LOG_STEP;
+    const uint64_t tiles = tiles_of(b, (uint32_t)n);
     b.ctl = (BinCtl*)p;
     b.report = slot.get();
     b.slot = slot.number();
     b.entries = entries;
     b.n = (uint32_t)n;
     b.ranking = ranking;
-    // about 256 items per bin, a thousand beyond 2^12 bins (more open ranges than that cost the scattered writes)
+    // about 256 items per bin, a thousand beyond 2^12 bins (more open ranges than that cost the scattered writes), 64 or
+    // 128 for small tiles
     b.bits = 4;
-    while (b.bits < BIN_BITS_MAX && ((b.bits < 12 ? 256ull : 1024ull) << b.bits) < n) ++b.bits;
+    while (b.bits < BIN_BITS_MAX && ((b.log_step == SMALL_LOG_STEP ? (n <= 65536 ? 64ull : 128ull) : b.bits < 12 ? 256ull : 1024ull) << b.bits) < n) ++b.bits;
     p += sizeof(BinCtl);
     b.group_sum = (ulonglong2*)p; p += group_bytes(tiles, ranking);
     b.by_tile = tiles <= CURSORS_MAX;
@@ -1511,19 +1536,20 @@ BinSort carve_bins(void* base, const atrex_entry_t* entries, uint64_t n, bool ra
 static_assert(sizeof(BinCtl) + 16u + (4u << 5) + 4u * 4u + 16u * 3u + 4u * 4u + 256u <= sizeof(ReleaseCtl) + 1024u + 1024u + 256u, "smallest case");
 
 cudaError_t launch_clear(const BinSort& b, cudaStream_t s) {
-    const uint32_t n = (uint32_t)((sizeof(BinCtl) + group_bytes((b.n + TILE_STEP - 1) / TILE_STEP, b.ranking) + (4ull << b.bits)) / 16);
+    const uint32_t n = (uint32_t)((sizeof(BinCtl) + group_bytes(tiles_of(b, b.n), b.ranking) + (4ull << b.bits)) / 16);
     return launch_chained(bin_clear_kernel, (n + BIN_THREADS - 1) / BIN_THREADS, BIN_THREADS, 0, s, (uint4*)b.ctl, n);
 }
 
 // Steps 2 to 5, behind the kernel that made the words.
 cudaError_t launch_bins(const BinSort& b, uint32_t coverage_ppm, atrex_entry_t* out, uint64_t out_cap, int n_sms, cudaStream_t s) {
-    const uint32_t bytes = 4u << b.bits, tiles = (b.n + TILE_STEP - 1) / TILE_STEP;
+    const uint32_t bytes = 4u << b.bits, tiles = tiles_of(b, b.n);
     uint32_t grid = (b.n + 4095) / 4096;
     if (grid > (uint32_t)n_sms) grid = (uint32_t)n_sms;
     cudaError_t e = launch_chained(bin_count_kernel, grid, SHARE_THREADS, bytes, s, b);
     if (e == cudaSuccess) e = launch_chained(bin_scan_kernel, 1, 1024, 0, s, b, coverage_ppm);
     if (e == cudaSuccess) e = launch_chained(bin_scatter_kernel, grid, SHARE_THREADS, b.n_cursors * 4 + (2u << b.bits), s, b);
-    if (e == cudaSuccess) e = launch_chained(bin_tile_kernel, tiles, TILE_THREADS, TILE_SMEM, s, b, out, (uint32_t)(out_cap < b.n ? out_cap : b.n));
+    auto* tile = b.log_step == SMALL_LOG_STEP ? bin_tile_kernel<SMALL_LOCAL_BINS> : bin_tile_kernel<TILE_LOCAL_BINS>;
+    if (e == cudaSuccess) e = launch_chained(tile, tiles, TILE_THREADS, TILE_SMEM, s, b, out, (uint32_t)(out_cap < b.n ? out_cap : b.n));
     return e;
 }
 
@@ -1619,7 +1645,7 @@ extern "C" int atrex_entries_rank(const atrex_entry_t* d_entries, uint64_t n, ui
         const BinSort b = carve_bins(d_scratch, d_entries, n, true, slot);
         if (launch_clear(b, s) != cudaSuccess) return ATREX_ERR_CUDA;
         const uint32_t want = ((uint32_t)n + 4 * BIN_THREADS - 1) / (4 * BIN_THREADS), most = 4u * (uint32_t)n_sms;
-        const uint32_t tiles = ((uint32_t)n + TILE_STEP - 1) / TILE_STEP, cap = (uint32_t)(out_cap < n ? out_cap : n);
+        const uint32_t tiles = tiles_of(b, (uint32_t)n), cap = (uint32_t)(out_cap < n ? out_cap : n);
         if (launch_chained(bin_phase_kernel, want < most ? want : most, BIN_THREADS, 0, s, b, phase) != cudaSuccess ||
             launch_bins(b, coverage_ppm, d_ranked, cap, n_sms, s) != cudaSuccess ||
             launch_chained(bin_share_kernel, tiles < CUM_CTAS * (uint32_t)n_sms ? tiles : CUM_CTAS * (uint32_t)n_sms, CUM_THREADS, 0, s, b, d_cum_share, cap) != cudaSuccess ||
