@@ -1398,6 +1398,137 @@ __global__ void __launch_bounds__(COUNT_THREADS) count_sort_kernel(const atrex_e
     finish_call(report, slot);
 }
 
+// A phase of a list of up to COUNT_RANK_MAX entries ranked in one kernel: an entry's place is the number of the phase's entries before
+// it, and the running sum before it the sum of theirs.  Every CTA reads all entries, puts the phase's side by side and places 32 of
+// them, a lane each, every warp counting over its own sixteenth.  Bound by the comparisons, some twenty instructions each (whole call,
+// one phase of two, in seven launches before: 100 entries 41 -> 18 us, 2 000 45 -> 23, 4 096 51 -> 30; all of one phase 4 096 52 -> 43.  Twice as
+// many entries are twice the CTAs and twice the comparisons of each: no gain in one phase).
+constexpr uint32_t COUNT_RANK_MAX = 4096;
+__global__ void __launch_bounds__(COUNT_THREADS) count_rank_kernel(const atrex_entry_t* entries, uint32_t n, uint32_t phase, uint32_t coverage_ppm,
+                                                                   atrex_entry_t* out, double* cum, uint32_t out_cap, BinReport* report, uint32_t slot) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    ulonglong2* s_wt = reinterpret_cast<ulonglong2*>(smem_raw);        // [n] the phase's entries in input order
+    ull* s_key = reinterpret_cast<ull*>(s_wt + n);
+    uint16_t* s_at = reinterpret_cast<uint16_t*>(s_key + n);
+    constexpr uint32_t WARPS = COUNT_THREADS / 32, EACH = COUNT_RANK_MAX / COUNT_THREADS, WORDS = COUNT_RANK_MAX / 32;
+    __shared__ ulonglong2 s_sum[WARPS][32];
+    __shared__ uint32_t s_count[WARPS][32], s_place[32], s_start[WORDS], s_counted;
+    __shared__ ull s_total[2];
+    const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5, base = blockIdx.x * 32;
+    if (threadIdx.x < 2) s_total[threadIdx.x] = 0;
+    grid_dependency_wait();
+    ull key[EACH], lo[EACH], hi[EACH], total_lo = 0, total_hi = 0;
+#pragma unroll
+    for (uint32_t u = 0; u < EACH; ++u) {
+        const uint32_t i = u * COUNT_THREADS + threadIdx.x;
+        key[u] = i < n ? entries[i].key : ~0ull;
+        lo[u] = i < n ? entries[i].wt_lo : 0ull;
+        hi[u] = i < n ? entries[i].wt_hi : 0ull;
+    }
+    grid_dependents_launch();
+    uint32_t votes[EACH];
+#pragma unroll
+    for (uint32_t u = 0; u < EACH; ++u) {
+        const bool mine = (uint32_t)(key[u] >> 48) == phase;
+        votes[u] = __ballot_sync(FULL, mine);
+        if (lane == 0) s_start[u * WARPS + w] = __popc(votes[u]);
+        if (mine) add128(total_lo, total_hi, lo[u], hi[u]);
+    }
+    __syncthreads();
+    if (w == 0) {                                        // where each word's entries start
+        static_assert(WORDS == 128, "four words a lane");
+        uint32_t c[4], own = 0;
+#pragma unroll
+        for (uint32_t j = 0; j < 4; ++j) own += c[j] = s_start[lane * 4 + j];
+        uint32_t incl = own;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t o = __shfl_up_sync(FULL, incl, d);
+            if (lane >= (uint32_t)d) incl += o;
+        }
+        uint32_t at = incl - own;
+#pragma unroll
+        for (uint32_t j = 0; j < 4; ++j) {
+            s_start[lane * 4 + j] = at;
+            at += c[j];
+        }
+        if (lane == 31) s_counted = incl;
+    }
+#pragma unroll
+    for (int d = 16; d; d >>= 1) {
+        const ull olo = __shfl_xor_sync(FULL, total_lo, d), ohi = __shfl_xor_sync(FULL, total_hi, d);
+        add128(total_lo, total_hi, olo, ohi);
+    }
+    if (lane == 0 && (total_lo | total_hi)) atomic_add128(&s_total[0], &s_total[1], total_lo, total_hi);
+    __syncthreads();
+#pragma unroll
+    for (uint32_t u = 0; u < EACH; ++u) {
+        if ((votes[u] & (1u << lane)) == 0) continue;
+        const uint32_t at = s_start[u * WARPS + w] + __popc(votes[u] & ((1u << lane) - 1u));
+        s_wt[at] = make_ulonglong2(lo[u], hi[u]);
+        s_key[at] = key[u];
+        s_at[at] = (uint16_t)(u * COUNT_THREADS + threadIdx.x);
+    }
+    __syncthreads();
+    const uint32_t m = s_counted, own = base + lane;
+    const ulonglong2 mine = own < m ? s_wt[own] : make_ulonglong2(0, 0);
+    const ull my_key = own < m ? s_key[own] : 0ull, my_lo = mine.x, my_hi = mine.y;
+    const uint32_t per = (m + WARPS - 1) / WARPS, first = base < m ? min(m, w * per) : m, end = min(m, first + per);
+    uint32_t before = 0;
+    ull sum_lo = 0, sum_hi = 0;
+#pragma unroll 4
+    for (uint32_t j = first; j < end; ++j) {
+        const ulonglong2 x = s_wt[j];
+        bool less = x.y > my_hi || (x.y == my_hi && x.x > my_lo);
+        if (x.x == my_lo && x.y == my_hi) less = s_key[j] < my_key || (s_key[j] == my_key && j < own);    // equal keys keep their input order
+        before += less ? 1u : 0u;
+        add128(sum_lo, sum_hi, less ? x.x : 0ull, less ? x.y : 0ull);
+    }
+    s_count[w][lane] = before;
+    s_sum[w][lane] = make_ulonglong2(sum_lo, sum_hi);
+    __syncthreads();
+    total_lo = s_total[0];
+    total_hi = s_total[1];
+    const bool too_large = (total_hi >> 44) != 0;        // T * 10^6 must fit 128 bits
+    if (w == 0) {
+        uint32_t place = 0;
+        ull ex_lo = 0, ex_hi = 0;
+#pragma unroll
+        for (uint32_t k = 0; k < WARPS; ++k) {
+            place += s_count[k][lane];
+            add128(ex_lo, ex_hi, s_sum[k][lane].x, s_sum[k][lane].y);
+        }
+        const bool ranked = own < m && !too_large;
+        s_place[lane] = ranked && place < out_cap ? place : ~0u;
+        if (ranked) {
+            // the smallest k with 10^6 * prefix_k >= ppm * T, i.e. prefix_k >= ceil(ppm * T / 10^6)
+            const unsigned __int128 total = ((unsigned __int128)total_hi << 64) | total_lo;
+            const unsigned __int128 need = ((unsigned __int128)coverage_ppm * total + 999999u) / 1000000u;
+            const unsigned __int128 ex = ((unsigned __int128)ex_hi << 64) | ex_lo, in = ex + (((unsigned __int128)my_hi << 64) | my_lo);
+            if (need != 0 && ex < need && in >= need) {
+                report->n_keep = (ull)place + 1;
+                report->covered_lo = (ull)in;
+                report->covered_hi = (ull)(in >> 64);
+                __threadfence_system();
+            }
+            if (place < out_cap) cum[place] = total != 0 ? __ddiv_rn(u128_to_f64_rn((ull)(in >> 64), (ull)in), u128_to_f64_rn(total_hi, total_lo)) : 0.0;
+        }
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 32) {
+        report->counter = s_counted;
+        report->total_lo = total_lo;
+        report->total_hi = total_hi;
+        report->too_large = too_large;
+        __threadfence_system();
+    }
+    __syncthreads();
+    const ull* src = reinterpret_cast<const ull*>(entries);
+    ull* dst = reinterpret_cast<ull*>(out);
+    for (uint32_t x = threadIdx.x; x < 32 * 6; x += COUNT_THREADS)
+        if (s_place[x / 6] != ~0u) dst[(size_t)s_place[x / 6] * 6 + x % 6] = src[(size_t)s_at[base + x / 6] * 6 + x % 6];
+    finish_call(report, slot);
+}
+
 // ---- host side
 
 struct Scratch {
@@ -1471,6 +1602,7 @@ int prepare_sort_kernels(int* n_sms) {
             cudaFuncSetAttribute(bin_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(4 * CURSORS_MAX + (2 << BIN_BITS_MAX))) != cudaSuccess ||
             cudaFuncSetAttribute(bin_tile_kernel<TILE_LOCAL_BINS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM) != cudaSuccess ||
             cudaFuncSetAttribute(bin_tile_kernel<SMALL_LOCAL_BINS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM) != cudaSuccess ||
+            cudaFuncSetAttribute(count_rank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(COUNT_RANK_MAX * 26)) != cudaSuccess ||
             cudaFuncSetAttribute(count_sort_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(COUNT_SORT_MAX * 8)) != cudaSuccess ||
             cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
             cudaGetLastError();
@@ -1642,15 +1774,21 @@ extern "C" int atrex_entries_rank(const atrex_entry_t* d_entries, uint64_t n, ui
     {
         ReportSlot slot(s);
         if (!slot.get()) return ATREX_ERR_NOMEM;
-        const BinSort b = carve_bins(d_scratch, d_entries, n, true, slot);
-        if (launch_clear(b, s) != cudaSuccess) return ATREX_ERR_CUDA;
-        const uint32_t want = ((uint32_t)n + 4 * BIN_THREADS - 1) / (4 * BIN_THREADS), most = 4u * (uint32_t)n_sms;
-        const uint32_t tiles = tiles_of(b, (uint32_t)n), cap = (uint32_t)(out_cap < n ? out_cap : n);
-        if (launch_chained(bin_phase_kernel, want < most ? want : most, BIN_THREADS, 0, s, b, phase) != cudaSuccess ||
-            launch_bins(b, coverage_ppm, d_ranked, cap, n_sms, s) != cudaSuccess ||
-            launch_chained(bin_share_kernel, tiles < CUM_CTAS * (uint32_t)n_sms ? tiles : CUM_CTAS * (uint32_t)n_sms, CUM_THREADS, 0, s, b, d_cum_share, cap) != cudaSuccess ||
-            slot.wait() != cudaSuccess)
-            return ATREX_ERR_CUDA;
+        const uint32_t cap = (uint32_t)(out_cap < n ? out_cap : n);
+        cudaError_t e;
+        if (n <= COUNT_RANK_MAX) {
+            e = launch_chained(count_rank_kernel, ((uint32_t)n + 31) / 32, COUNT_THREADS, (size_t)n * 26, s, d_entries, (uint32_t)n, phase, coverage_ppm,
+                               d_ranked, d_cum_share, cap, slot.get(), slot.number());
+        } else {
+            const BinSort b = carve_bins(d_scratch, d_entries, n, true, slot);
+            const uint32_t want = ((uint32_t)n + 4 * BIN_THREADS - 1) / (4 * BIN_THREADS), most = 4u * (uint32_t)n_sms, tiles = tiles_of(b, (uint32_t)n);
+            e = launch_clear(b, s);
+            if (e == cudaSuccess) e = launch_chained(bin_phase_kernel, want < most ? want : most, BIN_THREADS, 0, s, b, phase);
+            if (e == cudaSuccess) e = launch_bins(b, coverage_ppm, d_ranked, cap, n_sms, s);
+            if (e == cudaSuccess)
+                e = launch_chained(bin_share_kernel, tiles < CUM_CTAS * (uint32_t)n_sms ? tiles : CUM_CTAS * (uint32_t)n_sms, CUM_THREADS, 0, s, b, d_cum_share, cap);
+        }
+        if (e != cudaSuccess || slot.wait() != cudaSuccess) return ATREX_ERR_CUDA;
         const volatile BinReport* r = slot.get();
         if (r->too_large || !r->overflow) {
             h_result->n_phase = r->counter;
