@@ -1070,9 +1070,9 @@ __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ran
     }
     __syncthreads();
     each([&](ull item) { s_item[atomicAdd(&s_local[((uint32_t)(item >> 32) - low) >> shift], 1u)] = item; });
+    const uint32_t crowded = s_crowded;   // (read on this side of the barrier: bins with ties are added behind it)
     __syncthreads();
     // (a bin's cursor now stands at its end, its predecessor's at its start)
-    const uint32_t crowded = s_crowded;
     if (crowded <= TILE_CROWDED) {
         const uint32_t by_warp = crowded > TILE_CROWDED_FEW ? TILE_SMALL_CROWD : 0u;
         for (uint32_t k = w; k < crowded; k += n_warps) {

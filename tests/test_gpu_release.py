@@ -292,3 +292,32 @@ def test_crowded_weights(lib, n, crowd):
             exp_r, exp_c, exp_res = oracle.rank_phase(e, phase, ppm, out_cap=cap)
             assert got_res == exp_res and host(got_c, np.float64).tobytes() == exp_c.tobytes()
             assert host(got_r, lib.ENTRY_DTYPE).tobytes() == exp_r.tobytes()
+
+
+@pytest.mark.parametrize("n", [9_001, 400_000])                            # tiles of 512 and of 2 048 items
+@pytest.mark.parametrize("size", [7, 8, 24, 25])
+@pytest.mark.parametrize("groups", [1, 4, 32, 33, 100])
+def test_groups_of_ties_in_one_tile(lib, n, groups, size):
+    """Small groups of equal weights, and of keys that are equal or alike in their leading bits, side by side: around the sizes from which
+    on such a group counts as crowded, and the numbers of groups at which a tile is sorted in another way."""
+    rng = np.random.default_rng(n + 10 * groups + size)
+    e = np.zeros(n, dtype=oracle.ENTRY_DTYPE)
+    e["count"] = np.arange(n)
+    group = np.repeat(np.arange(groups, dtype=np.uint64), size)            # (all of them within one range of the first cut)
+    at = rng.permutation(n)[: groups * size]
+    e["wt_lo"] = np.exp2(rng.uniform(52, 62, n)).astype(np.uint64)
+    e["wt_lo"][at] = np.uint64(1 << 60) + (group << np.uint64(45))
+    for alike in (False, True):                                              # (rows of a group equal but for their counts, or not)
+        e["key"] = rng.integers(0, 1 << 51, n).astype(np.uint64)
+        e["key"][at] = np.uint64(1 << 50) + (group << np.uint64(33))
+        if alike:
+            e["key"][at] += rng.permutation(len(at)).astype(np.uint64)
+        d = dev(e)
+        assert host(lib.sort_entries_by_key(d, n), oracle.ENTRY_DTYPE).tobytes() == e[np.argsort(e["key"], kind="stable")].tobytes()
+        one = e.copy()
+        one["key"] &= np.uint64((1 << 48) - 1)                               # (all of phase 0)
+        ranked, cum, res = lib.rank_entries(dev(one), n, 0, 900_000)
+        order = np.lexsort((np.arange(n), one["key"], ~one["wt_lo"]))        # weight descending, key ascending, input order
+        assert host(ranked, lib.ENTRY_DTYPE).tobytes() == one[order].tobytes()
+        exp_r, exp_c, exp_res = oracle.rank_phase(one, 0, 900_000)           # (equal rows are the same to sums and cut)
+        assert res == exp_res and host(cum, np.float64).tobytes() == exp_c.tobytes()
