@@ -875,6 +875,7 @@ __device__ __noinline__ void sort_crowded_bin(const atrex_entry_t* entries, bool
         bitonic(size, [&](uint32_t a, uint32_t b) { return item_less(entries, ranking, s_item[from + a], s_item[from + b]); },
                 [&](uint32_t a, uint32_t b) { const ull x = s_item[from + a]; s_item[from + a] = s_item[from + b]; s_item[from + b] = x; });
     };
+    __syncthreads();                 // (the local bins have been read, and the segments of the call before this one)
     if (threadIdx.x == 0) {
         s_segments = 1;
         s_from[0] = b0;
