@@ -1541,9 +1541,9 @@ struct Scratch {
     ull* bsums;
 };
 
-inline uint64_t align256(uint64_t x) { return (x + 255u) & ~(uint64_t)255u; }
+constexpr uint64_t align256(uint64_t x) { return (x + 255u) & ~(uint64_t)255u; }
 
-uint64_t scratch_bytes_for(uint64_t n) {
+constexpr uint64_t scratch_bytes_for(uint64_t n) {
     const uint64_t tiles = (n + SORT_TILE - 1) / SORT_TILE, blocks = (n + SCAN_BLOCK - 1) / SCAN_BLOCK;
     return sizeof(ReleaseCtl) + 2 * align256(n * 8) + 2 * align256(n * 4) + align256(tiles * 256 * 4) +
            1024 + align256(blocks * 16) + 256;
@@ -1632,44 +1632,64 @@ int sort_by_word(const Scratch& sc, int cur, uint32_t m, ull differing_bits, cud
     return cur;
 }
 
-inline uint64_t group_bytes(uint64_t tiles, bool ranking) { return ranking ? (tiles + TILE_GROUP - 1) / TILE_GROUP * 16 : 0; }
+// How many tiles, bins and cursors a list of n entries gets, and the bytes that these take in front of the items.
+struct BinSizes {
+    uint32_t log_step, bits, n_cursors;
+    bool by_tile;
+    uint64_t tiles, group_bytes, bin_bytes, cursor_bytes;
+    constexpr BinSizes(uint64_t n, bool ranking)
+        : log_step(n <= (ranking ? SMALL_RANKING_MAX : SMALL_LIST_MAX) ? SMALL_LOG_STEP : TILE_LOG_STEP), bits(4), n_cursors(0), by_tile(false),
+          tiles((n + (1ull << log_step) - 1) >> log_step), group_bytes(ranking ? (tiles + TILE_GROUP - 1) / TILE_GROUP * 16 : 0), bin_bytes(0), cursor_bytes(0) {
+        // about 256 items per bin, a thousand beyond 2^12 bins (more open ranges than that cost the scattered writes), 64 or
+        // 128 for small tiles
+        while (bits < BIN_BITS_MAX && ((log_step == SMALL_LOG_STEP ? (n <= 65536 ? 64ull : 128ull) : bits < 12 ? 256ull : 1024ull) << bits) < n) ++bits;
+        by_tile = tiles <= CURSORS_MAX;
+        n_cursors = by_tile ? (uint32_t)tiles : 1u << bits;
+        bin_bytes = 4ull << bits;
+        cursor_bytes = 4ull * ((n_cursors + 3) & ~3u);
+    }
+    constexpr uint64_t control_bytes() const { return align256(sizeof(BinCtl) + group_bytes + bin_bytes + cursor_bytes + tiles * 16 + (tiles + 1) * 4); }
+    constexpr uint64_t bytes(uint64_t n) const { return control_bytes() + 2 * align256(n * 8) + n * 4; }
+};
+// (the scratch's size is the radix sort's, whose digit counts take more than the control area: on both sides of every line above)
+constexpr bool bins_fit(uint64_t n) { return BinSizes(n, false).bytes(n) <= scratch_bytes_for(n) && BinSizes(n, true).bytes(n) <= scratch_bytes_for(n); }
+static_assert(bins_fit(1) && bins_fit(COUNT_RANK_MAX + 1) && bins_fit(COUNT_SORT_MAX + 1) && bins_fit(65536) && bins_fit(65537) && bins_fit(SMALL_LIST_MAX) &&
+                  bins_fit(SMALL_LIST_MAX + 1) && bins_fit(SMALL_RANKING_MAX) && bins_fit(SMALL_RANKING_MAX + 1) && bins_fit(1u << 20) && bins_fit((1u << 20) + 1) &&
+                  bins_fit(1u << 22) && bins_fit((1u << 22) + 1) && bins_fit((uint64_t)CURSORS_MAX << TILE_LOG_STEP) &&
+                  bins_fit(((uint64_t)CURSORS_MAX << TILE_LOG_STEP) + 1) && bins_fit(ATREX_RELEASE_MAX_ENTRIES), "the binned sort's use of the scratch");
 
 // The scratch as the binned sort uses it.
 BinSort carve_bins(void* base, const atrex_entry_t* entries, uint64_t n, bool ranking, const ReportSlot& slot) {
     unsigned char* p = (unsigned char*)base;
     BinSort b;
-    b.log_step = n <= (ranking ? SMALL_RANKING_MAX : SMALL_LIST_MAX) ? SMALL_LOG_STEP : TILE_LOG_STEP;
-    const uint64_t tiles = tiles_of(b, (uint32_t)n);
+    const BinSizes z(n, ranking);
+    b.log_step = z.log_step;
+    b.bits = z.bits;
+    b.n_cursors = z.n_cursors;
+    b.by_tile = z.by_tile;
+    b.turns = b.n_cursors >= 2048 ? 2 : 1;
     b.ctl = (BinCtl*)p;
     b.report = slot.get();
     b.slot = slot.number();
     b.entries = entries;
     b.n = (uint32_t)n;
     b.ranking = ranking;
-    // about 256 items per bin, a thousand beyond 2^12 bins (more open ranges than that cost the scattered writes), 64 or
-    // 128 for small tiles
-    b.bits = 4;
-    while (b.bits < BIN_BITS_MAX && ((b.log_step == SMALL_LOG_STEP ? (n <= 65536 ? 64ull : 128ull) : b.bits < 12 ? 256ull : 1024ull) << b.bits) < n) ++b.bits;
     p += sizeof(BinCtl);
-    b.group_sum = (ulonglong2*)p; p += group_bytes(tiles, ranking);
-    b.by_tile = tiles <= CURSORS_MAX;
-    b.n_cursors = b.by_tile ? (uint32_t)tiles : 1u << b.bits;
-    b.turns = b.n_cursors >= 2048 ? 2 : 1;
-    b.bins = (uint32_t*)p;       p += 4ull << b.bits;
-    b.cursors = (uint32_t*)p;    p += 4ull * ((b.n_cursors + 3) & ~3u);
-    b.tile_sum = (ulonglong2*)p; p += tiles * 16;
-    b.tile_start = (uint32_t*)p; p += (tiles + 1) * 4;
-    p = (unsigned char*)base + align256(p - (unsigned char*)base);
+    b.group_sum = (ulonglong2*)p; p += z.group_bytes;
+    b.bins = (uint32_t*)p;       p += z.bin_bytes;
+    b.cursors = (uint32_t*)p;    p += z.cursor_bytes;
+    b.tile_sum = (ulonglong2*)p; p += z.tiles * 16;
+    b.tile_start = (uint32_t*)p;
+    p = (unsigned char*)base + z.control_bytes();
     b.words = (ull*)p;           p += align256(n * 8);
     b.items = (ull*)p;           p += align256(n * 8);
     b.idx = (uint32_t*)p;
     return b;
 }
-// (what it needs beyond the pairs is less than the radix sort's digit counts, as long as there are a few tiles)
-static_assert(sizeof(BinCtl) + 16u + (4u << 5) + 4u * 4u + 16u * 3u + 4u * 4u + 256u <= sizeof(ReleaseCtl) + 1024u + 1024u + 256u, "smallest case");
 
 cudaError_t launch_clear(const BinSort& b, cudaStream_t s) {
-    const uint32_t n = (uint32_t)((sizeof(BinCtl) + group_bytes(tiles_of(b, b.n), b.ranking) + (4ull << b.bits)) / 16);
+    const BinSizes z(b.n, b.ranking);
+    const uint32_t n = (uint32_t)((sizeof(BinCtl) + z.group_bytes + z.bin_bytes) / 16);
     return launch_chained(bin_clear_kernel, (n + BIN_THREADS - 1) / BIN_THREADS, BIN_THREADS, 0, s, (uint4*)b.ctl, n);
 }
 
