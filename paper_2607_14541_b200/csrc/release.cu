@@ -434,11 +434,16 @@ constexpr uint32_t TILE_GROUP = 64;         // tiles whose weighted times are su
 constexpr uint32_t TILE_CAP = 6144;         // ... and has at most this many items
 constexpr uint32_t TILE_LOCAL_BINS = 4096, SMALL_LOCAL_BINS = 1024, TILE_THREADS = 512, TILE_HELD = 5, GATHER_LOADS = 6;
 constexpr uint32_t TILE_CLASH_MAX = 24;     // larger local bins are crowded: some are sorted by a warp or the CTA each,
-constexpr uint32_t TILE_TIES = 8;           // from so many on, half of them alike in their leading bits, a local bin counts as crowded, too
 constexpr uint32_t TILE_CROWDED = 32;       // more of them send the tile to the comparison network
 constexpr uint32_t TILE_SMALL_CROWD = 64;   // sorted by a warp each, side by side, which takes 12 us; the whole CTA takes 4 for one,
 constexpr uint32_t TILE_CROWDED_FEW = 3;    // so that so many are sorted one after the other
-constexpr size_t TILE_SMEM = (size_t)TILE_CAP * 8 + TILE_LOCAL_BINS * 4;    // (what it leaves of two CTAs is L1 for the gather)
+// From so many items on, half of them alike in their leading bits, a local bin has ties: by insertion every comparison would read two
+// entries, so a warp sorts it (tile kernel of a ranking by insertion / now: 100 groups of 8 equal weights in one tile of 75 000 entries 66 / 36 us,
+// 100 of 24 116 / 50; every weight 8 times, 700 000 entries 187 / 126, 3 million 617 / 415, 24 times 1 780 / 496; up to 32 of those bins by the whole CTA
+// one after the other, the rest by insertion: 229, 178, 366, 1 213 and 2 074).
+constexpr uint32_t TILE_TIES = 8;
+constexpr size_t TILE_SMEM = (size_t)TILE_CAP * 8 + TILE_LOCAL_BINS * 4;    // (what it leaves of two CTAs is L1 for the gather; with
+// more than 1 KB of static shared memory beside it less is left: 10 % slower)
 constexpr uint32_t COUNT_SORT_MAX = 8192;   // up to here one kernel ranks every key by counting
 
 struct BinCtl {                  // at the start of the scratch, cleared by every call (with the bins behind it)
@@ -471,9 +476,10 @@ struct BinSort {                 // what the kernels share
     BinCtl* ctl;
     BinReport* report;
     const atrex_entry_t* entries;
-    ull* words;                  // [n] raw words: keys (key order), words (ranking); (ranking) later low words of the ranked weighted times
+    ull* words;                  // [n] raw words: keys (key order), words (ranking)
     uint32_t* idx;               // [n] (ranking) entry of each word
-    ull* items;                  // [n] in bin order: leading 32 bits of the word's place in the range, then the entry; later the high words
+    ulonglong2* ranked_wt;       // [n] (ranking) in the place of both once they are read: the ranked rows' weighted times
+    ull* items;                  // [n] in bin order: leading 32 bits of the word's place in the range, then the entry
     uint32_t* bins;              // [1 << bits] counts, then each bin's cursor number
     uint32_t* cursors;           // [n_cursors] where the next item of a tile (by_tile) or bin goes
     uint32_t* tile_start;        // [tiles + 1]
@@ -868,7 +874,8 @@ __device__ __forceinline__ void bitonic(uint32_t n, Less less, Swap swap) {
 constexpr uint32_t CROWD_BINS = 2048, CROWD_MAX = 4096, CROWD_CLASH_MAX = 64, CROWD_SEGMENTS = 32;
 __device__ __noinline__ void sort_crowded_bin(const atrex_entry_t* entries, bool ranking, ull* s_item, uint32_t b0, uint32_t n, uint32_t* s_bins) {
     __shared__ ull s_range[2];
-    __shared__ uint32_t s_warp[32], s_segments, s_from[CROWD_SEGMENTS], s_size[CROWD_SEGMENTS];
+    __shared__ uint32_t s_warp[32], s_segments;
+    __shared__ uint16_t s_from[CROWD_SEGMENTS], s_size[CROWD_SEGMENTS];
     uint16_t* s_list = reinterpret_cast<uint16_t*>(s_bins + CROWD_BINS);
     const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
     auto by_network = [&](uint32_t from, uint32_t size) {
@@ -878,8 +885,8 @@ __device__ __noinline__ void sort_crowded_bin(const atrex_entry_t* entries, bool
     __syncthreads();                 // (the local bins have been read, and the segments of the call before this one)
     if (threadIdx.x == 0) {
         s_segments = 1;
-        s_from[0] = b0;
-        s_size[0] = n;
+        s_from[0] = (uint16_t)b0;
+        s_size[0] = (uint16_t)n;
     }
     __syncthreads();
     for (uint32_t k = 0; k < min(s_segments, CROWD_SEGMENTS); ++k) {       // (the same for every thread)
@@ -945,8 +952,8 @@ __device__ __noinline__ void sort_crowded_bin(const atrex_entry_t* entries, bool
             if (c[u] > CROWD_CLASH_MAX) {
                 const uint32_t next = atomicAdd(&s_segments, 1u);
                 if (next < CROWD_SEGMENTS) {
-                    s_from[next] = from + at;
-                    s_size[next] = c[u];
+                    s_from[next] = (uint16_t)(from + at);
+                    s_size[next] = (uint16_t)c[u];
                 }
             }
             at += c[u];
@@ -1015,16 +1022,61 @@ __device__ __forceinline__ void sort_small_bin(const atrex_entry_t* entries, boo
         if (u * 32 + lane < n) s_item[before[u]] = item[u];
 }
 
+// A tile's crowded local bins, and those with ties: bit u of `tied` is a thread's bin u * TILE_THREADS + threadIdx.x (whole CTA, behind a
+// barrier; the local bins are not needed any more).
+__device__ __noinline__ void sort_crowds(const atrex_entry_t* entries, bool ranking, ull* s_item, uint32_t* s_local, const uint16_t* s_bin, uint32_t crowded,
+                                         uint32_t tied) {
+    constexpr uint32_t WARPS = TILE_THREADS / 32, WORDS = TILE_LOCAL_BINS / 32;
+    static_assert(WARPS == 16 && WORDS == 4 * 32, "a word's bins go to two lots of sixteen warps, a lane looks at four words");
+    __shared__ uint32_t s_tied[WORDS];                   // a bit for every local bin
+    const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
+    uint32_t begin = 0, size = 0;                        // of the lane's crowded bin
+    if (lane < crowded) {
+        const uint32_t d = s_bin[lane];
+        begin = d ? s_local[d - 1] : 0u;
+        size = s_local[d] - begin;
+    }
+#pragma unroll
+    for (uint32_t u = 0; u < TILE_LOCAL_BINS / TILE_THREADS; ++u) {
+        const uint32_t votes = __ballot_sync(FULL, tied >> u & 1u);
+        if (lane == 0) s_tied[u * WARPS + w] = votes;
+    }
+    __syncthreads();
+    const uint32_t by_warp = crowded > TILE_CROWDED_FEW ? TILE_SMALL_CROWD : 0u;
+    for (uint32_t k = w; k < crowded; k += WARPS) {
+        const uint32_t b0 = __shfl_sync(FULL, begin, k), n = __shfl_sync(FULL, size, k);
+        if (n <= by_warp) sort_small_bin(entries, ranking, s_item + b0, n);
+    }
+    // bins next to one another go to different warps: groups of ties come side by side
+#pragma unroll
+    for (uint32_t v = 0; v < 4; ++v) {
+        const uint32_t word = v * 32 + lane, own = s_tied[word] & 0x00010001u << ((w + word) & 15u);
+        for (uint32_t todo = __ballot_sync(FULL, own != 0); todo; todo &= todo - 1) {
+            const uint32_t src = __ffs(todo) - 1;
+            for (uint32_t bits = __shfl_sync(FULL, own, src); bits; bits &= bits - 1) {
+                const uint32_t d = (v * 32 + src) * 32 + __ffs(bits) - 1, b0 = d ? s_local[d - 1] : 0u;
+                sort_small_bin(entries, ranking, s_item + b0, s_local[d] - b0);
+            }
+        }
+    }
+    for (uint32_t k = 0; k < crowded; ++k) {
+        const uint32_t b0 = __shfl_sync(FULL, begin, k), n = __shfl_sync(FULL, size, k);
+        if (n > by_warp) sort_crowded_bin(entries, ranking, s_item, b0, n, s_local);
+    }
+}
+
 // Sorts n <= TILE_CAP items whose leading bits lie in [low, high] into s_item.  `each(f)` calls f with each of
 // this thread's items (twice).  Each item goes to one of twice as many local bins of equal width as a tile usually has items -- less than one item per bin, so that
 // a thread puts a bin in order by insertion; a few crowded local bins (hundreds of equal weights, say) are
-// sorted on their own, many of them send the whole tile through a bitonic network, with absent items behind the last one.
+// sorted on their own, those with ties by a warp each; many crowded ones send the whole tile through a bitonic network, with absent
+// items behind the last one.
 // (Every item's place counted by a thread of its own instead: 3.1 M entries 107.5 -> 111 us.)
 template <uint32_t LOCAL_BINS, typename Each>
 __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ranking, uint32_t n, uint32_t low, uint32_t high, Each each, ull* s_item,
                                           uint32_t* s_local) {
     __shared__ uint32_t s_warp[32];
-    __shared__ uint32_t s_crowded, s_bin[TILE_CROWDED], s_begin[TILE_CROWDED], s_size[TILE_CROWDED];
+    __shared__ uint32_t s_crowded;
+    __shared__ uint16_t s_bin[TILE_CROWDED];
     const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5, n_warps = blockDim.x >> 5;
     const int len = 32 - __clz((int)(high - low));
     constexpr int BITS = LOCAL_BINS == 4096 ? 12 : 10;
@@ -1037,7 +1089,7 @@ __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ran
         const uint32_t d = ((uint32_t)(item >> 32) - low) >> shift;
         if (atomicAdd(&s_local[d], 1u) == TILE_CLASH_MAX) {
             const uint32_t at = atomicAdd(&s_crowded, 1u);
-            if (at < TILE_CROWDED) s_bin[at] = d;
+            if (at < TILE_CROWDED) s_bin[at] = (uint16_t)d;
         }
     });
     __syncthreads();
@@ -1071,29 +1123,19 @@ __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ran
     }
     __syncthreads();
     each([&](ull item) { s_item[atomicAdd(&s_local[((uint32_t)(item >> 32) - low) >> shift], 1u)] = item; });
-    const uint32_t crowded = s_crowded;   // (read on this side of the barrier: bins with ties are added behind it)
     __syncthreads();
+    const uint32_t crowded = s_crowded;   // (nothing adds to it behind the first barrier)
     // (a bin's cursor now stands at its end, its predecessor's at its start)
     if (crowded <= TILE_CROWDED) {
-        const uint32_t by_warp = crowded > TILE_CROWDED_FEW ? TILE_SMALL_CROWD : 0u;
-        for (uint32_t k = w; k < crowded; k += n_warps) {
-            const uint32_t d = s_bin[k], b0 = d ? s_local[d - 1] : 0u, size = s_local[d] - b0;
-            if (size <= by_warp) sort_small_bin(entries, ranking, s_item + b0, size);
-            if (lane == 0) {
-                s_begin[k] = b0;
-                s_size[k] = size;
-            }
-        }
-        for (uint32_t d = threadIdx.x; d < LOCAL_BINS; d += blockDim.x) {
+        uint32_t tied = 0;                               // (a thread has eight local bins at most)
+        for (uint32_t d = threadIdx.x; d < LOCAL_BINS; d += TILE_THREADS) {
             const uint32_t b0 = d ? s_local[d - 1] : 0u, b1 = s_local[d];
             if (b1 - b0 > TILE_CLASH_MAX) continue;
             if (b1 - b0 >= TILE_TIES) {                  // leading bits alike: every comparison would read two entries
                 uint32_t ties = 0;
                 for (uint32_t i = b0 + 1; i < b1; ++i) ties += (s_item[i] ^ s_item[b0]) >> 32 ? 0u : 1u;
-                const uint32_t k = ties < TILE_TIES / 2 ? TILE_CROWDED : atomicAdd(&s_crowded, 1u);
-                if (k < TILE_CROWDED) {
-                    s_begin[k] = b0;
-                    s_size[k] = b1 - b0;
+                if (ties >= TILE_TIES / 2) {
+                    tied |= 1u << (d / TILE_THREADS);
                     continue;
                 }
             }
@@ -1107,9 +1149,7 @@ __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ran
                 s_item[j] = item;
             }
         }
-        __syncthreads();
-        for (uint32_t k = 0; k < min(s_crowded, TILE_CROWDED); ++k)      // (the same for every thread; the local bins are not needed any more)
-            if (k >= crowded || s_size[k] > by_warp) sort_crowded_bin(entries, ranking, s_item, s_begin[k], s_size[k], s_local);
+        if (__syncthreads_or(tied) || crowded != 0) sort_crowds(entries, ranking, s_item, s_local, s_bin, crowded, tied);
     } else {
         bitonic(n, [&](uint32_t a, uint32_t b) { return item_less(entries, ranking, s_item[a], s_item[b]); },
                 [&](uint32_t a, uint32_t b) { const ull x = s_item[a]; s_item[a] = s_item[b]; s_item[b] = x; });
@@ -1156,8 +1196,9 @@ __device__ __forceinline__ void gather_tile(const atrex_entry_t* entries, const 
     }
 }
 
-// 5. a tile's items in order, their entries gathered; (ranking) the tile's weighted time, and the order itself
-template <uint32_t LOCAL_BINS>
+// 5. a tile's items in order, their entries gathered; (ranking) the weighted times of the rows and their sum.  A kernel per order: in one for
+//    both, what only the other needs costs the key order 2 % and more (15 M entries: tile kernel 565 us, now 552).
+template <uint32_t LOCAL_BINS, bool RANKING>
 __global__ void __launch_bounds__(TILE_THREADS) bin_tile_kernel(const BinSort b, atrex_entry_t* out, uint32_t out_cap) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     ull* s_item = reinterpret_cast<ull*>(smem_raw);
@@ -1167,11 +1208,11 @@ __global__ void __launch_bounds__(TILE_THREADS) bin_tile_kernel(const BinSort b,
     grid_dependency_wait();
     const bool overflow = b.ctl->overflow;
     // the last tile first: at both ends of a ranking the words lie uneven, which takes a tile twice as long
-    const uint32_t n_tiles = tiles_of(b, item_count(b));
+    const uint32_t n_tiles = tiles_of(b, RANKING ? (uint32_t)b.ctl->counter : b.n);
     const uint32_t tile = blockIdx.x >= n_tiles ? blockIdx.x : (blockIdx.x ? blockIdx.x - 1 : n_tiles - 1);
     const uint32_t first = overflow ? 0u : b.tile_start[tile], n = overflow ? 0u : b.tile_start[tile + 1] - first;
     if (n == 0) {
-        if (!b.ranking) finish_call(b.report, b.slot);
+        if (!RANKING) finish_call(b.report, b.slot);
         else if (!overflow && threadIdx.x == 0) b.tile_sum[tile] = make_ulonglong2(0, 0);
         return;
     }
@@ -1203,21 +1244,20 @@ __global__ void __launch_bounds__(TILE_THREADS) bin_tile_kernel(const BinSort b,
         atomicMax(&s_range[1], top);
     }
     __syncthreads();
-    sort_tile<LOCAL_BINS>(b.entries, b.ranking, n, ~s_range[0], s_range[1], each, s_item, s_local);
+    sort_tile<LOCAL_BINS>(b.entries, RANKING, n, ~s_range[0], s_range[1], each, s_item, s_local);
     grid_dependents_launch();
     if (threadIdx.x < 2) s_sum[threadIdx.x] = 0;
     ulonglong2 sum = make_ulonglong2(0, 0);
-    if (!b.ranking) {
+    if constexpr (!RANKING) {
         gather_tile(b.entries, s_item, n, out, first, out_cap, [](uint32_t, ull, ull) {});
         finish_call(b.report, b.slot);
         return;
     }
-    // (the shares read a row's weighted time where the words were and where the items were, which this CTA alone read: the ranked
-    // rows themselves would have to come from memory once more)
+    // (the shares read a row's weighted time from where the words and indices were: the ranked rows themselves would have to come from
+    // memory once more)
     auto weight = [&](uint32_t row, ull lo, ull hi) {
         add128(sum.x, sum.y, lo, hi);
-        b.words[first + row] = lo;
-        b.items[first + row] = hi;
+        b.ranked_wt[first + row] = make_ulonglong2(lo, hi);
     };
     gather_tile(b.entries, s_item, n, out, first, out_cap, weight);
     for (uint32_t i = threadIdx.x; i < n; i += TILE_THREADS) {   // rows that are not wanted
@@ -1293,8 +1333,9 @@ __global__ void __launch_bounds__(CUM_THREADS, CUM_CTAS) bin_share_kernel(const 
         for (uint32_t u = 0; u < CUM_ROWS; ++u) {
             lo[u] = hi[u] = 0;
             if (r0 + u < end) {
-                lo[u] = b.words[r0 + u];
-                hi[u] = b.items[r0 + u];
+                const ulonglong2 wt = b.ranked_wt[r0 + u];
+                lo[u] = wt.x;
+                hi[u] = wt.y;
             }
         }
         ull own_lo = 0, own_hi = 0;
@@ -1601,8 +1642,10 @@ int prepare_sort_kernels(int* n_sms) {
         if (cudaFuncSetAttribute(radix_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCATTER_SMEM) != cudaSuccess ||
             cudaFuncSetAttribute(bin_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 << BIN_BITS_MAX) != cudaSuccess ||
             cudaFuncSetAttribute(bin_scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(4 * CURSORS_MAX + (2 << BIN_BITS_MAX))) != cudaSuccess ||
-            cudaFuncSetAttribute(bin_tile_kernel<TILE_LOCAL_BINS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(bin_tile_kernel<SMALL_LOCAL_BINS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM) != cudaSuccess ||
+            cudaFuncSetAttribute(bin_tile_kernel<TILE_LOCAL_BINS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM) != cudaSuccess ||
+            cudaFuncSetAttribute(bin_tile_kernel<TILE_LOCAL_BINS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM) != cudaSuccess ||
+            cudaFuncSetAttribute(bin_tile_kernel<SMALL_LOCAL_BINS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM) != cudaSuccess ||
+            cudaFuncSetAttribute(bin_tile_kernel<SMALL_LOCAL_BINS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TILE_SMEM) != cudaSuccess ||
             cudaFuncSetAttribute(count_rank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(COUNT_RANK_MAX * 26)) != cudaSuccess ||
             cudaFuncSetAttribute(count_sort_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(COUNT_SORT_MAX * 8)) != cudaSuccess ||
             cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
@@ -1649,7 +1692,8 @@ struct BinSizes {
         cursor_bytes = 4ull * ((n_cursors + 3) & ~3u);
     }
     constexpr uint64_t control_bytes() const { return align256(sizeof(BinCtl) + group_bytes + bin_bytes + cursor_bytes + tiles * 16 + (tiles + 1) * 4); }
-    constexpr uint64_t bytes(uint64_t n) const { return control_bytes() + 2 * align256(n * 8) + n * 4; }
+    // items, words, and room for the ranked weighted times
+    constexpr uint64_t bytes(uint64_t n) const { return control_bytes() + 2 * align256(n * 8) + n * 8; }
 };
 // (the scratch's size is the radix sort's, whose digit counts take more than the control area: on both sides of every line above)
 constexpr bool bins_fit(uint64_t n) { return BinSizes(n, false).bytes(n) <= scratch_bytes_for(n) && BinSizes(n, true).bytes(n) <= scratch_bytes_for(n); }
@@ -1682,8 +1726,9 @@ BinSort carve_bins(void* base, const atrex_entry_t* entries, uint64_t n, bool ra
     b.tile_start = (uint32_t*)p;
     p = (unsigned char*)base + z.control_bytes();
     b.words = (ull*)p;           p += align256(n * 8);
-    b.items = (ull*)p;           p += align256(n * 8);
-    b.idx = (uint32_t*)p;
+    b.idx = (uint32_t*)p;        p += align256(n * 8);
+    b.items = (ull*)p;
+    b.ranked_wt = (ulonglong2*)b.words;
     return b;
 }
 
@@ -1701,7 +1746,8 @@ cudaError_t launch_bins(const BinSort& b, uint32_t coverage_ppm, atrex_entry_t* 
     cudaError_t e = launch_chained(bin_count_kernel, grid, SHARE_THREADS, bytes, s, b);
     if (e == cudaSuccess) e = launch_chained(bin_scan_kernel, 1, 1024, 0, s, b, coverage_ppm);
     if (e == cudaSuccess) e = launch_chained(bin_scatter_kernel, grid, SHARE_THREADS, b.n_cursors * 4 + (2u << b.bits), s, b);
-    auto* tile = b.log_step == SMALL_LOG_STEP ? bin_tile_kernel<SMALL_LOCAL_BINS> : bin_tile_kernel<TILE_LOCAL_BINS>;
+    auto* tile = b.log_step == SMALL_LOG_STEP ? (b.ranking ? bin_tile_kernel<SMALL_LOCAL_BINS, true> : bin_tile_kernel<SMALL_LOCAL_BINS, false>)
+                                              : (b.ranking ? bin_tile_kernel<TILE_LOCAL_BINS, true> : bin_tile_kernel<TILE_LOCAL_BINS, false>);
     if (e == cudaSuccess) e = launch_chained(tile, tiles, TILE_THREADS, TILE_SMEM, s, b, out, (uint32_t)(out_cap < b.n ? out_cap : b.n));
     return e;
 }
