@@ -427,9 +427,11 @@ constexpr uint32_t SHARE_THREADS = 1024;     // counting and moving: one CTA per
 constexpr uint32_t CURSORS_MAX = 1u << 14;
 // A tile is the bins that start in one window of 2^log_step positions: 2 048, or 512 where a list is so short that larger tiles would
 // leave SMs without one and make every phase of a tile's sort longer (tile kernel, key order of 10 000 entries 12.7 -> 7.9 us, 150 000
-// 13.5 -> 9.3, 250 000 13.2 -> 15.4; one phase of two, 75 000 entries 27.9 -> 12.7, 250 000 25.5 -> 14.0, 400 000 no change in all).
-constexpr uint32_t TILE_LOG_STEP = 11, SMALL_LOG_STEP = 9;
-constexpr uint64_t SMALL_LIST_MAX = 150000, SMALL_RANKING_MAX = 300000;
+// 13.5 -> 9.3, 250 000 13.2 -> 15.4): up to there two tiles per SM are enough.  A ranking, of which the tiles of other phases are empty, takes windows of
+// 1 024 up to twice that (whole call with windows of 2 048 / 1 024 / 512: 155 000 entries of one phase 62 / 57 / 61 us, 250 000 62 / 60 / 66, 299 000
+// 66 / 63 / 70; a phase of two of 250 000 62 / 55 / 59; from 310 000 on no better than 2 048).
+constexpr uint32_t TILE_LOG_STEP = 11, MIDDLE_LOG_STEP = 10, SMALL_LOG_STEP = 9;
+constexpr uint64_t SMALL_LIST_MAX = 150000, MIDDLE_RANKING_MAX = 300000;
 constexpr uint32_t TILE_GROUP = 64;         // tiles whose weighted times are summed
 constexpr uint32_t TILE_CAP = 6144;         // ... and has at most this many items
 constexpr uint32_t TILE_LOCAL_BINS = 4096, SMALL_LOCAL_BINS = 1024, TILE_THREADS = 512, TILE_HELD = 5, GATHER_LOADS = 6;
@@ -1066,7 +1068,7 @@ __device__ __noinline__ void sort_crowds(const atrex_entry_t* entries, bool rank
 }
 
 // Sorts n <= TILE_CAP items whose leading bits lie in [low, high] into s_item.  `each(f)` calls f with each of
-// this thread's items (twice).  Each item goes to one of twice as many local bins of equal width as a tile usually has items -- less than one item per bin, so that
+// this thread's items (twice).  Each item goes to one of as many local bins of equal width as a tile usually has items, or twice as many, so that
 // a thread puts a bin in order by insertion; a few crowded local bins (hundreds of equal weights, say) are
 // sorted on their own, those with ties by a warp each; many crowded ones send the whole tile through a bitonic network, with absent
 // items behind the last one.
@@ -1681,11 +1683,11 @@ struct BinSizes {
     bool by_tile;
     uint64_t tiles, group_bytes, bin_bytes, cursor_bytes;
     constexpr BinSizes(uint64_t n, bool ranking)
-        : log_step(n <= (ranking ? SMALL_RANKING_MAX : SMALL_LIST_MAX) ? SMALL_LOG_STEP : TILE_LOG_STEP), bits(4), n_cursors(0), by_tile(false),
+        : log_step(n <= SMALL_LIST_MAX ? SMALL_LOG_STEP : ranking && n <= MIDDLE_RANKING_MAX ? MIDDLE_LOG_STEP : TILE_LOG_STEP), bits(4), n_cursors(0), by_tile(false),
           tiles((n + (1ull << log_step) - 1) >> log_step), group_bytes(ranking ? (tiles + TILE_GROUP - 1) / TILE_GROUP * 16 : 0), bin_bytes(0), cursor_bytes(0) {
         // about 256 items per bin, a thousand beyond 2^12 bins (more open ranges than that cost the scattered writes), 64 or
         // 128 for small tiles
-        while (bits < BIN_BITS_MAX && ((log_step == SMALL_LOG_STEP ? (n <= 65536 ? 64ull : 128ull) : bits < 12 ? 256ull : 1024ull) << bits) < n) ++bits;
+        while (bits < BIN_BITS_MAX && ((log_step < TILE_LOG_STEP ? (n <= 65536 ? 64ull : 128ull) : bits < 12 ? 256ull : 1024ull) << bits) < n) ++bits;
         by_tile = tiles <= CURSORS_MAX;
         n_cursors = by_tile ? (uint32_t)tiles : 1u << bits;
         bin_bytes = 4ull << bits;
@@ -1698,7 +1700,7 @@ struct BinSizes {
 // (the scratch's size is the radix sort's, whose digit counts take more than the control area: on both sides of every line above)
 constexpr bool bins_fit(uint64_t n) { return BinSizes(n, false).bytes(n) <= scratch_bytes_for(n) && BinSizes(n, true).bytes(n) <= scratch_bytes_for(n); }
 static_assert(bins_fit(1) && bins_fit(COUNT_RANK_MAX + 1) && bins_fit(COUNT_SORT_MAX + 1) && bins_fit(65536) && bins_fit(65537) && bins_fit(SMALL_LIST_MAX) &&
-                  bins_fit(SMALL_LIST_MAX + 1) && bins_fit(SMALL_RANKING_MAX) && bins_fit(SMALL_RANKING_MAX + 1) && bins_fit(1u << 20) && bins_fit((1u << 20) + 1) &&
+                  bins_fit(SMALL_LIST_MAX + 1) && bins_fit(MIDDLE_RANKING_MAX) && bins_fit(MIDDLE_RANKING_MAX + 1) && bins_fit(1u << 20) && bins_fit((1u << 20) + 1) &&
                   bins_fit(1u << 22) && bins_fit((1u << 22) + 1) && bins_fit((uint64_t)CURSORS_MAX << TILE_LOG_STEP) &&
                   bins_fit(((uint64_t)CURSORS_MAX << TILE_LOG_STEP) + 1) && bins_fit(ATREX_RELEASE_MAX_ENTRIES), "the binned sort's use of the scratch");
 
@@ -1746,7 +1748,7 @@ cudaError_t launch_bins(const BinSort& b, uint32_t coverage_ppm, atrex_entry_t* 
     cudaError_t e = launch_chained(bin_count_kernel, grid, SHARE_THREADS, bytes, s, b);
     if (e == cudaSuccess) e = launch_chained(bin_scan_kernel, 1, 1024, 0, s, b, coverage_ppm);
     if (e == cudaSuccess) e = launch_chained(bin_scatter_kernel, grid, SHARE_THREADS, b.n_cursors * 4 + (2u << b.bits), s, b);
-    auto* tile = b.log_step == SMALL_LOG_STEP ? (b.ranking ? bin_tile_kernel<SMALL_LOCAL_BINS, true> : bin_tile_kernel<SMALL_LOCAL_BINS, false>)
+    auto* tile = b.log_step < TILE_LOG_STEP ? (b.ranking ? bin_tile_kernel<SMALL_LOCAL_BINS, true> : bin_tile_kernel<SMALL_LOCAL_BINS, false>)
                                               : (b.ranking ? bin_tile_kernel<TILE_LOCAL_BINS, true> : bin_tile_kernel<TILE_LOCAL_BINS, false>);
     if (e == cudaSuccess) e = launch_chained(tile, tiles, TILE_THREADS, TILE_SMEM, s, b, out, (uint32_t)(out_cap < b.n ? out_cap : b.n));
     return e;

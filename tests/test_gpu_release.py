@@ -321,3 +321,14 @@ def test_groups_of_ties_in_one_tile(lib, n, groups, size):
         assert host(ranked, lib.ENTRY_DTYPE).tobytes() == one[order].tobytes()
         exp_r, exp_c, exp_res = oracle.rank_phase(one, 0, 900_000)           # (equal rows are the same to sums and cut)
         assert res == exp_res and host(cum, np.float64).tobytes() == exp_c.tobytes()
+
+
+@pytest.mark.parametrize("n", [4_097, 8_193, 65_536, 65_537, 150_000, 150_001, 300_000, 300_001])
+@pytest.mark.parametrize("phases", [1, 3])
+def test_where_tiles_and_bins_change(lib, n, phases):
+    """Both sides of the sizes at which a list gets larger tiles or fewer bins, with the whole list in one phase and spread over three."""
+    e = synthetic_entries(7 * n + phases, n, phases, "wide")
+    d = dev(e)
+    assert host(lib.sort_entries_by_key(d, n), oracle.ENTRY_DTYPE).tobytes() == oracle.sort_by_key(e).tobytes()
+    check_rank(lib, e, d, n, range(phases), ppms=(900_000,))
+    check_rank(lib, e, d, n, (0,), ppms=(0,), out_cap=n // phases - 1000)
