@@ -86,9 +86,9 @@ __device__ __forceinline__ uint32_t approx_key(float r, const double* roofline, 
 // that bin's keys fit the lanes (two rounds for a thousand spread-out values), where they are ranked.
 // A range of one value ends the search as well, so ties cost nothing; each round narrows the range at
 // least 64-fold, so there are at most eleven.  K: 32- or 64-bit keys, all ones = no usable score.
-// `bins`: SELECT_BINS words of this warp's.
+// `bins`: SELECT_BINS words of this warp's.  (In place, or as a call.)
 template <typename K, typename KeyAt>
-__device__ __noinline__ void warp_select(KeyAt key_at, uint32_t g, uint32_t k, uint32_t* bins, K* out_k, K* out_next) {
+__device__ __forceinline__ void warp_select_here(KeyAt key_at, uint32_t g, uint32_t k, uint32_t* bins, K* out_k, K* out_next) {
     constexpr K NONE = ~(K)0;
     const uint32_t lane = threadIdx.x & 31u;
     K lo = NONE, hi = 0;
@@ -169,6 +169,11 @@ __device__ __noinline__ void warp_select(KeyAt key_at, uint32_t g, uint32_t k, u
         *out_next = k + 1 < n ? in_list : next_above;
     }
     __syncwarp();   // `bins` may be overwritten from here on
+}
+
+template <typename K, typename KeyAt>
+__device__ __noinline__ void warp_select(KeyAt key_at, uint32_t g, uint32_t k, uint32_t* bins, K* out_k, K* out_next) {
+    warp_select_here<K>(key_at, g, k, bins, out_k, out_next);
 }
 
 // The middle of one operator's keys, by one warp: number of usable units, the lower and upper middle keys (no
@@ -903,12 +908,12 @@ __global__ void __launch_bounds__(1024)
 // the key's range, a warp finds the range that holds the middle, and the few units in it (or as close to it as
 // keys may err) are ranked by their exact scores.  Every step but the finding is spread over the whole CTA, and units stay
 // where they are, so that nothing is worked out about the grouping.  Where the middle's range holds too many units it is
-// cut again; what stays too many (ties) is searched among them.  Bound by latency at 48 warps per SM (loads, shared-memory
-// atomics, barriers: 40 % of the issue slots).  1 000 candidates x 12 001 units x 7 operators: 145 us by score_cta_kernel, 78;
+// cut again; what stays too many (ties) is searched among them.  Bound by latency at 45 warps per SM (loads, shared-memory
+// atomics, barriers: 52 % of the issue slots).  1 000 candidates x 12 001 units x 7 operators: 145 us by score_cta_kernel, 78;
 // with the next loads issued before a thread's units are worked on 116 (spills); strides not known at compile time 86.
 constexpr uint32_t NEAR_MAX = 32;             // units near an operator's middle that one warp ranks, a lane each
 constexpr uint32_t BINS_LOW = (127u - 7u) << 23, BINS_LOG_SPAN = 26;   // first cut: scores from 2^-7 to 2, what lies outside in the end bins
-constexpr uint32_t CUTS_MAX = 6;              // (each narrows the range 32-fold or more)
+constexpr uint32_t CUTS_MAX = 6;              // (each narrows the range 32-fold or more where the middles are in one range or two that touch)
 constexpr uint32_t NOWHERE = 0xFFFFFFFFu;     // no key is as close above it
 
 struct BinsLayout {
@@ -960,16 +965,97 @@ __device__ __forceinline__ Bin find_bin(const uint32_t* words, uint32_t W, uint3
     return {src * 2 * W + in, base + __shfl_sync(FULL, upto - c, in), __shfl_sync(FULL, c, in)};
 }
 
+struct BinsArgs {             // what the search of a candidate needs
+    const double *roofline_s, *t_cand, *w;
+    double* s_op_out;
+    uint32_t n_units, n_ops, log_bins;
+};
+
+// An operator that is searched, in its part of the list of units near the middles: where its units start, how many are in place, how
+// many of them lie below the middle's range.
+struct Segment {
+    uint32_t first, placed, below, pad;
+};
+// The operators whose middles their keys do not tell, by exact scores: of the units in their windows, or of all.  The units are brought
+// together by operator first (their numbers, where the keys were), so that a warp goes over its operator's units only: 5 000 candidates x 700
+// units x 10 operators, scores alike in their keys 614 -> 239 us, 1 000 x 12 001 x 7 of two values 4 840 -> 733, 1 500 x 16 320 x 255 14.8 -> 1.2 ms (every
+// warp over all units before; in place, as a call in the loop over candidates costs 2 to 4 % where nothing is searched).
+// (Whole CTA, behind a barrier and with one at its end.  searched: {any operator is, their units}, both 0 again at the end)
+template <int THREADS>
+__device__ __forceinline__ void search_operators(const BinsArgs& a, uint32_t cand, uint32_t* searched) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const uint32_t n_units = a.n_units, n_ops = a.n_ops;
+    const double *roofline_s = a.roofline_s, *t = a.t_cand + (size_t)cand * n_units;
+    const BinsLayout L(n_units, n_ops, a.log_bins, THREADS);
+    uint32_t *keys = reinterpret_cast<uint32_t*>(smem_raw), *flags = reinterpret_cast<uint32_t*>(smem_raw + L.bins);   // a bit per unit, in the
+    // counters' place (all 0 here; they are n / 8 words at least, or 512)
+    uint4* state = reinterpret_cast<uint4*>(smem_raw + L.state);
+    const uint2* window = reinterpret_cast<const uint2*>(smem_raw + L.window);
+    const uint8_t* ops = smem_raw + L.op;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, n_warps = THREADS / 32;
+    auto segment = [&](uint32_t op) { return reinterpret_cast<Segment*>(smem_raw + L.list) + op * (2 * NEAR_MAX / sizeof(Segment)); };
+    uint32_t* listed = reinterpret_cast<uint32_t*>(smem_raw + L.listed);
+    for (uint32_t op = threadIdx.x; op < n_ops; op += THREADS)
+        if (state[op].w >= GO_SEARCH) *segment(op) = Segment{atomicAdd(&searched[1], listed[op]), 0, 0, 0};
+    __syncthreads();
+    for (uint32_t j0 = warp * 32; j0 < n_units; j0 += THREADS) {
+        const uint32_t j = j0 + lane, op = j < n_units ? ops[j] : n_ops;
+        bool in = false;
+        if (op < n_ops && state[op].w >= GO_SEARCH) {
+            const uint32_t key = keys[j];
+            const uint2 win = window[op];
+            in = key - win.x <= win.y;
+            if (in && state[op].w == GO_SEARCH && key < state[op].x) atomicAdd(&segment(op)->below, 1u);
+        }
+        const uint32_t votes = __ballot_sync(FULL, in);
+        if (lane == 0) flags[j0 / 32] = votes;
+    }
+    __syncthreads();
+    uint16_t* units = reinterpret_cast<uint16_t*>(keys);
+    for (uint32_t j = threadIdx.x; j < n_units; j += THREADS) {
+        if (!(flags[j / 32] >> (j % 32) & 1u)) continue;
+        Segment* s = segment(ops[j]);
+        units[s->first + atomicAdd(&s->placed, 1u)] = (uint16_t)j;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) searched[0] = searched[1] = 0;
+    for (uint32_t i = threadIdx.x; i < (n_units + 31) / 32; i += THREADS) flags[i] = 0;
+    for (uint32_t op = warp; op < n_ops; op += n_warps) {
+        const uint4 st = state[op];
+        if (st.w < GO_SEARCH) continue;
+        const Segment g = *segment(op);
+        const uint32_t usable = st.w == GO_SEARCH_ALL ? g.placed : st.z, below = st.w == GO_SEARCH_ALL ? 0u : st.y - g.below;
+        const uint16_t* own = units + g.first;
+        auto key_at = [=](uint32_t i) {
+            const uint32_t j = own[i];
+            return exact_key(__ldg(roofline_s + j), __ldg(t + j), true);
+        };
+        ull k_lo, k_hi;
+        warp_select_here<ull>(key_at, g.placed, (usable - 1) / 2 - below, reinterpret_cast<uint32_t*>(smem_raw + L.spare) + warp * SELECT_BINS, &k_lo, &k_hi);
+        if (lane == 0) {
+            const double s = median_of_keys(k_lo, (usable & 1u) ? k_lo : k_hi, usable & 1u);
+            reinterpret_cast<double*>(smem_raw + L.prod)[op] = __dmul_rn(a.w[op], s);
+            if (a.s_op_out) a.s_op_out[(size_t)cand * n_ops + op] = s;
+            listed[op] = 0;
+            state[op].w = GO_NONE;
+        }
+    }
+    __syncthreads();
+}
+
 constexpr int bins_ctas(int threads) { return threads == 1024 ? 1 : 1536 / threads; }   // per SM, by registers
 template <int THREADS>
 __global__ void __launch_bounds__(THREADS, bins_ctas(THREADS))
     score_bins_kernel(const double* __restrict__ roofline_s, const uint32_t* __restrict__ unit_op, uint32_t n_units,
                       const double* __restrict__ t_cand, const uint8_t* __restrict__ correct, uint32_t n_cand,
                       const double* __restrict__ w, uint32_t n_ops, uint32_t log_bins, double* s_agg, double* s_op_out, ull* errors_out) {
+    __shared__ BinsArgs s_args;                                          // (for the search: held in registers for it they cost 1 to 2 % where nothing is searched)
+    if (threadIdx.x == 0) s_args = BinsArgs{roofline_s, t_cand, w, s_op_out, n_units, n_ops, log_bins};
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint32_t s_errors[2];
     constexpr uint32_t U = 4;                                            // units of a thread in flight
     __shared__ uint32_t s_cut;                                           // round of cuts that is still wanted
+    __shared__ uint32_t s_searched[2];                                   // (see search_operators)
     const BinsLayout L(n_units, n_ops, log_bins, THREADS);
     uint32_t* keys = reinterpret_cast<uint32_t*>(smem_raw);
     uint4* state = reinterpret_cast<uint4*>(smem_raw + L.state);
@@ -979,7 +1065,6 @@ __global__ void __launch_bounds__(THREADS, bins_ctas(THREADS))
     uint32_t* listed = reinterpret_cast<uint32_t*>(smem_raw + L.listed);
     uint16_t* list = reinterpret_cast<uint16_t*>(smem_raw + L.list);
     uint8_t* ops = smem_raw + L.op;                                      // n_ops: none
-    uint32_t* spare = reinterpret_cast<uint32_t*>(smem_raw + L.spare) + (threadIdx.x >> 5) * SELECT_BINS;
     const uint32_t warp = threadIdx.x >> 5, lane = threadIdx.x & 31u, n_warps = THREADS / 32;
     const uint32_t n_bins = 1u << log_bins, op_words = n_bins / 2, W = op_words / 32, first_shift = BINS_LOG_SPAN - log_bins;
     for (uint32_t j = threadIdx.x; j < n_units; j += THREADS) {
@@ -992,7 +1077,7 @@ __global__ void __launch_bounds__(THREADS, bins_ctas(THREADS))
         state[i].w = GO_NONE;
     }
     if (threadIdx.x == 0) {
-        s_errors[0] = s_errors[1] = s_cut = 0;
+        s_errors[0] = s_errors[1] = s_cut = s_searched[0] = s_searched[1] = 0;
         window[n_ops] = make_uint2(NOWHERE, 0);                          // (units without an operator)
     }
     __syncthreads();
@@ -1060,7 +1145,9 @@ __global__ void __launch_bounds__(THREADS, bins_ctas(THREADS))
                     m = st.z;
                 }
                 uint2 win = make_uint2(NOWHERE, 0);
-                if (st.w != GO_SEARCH_ALL) {
+                if (st.w == GO_SEARCH_ALL) {
+                    win = make_uint2(0, K_UNKNOWN);
+                } else {
                     st = make_uint4(0, 0, m, GO_NONE);
                     if (m != 0) {
                         const Bin low = find_bin(words, W, incl, own, (m - 1) / 2 - below);
@@ -1134,23 +1221,13 @@ __global__ void __launch_bounds__(THREADS, bins_ctas(THREADS))
                 const ull k_lo = __shfl_sync(FULL, x, __ffs(__ballot_sync(FULL, lane < n && less <= kl && kl < leq)) - 1);
                 const ull k_hi = __shfl_sync(FULL, x, __ffs(__ballot_sync(FULL, lane < n && less <= ku && ku < leq)) - 1);
                 s = median_of_keys(k_lo, k_hi, m & 1u);
-            } else if (st.w != GO_NONE) {
-                // too many units alike, or units whose keys say nothing: exact scores of those near the middle, or of all
-                const bool all = st.w == GO_SEARCH_ALL;
-                const uint2 win = window[op];
-                auto key_at = [=](uint32_t j) {
-                    const uint32_t key = keys[j];
-                    const bool in = ops[j] == op && (all ? key != K_ABSENT : key < K_UNKNOWN && key - win.x <= win.y);
-                    return in ? exact_key(__ldg(roofline_s + j), __ldg(t + j), true) : ~0ull;
-                };
-                uint32_t counted = 0;      // all: the usable units; else the listed ones below the middle's range
-                for (uint32_t j = lane; j < n_units; j += 32)
-                    if (ops[j] == op) counted += all ? (keys[j] != K_ABSENT ? 1u : 0u) : (keys[j] - win.x <= win.y && keys[j] < st.x ? 1u : 0u);
-                counted = __reduce_add_sync(FULL, counted);
-                const uint32_t usable = all ? counted : m, below = all ? 0u : st.y - counted;
-                ull k_lo, k_hi;
-                warp_select<ull>(key_at, n_units, (usable - 1) / 2 - below, spare, &k_lo, &k_hi);
-                s = median_of_keys(k_lo, (usable & 1u) ? k_lo : k_hi, usable & 1u);
+            } else if (st.w != GO_NONE) {            // too many units alike, or units whose keys say nothing
+                __syncwarp();
+                if (lane == 0) {
+                    state[op].w = max(st.w, GO_SEARCH);
+                    s_searched[0] = 1;
+                }
+                continue;
             }
             __syncwarp();
             if (lane == 0) {
@@ -1161,6 +1238,7 @@ __global__ void __launch_bounds__(THREADS, bins_ctas(THREADS))
             }
         }
         __syncthreads();
+        if (s_searched[0] != 0) search_operators<THREADS>(s_args, cand, s_searched);
         if (threadIdx.x == 0) {   // (the others go on to the next candidate: nothing of this is touched before two more barriers)
             double agg = 0.0;     // Eq. 6 in operator order
 #pragma unroll 4
@@ -1306,7 +1384,7 @@ extern "C" int atrex_score_aggregate(const double* d_roofline_s, const uint32_t*
         const uint32_t threads = bins_threads(n, n_ops, b, sms), log_bins = log_bins_for(n, n_ops);
         const size_t smem = BinsLayout(n, n_ops, log_bins, threads).total;
         auto* kernel = threads == 128 ? score_bins_kernel<128> : threads == 256 ? score_bins_kernel<256> : threads == 512 ? score_bins_kernel<512> : score_bins_kernel<1024>;
-        per_sm = (uint32_t)(SM_SMEM / (smem + 1024 + 16));
+        per_sm = (uint32_t)(SM_SMEM / (smem + 1024 + 64));
         if (per_sm > (uint32_t)bins_ctas((int)threads)) per_sm = (uint32_t)bins_ctas((int)threads);
         if (per_sm < 1) per_sm = 1;
         kernel<<<b < sms * per_sm ? b : sms * per_sm, threads, smem, (cudaStream_t)stream>>>(

@@ -138,3 +138,29 @@ def test_score_parity_by_counting(n_units, n_ops, batch, law):
     assert got[0].tobytes() == exp[0].tobytes()
     assert got[1].tobytes() == exp[1].tobytes()
     assert np.array_equal(got[2], exp[2])
+
+
+@pytest.mark.parametrize("n_units,n_ops,batch", [(64, 1, 2_000), (700, 10, 2_000), (1_001, 15, 1_500), (4_001, 31, 700), (16_320, 255, 3), (16_384, 1, 3)])
+def test_score_parity_where_operators_are_searched(n_units, n_ops, batch):
+    """Operators whose keys do not tell the middle beside others of the same candidate, and candidates without any behind them: per operator
+    and candidate, scores spread out, all alike, alike in their leading bits, of two values, or with one outside binary32."""
+    rng = np.random.default_rng(n_units + n_ops)
+    unit_op = rng.integers(0, n_ops, n_units).astype(np.uint32)
+    roof = np.exp(rng.uniform(np.log(1e-6), np.log(1e-1), n_units))
+    law = rng.integers(0, 5, (batch, n_ops))
+    law[::3] = 0
+    law = law[:, unit_op]
+    score = rng.uniform(0.01, 1.02, (batch, n_units))
+    score = np.where(law == 1, 0.25, score)
+    score = np.where(law == 2, 0.3 * (1 + np.floor(score * 4096) * 2.0 ** -34), score)
+    score = np.where(law == 3, np.where(score < 0.5, 0.01, 0.9), score)
+    t = roof[None, :] / score
+    t[law == 1] = np.broadcast_to(4.0 * roof, t.shape)[law == 1]         # (exactly one score)
+    t[:, ::61] *= np.where(law[:, ::61] == 4, 2.0 ** -300, 1.0)
+    ok = rng.random((batch, n_units)) < 0.8
+    w = rng.dirichlet(np.ones(n_ops))
+    exp = oracle.score_candidates(roof, unit_op, t, ok, w)
+    got = run_gpu(roof, unit_op, t, ok, w)
+    assert got[0].tobytes() == exp[0].tobytes()
+    assert got[1].tobytes() == exp[1].tobytes()
+    assert np.array_equal(got[2], exp[2])
