@@ -913,7 +913,7 @@ __global__ void __launch_bounds__(1024)
 // with the next loads issued before a thread's units are worked on 116 (spills); strides not known at compile time 86.
 constexpr uint32_t NEAR_MAX = 32;             // units near an operator's middle that one warp ranks, a lane each
 constexpr uint32_t BINS_LOW = (127u - 7u) << 23, BINS_LOG_SPAN = 26;   // first cut: scores from 2^-7 to 2, what lies outside in the end bins
-constexpr uint32_t CUTS_MAX = 6;              // (each narrows the range 32-fold or more where the middles are in one range or two that touch)
+constexpr uint32_t CUTS_MAX = 6;              // (each narrows the range sevenfold or more, 32-fold where the middles are in one range or two that touch)
 constexpr uint32_t NOWHERE = 0xFFFFFFFFu;     // no key is as close above it
 
 struct BinsLayout {
@@ -1160,7 +1160,8 @@ __global__ void __launch_bounds__(THREADS, bins_ctas(THREADS))
                         st.x = from;
                         st.y = below + low.before;
                         const uint32_t in = up.before + up.n - low.before;
-                        st.w = in <= NEAR_MAX ? GO_RANK : (shift == 0 || round == CUTS_MAX ? GO_SEARCH : GO_CUT);
+                        const bool far = (up.at - low.at) * 8 > n_bins;          // two middles that a cut would only trim the outsides of
+                        st.w = in <= NEAR_MAX ? GO_RANK : (shift == 0 || round == CUTS_MAX || far ? GO_SEARCH : GO_CUT);
                         if (st.w == GO_CUT) {
                             const int len = 32 - __clz((int)(to - from));
                             win = make_uint2(from, len > (int)log_bins ? len - log_bins : 0u);
