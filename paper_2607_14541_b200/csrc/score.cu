@@ -1282,11 +1282,14 @@ uint32_t cta_threads(uint32_t n, uint32_t n_ops, uint32_t b, uint32_t sms) {
     return n <= 30 * n_ops && (n <= 800 || b <= 8 * sms) ? 128u : 256u;
 }
 
-// One candidate per CTA by counting (score_bins_kernel), from groups of 64 units on in the mean: there it is the fastest for
-// every number of candidates (us, counting / the better of the other two: 6 000 units in 90 operators, 600 candidates 60 / 69,
-// 5 000 387 / 421; 700 in 10, 1 500 22.5 / 26.6; 12 001 in 7, 1 000 78 / 145), below, its two steps of a warp per operator
+// One candidate per CTA by counting (score_bins_kernel), from groups of 64 units on in the mean (us, counting / the better of
+// the other two: 6 000 units in 90 operators, 600 candidates 60 / 69, 5 000 387 / 421; 700 in 10, 1 500 22.5 / 26.6; 12 001 in 7, 1 000
+// 78 / 145; but 1 000 in 15, 5 000 78 / 74); below, its two steps of a warp per operator
 // outweigh what it saves (6 000 in 150, 500 candidates 73 / 78; 8 000 in 200, 3 000 487 / 438; 3 000 in 300, 5 000 950 / 226).
-constexpr uint32_t BINS_GROUP_MIN = 64;
+// Up to 500 units, a warp per candidate is quicker once it is by_warps' choice (100 in 1, 20 000 candidates 57 / 35, 100 000 268 / 141; 200 in 2,
+// 13 000 49 / 39; 300 in 4, 45 000 209 / 196; 500 in 2, 13 000 69 / 55, in 7, 45 000 338 / 311, though 4 500 39 / 47; scores alike in their keys, 500 in
+// 7, 13 000 482 / 234), and not above (550 in 2, 13 000 66 / 74, in 7 100 / 104; 600 in 4, 20 000 122 / 130).
+constexpr uint32_t BINS_GROUP_MIN = 64, BINS_UNITS_FEW = 500;
 constexpr uint32_t BINS_OPS_MAX = 255;        // (a unit's operator is kept in a byte, n_ops where it has none)
 
 // Its threads.  A candidate's latency falls with the threads as long as SMs would idle; with several candidates per SM, CTAs
@@ -1381,7 +1384,8 @@ extern "C" int atrex_score_aggregate(const double* d_roofline_s, const uint32_t*
         if (k * c > warps * per_sm) warps = k, per_sm = c;
     }
     const uint32_t sms = (uint32_t)n_sms, held = warps * per_sm;
-    if (n >= BINS_GROUP_MIN * n_ops && n_ops <= BINS_OPS_MAX) {
+    const bool warp_each = by_warps(n, n_ops, b, sms, held) && slots + n < SLOT_MASK;
+    if (n >= BINS_GROUP_MIN * n_ops && n_ops <= BINS_OPS_MAX && !(warp_each && n <= BINS_UNITS_FEW)) {
         const uint32_t threads = bins_threads(n, n_ops, b, sms), log_bins = log_bins_for(n, n_ops);
         const size_t smem = BinsLayout(n, n_ops, log_bins, threads).total;
         auto* kernel = threads == 128 ? score_bins_kernel<128> : threads == 256 ? score_bins_kernel<256> : threads == 512 ? score_bins_kernel<512> : score_bins_kernel<1024>;
@@ -1390,7 +1394,7 @@ extern "C" int atrex_score_aggregate(const double* d_roofline_s, const uint32_t*
         if (per_sm < 1) per_sm = 1;
         kernel<<<b < sms * per_sm ? b : sms * per_sm, threads, smem, (cudaStream_t)stream>>>(
             d_roofline_s, d_unit_op, n, d_t_cand, d_correct, b, d_w, n_ops, log_bins, d_s_agg, d_s_op, errors);
-    } else if (by_warps(n, n_ops, b, sms, held) && slots + n < SLOT_MASK) {
+    } else if (warp_each) {
         const uint32_t want = (b + warps - 1) / warps, most = (uint32_t)n_sms * per_sm;
         const size_t warp_smem = wl.warps + (size_t)wl.warp_bytes * warps;
         auto* kernel = pairs ? score_warp_kernel<true> : score_warp_kernel<false>;

@@ -164,3 +164,22 @@ def test_score_parity_where_operators_are_searched(n_units, n_ops, batch):
     assert got[0].tobytes() == exp[0].tobytes()
     assert got[1].tobytes() == exp[1].tobytes()
     assert np.array_equal(got[2], exp[2])
+
+
+@pytest.mark.parametrize("batch", [2_367, 2_368])
+@pytest.mark.parametrize("n_units,n_ops", [(64, 1), (500, 1), (500, 7), (501, 7)])
+def test_score_parity_between_counting_and_warps(n_units, n_ops, batch):
+    """Large groups of few units: a CTA per candidate that counts them, or from 16 candidates per SM on a warp."""
+    rng = np.random.default_rng(n_units + batch)
+    unit_op = rng.integers(0, n_ops, n_units).astype(np.uint32)
+    roof = np.exp(rng.uniform(np.log(1e-6), np.log(1e-1), n_units))
+    t = roof[None, :] / rng.uniform(0.01, 1.02, (batch, n_units))
+    t[0::5] = roof / np.round(rng.uniform(0.1, 1.0, n_units), 1)          # ties
+    t[1::7] = roof / (0.3 * (1 + rng.integers(0, 1 << 12, n_units) * 2.0 ** -34))
+    ok = rng.random((batch, n_units)) < 0.8
+    w = rng.dirichlet(np.ones(n_ops))
+    exp = oracle.score_candidates(roof, unit_op, t, ok, w)
+    got = run_gpu(roof, unit_op, t, ok, w)
+    assert got[0].tobytes() == exp[0].tobytes()
+    assert got[1].tobytes() == exp[1].tobytes()
+    assert np.array_equal(got[2], exp[2])
