@@ -598,7 +598,7 @@ __global__ void __launch_bounds__(BIN_THREADS) bin_keys_kernel(const BinSort b) 
 
 // 1b. (ranking) the phase's entries: words and indices side by side in any order, word range, exact total.  Bound by the entries' DRAM
 //     reads, 4.4 TB/s (weights asked for once the phase was known: 3.1 M entries 38 us, now 34; 15 M 154, now 130; the next round's lines
-//     prefetched into L2 as well: 40 and 140).
+//     prefetched into L2 as well: 40 and 140; a list in key order, where most warps have nothing to take, one phase of eight of 12 M 100 and 100).
 __global__ void __launch_bounds__(BIN_THREADS) bin_phase_kernel(const BinSort b, uint32_t phase) {
     constexpr uint32_t PER = 4;
     __shared__ ull s_part[32];

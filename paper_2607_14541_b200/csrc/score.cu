@@ -14,7 +14,7 @@
 // that out once and then goes through its candidates.  Three kernels:
 //   score_warp_kernel  one candidate per warp, no barriers: many candidates of few units
 //   score_cta_kernel   one candidate per CTA: few candidates, or more units than a warp should hold
-//   score_bins_kernel  one candidate per CTA, no grouping: operators of 64 units and more
+//   score_bins_kernel  one candidate per CTA, no grouping: operators of 64 units and more, but for many candidates of up to 500 units
 // The kernel before these (one candidate per CTA, grouping redone for every candidate, exact scores ranked
 // against each other) was bound by its barriers and shared-memory atomics: 65 536 candidates x 440 units x
 // 30 operators in 594 us, 1 000 x 12 001 units x 7 operators in 1 179 us.

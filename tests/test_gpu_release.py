@@ -259,11 +259,11 @@ def test_equal_keys_keep_their_order(lib, n):
     assert host(lib.sort_entries_by_key(dev(e), n), oracle.ENTRY_DTYPE).tobytes() == e[np.argsort(e["key"], kind="stable")].tobytes()
 
 
-@pytest.mark.parametrize("n", [3_000, 9_001, 40_000, 700_001])
+@pytest.mark.parametrize("n", [3_000, 5_000, 9_001, 40_000, 700_001])
 @pytest.mark.parametrize("crowd", ["alike", "close", "alike and close", "alike, equal keys", "steps"])
 def test_crowded_weights(lib, n, crowd):
     """Hundreds to thousands of weights in one place of a wide scale: equal ones (their keys decide, or the input order), some that only
-    the last bits tell apart, both, and many values of a hundred equal ones each."""
+    the last bits tell apart, both, and many values of a hundred equal ones each.  (3 000 entries are ranked by counting, the others in tiles.)"""
     rng = np.random.default_rng(n + len(crowd))
     e = np.zeros(n, dtype=oracle.ENTRY_DTYPE)
     e["key"] = rng.permutation(np.arange(n, dtype=np.uint64) * np.uint64(977))
@@ -332,3 +332,26 @@ def test_where_tiles_and_bins_change(lib, n, phases):
     assert host(lib.sort_entries_by_key(d, n), oracle.ENTRY_DTYPE).tobytes() == oracle.sort_by_key(e).tobytes()
     check_rank(lib, e, d, n, range(phases), ppms=(900_000,))
     check_rank(lib, e, d, n, (0,), ppms=(0,), out_cap=n // phases - 1000)
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 511, 512, 513, 4_096])
+@pytest.mark.parametrize("phases", [1, 5])
+def test_rankings_by_counting(lib, n, phases):
+    """Lists that one kernel ranks: equal weights, equal rows, 128-bit weights, phases in any order or one behind the other, few rows wanted."""
+    rng = np.random.default_rng(n + phases)
+    for sorted_phases in (False, True):
+        e = np.zeros(n, dtype=oracle.ENTRY_DTYPE)
+        phase = rng.integers(0, phases, n).astype(np.uint64)
+        e["key"] = (np.sort(phase) if sorted_phases else phase) << np.uint64(48) | rng.integers(0, max(2, n // 2), n).astype(np.uint64)
+        e["count"] = np.arange(n)
+        e["wt_lo"] = rng.integers(0, 4, n).astype(np.uint64) * np.uint64(1 << 62)
+        e["wt_hi"] = rng.integers(0, 3, n).astype(np.uint64) * np.uint64(1 << 30)
+        d = dev(e)
+        for p in range(phases):
+            for ppm, cap in [(0, None), (750_000, n // 2), (1_000_000, 1)]:
+                got_r, got_c, got_res = lib.rank_entries(d, n, p, ppm, out_cap=cap)
+                exp_r, exp_c, exp_res = oracle.rank_phase(e, p, ppm, out_cap=cap)
+                own = e[(e["key"] >> np.uint64(48)) == p]
+                order = np.lexsort((np.arange(len(own)), own["key"], ~own["wt_lo"], ~own["wt_hi"]))
+                assert got_res == exp_res and host(got_c, np.float64).tobytes() == exp_c.tobytes()
+                assert host(got_r, lib.ENTRY_DTYPE).tobytes() == own[order][:len(exp_c)].tobytes()
