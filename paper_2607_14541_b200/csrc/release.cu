@@ -874,7 +874,7 @@ __device__ __forceinline__ void bitonic(uint32_t n, Less less, Swap swap) {
 // of them at the clamp of their weights: the tile that held those went through a network as a whole, kernel 90 us, now 75 with the weighted
 // times written for the shares; 7.5 M rows, 7 500 of them: 572, now 367)
 constexpr uint32_t CROWD_BINS = 2048, CROWD_MAX = 4096, CROWD_CLASH_MAX = 64, CROWD_SEGMENTS = 32;
-__device__ __noinline__ void sort_crowded_bin(const atrex_entry_t* entries, bool ranking, ull* s_item, uint32_t b0, uint32_t n, uint32_t* s_bins) {
+__device__ __forceinline__ void sort_crowded_bin(const atrex_entry_t* entries, bool ranking, ull* s_item, uint32_t b0, uint32_t n, uint32_t* s_bins) {
     __shared__ ull s_range[2];
     __shared__ uint32_t s_warp[32], s_segments;
     __shared__ uint16_t s_from[CROWD_SEGMENTS], s_size[CROWD_SEGMENTS];
@@ -1024,10 +1024,19 @@ __device__ __forceinline__ void sort_small_bin(const atrex_entry_t* entries, boo
         if (u * 32 + lane < n) s_item[before[u]] = item[u];
 }
 
-// A tile's crowded local bins, and those with ties: bit u of `tied` is a thread's bin u * TILE_THREADS + threadIdx.x (whole CTA, behind a
-// barrier; the local bins are not needed any more).
+// Crowded local bins of up to TILE_SMALL_CROWD items, a warp each (the others go on).
+__device__ __forceinline__ void sort_small_crowds(const atrex_entry_t* entries, bool ranking, ull* s_item, const uint32_t* s_local, const uint16_t* s_bin,
+                                                  uint32_t crowded) {
+    for (uint32_t k = threadIdx.x >> 5; k < crowded; k += TILE_THREADS / 32) {
+        const uint32_t d = s_bin[k], b0 = d ? s_local[d - 1] : 0u, n = s_local[d] - b0;
+        if (n <= TILE_SMALL_CROWD) sort_small_bin(entries, ranking, s_item + b0, n);
+    }
+}
+
+// A tile's other crowded local bins, and those with ties: bit u of `tied` is a thread's bin u * TILE_THREADS + threadIdx.x (whole CTA, behind a
+// barrier; the local bins are not needed any more).  A function of its own, as in place it costs every tile registers.
 __device__ __noinline__ void sort_crowds(const atrex_entry_t* entries, bool ranking, ull* s_item, uint32_t* s_local, const uint16_t* s_bin, uint32_t crowded,
-                                         uint32_t tied) {
+                                         uint32_t tied, bool any_tied) {
     constexpr uint32_t WARPS = TILE_THREADS / 32, WORDS = TILE_LOCAL_BINS / 32;
     static_assert(WARPS == 16 && WORDS == 4 * 32, "a word's bins go to two lots of sixteen warps, a lane looks at four words");
     __shared__ uint32_t s_tied[WORDS];                   // a bit for every local bin
@@ -1038,32 +1047,30 @@ __device__ __noinline__ void sort_crowds(const atrex_entry_t* entries, bool rank
         begin = d ? s_local[d - 1] : 0u;
         size = s_local[d] - begin;
     }
+    if (any_tied) {
 #pragma unroll
-    for (uint32_t u = 0; u < TILE_LOCAL_BINS / TILE_THREADS; ++u) {
-        const uint32_t votes = __ballot_sync(FULL, tied >> u & 1u);
-        if (lane == 0) s_tied[u * WARPS + w] = votes;
-    }
-    __syncthreads();
-    const uint32_t by_warp = crowded > TILE_CROWDED_FEW ? TILE_SMALL_CROWD : 0u;
-    for (uint32_t k = w; k < crowded; k += WARPS) {
-        const uint32_t b0 = __shfl_sync(FULL, begin, k), n = __shfl_sync(FULL, size, k);
-        if (n <= by_warp) sort_small_bin(entries, ranking, s_item + b0, n);
-    }
-    // bins next to one another go to different warps: groups of ties come side by side
+        for (uint32_t u = 0; u < TILE_LOCAL_BINS / TILE_THREADS; ++u) {
+            const uint32_t votes = __ballot_sync(FULL, tied >> u & 1u);
+            if (lane == 0) s_tied[u * WARPS + w] = votes;
+        }
+        __syncthreads();
+        // bins next to one another go to different warps: groups of ties come side by side
 #pragma unroll
-    for (uint32_t v = 0; v < 4; ++v) {
-        const uint32_t word = v * 32 + lane, own = s_tied[word] & 0x00010001u << ((w + word) & 15u);
-        for (uint32_t todo = __ballot_sync(FULL, own != 0); todo; todo &= todo - 1) {
-            const uint32_t src = __ffs(todo) - 1;
-            for (uint32_t bits = __shfl_sync(FULL, own, src); bits; bits &= bits - 1) {
-                const uint32_t d = (v * 32 + src) * 32 + __ffs(bits) - 1, b0 = d ? s_local[d - 1] : 0u;
-                sort_small_bin(entries, ranking, s_item + b0, s_local[d] - b0);
+        for (uint32_t v = 0; v < 4; ++v) {
+            const uint32_t word = v * 32 + lane, own = s_tied[word] & 0x00010001u << ((w + word) & 15u);
+            for (uint32_t todo = __ballot_sync(FULL, own != 0); todo; todo &= todo - 1) {
+                const uint32_t src = __ffs(todo) - 1;
+                for (uint32_t bits = __shfl_sync(FULL, own, src); bits; bits &= bits - 1) {
+                    const uint32_t d = (v * 32 + src) * 32 + __ffs(bits) - 1, b0 = d ? s_local[d - 1] : 0u;
+                    sort_small_bin(entries, ranking, s_item + b0, s_local[d] - b0);
+                }
             }
         }
     }
+    const uint32_t sorted = crowded > TILE_CROWDED_FEW ? TILE_SMALL_CROWD : 0u;
     for (uint32_t k = 0; k < crowded; ++k) {
         const uint32_t b0 = __shfl_sync(FULL, begin, k), n = __shfl_sync(FULL, size, k);
-        if (n > by_warp) sort_crowded_bin(entries, ranking, s_item, b0, n, s_local);
+        if (n > sorted) sort_crowded_bin(entries, ranking, s_item, b0, n, s_local);
     }
 }
 
@@ -1129,6 +1136,7 @@ __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ran
     const uint32_t crowded = s_crowded;   // (nothing adds to it behind the first barrier)
     // (a bin's cursor now stands at its end, its predecessor's at its start)
     if (crowded <= TILE_CROWDED) {
+        if (crowded > TILE_CROWDED_FEW) sort_small_crowds(entries, ranking, s_item, s_local, s_bin, crowded);   // (beside the insertion)
         uint32_t tied = 0;                               // (a thread has eight local bins at most)
         for (uint32_t d = threadIdx.x; d < LOCAL_BINS; d += TILE_THREADS) {
             const uint32_t b0 = d ? s_local[d - 1] : 0u, b1 = s_local[d];
@@ -1151,7 +1159,8 @@ __device__ __forceinline__ void sort_tile(const atrex_entry_t* entries, bool ran
                 s_item[j] = item;
             }
         }
-        if (__syncthreads_or(tied) || crowded != 0) sort_crowds(entries, ranking, s_item, s_local, s_bin, crowded, tied);
+        const bool any_tied = __syncthreads_or(tied) != 0;
+        if (any_tied || crowded != 0) sort_crowds(entries, ranking, s_item, s_local, s_bin, crowded, tied, any_tied);
     } else {
         bitonic(n, [&](uint32_t a, uint32_t b) { return item_less(entries, ranking, s_item[a], s_item[b]); },
                 [&](uint32_t a, uint32_t b) { const ull x = s_item[a]; s_item[a] = s_item[b]; s_item[b] = x; });
