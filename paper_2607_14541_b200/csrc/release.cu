@@ -871,7 +871,7 @@ __device__ __forceinline__ void bitonic(uint32_t n, Less less, Swap swap) {
 // smallest and the largest of what their leading bits left out -- the weighted times' 57 bits, or the keys where those are all
 // alike --, bins that are still crowded again, and so on.  Items that nothing tells apart but their entries' order, and more than CROWD_MAX, go
 // through the network, which reads entries at every comparison.  `s_bins`: CROWD_BINS + CROWD_MAX / 2 words.  (1.6 M rows, 1 600
-// of them at the clamp of their weights: the tile that held those went through a network as a whole, kernel 90 us, now 75 with the weighted
+// of them at the clamp of their weights: the tile that held those went through a network as a whole, kernel 90 us, now 80 with the weighted
 // times written for the shares; 7.5 M rows, 7 500 of them: 572, now 367)
 constexpr uint32_t CROWD_BINS = 2048, CROWD_MAX = 4096, CROWD_CLASH_MAX = 64, CROWD_SEGMENTS = 32;
 __device__ __forceinline__ void sort_crowded_bin(const atrex_entry_t* entries, bool ranking, ull* s_item, uint32_t b0, uint32_t n, uint32_t* s_bins) {
@@ -1208,7 +1208,7 @@ __device__ __forceinline__ void gather_tile(const atrex_entry_t* entries, const 
 }
 
 // 5. a tile's items in order, their entries gathered; (ranking) the weighted times of the rows and their sum.  A kernel per order: in one for
-//    both, what only the other needs costs the key order 2 % and more (15 M entries: tile kernel 565 us, now 552).
+//    both, what only the other needs costs the key order 2 % and more (15 M entries: tile kernel 565 us, now 548).
 template <uint32_t LOCAL_BINS, bool RANKING>
 __global__ void __launch_bounds__(TILE_THREADS) bin_tile_kernel(const BinSort b, atrex_entry_t* out, uint32_t out_cap) {
     extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -908,8 +908,8 @@ __global__ void __launch_bounds__(1024)
 // the key's range, a warp finds the range that holds the middle, and the few units in it (or as close to it as
 // keys may err) are ranked by their exact scores.  Every step but the finding is spread over the whole CTA, and units stay
 // where they are, so that nothing is worked out about the grouping.  Where the middle's range holds too many units it is
-// cut again; what stays too many (ties) is searched among them.  Bound by latency at 45 warps per SM (loads, shared-memory
-// atomics, barriers: 52 % of the issue slots).  1 000 candidates x 12 001 units x 7 operators: 145 us by score_cta_kernel, 78;
+// cut again; what stays too many (ties) is searched among them.  Bound by latency at 44 warps per SM (loads, shared-memory
+// atomics, barriers: 51 % of the issue slots).  1 000 candidates x 12 001 units x 7 operators: 145 us by score_cta_kernel, 78;
 // with the next loads issued before a thread's units are worked on 116 (spills); strides not known at compile time 86.
 constexpr uint32_t NEAR_MAX = 32;             // units near an operator's middle that one warp ranks, a lane each
 constexpr uint32_t BINS_LOW = (127u - 7u) << 23, BINS_LOG_SPAN = 26;   // first cut: scores from 2^-7 to 2, what lies outside in the end bins
